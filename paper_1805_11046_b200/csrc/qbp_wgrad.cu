@@ -90,6 +90,7 @@ struct WgradParams {
     const long long *rowterm, *colterm;
     const qbp_qparams *qx, *qg;
     long long *acc_out; float *dW;
+    int dW_vec;                      // dW starts on a 16-byte boundary
     int *status;
     // Convolution: per-channel totals of the stored codes over all positions (x: [C]; the 16-bit gradient codes
     // 256 * hi + lo: [N]) that the kernels which wrote the codes left.  The class tables then hold the border classes
@@ -377,6 +378,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
     __shared__ uint32_t tmem_slot;
     __shared__ int4 s_load[kWgMaxLoads];      // (destination offset in the stage, 0 x / 1 hi / 2 lo, channel offset, tap dw | dh << 16)
     __shared__ int s_counts[1];               // loads per stage
+    __shared__ long long s_cterm[128];        // direct epilogue: the tile's column terms
 
     const uint32_t raw_addr = smem_u32(smem_raw);
     uint8_t *smem = smem_raw + ((1024u - (raw_addr & 1023u)) & 1023u);
@@ -537,6 +539,11 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
                 if (tl[i]) atomicAdd(P.cls_lo + i, (unsigned long long)(long long)tl[i]);
             }
         }
+        if (P.direct) {
+            const int t = threadIdx.x - 64;
+            if (t < P.bn) s_cterm[t] = (int64_t)n0 + t < P.N ? P.colterm[n0 + t] : 0;
+            named_barrier(3, 128);
+        }
         if (k_iters > 0 && !mbar_wait_warp(&acc_bar, 0)) timed_out = true;
         tc_fence_after();
         if (!timed_out && k_iters > 0) {
@@ -564,14 +571,27 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
                     }
                     if (!valid) continue;
                     if (P.direct) {
-                        // the whole reduction is here: zero-points, scale, store
+                        // the whole reduction is here: zero-points, scale, store (N is a multiple of 16: groups of four
+                        // columns are whole; the column terms come from shared memory -- read per element from global
+                        // memory, between stores they might alias, they cost a load latency each)
+                        const int64_t at_out = k * P.N + n0 + c0;
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) {
-                            const int64_t n = (int64_t)n0 + c0 + e;
-                            if (n < P.N) {
-                                const long long acc = 256ll * (long long)(int)rh[e] + (long long)(int)rl[e] + rterm + P.colterm[n];
-                                if (P.acc_out) P.acc_out[k * P.N + n] = acc;
-                                if (P.dW) P.dW[k * P.N + n] = __fmul_rn((float)acc, scale);
+                        for (int e = 0; e < 32; e += 4) {
+                            if ((int64_t)n0 + c0 + e >= P.N) break;
+                            long long a4[4];
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) a4[q] = 256ll * (long long)(int)rh[e + q] + (long long)(int)rl[e + q] + rterm + s_cterm[c0 + e + q];
+                            if (P.acc_out) {
+                                long long *dst = P.acc_out + at_out + e;
+#pragma unroll
+                                for (int q = 0; q < 4; ++q) dst[q] = a4[q];
+                            }
+                            if (P.dW) {
+                                const float4 v = make_float4(__fmul_rn((float)a4[0], scale), __fmul_rn((float)a4[1], scale),
+                                                             __fmul_rn((float)a4[2], scale), __fmul_rn((float)a4[3], scale));
+                                float *dst = P.dW + at_out + e;
+                                if (P.dW_vec) *reinterpret_cast<float4 *>(dst) = v;
+                                else { dst[0] = v.x; dst[1] = v.y; dst[2] = v.z; dst[3] = v.w; }
                             }
                         }
                     } else if (P.conv) {
@@ -879,14 +899,12 @@ __global__ void wgrad_terms_kernel(const long long *__restrict__ sx, const long 
 
 // Adds the CTAs' partials, applies the zero-points and dequantises:
 //   acc = raw - zg * SX - zx * SG + count * zx * zg
-// where SX / SG / count are taken over the positions at which the tap is inside
-// the image.  Output element e: plain [k][n]; conv [k][tap][c].
+// Plain product [k][n]: SX / SG are the column sums, count = M.  kWgFinalizeLanes lanes per output element share its slices (an
+// element's partials are few hundred bytes each, far apart: one thread walking them alone is bound by latency).
 __global__ void __launch_bounds__(256) wgrad_finalize_kernel(const WgradParams P, const long long *__restrict__ sx,
                                                              const long long *__restrict__ shi,
                                                              const long long *__restrict__ slo, int64_t total)
 {
-    // kWgFinalizeLanes lanes per output element share its slices (an element's partials are few hundred bytes each, far apart:
-    // one thread walking them alone is bound by latency)
     constexpr int kLanes = kWgFinalizeLanes;
     const int64_t e_raw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kLanes;
     const int part_lane = threadIdx.x % kLanes;
@@ -894,55 +912,18 @@ __global__ void __launch_bounds__(256) wgrad_finalize_kernel(const WgradParams P
     const int64_t e = live ? e_raw : total - 1;           // (idle lanes of the last warp compute a duplicate and do not store)
     // (signed low bytes: the limbs hold g16 - 128, against the zero-point zg - 128)
     const long long zx = P.qx->zero_point, zg = P.qg->zero_point - (P.lo_signed ? 128 : 0);
-    long long SX = 0, SG = 0, count = 0;
-    int at, row, n;                                     // accumulator tile, row in it, output column of g
-    if (!P.conv) {
-        const int64_t k = e / P.N;
-        n = (int)(e % P.N);
-        at = (int)(k / 128); row = (int)(k % 128);
-        SX = sx[k];
-        SG = 256 * shi[n] + slo[n];
-        count = P.M;
-    } else {
-        const int c = (int)(e % P.C);
-        const int tap = (int)((e / P.C) % P.taps);
-        n = (int)(e / ((int64_t)P.C * P.taps));
-        const int r = tap / P.S, s = tap % P.S, pad = P.pad;
-        at = (tap / P.a_chunks) * P.tiles_c + c / P.rb_a;
-        row = (tap % P.a_chunks) * P.rb_a + c % P.rb_a;
-        // positions of g that see this tap: p - pad + r in [0,H)  <=>  not (r<pad and first row), not (r>pad and last row);
-        // positions of x that are seen:      h + pad - r in [0,H)  <=>  not (r<pad and last row),  not (r>pad and first row).
-        if (P.tot_x) {
-            // totals over all positions, less the border classes this tap does not see (the interior always counts)
-            SX = P.tot_x[c]; SG = P.tot_g[n];
-            if (P.lo_signed && P.tot_g_plain) SG -= 128ll * P.Nimg * P.H * P.W;
-            for (int cls = 1; cls < 16; ++cls) {
-                const bool top = cls & 1, bottom = cls & 2, left = cls & 4, right = cls & 8;
-                const bool g_ok = !((r < pad && top) || (r > pad && bottom) || (s < pad && left) || (s > pad && right));
-                const bool x_ok = !((r < pad && bottom) || (r > pad && top) || (s < pad && right) || (s > pad && left));
-                if (!g_ok) SG -= 256 * shi[cls * P.N + n] + slo[cls * P.N + n];
-                if (!x_ok) SX -= sx[cls * P.C + c];
-            }
-        } else
-        for (int cls = 0; cls < 16; ++cls) {
-            const bool top = cls & 1, bottom = cls & 2, left = cls & 4, right = cls & 8;
-            const bool g_ok = !((r < pad && top) || (r > pad && bottom) || (s < pad && left) || (s > pad && right));
-            const bool x_ok = !((r < pad && bottom) || (r > pad && top) || (s < pad && right) || (s > pad && left));
-            if (g_ok) SG += 256 * shi[cls * P.N + n] + slo[cls * P.N + n];
-            if (x_ok) SX += sx[cls * P.C + c];
-        }
-        const long long rows_ok = P.H - (r < pad ? pad - r : r - pad), cols_ok = P.W - (s < pad ? pad - s : s - pad);
-        count = (long long)P.Nimg * (rows_ok > 0 ? rows_ok : 0) * (cols_ok > 0 ? cols_ok : 0);
-    }
+    const int64_t k = e / P.N;
+    const int n = (int)(e % P.N);
+    const int at = (int)(k / 128), row = (int)(k % 128);  // accumulator tile, row in it
+    const long long SX = sx[k], SG = 256 * shi[n] + slo[n];
     // the CTAs of this element's item
     const int ag = at / P.ma, j = at % P.ma, tb = n / P.bn, col = n % P.bn;
     const int item = ag * P.tiles_b + tb;
     const int full_items = P.ctas_full / P.s_full;
     const int first = item < full_items ? item * P.s_full : P.ctas_full + (item - full_items) * P.s_last;
     const int slices = item < full_items ? P.s_full : P.s_last;
-    const int64_t off = P.conv ? ((int64_t)j * P.bn + col) * 128 + row : ((int64_t)j * 128 + row) * P.bn + col;
     long long raw = 0;
-    const long long *src = P.part + (int64_t)first * P.part_stride + off;
+    const long long *src = P.part + (int64_t)first * P.part_stride + ((int64_t)j * 128 + row) * P.bn + col;
     int sl = part_lane;
     for (; sl + 7 * kLanes < slices; sl += 8 * kLanes) {
         long long v[8];
@@ -955,9 +936,108 @@ __global__ void __launch_bounds__(256) wgrad_finalize_kernel(const WgradParams P
 #pragma unroll
     for (int o = 1; o < kLanes; o <<= 1) raw += __shfl_xor_sync(0xffffffffu, raw, o);
     if (!live || part_lane != 0) return;
-    const long long acc = raw - zg * SX - zx * SG + count * zx * zg;
+    const long long acc = raw - zg * SX - zx * SG + P.M * zx * zg;
     if (P.acc_out) P.acc_out[e] = acc;
     if (P.dW) P.dW[e] = __fmul_rn((float)acc, __fmul_rn(P.qx->scale, P.qg->scale));
+}
+
+// The part of SX (of_x: over the positions of x that tap (r, s) sees) or SG (over the positions of g at which it is inside
+// the image) that four of the sixteen border classes contribute (cls = 4 i + q): with totals, what those classes take off the
+// total; without, what they hold.
+__device__ __forceinline__ long long wg_class_part(const WgradParams &P, bool of_x, int ch, int r, int s, int q,
+                                                   const long long *__restrict__ ta, const long long *__restrict__ tb)
+{
+    const int pad = P.pad, width = of_x ? P.C : (int)P.N;
+    const bool totals = P.tot_x != nullptr;
+    long long sum = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int cls = 4 * i + q;
+        const bool top = cls & 1, bottom = cls & 2, left = cls & 4, right = cls & 8;
+        // positions of g that see this tap: p - pad + r in [0,H)  <=>  not (r<pad and first row), not (r>pad and last row);
+        // positions of x that are seen:      h + pad - r in [0,H)  <=>  not (r<pad and last row),  not (r>pad and first row).
+        const bool ok = of_x ? !((r < pad && bottom) || (r > pad && top) || (s < pad && right) || (s > pad && left))
+                             : !((r < pad && top) || (r > pad && bottom) || (s < pad && left) || (s > pad && right));
+        if (ok != totals) {               // (totals: the classes not seen; the interior always is)
+            const long long v = of_x ? ta[cls * width + ch] : 256 * ta[cls * width + ch] + tb[cls * width + ch];
+            sum += totals ? -v : v;
+        }
+    }
+    return sum;
+}
+
+// The same for a convolution, output [n][tap][c].  A block takes 64 channels of one tap and NB output channels: the class
+// sums behind SX and SG are added up once per block instead of once per element (thirty and more loads each, which made
+// this kernel 78 us for a 256 -> 256 channel 3x3 filter, five times what its partials take to read), four groups
+// of 64 threads share the slices, each thread with eight loads in flight, and meet in shared memory.
+template <int NB>
+__global__ void __launch_bounds__(256) wgrad_conv_finalize_kernel(const WgradParams P, const long long *__restrict__ sx,
+                                                                  const long long *__restrict__ shi,
+                                                                  const long long *__restrict__ slo)
+{
+    constexpr int U = 8 / NB;                              // slices in flight per output channel
+    __shared__ long long s_part[NB][4][64], s_sx[4][64], s_sg[4][NB];
+    const int cblocks = (P.C + 63) / 64;
+    const int tap = (int)blockIdx.x / cblocks, c = ((int)blockIdx.x % cblocks) * 64 + (threadIdx.x & 63);
+    const int q = threadIdx.x >> 6;
+    const int n0 = (int)blockIdx.y * NB;
+    const int r = tap / P.S, s = tap % P.S, pad = P.pad;
+    const bool c_ok = c < P.C;
+    // the CTAs of this channel's items
+    const int at = (tap / P.a_chunks) * P.tiles_c + (c_ok ? c : 0) / P.rb_a, row = (tap % P.a_chunks) * P.rb_a + (c_ok ? c : 0) % P.rb_a;
+    const int ag = at / P.ma, j = at % P.ma, full_items = P.ctas_full / P.s_full;
+    long long raw[NB];
+    const long long *src[NB];
+    int slices = 0;
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        const int n = min(n0 + i, (int)P.N - 1);
+        const int item = ag * P.tiles_b + n / P.bn;
+        const int first = item < full_items ? item * P.s_full : P.ctas_full + (item - full_items) * P.s_last;
+        slices = item < full_items ? P.s_full : P.s_last;  // (the same for all: it depends on the A group alone)
+        src[i] = P.part + (int64_t)first * P.part_stride + ((int64_t)j * P.bn + n % P.bn) * 128 + row;
+        raw[i] = 0;
+    }
+    if (c_ok) {
+        int sl = q;
+        for (; sl + 4 * (U - 1) < slices; sl += 4 * U) {
+            long long v[NB][U];
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+#pragma unroll
+                for (int u = 0; u < U; ++u) v[i][u] = __ldcs(src[i] + (int64_t)(sl + 4 * u) * P.part_stride);
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+#pragma unroll
+                for (int u = 0; u < U; ++u) raw[i] += v[i][u];
+        }
+        for (; sl < slices; sl += 4)
+#pragma unroll
+            for (int i = 0; i < NB; ++i) raw[i] += __ldcs(src[i] + (int64_t)sl * P.part_stride);
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) s_part[i][q][threadIdx.x & 63] = raw[i];
+    s_sx[q][threadIdx.x & 63] = c_ok ? wg_class_part(P, true, c, r, s, q, sx, nullptr) : 0;
+    if ((threadIdx.x & 63) < NB) s_sg[q][threadIdx.x & 63] = wg_class_part(P, false, min(n0 + (int)(threadIdx.x & 63), (int)P.N - 1), r, s, q, shi, slo);
+    __syncthreads();
+    // (signed low bytes: the limbs hold g16 - 128, against the zero-point zg - 128)
+    const long long zx = P.qx->zero_point, zg = P.qg->zero_point - (P.lo_signed ? 128 : 0);
+    const long long rows_ok = P.H - (r < pad ? pad - r : r - pad), cols_ok = P.W - (s < pad ? pad - s : s - pad);
+    const long long count = (long long)P.Nimg * (rows_ok > 0 ? rows_ok : 0) * (cols_ok > 0 ? cols_ok : 0);
+    const float scale = __fmul_rn(P.qx->scale, P.qg->scale);
+    for (int i = threadIdx.x; i < NB * 64; i += 256) {
+        const int cl = i & 63, nl = i >> 6, n = n0 + nl, co = ((int)blockIdx.x % cblocks) * 64 + cl;
+        if (n >= P.N || co >= P.C) continue;
+        long long SX = s_sx[0][cl] + s_sx[1][cl] + s_sx[2][cl] + s_sx[3][cl], SG = s_sg[0][nl] + s_sg[1][nl] + s_sg[2][nl] + s_sg[3][nl];
+        if (P.tot_x) {
+            SX += P.tot_x[co]; SG += P.tot_g[n];
+            if (P.lo_signed && P.tot_g_plain) SG -= 128ll * P.Nimg * P.H * P.W;
+        }
+        const long long acc = s_part[nl][0][cl] + s_part[nl][1][cl] + s_part[nl][2][cl] + s_part[nl][3][cl] - zg * SX - zx * SG + count * zx * zg;
+        const int64_t e = ((int64_t)n * P.taps + tap) * P.C + co;
+        if (P.acc_out) P.acc_out[e] = acc;
+        if (P.dW) P.dW[e] = __fmul_rn((float)acc, scale);
+    }
 }
 
 // Pixel box of `rows` = bw x bh x bn positions (powers of two) that needs the fewest steps.
@@ -1036,6 +1116,8 @@ static void plan_wgrad(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, 
     // the groups that takes (5 tiles: 3 + 2 rather than 4 + 1 -- a stage of few MMAs is bound by its fixed costs)
     const int ma_max = std::max(1, std::min({kWgMaxTiles, 512 / (2 * P.bn), P.a_tiles}));
     P.a_groups = (P.a_tiles + ma_max - 1) / ma_max;
+    // (a plain product whose tiles do not fill the machine: one A tile per CTA)
+    if (!d && (int64_t)P.a_tiles * P.tiles_b <= sm_count()) P.a_groups = P.a_tiles;
     P.ma = (P.a_tiles + P.a_groups - 1) / P.a_groups;
     int cols = 32; while (cols < P.ma * 2 * P.bn) cols <<= 1;
     P.tmem_cols = cols;
@@ -1112,6 +1194,8 @@ static void plan_wgrad(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, 
         int64_t s = (int64_t)T * cost(tiles) / weight;
         s = std::max<int64_t>(s, min_slices);
         s = std::max<int64_t>(1, std::min<int64_t>(s, P.iters_total));
+        // a short plain reduction (at most 1024 rows) stays whole: no partials and no second kernel
+        if (!d && P.iters_total <= 8) s = 1;
         return (int)s;
     };
     P.s_full = slices_for(P.ma);
@@ -1306,7 +1390,7 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
 
     P.part = (long long *)part; P.status = status;
     P.rowterm = (const long long *)rowterm; P.colterm = (const long long *)colterm;
-    P.qx = qx; P.qg = qg16; P.acc_out = (long long *)acc_out; P.dW = dW;
+    P.qx = qx; P.qg = qg16; P.acc_out = (long long *)acc_out; P.dW = dW; P.dW_vec = aligned16(dW) ? 1 : 0;
     const uint32_t kr = (uint32_t)P.kr, rb_a = (uint32_t)P.rb_a, rb_b = (uint32_t)P.bn;
     if (!d) {
         if ((rc = make_map_2d(&P.mapX, x, M, K, kr, rb_a))) return rc;
@@ -1337,7 +1421,17 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
     QBP_TRACE_BEGIN(st);
     kernel<<<pl.grid, kWgThreads, pl.smem, st>>>(P);
     QBP_LAUNCH_OK("qbp_wgrad_kernel");
-    if (!P.direct) {
+    if (d) {
+        // output channels per block: as many as still leave four blocks per SM
+        const int64_t per_n = (int64_t)P.taps * ((d->C + 63) / 64);
+        const int nb = per_n * (d->K / 8) >= 4ll * sm_count() ? 8 : per_n * (d->K / 4) >= 4ll * sm_count() ? 4 : 2;
+        const dim3 grid((unsigned)per_n, (unsigned)((d->K + nb - 1) / nb));
+        QBP_TRACE_BEGIN(st);
+        if (nb == 8)      wgrad_conv_finalize_kernel<8><<<grid, 256, 0, st>>>(P, (const long long *)sx, (const long long *)shi, (const long long *)slo);
+        else if (nb == 4) wgrad_conv_finalize_kernel<4><<<grid, 256, 0, st>>>(P, (const long long *)sx, (const long long *)shi, (const long long *)slo);
+        else              wgrad_conv_finalize_kernel<2><<<grid, 256, 0, st>>>(P, (const long long *)sx, (const long long *)shi, (const long long *)slo);
+        QBP_LAUNCH_OK("wgrad_finalize_kernel");
+    } else if (!P.direct) {
         const int blocks = (int)((outs * kWgFinalizeLanes + 255) / 256);
         QBP_TRACE_BEGIN(st);
         wgrad_finalize_kernel<<<blocks, 256, 0, st>>>(P, (const long long *)sx, (const long long *)shi, (const long long *)slo, outs);

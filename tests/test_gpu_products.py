@@ -411,3 +411,33 @@ def test_conv_at_full_size_is_reproducible(B, mode):
             assert not bool(torch.isnan(out).any())
         else:
             assert int((bits != ref).sum()) == 0, f"run {rep} differs from run 0"
+
+
+# ------------------------------------------- the weight gradient's two ways of finishing
+@pytest.mark.parametrize("M,N,K,shift", [(16, 16, 16, 0), (64, 128, 256, 0), (64, 128, 256, 1), (496, 112, 1008, 0), (1024, 144, 272, 0),
+                                         (1040, 128, 272, 0)])
+def test_wgrad_plain_whole_and_split_reductions(B, M, N, K, shift):
+    """At most 1024 rows stay whole (the product applies the zero-points itself), one more step of rows is split; one A
+    tile per CTA while the tiles do not fill the machine; dW on a 16-byte boundary and 4 bytes off it."""
+    import torch
+    X = random_codes((M, K), 51); G = np.random.Generator(np.random.PCG64(52)).integers(-32768, 32768, (M, N)).astype(np.int16)
+    hi, lo = O.limb_split(G)
+    dW = torch.full((K * N + 4,), float("nan"), dtype=torch.float32, device="cuda")[shift:shift + K * N].view(K, N)
+    acc, _, ws = B.qbp_wgrad_s16(to_dev(X), _qp(B, 0.5, -7), to_dev(hi), to_dev(lo), _qp(B, 0.25, 311), want_acc=True, dW=dW)
+    oacc, oout = O.gemm_s16s8(X, -7, G, 311, 0.5, 0.25)
+    assert B.status_word(ws) == 0
+    assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
+
+
+@pytest.mark.parametrize("N,H,W,C,K,R", [(2, 6, 6, 32, 32, 1), (2, 9, 7, 96, 160, 3), (2, 7, 9, 160, 192, 3), (3, 6, 5, 256, 256, 3)])
+def test_wgrad_conv_finalize_block_shapes(B, N, H, W, C, K, R):
+    """The kernel that adds the partials with two, four and eight output channels per block; channel blocks half filled and
+    spanning two accumulator tiles."""
+    pad = (R - 1) // 2
+    d = B.conv_desc(N, H, W, C, K, R, R, 1, pad); od = O.conv_desc(N, H, W, C, K, R, R, 1, pad)
+    X = random_codes((N, H, W, C), 53); G = np.random.Generator(np.random.PCG64(54)).integers(-32768, 32768, (N, H, W, K)).astype(np.int16)
+    hi, lo = O.limb_split(G)
+    acc, dW, ws = B.qbp_wgrad_s16(to_dev(X), _qp(B, 0.5, 9), to_dev(hi), to_dev(lo), _qp(B, 0.25, -77), d=d, want_acc=True)
+    oacc, oout = O.conv_wgrad_s16(od, X, 9, G, -77, 0.5, 0.25)
+    assert B.status_word(ws) == 0
+    assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
