@@ -80,11 +80,17 @@ static SideStream *side_stream()
     return c.ok ? &c : nullptr;
 }
 // Runs what the caller enqueues on `side` between the event `fork` (already recorded on st) and the rest of st.
-static int side_begin(SideStream *sd) { QBP_CUDA_OK(cudaStreamWaitEvent(sd->s, sd->fork, 0)); return QBP_OK; }
+static int side_begin(SideStream *sd)
+{
+    QBP_CUDA_OK(cudaStreamWaitEvent(sd->s, sd->fork, 0));
+    launch_next_in_full();
+    return QBP_OK;
+}
 static int side_end(SideStream *sd, cudaStream_t st)
 {
     QBP_CUDA_OK(cudaEventRecord(sd->join, sd->s));
     QBP_CUDA_OK(cudaStreamWaitEvent(st, sd->join, 0));
+    launch_next_in_full();
     return QBP_OK;
 }
 

@@ -445,6 +445,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_trigger();                       // (tensor memory is allocated)
+    pdl_wait();
     const uint32_t tmem_base = tmem_slot;
     const uint32_t buf_cols = (uint32_t)(P.msub * P.bn);
     bool timed_out = false;
@@ -835,6 +837,7 @@ __global__ void gemm_terms_kernel(const int32_t *ra32, const long long *ra64, co
                                   int64_t M, int64_t N, int64_t K, const qbp_qparams *qa, const qbp_qparams *qb,
                                   int32_t *rowterm, int32_t *colterm)
 {
+    pdl_enter();
     const int za = qa->zero_point, zb = qb->zero_point;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < M) {
@@ -854,6 +857,7 @@ __global__ void gemm_terms_kernel(const int32_t *ra32, const long long *ra64, co
 __global__ void conv_colterm_kernel(const int32_t *wsum32, const long long *wsum64, int N, int R, int S, int pad,
                                     int dgrad, const qbp_qparams *q_in, int32_t *colterm)
 {
+    pdl_enter();
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     const int cls = blockIdx.y;
     if (n >= N) return;
@@ -883,6 +887,7 @@ __global__ void __launch_bounds__(1024) filter_prep_kernel(const float *__restri
                                                             const qbp_qparams *__restrict__ q_in, int8_t *__restrict__ codes,
                                                             qbp_qparams *__restrict__ qp_out, int32_t *__restrict__ colterm)
 {
+    pdl_enter();
     extern __shared__ int s_wsum[];                      // [K * taps]
     __shared__ float s_lo[32], s_hi[32];
     __shared__ float s_inv, s_zp;
@@ -942,6 +947,7 @@ __global__ void __launch_bounds__(1024) filter_dgrad_colterm_kernel(const int8_t
                                                                      int S, int pad, const qbp_qparams *__restrict__ q_g,
                                                                      int32_t *__restrict__ colterm)
 {
+    pdl_enter();
     extern __shared__ int s_wsum[];                      // [taps * C]
     const int cols4 = taps * C / 4;
     for (int j = threadIdx.x; j < cols4; j += 1024) {
@@ -978,6 +984,7 @@ __global__ void __launch_bounds__(256) conv_rowterm_kernel(const int32_t *__rest
                                                            FastDiv dW, int pad, int Cred, const qbp_qparams *q_in,
                                                            const qbp_qparams *q_w, int32_t *__restrict__ rowterm)
 {
+    pdl_enter();
     const int i = (int)blockIdx.x * 256 + (int)threadIdx.x;
     if (i >= HW) return;
     int p, q;
@@ -1009,6 +1016,7 @@ __global__ void __launch_bounds__(128) colstat_finalize_kernel(const float *__re
                                                                double *__restrict__ col_sum, float *__restrict__ col_min,
                                                                float *__restrict__ col_max)
 {
+    pdl_enter();
     const int c = blockIdx.x;
     float lo = INFINITY, hi = -INFINITY;
     double sum = 0.0;
@@ -1042,7 +1050,7 @@ int launch_filter_dgrad_colterm(const qbp_conv_desc *d, const int8_t *codes, con
 {
     const int taps = d->R * d->S;
     QBP_TRACE_BEGIN(st);
-    filter_dgrad_colterm_kernel<<<1, 1024, sizeof(int) * (size_t)taps * d->C, st>>>(codes, d->K, taps, d->C, d->R, d->S, d->pad, q_g, colterm);
+    launch(filter_dgrad_colterm_kernel, 1, 1024, sizeof(int) * (size_t)taps * d->C, st, codes, d->K, taps, d->C, d->R, d->S, d->pad, q_g, colterm);
     QBP_LAUNCH_OK("filter_dgrad_colterm_kernel");
     return QBP_OK;
 }
@@ -1052,7 +1060,7 @@ int launch_filter_prep(const qbp_conv_desc *d, const float *w, const qbp_qparams
 {
     const int taps = d->R * d->S;
     QBP_TRACE_BEGIN(st);
-    filter_prep_kernel<<<1, 1024, sizeof(int) * (size_t)d->K * taps, st>>>(w, d->K, taps, d->C, d->R, d->S, d->pad, q_in, codes, qw, colterm);
+    launch(filter_prep_kernel, 1, 1024, sizeof(int) * (size_t)d->K * taps, st, w, d->K, taps, d->C, d->R, d->S, d->pad, q_in, codes, qw, colterm);
     QBP_LAUNCH_OK("filter_prep_kernel");
     return QBP_OK;
 }
@@ -1080,6 +1088,7 @@ static size_t colstat_ws_bytes(int64_t N, bool conv = false)
 // Parameters of the requantisation in a product's epilogue from the caller's clamping values.
 __global__ void epilogue_qparams_kernel(const qbp_qparams *__restrict__ range, qbp_qparams *__restrict__ qp8)
 {
+    pdl_enter();
     *qp8 = make_qparams(range->vmin, range->vmax, 8);
 }
 
@@ -1109,7 +1118,7 @@ static int launch_epilogue_qparams(const qbp_epilogue *ep, cudaStream_t st)
 {
     if (!ep->q_out) return QBP_OK;
     QBP_TRACE_BEGIN(st);
-    epilogue_qparams_kernel<<<1, 1, 0, st>>>(ep->requant_range, ep->qp_out);
+    launch(epilogue_qparams_kernel, 1, 1, 0, st, ep->requant_range, ep->qp_out);
     QBP_LAUNCH_OK("epilogue_qparams_kernel");
     return QBP_OK;
 }
@@ -1117,7 +1126,7 @@ static int launch_epilogue_qparams(const qbp_epilogue *ep, cudaStream_t st)
 static int finish_epilogue(const qbp_epilogue *ep, const ColStatParts &parts, int64_t N, cudaStream_t st)
 {
     QBP_TRACE_BEGIN(st);
-    colstat_finalize_kernel<<<(int)N, 128, 0, st>>>(parts.lo, parts.hi, parts.sum, parts.rows, (int)N, ep->col_sum, ep->col_min, ep->col_max);
+    launch(colstat_finalize_kernel, (int)N, 128, 0, st, parts.lo, parts.hi, parts.sum, parts.rows, (int)N, ep->col_sum, ep->col_min, ep->col_max);
     QBP_LAUNCH_OK("colstat_finalize_kernel");
     return QBP_OK;
 }
@@ -1213,8 +1222,8 @@ static int launch_mma(MmaParams &P, int tiles_m, bool clear_status, cudaStream_t
     }
     P.grid = grid;
     QBP_TRACE_BEGIN(st);
-    if (tail) qbp_mma_kernel<true><<<grid, kMmaThreads, smem, st>>>(P);
-    else      qbp_mma_kernel<false><<<grid, kMmaThreads, smem, st>>>(P);
+    if (tail) launch(qbp_mma_kernel<true>, grid, kMmaThreads, smem, st, P);
+    else      launch(qbp_mma_kernel<false>, grid, kMmaThreads, smem, st, P);
     QBP_LAUNCH_OK("qbp_mma_kernel");
     return QBP_OK;
 }
@@ -1361,8 +1370,7 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
     const int32_t *ra32 = a_sums ? a_sums : (const int32_t *)tmp_m, *cb32 = b_sums ? b_sums : (const int32_t *)tmp_n;
     const int64_t mx = std::max(M, N);
     QBP_TRACE_BEGIN(st);
-    gemm_terms_kernel<<<(int)((mx + 255) / 256), 256, 0, st>>>(
-        a32 ? ra32 : nullptr, a32 ? nullptr : (const long long *)tmp_m,
+    launch(gemm_terms_kernel, (int)((mx + 255) / 256), 256, 0, st, a32 ? ra32 : nullptr, a32 ? nullptr : (const long long *)tmp_m,
         b32 ? cb32 : nullptr, b32 ? nullptr : (const long long *)tmp_n, M, N, K, qa, qb,
         rowterm, colterm);
     QBP_LAUNCH_OK("gemm_terms_kernel");
@@ -1520,14 +1528,12 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
             else        rc = launch_colsum(wgt, true, d->K, (int64_t)taps * d->C, wsum, st);                    // [tap][c]
             if (rc) return rc;
             QBP_TRACE_BEGIN(st);
-            conv_colterm_kernel<<<dim3((Nout + 127) / 128, 16), 128, 0, st>>>(
-                dgrad ? nullptr : (const int32_t *)wsum, dgrad ? (const long long *)wsum : nullptr, Nout, d->R, d->S, d->pad,
+            launch(conv_colterm_kernel, dim3((Nout + 127) / 128, 16), 128, 0, st, dgrad ? nullptr : (const int32_t *)wsum, dgrad ? (const long long *)wsum : nullptr, Nout, d->R, d->S, d->pad,
                 dgrad ? 1 : 0, q_in, colterm);
             QBP_LAUNCH_OK("conv_colterm_kernel");
         }
         QBP_TRACE_BEGIN(st);
-        conv_rowterm_kernel<<<dim3((unsigned)((d->H * d->W + 255) / 256), (unsigned)d->N), 256, 0, st>>>(
-            chan_sum, d->H * d->W, d->H, d->W, make_fastdiv(d->W), d->pad, Cred, q_in, q_w, rowterm);
+        launch(conv_rowterm_kernel, dim3((unsigned)((d->H * d->W + 255) / 256), (unsigned)d->N), 256, 0, st, chan_sum, d->H * d->W, d->H, d->W, make_fastdiv(d->W), d->pad, Cred, q_in, q_w, rowterm);
         QBP_LAUNCH_OK("conv_rowterm_kernel");
     }
 

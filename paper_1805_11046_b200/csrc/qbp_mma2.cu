@@ -205,6 +205,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
     __syncthreads();
     cluster_sync_all();                  // both CTAs' barriers are initialised before either signals the other
     tc_fence_after();
+    pdl_trigger();                       // (tensor memory is allocated, in both CTAs)
+    pdl_wait();
     const uint32_t tmem_base = tmem_slot;
     bool timed_out = false;
 
@@ -397,7 +399,7 @@ int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const 
     QBP_SMEM_OPT_IN(configured, qbp_mma2_kernel, k2Smem);
     if (clear_status) QBP_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
     QBP_TRACE_BEGIN(st);
-    qbp_mma2_kernel<<<2 * P.pairs, k2Threads, smem, st>>>(P);
+    launch(qbp_mma2_kernel, 2 * P.pairs, k2Threads, smem, st, P);
     QBP_LAUNCH_OK("qbp_mma2_kernel");
     return QBP_OK;
 }

@@ -57,6 +57,7 @@ static cudaEvent_t pool_event()
     cudaEventCreate(&e);
     return e;
 }
+bool trace_is_on() { return g_trace_on; }
 void trace_begin(cudaStream_t st)
 {
     if (!g_trace_on) return;
@@ -83,6 +84,7 @@ template <int VEC>
 __global__ void __launch_bounds__(kThreads) range_partial_kernel(const float *__restrict__ x, int64_t n,
                                                                  float2 *__restrict__ partials, int keep_rev)
 {
+    pdl_enter();
     float lo = INFINITY, hi = -INFINITY;
     const int64_t nv = n / VEC;
     const int64_t stride = (int64_t)gridDim.x * kThreads * kRangeUnroll;
@@ -120,6 +122,7 @@ __global__ void __launch_bounds__(kThreads) range_partial_kernel(const float *__
 __global__ void __launch_bounds__(kThreads) range_finalize_kernel(const float2 *__restrict__ partials, int nparts,
                                                                   qbp_qparams *qp8, qbp_qparams *qp16)
 {
+    pdl_enter();
     float lo = INFINITY, hi = -INFINITY;
     for (int i = threadIdx.x; i < nparts; i += kThreads) {
         float2 p = partials[i];
@@ -143,6 +146,7 @@ template <int VEC>
 __global__ void __launch_bounds__(kThreads) chunk_range_partial_kernel(const float *__restrict__ x, int64_t n_chunk,
                                                                        float2 *__restrict__ partials)
 {
+    pdl_enter();
     x += (int64_t)blockIdx.y * n_chunk;
     float lo = INFINITY, hi = -INFINITY;
     const int64_t nv = n_chunk / VEC;              // (VEC = 4 only when n_chunk is a multiple of 4)
@@ -182,6 +186,7 @@ __global__ void __launch_bounds__(kThreads) chunk_range_finalize_kernel(const fl
                                                                         int blocks_per_chunk, float2 *__restrict__ per_chunk,
                                                                         qbp_qparams *__restrict__ out)
 {
+    pdl_enter();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int k = warp; k < chunks; k += kThreads / 32) {
         float lo = INFINITY, hi = -INFINITY;
@@ -207,6 +212,7 @@ __global__ void __launch_bounds__(kThreads) chunk_range_finalize_kernel(const fl
 __global__ void qparams_from_range_kernel(const qbp_qparams *__restrict__ in, int count, int bits,
                                           qbp_qparams *__restrict__ out)
 {
+    pdl_enter();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < count) out[i] = make_qparams(in[i].vmin, in[i].vmax, bits);
 }
@@ -217,6 +223,7 @@ __global__ void __launch_bounds__(kScanThreads) chan_range_partial_kernel(const 
                                                                           int C, int tw, float *__restrict__ part_lo,
                                                                           float *__restrict__ part_hi)
 {
+    pdl_enter();
     const ScanPos p = scan_pos<VEC>(C, tw);
     const int rpb = kScanThreads / tw;
     float lo[VEC], hi[VEC];
@@ -265,6 +272,7 @@ __global__ void __launch_bounds__(kThreads) chan_range_finalize_kernel(const flo
                                                                        const float *__restrict__ part_hi, int nparts,
                                                                        int C, int bits, qbp_qparams *__restrict__ qp)
 {
+    pdl_enter();
     int c = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
     if (c >= C) return;
     float lo = INFINITY, hi = -INFINITY;
@@ -369,6 +377,7 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const float *__restr
                                                             uint32_t id16, const __grid_constant__ PhiloxKeys keys,
                                                             QuantOut o, int smem_cols, uint64_t index_base)
 {
+    pdl_enter();
     if (VEC == 1) {
         const int64_t stride = (int64_t)gridDim.x * kThreads;
         for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += stride)
@@ -528,6 +537,7 @@ template <bool IS_SIGNED>
 __global__ void __launch_bounds__(kThreads) rowsum_kernel(const uint8_t *__restrict__ q, int64_t rows, int cols,
                                                           int G, int32_t *__restrict__ sums)
 {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int gl = lane % G;
     const int64_t groups_per_block = kThreads / G;
@@ -557,6 +567,7 @@ template <bool IS_SIGNED>
 __global__ void __launch_bounds__(kThreads) colsum_kernel(const uint8_t *__restrict__ q, int64_t rows, int cols,
                                                           unsigned long long *__restrict__ sums)
 {
+    pdl_enter();
     const int cv = cols >> 4;
     const int slab0 = blockIdx.y * kThreads;                 // first column group of this slab
     const int tw = (cv - slab0) < kThreads ? (cv - slab0) : kThreads;
@@ -608,12 +619,12 @@ static int launch_range(const float *x, int64_t n, float2 *partials, qbp_qparams
                           (n + per_block - 1) / per_block);
         if (nparts > kMaxParts) nparts = kMaxParts;
         QBP_TRACE_BEGIN(st);
-        if (vec) range_partial_kernel<4><<<nparts, kThreads, 0, st>>>(x, n, partials, keep_rev);
-        else     range_partial_kernel<1><<<nparts, kThreads, 0, st>>>(x, n, partials, keep_rev);
+        if (vec) launch(range_partial_kernel<4>, nparts, kThreads, 0, st, x, n, partials, keep_rev);
+        else     launch(range_partial_kernel<1>, nparts, kThreads, 0, st, x, n, partials, keep_rev);
         QBP_LAUNCH_OK("range_partial_kernel");
     }
     QBP_TRACE_BEGIN(st);
-    range_finalize_kernel<<<1, kThreads, 0, st>>>(partials, nparts, qp8, qp16);
+    launch(range_finalize_kernel, 1, kThreads, 0, st, partials, nparts, qp8, qp16);
     QBP_LAUNCH_OK("range_finalize_kernel");
     if (after_range) QBP_CUDA_OK(cudaEventRecord(after_range, st));
     return QBP_OK;
@@ -639,12 +650,12 @@ static int launch_chan_range(const float *x, int64_t rows, int64_t cols, int bit
         nparts = g.nbx;
         dim3 grid(g.nbx, g.slabs);
         QBP_TRACE_BEGIN(st);
-        if (g.vec == 4) chan_range_partial_kernel<4><<<grid, kScanThreads, 0, st>>>(x, rows, (int)cols, g.tw, part_lo, part_hi);
-        else            chan_range_partial_kernel<1><<<grid, kScanThreads, 0, st>>>(x, rows, (int)cols, g.tw, part_lo, part_hi);
+        if (g.vec == 4) launch(chan_range_partial_kernel<4>, grid, kScanThreads, 0, st, x, rows, (int)cols, g.tw, part_lo, part_hi);
+        else            launch(chan_range_partial_kernel<1>, grid, kScanThreads, 0, st, x, rows, (int)cols, g.tw, part_lo, part_hi);
         QBP_LAUNCH_OK("chan_range_partial_kernel");
     }
     QBP_TRACE_BEGIN(st);
-    chan_range_finalize_kernel<<<(int)((cols + 7) / 8), kThreads, 0, st>>>(part_lo, part_hi, nparts, (int)cols, bits, qp);
+    launch(chan_range_finalize_kernel, (int)((cols + 7) / 8), kThreads, 0, st, part_lo, part_hi, nparts, (int)cols, bits, qp);
     QBP_LAUNCH_OK("chan_range_finalize_kernel");
     return QBP_OK;
 }
@@ -675,7 +686,7 @@ static int launch_quantize(const float *x, int64_t n, int64_t cols, int perch, i
     do {                                                                                                                \
         const int grid = grid_for(blocks_per_sm(quantize_kernel<SR_, VEC_, PC_, TOT_>, kThreads), groups);              \
         QBP_TRACE_BEGIN(st);                                                                                            \
-        quantize_kernel<SR_, VEC_, PC_, TOT_><<<grid, kThreads, (VEC_) == 4 ? smem : 0, st>>>(x, n, c, qp8, id8, qp16, id16,  \
+        launch(quantize_kernel<SR_, VEC_, PC_, TOT_>, grid, kThreads, (VEC_) == 4 ? smem : 0, st, x, n, c, qp8, id8, qp16, id16,  \
                                                                                          key, o, (VEC_) == 4 ? smem_cols : 0, index_base); \
     } while (0)
 #define QBP_QUANT(SR_, VEC_, PC_) QBP_QUANT2(SR_, VEC_, PC_, false)
@@ -714,8 +725,8 @@ int launch_rowsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int
     const int grid = grid_for(is_signed ? blocks_per_sm(rowsum_kernel<true>, kThreads) : blocks_per_sm(rowsum_kernel<false>, kThreads),
                               (rows + groups - 1) / groups);
     QBP_TRACE_BEGIN(st);
-    if (is_signed) rowsum_kernel<true><<<grid, kThreads, 0, st>>>((const uint8_t *)q, rows, (int)cols, G, sums);
-    else           rowsum_kernel<false><<<grid, kThreads, 0, st>>>((const uint8_t *)q, rows, (int)cols, G, sums);
+    if (is_signed) launch(rowsum_kernel<true>, grid, kThreads, 0, st, (const uint8_t *)q, rows, (int)cols, G, sums);
+    else           launch(rowsum_kernel<false>, grid, kThreads, 0, st, (const uint8_t *)q, rows, (int)cols, G, sums);
     QBP_LAUNCH_OK("rowsum_kernel");
     return QBP_OK;
 }
@@ -733,8 +744,8 @@ int launch_colsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int
     int64_t grid = grid_for(blocks_per_sm(colsum_kernel<true>, kThreads), (rows + rpb - 1) / rpb) / slabs;
     if (grid < min_blocks) grid = min_blocks;
     QBP_TRACE_BEGIN(st);
-    if (is_signed) colsum_kernel<true><<<dim3((unsigned)grid, (unsigned)slabs), kThreads, 0, st>>>((const uint8_t *)q, rows, (int)cols, (unsigned long long *)sums);
-    else           colsum_kernel<false><<<dim3((unsigned)grid, (unsigned)slabs), kThreads, 0, st>>>((const uint8_t *)q, rows, (int)cols, (unsigned long long *)sums);
+    if (is_signed) launch(colsum_kernel<true>, dim3((unsigned)grid, (unsigned)slabs), kThreads, 0, st, (const uint8_t *)q, rows, (int)cols, (unsigned long long *)sums);
+    else           launch(colsum_kernel<false>, dim3((unsigned)grid, (unsigned)slabs), kThreads, 0, st, (const uint8_t *)q, rows, (int)cols, (unsigned long long *)sums);
     QBP_LAUNCH_OK("colsum_kernel");
     return QBP_OK;
 }
@@ -771,7 +782,7 @@ static int quantize_any(int bits, const float *x, int64_t rows, int64_t cols, in
     if (range_in) {
         const int count = perch ? (int)cols : 1;
         QBP_TRACE_BEGIN(st);
-        qparams_from_range_kernel<<<(count + 255) / 256, 256, 0, st>>>(range_in, count, bits, qp_out);
+        launch(qparams_from_range_kernel, (count + 255) / 256, 256, 0, st, range_in, count, bits, qp_out);
         QBP_LAUNCH_OK("qparams_from_range_kernel");
     } else {
         if (!ws || ws_bytes < quant_ws_bytes(cols, granularity))
@@ -845,7 +856,7 @@ int bifurcate_with_range_partials(const float *g, int64_t rows, int64_t cols, ui
                                   int64_t *tot16, bool lo_signed, cudaEvent_t after_range)
 {
     QBP_TRACE_BEGIN(st);
-    range_finalize_kernel<<<1, kThreads, 0, st>>>(partials, nparts, qp8, qp16);
+    launch(range_finalize_kernel, 1, kThreads, 0, st, partials, nparts, qp8, qp16);
     QBP_LAUNCH_OK("range_finalize_kernel");
     if (after_range) QBP_CUDA_OK(cudaEventRecord(after_range, st));
     return bifurcate_tail(g, rows, cols, seed, tensor_id8, tensor_id16, q8, qp8, row_sums8, hi, lo, qp16, st, 0, tot16, lo_signed);
@@ -856,7 +867,7 @@ int launch_range_finalize(const float2 *partials, int nparts, qbp_qparams *qp8, 
                           cudaEvent_t after_range)
 {
     QBP_TRACE_BEGIN(st);
-    range_finalize_kernel<<<1, kThreads, 0, st>>>(partials, nparts, qp8, qp16);
+    launch(range_finalize_kernel, 1, kThreads, 0, st, partials, nparts, qp8, qp16);
     QBP_LAUNCH_OK("range_finalize_kernel");
     if (after_range) QBP_CUDA_OK(cudaEventRecord(after_range, st));
     return QBP_OK;
@@ -944,11 +955,11 @@ extern "C" __attribute__((visibility("default"))) int qbp_range_chunked(const fl
     int bpc = (int)std::max<int64_t>(1, std::min<int64_t>((n_chunk + per_block - 1) / per_block, wave / chunks));
     bpc = (int)std::min<int64_t>(bpc, kMaxParts / chunks);
     QBP_TRACE_BEGIN(st);
-    if (vec) chunk_range_partial_kernel<4><<<dim3(bpc, (unsigned)chunks), kThreads, 0, st>>>(x, n_chunk, parts);
-    else     chunk_range_partial_kernel<1><<<dim3(bpc, (unsigned)chunks), kThreads, 0, st>>>(x, n_chunk, parts);
+    if (vec) launch(chunk_range_partial_kernel<4>, dim3(bpc, (unsigned)chunks), kThreads, 0, st, x, n_chunk, parts);
+    else     launch(chunk_range_partial_kernel<1>, dim3(bpc, (unsigned)chunks), kThreads, 0, st, x, n_chunk, parts);
     QBP_LAUNCH_OK("chunk_range_partial_kernel");
     QBP_TRACE_BEGIN(st);
-    chunk_range_finalize_kernel<<<1, kThreads, 0, st>>>(parts, (int)chunks, bpc, per_chunk, range_out);
+    launch(chunk_range_finalize_kernel, 1, kThreads, 0, st, parts, (int)chunks, bpc, per_chunk, range_out);
     QBP_LAUNCH_OK("chunk_range_finalize_kernel");
     return QBP_OK;
 }
@@ -1011,6 +1022,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_bifurcate(const float 
 __global__ void qparams_pair_from_range_kernel(const qbp_qparams *__restrict__ in, qbp_qparams *__restrict__ qp8,
                                                qbp_qparams *__restrict__ qp16)
 {
+    pdl_enter();
     *qp8 = make_qparams(in->vmin, in->vmax, 8);
     *qp16 = make_qparams(in->vmin, in->vmax, 16);
 }
@@ -1027,7 +1039,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_bifurcate_shard(const 
     if (((uintptr_t)g & 3) != 0) return fail(QBP_ERR_INVALID_ARG, "bifurcate_shard: g is not 4-byte aligned");
     if (index_base % 4) return fail(QBP_ERR_INVALID_ARG, "bifurcate_shard: index_base must be a multiple of 4");
     QBP_TRACE_BEGIN(st);
-    qparams_pair_from_range_kernel<<<1, 1, 0, st>>>(range_in, qp8, qp16);
+    launch(qparams_pair_from_range_kernel, 1, 1, 0, st, range_in, qp8, qp16);
     QBP_LAUNCH_OK("qparams_pair_from_range_kernel");
     return bifurcate_tail(g, rows, cols, seed, tensor_id8, tensor_id16, q8, qp8, row_sums8, hi, lo, qp16, st, index_base);
 }
@@ -1037,6 +1049,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_bifurcate_shard(const 
 __global__ void dequant_s64_kernel(const long long *__restrict__ acc, int64_t n, const qbp_qparams *qa,
                                    const qbp_qparams *qb, float *__restrict__ out)
 {
+    pdl_enter();
     const float s = __fmul_rn(qa->scale, qb->scale);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         out[i] = __fmul_rn((float)acc[i], s);
@@ -1050,7 +1063,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_dequant_s64(const int6
     if (count == 0) return QBP_OK;
     const int grid = (int)std::min<int64_t>((count + 255) / 256, (int64_t)sm_count() * 8);
     QBP_TRACE_BEGIN(st);
-    dequant_s64_kernel<<<grid, 256, 0, st>>>((const long long *)acc, count, qa, qb, out);
+    launch(dequant_s64_kernel, grid, 256, 0, st, (const long long *)acc, count, qa, qb, out);
     QBP_LAUNCH_OK("dequant_s64_kernel");
     return QBP_OK;
 }
@@ -1061,6 +1074,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_dequant_s64(const int6
 __global__ void __launch_bounds__(256) sgd_update_kernel(float *__restrict__ w, const float *__restrict__ dw,
                                                          float *__restrict__ vbuf, int64_t n, float lr, float mu, float wd)
 {
+    pdl_enter();
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
         const float wi = w[i];
         float g = __fadd_rn(dw[i], __fmul_rn(wd, wi));
@@ -1077,7 +1091,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_sgd_update(float *w, c
     if (count == 0) return QBP_OK;
     const int grid = (int)std::min<int64_t>((count + 255) / 256, (int64_t)sm_count() * 8);
     QBP_TRACE_BEGIN(st);
-    sgd_update_kernel<<<grid, 256, 0, st>>>(w, dw, momentum_buf, count, lr, momentum, weight_decay);
+    launch(sgd_update_kernel, grid, 256, 0, st, w, dw, momentum_buf, count, lr, momentum, weight_decay);
     QBP_LAUNCH_OK("sgd_update_kernel");
     return QBP_OK;
 }

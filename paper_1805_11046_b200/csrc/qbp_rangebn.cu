@@ -21,6 +21,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_stats_kernel(const float *__r
                                                                 float *__restrict__ part_lo, float *__restrict__ part_hi,
                                                                 double *__restrict__ part_sum)
 {
+    pdl_enter();
     const ScanPos p = scan_pos<VEC>(C, tw);
     const int rpb = kScanThreads / tw;
     float lo[VEC], hi[VEC];
@@ -81,6 +82,7 @@ __global__ void __launch_bounds__(128) bn_stats_finalize_kernel(const float *__r
                                                                 float *__restrict__ vmin, float *__restrict__ vmax,
                                                                 double *__restrict__ sum_out)
 {
+    pdl_enter();
     const int c = blockIdx.x;
     float lo = INFINITY, hi = -INFINITY;
     double sum = 0.0;
@@ -109,6 +111,7 @@ __global__ void bn_mean_from_sum_kernel(const double *__restrict__ col_sum, cons
                                         const float *__restrict__ col_max, int C, int64_t n, float *__restrict__ mean,
                                         float *__restrict__ vmin, float *__restrict__ vmax)
 {
+    pdl_enter();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= C) return;
     mean[c] = (float)(col_sum[c] / (double)n);
@@ -132,6 +135,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_apply_kernel(const float *__r
                                                                 const float *__restrict__ beta, float Cn,
                                                                 float *__restrict__ y, BnRequant R, int reverse)
 {
+    pdl_enter();
     const ScanPos p = scan_pos<VEC>(C, tw);
     // (with row sums the idle threads of a ragged last slab take part in the shuffles: tw <= 32 then, one slab)
     if (!p.active && !(REQUANT && (R.rowsum || R.chansum))) return;
@@ -230,6 +234,7 @@ __global__ void __launch_bounds__(256) bn_out_range_kernel(const float *__restri
                                                            qbp_qparams *__restrict__ out, qbp_qparams *__restrict__ qp8_out,
                                                            float4 *__restrict__ fold)
 {
+    pdl_enter();
     float lo = INFINITY, hi = -INFINITY;
     for (int c = threadIdx.x; c < C; c += 256) {
         float s = bn_scale(vmin[c], vmax[c], Cn);
@@ -268,6 +273,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_stats_kernel(const float 
                                                                     double *__restrict__ part_dyx,
                                                                     float *__restrict__ ext)
 {
+    pdl_enter();
     const ScanPos p = scan_pos<VEC>(C, tw);
     const int rpb = kScanThreads / tw;
     double sdy[VEC], sdyx[VEC];
@@ -392,6 +398,7 @@ __global__ void __launch_bounds__(128) bn_bwd_finalize_kernel(const double *__re
                                                               const float *__restrict__ beta = nullptr,
                                                               float2 *__restrict__ relu_thr = nullptr)
 {
+    pdl_enter();
     const int c = blockIdx.x;
     double a = 0.0, b = 0.0;
     for (int i = threadIdx.x; i < nparts; i += 128) {
@@ -483,6 +490,7 @@ __global__ void __launch_bounds__(kScanThreads, 3) bn_bwd_apply_bifurcate_kernel
     uint32_t lo_flip, int32_t *__restrict__ rowsum8, unsigned long long *__restrict__ chansum16,
     const float2 *__restrict__ relu_thr)
 {
+    pdl_enter();
     const bool rowsum_pieces = tw > 32 || gridDim.y > 1;
     const ScanPos p = scan_pos<4>(C, tw);
     uint32_t cs16[4] = {0u, 0u, 0u, 0u};          // unsigned codes of this thread's rows (fewer than 65536 rows)
@@ -604,6 +612,7 @@ __global__ void bn_bwd_coef_kernel(const double *__restrict__ sum_dy, const doub
                                    const float *__restrict__ gamma, double Cn, float *__restrict__ dgamma,
                                    float *__restrict__ dbeta, float2 *__restrict__ coef)
 {
+    pdl_enter();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= C) return;
     const double a = sum_dy[c], b = sum_dyx[c];
@@ -627,6 +636,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_apply_kernel(const float 
                                                                     float *__restrict__ dx,
                                                                     float2 *__restrict__ range_parts)
 {
+    pdl_enter();
     const ScanPos p = scan_pos<VEC>(C, tw);
     float rlo = INFINITY, rhi = -INFINITY;
     if (p.active) {
@@ -742,7 +752,7 @@ static int bn_fwd_apply_launch(const float *x, int64_t n_rows, int64_t n_stat, i
     const float Cn = (float)(1.0 / std::sqrt(2.0 * std::log((double)n_stat)));
     if (out_range || requant) {
         QBP_TRACE_BEGIN(st);
-        bn_out_range_kernel<<<1, 256, 0, st>>>(save_mean, save_min, save_max, gamma, beta, (int)C, Cn, relu, out_range,
+        launch(bn_out_range_kernel, 1, 256, 0, st, save_mean, save_min, save_max, gamma, beta, (int)C, Cn, relu, out_range,
                                                requant ? rq->qp : nullptr, nullptr);
         QBP_LAUNCH_OK("bn_out_range_kernel");
     }
@@ -760,7 +770,7 @@ static int bn_fwd_apply_launch(const float *x, int64_t n_rows, int64_t n_stat, i
         }
     }
     QBP_TRACE_BEGIN(st);
-#define QBP_BN_APPLY(V, RL, RQ) bn_apply_kernel<V, RL, RQ><<<grid_apply, kScanThreads, 0, st>>>(x, n_rows, (int)C, ga.tw, save_mean, save_min, save_max, gamma, beta, Cn, y, R, reverse ? 1 : 0)
+#define QBP_BN_APPLY(V, RL, RQ) launch(bn_apply_kernel<V, RL, RQ>, grid_apply, kScanThreads, 0, st, x, n_rows, (int)C, ga.tw, save_mean, save_min, save_max, gamma, beta, Cn, y, R, reverse ? 1 : 0)
     if (ga.vec == 4) {
         if (requant) { if (relu) QBP_BN_APPLY(4, true, true); else QBP_BN_APPLY(4, false, true); }
         else         { if (relu) QBP_BN_APPLY(4, true, false); else QBP_BN_APPLY(4, false, false); }
@@ -789,11 +799,11 @@ static int bn_fwd_stats_launch(const float *x, int64_t n, int64_t C, float *mean
                                               : blocks_per_sm(bn_stats_kernel<1>, kScanThreads));
     const dim3 grid(g.nbx, g.slabs);
     QBP_TRACE_BEGIN(st);
-    if (g.vec == 4) bn_stats_kernel<4><<<grid, kScanThreads, 0, st>>>(x, n, (int)C, g.tw, plo, phi, psum);
-    else            bn_stats_kernel<1><<<grid, kScanThreads, 0, st>>>(x, n, (int)C, g.tw, plo, phi, psum);
+    if (g.vec == 4) launch(bn_stats_kernel<4>, grid, kScanThreads, 0, st, x, n, (int)C, g.tw, plo, phi, psum);
+    else            launch(bn_stats_kernel<1>, grid, kScanThreads, 0, st, x, n, (int)C, g.tw, plo, phi, psum);
     QBP_LAUNCH_OK("bn_stats_kernel");
     QBP_TRACE_BEGIN(st);
-    bn_stats_finalize_kernel<<<(int)C, 128, 0, st>>>(plo, phi, psum, g.nbx, (int)C, n, mean, vmin, vmax, sum_out);
+    launch(bn_stats_finalize_kernel, (int)C, 128, 0, st, plo, phi, psum, g.nbx, (int)C, n, mean, vmin, vmax, sum_out);
     QBP_LAUNCH_OK("bn_stats_finalize_kernel");
     return QBP_OK;
 }
@@ -843,7 +853,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_rangebn_fwd_apply(cons
     if (!x || !col_sum || !col_min || !col_max || !save_mean || !save_min || !save_max)
         return fail(QBP_ERR_INVALID_ARG, "rangebn_fwd_apply: NULL argument");
     QBP_TRACE_BEGIN(st);
-    bn_mean_from_sum_kernel<<<(int)((C + 255) / 256), 256, 0, st>>>(col_sum, col_min, col_max, (int)C, n_stat, save_mean, save_min, save_max);
+    launch(bn_mean_from_sum_kernel, (int)((C + 255) / 256), 256, 0, st, col_sum, col_min, col_max, (int)C, n_stat, save_mean, save_min, save_max);
     QBP_LAUNCH_OK("bn_mean_from_sum_kernel");
     return bn_fwd_apply_launch(x, n_rows, n_stat, C, gamma, beta, relu, y, save_mean, save_min, save_max, out_range, rq, st);
 }
@@ -860,10 +870,10 @@ int qbp::rangebn_fold_from_parts(int64_t n, int64_t C, const float *gamma, const
     if (n < 2 || C <= 0) return fail(QBP_ERR_INVALID_ARG, "rangebn: needs n >= 2 rows");
     const float Cn = (float)(1.0 / std::sqrt(2.0 * std::log((double)n)));
     QBP_TRACE_BEGIN(st);
-    bn_stats_finalize_kernel<<<(int)C, 128, 0, st>>>(parts.lo, parts.hi, parts.sum, parts.rows, (int)C, n, save_mean, save_min, save_max, nullptr);
+    launch(bn_stats_finalize_kernel, (int)C, 128, 0, st, parts.lo, parts.hi, parts.sum, parts.rows, (int)C, n, save_mean, save_min, save_max, nullptr);
     QBP_LAUNCH_OK("bn_stats_finalize_kernel");
     QBP_TRACE_BEGIN(st);
-    bn_out_range_kernel<<<1, 256, 0, st>>>(save_mean, save_min, save_max, gamma, beta, (int)C, Cn, relu, nullptr, qp8_out, fold);
+    launch(bn_out_range_kernel, 1, 256, 0, st, save_mean, save_min, save_max, gamma, beta, (int)C, Cn, relu, nullptr, qp8_out, fold);
     QBP_LAUNCH_OK("bn_out_range_kernel");
     return QBP_OK;
 }
@@ -878,7 +888,7 @@ int qbp::rangebn_fwd_from_parts(const float *x, int64_t n, int64_t C, const floa
         return fail(QBP_ERR_INVALID_ARG, "rangebn_fwd: NULL tensor");
     if (n < 2 || C <= 0) return fail(QBP_ERR_INVALID_ARG, "rangebn_fwd: needs n >= 2 rows");
     QBP_TRACE_BEGIN(st);
-    bn_stats_finalize_kernel<<<(int)C, 128, 0, st>>>(parts.lo, parts.hi, parts.sum, parts.rows, (int)C, n, save_mean, save_min, save_max, nullptr);
+    launch(bn_stats_finalize_kernel, (int)C, 128, 0, st, parts.lo, parts.hi, parts.sum, parts.rows, (int)C, n, save_mean, save_min, save_max, nullptr);
     QBP_LAUNCH_OK("bn_stats_finalize_kernel");
     // (the product that left the statistics has just written x: its tail is in the L2)
     return bn_fwd_apply_launch(x, n, n, C, gamma, beta, relu, y, save_mean, save_min, save_max, out_range, rq, st, true);
@@ -911,7 +921,7 @@ static int bn_bwd_stats_launch(const float *dy, const float *x, int64_t n_rows, 
     const double Cnd = 1.0 / std::sqrt(2.0 * std::log((double)n_stat));
     const float Cn = (float)Cnd;
     QBP_TRACE_BEGIN(st);
-#define QBP_BN_BSTATS(V, R, E) bn_bwd_stats_kernel<V, R, E><<<grid, kScanThreads, 0, st>>>(dy, x, n_rows, (int)C, g.tw, save_mean, save_min, save_max, gamma, beta, Cn, pa, pb, ext)
+#define QBP_BN_BSTATS(V, R, E) launch(bn_bwd_stats_kernel<V, R, E>, grid, kScanThreads, 0, st, dy, x, n_rows, (int)C, g.tw, save_mean, save_min, save_max, gamma, beta, Cn, pa, pb, ext)
     if (ext) {
         if (g.vec != 4) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "rangebn_bwd: the pass with dy extremes needs aligned tensors and C a multiple of 4");
         if (relu) QBP_BN_BSTATS(4, true, true); else QBP_BN_BSTATS(4, false, true);
@@ -920,7 +930,7 @@ static int bn_bwd_stats_launch(const float *dy, const float *x, int64_t n_rows, 
 #undef QBP_BN_BSTATS
     QBP_LAUNCH_OK("bn_bwd_stats_kernel");
     QBP_TRACE_BEGIN(st);
-    bn_bwd_finalize_kernel<<<(int)C, 128, 0, st>>>(pa, pb, g.nbx, (int)C, n_stat, gamma, Cnd, dgamma, dbeta, coef, sum_dy, sum_dyx,
+    launch(bn_bwd_finalize_kernel, (int)C, 128, 0, st, pa, pb, g.nbx, (int)C, n_stat, gamma, Cnd, dgamma, dbeta, coef, sum_dy, sum_dyx,
                                                    ext, save_min, save_max, Cn, chan_range, save_mean, beta, relu_thr);
     QBP_LAUNCH_OK("bn_bwd_finalize_kernel");
     return QBP_OK;
@@ -939,7 +949,7 @@ static int bn_bwd_apply_launch(const float *dy, const float *x, int64_t n_rows, 
     const dim3 grid_apply(ga.nbx, ga.slabs);
     const float Cn = (float)(1.0 / std::sqrt(2.0 * std::log((double)n_stat)));
     QBP_TRACE_BEGIN(st);
-#define QBP_BN_BAPPLY(V, R, G) bn_bwd_apply_kernel<V, R, G><<<grid_apply, kScanThreads, 0, st>>>(dy, x, n_rows, (int)C, ga.tw, save_mean, save_min, save_max, gamma, beta, Cn, coef, dx, range_parts)
+#define QBP_BN_BAPPLY(V, R, G) launch(bn_bwd_apply_kernel<V, R, G>, grid_apply, kScanThreads, 0, st, dy, x, n_rows, (int)C, ga.tw, save_mean, save_min, save_max, gamma, beta, Cn, coef, dx, range_parts)
     if (range_parts) {
         if (ga.vec == 4) { if (relu) QBP_BN_BAPPLY(4, true, true); else QBP_BN_BAPPLY(4, false, true); }
         else             { if (relu) QBP_BN_BAPPLY(1, true, true); else QBP_BN_BAPPLY(1, false, true); }
@@ -1000,7 +1010,7 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
     int32_t *row_sums_arg = row_sums8;
     if (row_sums8 && (ga.tw > 32 || ga.slabs > 1)) QBP_CUDA_OK(cudaMemsetAsync(row_sums8, 0, sizeof(int32_t) * (size_t)n, st));
     QBP_TRACE_BEGIN(st);
-#define QBP_BN_BAB(R, G, T) do { static PerDeviceOnce once_; QBP_SMEM_OPT_IN(once_, (bn_bwd_apply_bifurcate_kernel<R, G, T>), kBabRingBytes); bn_bwd_apply_bifurcate_kernel<R, G, T><<<grid, kScanThreads, kBabRingBytes, st>>>(dy, x, n, (int)C, ga.tw, save_mean, save_min, save_max, gamma, beta, Cn, coef, g_out, qp8, qp16, id8, id16, keys, reinterpret_cast<uint32_t *>(q8), reinterpret_cast<uint32_t *>(hi), reinterpret_cast<uint32_t *>(lo), flip, row_sums_arg, reinterpret_cast<unsigned long long *>(tot16), relu_thr); } while (0)
+#define QBP_BN_BAB(R, G, T) do { static PerDeviceOnce once_; QBP_SMEM_OPT_IN(once_, (bn_bwd_apply_bifurcate_kernel<R, G, T>), kBabRingBytes); launch(bn_bwd_apply_bifurcate_kernel<R, G, T>, grid, kScanThreads, kBabRingBytes, st, dy, x, n, (int)C, ga.tw, save_mean, save_min, save_max, gamma, beta, Cn, coef, g_out, qp8, qp16, id8, id16, keys, reinterpret_cast<uint32_t *>(q8), reinterpret_cast<uint32_t *>(hi), reinterpret_cast<uint32_t *>(lo), flip, row_sums_arg, reinterpret_cast<unsigned long long *>(tot16), relu_thr); } while (0)
 #define QBP_BN_BAB2(R, G) do { if (tot16) QBP_BN_BAB(R, G, true); else QBP_BN_BAB(R, G, false); } while (0)
     if (g_out) { if (relu) QBP_BN_BAB2(true, true); else QBP_BN_BAB2(false, true); }
     else       { if (relu) QBP_BN_BAB2(true, false); else QBP_BN_BAB2(false, false); }
@@ -1073,7 +1083,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_rangebn_bwd_apply(cons
     float2 *coef = w.take<float2>((size_t)C);
     const double Cnd = 1.0 / std::sqrt(2.0 * std::log((double)n_stat));
     QBP_TRACE_BEGIN(st);
-    bn_bwd_coef_kernel<<<(int)((C + 255) / 256), 256, 0, st>>>(sum_dy, sum_dyxhat, (int)C, n_stat, gamma, Cnd, dgamma, dbeta, coef);
+    launch(bn_bwd_coef_kernel, (int)((C + 255) / 256), 256, 0, st, sum_dy, sum_dyxhat, (int)C, n_stat, gamma, Cnd, dgamma, dbeta, coef);
     QBP_LAUNCH_OK("bn_bwd_coef_kernel");
     return bn_bwd_apply_launch(dy, x, n_rows, n_stat, C, gamma, beta, relu, save_mean, save_min, save_max, coef, dx, nullptr, nullptr, st);
 }

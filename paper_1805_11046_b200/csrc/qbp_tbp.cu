@@ -21,6 +21,7 @@ template <int VEC>
 __global__ void __launch_bounds__(kTbpThreads) binarize_kernel(const float *__restrict__ x, int64_t n, int8_t *__restrict__ q,
                                                                qbp_qparams *__restrict__ qp_out)
 {
+    pdl_enter();
     if (qp_out && blockIdx.x == 0 && threadIdx.x == 0) {
         qbp_qparams r; r.scale = 1.0f; r.zero_point = 0; r.vmin = -1.0f; r.vmax = 1.0f;
         *qp_out = r;
@@ -60,6 +61,7 @@ __global__ void __launch_bounds__(kTbpThreads) stc_ternarize_kernel(const float 
                                                                     int8_t *__restrict__ q, int8_t *__restrict__ hi,
                                                                     uint8_t *__restrict__ lo, qbp_qparams *__restrict__ qp_out)
 {
+    pdl_enter();
     const float s = fmaxf(-rng->vmin, rng->vmax);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         qbp_qparams r;
@@ -129,8 +131,8 @@ static int stc_ternarize_impl(const float *g, int64_t n, int samples, uint64_t s
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((items + kTbpThreads - 1) / kTbpThreads, (int64_t)sm_count() * 8));
     const PhiloxKeys keys = philox_keys_host(seed);
     QBP_TRACE_BEGIN(st);
-    if (vec) stc_ternarize_kernel<4><<<grid, kTbpThreads, 0, st>>>(g, n, rng, samples, tensor_id, keys, q, hi, lo, qp_out);
-    else     stc_ternarize_kernel<1><<<grid, kTbpThreads, 0, st>>>(g, n, rng, samples, tensor_id, keys, q, hi, lo, qp_out);
+    if (vec) launch(stc_ternarize_kernel<4>, grid, kTbpThreads, 0, st, g, n, rng, samples, tensor_id, keys, q, hi, lo, qp_out);
+    else     launch(stc_ternarize_kernel<1>, grid, kTbpThreads, 0, st, g, n, rng, samples, tensor_id, keys, q, hi, lo, qp_out);
     QBP_LAUNCH_OK("stc_ternarize_kernel");
     return QBP_OK;
 }
@@ -141,6 +143,7 @@ static int stc_ternarize_impl(const float *g, int64_t n, int samples, uint64_t s
 __global__ void __launch_bounds__(256) pack_bits_kernel(const int8_t *__restrict__ codes, int64_t rows, int64_t cols, int mask,
                                                         uint32_t *__restrict__ words)
 {
+    pdl_enter();
     const int64_t wpr = (cols + 31) / 32;
     const int lane = threadIdx.x & 31;
     for (int64_t word = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); word < rows * wpr; word += (int64_t)gridDim.x * 8) {
@@ -163,6 +166,7 @@ __global__ void __launch_bounds__(256) xnor_gemm_bits_kernel(int M, int N, int K
                                                              const uint32_t *__restrict__ S, const uint32_t *__restrict__ B,
                                                              int32_t *__restrict__ C)
 {
+    pdl_enter();
     __shared__ uint32_t sA[64][33], sB[64][33], sS[GATED ? 64 : 1][33];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
@@ -216,8 +220,8 @@ static int xnor_bits_launch(bool gated, int64_t M, int64_t N, int64_t K, const u
     const dim3 grid((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64));
     const int wpr = (int)((K + 31) / 32);
     QBP_TRACE_BEGIN(st);
-    if (gated) xnor_gemm_bits_kernel<true><<<grid, 256, 0, st>>>((int)M, (int)N, (int)K, wpr, A, S, B, C);
-    else       xnor_gemm_bits_kernel<false><<<grid, 256, 0, st>>>((int)M, (int)N, (int)K, wpr, A, nullptr, B, C);
+    if (gated) launch(xnor_gemm_bits_kernel<true>, grid, 256, 0, st, (int)M, (int)N, (int)K, wpr, A, S, B, C);
+    else       launch(xnor_gemm_bits_kernel<false>, grid, 256, 0, st, (int)M, (int)N, (int)K, wpr, A, nullptr, B, C);
     QBP_LAUNCH_OK("xnor_gemm_bits_kernel");
     return QBP_OK;
 }
@@ -235,7 +239,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_pack_bits(const int8_t
     const int64_t total = rows * ((cols + 31) / 32);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((total + 7) / 8, (int64_t)sm_count() * 16));
     QBP_TRACE_BEGIN(st);
-    pack_bits_kernel<<<grid, 256, 0, st>>>(codes, rows, cols, mask, words);
+    launch(pack_bits_kernel, grid, 256, 0, st, codes, rows, cols, mask, words);
     QBP_LAUNCH_OK("pack_bits_kernel");
     return QBP_OK;
 }
@@ -262,8 +266,8 @@ extern "C" __attribute__((visibility("default"))) int qbp_binarize_s8(const floa
     const int64_t items = vec ? (n + 3) / 4 : n;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((items + kTbpThreads - 1) / kTbpThreads, (int64_t)sm_count() * 8));
     QBP_TRACE_BEGIN(st);
-    if (vec) binarize_kernel<4><<<grid, kTbpThreads, 0, st>>>(x, n, q, qp_out);
-    else     binarize_kernel<1><<<grid, kTbpThreads, 0, st>>>(x, n, q, qp_out);
+    if (vec) launch(binarize_kernel<4>, grid, kTbpThreads, 0, st, x, n, q, qp_out);
+    else     launch(binarize_kernel<1>, grid, kTbpThreads, 0, st, x, n, q, qp_out);
     QBP_LAUNCH_OK("binarize_kernel");
     return QBP_OK;
 }

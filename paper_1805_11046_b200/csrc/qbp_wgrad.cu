@@ -446,6 +446,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_trigger();                       // (tensor memory is allocated)
+    pdl_wait();
     const uint32_t tmem_base = tmem_slot;
     bool timed_out = false;
 
@@ -633,6 +635,7 @@ template <bool IS_SIGNED>
 __global__ void __launch_bounds__(256) class_sums_kernel(const uint8_t *__restrict__ q, int pixels, int H, int W,
                                                          int C, unsigned long long *__restrict__ sums)
 {
+    pdl_enter();
     extern __shared__ int s_acc[];                       // [16][C]
     for (int i = threadIdx.x; i < 16 * C; i += 256) s_acc[i] = 0;
     __syncthreads();
@@ -783,6 +786,7 @@ template <bool IS_SIGNED>
 __global__ void __launch_bounds__(256, 3) row_class_sums_kernel(const uint8_t *__restrict__ q, int Nimg, int H, int W,
                                                                 int C, int gs, unsigned long long *__restrict__ sums)
 {
+    pdl_enter();
     row_class_sums_body<IS_SIGNED>(q, Nimg, H, W, C, gs, sums);
 }
 
@@ -792,6 +796,7 @@ __global__ void __launch_bounds__(256, 3) row_class_sums3_kernel(const uint8_t *
                                                                  const uint8_t *__restrict__ lo, int Nimg, int H, int W, int C,
                                                                  int gs, unsigned long long *__restrict__ sums, int lo_signed)
 {
+    pdl_enter();
     if (blockIdx.z == 0)      row_class_sums_body<true>(x, Nimg, H, W, C, gs, sums);
     else if (blockIdx.z == 1) row_class_sums_body<true>(hi, Nimg, H, W, C, gs, sums + 16 * C);
     else if (lo_signed)       row_class_sums_body<true>(lo, Nimg, H, W, C, gs, sums + 32 * C);
@@ -810,6 +815,7 @@ __global__ void __launch_bounds__(256) border_class_sums_kernel(const uint8_t *_
                                                                 unsigned long long *__restrict__ sums_hi,
                                                                 unsigned long long *__restrict__ sums_lo, int lo_signed)
 {
+    pdl_enter();
     extern __shared__ int s_acc[];                       // [16][C]
     const uint8_t *q = blockIdx.z == 0 ? x : blockIdx.z == 1 ? hi : lo;
     unsigned long long *sums = blockIdx.z == 0 ? sums_x : blockIdx.z == 1 ? sums_hi : sums_lo;
@@ -891,6 +897,7 @@ __global__ void wgrad_terms_kernel(const long long *__restrict__ sx, const long 
                                    const qbp_qparams *qx, const qbp_qparams *qg, long long *__restrict__ rowterm,
                                    long long *__restrict__ colterm, int zg_shift)
 {
+    pdl_enter();
     const long long zx = qx->zero_point, zg = qg->zero_point - zg_shift;      // (signed low bytes: lo - 128 against zg - 128)
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < K) rowterm[i] = -zg * sx[i] + M * zx * zg;
@@ -905,6 +912,7 @@ __global__ void __launch_bounds__(256) wgrad_finalize_kernel(const WgradParams P
                                                              const long long *__restrict__ shi,
                                                              const long long *__restrict__ slo, int64_t total)
 {
+    pdl_enter();
     constexpr int kLanes = kWgFinalizeLanes;
     const int64_t e_raw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kLanes;
     const int part_lane = threadIdx.x % kLanes;
@@ -975,6 +983,7 @@ __global__ void __launch_bounds__(256) wgrad_conv_finalize_kernel(const WgradPar
                                                                   const long long *__restrict__ shi,
                                                                   const long long *__restrict__ slo)
 {
+    pdl_enter();
     constexpr int U = 8 / NB;                              // slices in flight per output channel
     __shared__ long long s_part[NB][4][64], s_sx[4][64], s_sg[4][NB];
     const int cblocks = (P.C + 63) / 64;
@@ -1242,8 +1251,7 @@ static int launch_class_sums(const void *q, int64_t pixels, int H, int W, int C,
         int64_t grid_x = std::min<int64_t>(rows, std::max<int64_t>(1, (int64_t)sm_count() * 3 / slabs));
         grid_x = std::max<int64_t>(grid_x, rows / (1 << 22) + 1);
         QBP_TRACE_BEGIN(st);
-        row_class_sums_kernel<IS_SIGNED><<<dim3((unsigned)grid_x, (unsigned)slabs), 256, (size_t)12 * gs * 16 * sizeof(int), st>>>(
-            (const uint8_t *)q, Nimg, H, W, C, gs, (unsigned long long *)sums);
+        launch(row_class_sums_kernel<IS_SIGNED>, dim3((unsigned)grid_x, (unsigned)slabs), 256, (size_t)12 * gs * 16 * sizeof(int), st, (const uint8_t *)q, Nimg, H, W, C, gs, (unsigned long long *)sums);
         QBP_LAUNCH_OK("class_sums_kernel");
         return QBP_OK;
     }
@@ -1254,7 +1262,7 @@ static int launch_class_sums(const void *q, int64_t pixels, int H, int W, int C,
     int64_t grid = std::min<int64_t>((pixels + 8 * rpb - 1) / (8 * rpb), (int64_t)sm_count() * bps);
     grid = std::max<int64_t>(grid, pixels / (1 << 22) + 1);
     QBP_TRACE_BEGIN(st);
-    class_sums_kernel<IS_SIGNED><<<(unsigned)grid, 256, smem, st>>>((const uint8_t *)q, (int)pixels, H, W, C, (unsigned long long *)sums);
+    launch(class_sums_kernel<IS_SIGNED>, (unsigned)grid, 256, smem, st, (const uint8_t *)q, (int)pixels, H, W, C, (unsigned long long *)sums);
     QBP_LAUNCH_OK("class_sums_kernel");
     return QBP_OK;
 }
@@ -1338,8 +1346,7 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
             QBP_SMEM_OPT_IN(configured, border_class_sums_kernel, 96 * 1024);
             const int gx = (int)std::min<int64_t>((d->N + 3) / 4, 128);      // one group of four images per block when possible
             QBP_TRACE_BEGIN(st);
-            border_class_sums_kernel<<<dim3((unsigned)gx, 1, 3), 256, (size_t)std::max(K, N) * 16 * sizeof(int), st>>>(
-                (const uint8_t *)x, (const uint8_t *)g_hi, g_lo, d->N, d->H, d->W, (int)K, (int)N, (unsigned long long *)sx,
+            launch(border_class_sums_kernel, dim3((unsigned)gx, 1, 3), 256, (size_t)std::max(K, N) * 16 * sizeof(int), st, (const uint8_t *)x, (const uint8_t *)g_hi, g_lo, d->N, d->H, d->W, (int)K, (int)N, (unsigned long long *)sx,
                 (unsigned long long *)shi, (unsigned long long *)slo, lo_signed ? 1 : 0);
             QBP_LAUNCH_OK("border_class_sums_kernel");
         }
@@ -1361,8 +1368,7 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
         int64_t grid_x = std::min<int64_t>(rows, std::max<int64_t>(1, (int64_t)sm_count() / slabs));
         grid_x = std::max<int64_t>(grid_x, rows / (1 << 22) + 1);
         QBP_TRACE_BEGIN(st);
-        row_class_sums3_kernel<<<dim3((unsigned)grid_x, (unsigned)slabs, 3), 256, (size_t)12 * gs * 16 * sizeof(int), st>>>(
-            (const uint8_t *)x, (const uint8_t *)g_hi, (const uint8_t *)g_lo, (int)(rows / d->H), d->H, d->W, (int)K, gs,
+        launch(row_class_sums3_kernel, dim3((unsigned)grid_x, (unsigned)slabs, 3), 256, (size_t)12 * gs * 16 * sizeof(int), st, (const uint8_t *)x, (const uint8_t *)g_hi, (const uint8_t *)g_lo, (int)(rows / d->H), d->H, d->W, (int)K, gs,
             (unsigned long long *)sx, lo_signed ? 1 : 0);
         QBP_LAUNCH_OK("class_sums_kernel");
     } else if (d) {
@@ -1377,7 +1383,7 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
         if (P.direct || pair_kernel) {
             const int64_t mx = std::max(K, N);
             QBP_TRACE_BEGIN(st);
-            wgrad_terms_kernel<<<(unsigned)((mx + 255) / 256), 256, 0, st>>>((const long long *)sx, (const long long *)shi,
+            launch(wgrad_terms_kernel, (unsigned)((mx + 255) / 256), 256, 0, st, (const long long *)sx, (const long long *)shi,
                                                                             (const long long *)slo, M, N, K, qx, qg16,
                                                                             (long long *)rowterm, (long long *)colterm, lo_signed ? 128 : 0);
             QBP_LAUNCH_OK("wgrad_terms_kernel");
@@ -1419,7 +1425,7 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
     static PerDeviceOnce configured[9];
     QBP_SMEM_OPT_IN(configured[layout_id], kernel, kWgSmem);
     QBP_TRACE_BEGIN(st);
-    kernel<<<pl.grid, kWgThreads, pl.smem, st>>>(P);
+    launch(kernel, pl.grid, kWgThreads, pl.smem, st, P);
     QBP_LAUNCH_OK("qbp_wgrad_kernel");
     if (d) {
         // output channels per block: as many as still leave four blocks per SM
@@ -1427,14 +1433,14 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
         const int nb = per_n * (d->K / 8) >= 4ll * sm_count() ? 8 : per_n * (d->K / 4) >= 4ll * sm_count() ? 4 : 2;
         const dim3 grid((unsigned)per_n, (unsigned)((d->K + nb - 1) / nb));
         QBP_TRACE_BEGIN(st);
-        if (nb == 8)      wgrad_conv_finalize_kernel<8><<<grid, 256, 0, st>>>(P, (const long long *)sx, (const long long *)shi, (const long long *)slo);
-        else if (nb == 4) wgrad_conv_finalize_kernel<4><<<grid, 256, 0, st>>>(P, (const long long *)sx, (const long long *)shi, (const long long *)slo);
-        else              wgrad_conv_finalize_kernel<2><<<grid, 256, 0, st>>>(P, (const long long *)sx, (const long long *)shi, (const long long *)slo);
+        if (nb == 8)      launch(wgrad_conv_finalize_kernel<8>, grid, 256, 0, st, P, (const long long *)sx, (const long long *)shi, (const long long *)slo);
+        else if (nb == 4) launch(wgrad_conv_finalize_kernel<4>, grid, 256, 0, st, P, (const long long *)sx, (const long long *)shi, (const long long *)slo);
+        else              launch(wgrad_conv_finalize_kernel<2>, grid, 256, 0, st, P, (const long long *)sx, (const long long *)shi, (const long long *)slo);
         QBP_LAUNCH_OK("wgrad_finalize_kernel");
     } else if (!P.direct) {
         const int blocks = (int)((outs * kWgFinalizeLanes + 255) / 256);
         QBP_TRACE_BEGIN(st);
-        wgrad_finalize_kernel<<<blocks, 256, 0, st>>>(P, (const long long *)sx, (const long long *)shi, (const long long *)slo, outs);
+        launch(wgrad_finalize_kernel, blocks, 256, 0, st, P, (const long long *)sx, (const long long *)shi, (const long long *)slo, outs);
         QBP_LAUNCH_OK("wgrad_finalize_kernel");
     }
     return QBP_OK;

@@ -151,6 +151,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
     __syncthreads();
     w2_cluster_sync();                   // both CTAs' barriers are initialised before either signals the other
     tc_fence_after();
+    pdl_trigger();                       // (tensor memory is allocated, in both CTAs)
+    pdl_wait();
     const uint32_t tmem_base = tmem_slot;
     bool timed_out = false;
 
@@ -334,7 +336,7 @@ int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qp
     static PerDeviceOnce configured;
     QBP_SMEM_OPT_IN(configured, qbp_wgrad2_kernel, kW2Smem);
     QBP_TRACE_BEGIN(st);
-    qbp_wgrad2_kernel<<<2 * P.pairs, kW2Threads, kW2Smem, st>>>(P);
+    launch(qbp_wgrad2_kernel, 2 * P.pairs, kW2Threads, kW2Smem, st, P);
     QBP_LAUNCH_OK("qbp_wgrad2_kernel");
     return QBP_OK;
 }
