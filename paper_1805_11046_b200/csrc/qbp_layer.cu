@@ -102,7 +102,7 @@ static size_t step_scratch_bytes(const qbp_layer_desc *L, const LayerShape &s)
         b = std::max(b, qbp_conv_s8_workspace_bytes(QBP_CONV_FPROP, &L->conv));
         b = std::max(b, qbp_wgrad_s16_workspace_bytes(&L->conv, 0, 0, 0));
     } else {
-        b = std::max(b, qbp_gemm_s8_workspace_bytes(s.rows, std::max(s.cin, s.cout), std::max(s.cin, s.cout)));
+        b = std::max({b, qbp_gemm_s8_workspace_bytes(s.rows, s.cout, s.cin), qbp_gemm_s8_workspace_bytes(s.rows, s.cin, s.cout)});
         b = std::max(b, qbp_wgrad_s16_workspace_bytes(nullptr, s.rows, s.cout, s.cin));
     }
     return align_up(b, 256);
@@ -225,7 +225,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_fwd_chained(cons
     int32_t *row_sums = reinterpret_cast<int32_t *>(static_cast<char *>(ws) + scratch);
     const int32_t *in_sums = s.conv ? row_sums : nullptr;
     // (a small filter's launch runs beside the pass that writes the input codes)
-    const bool small_filter = s.conv && filter_prep_supported(&L->conv, w, saved->w_codes);
+    const bool small_filter = s.conv && L->conv.R == 3 && filter_prep_supported(&L->conv, w, saved->w_codes);
     SideStream *sd = (x && small_filter) ? side_stream() : nullptr;
     if (x) {
         bool left = false;
@@ -319,7 +319,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_bwd(const qbp_la
     int64_t *tot_g = totals ? tot_g_buffer(L, s, ws) : nullptr;
     // (a small filter: the layer gradient's column terms in one launch, beside the bifurcation -- they need the
     // gradient's parameters only; else two kernels inside the product's call)
-    const bool small = s.conv && (int64_t)L->conv.R * L->conv.S * L->conv.C <= 12288 && s.w_elems <= 49152 && L->conv.C % 4 == 0;
+    const bool small = s.conv && L->conv.R == 3 && (int64_t)L->conv.R * L->conv.S * L->conv.C <= 12288 && s.w_elems <= 49152 && L->conv.C % 4 == 0;
     SideStream *sd = small ? side_stream() : nullptr;
     // Range BN backward and the two copies of its result.  Where the shape allows, in two passes over (dy, z): the
     // statistics pass also takes the extremes of dy, from which the exact range of the gradient follows (Section 4:

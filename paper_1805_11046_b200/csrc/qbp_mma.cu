@@ -211,8 +211,13 @@ struct MmaParams {
     // output
     int64_t M, N;                 // rows / columns of the output matrix
     int32_t *acc_out; float *out;
+    // zero-point correction: acc + rowterm[m] + colterm[class][n] (3 x 3 convolutions, precomputed), or, in the RAW
+    // instances (GEMM, 1 x 1 convolutions), from the code sums themselves:
+    //   rowterm = -zb * a_sums[m] + k_len * za * zb,  colterm = -za * b_sums[n]
     const int32_t *rowterm;       // [M]
     const int32_t *colterm;       // [ncls][N]
+    int raw_sums, k_len;
+    CodeSums a_sums, b_sums;
     const qbp_qparams *qa, *qb;
     int *status;
     int kblock;                   // GEMM: reduction elements per k iteration
@@ -402,7 +407,8 @@ __device__ __forceinline__ void issue_stage(const MmaParams &P, uint32_t a_lo, u
 // Epilogue: tcgen05.ld -> zero-point terms -> fp32 -> swizzled staging slab -> TMA store per warp.
 // TAIL: the instance with the optional normalise / ReLU / requantise tail of the epilogue (the plain instance, which the
 // bandwidth-bound convolutions of a training step use, carries none of it).
-template <bool TAIL>
+// RAW: the instance whose zero-point correction starts from the operands' code sums (no border classes): a launch less.
+template <bool TAIL, bool RAW>
 __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_constant__ MmaParams P)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -598,10 +604,14 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
         const int bar_id = P.msub == 2 ? 1 : 1 + group, bar_cnt = P.msub == 2 ? 256 : 128;
         const int gt = P.msub == 2 ? threadIdx.x - 64 : (threadIdx.x - 64) & 127;     // thread index within the barrier group
         int32_t *region = s_cterm + (P.cterm_all || P.msub == 2 ? 0 : group * P.ncls * P.bn);
+        int neg_za = 0, neg_zb = 0, k_zz = 0;
+        if (RAW) { neg_za = -P.qa->zero_point; neg_zb = -P.qb->zero_point; k_zz = P.k_len * neg_za * neg_zb; }
+        auto row_term = [&](int64_t m) { return RAW ? neg_zb * (int)P.a_sums.at(m) + k_zz : __ldg(P.rowterm + m); };
+        auto col_term = [&](int64_t i) { return RAW ? neg_za * (int)P.b_sums.at(i) : __ldg(P.colterm + i); };
         if (P.cterm_all || (TAIL && P.ep_fold)) {
             // the whole column-term table fits: fill it once (and the per-column constants of the normalisation)
             if (P.cterm_all)
-                for (int i = threadIdx.x - 64; i < P.ncls * (int)P.N; i += 32 * P.ewarps) s_cterm[i] = __ldg(P.colterm + i);
+                for (int i = threadIdx.x - 64; i < P.ncls * (int)P.N; i += 32 * P.ewarps) s_cterm[i] = col_term(i);
             if (TAIL && P.ep_fold)
                 for (int i = threadIdx.x - 64; i < (int)P.N; i += 32 * P.ewarps) s_fold[i] = __ldg(P.ep_fold + i);
             named_barrier(4, 32 * P.ewarps);
@@ -624,7 +634,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
                 const int n = o.img0 + dn, p = o.h0 + dh, q = o.w0 + dw;
                 ri.valid = n < P.Nimg && p < P.H && q < P.W;
                 ri.m = ((int64_t)n * P.H + p) * P.W + q;
-                ri.cls = (p == 0 ? 1 : 0) | (p == P.H - 1 ? 2 : 0) | (q == 0 ? 4 : 0) | (q == P.W - 1 ? 8 : 0);
+                ri.cls = RAW ? 0 : (p == 0 ? 1 : 0) | (p == P.H - 1 ? 2 : 0) | (q == 0 ? 4 : 0) | (q == P.W - 1 ? 8 : 0);
                 const int r0 = quad * 32;            // this warp's 32 rows are a sub-box of the pixel box
                 ri.sx = o.w0 + (r0 & ((1 << P.bw_log2) - 1));
                 ri.sy = o.h0 + ((r0 >> P.bw_log2) & ((1 << P.bh_log2) - 1));
@@ -640,19 +650,19 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
         uint32_t buf = P.msub == 2 ? 0u : (uint32_t)group, fph = 0;
         TileOrigin o = tile_origin(P, tile < P.tiles_total ? tile : 0);
         RowInfo ri = row_info(o);
-        int rterm = (tile < P.tiles_total && ri.valid) ? __ldg(P.rowterm + ri.m) : 0;
+        int rterm = (tile < P.tiles_total && ri.valid) ? row_term(ri.m) : 0;
         for (; tile < P.tiles_total; tile += tile_step) {
             // the next tile's row term is fetched now, so that its latency hides behind this tile
             const int tile_next = tile + tile_step;
             const TileOrigin o_next = tile_origin(P, tile_next < P.tiles_total ? tile_next : 0);
             const RowInfo ri_next = row_info(o_next);
-            const int rterm_next = (tile_next < P.tiles_total && ri_next.valid) ? __ldg(P.rowterm + ri_next.m) : 0;
+            const int rterm_next = (tile_next < P.tiles_total && ri_next.valid) ? row_term(ri_next.m) : 0;
             if (!P.cterm_all) {
                 // column terms of this tile into shared memory (the previous tile's readers are done first)
                 named_barrier(bar_id, bar_cnt);
                 for (int i = gt; i < P.ncls * P.bn; i += bar_cnt) {
                     const int cls = i / P.bn, n = o.n0 + i % P.bn;
-                    region[i] = n < P.N ? __ldg(P.colterm + (int64_t)cls * P.N + n) : 0;
+                    region[i] = n < P.N ? col_term((int64_t)cls * P.N + n) : 0;
                 }
                 named_barrier(bar_id, bar_cnt);
             }
@@ -831,52 +841,6 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
 }
 
 // ================================================= zero-point correction terms
-// GEMM: rowterm[m] = -zb * sum_k A[m,k] + K*za*zb ; colterm[n] = -za * sum_k B[k,n].
-// The code sums arrive as int32 (sums along stored rows) or int64 (along stored columns).
-__global__ void gemm_terms_kernel(const int32_t *ra32, const long long *ra64, const int32_t *cb32, const long long *cb64,
-                                  int64_t M, int64_t N, int64_t K, const qbp_qparams *qa, const qbp_qparams *qb,
-                                  int32_t *rowterm, int32_t *colterm)
-{
-    pdl_enter();
-    const int za = qa->zero_point, zb = qb->zero_point;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < M) {
-        const int ra = ra32 ? ra32[i] : (int)ra64[i];
-        rowterm[i] = -zb * ra + (int)K * za * zb;
-    }
-    if (i < N) {
-        const int cb = cb32 ? cb32[i] : (int)cb64[i];
-        colterm[i] = -za * cb;
-    }
-}
-
-// colterm[cls][n] = -z_in * sum over the taps valid for border class cls of the
-// filter's code sum for that tap and output column n.  cls bits: 1 first row,
-// 2 last row, 4 first column, 8 last column.  wsum32: [n][tap] (forward: sums over
-// the input channels); wsum64: [tap][n] (layer gradient: sums over the output channels).
-__global__ void conv_colterm_kernel(const int32_t *wsum32, const long long *wsum64, int N, int R, int S, int pad,
-                                    int dgrad, const qbp_qparams *q_in, int32_t *colterm)
-{
-    pdl_enter();
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    const int cls = blockIdx.y;
-    if (n >= N) return;
-    const bool top = cls & 1, bottom = cls & 2, left = cls & 4, right = cls & 8;
-    long long sum = 0;
-    for (int r = 0; r < R; ++r) {
-        // forward: tap row r reads input row p - pad + r; layer gradient: gradient row h + pad - r
-        const bool low = dgrad ? r > pad : r < pad, high = dgrad ? r < pad : r > pad;
-        if ((low && top) || (high && bottom)) continue;
-        for (int s = 0; s < S; ++s) {
-            const bool lo_c = dgrad ? s > pad : s < pad, hi_c = dgrad ? s < pad : s > pad;
-            if ((lo_c && left) || (hi_c && right)) continue;
-            const int tap = r * S + s;
-            sum += wsum32 ? (long long)wsum32[(int64_t)n * R * S + tap] : wsum64[(int64_t)tap * N + n];
-        }
-    }
-    colterm[cls * N + n] = -q_in->zero_point * (int)sum;
-}
-
 // A small filter in one launch (Appendix B's quantiser for the weights, then what the forward convolution's zero-point
 // correction needs of them): min / max scan, scale and zero-point, nearest 8-bit codes, the code sums of every
 // (output channel, tap) over the input channels, and the forward column terms
@@ -976,38 +940,66 @@ __global__ void __launch_bounds__(1024) filter_dgrad_colterm_kernel(const int8_t
     }
 }
 
-// rowterm[pixel] = -z_w * (sum of the input's channel sums over the taps inside the image)
-//                   + (taps inside) * Cred * z_in * z_w          (pad is 0 or 1)
-// blockIdx.y = image, blockIdx.x * 256 + threadIdx.x = position inside it; the nine taps unrolled under predicates
-// and the one division by a multiply-high (with plain divisions and loops this kernel ran 260 instructions per pixel).
-__global__ void __launch_bounds__(256) conv_rowterm_kernel(const int32_t *__restrict__ chan_sum, int HW, int H, int W,
-                                                           FastDiv dW, int pad, int Cred, const qbp_qparams *q_in,
-                                                           const qbp_qparams *q_w, int32_t *__restrict__ rowterm)
+// The correction terms of a 3 x 3 convolution.
+// Blocks below `row_blocks`: rowterm[pixel] = -z_w * (sum of the input's channel sums over the taps inside the image)
+//                   + (taps inside) * Cred * z_in * z_w
+// a block = 256 positions of one image (the nine taps unrolled under predicates and the divisions by multiply-high: with
+// plain divisions and loops this ran 260 instructions per pixel).
+// The rest: colterm[cls][n] = -z_in * sum over the taps valid for border class cls of the filter's code sum for that tap and
+// output column n.  cls bits: 1 first row, 2 last row, 4 first column, 8 last column.  Sums of the filter: forward [n][tap]
+// (over the input channels), layer gradient [tap][n] (over the output channels).
+struct ConvTerms {
+    const int32_t *chan_sum; int HW, H, W; FastDiv dW, dB;     // dB: blocks per image
+    int Cred, row_blocks;
+    const qbp_qparams *q_in, *q_w;
+    int32_t *rowterm;
+    CodeSums w_sums; int N, dgrad;
+    int32_t *colterm;
+};
+__global__ void __launch_bounds__(256) conv_terms_kernel(const __grid_constant__ ConvTerms T)
 {
     pdl_enter();
-    const int i = (int)blockIdx.x * 256 + (int)threadIdx.x;
-    if (i >= HW) return;
+    if ((int)blockIdx.x >= T.row_blocks) {
+        const int i = ((int)blockIdx.x - T.row_blocks) * 256 + (int)threadIdx.x;
+        if (i >= 16 * T.N) return;
+        const int cls = i / T.N, n = i - cls * T.N;
+        const bool top = cls & 1, bottom = cls & 2, left = cls & 4, right = cls & 8;
+        int sum = 0;
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+            // forward: tap row r reads input row p - 1 + r; layer gradient: gradient row h + 1 - r
+            const int r = T.dgrad ? 2 - tap / 3 : tap / 3, s = T.dgrad ? 2 - tap % 3 : tap % 3;
+            if ((r == 0 && top) || (r == 2 && bottom) || (s == 0 && left) || (s == 2 && right)) continue;
+            sum += (int)T.w_sums.at(T.dgrad ? (int64_t)tap * T.N + n : (int64_t)n * 9 + tap);
+        }
+        T.colterm[i] = -T.q_in->zero_point * sum;
+        return;
+    }
+    int img, bi;
+    T.dB.divmod((int)blockIdx.x, img, bi);
+    const int i = bi * 256 + (int)threadIdx.x;
+    if (i >= T.HW) return;
     int p, q;
-    dW.divmod(i, p, q);
-    const int m = (int)blockIdx.y * HW + i;                  // (fewer than 2^31 positions)
-    const bool up = pad && p > 0, down = pad && p + 1 < H, left = pad && q > 0, right = pad && q + 1 < W;
-    const int32_t *c = chan_sum + m;
+    T.dW.divmod(i, p, q);
+    const int m = img * T.HW + i;                            // (fewer than 2^31 positions)
+    const bool up = p > 0, down = p + 1 < T.H, left = q > 0, right = q + 1 < T.W;
+    const int32_t *c = T.chan_sum + m;
     int box = __ldg(c);
     if (left) box += __ldg(c - 1);
     if (right) box += __ldg(c + 1);
     if (up) {
-        box += __ldg(c - W);
-        if (left) box += __ldg(c - W - 1);
-        if (right) box += __ldg(c - W + 1);
+        box += __ldg(c - T.W);
+        if (left) box += __ldg(c - T.W - 1);
+        if (right) box += __ldg(c - T.W + 1);
     }
     if (down) {
-        box += __ldg(c + W);
-        if (left) box += __ldg(c + W - 1);
-        if (right) box += __ldg(c + W + 1);
+        box += __ldg(c + T.W);
+        if (left) box += __ldg(c + T.W - 1);
+        if (right) box += __ldg(c + T.W + 1);
     }
     const int taps = (1 + (up ? 1 : 0) + (down ? 1 : 0)) * (1 + (left ? 1 : 0) + (right ? 1 : 0));
-    const int za = q_in->zero_point, zb = q_w->zero_point;
-    rowterm[m] = -zb * box + taps * Cred * za * zb;
+    const int za = T.q_in->zero_point, zb = T.q_w->zero_point;
+    T.rowterm[m] = -zb * box + taps * T.Cred * za * zb;
 }
 
 // Per-column sum / min / max from the epilogue warps' partial rows: one block of 128 threads per column.
@@ -1209,9 +1201,11 @@ static int launch_mma(MmaParams &P, int tiles_m, bool clear_status, cudaStream_t
     P.d_tiles_h = make_fastdiv(P.mode == MODE_GEMM ? 1 : P.tiles_h);
     const size_t smem = (size_t)fixed + P.b_res_bytes + (size_t)stages * stage_bytes;
     const bool tail = P.ep_fold || P.ep_relu || P.ep_q;
-    static PerDeviceOnce configured[2];
-    if (tail) QBP_SMEM_OPT_IN(configured[1], qbp_mma_kernel<true>, kSmemBudget);
-    else      QBP_SMEM_OPT_IN(configured[0], qbp_mma_kernel<false>, kSmemBudget);
+    static PerDeviceOnce configured[4];
+    const int id = (tail ? 2 : 0) + (P.raw_sums ? 1 : 0);
+    void (*kernel)(const MmaParams) = id == 0 ? qbp_mma_kernel<false, false> : id == 1 ? qbp_mma_kernel<false, true>
+                                    : id == 2 ? qbp_mma_kernel<true, false> : qbp_mma_kernel<true, true>;
+    QBP_SMEM_OPT_IN(configured[id], kernel, kSmemBudget);
     if (clear_status) QBP_CUDA_OK(cudaMemsetAsync(P.status, 0, sizeof(int), st));
     // one CTA per SM (its shared-memory ring fills the SM), each walking its share of the tiles
     int grid = std::min(P.tiles_total, sm_count());
@@ -1222,22 +1216,29 @@ static int launch_mma(MmaParams &P, int tiles_m, bool clear_status, cudaStream_t
     }
     P.grid = grid;
     QBP_TRACE_BEGIN(st);
-    if (tail) launch(qbp_mma_kernel<true>, grid, kMmaThreads, smem, st, P);
-    else      launch(qbp_mma_kernel<false>, grid, kMmaThreads, smem, st, P);
+    launch(kernel, grid, kMmaThreads, smem, st, P);
     QBP_LAUNCH_OK("qbp_mma_kernel");
     return QBP_OK;
 }
 
-static size_t gemm_ws_bytes(int64_t M, int64_t N)
+static size_t gemm_ws_bytes(int64_t M, int64_t N, int64_t K)
 {
-    return 256 + align_up(sizeof(int32_t) * M, 256) + align_up(sizeof(int32_t) * N, 256) +
-           align_up(sizeof(int64_t) * M, 256) + align_up(sizeof(int64_t) * N, 256) + colstat_ws_bytes(N);
+    // (code sums of either operand, stored either way round)
+    auto sums = [&](int64_t n) { return align_up(sizeof(int32_t) * std::max(sum_elems(n, K, false), sum_elems(K, n, true)), 256); };
+    return 256 + sums(M) + sums(N) + colstat_ws_bytes(N);
 }
 
 bool conv_supported(const qbp_conv_desc *d)
 {
     return d->stride == 1 && d->R == d->S && (d->R == 1 || d->R == 3) && d->pad == (d->R - 1) / 2 && d->N > 0 &&
            d->H > 0 && d->W > 0 && d->C > 0 && d->K > 0 && d->C % 16 == 0 && d->K % 16 == 0;
+}
+
+// The filter's code sums: forward [K][taps], layer gradient pieces of [taps * C].
+static size_t filter_sum_elems(const qbp_conv_desc *d)
+{
+    const int64_t taps = (int64_t)d->R * d->S;
+    return std::max(sum_elems(d->K * taps, d->C, false), sum_elems(d->K, taps * d->C, true));
 }
 
 // What the product itself carves from the workspace, and with the room for the column statistics' partial rows
@@ -1247,7 +1248,7 @@ static size_t conv_core_ws_bytes(const qbp_conv_desc *d)
     const int64_t pix = (int64_t)d->N * d->H * d->W;
     const int64_t nmax = std::max(d->C, d->K);
     return 256 + align_up(sizeof(int32_t) * pix, 256) * 2 + align_up(sizeof(int32_t) * 16 * nmax, 256) +
-           align_up(sizeof(int64_t) * (int64_t)d->R * d->S * nmax, 256);
+           align_up(sizeof(int32_t) * filter_sum_elems(d), 256);
 }
 static size_t conv_ws_bytes(const qbp_conv_desc *d)
 {
@@ -1299,8 +1300,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_selftest_bounded_wait(
 
 extern "C" __attribute__((visibility("default"))) size_t qbp_gemm_s8_workspace_bytes(int64_t M, int64_t N, int64_t K)
 {
-    (void)K;
-    return gemm_ws_bytes(M > 0 ? M : 1, N > 0 ? N : 1);
+    return gemm_ws_bytes(M > 0 ? M : 1, N > 0 ? N : 1, K > 0 ? K : 1);
 }
 
 extern "C" __attribute__((visibility("default"))) int qbp_gemm_s8(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A,
@@ -1330,8 +1330,8 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
     if (!acc_out && !C && !(ep && ep->q_out)) return fail(QBP_ERR_INVALID_ARG, "gemm_s8: acc_out and C are both NULL");
     if (!aligned16(A) || !aligned16(B) || (C && !aligned16(C)) || (acc_out && !aligned16(acc_out)))
         return fail(QBP_ERR_INVALID_ARG, "gemm_s8: operands must be 16-byte aligned");
-    if (!ws || ws_bytes < gemm_ws_bytes(M, N))
-        return fail(QBP_ERR_WORKSPACE, "gemm_s8: workspace of %zu bytes needed, %zu given", gemm_ws_bytes(M, N), ws_bytes);
+    if (!ws || ws_bytes < gemm_ws_bytes(M, N, K))
+        return fail(QBP_ERR_WORKSPACE, "gemm_s8: workspace of %zu bytes needed, %zu given", gemm_ws_bytes(M, N, K), ws_bytes);
 
     bool stats = false, has_tail = false;
     EpilogueTail tail;
@@ -1343,42 +1343,27 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
     WsCarver w(ws, ws_bytes);
     int *status = w.take<int>(1);
     if (ext_status) status = ext_status;         // the caller's sticky word: raised here, never cleared
-    int32_t *rowterm = w.take<int32_t>(M);
-    int32_t *colterm = w.take<int32_t>(N);
-    int64_t *tmp_m = w.take<int64_t>(M);
-    int64_t *tmp_n = w.take<int64_t>(N);
+    // code sums along the reduction, the caller's or of this call's own (one launch for both operands)
+    const SumJob a_job = transA ? SumJob{A, K, M, 1, 1, nullptr} : SumJob{A, M, K, 0, 1, nullptr};
+    const SumJob b_job = transB ? SumJob{B, N, K, 0, 1, nullptr} : SumJob{B, K, N, 1, 1, nullptr};
+    SumJob jobs[2];
+    int njobs = 0;
+    CodeSums asum = sums_of(a_sums), bsum = sums_of(b_sums);
+    if (!a_sums) { jobs[njobs] = a_job; jobs[njobs].out = w.take<int32_t>(sum_elems(a_job.rows, a_job.cols, a_job.over_rows)); asum = sums_of(jobs[njobs++]); }
+    if (!b_sums) { jobs[njobs] = b_job; jobs[njobs].out = w.take<int32_t>(sum_elems(b_job.rows, b_job.cols, b_job.over_rows)); bsum = sums_of(jobs[njobs++]); }
     ColStatParts parts{nullptr, nullptr, nullptr, 0};
     if (stats) {
         const size_t cells = (size_t)colstat_rows_max() * (size_t)N;
         parts.lo = w.take<float>(cells); parts.hi = w.take<float>(cells); parts.sum = w.take<double>(cells);
     }
 
-    // code sums along the reduction
     int rc = QBP_OK;
-    // (sums along stored rows are int32, along stored columns int64; the caller's are int32 either way)
-    const bool a32 = a_sums || !transA, b32 = b_sums || transB;
-    if (!a_sums) {
-        if (!transA) rc = launch_rowsum(A, true, M, K, (int32_t *)tmp_m, st);
-        else         rc = launch_colsum(A, true, K, M, tmp_m, st);
-        if (rc) return rc;
-    }
-    if (!b_sums) {
-        if (transB) rc = launch_rowsum(B, true, N, K, (int32_t *)tmp_n, st);
-        else        rc = launch_colsum(B, true, K, N, tmp_n, st);
-        if (rc) return rc;
-    }
-    const int32_t *ra32 = a_sums ? a_sums : (const int32_t *)tmp_m, *cb32 = b_sums ? b_sums : (const int32_t *)tmp_n;
-    const int64_t mx = std::max(M, N);
-    QBP_TRACE_BEGIN(st);
-    launch(gemm_terms_kernel, (int)((mx + 255) / 256), 256, 0, st, a32 ? ra32 : nullptr, a32 ? nullptr : (const long long *)tmp_m,
-        b32 ? cb32 : nullptr, b32 ? nullptr : (const long long *)tmp_n, M, N, K, qa, qb,
-        rowterm, colterm);
-    QBP_LAUNCH_OK("gemm_terms_kernel");
+    if (njobs && (rc = launch_code_sums(jobs, njobs, st))) return rc;
 
     // large products run on CTA pairs (256 x 256 tiles across two SMs); the column statistics are the
     // single-CTA kernel's (at most 256 columns: narrow either way)
     if (gemm2_eligible(M, N, K) && !stats && !has_tail)
-        return launch_gemm2(transA, transB, M, N, K, A, qa, B, qb, acc_out, C, rowterm, colterm, status, !ext_status, st);
+        return launch_gemm2(transA, transB, M, N, K, A, qa, B, qb, acc_out, C, asum, bsum, status, !ext_status, st);
 
     MmaParams P{};
     P.mode = MODE_GEMM;
@@ -1416,7 +1401,7 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
     P.tiles_n = (int)((N + P.bn - 1) / P.bn);
     P.M = M; P.N = N;
     P.acc_out = acc_out; P.out = C;
-    P.rowterm = rowterm; P.colterm = colterm; P.qa = qa; P.qb = qb; P.status = status;
+    P.raw_sums = 1; P.k_len = (int)K; P.a_sums = asum; P.b_sums = bsum; P.qa = qa; P.qb = qb; P.status = status;
     if (stats) { P.st_lo = parts.lo; P.st_hi = parts.hi; P.st_sum = parts.sum; }
     bool fused_row_sums = false;
     if (has_tail) {
@@ -1517,32 +1502,37 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
     int32_t *rowterm = w.take<int32_t>(pix);
     int32_t *chan_sum = w.take<int32_t>(pix);
     int32_t *colterm = w.take<int32_t>(16 * nmax);
-    int64_t *wsum = w.take<int64_t>((int64_t)taps * nmax);
+    int32_t *wsum = w.take<int32_t>(filter_sum_elems(d));
+    const SumJob w_job = dgrad ? SumJob{wgt, d->K, (int64_t)taps * d->C, 1, 1, wsum} : SumJob{wgt, (int64_t)d->K * taps, d->C, 0, 1, wsum};
+    const bool own_colterm = !(tail && tail->colterm);       // (else: the column terms came with the filter's codes)
+    const bool raw_sums = d->R == 1;                         // (1 x 1: no borders, the kernel works on the sums themselves)
 
     int rc = QBP_OK;
+    if (in_chan_sum) chan_sum = const_cast<int32_t *>(in_chan_sum);
+    if (tail && tail->colterm) colterm = const_cast<int32_t *>(tail->colterm);
     if (!(tail && tail->keep_terms)) {
-        if (in_chan_sum) chan_sum = const_cast<int32_t *>(in_chan_sum);
-        else if ((rc = launch_rowsum(in, true, pix, Cred, chan_sum, st))) return rc;
-        if (!(tail && tail->colterm)) {          // (else: the column terms came with the filter's codes)
-            if (!dgrad) rc = launch_rowsum(wgt, true, (int64_t)d->K * taps, d->C, (int32_t *)wsum, st);   // [k][tap]
-            else        rc = launch_colsum(wgt, true, d->K, (int64_t)taps * d->C, wsum, st);                    // [tap][c]
-            if (rc) return rc;
+        SumJob jobs[2];
+        int njobs = 0;
+        if (!in_chan_sum) jobs[njobs++] = SumJob{in, pix, Cred, 0, 1, chan_sum};
+        if (own_colterm) jobs[njobs++] = w_job;
+        if (njobs && (rc = launch_code_sums(jobs, njobs, st))) return rc;
+        if (!raw_sums) {
+            ConvTerms T{};
+            const int per_img = (d->H * d->W + 255) / 256;
+            T.chan_sum = chan_sum; T.HW = d->H * d->W; T.H = d->H; T.W = d->W; T.dW = make_fastdiv(d->W); T.dB = make_fastdiv(per_img);
+            T.Cred = Cred; T.row_blocks = per_img * d->N; T.q_in = q_in; T.q_w = q_w; T.rowterm = rowterm;
+            T.w_sums = sums_of(w_job); T.N = Nout; T.dgrad = dgrad ? 1 : 0; T.colterm = colterm;
             QBP_TRACE_BEGIN(st);
-            launch(conv_colterm_kernel, dim3((Nout + 127) / 128, 16), 128, 0, st, dgrad ? nullptr : (const int32_t *)wsum, dgrad ? (const long long *)wsum : nullptr, Nout, d->R, d->S, d->pad,
-                dgrad ? 1 : 0, q_in, colterm);
-            QBP_LAUNCH_OK("conv_colterm_kernel");
+            launch(conv_terms_kernel, T.row_blocks + (own_colterm ? (16 * Nout + 255) / 256 : 0), 256, 0, st, T);
+            QBP_LAUNCH_OK("conv_terms_kernel");
         }
-        QBP_TRACE_BEGIN(st);
-        launch(conv_rowterm_kernel, dim3((unsigned)((d->H * d->W + 255) / 256), (unsigned)d->N), 256, 0, st, chan_sum, d->H * d->W, d->H, d->W, make_fastdiv(d->W), d->pad, Cred, q_in, q_w, rowterm);
-        QBP_LAUNCH_OK("conv_rowterm_kernel");
     }
 
     MmaParams P{};
     P.mode = dgrad ? MODE_DGRAD : MODE_FPROP;
-    P.msub = 1; P.ncls = 16; P.nslab = 1;
+    P.msub = 1; P.ncls = raw_sums ? 1 : 16; P.nslab = 1;
     if (stats) { P.st_lo = stats->lo; P.st_hi = stats->hi; P.st_sum = stats->sum; }
     if (tail) { P.ep_fold = tail->fold; P.ep_relu = tail->relu; P.ep_rq = tail->rq; P.ep_q = tail->q; }
-    if (tail && tail->colterm) colterm = const_cast<int32_t *>(tail->colterm);
     P.H = d->H; P.W = d->W; P.Nimg = d->N; P.pad = d->pad; P.S = d->S; P.Cred = Cred;
     const uint32_t cb = Cred % 128 == 0 ? 128u : Cred % 64 == 0 ? 64u : 32u;      // reduction bytes per stage row
     P.chunk_bytes = (int)cb;
@@ -1606,6 +1596,7 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
     P.idesc = make_idesc(true, true, P.a.major, P.b.major, 128, (uint32_t)P.bn);
     P.acc_out = acc_out; P.out = out;
     P.rowterm = rowterm; P.colterm = colterm; P.qa = q_in; P.qb = q_w; P.status = status;
+    P.raw_sums = raw_sums ? 1 : 0; P.k_len = Cred; P.a_sums = sums_of(chan_sum); P.b_sums = sums_of(w_job);
     // each row's code sum comes from the epilogue when one column tile holds the whole row, else from a pass over the codes
     const bool fused_row_sums = want_codes && tail->row_sums && P.tiles_n == 1;
     if (fused_row_sums) P.ep_rowsum = tail->row_sums;

@@ -12,6 +12,32 @@ namespace qbp {
 // ---- sums of stored codes (qbp_quant.cu) -------------------------------------
 int launch_rowsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int32_t *sums, cudaStream_t st);
 int launch_colsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int64_t *sums, cudaStream_t st);
+// Sums of stored codes as a product takes them for its zero-point correction: element i is the sum of `pieces` int32
+// values p[i], p[i + stride], ... (sums along the rows of a tensor in pieces of its columns, so that nothing has to start at
+// zero and no atomics are needed).
+struct CodeSums {
+    const int32_t *p; int pieces; int64_t stride;
+#ifdef __CUDACC__
+    __device__ __forceinline__ long long at(int64_t i) const
+    {
+        long long s = 0;
+#pragma unroll 4
+        for (int k = 0; k < pieces; ++k) s += __ldg(p + (int64_t)k * stride + i);
+        return s;
+    }
+#endif
+};
+inline CodeSums sums_of(const int32_t *p) { return CodeSums{p, 1, 0}; }
+// Up to four such sums in one launch (code_sums_kernel): per row (over_rows = 0: out [rows]), or per column over the rows
+// (over_rows = 1: out [sum_pieces(rows, cols)][cols]).  cols a multiple of 16, q 16-byte aligned, fewer than 2^31 rows.
+struct SumJob { const void *q; int64_t rows, cols; int over_rows, is_signed; int32_t *out; };
+int sum_pieces(int64_t rows, int64_t cols);
+inline size_t sum_elems(int64_t rows, int64_t cols, bool over_rows) { return over_rows ? (size_t)sum_pieces(rows, cols) * (size_t)cols : (size_t)rows; }
+inline CodeSums sums_of(const SumJob &j)
+{
+    return j.over_rows ? CodeSums{j.out, sum_pieces(j.rows, j.cols), j.cols} : sums_of(j.out);
+}
+int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st);
 
 // ---- per-tensor range scan (qbp_quant.cu): *qp = 8-bit parameters of [min(lowest, 0), max(highest, 0)] -------------
 size_t range_scan_ws_bytes();
@@ -58,7 +84,7 @@ int rangebn_fold_from_parts(int64_t n, int64_t C, const float *gamma, const floa
 // column, as rangebn_fold_from_parts leaves them), ReLU, and 8-bit codes of the result with parameters *rq
 // (q [M x N], row_sums [M] nullable).  keep_terms: the zero-point term kernels ran for the same operands in the
 // call just before on the same workspace and are not run again.
-// colterm (nullable): the column terms [16][N] of this product, already computed (launch_filter_prep).
+// colterm (nullable; 3 x 3): the column terms [16][N] of this product, already computed (launch_filter_prep).
 struct EpilogueTail { const float4 *fold; int relu; const qbp_qparams *rq; int8_t *q; int32_t *row_sums; int keep_terms; const int32_t *colterm; };
 // A small filter quantised and its forward column terms computed in one launch (qbp_mma.cu).
 bool filter_prep_supported(const qbp_conv_desc *d, const float *w, const int8_t *codes);
@@ -112,14 +138,14 @@ int make_map_out_2d(CUtensorMap *map, float *base, uint64_t rows, uint64_t cols)
 // ---- the dense product on CTA pairs (qbp_mma2.cu) -------------------------------
 bool gemm2_eligible(int64_t M, int64_t N, int64_t K);
 int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,
-                 const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const int32_t *rowterm,
-                 const int32_t *colterm, int *status, bool clear_status, cudaStream_t st);
+                 const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const CodeSums &a_sums,
+                 const CodeSums &b_sums, int *status, bool clear_status, cudaStream_t st);
 
 // ---- the dense weight gradient on CTA pairs (qbp_wgrad2.cu) ----------------------
 bool wgrad2_eligible(int64_t M, int64_t N, int64_t K);
 int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qparams *qx, const int8_t *g_hi,
-                  const uint8_t *g_lo, const qbp_qparams *qg16, int64_t *acc_out, float *dW, const long long *rowterm,
-                  const long long *colterm, int *status, cudaStream_t st, bool lo_signed = false);
+                  const uint8_t *g_lo, const qbp_qparams *qg16, int64_t *acc_out, float *dW, const CodeSums &sx,
+                  const CodeSums &shi, const CodeSums &slo, int *status, cudaStream_t st, bool lo_signed = false);
 
 // ---- shared-memory operand descriptors ---------------------------------------
 // How one operand tile of a pipeline stage is laid out and walked by the MMAs.

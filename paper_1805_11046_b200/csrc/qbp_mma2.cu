@@ -38,7 +38,8 @@ struct Mma2Params {
     FastDiv d_group;
     int64_t M, N;
     int32_t *acc_out; float *out;
-    const int32_t *rowterm, *colterm;
+    CodeSums a_sums, b_sums;         // along the reduction: rowterm = -zb * a_sums[m] + K * za * zb, colterm = -za * b_sums[n]
+    int k_len;
     const qbp_qparams *qa, *qb;
     int *status;
 };
@@ -265,6 +266,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
         const int row = quad * 32 + lane;
         uint8_t *slab = staging + (size_t)ew * k2Slab;
         const float scale = __fmul_rn(P.qa->scale, P.qb->scale);
+        const int neg_za = -P.qa->zero_point, neg_zb = -P.qb->zero_point, k_zz = P.k_len * neg_za * neg_zb;
         const uint32_t leader_empty0 = map_to_cta(&acc_empty[0], 0), leader_empty1 = map_to_cta(&acc_empty[1], 0);
         uint32_t buf = 0, fph = 0;
         for (int tile = pair; tile < P.tiles_total; tile += P.pairs) {
@@ -272,10 +274,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
             const int64_t m = (int64_t)o.m0 + 256 * sub + 128 * (int)rank + row;
             const bool valid = m < P.M;
             const bool slab_in = (int64_t)o.m0 + 256 * sub + 128 * (int)rank + quad * 32 < P.M;
-            const int rterm = valid ? __ldg(P.rowterm + m) : 0;
+            const int rterm = valid ? neg_zb * (int)P.a_sums.at(m) + k_zz : 0;
             // column terms of this tile (the previous tile's readers are done first)
             named_barrier(1, 32 * k2EpiWarps);
-            if (et < 256) s_cterm[et] = o.n0 + et < P.N ? __ldg(P.colterm + o.n0 + et) : 0;
+            if (et < 256) s_cterm[et] = o.n0 + et < P.N ? neg_za * (int)P.b_sums.at(o.n0 + et) : 0;
             named_barrier(1, 32 * k2EpiWarps);
             const int64_t ncol = P.N - o.n0;
             const int nchunks = (int)((ncol < 256 ? ncol : 256) + 31) / 32;
@@ -362,8 +364,8 @@ bool gemm2_eligible(int64_t M, int64_t N, int64_t K)
 }
 
 int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,
-                 const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const int32_t *rowterm,
-                 const int32_t *colterm, int *status, bool clear_status, cudaStream_t st)
+                 const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const CodeSums &a_sums,
+                 const CodeSums &b_sums, int *status, bool clear_status, cudaStream_t st)
 {
     Mma2Params P{};
     int rc;
@@ -393,7 +395,7 @@ int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const 
     if (stages < 2 * P.cg) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "gemm_s8: the pair kernel's ring does not fit");
     P.stages = stages;
     P.M = M; P.N = N; P.acc_out = acc_out; P.out = C;
-    P.rowterm = rowterm; P.colterm = colterm; P.qa = qa; P.qb = qb; P.status = status;
+    P.a_sums = a_sums; P.b_sums = b_sums; P.k_len = (int)K; P.qa = qa; P.qb = qb; P.status = status;
     const size_t smem = 1024 + (size_t)stages * stage_bytes + k2EpiWarps * k2Slab;
     static PerDeviceOnce configured;
     QBP_SMEM_OPT_IN(configured, qbp_mma2_kernel, k2Smem);

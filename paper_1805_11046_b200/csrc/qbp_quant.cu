@@ -6,6 +6,7 @@
 // flight per thread, warp-shuffle + shared-memory reductions, grids sized to
 // fill every SM.  Also hosts the library's error-reporting state.
 #include "qbp_colscan.cuh"
+#include "qbp_mma.cuh"
 
 #include <algorithm>
 #include <cstring>
@@ -597,7 +598,131 @@ __global__ void __launch_bounds__(kThreads) colsum_kernel(const uint8_t *__restr
         atomicAdd(&sums[slab0 * 16 + c], (unsigned long long)(long long)s_acc[c]);
 }
 
+// The sums of up to four code tensors in one launch (see SumJob).  Unsigned codes are summed as codes - 128 (top bit
+// flipped) and 128 per code is added at the end, so that one form of the dot product serves both.
+// Per row: a group of G lanes per row, four 16-byte loads in flight.  Per column: a block takes a strip of 128 columns
+// (eight 16-byte groups across, 32 rows high) over one piece of the rows, eight rows in flight per thread; its rows
+// meet by shuffle and in 4 KB of shared memory.
+// Bound by the read of the codes (134 MB for the operands of an 8192^3 product: 24 us with their launch, where a launch per
+// operand, a memset and a launch for the correction terms took 57).
+struct SumJobDev { const uint8_t *q; int64_t rows; int cols, over_rows, first, blocks, G, pieces; uint32_t flip; int32_t *out; };
+struct SumJobs { SumJobDev j[4]; int count; };
+__global__ void __launch_bounds__(kThreads) code_sums_kernel(const __grid_constant__ SumJobs J)
+{
+    pdl_enter();
+    int k = 0;
+    while (k + 1 < J.count && (int)blockIdx.x >= J.j[k + 1].first) ++k;
+    const SumJobDev &j = J.j[k];
+    const int bid = (int)blockIdx.x - j.first, cv = j.cols >> 4, lane = threadIdx.x & 31;
+    const uint32_t flip = j.flip;
+    if (!j.over_rows) {
+        const int G = j.G, gl = lane % G;
+        const int groups_per_block = kThreads / G;
+        // (the loop bound is the block's, so that the shuffles see whole warps)
+        for (int64_t rb = (int64_t)bid * groups_per_block; rb < j.rows; rb += (int64_t)j.blocks * groups_per_block) {
+            const int64_t r = rb + threadIdx.x / G;
+            const bool in = r < j.rows;
+            const uint4 *row = reinterpret_cast<const uint4 *>(j.q + (in ? r : 0) * j.cols);
+            int acc = 0;
+            auto add = [&](const uint4 &v) {
+                acc = __dp4a((int)(v.x ^ flip), 0x01010101, acc); acc = __dp4a((int)(v.y ^ flip), 0x01010101, acc);
+                acc = __dp4a((int)(v.z ^ flip), 0x01010101, acc); acc = __dp4a((int)(v.w ^ flip), 0x01010101, acc);
+            };
+            int c = in ? gl : cv;
+            for (; c + 3 * G < cv; c += 4 * G) {
+                uint4 v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = __ldg(row + c + u * G);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) add(v[u]);
+            }
+            for (; c < cv; c += G) add(__ldg(row + c));
+            for (int o = G >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (in && gl == 0) j.out[r] = acc + (flip ? 128 * j.cols : 0);
+        }
+        return;
+    }
+    __shared__ int s_acc[kThreads / 32][128];
+    const int strips = (cv + 7) / 8, strip = bid % strips, piece = bid / strips;
+    const int64_t r_begin = j.rows * piece / j.pieces, r_end = j.rows * (piece + 1) / j.pieces;
+    const int g = strip * 8 + (lane & 7), ty = (int)(threadIdx.x >> 5) * 4 + (lane >> 3);
+    int acc[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) acc[e] = 0;
+    if (g < cv) {
+        constexpr int U = 8;
+        const uint8_t *base = j.q + (int64_t)g * 16;
+        for (int64_t r = r_begin + ty; r < r_end; r += 32 * U) {
+            uint4 v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (r + 32 * u < r_end) v[u] = __ldg(reinterpret_cast<const uint4 *>(base + (r + 32 * u) * j.cols));
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (r + 32 * u >= r_end) break;
+                const uint32_t w[4] = {v[u].x ^ flip, v[u].y ^ flip, v[u].z ^ flip, v[u].w ^ flip};
+#pragma unroll
+                for (int e = 0; e < 16; ++e) acc[e] = __dp4a((int)w[e >> 2], 1 << (8 * (e & 3)), acc[e]);
+            }
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 8);
+        acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 16);
+    }
+    if (lane < 8) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) s_acc[threadIdx.x >> 5][lane * 16 + e] = acc[e];
+    }
+    __syncthreads();
+    const int c = strip * 128 + (int)threadIdx.x;
+    if (threadIdx.x < 128 && c < j.cols) {
+        int sum = 0;
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w) sum += s_acc[w][threadIdx.x];
+        j.out[(int64_t)piece * j.cols + c] = sum + (flip ? 128 * (int)(r_end - r_begin) : 0);
+    }
+}
+
 // ----------------------------------------------------------------- launchers
+// Pieces of the rows in a column sum: enough blocks for two per SM, at least 128 rows each (four per thread row), at most 32
+// pieces (the reader adds them up) -- but at most 2^22 rows each, so that a piece fits int32 (255 * 2^22 < 2^31).
+int sum_pieces(int64_t rows, int64_t cols)
+{
+    const int64_t strips = (cols + 127) / 128;
+    int64_t p = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(2ll * sm_count() / strips, 32), rows / 128));
+    return (int)std::max<int64_t>(p, (rows >> 22) + 1);
+}
+
+int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st)
+{
+    SumJobs J{};
+    int first = 0;
+    for (int i = 0; i < count; ++i) {
+        const SumJob &s = jobs[i];
+        if (s.cols % 16 || !aligned16(s.q)) return fail(QBP_ERR_INVALID_ARG, "code sums need 16-byte aligned rows (cols %% 16 == 0)");
+        SumJobDev &j = J.j[i];
+        j.q = static_cast<const uint8_t *>(s.q); j.rows = s.rows; j.cols = (int)s.cols; j.over_rows = s.over_rows; j.out = s.out;
+        j.flip = s.is_signed ? 0u : 0x80808080u; j.first = first; j.G = 1; j.pieces = 1;
+        if (s.over_rows) {
+            j.pieces = sum_pieces(s.rows, s.cols);
+            j.blocks = j.pieces * (int)((s.cols + 127) / 128);
+        } else {
+            while (j.G < 32 && j.G < s.cols / 16) j.G <<= 1;
+            const int64_t groups = kThreads / j.G;
+            j.blocks = (int)std::max<int64_t>(1, std::min<int64_t>((s.rows + groups - 1) / groups, 4ll * sm_count()));
+        }
+        first += j.blocks;
+    }
+    J.count = count;
+    if (first == 0) return QBP_OK;
+    QBP_TRACE_BEGIN(st);
+    launch(code_sums_kernel, first, kThreads, 0, st, J);
+    QBP_LAUNCH_OK("code_sums_kernel");
+    return QBP_OK;
+}
+
 // One wave: `bps` resident blocks per SM (the kernel's occupancy), never more blocks than work groups.
 static int grid_for(int bps, int64_t n_groups)
 {

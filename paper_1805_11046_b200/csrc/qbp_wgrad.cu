@@ -86,8 +86,8 @@ struct WgradParams {
     int64_t M, N, K;
     long long *part;                 // int64 partials, one block of part_stride values per CTA
     int64_t part_stride;             // ma * 128 * bn, padded
-    // direct epilogue (plain): acc = raw + rowterm[k] + colterm[n]
-    const long long *rowterm, *colterm;
+    // plain product: code sums over the M rows (acc = raw - zg * sx[k] - zx * (256 * shi[n] + slo[n]) + M * zx * zg)
+    CodeSums sx, shi, slo;
     const qbp_qparams *qx, *qg;
     long long *acc_out; float *dW;
     int dW_vec;                      // dW starts on a 16-byte boundary
@@ -543,13 +543,16 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
         }
         if (P.direct) {
             const int t = threadIdx.x - 64;
-            if (t < P.bn) s_cterm[t] = (int64_t)n0 + t < P.N ? P.colterm[n0 + t] : 0;
+            const long long zx = P.qx->zero_point;
+            if (t < P.bn) s_cterm[t] = (int64_t)n0 + t < P.N ? -zx * (256 * P.shi.at(n0 + t) + P.slo.at(n0 + t)) : 0;
             named_barrier(3, 128);
         }
         if (k_iters > 0 && !mbar_wait_warp(&acc_bar, 0)) timed_out = true;
         tc_fence_after();
         if (!timed_out && k_iters > 0) {
             const float scale = P.direct ? __fmul_rn(P.qx->scale, P.qg->scale) : 0.0f;
+            // (signed low bytes: the limbs hold g16 - 128, against the zero-point zg - 128)
+            const long long zg_d = P.direct ? P.qg->zero_point - (P.lo_signed ? 128 : 0) : 0, zz_d = P.direct ? P.M * P.qx->zero_point * zg_d : 0;
             long long *part = P.part + (int64_t)blockIdx.x * P.part_stride;
             for (int j = 0; j < n_tiles; ++j) {
                 const int at = ag * P.ma + j;
@@ -557,7 +560,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
                 const int64_t k = (int64_t)at * 128 + row;                  // plain: output row
                 if (!P.conv) valid = valid && k < P.K;
                 else         valid = valid && (at % P.tiles_c) * P.rb_a + row % P.rb_a < P.C;
-                const long long rterm = (P.direct && valid) ? P.rowterm[k] : 0;
+                const long long rterm = (P.direct && valid) ? -zg_d * P.sx.at(k) + zz_d : 0;
                 const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(j * 2 * P.bn);
                 for (int c0 = 0; c0 < P.bn; c0 += 32) {
                     uint32_t rh[32], rl[32];
@@ -891,26 +894,11 @@ __global__ void __launch_bounds__(256) border_class_sums_kernel(const uint8_t *_
         if (s_acc[i] != 0) atomicAdd(&sums[i], (unsigned long long)(long long)s_acc[i]);
 }
 
-// Plain product, direct epilogue: rowterm[k] = -zg * SX[k] + M*zx*zg, colterm[n] = -zx * (256*SHI[n] + SLO[n]).
-__global__ void wgrad_terms_kernel(const long long *__restrict__ sx, const long long *__restrict__ shi,
-                                   const long long *__restrict__ slo, int64_t M, int64_t N, int64_t K,
-                                   const qbp_qparams *qx, const qbp_qparams *qg, long long *__restrict__ rowterm,
-                                   long long *__restrict__ colterm, int zg_shift)
-{
-    pdl_enter();
-    const long long zx = qx->zero_point, zg = qg->zero_point - zg_shift;      // (signed low bytes: lo - 128 against zg - 128)
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < K) rowterm[i] = -zg * sx[i] + M * zx * zg;
-    if (i < N) colterm[i] = -zx * (256 * shi[i] + slo[i]);
-}
-
 // Adds the CTAs' partials, applies the zero-points and dequantises:
 //   acc = raw - zg * SX - zx * SG + count * zx * zg
 // Plain product [k][n]: SX / SG are the column sums, count = M.  kWgFinalizeLanes lanes per output element share its slices (an
 // element's partials are few hundred bytes each, far apart: one thread walking them alone is bound by latency).
-__global__ void __launch_bounds__(256) wgrad_finalize_kernel(const WgradParams P, const long long *__restrict__ sx,
-                                                             const long long *__restrict__ shi,
-                                                             const long long *__restrict__ slo, int64_t total)
+__global__ void __launch_bounds__(256) wgrad_finalize_kernel(const __grid_constant__ WgradParams P, int64_t total)
 {
     pdl_enter();
     constexpr int kLanes = kWgFinalizeLanes;
@@ -923,7 +911,6 @@ __global__ void __launch_bounds__(256) wgrad_finalize_kernel(const WgradParams P
     const int64_t k = e / P.N;
     const int n = (int)(e % P.N);
     const int at = (int)(k / 128), row = (int)(k % 128);  // accumulator tile, row in it
-    const long long SX = sx[k], SG = 256 * shi[n] + slo[n];
     // the CTAs of this element's item
     const int ag = at / P.ma, j = at % P.ma, tb = n / P.bn, col = n % P.bn;
     const int item = ag * P.tiles_b + tb;
@@ -944,6 +931,7 @@ __global__ void __launch_bounds__(256) wgrad_finalize_kernel(const WgradParams P
 #pragma unroll
     for (int o = 1; o < kLanes; o <<= 1) raw += __shfl_xor_sync(0xffffffffu, raw, o);
     if (!live || part_lane != 0) return;
+    const long long SX = P.sx.at(k), SG = 256 * P.shi.at(n) + P.slo.at(n);
     const long long acc = raw - zg * SX - zx * SG + P.M * zx * zg;
     if (P.acc_out) P.acc_out[e] = acc;
     if (P.dW) P.dW[e] = __fmul_rn((float)acc, __fmul_rn(P.qx->scale, P.qg->scale));
@@ -979,7 +967,7 @@ __device__ __forceinline__ long long wg_class_part(const WgradParams &P, bool of
 // this kernel 78 us for a 256 -> 256 channel 3x3 filter, five times what its partials take to read), four groups
 // of 64 threads share the slices, each thread with eight loads in flight, and meet in shared memory.
 template <int NB>
-__global__ void __launch_bounds__(256) wgrad_conv_finalize_kernel(const WgradParams P, const long long *__restrict__ sx,
+__global__ void __launch_bounds__(256) wgrad_conv_finalize_kernel(const __grid_constant__ WgradParams P, const long long *__restrict__ sx,
                                                                   const long long *__restrict__ shi,
                                                                   const long long *__restrict__ slo)
 {
@@ -1218,9 +1206,8 @@ static void plan_wgrad(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, 
 
 static size_t wgrad_ws_bytes(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K)
 {
-    const int64_t cx = d ? d->C : K, cg = d ? d->K : N;
-    const size_t sums = align_up(sizeof(int64_t) * 16 * cx, 256) + 2 * align_up(sizeof(int64_t) * 16 * cg, 256);
-    const size_t terms = align_up(sizeof(int64_t) * cx, 256) + align_up(sizeof(int64_t) * cg, 256);
+    const size_t sums = d ? align_up(sizeof(int64_t) * 16 * (size_t)d->C, 256) + 2 * align_up(sizeof(int64_t) * 16 * (size_t)d->K, 256)
+                          : align_up(sizeof(int32_t) * sum_elems(M, K, true), 256) + 2 * align_up(sizeof(int32_t) * sum_elems(M, N, true), 256);
     // (the split, and with it the partials, may differ between the two forms of the low limb: room for either)
     size_t part = 0;
     for (int lo_signed = 0; lo_signed < 2; ++lo_signed) {
@@ -1228,7 +1215,7 @@ static size_t wgrad_ws_bytes(const qbp_conv_desc *d, int64_t M, int64_t N, int64
         plan_wgrad(d, M, N, K, pl, lo_signed != 0);
         part = std::max(part, pl.P.direct ? (size_t)0 : align_up(sizeof(int64_t) * (size_t)pl.grid * (size_t)pl.P.part_stride, 256));
     }
-    return 256 + sums + terms + part;
+    return 256 + sums + part;
 }
 
 template <bool IS_SIGNED>
@@ -1320,11 +1307,10 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
     WsCarver w(ws, ws_bytes);
     int *status = w.take<int>(1);
     if (ext_status) status = ext_status;         // the caller's sticky word: raised here, never cleared
-    int64_t *sx = w.take<int64_t>(16 * K);
-    int64_t *shi = w.take<int64_t>(16 * N);
-    int64_t *slo = w.take<int64_t>(16 * N);
-    int64_t *rowterm = w.take<int64_t>(K);
-    int64_t *colterm = w.take<int64_t>(N);
+    int64_t *sx = nullptr, *shi = nullptr, *slo = nullptr;       // convolution: per border class
+    SumJob jobs[3] = {{x, M, K, 1, 1, nullptr}, {g_hi, M, N, 1, 1, nullptr}, {g_lo, M, N, 1, lo_signed ? 1 : 0, nullptr}};
+    if (d) { sx = w.take<int64_t>(16 * K); shi = w.take<int64_t>(16 * N); slo = w.take<int64_t>(16 * N); }
+    else for (SumJob &j : jobs) j.out = w.take<int32_t>(sum_elems(j.rows, j.cols, true));
     int64_t *part = P.direct ? nullptr : w.take<int64_t>((size_t)pl.grid * (size_t)P.part_stride);
 
     // large plain products run on CTA pairs (256 x 256 tiles across two SMs, the whole reduction in one pair)
@@ -1377,25 +1363,14 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
         if ((rc = lo_signed ? launch_class_sums<true>(g_lo, M, d->H, d->W, (int)N, slo, st)
                             : launch_class_sums<false>(g_lo, M, d->H, d->W, (int)N, slo, st))) return rc;
     } else {
-        if ((rc = launch_colsum(x, true, M, K, sx, st))) return rc;
-        if ((rc = launch_colsum(g_hi, true, M, N, shi, st))) return rc;
-        if ((rc = launch_colsum(g_lo, lo_signed, M, N, slo, st))) return rc;
-        if (P.direct || pair_kernel) {
-            const int64_t mx = std::max(K, N);
-            QBP_TRACE_BEGIN(st);
-            launch(wgrad_terms_kernel, (unsigned)((mx + 255) / 256), 256, 0, st, (const long long *)sx, (const long long *)shi,
-                                                                            (const long long *)slo, M, N, K, qx, qg16,
-                                                                            (long long *)rowterm, (long long *)colterm, lo_signed ? 128 : 0);
-            QBP_LAUNCH_OK("wgrad_terms_kernel");
-        }
+        if ((rc = launch_code_sums(jobs, 3, st))) return rc;
+        P.sx = sums_of(jobs[0]); P.shi = sums_of(jobs[1]); P.slo = sums_of(jobs[2]);
     }
     if (!ext_status) QBP_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
     if (pair_kernel)
-        return launch_wgrad2(M, N, K, x, qx, g_hi, g_lo, qg16, acc_out, dW, (const long long *)rowterm,
-                             (const long long *)colterm, status, st, lo_signed);
+        return launch_wgrad2(M, N, K, x, qx, g_hi, g_lo, qg16, acc_out, dW, P.sx, P.shi, P.slo, status, st, lo_signed);
 
     P.part = (long long *)part; P.status = status;
-    P.rowterm = (const long long *)rowterm; P.colterm = (const long long *)colterm;
     P.qx = qx; P.qg = qg16; P.acc_out = (long long *)acc_out; P.dW = dW; P.dW_vec = aligned16(dW) ? 1 : 0;
     const uint32_t kr = (uint32_t)P.kr, rb_a = (uint32_t)P.rb_a, rb_b = (uint32_t)P.bn;
     if (!d) {
@@ -1440,7 +1415,7 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
     } else if (!P.direct) {
         const int blocks = (int)((outs * kWgFinalizeLanes + 255) / 256);
         QBP_TRACE_BEGIN(st);
-        launch(wgrad_finalize_kernel, blocks, 256, 0, st, P, (const long long *)sx, (const long long *)shi, (const long long *)slo, outs);
+        launch(wgrad_finalize_kernel, blocks, 256, 0, st, P, outs);
         QBP_LAUNCH_OK("wgrad_finalize_kernel");
     }
     return QBP_OK;

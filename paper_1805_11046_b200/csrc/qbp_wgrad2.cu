@@ -42,7 +42,8 @@ struct Wgrad2Params {
     FastDiv d_group;
     int64_t M, N, K;                 // reduction rows; output columns; output rows
     long long *acc_out; float *dW;
-    const long long *rowterm, *colterm;
+    CodeSums sx, shi, slo;           // code sums over the M rows: rowterm = -zg * sx[k] + M * zx * zg, colterm = -zx * (256 * shi[n] + slo[n])
+    int zg_shift;                    // 128 for signed low bytes (lo - 128 against zg - 128)
     const qbp_qparams *qx, *qg;
     int *status;
 };
@@ -211,6 +212,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
         const int row = quad * 32 + lane;
         uint8_t *slab = staging + (size_t)ew * kW2Slab;
         const float scale = __fmul_rn(P.qx->scale, P.qg->scale);
+        const long long zx = P.qx->zero_point, zg = P.qg->zero_point - P.zg_shift;
         const uint32_t leader_empty = w2_map_to_cta(&acc_empty, 0);
         uint32_t fph = 0;
         for (int tile = pair; tile < P.tiles_total; tile += P.pairs) {
@@ -218,8 +220,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
             const int64_t k = (int64_t)o.k0 + 128 * (int)rank + row;                  // output row
             const bool valid = k < P.K;
             const bool slab_in = (int64_t)o.k0 + 128 * (int)rank + quad * 32 < P.K;
-            const long long rterm = valid ? P.rowterm[k] : 0;
+            const long long rterm = valid ? -zg * P.sx.at(k) + P.M * zx * zg : 0;
             const int64_t ncol = P.N - o.n0;
+            // lane l takes the column terms of column l of this warp's four chunks, while the MMAs run
+            long long ct[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int n = (half * 4 + i) * 32 + lane;
+                ct[i] = n < ncol ? -zx * (256 * P.shi.at(o.n0 + n) + P.slo.at(o.n0 + n)) : 0;
+            }
             const int nchunks = (int)((ncol < 256 ? ncol : 256) + 31) / 32;
             if (!timed_out && !mbar_wait_warp(&acc_full, fph)) timed_out = true;
             fph ^= 1u;
@@ -245,8 +254,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
                         if (lane == 0) w2_arrive_cluster(leader_empty);
                     }
                     const int lim = (int)(ncol - c0 < 32 ? ncol - c0 : 32);
-                    // lane l fetches the column term of column c0 + l; the row's 32 sums take them by shuffle
-                    const long long my_cterm = lane < lim ? __ldg(P.colterm + o.n0 + c0 + lane) : 0;
+                    // (lane l holds the column term of column c0 + l; the row's 32 sums take them by shuffle)
+                    const int ci = c - c_begin;
+                    const long long my_cterm = ci == 0 ? ct[0] : ci == 1 ? ct[1] : ci == 2 ? ct[2] : ct[3];
                     if (P.dW) {
                         if (lane == 0) tma_store_wait_read();
                         __syncwarp();
@@ -311,8 +321,8 @@ bool wgrad2_eligible(int64_t M, int64_t N, int64_t K)
 }
 
 int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qparams *qx, const int8_t *g_hi,
-                  const uint8_t *g_lo, const qbp_qparams *qg16, int64_t *acc_out, float *dW, const long long *rowterm,
-                  const long long *colterm, int *status, cudaStream_t st, bool lo_signed)
+                  const uint8_t *g_lo, const qbp_qparams *qg16, int64_t *acc_out, float *dW, const CodeSums &sx,
+                  const CodeSums &shi, const CodeSums &slo, int *status, cudaStream_t st, bool lo_signed)
 {
     Wgrad2Params P{};
     int rc;
@@ -332,7 +342,7 @@ int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qp
     P.d_group = make_fastdiv(kW2GroupM * P.tiles_n);
     P.M = M; P.N = N; P.K = K;
     P.acc_out = (long long *)acc_out; P.dW = dW;
-    P.rowterm = rowterm; P.colterm = colterm; P.qx = qx; P.qg = qg16; P.status = status;
+    P.sx = sx; P.shi = shi; P.slo = slo; P.zg_shift = lo_signed ? 128 : 0; P.qx = qx; P.qg = qg16; P.status = status;
     static PerDeviceOnce configured;
     QBP_SMEM_OPT_IN(configured, qbp_wgrad2_kernel, kW2Smem);
     QBP_TRACE_BEGIN(st);
