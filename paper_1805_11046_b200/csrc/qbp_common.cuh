@@ -42,11 +42,9 @@ void trace_end(const char *name, cudaStream_t st);
 // before: launch() marks every kernel as a programmatic dependent of its predecessor, each kernel says at its start that
 // its successor may be scheduled (pdl_trigger: the successor's blocks then take the slots that come free) and waits,
 // before it touches global memory, until the predecessor has completed and its writes are visible (pdl_wait).  A chain of
-// dependent small kernels then costs about 2 us each instead of 4 to 5.  While launches are timed one by one, and for the
-// first kernel after a join with another stream (launch_next_in_full), the dependency is the ordinary one.
+// dependent small kernels then costs about 2 us each instead of 4 to 5.  While launches are timed one by one the dependency
+// is the ordinary one.
 bool trace_is_on();
-inline bool &full_dependency_next() { thread_local bool f = false; return f; }
-inline void launch_next_in_full() { full_dependency_next() = true; }
 template <typename... P, typename... A>
 inline void launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A &&...args)
 {
@@ -56,8 +54,7 @@ inline void launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t sme
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = (full_dependency_next() || trace_is_on()) ? 0 : 1;
-    full_dependency_next() = false;
+    cfg.numAttrs = trace_is_on() ? 0 : 1;
     (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);     // (an error is found by QBP_LAUNCH_OK)
 }
 
@@ -101,6 +98,14 @@ struct WsCarver {
     }
     bool ok() const { return base != nullptr && off <= cap; }
 };
+
+// Where a kernel that quantises per tensor takes its range from: the (min, max) pairs that the kernel before left (per block or
+// per channel; `parts`), clamping values the caller gave (`given`), or -- both NULL -- finished records at qp8 / qp16.  In the
+// first two cases every block works out the parameters itself (about a microsecond, most of it behind its first loads;
+// a launch of its own for it costs two and more) and the first block leaves the records at qp8 / qp16 (each nullable).
+struct RangeSrc { const float2 *parts; int nparts; const qbp_qparams *given; qbp_qparams *qp8, *qp16; };
+// Regions of 32-bit words that a kernel clears on the way (a status word, sums that a later kernel adds to).
+struct ZeroJobs { uint32_t *p[2]; int64_t words[2]; };
 
 // -------------------------------------------------------------- device side
 #ifdef __CUDACC__
@@ -269,6 +274,60 @@ __device__ __forceinline__ float warp_max(float v)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
+}
+
+// The whole block's (min, max) of per-thread values (threads a multiple of 32, at most 1024; once per kernel).
+__device__ __forceinline__ float2 block_min_max(float lo, float hi)
+{
+    __shared__ float2 s_red[32];
+    lo = warp_min(lo); hi = warp_max(hi);
+    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = make_float2(lo, hi);
+    __syncthreads();
+    float2 r = s_red[0];
+    for (unsigned w = 1; w < blockDim.x / 32; ++w) { const float2 t = s_red[w]; r.x = fminf(r.x, t.x); r.y = fmaxf(r.y, t.y); }
+    return r;
+}
+// ... of (min, max) pairs in memory.
+__device__ __forceinline__ float2 block_range(const float2 *__restrict__ parts, int nparts)
+{
+    float lo = INFINITY, hi = -INFINITY;
+    for (int i = threadIdx.x; i < nparts; i += blockDim.x) { const float2 t = __ldg(parts + i); lo = fminf(lo, t.x); hi = fmaxf(hi, t.y); }
+    return block_min_max(lo, hi);
+}
+// A thread's share of the clearing, `threads` threads taking part.
+__device__ __forceinline__ void run_zero_jobs(const ZeroJobs &z, int64_t thread, int64_t threads)
+{
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        for (int64_t i = thread; i < z.words[k]; i += threads) z.p[k][i] = 0u;
+}
+struct QParamsReg { float inv, zp_u; };       // 1 / scale and the unsigned zero-point
+__device__ __forceinline__ QParamsReg qparams_reg(const qbp_qparams &qp, int bits)
+{
+    QParamsReg r;
+    r.inv = __fdiv_rn(1.0f, qp.scale);
+    r.zp_u = (float)(qp.zero_point + (1 << (bits - 1)));
+    return r;
+}
+// The parameters of the copies that are wanted, by a whole block; `first`: the block that leaves the records.
+__device__ __forceinline__ void resolve_range(const RangeSrc &R, bool want8, bool want16, bool first, QParamsReg &p8, QParamsReg &p16)
+{
+    if (!R.parts && !R.given) {
+        if (want8) p8 = qparams_reg(*R.qp8, 8);
+        if (want16) p16 = qparams_reg(*R.qp16, 16);
+        return;
+    }
+    const float2 r = R.given ? make_float2(R.given->vmin, R.given->vmax) : block_range(R.parts, R.nparts);
+    if (want8) {
+        const qbp_qparams q = make_qparams(r.x, r.y, 8);
+        if (first && threadIdx.x == 0 && R.qp8) *R.qp8 = q;
+        p8 = qparams_reg(q, 8);
+    }
+    if (want16) {
+        const qbp_qparams q = make_qparams(r.x, r.y, 16);
+        if (first && threadIdx.x == 0 && R.qp16) *R.qp16 = q;
+        p16 = qparams_reg(q, 16);
+    }
 }
 
 // ---- sm_100a PTX wrappers ---------------------------------------------------

@@ -57,46 +57,9 @@ static int layer_shape(const qbp_layer_desc *L, LayerShape &s)
 // the steps share (they run one after another on the stream), then the buffers that live across steps.
 constexpr size_t kLayerHead = 256;
 
-// A small filter's kernels (one block each, some ten microseconds of latency) need the quantiser parameters of the
-// activation or gradient they are paired with, but not its codes: they run on a stream of the library's own beside
-// the pass that writes those codes, forked from the caller's stream after the parameters and joined before the
-// product.  One stream and two events per host thread and device, made at first use (a first call should therefore
-// come before any stream capture); when they cannot be made the kernels simply run in line.
-struct SideStream { cudaStream_t s; cudaEvent_t fork, join; bool ok; };
-static SideStream *side_stream()
-{
-    thread_local SideStream cache[kMaxDevices] = {};
-    thread_local bool tried[kMaxDevices] = {};
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
-    SideStream &c = cache[dev];
-    if (!tried[dev]) {
-        tried[dev] = true;
-        c.ok = cudaStreamCreateWithFlags(&c.s, cudaStreamNonBlocking) == cudaSuccess &&
-               cudaEventCreateWithFlags(&c.fork, cudaEventDisableTiming) == cudaSuccess &&
-               cudaEventCreateWithFlags(&c.join, cudaEventDisableTiming) == cudaSuccess;
-        if (!c.ok) (void)cudaGetLastError();
-    }
-    return c.ok ? &c : nullptr;
-}
-// Runs what the caller enqueues on `side` between the event `fork` (already recorded on st) and the rest of st.
-static int side_begin(SideStream *sd)
-{
-    QBP_CUDA_OK(cudaStreamWaitEvent(sd->s, sd->fork, 0));
-    launch_next_in_full();
-    return QBP_OK;
-}
-static int side_end(SideStream *sd, cudaStream_t st)
-{
-    QBP_CUDA_OK(cudaEventRecord(sd->join, sd->s));
-    QBP_CUDA_OK(cudaStreamWaitEvent(st, sd->join, 0));
-    launch_next_in_full();
-    return QBP_OK;
-}
-
 static size_t step_scratch_bytes(const qbp_layer_desc *L, const LayerShape &s)
 {
-    size_t b = qbp_quantize_workspace_bytes(s.rows, std::max(s.cin, s.cout), QBP_PER_TENSOR);
+    size_t b = std::max(quantize_operands_ws_bytes(), qbp_quantize_workspace_bytes(s.rows, std::max(s.cin, s.cout), QBP_PER_TENSOR));
     b = std::max(b, qbp_rangebn_workspace_bytes(s.rows, s.cout));
     if (s.conv) {
         b = std::max(b, qbp_conv_s8_workspace_bytes(QBP_CONV_FPROP, &L->conv));
@@ -108,34 +71,53 @@ static size_t step_scratch_bytes(const qbp_layer_desc *L, const LayerShape &s)
     return align_up(b, 256);
 }
 
-// Buffers that live across steps, behind the shared step scratch: the per-row sums of the codes feeding the
-// next product (written by the quantiser that makes the codes) and the range partials of the gradient
-// (written by the Range BN backward pass that makes the gradient).
 // (a convolution's epilogue takes the output's per-channel statistics for any number of channels that leaves a CTA one
 // column tile: 256 channels per tile, one CTA per SM)
 static bool epilogue_stats(const LayerShape &s) { return s.conv && (s.cout + 255) / 256 <= sm_count(); }
 static size_t colstat_cells(const LayerShape &s) { return epilogue_stats(s) ? (size_t)colstat_rows_max() * (size_t)s.cout : 0; }
-static size_t chained_bytes(const LayerShape &s)
+// The layer's own pieces of the workspace, in order.
+struct LayerWs {
+    int *status;                 // byte 0 of the workspace
+    void *scratch; size_t scratch_bytes;
+    int32_t *row_sums;           // [rows] code sums of the operand of the next product
+    float2 *range_parts;         // range partials of the gradient
+    ColStatParts parts;          // per-channel (sum, min, max) partials of the output, from the convolution's epilogue
+    float4 *fold;                // per-channel constants of the normalisation, for the recompute fusion
+    int64_t *tot_g;              // [cout] per-channel totals of the 16-bit gradient codes, and behind them ...
+    int64_t *wg_table;           // ... the table of the weight gradient's sums (convolution): cleared together
+    int64_t clear_words;
+    int32_t *w_sums;             // the weights' code sums: forward, then layer gradient
+    SumJob wg_sums[6];           // the weight gradient's code sums (count: wg_count)
+    int wg_count;
+    size_t bytes;
+};
+static SumJob weight_sum_job(const qbp_layer_desc *L, const LayerShape &s, bool bwd, const int8_t *w, int32_t *out)
 {
-    // ... and the per-channel (sum, min, max) partials of the layer output that the convolution's epilogue leaves
-    // for the Range BN forward, and the per-channel constants of the normalisation for the recompute fusion
-    return align_up(sizeof(int32_t) * (size_t)s.rows, 256) + align_up(sizeof(float2) * rangebn_range_parts_capacity(s.cout), 256) +
-           2 * align_up(sizeof(float) * colstat_cells(s), 256) + align_up(sizeof(double) * colstat_cells(s), 256) +
-           align_up(sizeof(float4) * (size_t)s.cout, 256) + align_up(sizeof(int32_t) * 16 * (size_t)std::max(s.cin, s.cout), 256) +
-           align_up(sizeof(int64_t) * (size_t)s.cout, 256);
+    if (s.conv) return filter_sum_job(&L->conv, bwd, w, out);
+    return bwd ? SumJob{w, s.cin, s.cout, kSumRows, 1, out} : SumJob{w, s.cin, s.cout, kSumCols, 1, out};
 }
-// The forward column terms that come with the filter's codes (the piece before the last of the region above).
-static int32_t *colterm_buffer(const qbp_layer_desc *L, const LayerShape &s, void *ws_after_head)
+static LayerWs layer_ws(const qbp_layer_desc *L, const LayerShape &s, void *ws, const int8_t *x = nullptr, const int8_t *hi = nullptr,
+                        const uint8_t *lo = nullptr)
 {
-    return reinterpret_cast<int32_t *>(static_cast<char *>(ws_after_head) + step_scratch_bytes(L, s) + chained_bytes(s) -
-                                       align_up(sizeof(int64_t) * (size_t)s.cout, 256) -
-                                       align_up(sizeof(int32_t) * 16 * (size_t)std::max(s.cin, s.cout), 256));
-}
-// The per-channel totals of the 16-bit gradient codes (last piece of the region above).
-static int64_t *tot_g_buffer(const qbp_layer_desc *L, const LayerShape &s, void *ws_after_head)
-{
-    return reinterpret_cast<int64_t *>(static_cast<char *>(ws_after_head) + step_scratch_bytes(L, s) + chained_bytes(s) -
-                                       align_up(sizeof(int64_t) * (size_t)s.cout, 256));
+    LayerWs l{};
+    WsCarver c(ws, SIZE_MAX);
+    l.status = c.take<int>(kLayerHead / sizeof(int));
+    l.scratch_bytes = step_scratch_bytes(L, s);
+    l.scratch = c.take<char>(l.scratch_bytes);
+    l.row_sums = c.take<int32_t>((size_t)s.rows);
+    l.range_parts = c.take<float2>(rangebn_range_parts_capacity(s.cout));
+    const size_t cells = colstat_cells(s);
+    if (cells) { l.parts.lo = c.take<float>(cells); l.parts.hi = c.take<float>(cells); l.parts.sum = c.take<double>(cells); }
+    l.fold = c.take<float4>((size_t)s.cout);
+    const qbp_conv_desc *d = s.conv ? &L->conv : nullptr;
+    l.tot_g = c.take<int64_t>((size_t)s.cout + wgrad_sum_table(d));
+    l.wg_table = l.tot_g + s.cout;
+    l.clear_words = 2 * ((int64_t)s.cout + (int64_t)wgrad_sum_table(d));
+    l.w_sums = c.take<int32_t>(std::max(sum_elems(weight_sum_job(L, s, false, nullptr, nullptr)), sum_elems(weight_sum_job(L, s, true, nullptr, nullptr))));
+    l.wg_count = wgrad_sum_jobs(d, s.rows, s.cout, s.cin, x, hi, lo, true, d ? l.wg_table : nullptr, l.wg_sums);
+    for (int i = 0; i < l.wg_count && !d; ++i) l.wg_sums[i].out = c.take<int32_t>(sum_elems(l.wg_sums[i]));
+    l.bytes = c.off;
+    return l;
 }
 
 // Recompute instead of store (motivated by Section 7's memory and bandwidth argument): convolution -> Range BN
@@ -145,16 +127,16 @@ static int64_t *tot_g_buffer(const qbp_layer_desc *L, const LayerShape &s, void 
 static int conv_rangebn_recompute(const qbp_conv_desc *d, const int8_t *x_codes, const qbp_qparams *qx, const int32_t *in_sums,
                                   const int8_t *w_codes, const qbp_qparams *qw, const float *gamma, const float *beta, int relu,
                                   float *save_mean, float *save_min, float *save_max, const qbp_requant *out,
-                                  ColStatParts parts, float4 *fold, const int32_t *colterm, int *status, void *ws, size_t scratch,
+                                  ColStatParts parts, float4 *fold, const CodeSums &w_sums, int *status, void *ws, size_t scratch,
                                   cudaStream_t st)
 {
     const int64_t rows = (int64_t)d->N * d->H * d->W;
-    const EpilogueTail first{nullptr, 0, nullptr, nullptr, nullptr, 0, colterm};
+    const EpilogueTail first{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums};
     int rc = conv_s8_impl(QBP_CONV_FPROP, d, x_codes, qx, w_codes, qw, nullptr, nullptr, in_sums, &parts, status, ws, scratch, st,
-                          colterm ? &first : nullptr);
+                          &first);
     if (rc) return rc;
     if ((rc = rangebn_fold_from_parts(rows, d->K, gamma, beta, relu, save_mean, save_min, save_max, parts, out->qp, fold, st))) return rc;
-    const EpilogueTail tail{fold, relu, out->qp, out->q, out->row_sums, 1, colterm};
+    const EpilogueTail tail{fold, relu, out->qp, out->q, out->row_sums, 1, &w_sums};
     rc = conv_s8_impl(QBP_CONV_FPROP, d, x_codes, qx, w_codes, qw, nullptr, nullptr, in_sums, nullptr, status, ws, scratch, st, &tail);
     if (rc || !out->chan_sums) return rc;
     return launch_colsum(out->q, true, rows, d->K, out->chan_sums, st);
@@ -168,7 +150,7 @@ extern "C" __attribute__((visibility("default"))) size_t qbp_layer_workspace_byt
 {
     LayerShape s;
     if (layer_shape(L, s)) return 0;
-    return kLayerHead + step_scratch_bytes(L, s) + chained_bytes(s);
+    return layer_ws(L, s, nullptr).bytes;
 }
 
 extern "C" __attribute__((visibility("default"))) int qbp_layer_fwd(const qbp_layer_desc *L, const float *x,
@@ -210,78 +192,53 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_fwd_chained(cons
     if (want_totals && s.rows >= (1ll << 22)) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "layer_fwd: x_chan_sums for fewer than 2^22 positions");
     if (want_totals && in && in->chan_sums && in->chan_sums != saved->x_chan_sums)
         return fail(QBP_ERR_INVALID_ARG, "layer_fwd: in->chan_sums must be the layer's saved x_chan_sums");
-    if (!ws || ws_bytes < qbp_layer_workspace_bytes(L))
-        return fail(QBP_ERR_WORKSPACE, "layer_fwd: workspace of %zu bytes needed, %zu given",
-                    qbp_layer_workspace_bytes(L), ws_bytes);
-    const size_t scratch = step_scratch_bytes(L, s);
+    const LayerWs l = layer_ws(L, s, ws);
+    if (!ws || ws_bytes < l.bytes)
+        return fail(QBP_ERR_WORKSPACE, "layer_fwd: workspace of %zu bytes needed, %zu given", l.bytes, ws_bytes);
     cudaStream_t st = (cudaStream_t)stream;
-    int *status = static_cast<int *>(ws);
-    QBP_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
-    ws = static_cast<char *>(ws) + kLayerHead;
+    int *status = l.status;
 
     // activations: nearest rounding, clamping values = min and max (Appendix B) -- or already quantised by the
-    // Range BN of the layer before (Section 4)
-    // (convolution: each pixel's code sum is needed for the zero-point correction of the product)
-    int32_t *row_sums = reinterpret_cast<int32_t *>(static_cast<char *>(ws) + scratch);
-    const int32_t *in_sums = s.conv ? row_sums : nullptr;
-    // (a small filter's launch runs beside the pass that writes the input codes)
-    const bool small_filter = s.conv && L->conv.R == 3 && filter_prep_supported(&L->conv, w, saved->w_codes);
-    SideStream *sd = (x && small_filter) ? side_stream() : nullptr;
-    if (x) {
-        bool left = false;
-        rc = quantize_s8_with_totals(x, s.rows, s.cin, saved->x_codes, saved->qx, s.conv ? row_sums : nullptr,
-                                     want_totals ? saved->x_chan_sums : nullptr, &left, ws, scratch, st, sd ? sd->fork : nullptr);
-        if (rc) return rc;
-        // (a shape the quantiser cannot take the totals of: one pass over the codes)
-        if (want_totals && !left && (rc = launch_colsum(saved->x_codes, true, s.rows, s.cin, saved->x_chan_sums, st))) return rc;
-    } else if (s.conv) {
-        if (in->row_sums) in_sums = in->row_sums;
-        else if ((rc = launch_rowsum(in->q, true, s.rows, s.cin, row_sums, st))) return rc;
-        if (want_totals && !in->chan_sums && (rc = launch_colsum(in->q, true, s.rows, s.cin, saved->x_chan_sums, st))) return rc;
-    }
-    // weights: nearest rounding, clamping values = min and max (a small filter: scan, codes, code sums and the forward
-    // product's column terms in one launch)
+    // Range BN of the layer before (Section 4); weights the same.  (the first launch also clears the status word)
     const int64_t w_rows = s.conv ? (int64_t)L->conv.K * L->conv.R * L->conv.S : s.cin;
-    const int32_t *colterm = nullptr;
-    if (small_filter) {
-        int32_t *ct = colterm_buffer(L, s, ws);
-        if (sd && (rc = side_begin(sd))) return rc;
-        if ((rc = launch_filter_prep(&L->conv, w, saved->qx, saved->w_codes, saved->qw, ct, sd ? sd->s : st))) return rc;
-        if (sd && (rc = side_end(sd, st))) return rc;
-        colterm = ct;
-    } else {
-        rc = qbp_quantize_s8(w, w_rows, s.w_elems / w_rows, QBP_PER_TENSOR, QBP_ROUND_NEAREST, 0, 0, nullptr,
-                             saved->w_codes, saved->qw, nullptr, nullptr, ws, scratch, stream);
-        if (rc) return rc;
-    }
-    const EpilogueTail with_colterm{nullptr, 0, nullptr, nullptr, nullptr, 0, colterm};
-    ColStatParts parts{nullptr, nullptr, nullptr, 0};
-    if (epilogue_stats(s)) {
-        char *base = static_cast<char *>(ws) + scratch + align_up(sizeof(int32_t) * (size_t)s.rows, 256) +
-                     align_up(sizeof(float2) * rangebn_range_parts_capacity(s.cout), 256);
-        parts.lo = reinterpret_cast<float *>(base);
-        parts.hi = reinterpret_cast<float *>(base + align_up(sizeof(float) * colstat_cells(s), 256));
-        parts.sum = reinterpret_cast<double *>(base + 2 * align_up(sizeof(float) * colstat_cells(s), 256));
-    }
-    if (recompute) {
-        float4 *fold = reinterpret_cast<float4 *>(reinterpret_cast<char *>(parts.sum) + align_up(sizeof(double) * colstat_cells(s), 256));
+    QuantOperand xo{x, s.rows, s.cin, saved->x_codes, saved->qx, l.row_sums, want_totals ? saved->x_chan_sums : nullptr};
+    QuantOperand wo{w, w_rows, s.w_elems / w_rows, saved->w_codes, saved->qw, s.conv ? l.w_sums : nullptr, nullptr};
+    // (an input that came without its channel totals: cleared with the rest, summed up below; a filter has cin columns)
+    const bool chained_totals = !x && want_totals && !in->chan_sums;
+    if (chained_totals) wo.tot = saved->x_chan_sums;
+    if ((rc = quantize_operands(x ? &xo : nullptr, &wo, status, l.scratch, l.scratch_bytes, st))) return rc;
+    // what the products need beside the codes: each input row's code sum (convolution: each pixel's), the weights' sums,
+    // each input channel's total -- whatever the quantising kernel did not leave, in one launch
+    SumJob jobs[3];
+    int njobs = 0;
+    const int32_t *in_sums = l.row_sums;
+    if (in && in->row_sums) in_sums = in->row_sums;
+    else if (!xo.row_sums_left) jobs[njobs++] = SumJob{saved->x_codes, s.rows, s.cin, kSumRows, 1, l.row_sums};
+    const SumJob w_job = weight_sum_job(L, s, false, saved->w_codes, l.w_sums);
+    if (!wo.row_sums_left) jobs[njobs++] = w_job;
+    if ((want_totals && x && !xo.tot_left) || chained_totals)
+        jobs[njobs++] = SumJob{saved->x_codes, s.rows, s.cin, kSumCols, 1, nullptr, 0, 0, saved->x_chan_sums};
+    if (njobs && (rc = launch_code_sums(jobs, njobs, st))) return rc;
+    const CodeSums w_sums = sums_of(w_job), x_sums = sums_of(in_sums);
+    ColStatParts parts = l.parts;
+    if (recompute)
         return conv_rangebn_recompute(&L->conv, saved->x_codes, saved->qx, in_sums, saved->w_codes, saved->qw, gamma, beta, L->relu,
-                                      saved->save_mean, saved->save_min, saved->save_max, out, parts, fold, colterm, status, ws,
-                                      scratch, st);
-    }
+                                      saved->save_mean, saved->save_min, saved->save_max, out, parts, l.fold, w_sums, status,
+                                      l.scratch, l.scratch_bytes, st);
+    const EpilogueTail with_sums{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums};
     if (s.conv)
         rc = conv_s8_impl(QBP_CONV_FPROP, &L->conv, saved->x_codes, saved->qx, saved->w_codes, saved->qw, nullptr, saved->z,
-                          in_sums, parts.sum ? &parts : nullptr, status, ws, scratch, st, colterm ? &with_colterm : nullptr);
+                          in_sums, parts.sum ? &parts : nullptr, status, l.scratch, l.scratch_bytes, st, &with_sums);
     else
         rc = gemm_s8_impl(0, 0, s.rows, s.cout, s.cin, saved->x_codes, saved->qx, saved->w_codes, saved->qw, nullptr,
-                          saved->z, nullptr, status, ws, scratch, st);
+                          saved->z, nullptr, status, l.scratch, l.scratch_bytes, st, &x_sums, &w_sums);
     if (rc) return rc;
     // the convolution's epilogue has left the statistics of z: no pass over z for them
     if (parts.sum)
         return rangebn_fwd_from_parts(saved->z, s.rows, s.cout, gamma, beta, L->relu, y, saved->save_mean, saved->save_min,
                                       saved->save_max, parts, nullptr, out, st);
     return qbp_rangebn_fwd_q8(saved->z, s.rows, s.cout, gamma, beta, L->relu, y, saved->save_mean, saved->save_min,
-                              saved->save_max, nullptr, out, ws, scratch, stream);
+                              saved->save_max, nullptr, out, l.scratch, l.scratch_bytes, stream);
 }
 
 extern "C" __attribute__((visibility("default"))) int qbp_layer_bwd(const qbp_layer_desc *L, const qbp_layer_ctx *saved,
@@ -294,33 +251,35 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_bwd(const qbp_la
     int rc = layer_shape(L, s);
     if (rc) return rc;
     if (!saved || !dy || !dx || !dw) return fail(QBP_ERR_INVALID_ARG, "layer_bwd: NULL argument");
-    if (!ws || ws_bytes < qbp_layer_workspace_bytes(L))
-        return fail(QBP_ERR_WORKSPACE, "layer_bwd: workspace of %zu bytes needed, %zu given",
-                    qbp_layer_workspace_bytes(L), ws_bytes);
     if (!saved->g8 || !saved->qg8 || !saved->g_hi || !saved->g_lo || !saved->qg16 || !saved->z)
         return fail(QBP_ERR_INVALID_ARG, "layer_bwd: the saved-state record has a NULL buffer (the backward pass needs z and the gradient buffers)");
-    const size_t scratch = step_scratch_bytes(L, s);
     float *g = saved->g;
     int8_t *g8 = saved->g8, *ghi = saved->g_hi;
     uint8_t *glo = saved->g_lo;
     qbp_qparams *qp8 = saved->qg8, *qp16 = saved->qg16;
+    const LayerWs l = layer_ws(L, s, ws, saved->x_codes, ghi, glo);
+    if (!ws || ws_bytes < l.bytes)
+        return fail(QBP_ERR_WORKSPACE, "layer_bwd: workspace of %zu bytes needed, %zu given", l.bytes, ws_bytes);
 
     cudaStream_t st = (cudaStream_t)stream;
-    int *status = static_cast<int *>(ws);          // the forward call cleared it; the backward only ever raises it
-    ws = static_cast<char *>(ws) + kLayerHead;
-    int32_t *row_sums = reinterpret_cast<int32_t *>(static_cast<char *>(ws) + scratch);
-    float2 *range_parts = reinterpret_cast<float2 *>(static_cast<char *>(ws) + scratch + align_up(sizeof(int32_t) * (size_t)s.rows, 256));
+    int *status = l.status;                        // the forward call cleared it; the backward only ever raises it
     // two copies of the gradient: 8 bits for the layer gradient, 16 bits for the weight gradient
     // (convolution with the input's per-channel code totals at hand: the bifurcation leaves the gradient's, and the
-    // weight gradient reads only the border positions again for its zero-point terms)
+    // weight gradient reads only the edges of the images again for its zero-point terms)
     // ... and when the weight-gradient product has a spare chunk of MMA rows, it takes the gradient's totals itself
     const bool self_totals = s.conv && saved->x_chan_sums && wgrad_self_totals(&L->conv) && s.rows < (1ll << 22);
     const bool totals = s.conv && saved->x_chan_sums && (self_totals || quantizer_totals_supported(s.cout)) && s.rows < (1ll << 22);
-    int64_t *tot_g = totals ? tot_g_buffer(L, s, ws) : nullptr;
-    // (a small filter: the layer gradient's column terms in one launch, beside the bifurcation -- they need the
-    // gradient's parameters only; else two kernels inside the product's call)
-    const bool small = s.conv && L->conv.R == 3 && (int64_t)L->conv.R * L->conv.S * L->conv.C <= 12288 && s.w_elems <= 49152 && L->conv.C % 4 == 0;
-    SideStream *sd = small ? side_stream() : nullptr;
+    int64_t *tot_g = totals ? l.tot_g : nullptr;
+    // the code sums that the two products need: of the weights and the input beside the statistics of the Range BN backward ...
+    SumJob early[kMaxSumJobs], late[kMaxSumJobs];
+    int nearly = 0, nlate = 0;
+    const SumJob w_job = weight_sum_job(L, s, true, saved->w_codes, l.w_sums);
+    early[nearly++] = w_job;
+    for (int i = totals ? 3 : 0; i < l.wg_count; ++i) {
+        if (i % 3 == 0) early[nearly++] = l.wg_sums[i];
+        else            late[nlate++] = l.wg_sums[i];          // ... of the gradient's copies once they are there
+    }
+    if (!s.conv) late[nlate++] = SumJob{g8, s.rows, s.cout, kSumRows, 1, l.row_sums};
     // Range BN backward and the two copies of its result.  Where the shape allows, in two passes over (dy, z): the
     // statistics pass also takes the extremes of dy, from which the exact range of the gradient follows (Section 4:
     // the range without a scan), and the second pass quantises the gradient as it computes it -- the fp32 gradient is
@@ -330,36 +289,37 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_bwd(const qbp_la
     if (two_pass) {
         rc = rangebn_bwd_bifurcate_impl(dy, saved->z, s.rows, s.cout, gamma, beta, L->relu, saved->save_mean, saved->save_min,
                                         saved->save_max, g, dgamma, dbeta, L->seed, L->tensor_id8, L->tensor_id16, g8, qp8,
-                                        s.conv ? row_sums : nullptr, ghi, glo, qp16, true, ws, scratch, st, sd ? sd->fork : nullptr,
-                                        self_totals ? nullptr : tot_g);
+                                        s.conv ? l.row_sums : nullptr, ghi, glo, qp16, true, l.scratch, l.scratch_bytes, st,
+                                        self_totals ? nullptr : tot_g, l.tot_g, s.conv ? l.clear_words : 0, early, nearly);
     } else {
         if (!g) return fail(QBP_ERR_INVALID_ARG, "layer_bwd: this shape needs saved->g (the fp32 gradient is written and read back)");
+        if (s.conv) QBP_CUDA_OK(cudaMemsetAsync(l.tot_g, 0, sizeof(uint32_t) * (size_t)l.clear_words, st));
         int nparts = 0;
         rc = rangebn_bwd_impl(dy, saved->z, s.rows, s.cout, gamma, beta, L->relu, saved->save_mean, saved->save_min,
-                              saved->save_max, g, dgamma, dbeta, ws, scratch, range_parts, &nparts, st);
+                              saved->save_max, g, dgamma, dbeta, l.scratch, l.scratch_bytes, l.range_parts, &nparts, st);
         if (rc) return rc;
         rc = bifurcate_with_range_partials(g, s.rows, s.cout, L->seed, L->tensor_id8, L->tensor_id16, g8, qp8,
-                                           s.conv ? row_sums : nullptr, ghi, glo, qp16, range_parts, nparts, st,
-                                           self_totals ? nullptr : tot_g, true, sd ? sd->fork : nullptr);
+                                           s.conv ? l.row_sums : nullptr, ghi, glo, qp16, l.range_parts, nparts, st,
+                                           self_totals ? nullptr : tot_g, true);
+        if (!rc) rc = launch_code_sums(early, nearly, st);
     }
     if (rc) return rc;
+    // (a 3 x 3 convolution: in the launch of the layer gradient's correction terms)
+    const bool with_terms = s.conv && L->conv.R == 3;
+    if (!with_terms && nlate && (rc = launch_code_sums(late, nlate, st))) return rc;
+    const CodeSums w_sums = sums_of(w_job), g_sums = sums_of(l.row_sums);
     if (s.conv) {
-        int32_t *ct = small ? colterm_buffer(L, s, ws) : nullptr;
-        if (small) {
-            if (sd && (rc = side_begin(sd))) return rc;
-            if ((rc = launch_filter_dgrad_colterm(&L->conv, saved->w_codes, qp8, ct, sd ? sd->s : st))) return rc;
-            if (sd && (rc = side_end(sd, st))) return rc;
-        }
-        const EpilogueTail with_colterm{nullptr, 0, nullptr, nullptr, nullptr, 0, ct};
-        rc = conv_s8_impl(QBP_CONV_DGRAD, &L->conv, g8, qp8, saved->w_codes, saved->qw, nullptr, dx, row_sums, nullptr, status, ws, scratch, st,
-                          small ? &with_colterm : nullptr);
+        const EpilogueTail with_sums{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums, late, with_terms ? nlate : 0};
+        rc = conv_s8_impl(QBP_CONV_DGRAD, &L->conv, g8, qp8, saved->w_codes, saved->qw, nullptr, dx, l.row_sums, nullptr, status,
+                          l.scratch, l.scratch_bytes, st, &with_sums);
         if (rc) return rc;
-        return wgrad_s16_impl(&L->conv, 0, 0, 0, saved->x_codes, saved->qx, ghi, glo, qp16, nullptr, dw, status, ws, scratch, st,
-                              totals ? saved->x_chan_sums : nullptr, tot_g, !self_totals, true);
+        return wgrad_s16_impl(&L->conv, 0, 0, 0, saved->x_codes, saved->qx, ghi, glo, qp16, nullptr, dw, status, l.scratch, l.scratch_bytes,
+                              st, totals ? saved->x_chan_sums : nullptr, tot_g, !self_totals, true, l.wg_sums);
     }
     // dx [batch x in] = g8 [batch x out] . w^T, w stored [in x out]
-    rc = gemm_s8_impl(0, 1, s.rows, s.cin, s.cout, g8, qp8, saved->w_codes, saved->qw, nullptr, dx, nullptr, status, ws, scratch, st);
+    rc = gemm_s8_impl(0, 1, s.rows, s.cin, s.cout, g8, qp8, saved->w_codes, saved->qw, nullptr, dx, nullptr, status, l.scratch,
+                      l.scratch_bytes, st, &g_sums, &w_sums);
     if (rc) return rc;
-    return wgrad_s16_impl(nullptr, s.rows, s.cout, s.cin, saved->x_codes, saved->qx, ghi, glo, qp16, nullptr, dw, status, ws,
-                          scratch, st, nullptr, nullptr, true, true);
+    return wgrad_s16_impl(nullptr, s.rows, s.cout, s.cin, saved->x_codes, saved->qx, ghi, glo, qp16, nullptr, dw, status, l.scratch,
+                          l.scratch_bytes, st, nullptr, nullptr, true, true, l.wg_sums);
 }

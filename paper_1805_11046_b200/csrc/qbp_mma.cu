@@ -19,6 +19,7 @@
 // where, for a convolution, class(m) says which taps of output pixel m fall
 // inside the image (real-zero padding contributes nothing).
 #include "qbp_mma.cuh"
+#include "qbp_sums.cuh"
 
 #include <algorithm>
 
@@ -841,105 +842,6 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
 }
 
 // ================================================= zero-point correction terms
-// A small filter in one launch (Appendix B's quantiser for the weights, then what the forward convolution's zero-point
-// correction needs of them): min / max scan, scale and zero-point, nearest 8-bit codes, the code sums of every
-// (output channel, tap) over the input channels, and the forward column terms
-//   colterm[cls][k] = -z_in * sum over the taps valid for border class cls of wsum[k][tap].
-// One block of 1024 threads; w [K][taps][C] fp32, C a multiple of 4, 16-byte aligned.  The operation order of the
-// quantiser is the library's (make_qparams, quantize_code), so the codes are those of qbp_quantize_s8.
-__global__ void __launch_bounds__(1024) filter_prep_kernel(const float *__restrict__ w, int K, int taps, int C, int R, int S, int pad,
-                                                            const qbp_qparams *__restrict__ q_in, int8_t *__restrict__ codes,
-                                                            qbp_qparams *__restrict__ qp_out, int32_t *__restrict__ colterm)
-{
-    pdl_enter();
-    extern __shared__ int s_wsum[];                      // [K * taps]
-    __shared__ float s_lo[32], s_hi[32];
-    __shared__ float s_inv, s_zp;
-    const int n4 = K * taps * C / 4;
-    const int rows = K * taps;
-    float lo = INFINITY, hi = -INFINITY;
-    for (int i = threadIdx.x; i < n4; i += 1024) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(w) + i);
-        lo = fminf(fminf(lo, fminf(v.x, v.y)), fminf(v.z, v.w));
-        hi = fmaxf(fmaxf(hi, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
-    }
-    lo = warp_min(lo); hi = warp_max(hi);
-    if ((threadIdx.x & 31) == 0) { s_lo[threadIdx.x >> 5] = lo; s_hi[threadIdx.x >> 5] = hi; }
-    for (int i = threadIdx.x; i < rows; i += 1024) s_wsum[i] = 0;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        lo = warp_min(s_lo[threadIdx.x]); hi = warp_max(s_hi[threadIdx.x]);
-        if (threadIdx.x == 0) {
-            const qbp_qparams qp = make_qparams(lo, hi, 8);
-            *qp_out = qp;
-            s_inv = __fdiv_rn(1.0f, qp.scale); s_zp = (float)(qp.zero_point + 128);
-        }
-    }
-    __syncthreads();
-    const float inv = s_inv, zp_u = s_zp;
-    const int c4 = C / 4;                                 // vectors per (k, tap) row
-    for (int i = threadIdx.x; i < n4; i += 1024) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(w) + i);
-        const uint32_t c0 = (uint32_t)quantize_code<false>(v.x, inv, zp_u, 255.0f, 0u), c1 = (uint32_t)quantize_code<false>(v.y, inv, zp_u, 255.0f, 0u);
-        const uint32_t c2 = (uint32_t)quantize_code<false>(v.z, inv, zp_u, 255.0f, 0u), c3 = (uint32_t)quantize_code<false>(v.w, inv, zp_u, 255.0f, 0u);
-        const uint32_t packed = (c0 | (c1 << 8) | (c2 << 16) | (c3 << 24)) ^ 0x80808080u;
-        reinterpret_cast<uint32_t *>(codes)[i] = packed;
-        atomicAdd(&s_wsum[i / c4], __dp4a((int)packed, 0x01010101, 0));
-    }
-    __syncthreads();
-    const int zin = q_in->zero_point;
-    for (int i = threadIdx.x; i < 16 * K; i += 1024) {
-        const int cls = i / K, k = i - cls * K;
-        const bool top = cls & 1, bottom = cls & 2, left = cls & 4, right = cls & 8;
-        int sum = 0;
-        for (int r = 0; r < R; ++r) {
-            if ((r < pad && top) || (r > pad && bottom)) continue;
-            for (int t = 0; t < S; ++t) {
-                if ((t < pad && left) || (t > pad && right)) continue;
-                sum += s_wsum[k * taps + r * S + t];
-            }
-        }
-        colterm[i] = -zin * sum;
-    }
-}
-
-// The layer-gradient product's column terms from a small filter's codes in one launch: the code sums of every
-// (tap, input channel) over the output channels, then
-//   colterm[cls][c] = -z_g * sum over the taps valid for border class cls (gradient orientation) of wsum[tap][c].
-// One block of 1024 threads; codes [K][taps * C], C a multiple of 4.
-__global__ void __launch_bounds__(1024) filter_dgrad_colterm_kernel(const int8_t *__restrict__ codes, int K, int taps, int C, int R,
-                                                                     int S, int pad, const qbp_qparams *__restrict__ q_g,
-                                                                     int32_t *__restrict__ colterm)
-{
-    pdl_enter();
-    extern __shared__ int s_wsum[];                      // [taps * C]
-    const int cols4 = taps * C / 4;
-    for (int j = threadIdx.x; j < cols4; j += 1024) {
-        int a0 = 0, a1 = 0, a2 = 0, a3 = 0;
-        for (int k = 0; k < K; ++k) {
-            const int v = (int)__ldg(reinterpret_cast<const uint32_t *>(codes) + (int64_t)k * cols4 + j);
-            a0 = __dp4a(v, 0x00000001, a0); a1 = __dp4a(v, 0x00000100, a1); a2 = __dp4a(v, 0x00010000, a2); a3 = __dp4a(v, 0x01000000, a3);
-        }
-        s_wsum[4 * j] = a0; s_wsum[4 * j + 1] = a1; s_wsum[4 * j + 2] = a2; s_wsum[4 * j + 3] = a3;
-    }
-    __syncthreads();
-    const int zg = q_g->zero_point;
-    for (int i = threadIdx.x; i < 16 * C; i += 1024) {
-        const int cls = i / C, c = i - cls * C;
-        const bool top = cls & 1, bottom = cls & 2, left = cls & 4, right = cls & 8;
-        int sum = 0;
-        for (int r = 0; r < R; ++r) {
-            // gradient row h + pad - r feeds input row h: tap rows below the centre fall off the first row
-            if ((r > pad && top) || (r < pad && bottom)) continue;
-            for (int t = 0; t < S; ++t) {
-                if ((t > pad && left) || (t < pad && right)) continue;
-                sum += s_wsum[(r * S + t) * C + c];
-            }
-        }
-        colterm[i] = -zg * sum;
-    }
-}
-
 // The correction terms of a 3 x 3 convolution.
 // Blocks below `row_blocks`: rowterm[pixel] = -z_w * (sum of the input's channel sums over the taps inside the image)
 //                   + (taps inside) * Cred * z_in * z_w
@@ -956,11 +858,14 @@ struct ConvTerms {
     CodeSums w_sums; int N, dgrad;
     int32_t *colterm;
 };
-__global__ void __launch_bounds__(256) conv_terms_kernel(const __grid_constant__ ConvTerms T)
+// The first `sum_blocks` blocks take code sums that a later product needs (a launch less, and they overlap).
+__global__ void __launch_bounds__(256, 6) conv_terms_kernel(const __grid_constant__ ConvTerms T, const __grid_constant__ SumJobs J, int sum_blocks)
 {
     pdl_enter();
-    if ((int)blockIdx.x >= T.row_blocks) {
-        const int i = ((int)blockIdx.x - T.row_blocks) * 256 + (int)threadIdx.x;
+    if ((int)blockIdx.x < sum_blocks) { code_sums_block(J, (int)blockIdx.x); return; }
+    const int block = (int)blockIdx.x - sum_blocks;
+    if (block >= T.row_blocks) {
+        const int i = (block - T.row_blocks) * 256 + (int)threadIdx.x;
         if (i >= 16 * T.N) return;
         const int cls = i / T.N, n = i - cls * T.N;
         const bool top = cls & 1, bottom = cls & 2, left = cls & 4, right = cls & 8;
@@ -976,7 +881,7 @@ __global__ void __launch_bounds__(256) conv_terms_kernel(const __grid_constant__
         return;
     }
     int img, bi;
-    T.dB.divmod((int)blockIdx.x, img, bi);
+    T.dB.divmod(block, img, bi);
     const int i = bi * 256 + (int)threadIdx.x;
     if (i >= T.HW) return;
     int p, q;
@@ -1029,33 +934,6 @@ __global__ void __launch_bounds__(128) colstat_finalize_kernel(const float *__re
 }
 
 int colstat_rows_max() { return sm_count(); }
-
-// Whether filter_prep_kernel takes this filter: small enough for one block and its shared-memory table.
-bool filter_prep_supported(const qbp_conv_desc *d, const float *w, const int8_t *codes)
-{
-    const int64_t elems = (int64_t)d->K * d->R * d->S * d->C;
-    // (one block: beyond some 48 K elements the five launches it replaces are faster)
-    return d->C % 4 == 0 && elems <= 49152 && (int64_t)d->K * d->R * d->S <= 8192 && aligned16(w) && ((uintptr_t)codes & 3) == 0;
-}
-
-int launch_filter_dgrad_colterm(const qbp_conv_desc *d, const int8_t *codes, const qbp_qparams *q_g, int32_t *colterm, cudaStream_t st)
-{
-    const int taps = d->R * d->S;
-    QBP_TRACE_BEGIN(st);
-    launch(filter_dgrad_colterm_kernel, 1, 1024, sizeof(int) * (size_t)taps * d->C, st, codes, d->K, taps, d->C, d->R, d->S, d->pad, q_g, colterm);
-    QBP_LAUNCH_OK("filter_dgrad_colterm_kernel");
-    return QBP_OK;
-}
-
-int launch_filter_prep(const qbp_conv_desc *d, const float *w, const qbp_qparams *q_in, int8_t *codes, qbp_qparams *qw,
-                       int32_t *colterm, cudaStream_t st)
-{
-    const int taps = d->R * d->S;
-    QBP_TRACE_BEGIN(st);
-    launch(filter_prep_kernel, 1, 1024, sizeof(int) * (size_t)d->K * taps, st, w, d->K, taps, d->C, d->R, d->S, d->pad, q_in, codes, qw, colterm);
-    QBP_LAUNCH_OK("filter_prep_kernel");
-    return QBP_OK;
-}
 
 // Self-test of the bounded wait (diagnostics): one warp waits on an mbarrier on which nothing ever arrives, with
 // the wait wrappers the product kernels use and a limit of `limit` cycles; the wait gives up, the status word is
@@ -1153,7 +1031,7 @@ static bool halo_fits(MmaParams &P, uint32_t halo_tile_bytes)
     return P.tiles_n == 1 && fixed + align_up((size_t)P.b.tile_bytes * P.k_iters, 1024) + 3u * halo_tile_bytes <= kSmemBudget;
 }
 
-static int launch_mma(MmaParams &P, int tiles_m, bool clear_status, cudaStream_t st)
+static int launch_mma(MmaParams &P, int tiles_m, cudaStream_t st)
 {
     const uint32_t fixed = fixed_smem(P);
     const uint32_t budget = kSmemBudget - fixed;
@@ -1206,7 +1084,6 @@ static int launch_mma(MmaParams &P, int tiles_m, bool clear_status, cudaStream_t
     void (*kernel)(const MmaParams) = id == 0 ? qbp_mma_kernel<false, false> : id == 1 ? qbp_mma_kernel<false, true>
                                     : id == 2 ? qbp_mma_kernel<true, false> : qbp_mma_kernel<true, true>;
     QBP_SMEM_OPT_IN(configured[id], kernel, kSmemBudget);
-    if (clear_status) QBP_CUDA_OK(cudaMemsetAsync(P.status, 0, sizeof(int), st));
     // one CTA per SM (its shared-memory ring fills the SM), each walking its share of the tiles
     int grid = std::min(P.tiles_total, sm_count());
     if (P.stat_local) {
@@ -1224,7 +1101,7 @@ static int launch_mma(MmaParams &P, int tiles_m, bool clear_status, cudaStream_t
 static size_t gemm_ws_bytes(int64_t M, int64_t N, int64_t K)
 {
     // (code sums of either operand, stored either way round)
-    auto sums = [&](int64_t n) { return align_up(sizeof(int32_t) * std::max(sum_elems(n, K, false), sum_elems(K, n, true)), 256); };
+    auto sums = [&](int64_t n) { return align_up(sizeof(int32_t) * std::max(sum_elems(n, K, kSumRows), sum_elems(K, n, kSumCols)), 256); };
     return 256 + sums(M) + sums(N) + colstat_ws_bytes(N);
 }
 
@@ -1235,10 +1112,16 @@ bool conv_supported(const qbp_conv_desc *d)
 }
 
 // The filter's code sums: forward [K][taps], layer gradient pieces of [taps * C].
-static size_t filter_sum_elems(const qbp_conv_desc *d)
+size_t filter_sum_elems(const qbp_conv_desc *d)
 {
     const int64_t taps = (int64_t)d->R * d->S;
-    return std::max(sum_elems(d->K * taps, d->C, false), sum_elems(d->K, taps * d->C, true));
+    return std::max(sum_elems(d->K * taps, d->C, kSumRows), sum_elems(d->K, taps * d->C, kSumCols));
+}
+
+SumJob filter_sum_job(const qbp_conv_desc *d, bool dgrad, const int8_t *w, int32_t *out)
+{
+    const int64_t taps = (int64_t)d->R * d->S;
+    return dgrad ? SumJob{w, d->K, taps * d->C, kSumCols, 1, out} : SumJob{w, d->K * taps, d->C, kSumRows, 1, out};
 }
 
 // What the product itself carves from the workspace, and with the room for the column statistics' partial rows
@@ -1315,12 +1198,14 @@ extern "C" __attribute__((visibility("default"))) int qbp_gemm_s8_sums(int trans
                            const int32_t *b_sums, int32_t *acc_out, float *C, const qbp_epilogue *ep, void *ws,
                            size_t ws_bytes, void *stream)
 {
-    return gemm_s8_impl(transA, transB, M, N, K, A, qa, B, qb, acc_out, C, ep, nullptr, ws, ws_bytes, (cudaStream_t)stream, a_sums, b_sums);
+    const CodeSums as = sums_of(a_sums), bs = sums_of(b_sums);
+    return gemm_s8_impl(transA, transB, M, N, K, A, qa, B, qb, acc_out, C, ep, nullptr, ws, ws_bytes, (cudaStream_t)stream,
+                        a_sums ? &as : nullptr, b_sums ? &bs : nullptr);
 }
 
 int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,
                       const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const qbp_epilogue *ep,
-                      int *ext_status, void *ws, size_t ws_bytes, cudaStream_t st, const int32_t *a_sums, const int32_t *b_sums)
+                      int *ext_status, void *ws, size_t ws_bytes, cudaStream_t st, const CodeSums *a_sums, const CodeSums *b_sums)
 {
     if (M <= 0 || N <= 0 || K <= 0) return fail(QBP_ERR_INVALID_ARG, "gemm_s8: M, N, K must be positive");
     if (M % 16 || N % 16 || K % 16) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "gemm_s8: M, N, K must be multiples of 16");
@@ -1344,13 +1229,13 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
     int *status = w.take<int>(1);
     if (ext_status) status = ext_status;         // the caller's sticky word: raised here, never cleared
     // code sums along the reduction, the caller's or of this call's own (one launch for both operands)
-    const SumJob a_job = transA ? SumJob{A, K, M, 1, 1, nullptr} : SumJob{A, M, K, 0, 1, nullptr};
-    const SumJob b_job = transB ? SumJob{B, N, K, 0, 1, nullptr} : SumJob{B, K, N, 1, 1, nullptr};
+    const SumJob a_job = transA ? SumJob{A, K, M, kSumCols, 1, nullptr} : SumJob{A, M, K, kSumRows, 1, nullptr};
+    const SumJob b_job = transB ? SumJob{B, N, K, kSumRows, 1, nullptr} : SumJob{B, K, N, kSumCols, 1, nullptr};
     SumJob jobs[2];
     int njobs = 0;
-    CodeSums asum = sums_of(a_sums), bsum = sums_of(b_sums);
-    if (!a_sums) { jobs[njobs] = a_job; jobs[njobs].out = w.take<int32_t>(sum_elems(a_job.rows, a_job.cols, a_job.over_rows)); asum = sums_of(jobs[njobs++]); }
-    if (!b_sums) { jobs[njobs] = b_job; jobs[njobs].out = w.take<int32_t>(sum_elems(b_job.rows, b_job.cols, b_job.over_rows)); bsum = sums_of(jobs[njobs++]); }
+    CodeSums asum = a_sums ? *a_sums : CodeSums{}, bsum = b_sums ? *b_sums : CodeSums{};
+    if (!a_sums) { jobs[njobs] = a_job; jobs[njobs].out = w.take<int32_t>(sum_elems(a_job)); asum = sums_of(jobs[njobs++]); }
+    if (!b_sums) { jobs[njobs] = b_job; jobs[njobs].out = w.take<int32_t>(sum_elems(b_job)); bsum = sums_of(jobs[njobs++]); }
     ColStatParts parts{nullptr, nullptr, nullptr, 0};
     if (stats) {
         const size_t cells = (size_t)colstat_rows_max() * (size_t)N;
@@ -1358,12 +1243,14 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
     }
 
     int rc = QBP_OK;
-    if (njobs && (rc = launch_code_sums(jobs, njobs, st))) return rc;
+    ZeroJobs zero{};
+    if (!ext_status) { zero.p[0] = reinterpret_cast<uint32_t *>(status); zero.words[0] = 1; }
+    if ((rc = launch_code_sums(jobs, njobs, st, zero))) return rc;
 
     // large products run on CTA pairs (256 x 256 tiles across two SMs); the column statistics are the
     // single-CTA kernel's (at most 256 columns: narrow either way)
     if (gemm2_eligible(M, N, K) && !stats && !has_tail)
-        return launch_gemm2(transA, transB, M, N, K, A, qa, B, qb, acc_out, C, asum, bsum, status, !ext_status, st);
+        return launch_gemm2(transA, transB, M, N, K, A, qa, B, qb, acc_out, C, asum, bsum, status, st);
 
     MmaParams P{};
     P.mode = MODE_GEMM;
@@ -1410,7 +1297,7 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
         fused_row_sums = tail.q && tail.row_sums && P.tiles_n == 1;
         if (fused_row_sums) P.ep_rowsum = tail.row_sums;
     }
-    if ((rc = launch_mma(P, (int)((M + 128 * P.msub - 1) / (128 * P.msub)), !ext_status, st))) return rc;
+    if ((rc = launch_mma(P, (int)((M + 128 * P.msub - 1) / (128 * P.msub)), st))) return rc;
     if (stats) { parts.rows = P.grid; return finish_epilogue(ep, parts, N, st); }
     if (has_tail && tail.q && tail.row_sums && !fused_row_sums) return launch_rowsum(tail.q, true, M, N, tail.row_sums, st);
     return QBP_OK;
@@ -1503,27 +1390,33 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
     int32_t *chan_sum = w.take<int32_t>(pix);
     int32_t *colterm = w.take<int32_t>(16 * nmax);
     int32_t *wsum = w.take<int32_t>(filter_sum_elems(d));
-    const SumJob w_job = dgrad ? SumJob{wgt, d->K, (int64_t)taps * d->C, 1, 1, wsum} : SumJob{wgt, (int64_t)d->K * taps, d->C, 0, 1, wsum};
-    const bool own_colterm = !(tail && tail->colterm);       // (else: the column terms came with the filter's codes)
+    const SumJob w_job = filter_sum_job(d, dgrad, wgt, wsum);
+    const bool own_wsums = !(tail && tail->w_sums);
+    const CodeSums w_sums = own_wsums ? sums_of(w_job) : *tail->w_sums;
     const bool raw_sums = d->R == 1;                         // (1 x 1: no borders, the kernel works on the sums themselves)
 
     int rc = QBP_OK;
     if (in_chan_sum) chan_sum = const_cast<int32_t *>(in_chan_sum);
-    if (tail && tail->colterm) colterm = const_cast<int32_t *>(tail->colterm);
-    if (!(tail && tail->keep_terms)) {
+    ZeroJobs zero{};
+    if (!ext_status) { zero.p[0] = reinterpret_cast<uint32_t *>(status); zero.words[0] = 1; }
+    if (tail && tail->keep_terms) { if ((rc = launch_code_sums(nullptr, 0, st, zero))) return rc; }
+    else {
         SumJob jobs[2];
         int njobs = 0;
-        if (!in_chan_sum) jobs[njobs++] = SumJob{in, pix, Cred, 0, 1, chan_sum};
-        if (own_colterm) jobs[njobs++] = w_job;
-        if (njobs && (rc = launch_code_sums(jobs, njobs, st))) return rc;
+        if (!in_chan_sum) jobs[njobs++] = SumJob{in, pix, Cred, kSumRows, 1, chan_sum};
+        if (own_wsums) jobs[njobs++] = w_job;
+        if ((rc = launch_code_sums(jobs, njobs, st, zero))) return rc;
         if (!raw_sums) {
             ConvTerms T{};
             const int per_img = (d->H * d->W + 255) / 256;
             T.chan_sum = chan_sum; T.HW = d->H * d->W; T.H = d->H; T.W = d->W; T.dW = make_fastdiv(d->W); T.dB = make_fastdiv(per_img);
             T.Cred = Cred; T.row_blocks = per_img * d->N; T.q_in = q_in; T.q_w = q_w; T.rowterm = rowterm;
-            T.w_sums = sums_of(w_job); T.N = Nout; T.dgrad = dgrad ? 1 : 0; T.colterm = colterm;
+            T.w_sums = w_sums; T.N = Nout; T.dgrad = dgrad ? 1 : 0; T.colterm = colterm;
+            SumJobs J{};
+            int sum_blocks = 0;
+            if (tail && tail->extra_count && (rc = fill_sum_jobs(tail->extra, tail->extra_count, J, &sum_blocks))) return rc;
             QBP_TRACE_BEGIN(st);
-            launch(conv_terms_kernel, T.row_blocks + (own_colterm ? (16 * Nout + 255) / 256 : 0), 256, 0, st, T);
+            launch(conv_terms_kernel, sum_blocks + T.row_blocks + (16 * Nout + 255) / 256, 256, 0, st, T, J, sum_blocks);
             QBP_LAUNCH_OK("conv_terms_kernel");
         }
     }
@@ -1596,11 +1489,11 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
     P.idesc = make_idesc(true, true, P.a.major, P.b.major, 128, (uint32_t)P.bn);
     P.acc_out = acc_out; P.out = out;
     P.rowterm = rowterm; P.colterm = colterm; P.qa = q_in; P.qb = q_w; P.status = status;
-    P.raw_sums = raw_sums ? 1 : 0; P.k_len = Cred; P.a_sums = sums_of(chan_sum); P.b_sums = sums_of(w_job);
+    P.raw_sums = raw_sums ? 1 : 0; P.k_len = Cred; P.a_sums = sums_of(chan_sum); P.b_sums = w_sums;
     // each row's code sum comes from the epilogue when one column tile holds the whole row, else from a pass over the codes
     const bool fused_row_sums = want_codes && tail->row_sums && P.tiles_n == 1;
     if (fused_row_sums) P.ep_rowsum = tail->row_sums;
-    if ((rc = launch_mma(P, P.tiles_w * P.tiles_h * tiles_img, !ext_status, st))) return rc;
+    if ((rc = launch_mma(P, P.tiles_w * P.tiles_h * tiles_img, st))) return rc;
     if (stats) stats->rows = P.grid;
     if (want_codes && tail->row_sums && !fused_row_sums) return launch_rowsum(tail->q, true, pix, Nout, tail->row_sums, st);
     return QBP_OK;

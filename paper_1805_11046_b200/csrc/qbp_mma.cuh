@@ -28,20 +28,34 @@ struct CodeSums {
 #endif
 };
 inline CodeSums sums_of(const int32_t *p) { return CodeSums{p, 1, 0}; }
-// Up to four such sums in one launch (code_sums_kernel): per row (over_rows = 0: out [rows]), or per column over the rows
-// (over_rows = 1: out [sum_pieces(rows, cols)][cols]).  cols a multiple of 16, q 16-byte aligned, fewer than 2^31 rows.
-struct SumJob { const void *q; int64_t rows, cols; int over_rows, is_signed; int32_t *out; };
+// Up to eight such sums in one launch (code_sums_kernel), by kind:
+//   kSumRows   per row: out [rows]
+//   kSumCols   per column over the rows, in pieces: out [sum_pieces(rows, cols)][cols]
+//   kSumEdges  rows = the positions of N images of H x W, cols = channels: per channel over the positions of the first row, last
+//              row, first column, last column and the four corners (first row: first, last column; last row: the same) of
+//              every image: added to out64 [8][cols], which is zero beforehand
+// out64 (kSumCols): the whole sums are added to out64 [cols], which is zero beforehand, instead.
+// cols a multiple of 16, q 16-byte aligned, fewer than 2^31 rows.  zero: up to two regions of 32-bit words the launch clears (a
+// status word, sums that a later kernel adds to).
+enum { kSumRows = 0, kSumCols = 1, kSumEdges = 2 };
+struct SumJob { const void *q; int64_t rows, cols; int kind, is_signed; int32_t *out; int H = 0, W = 0; int64_t *out64 = nullptr; };
+constexpr int kMaxSumJobs = 8;
 int sum_pieces(int64_t rows, int64_t cols);
-inline size_t sum_elems(int64_t rows, int64_t cols, bool over_rows) { return over_rows ? (size_t)sum_pieces(rows, cols) * (size_t)cols : (size_t)rows; }
+int edge_pieces(int64_t rows, int H, int W);
+inline size_t sum_elems(int64_t rows, int64_t cols, int kind)
+{
+    return kind == kSumRows ? (size_t)rows : kind == kSumCols ? (size_t)sum_pieces(rows, cols) * (size_t)cols : 8 * (size_t)cols;
+}
+inline size_t sum_elems(const SumJob &j) { return sum_elems(j.rows, j.cols, j.kind); }
 inline CodeSums sums_of(const SumJob &j)
 {
-    return j.over_rows ? CodeSums{j.out, sum_pieces(j.rows, j.cols), j.cols} : sums_of(j.out);
+    return j.kind == kSumRows ? sums_of(j.out) : CodeSums{j.out, sum_pieces(j.rows, j.cols), j.cols};
 }
-int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st);
+int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st, const ZeroJobs &zero = ZeroJobs{});
 
-// ---- per-tensor range scan (qbp_quant.cu): *qp = 8-bit parameters of [min(lowest, 0), max(highest, 0)] -------------
+// ---- per-tensor range scan (qbp_quant.cu): leaves *nparts (min, max) pairs at ws, for RangeSrc::parts -------------
 size_t range_scan_ws_bytes();
-int range_scan(const float *x, int64_t n, void *ws, size_t ws_bytes, qbp_qparams *qp, cudaStream_t st);
+int range_scan(const float *x, int64_t n, void *ws, size_t ws_bytes, int *nparts, cudaStream_t st);
 
 // ---- pieces the whole-layer composition chains without a pass of their own ------
 // Range BN backward that also leaves per-block (min, max) of dx (qbp_rangebn.cu), and the gradient
@@ -57,20 +71,24 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
                                int relu, const float *save_mean, const float *save_min, const float *save_max, float *g_out,
                                float *dgamma, float *dbeta, uint64_t seed, uint32_t id8, uint32_t id16, int8_t *q8,
                                qbp_qparams *qp8, int32_t *row_sums8, int8_t *hi, uint8_t *lo, qbp_qparams *qp16, bool lo_signed,
-                               void *ws, size_t ws_bytes, cudaStream_t st, cudaEvent_t after_range = nullptr,
-                               int64_t *tot16 = nullptr);      // tot16 (nullable) [C]: per-channel totals of the stored 16-bit codes
-int launch_range_finalize(const float2 *partials, int nparts, qbp_qparams *qp8, qbp_qparams *qp16, cudaStream_t st,
-                          cudaEvent_t after_range = nullptr);
+                               void *ws, size_t ws_bytes, cudaStream_t st, int64_t *tot16 = nullptr, void *clear = nullptr,
+                               int64_t clear_words = 0, const SumJob *extra = nullptr, int extra_count = 0);
+// (tot16 (nullable) [C]: per-channel totals of the stored 16-bit codes; clear: 32-bit words cleared at the start, tot16 among
+// them; extra: code sums taken beside the per-channel reduction)
 int bifurcate_with_range_partials(const float *g, int64_t rows, int64_t cols, uint64_t seed, uint32_t tensor_id8,
                                   uint32_t tensor_id16, int8_t *q8, qbp_qparams *qp8, int32_t *row_sums8, int8_t *hi,
                                   uint8_t *lo, qbp_qparams *qp16, const float2 *partials, int nparts, cudaStream_t st,
-                                  int64_t *tot16 = nullptr, bool lo_signed = false, cudaEvent_t after_range = nullptr);
-// after_range (here and in quantize_s8_with_totals; nullable): an event recorded on the stream as soon as the quantiser's
-// parameters are enqueued, before the pass that writes the codes.
-// Whether the quantising kernels can leave per-channel totals for a tensor of `cols` channels.
+                                  int64_t *tot16 = nullptr, bool lo_signed = false);
+// The layer's operands quantised to 8 bits (nearest rounding, clamping values = min and max): the activation (nullable) and the
+// weights, in two launches.  row_sums [rows] / tot [cols] (each nullable): wanted sums of the stored codes; *_left: whether the
+// quantising kernel left them (it depends on the shape; the caller sums the codes up otherwise).  tot is cleared either way.
+struct QuantOperand {
+    const float *v; int64_t rows, cols; int8_t *q; qbp_qparams *qp; int32_t *row_sums; int64_t *tot;
+    bool row_sums_left = false, tot_left = false;
+};
+size_t quantize_operands_ws_bytes();
+int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, size_t ws_bytes, cudaStream_t st);
 bool quantizer_totals_supported(int64_t cols);
-int quantize_s8_with_totals(const float *x, int64_t rows, int64_t cols, int8_t *q, qbp_qparams *qp_out, int32_t *row_sums,
-                            int64_t *tot8, bool *left, void *ws, size_t ws_bytes, cudaStream_t st, cudaEvent_t after_range = nullptr);
 // The convolution products with the per-pixel channel sums of the input codes supplied by the caller
 // (nullable: computed here) (qbp_mma.cu).
 // Per-column (sum, min, max) of a product's fp32 output as partial rows [rows][N], one per CTA
@@ -84,14 +102,12 @@ int rangebn_fold_from_parts(int64_t n, int64_t C, const float *gamma, const floa
 // column, as rangebn_fold_from_parts leaves them), ReLU, and 8-bit codes of the result with parameters *rq
 // (q [M x N], row_sums [M] nullable).  keep_terms: the zero-point term kernels ran for the same operands in the
 // call just before on the same workspace and are not run again.
-// colterm (nullable; 3 x 3): the column terms [16][N] of this product, already computed (launch_filter_prep).
-struct EpilogueTail { const float4 *fold; int relu; const qbp_qparams *rq; int8_t *q; int32_t *row_sums; int keep_terms; const int32_t *colterm; };
-// A small filter quantised and its forward column terms computed in one launch (qbp_mma.cu).
-bool filter_prep_supported(const qbp_conv_desc *d, const float *w, const int8_t *codes);
-int launch_filter_prep(const qbp_conv_desc *d, const float *w, const qbp_qparams *q_in, int8_t *codes, qbp_qparams *qw,
-                       int32_t *colterm, cudaStream_t st);
-// ... and the layer-gradient product's column terms [16][C] from such a filter's codes, in one launch.
-int launch_filter_dgrad_colterm(const qbp_conv_desc *d, const int8_t *codes, const qbp_qparams *q_g, int32_t *colterm, cudaStream_t st);
+// w_sums (nullable): the filter's code sums (forward [K * taps], layer gradient [taps * C]) are there already.
+// extra [extra_count] (3 x 3): code sums of a later product, taken in the launch that makes this one's correction terms.
+struct EpilogueTail { const float4 *fold; int relu; const qbp_qparams *rq; int8_t *q; int32_t *row_sums; int keep_terms; const CodeSums *w_sums;
+                      const SumJob *extra = nullptr; int extra_count = 0; };
+size_t filter_sum_elems(const qbp_conv_desc *d);
+SumJob filter_sum_job(const qbp_conv_desc *d, bool dgrad, const int8_t *w, int32_t *out);
 
 // ext_status (here and below; nullable): a status word the caller owns and has cleared -- the product raises it when
 // a bounded wait runs out and never clears it; NULL: the word is the first int of `ws`, cleared by the call itself.
@@ -100,8 +116,8 @@ int conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const qbp_q
                  int *ext_status, void *ws, size_t ws_bytes, cudaStream_t st, const EpilogueTail *tail = nullptr);
 int gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,
                  const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const qbp_epilogue *ep,
-                 int *ext_status, void *ws, size_t ws_bytes, cudaStream_t st, const int32_t *a_sums = nullptr,
-                 const int32_t *b_sums = nullptr);
+                 int *ext_status, void *ws, size_t ws_bytes, cudaStream_t st, const CodeSums *a_sums = nullptr,
+                 const CodeSums *b_sums = nullptr);
 // tot_x [C] / tot_g16 [K] (convolution; nullable, both or none): per-channel totals of the stored x codes and of the
 // stored 16-bit gradient codes (256 * hi + lo) over all positions, left by the kernels that wrote the codes.
 // lo_signed: g_lo holds the low bytes with the top bit flipped, i.e. the signed bytes lo - 128 (lo_signed in
@@ -111,10 +127,17 @@ int gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, const 
 int wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qparams *qx,
                    const int8_t *g_hi, const uint8_t *g_lo, const qbp_qparams *qg16, int64_t *acc_out, float *dW,
                    int *ext_status, void *ws, size_t ws_bytes, cudaStream_t st, const int64_t *tot_x = nullptr,
-                   const int64_t *tot_g16 = nullptr, bool tot_g_filled = true, bool lo_signed = false);
-// tot_g_filled == false: tot_g16 is a buffer [K] that the product fills itself (possible when wgrad_self_totals(d)).
+                   const int64_t *tot_g16 = nullptr, bool tot_g_filled = true, bool lo_signed = false,
+                   const SumJob *done_sums = nullptr);
+// The sums behind the zero-point terms.  Plain product: the columns of x, hi, lo in pieces (3 jobs).  Convolution: the same
+// added to one cleared table of int64 (tab: x [C], hi [N], lo [N]; 3 x 3: then [8][C], [8][N], [8][N] over the images' edges;
+// 3 or 6 jobs); with totals (tot_x, tot_g16) the first three are not needed.  done_sums (above): the caller has run the needed
+// ones into these buffers, and has cleared tot_g16 when tot_g_filled is false.
+int wgrad_sum_jobs(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, const int8_t *x, const int8_t *hi, const uint8_t *lo,
+                   bool lo_signed, int64_t *tab, SumJob (&jobs)[6]);
+size_t wgrad_sum_table(const qbp_conv_desc *d);        // int64 entries of tab (0: plain)
+// tot_g_filled == false: tot_g16 is a cleared buffer [K] that the product fills itself (possible when wgrad_self_totals(d)).
 bool wgrad_self_totals(const qbp_conv_desc *d);
-// Bifurcation with optional per-channel totals of the 16-bit codes (tot16 [cols], zeroed here) -- see above.
 // Shapes the convolution products / the convolution weight gradient implement.
 bool conv_supported(const qbp_conv_desc *d);
 bool wgrad_conv_supported(const qbp_conv_desc *d);
@@ -139,7 +162,7 @@ int make_map_out_2d(CUtensorMap *map, float *base, uint64_t rows, uint64_t cols)
 bool gemm2_eligible(int64_t M, int64_t N, int64_t K);
 int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,
                  const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const CodeSums &a_sums,
-                 const CodeSums &b_sums, int *status, bool clear_status, cudaStream_t st);
+                 const CodeSums &b_sums, int *status, cudaStream_t st);
 
 // ---- the dense weight gradient on CTA pairs (qbp_wgrad2.cu) ----------------------
 bool wgrad2_eligible(int64_t M, int64_t N, int64_t K);

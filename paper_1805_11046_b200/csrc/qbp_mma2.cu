@@ -365,7 +365,7 @@ bool gemm2_eligible(int64_t M, int64_t N, int64_t K)
 
 int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,
                  const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const CodeSums &a_sums,
-                 const CodeSums &b_sums, int *status, bool clear_status, cudaStream_t st)
+                 const CodeSums &b_sums, int *status, cudaStream_t st)
 {
     Mma2Params P{};
     int rc;
@@ -399,7 +399,6 @@ int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const 
     const size_t smem = 1024 + (size_t)stages * stage_bytes + k2EpiWarps * k2Slab;
     static PerDeviceOnce configured;
     QBP_SMEM_OPT_IN(configured, qbp_mma2_kernel, k2Smem);
-    if (clear_status) QBP_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
     QBP_TRACE_BEGIN(st);
     launch(qbp_mma2_kernel, 2 * P.pairs, k2Threads, smem, st, P);
     QBP_LAUNCH_OK("qbp_mma2_kernel");

@@ -7,6 +7,7 @@
 // fill every SM.  Also hosts the library's error-reporting state.
 #include "qbp_colscan.cuh"
 #include "qbp_mma.cuh"
+#include "qbp_sums.cuh"
 
 #include <algorithm>
 #include <cstring>
@@ -81,22 +82,29 @@ constexpr int kMaxParts = 4096;          // upper bound on per-tensor scan block
 // ------------------------------------------------------- per-tensor range
 // keep_rev: the tensor is walked from its end with loads that leave the lines in the L2 -- for the layer's input, whose
 // quantiser follows from the front and so finds the first 100 MB there (scan +3 us, quantiser -3 us, step -2.5 us).
+// Up to two tensors in one launch (a layer's weights, b, beside its activation, a): the first b.blocks blocks take b.
+struct ScanJob { const float *x; int64_t n; float2 *parts; int blocks, keep_rev; };
 template <int VEC>
-__global__ void __launch_bounds__(kThreads) range_partial_kernel(const float *__restrict__ x, int64_t n,
-                                                                 float2 *__restrict__ partials, int keep_rev)
+__global__ void __launch_bounds__(kThreads) range_partial_kernel(const __grid_constant__ ScanJob a, const __grid_constant__ ScanJob b,
+                                                                 const __grid_constant__ ZeroJobs zero)
 {
     pdl_enter();
+    const bool second = (int)blockIdx.x < b.blocks;
+    const ScanJob &J = second ? b : a;
+    const int block = second ? (int)blockIdx.x : (int)blockIdx.x - b.blocks;
+    run_zero_jobs(zero, (int64_t)blockIdx.x * kThreads + threadIdx.x, (int64_t)gridDim.x * kThreads);
+    const float *__restrict__ x = J.x;
     float lo = INFINITY, hi = -INFINITY;
-    const int64_t nv = n / VEC;
-    const int64_t stride = (int64_t)gridDim.x * kThreads * kRangeUnroll;
-    for (int64_t base = (int64_t)blockIdx.x * kThreads * kRangeUnroll; base < nv; base += stride) {
+    const int64_t nv = J.n / VEC;
+    const int64_t stride = (int64_t)J.blocks * kThreads * kRangeUnroll;
+    for (int64_t base = (int64_t)block * kThreads * kRangeUnroll; base < nv; base += stride) {
         VecF<VEC> v[kRangeUnroll];
         bool ok[kRangeUnroll];
 #pragma unroll
         for (int u = 0; u < kRangeUnroll; ++u) {
             int64_t i = base + u * kThreads + threadIdx.x;
             ok[u] = i < nv;
-            if (ok[u]) { if (keep_rev) v[u].load(x + (nv - 1 - i) * VEC); else v[u].load_stream(x + i * VEC); }
+            if (ok[u]) { if (J.keep_rev) v[u].load(x + (nv - 1 - i) * VEC); else v[u].load_stream(x + i * VEC); }
         }
 #pragma unroll
         for (int u = 0; u < kRangeUnroll; ++u)
@@ -105,39 +113,18 @@ __global__ void __launch_bounds__(kThreads) range_partial_kernel(const float *__
                 for (int e = 0; e < VEC; ++e) { lo = fminf(lo, v[u].v[e]); hi = fmaxf(hi, v[u].v[e]); }
             }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        for (int64_t i = nv * VEC; i < n; ++i) { lo = fminf(lo, x[i]); hi = fmaxf(hi, x[i]); }
-    lo = warp_min(lo); hi = warp_max(hi);
-    __shared__ float s_lo[kThreads / 32], s_hi[kThreads / 32];
-    if ((threadIdx.x & 31) == 0) { s_lo[threadIdx.x >> 5] = lo; s_hi[threadIdx.x >> 5] = hi; }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        lo = threadIdx.x < kThreads / 32 ? s_lo[threadIdx.x] : INFINITY;
-        hi = threadIdx.x < kThreads / 32 ? s_hi[threadIdx.x] : -INFINITY;
-        lo = warp_min(lo); hi = warp_max(hi);
-        if (threadIdx.x == 0) partials[blockIdx.x] = make_float2(lo, hi);
-    }
+    if (block == 0 && threadIdx.x == 0)
+        for (int64_t i = nv * VEC; i < J.n; ++i) { lo = fminf(lo, x[i]); hi = fmaxf(hi, x[i]); }
+    const float2 r = block_min_max(lo, hi);
+    if (threadIdx.x == 0) J.parts[block] = r;
 }
 
-// One block: combine the partial ranges, emit the parameters for 8 and/or 16 bits.
-__global__ void __launch_bounds__(kThreads) range_finalize_kernel(const float2 *__restrict__ partials, int nparts,
-                                                                  qbp_qparams *qp8, qbp_qparams *qp16)
+// The parameters of an empty tensor.
+__global__ void empty_qparams_kernel(qbp_qparams *qp8, qbp_qparams *qp16)
 {
     pdl_enter();
-    float lo = INFINITY, hi = -INFINITY;
-    for (int i = threadIdx.x; i < nparts; i += kThreads) {
-        float2 p = partials[i];
-        lo = fminf(lo, p.x); hi = fmaxf(hi, p.y);
-    }
-    lo = warp_min(lo); hi = warp_max(hi);
-    __shared__ float s_lo[kThreads / 32], s_hi[kThreads / 32];
-    if ((threadIdx.x & 31) == 0) { s_lo[threadIdx.x >> 5] = lo; s_hi[threadIdx.x >> 5] = hi; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 0; w < kThreads / 32; ++w) { lo = fminf(lo, s_lo[w]); hi = fmaxf(hi, s_hi[w]); }
-        if (qp8) *qp8 = make_qparams(lo, hi, 8);
-        if (qp16) *qp16 = make_qparams(lo, hi, 16);
-    }
+    if (qp8) *qp8 = make_qparams(0.0f, 0.0f, 8);
+    if (qp16) *qp16 = make_qparams(0.0f, 0.0f, 16);
 }
 
 // ---------------------------------------------- chunk-averaged clamping values
@@ -303,27 +290,25 @@ struct QuantOut {
     uint32_t lo_flip;
 };
 
-struct QParamsReg { float inv, zp_u; };
-
-__device__ __forceinline__ QParamsReg load_qp(const qbp_qparams *qp, int bits)
-{
-    QParamsReg r;
-    r.inv = __fdiv_rn(1.0f, qp->scale);
-    r.zp_u = (float)(qp->zero_point + (1 << (bits - 1)));
-    return r;
-}
+// One tensor of a quantising launch.
+struct QuantJob {
+    const float *x; int64_t n; int cols;
+    RangeSrc r;                  // per channel: the records [cols] at r.qp8 / r.qp16
+    uint32_t id8, id16; QuantOut o; int smem_cols; uint64_t index_base;
+};
 
 // Scalar path: unaligned tensors, per-element tails.  One Philox block per element.
 template <bool SR>
-__device__ __forceinline__ void quantize_scalar(const float *x, int64_t i, int cols, bool perch,
-                                                const qbp_qparams *qp8, uint32_t id8, const qbp_qparams *qp16,
-                                                uint32_t id16, const PhiloxKeys &key, const QuantOut &o, uint64_t index_base)
+__device__ __forceinline__ void quantize_scalar(const QuantJob &J, int64_t i, bool perch, const QParamsReg &t8, const QParamsReg &t16,
+                                                const PhiloxKeys &key)
 {
-    const int c = perch ? (int)(i % cols) : 0;
-    const float v = x[i];
-    const uint64_t j = ((uint64_t)i + index_base) >> 2;          // (index_base is a multiple of 4: word i & 3 is unchanged)
+    const QuantOut &o = J.o;
+    const uint32_t id8 = J.id8, id16 = J.id16;
+    const int c = perch ? (int)(i % J.cols) : 0;
+    const float v = J.x[i];
+    const uint64_t j = ((uint64_t)i + J.index_base) >> 2;          // (index_base is a multiple of 4: word i & 3 is unchanged)
     if (o.q8) {
-        QParamsReg p = load_qp(qp8 + c, 8);
+        const QParamsReg p = perch ? qparams_reg(J.r.qp8[c], 8) : t8;
         uint32_t rnd = 0;
         if (SR) {
             uint4 b = philox4x32_10(make_uint4((uint32_t)j, (uint32_t)(j >> 32), id8, 0u), key);
@@ -333,7 +318,7 @@ __device__ __forceinline__ void quantize_scalar(const float *x, int64_t i, int c
         o.q8[i] = (int8_t)(quantize_code<SR>(v, p.inv, p.zp_u, 255.0f, rnd) - 128);
     }
     if (o.q16 || o.hi || o.lo) {
-        QParamsReg p = load_qp(qp16 + c, 16);
+        const QParamsReg p = perch ? qparams_reg(J.r.qp16[c], 16) : t16;
         uint32_t rnd = 0;
         if (SR) {
             uint4 b = philox4x32_10(make_uint4((uint32_t)j, (uint32_t)(j >> 32), id16, 0u), key);
@@ -372,35 +357,35 @@ __device__ __forceinline__ uint32_t pack_bytes2(const uint32_t (&c)[4])
 // count when rounding stochastically) carries none of the per-channel parameter handling.
 // TOTALS: the instance that also leaves the per-channel totals (the others carry none of that work).
 template <bool SR, int VEC, bool PERCH, bool TOTALS>
-__global__ void __launch_bounds__(kThreads) quantize_kernel(const float *__restrict__ x, int64_t n, int cols,
-                                                            const qbp_qparams *__restrict__ qp8,
-                                                            uint32_t id8, const qbp_qparams *__restrict__ qp16,
-                                                            uint32_t id16, const __grid_constant__ PhiloxKeys keys,
-                                                            QuantOut o, int smem_cols, uint64_t index_base)
+__device__ __forceinline__ void quantize_body(const QuantJob &J, const PhiloxKeys &keys, int block, int blocks)
 {
-    pdl_enter();
-    if (VEC == 1) {
-        const int64_t stride = (int64_t)gridDim.x * kThreads;
-        for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += stride)
-            quantize_scalar<SR>(x, i, cols, PERCH, qp8, id8, qp16, id16, keys, o, index_base);
-        return;
-    }
+    const float *__restrict__ x = J.x;
+    const int64_t n = J.n;
+    const int cols = J.cols, smem_cols = J.smem_cols;
+    const QuantOut &o = J.o;
+    const uint32_t id8 = J.id8, id16 = J.id16;
+    const uint64_t index_base = J.index_base;
     const bool want8 = o.q8 != nullptr, want16 = o.q16 || o.hi || o.lo;
     QParamsReg p8 = {0, 0}, p16 = {0, 0};
+    if (!PERCH) resolve_range(J.r, want8, want16, block == 0, p8, p16);
+    const QParamsReg t8 = p8, t16 = p16;
+    if (VEC == 1) {
+        const int64_t stride = (int64_t)blocks * kThreads;
+        for (int64_t i = (int64_t)block * kThreads + threadIdx.x; i < n; i += stride) quantize_scalar<SR>(J, i, PERCH, t8, t16, keys);
+        return;
+    }
     // per channel: (1/scale, zero-point) of every channel once per block in shared memory (when the launcher
     // gave it room), instead of a division per element
     extern __shared__ float2 s_qp[];                         // [cols] for 8 bits, then [cols] for 16 bits
     const bool table = PERCH && smem_cols > 0;
     if (table) {
         for (int c = threadIdx.x; c < cols; c += kThreads) {
-            if (want8)  { QParamsReg t = load_qp(qp8 + c, 8);   s_qp[c] = make_float2(t.inv, t.zp_u); }
-            if (want16) { QParamsReg t = load_qp(qp16 + c, 16); s_qp[cols + c] = make_float2(t.inv, t.zp_u); }
+            if (want8)  { QParamsReg t = qparams_reg(J.r.qp8[c], 8);   s_qp[c] = make_float2(t.inv, t.zp_u); }
+            if (want16) { QParamsReg t = qparams_reg(J.r.qp16[c], 16); s_qp[cols + c] = make_float2(t.inv, t.zp_u); }
         }
         __syncthreads();
     }
     if (!PERCH) {
-        if (want8) p8 = load_qp(qp8, 8);
-        if (want16) p16 = load_qp(qp16, 16);
         // the stochastic codes are taken in fixed point with 16 fraction bits: fold the factor into the parameters
         if (SR) { p8.inv *= 65536.0f; p8.zp_u *= 65536.0f; p16.inv *= 65536.0f; p16.zp_u *= 65536.0f; }
     }
@@ -409,8 +394,8 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const float *__restr
     int cs8[4] = {0, 0, 0, 0};                               // this thread's channels: totals of the stored 8-bit codes
     unsigned cs16[4] = {0, 0, 0, 0};                         // ... and of the unsigned 16-bit codes (fewer than 65536 per thread)
     const int64_t nv = n >> 2;
-    const int64_t stride = (int64_t)gridDim.x * kThreads * kUnroll;
-    for (int64_t base = (int64_t)blockIdx.x * kThreads * kUnroll; base < nv; base += stride) {
+    const int64_t stride = (int64_t)blocks * kThreads * kUnroll;
+    for (int64_t base = (int64_t)block * kThreads * kUnroll; base < nv; base += stride) {
         float4 v[kUnroll];
         bool ok[kUnroll];
 #pragma unroll
@@ -444,7 +429,7 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const float *__restr
                 for (int e = 0; e < 4; ++e) {
                     if (PERCH) {
                         if (table) { const float2 t = s_qp[c0 + e]; p8.inv = t.x; p8.zp_u = t.y; }
-                        else p8 = load_qp(qp8 + c0 + e, 8);
+                        else p8 = qparams_reg(J.r.qp8[c0 + e], 8);
                         if (SR) { p8.inv *= 65536.0f; p8.zp_u *= 65536.0f; }
                     }
                     c[e] = SR ? quantize_sr8_byte2(xs[e], p8.inv, p8.zp_u, r[e])
@@ -465,7 +450,7 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const float *__restr
                 for (int e = 0; e < 4; ++e) {
                     if (PERCH) {
                         if (table) { const float2 t = s_qp[cols + c0 + e]; p16.inv = t.x; p16.zp_u = t.y; }
-                        else p16 = load_qp(qp16 + c0 + e, 16);
+                        else p16 = qparams_reg(J.r.qp16[c0 + e], 16);
                         if (SR) { p16.inv *= 65536.0f; p16.zp_u *= 65536.0f; }
                     }
                     // (stochastic: the code sits in the upper half of the word, i.e. bytes 3 and 2)
@@ -505,9 +490,8 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const float *__restr
             }
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        for (int64_t i = nv << 2; i < n; ++i)
-            quantize_scalar<SR>(x, i, cols, PERCH, qp8, id8, qp16, id16, keys, o, index_base);
+    if (block == 0 && threadIdx.x == 0)
+        for (int64_t i = nv << 2; i < n; ++i) quantize_scalar<SR>(J, i, PERCH, t8, t16, keys);
     if (TOTALS && !PERCH && (o.chansum8 || o.chansum16)) {
         // (cols / 4 divides the block size and the grid stride: the thread's channels are 4 * (threadIdx.x mod cols / 4) ...)
         // (a block sees fewer than 65536 rows -- the launcher's rule -- so its totals fit int32)
@@ -517,7 +501,7 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const float *__restr
         const int c0 = 4 * (threadIdx.x & ((cols >> 2) - 1));
         // how many elements this thread quantised per channel: the 16-bit totals were taken over unsigned codes
         int64_t mine = 0;
-        for (int64_t base = (int64_t)blockIdx.x * kThreads * kUnroll; base < nv; base += stride)
+        for (int64_t base = (int64_t)block * kThreads * kUnroll; base < nv; base += stride)
             for (int u = 0; u < kUnroll; ++u) mine += (base + u * kThreads + threadIdx.x < nv) ? 1 : 0;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -532,157 +516,29 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const float *__restr
     }
 }
 
-// Row sums of stored 8-bit codes: a group of G lanes per row (G = smallest power
-// of two covering cols/16, at most 32), 16-byte loads.
-template <bool IS_SIGNED>
-__global__ void __launch_bounds__(kThreads) rowsum_kernel(const uint8_t *__restrict__ q, int64_t rows, int cols,
-                                                          int G, int32_t *__restrict__ sums)
+template <bool SR, int VEC, bool PERCH, bool TOTALS>
+__global__ void __launch_bounds__(kThreads) quantize_kernel(const __grid_constant__ QuantJob J, const __grid_constant__ PhiloxKeys keys)
 {
     pdl_enter();
-    const int lane = threadIdx.x & 31;
-    const int gl = lane % G;
-    const int64_t groups_per_block = kThreads / G;
-    const int cv = cols >> 4;
-    for (int64_t r = (int64_t)blockIdx.x * groups_per_block + threadIdx.x / G; r < rows;
-         r += (int64_t)gridDim.x * groups_per_block) {
-        int acc = 0;
-        const uint4 *row = reinterpret_cast<const uint4 *>(q + r * cols);
-        for (int c = gl; c < cv; c += G) {
-            uint4 v = __ldg(row + c);
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                acc = IS_SIGNED ? __dp4a((int)w[k], 0x01010101, acc) : (int)__dp4a(w[k], 0x01010101u, (uint32_t)acc);
-        }
-        for (int o = G >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (gl == 0) sums[r] = acc;
-    }
+    quantize_body<SR, VEC, PERCH, TOTALS>(J, keys, (int)blockIdx.x, (int)gridDim.x);
 }
 
-// Column sums (over rows) of stored 8-bit codes (signed or unsigned) into int64.  blockIdx.y
-// selects a slab of up to 256 column groups (16 codes each); inside a slab a
-// thread owns one group and every (256 / groups)-th row.  Block partials meet in
-// shared memory, then one atomic per column and block.  The destination must be
-// zeroed beforehand.
-template <bool IS_SIGNED>
-__global__ void __launch_bounds__(kThreads) colsum_kernel(const uint8_t *__restrict__ q, int64_t rows, int cols,
-                                                          unsigned long long *__restrict__ sums)
+// A layer's weights (the first b_blocks blocks) and activation in one launch; nearest rounding, per tensor.
+template <bool TOTALS>
+__global__ void __launch_bounds__(kThreads) quantize_pair_kernel(const __grid_constant__ QuantJob a, const __grid_constant__ QuantJob b, int b_blocks)
 {
     pdl_enter();
-    const int cv = cols >> 4;
-    const int slab0 = blockIdx.y * kThreads;                 // first column group of this slab
-    const int tw = (cv - slab0) < kThreads ? (cv - slab0) : kThreads;
-    const int rpb = kThreads / tw;
-    const int tx = threadIdx.x % tw, ty = threadIdx.x / tw;
-    __shared__ int s_acc[kThreads * 16];
-    for (int c = threadIdx.x; c < tw * 16; c += kThreads) s_acc[c] = 0;
-    __syncthreads();
-    if (ty < rpb) {
-        int acc[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) acc[e] = 0;
-        for (int64_t r = (int64_t)blockIdx.x * rpb + ty; r < rows; r += (int64_t)gridDim.x * rpb) {
-            uint4 v = __ldg(reinterpret_cast<const uint4 *>(q + r * cols) + slab0 + tx);
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-#pragma unroll
-                for (int b = 0; b < 4; ++b)
-                    acc[k * 4 + b] += IS_SIGNED ? (int)(int8_t)(w[k] >> (8 * b)) : (int)((w[k] >> (8 * b)) & 0xFFu);
-        }
-#pragma unroll
-        for (int e = 0; e < 16; ++e) atomicAdd(&s_acc[tx * 16 + e], acc[e]);
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c < tw * 16; c += kThreads)
-        atomicAdd(&sums[slab0 * 16 + c], (unsigned long long)(long long)s_acc[c]);
+    const PhiloxKeys none = {};
+    if ((int)blockIdx.x < b_blocks) quantize_body<false, 4, false, false>(b, none, (int)blockIdx.x, b_blocks);
+    else                            quantize_body<false, 4, false, TOTALS>(a, none, (int)blockIdx.x - b_blocks, (int)gridDim.x - b_blocks);
 }
 
-// The sums of up to four code tensors in one launch (see SumJob).  Unsigned codes are summed as codes - 128 (top bit
-// flipped) and 128 per code is added at the end, so that one form of the dot product serves both.
-// Per row: a group of G lanes per row, four 16-byte loads in flight.  Per column: a block takes a strip of 128 columns
-// (eight 16-byte groups across, 32 rows high) over one piece of the rows, eight rows in flight per thread; its rows
-// meet by shuffle and in 4 KB of shared memory.
-// Bound by the read of the codes (134 MB for the operands of an 8192^3 product: 24 us with their launch, where a launch per
-// operand, a memset and a launch for the correction terms took 57).
-struct SumJobDev { const uint8_t *q; int64_t rows; int cols, over_rows, first, blocks, G, pieces; uint32_t flip; int32_t *out; };
-struct SumJobs { SumJobDev j[4]; int count; };
-__global__ void __launch_bounds__(kThreads) code_sums_kernel(const __grid_constant__ SumJobs J)
+// The sums of up to eight code tensors in a launch of their own (see qbp_sums.cuh).
+__global__ void __launch_bounds__(kSumThreads) code_sums_kernel(const __grid_constant__ SumJobs J)
 {
     pdl_enter();
-    int k = 0;
-    while (k + 1 < J.count && (int)blockIdx.x >= J.j[k + 1].first) ++k;
-    const SumJobDev &j = J.j[k];
-    const int bid = (int)blockIdx.x - j.first, cv = j.cols >> 4, lane = threadIdx.x & 31;
-    const uint32_t flip = j.flip;
-    if (!j.over_rows) {
-        const int G = j.G, gl = lane % G;
-        const int groups_per_block = kThreads / G;
-        // (the loop bound is the block's, so that the shuffles see whole warps)
-        for (int64_t rb = (int64_t)bid * groups_per_block; rb < j.rows; rb += (int64_t)j.blocks * groups_per_block) {
-            const int64_t r = rb + threadIdx.x / G;
-            const bool in = r < j.rows;
-            const uint4 *row = reinterpret_cast<const uint4 *>(j.q + (in ? r : 0) * j.cols);
-            int acc = 0;
-            auto add = [&](const uint4 &v) {
-                acc = __dp4a((int)(v.x ^ flip), 0x01010101, acc); acc = __dp4a((int)(v.y ^ flip), 0x01010101, acc);
-                acc = __dp4a((int)(v.z ^ flip), 0x01010101, acc); acc = __dp4a((int)(v.w ^ flip), 0x01010101, acc);
-            };
-            int c = in ? gl : cv;
-            for (; c + 3 * G < cv; c += 4 * G) {
-                uint4 v[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) v[u] = __ldg(row + c + u * G);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) add(v[u]);
-            }
-            for (; c < cv; c += G) add(__ldg(row + c));
-            for (int o = G >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (in && gl == 0) j.out[r] = acc + (flip ? 128 * j.cols : 0);
-        }
-        return;
-    }
-    __shared__ int s_acc[kThreads / 32][128];
-    const int strips = (cv + 7) / 8, strip = bid % strips, piece = bid / strips;
-    const int64_t r_begin = j.rows * piece / j.pieces, r_end = j.rows * (piece + 1) / j.pieces;
-    const int g = strip * 8 + (lane & 7), ty = (int)(threadIdx.x >> 5) * 4 + (lane >> 3);
-    int acc[16];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) acc[e] = 0;
-    if (g < cv) {
-        constexpr int U = 8;
-        const uint8_t *base = j.q + (int64_t)g * 16;
-        for (int64_t r = r_begin + ty; r < r_end; r += 32 * U) {
-            uint4 v[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (r + 32 * u < r_end) v[u] = __ldg(reinterpret_cast<const uint4 *>(base + (r + 32 * u) * j.cols));
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (r + 32 * u >= r_end) break;
-                const uint32_t w[4] = {v[u].x ^ flip, v[u].y ^ flip, v[u].z ^ flip, v[u].w ^ flip};
-#pragma unroll
-                for (int e = 0; e < 16; ++e) acc[e] = __dp4a((int)w[e >> 2], 1 << (8 * (e & 3)), acc[e]);
-            }
-        }
-    }
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 8);
-        acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 16);
-    }
-    if (lane < 8) {
-#pragma unroll
-        for (int e = 0; e < 16; ++e) s_acc[threadIdx.x >> 5][lane * 16 + e] = acc[e];
-    }
-    __syncthreads();
-    const int c = strip * 128 + (int)threadIdx.x;
-    if (threadIdx.x < 128 && c < j.cols) {
-        int sum = 0;
-#pragma unroll
-        for (int w = 0; w < kThreads / 32; ++w) sum += s_acc[w][threadIdx.x];
-        j.out[(int64_t)piece * j.cols + c] = sum + (flip ? 128 * (int)(r_end - r_begin) : 0);
-    }
+    run_zero_jobs(J.zero, (int64_t)blockIdx.x * kSumThreads + threadIdx.x, (int64_t)gridDim.x * kSumThreads);
+    code_sums_block(J, (int)blockIdx.x);
 }
 
 // ----------------------------------------------------------------- launchers
@@ -695,30 +551,52 @@ int sum_pieces(int64_t rows, int64_t cols)
     return (int)std::max<int64_t>(p, (rows >> 22) + 1);
 }
 
-int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st)
+// The same for the edges of N images: some 256 positions of the longest edge each, at most 16.
+int edge_pieces(int64_t rows, int H, int W)
 {
-    SumJobs J{};
+    const int64_t longest = rows / ((int64_t)H * W) * std::max(H, W);
+    return (int)std::max<int64_t>(std::max<int64_t>(1, std::min<int64_t>(16, longest / 256)), (longest >> 22) + 1);
+}
+
+int fill_sum_jobs(const SumJob *jobs, int count, SumJobs &J, int *blocks)
+{
     int first = 0;
     for (int i = 0; i < count; ++i) {
         const SumJob &s = jobs[i];
         if (s.cols % 16 || !aligned16(s.q)) return fail(QBP_ERR_INVALID_ARG, "code sums need 16-byte aligned rows (cols %% 16 == 0)");
         SumJobDev &j = J.j[i];
-        j.q = static_cast<const uint8_t *>(s.q); j.rows = s.rows; j.cols = (int)s.cols; j.over_rows = s.over_rows; j.out = s.out;
-        j.flip = s.is_signed ? 0u : 0x80808080u; j.first = first; j.G = 1; j.pieces = 1;
-        if (s.over_rows) {
-            j.pieces = sum_pieces(s.rows, s.cols);
-            j.blocks = j.pieces * (int)((s.cols + 127) / 128);
-        } else {
+        j.q = static_cast<const uint8_t *>(s.q); j.rows = s.rows; j.cols = (int)s.cols; j.kind = s.kind; j.out = s.out; j.out64 = s.out64;
+        j.flip = s.is_signed ? 0u : 0x80808080u; j.first = first; j.G = 1; j.pieces = 1; j.H = s.H; j.W = s.W;
+        while ((16 << j.lg_log2) < s.cols && j.lg_log2 < 3) ++j.lg_log2;
+        const int strips = (int)((s.cols / 16 + (1 << j.lg_log2) - 1) >> j.lg_log2);
+        if (s.kind == kSumRows) {
             while (j.G < 32 && j.G < s.cols / 16) j.G <<= 1;
-            const int64_t groups = kThreads / j.G;
+            const int64_t groups = kSumThreads / j.G;
             j.blocks = (int)std::max<int64_t>(1, std::min<int64_t>((s.rows + groups - 1) / groups, 4ll * sm_count()));
+        } else {
+            j.pieces = s.kind == kSumCols ? sum_pieces(s.rows, s.cols) : edge_pieces(s.rows, s.H, s.W);
+            j.blocks = strips * (s.kind == kSumCols ? j.pieces : 4 * j.pieces + 4);
         }
         first += j.blocks;
     }
     J.count = count;
-    if (first == 0) return QBP_OK;
+    *blocks = first;
+    return QBP_OK;
+}
+
+int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st, const ZeroJobs &zero)
+{
+    if (count == 0) {
+        for (int k = 0; k < 2; ++k)
+            if (zero.words[k]) QBP_CUDA_OK(cudaMemsetAsync(zero.p[k], 0, sizeof(uint32_t) * (size_t)zero.words[k], st));
+        return QBP_OK;
+    }
+    SumJobs J{};
+    int blocks = 0;
+    if (int rc = fill_sum_jobs(jobs, count, J, &blocks)) return rc;
+    J.zero = zero;
     QBP_TRACE_BEGIN(st);
-    launch(code_sums_kernel, first, kThreads, 0, st, J);
+    launch(code_sums_kernel, blocks, kSumThreads, 0, st, J);
     QBP_LAUNCH_OK("code_sums_kernel");
     return QBP_OK;
 }
@@ -731,37 +609,43 @@ static int grid_for(int bps, int64_t n_groups)
     return (int)(g < 1 ? 1 : g);
 }
 
-// after_range (nullable): recorded on the stream once the parameters are enqueued -- a caller that has work for
-// another stream which needs only them (and not the codes) starts it from there.
-static int launch_range(const float *x, int64_t n, float2 *partials, qbp_qparams *qp8, qbp_qparams *qp16,
-                        cudaStream_t st, cudaEvent_t after_range = nullptr, int keep_rev = 0)
+// Blocks of the scan of one tensor: one wave at most.
+static int scan_blocks(int64_t n, bool vec)
 {
-    int nparts = 0;
-    if (n > 0) {
-        const bool vec = aligned16(x);
-        const int64_t per_block = (int64_t)kThreads * kRangeUnroll * (vec ? 4 : 1);
-        nparts = grid_for(vec ? blocks_per_sm(range_partial_kernel<4>, kThreads) : blocks_per_sm(range_partial_kernel<1>, kThreads),
-                          (n + per_block - 1) / per_block);
-        if (nparts > kMaxParts) nparts = kMaxParts;
-        QBP_TRACE_BEGIN(st);
-        if (vec) launch(range_partial_kernel<4>, nparts, kThreads, 0, st, x, n, partials, keep_rev);
-        else     launch(range_partial_kernel<1>, nparts, kThreads, 0, st, x, n, partials, keep_rev);
-        QBP_LAUNCH_OK("range_partial_kernel");
-    }
+    if (n <= 0) return 0;
+    const int64_t per_block = (int64_t)kThreads * kRangeUnroll * (vec ? 4 : 1);
+    const int g = grid_for(vec ? blocks_per_sm(range_partial_kernel<4>, kThreads) : blocks_per_sm(range_partial_kernel<1>, kThreads), (n + per_block - 1) / per_block);
+    return std::min(g, kMaxParts);
+}
+
+// Leaves *nparts (min, max) pairs of the n elements at `partials`.
+static int launch_range(const float *x, int64_t n, float2 *partials, int *nparts, cudaStream_t st, const ZeroJobs &zero = ZeroJobs{})
+{
+    const bool vec = aligned16(x);
+    const ScanJob a{x, n, partials, scan_blocks(n, vec), 0}, none{};
+    *nparts = a.blocks;
+    if (a.blocks == 0) return QBP_OK;
     QBP_TRACE_BEGIN(st);
-    launch(range_finalize_kernel, 1, kThreads, 0, st, partials, nparts, qp8, qp16);
-    QBP_LAUNCH_OK("range_finalize_kernel");
-    if (after_range) QBP_CUDA_OK(cudaEventRecord(after_range, st));
+    if (vec) launch(range_partial_kernel<4>, a.blocks, kThreads, 0, st, a, none, zero);
+    else     launch(range_partial_kernel<1>, a.blocks, kThreads, 0, st, a, none, zero);
+    QBP_LAUNCH_OK("range_partial_kernel");
     return QBP_OK;
 }
 
-// The per-tensor scan for callers in other files: *qp receives the 8-bit parameters of the tensor's range widened to
-// hold 0 (vmin = min(lowest, 0), vmax = max(highest, 0)).
+// The per-tensor scan for callers in other files.
 size_t range_scan_ws_bytes() { return align_up(sizeof(float2) * kMaxParts, 256); }
-int range_scan(const float *x, int64_t n, void *ws, size_t ws_bytes, qbp_qparams *qp, cudaStream_t st)
+int range_scan(const float *x, int64_t n, void *ws, size_t ws_bytes, int *nparts, cudaStream_t st)
 {
     if (!ws || ws_bytes < range_scan_ws_bytes()) return fail(QBP_ERR_WORKSPACE, "range scan: workspace too small");
-    return launch_range(x, n, static_cast<float2 *>(ws), qp, nullptr, st);
+    return launch_range(x, n, static_cast<float2 *>(ws), nparts, st);
+}
+
+static int launch_empty_qparams(qbp_qparams *qp8, qbp_qparams *qp16, cudaStream_t st)
+{
+    QBP_TRACE_BEGIN(st);
+    launch(empty_qparams_kernel, 1, 1, 0, st, qp8, qp16);
+    QBP_LAUNCH_OK("empty_qparams_kernel");
+    return QBP_OK;
 }
 
 static int launch_chan_range(const float *x, int64_t rows, int64_t cols, int bits, float *part_lo, float *part_hi,
@@ -785,34 +669,37 @@ static int launch_chan_range(const float *x, int64_t rows, int64_t cols, int bit
     return QBP_OK;
 }
 
-static int launch_quantize(const float *x, int64_t n, int64_t cols, int perch, int rounding,
-                           const qbp_qparams *qp8, uint32_t id8, const qbp_qparams *qp16, uint32_t id16,
-                           uint64_t seed, const QuantOut &o, cudaStream_t st, uint64_t index_base = 0)
+// Whether a tensor takes the vector path.
+static bool quant_vec(const float *x, int64_t cols, int perch, const QuantOut &o)
+{
+    return aligned16(x) && (!perch || cols % 4 == 0) && (!o.q8 || ((uintptr_t)o.q8 & 3) == 0) && (!o.q16 || ((uintptr_t)o.q16 & 7) == 0) &&
+           (!o.hi || ((uintptr_t)o.hi & 3) == 0) && (!o.lo || ((uintptr_t)o.lo & 3) == 0);
+}
+
+static int launch_quantize(const float *x, int64_t n, int64_t cols, int perch, int rounding, const RangeSrc &r, uint32_t id8,
+                           uint32_t id16, uint64_t seed, const QuantOut &o, cudaStream_t st, uint64_t index_base = 0)
 {
     if (n == 0) return QBP_OK;
-    const bool vec = aligned16(x) && (!perch || cols % 4 == 0) &&
-                     (!o.q8 || ((uintptr_t)o.q8 & 3) == 0) && (!o.q16 || ((uintptr_t)o.q16 & 7) == 0) &&
-                     (!o.hi || ((uintptr_t)o.hi & 3) == 0) && (!o.lo || ((uintptr_t)o.lo & 3) == 0);
+    const bool vec = quant_vec(x, cols, perch, o);
     if (o.rowsum8 && !vec) return fail(QBP_ERR_INVALID_ARG, "quantize: fused row sums need the vector path");
     const int64_t per_block = (int64_t)kThreads * (vec ? 4 * kUnroll : 1);
     const bool sr = rounding == QBP_ROUND_STOCHASTIC;
     const PhiloxKeys key = philox_keys_host(seed);
-    const int c = (int)cols;
     // per-channel parameter table: 2 x cols x 8 bytes of dynamic shared memory when that stays within 32 KB
-    const int smem_cols = (perch && vec && cols <= 2048) ? c : 0;
+    const int smem_cols = (perch && vec && cols <= 2048) ? (int)cols : 0;
     const bool totals = o.chansum8 || o.chansum16;
     // (fewer than 2^22 rows: with a grid of at least one block per SM, or one block per 1024 vectors, a block sees
     // fewer than 65536 of them, and its int32 totals of 16-bit codes cannot overflow)
-    if (totals && !(vec && !perch && cols % 4 == 0 && cols / 4 <= kThreads && ((cols / 4) & (cols / 4 - 1)) == 0 && n / cols < (1ll << 22)))
+    if (totals && !(vec && !perch && quantizer_totals_supported(cols) && n / cols < (1ll << 22)))
         return fail(QBP_ERR_INVALID_ARG, "quantize: per-channel totals need the vector path and cols / 4 a power of two <= %d", kThreads);
-    const size_t smem = totals ? (size_t)cols * 2 * sizeof(int) : (size_t)smem_cols * 2 * sizeof(float2);
+    const size_t smem = !vec ? 0 : totals ? (size_t)cols * 2 * sizeof(int) : (size_t)smem_cols * 2 * sizeof(float2);
     const int64_t groups = (n + per_block - 1) / per_block;
+    const QuantJob J{x, n, (int)cols, r, id8, id16, o, smem_cols, index_base};
 #define QBP_QUANT2(SR_, VEC_, PC_, TOT_)                                                                                \
     do {                                                                                                                \
         const int grid = grid_for(blocks_per_sm(quantize_kernel<SR_, VEC_, PC_, TOT_>, kThreads), groups);              \
         QBP_TRACE_BEGIN(st);                                                                                            \
-        launch(quantize_kernel<SR_, VEC_, PC_, TOT_>, grid, kThreads, (VEC_) == 4 ? smem : 0, st, x, n, c, qp8, id8, qp16, id16,  \
-                                                                                         key, o, (VEC_) == 4 ? smem_cols : 0, index_base); \
+        launch(quantize_kernel<SR_, VEC_, PC_, TOT_>, grid, kThreads, smem, st, J, key);                                \
     } while (0)
 #define QBP_QUANT(SR_, VEC_, PC_) QBP_QUANT2(SR_, VEC_, PC_, false)
     if (totals) {           // (vector path, per tensor: checked above)
@@ -839,40 +726,17 @@ static bool can_fuse_rowsums(const float *x, const void *q8, int64_t cols, const
            (!o.q16 || ((uintptr_t)o.q16 & 7) == 0) && (!o.hi || ((uintptr_t)o.hi & 3) == 0) && (!o.lo || ((uintptr_t)o.lo & 3) == 0);
 }
 
-// Row / column sums of stored codes; used by the quantiser's optional outputs
-// and by the integer products' zero-point corrections.
+// Row / column sums of stored codes, complete.
 int launch_rowsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int32_t *sums, cudaStream_t st)
 {
-    if (rows == 0) return QBP_OK;
-    if (cols % 16 || !aligned16(q)) return fail(QBP_ERR_INVALID_ARG, "row sums need 16-byte aligned rows (cols %% 16 == 0)");
-    int G = 1; while (G < 32 && G < cols / 16) G <<= 1;
-    const int64_t groups = kThreads / G;
-    const int grid = grid_for(is_signed ? blocks_per_sm(rowsum_kernel<true>, kThreads) : blocks_per_sm(rowsum_kernel<false>, kThreads),
-                              (rows + groups - 1) / groups);
-    QBP_TRACE_BEGIN(st);
-    if (is_signed) launch(rowsum_kernel<true>, grid, kThreads, 0, st, (const uint8_t *)q, rows, (int)cols, G, sums);
-    else           launch(rowsum_kernel<false>, grid, kThreads, 0, st, (const uint8_t *)q, rows, (int)cols, G, sums);
-    QBP_LAUNCH_OK("rowsum_kernel");
-    return QBP_OK;
+    const SumJob job{q, rows, cols, kSumRows, is_signed ? 1 : 0, sums};
+    return rows == 0 ? QBP_OK : launch_code_sums(&job, 1, st);
 }
-
 int launch_colsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int64_t *sums, cudaStream_t st)
 {
-    if (cols % 16 || !aligned16(q)) return fail(QBP_ERR_INVALID_ARG, "column sums need cols %% 16 == 0");
-    QBP_CUDA_OK(cudaMemsetAsync(sums, 0, sizeof(int64_t) * cols, st));
-    if (rows == 0) return QBP_OK;
-    const int cv = (int)(cols / 16);
-    const int slabs = (cv + kThreads - 1) / kThreads;
-    const int rpb = kThreads / (cv < kThreads ? cv : kThreads);
-    // each thread keeps int32 partials over at most 2^22 rows: 255 * 2^22 < 2^31
-    int64_t min_blocks = (rows >> 22) + 1;
-    int64_t grid = grid_for(blocks_per_sm(colsum_kernel<true>, kThreads), (rows + rpb - 1) / rpb) / slabs;
-    if (grid < min_blocks) grid = min_blocks;
-    QBP_TRACE_BEGIN(st);
-    if (is_signed) launch(colsum_kernel<true>, dim3((unsigned)grid, (unsigned)slabs), kThreads, 0, st, (const uint8_t *)q, rows, (int)cols, (unsigned long long *)sums);
-    else           launch(colsum_kernel<false>, dim3((unsigned)grid, (unsigned)slabs), kThreads, 0, st, (const uint8_t *)q, rows, (int)cols, (unsigned long long *)sums);
-    QBP_LAUNCH_OK("colsum_kernel");
-    return QBP_OK;
+    const SumJob job{q, rows, cols, kSumCols, is_signed ? 1 : 0, nullptr, 0, 0, sums};
+    QBP_CUDA_OK(cudaMemsetAsync(sums, 0, sizeof(int64_t) * (size_t)cols, st));
+    return rows == 0 ? QBP_OK : launch_code_sums(&job, 1, st);
 }
 
 static int check_common(const float *x, int64_t rows, int64_t cols, int granularity, int rounding,
@@ -898,17 +762,21 @@ static size_t quant_ws_bytes(int64_t cols, int granularity)
 // Shared body of the 8- and 16-bit entry points.
 static int quantize_any(int bits, const float *x, int64_t rows, int64_t cols, int granularity, int rounding,
                         uint64_t seed, uint32_t tensor_id, const qbp_qparams *range_in, const QuantOut &o,
-                        qbp_qparams *qp_out, void *ws, size_t ws_bytes, cudaStream_t st, cudaEvent_t after_range = nullptr,
-                        int keep_rev = 0)
+                        qbp_qparams *qp_out, void *ws, size_t ws_bytes, cudaStream_t st)
 {
     int rc = check_common(x, rows, cols, granularity, rounding, qp_out);
     if (rc) return rc;
     const int perch = granularity == QBP_PER_CHANNEL;
-    if (range_in) {
+    const int64_t n = rows * cols;
+    qbp_qparams *qp8 = bits == 8 ? qp_out : nullptr, *qp16 = bits == 16 ? qp_out : nullptr;
+    RangeSrc r{nullptr, 0, nullptr, qp8, qp16};
+    if (range_in && (perch || n == 0)) {
         const int count = perch ? (int)cols : 1;
         QBP_TRACE_BEGIN(st);
         launch(qparams_from_range_kernel, (count + 255) / 256, 256, 0, st, range_in, count, bits, qp_out);
         QBP_LAUNCH_OK("qparams_from_range_kernel");
+    } else if (range_in) {
+        r.given = range_in;
     } else {
         if (!ws || ws_bytes < quant_ws_bytes(cols, granularity))
             return fail(QBP_ERR_WORKSPACE, "quantize: workspace of %zu bytes needed, %zu given",
@@ -918,13 +786,16 @@ static int quantize_any(int bits, const float *x, int64_t rows, int64_t cols, in
             float *plo = w.take<float>((size_t)kScanMaxStrips * cols);
             float *phi = w.take<float>((size_t)kScanMaxStrips * cols);
             rc = launch_chan_range(x, rows, cols, bits, plo, phi, qp_out, st);
+        } else if (n == 0) {
+            rc = launch_empty_qparams(qp8, qp16, st);
         } else {
             float2 *parts = w.take<float2>(kMaxParts);
-            rc = launch_range(x, rows * cols, parts, bits == 8 ? qp_out : nullptr, bits == 16 ? qp_out : nullptr, st, after_range, keep_rev);
+            rc = launch_range(x, n, parts, &r.nparts, st);
+            r.parts = parts;
         }
         if (rc) return rc;
     }
-    return launch_quantize(x, rows * cols, cols, perch, rounding, qp_out, tensor_id, qp_out, tensor_id, seed, o, st);
+    return launch_quantize(x, n, cols, perch, rounding, r, tensor_id, tensor_id, seed, o, st);
 }
 
 // ------------------------------------------------- built-in scratch (no allocation)
@@ -955,20 +826,17 @@ static int static_scratch_address(void **out)
     return QBP_OK;
 }
 
-// The quantising half of the bifurcation, once qp8 / qp16 are known.
+// The quantising half of the bifurcation.
 static int bifurcate_tail(const float *g, int64_t rows, int64_t cols, uint64_t seed, uint32_t tensor_id8,
-                          uint32_t tensor_id16, int8_t *q8, qbp_qparams *qp8, int32_t *row_sums8, int8_t *hi, uint8_t *lo,
-                          qbp_qparams *qp16, cudaStream_t st, uint64_t index_base = 0, int64_t *tot16 = nullptr,
-                          bool lo_signed = false)
+                          uint32_t tensor_id16, int8_t *q8, const RangeSrc &r, int32_t *row_sums8, int8_t *hi, uint8_t *lo,
+                          cudaStream_t st, uint64_t index_base = 0, int64_t *tot16 = nullptr, bool lo_signed = false)
 {
     QuantOut o = {q8, nullptr, hi, lo, nullptr, 0, 0, nullptr, nullptr, lo_signed ? 0x80808080u : 0u};
-    if (tot16 && rows * cols > 0) {                       // (the caller asked quantizer_totals_supported(cols) first)
-        QBP_CUDA_OK(cudaMemsetAsync(tot16, 0, sizeof(int64_t) * (size_t)cols, st));
+    if (tot16 && rows * cols > 0)                         // (cleared by the caller, who asked quantizer_totals_supported(cols) first)
         o.chansum16 = reinterpret_cast<unsigned long long *>(tot16);
-    }
     const bool fused = row_sums8 && rows * cols > 0 && can_fuse_rowsums(g, q8, cols, o);
     if (fused) { o.rowsum8 = row_sums8; o.rs_group = (int)(cols / 4); o.rs_shift = 31 - __builtin_clz((unsigned)o.rs_group); }
-    int rc = launch_quantize(g, rows * cols, cols, 0, QBP_ROUND_STOCHASTIC, qp8, tensor_id8, qp16, tensor_id16, seed, o, st, index_base);
+    int rc = launch_quantize(g, rows * cols, cols, 0, QBP_ROUND_STOCHASTIC, r, tensor_id8, tensor_id16, seed, o, st, index_base);
     if (rc) return rc;
     if (row_sums8 && !fused) return launch_rowsum(q8, true, rows, cols, row_sums8, st);
     return QBP_OK;
@@ -978,24 +846,10 @@ static int bifurcate_tail(const float *g, int64_t rows, int64_t cols, uint64_t s
 int bifurcate_with_range_partials(const float *g, int64_t rows, int64_t cols, uint64_t seed, uint32_t tensor_id8,
                                   uint32_t tensor_id16, int8_t *q8, qbp_qparams *qp8, int32_t *row_sums8, int8_t *hi,
                                   uint8_t *lo, qbp_qparams *qp16, const float2 *partials, int nparts, cudaStream_t st,
-                                  int64_t *tot16, bool lo_signed, cudaEvent_t after_range)
+                                  int64_t *tot16, bool lo_signed)
 {
-    QBP_TRACE_BEGIN(st);
-    launch(range_finalize_kernel, 1, kThreads, 0, st, partials, nparts, qp8, qp16);
-    QBP_LAUNCH_OK("range_finalize_kernel");
-    if (after_range) QBP_CUDA_OK(cudaEventRecord(after_range, st));
-    return bifurcate_tail(g, rows, cols, seed, tensor_id8, tensor_id16, q8, qp8, row_sums8, hi, lo, qp16, st, 0, tot16, lo_signed);
-}
-
-// The parameters of both copies from per-block (or per-channel) (min, max) pairs.
-int launch_range_finalize(const float2 *partials, int nparts, qbp_qparams *qp8, qbp_qparams *qp16, cudaStream_t st,
-                          cudaEvent_t after_range)
-{
-    QBP_TRACE_BEGIN(st);
-    launch(range_finalize_kernel, 1, kThreads, 0, st, partials, nparts, qp8, qp16);
-    QBP_LAUNCH_OK("range_finalize_kernel");
-    if (after_range) QBP_CUDA_OK(cudaEventRecord(after_range, st));
-    return QBP_OK;
+    return bifurcate_tail(g, rows, cols, seed, tensor_id8, tensor_id16, q8, RangeSrc{partials, nparts, nullptr, qp8, qp16}, row_sums8,
+                          hi, lo, st, 0, tot16, lo_signed);
 }
 
 bool quantizer_totals_supported(int64_t cols)
@@ -1003,23 +857,67 @@ bool quantizer_totals_supported(int64_t cols)
     return cols % 4 == 0 && cols / 4 <= kThreads && ((cols / 4) & (cols / 4 - 1)) == 0;
 }
 
-// The layer's activation quantiser: qbp_quantize_s8 (per tensor, nearest) that also leaves the per-channel totals
-// of the codes (tot8 [cols], zeroed here) when the tensor's shape allows it; *left says whether it did.
-int quantize_s8_with_totals(const float *x, int64_t rows, int64_t cols, int8_t *q, qbp_qparams *qp_out, int32_t *row_sums,
-                            int64_t *tot8, bool *left, void *ws, size_t ws_bytes, cudaStream_t st, cudaEvent_t after_range)
+size_t quantize_operands_ws_bytes() { return 2 * align_up(sizeof(float2) * kMaxParts, 256); }
+int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, size_t ws_bytes, cudaStream_t st)
 {
-    *left = false;
-    QuantOut o = {q, nullptr, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr};
-    const bool fused = row_sums && rows * cols > 0 && can_fuse_rowsums(x, q, cols, o);
-    if (fused) { o.rowsum8 = row_sums; o.rs_group = (int)(cols / 4); o.rs_shift = 31 - __builtin_clz((unsigned)o.rs_group); }
-    if (tot8 && rows * cols > 0 && quantizer_totals_supported(cols) && aligned16(x) && ((uintptr_t)q & 3) == 0) {
-        QBP_CUDA_OK(cudaMemsetAsync(tot8, 0, sizeof(int64_t) * (size_t)cols, st));
-        o.chansum8 = reinterpret_cast<unsigned long long *>(tot8);
-        *left = true;
+    if (!ws || ws_bytes < quantize_operands_ws_bytes()) return fail(QBP_ERR_WORKSPACE, "quantize: workspace too small");
+    WsCarver c(ws, ws_bytes);
+    QuantOperand *ops[2] = {x, w};
+    QuantOut o[2];
+    float2 *parts[2];
+    bool vec[2] = {true, true};
+    ZeroJobs zero{{reinterpret_cast<uint32_t *>(status), nullptr}, {status ? 1 : 0, 0}};
+    for (int i = 0; i < 2; ++i) {
+        parts[i] = c.take<float2>(kMaxParts);
+        if (!ops[i]) continue;
+        QuantOperand &op = *ops[i];
+        if (int rc = check_common(op.v, op.rows, op.cols, QBP_PER_TENSOR, QBP_ROUND_NEAREST, op.qp)) return rc;
+        o[i] = QuantOut{op.q, nullptr, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr, 0u};
+        if (op.row_sums && can_fuse_rowsums(op.v, op.q, op.cols, o[i])) {
+            o[i].rowsum8 = op.row_sums; o[i].rs_group = (int)(op.cols / 4); o[i].rs_shift = 31 - __builtin_clz((unsigned)o[i].rs_group);
+            op.row_sums_left = true;
+        }
+        vec[i] = quant_vec(op.v, op.cols, 0, o[i]);
+        if (op.tot) {
+            zero.p[1] = reinterpret_cast<uint32_t *>(op.tot); zero.words[1] = 2 * op.cols;
+            if (i == 0 && vec[i] && quantizer_totals_supported(op.cols)) { o[i].chansum8 = reinterpret_cast<unsigned long long *>(op.tot); op.tot_left = true; }
+        }
     }
-    int rc = quantize_any(8, x, rows, cols, QBP_PER_TENSOR, QBP_ROUND_NEAREST, 0, 0, nullptr, o, qp_out, ws, ws_bytes, st, after_range, 1);
-    if (rc) return rc;
-    if (row_sums && !fused) return launch_rowsum(q, true, rows, cols, row_sums, st);
+    // the scans (and what they clear on the way), then the codes; the weights ride along with the activation
+    if (x && vec[0] && vec[1]) {
+        const int64_t nx = x->rows * x->cols, nw = w->rows * w->cols;
+        ScanJob a{x->v, nx, parts[0], scan_blocks(nx, true), 1}, b{w->v, nw, parts[1], scan_blocks(nw, true), 0};
+        // one wave in all: each tensor its share
+        const int wave = std::min(kMaxParts, sm_count() * blocks_per_sm(range_partial_kernel<4>, kThreads));
+        if (a.blocks + b.blocks > wave) {
+            b.blocks = std::max(1, std::min(b.blocks, (int)(wave * nw / (nx + nw))));
+            a.blocks = std::min(a.blocks, wave - b.blocks);
+        }
+        QBP_TRACE_BEGIN(st);
+        launch(range_partial_kernel<4>, a.blocks + b.blocks, kThreads, 0, st, a, b, zero);
+        QBP_LAUNCH_OK("range_partial_kernel");
+        const QuantJob ja{x->v, nx, (int)x->cols, RangeSrc{parts[0], a.blocks, nullptr, x->qp, nullptr}, 0, 0, o[0], 0, 0};
+        const QuantJob jb{w->v, nw, (int)w->cols, RangeSrc{parts[1], b.blocks, nullptr, w->qp, nullptr}, 0, 0, o[1], 0, 0};
+        const int64_t per_block = (int64_t)kThreads * 4 * kUnroll;
+        const bool totals = o[0].chansum8 != nullptr;
+        const int qwave = sm_count() * (totals ? blocks_per_sm(quantize_pair_kernel<true>, kThreads) : blocks_per_sm(quantize_pair_kernel<false>, kThreads));
+        int64_t ga = (nx + per_block - 1) / per_block, gb = (nw + per_block - 1) / per_block;
+        if (ga + gb > qwave) { gb = std::max<int64_t>(1, std::min(gb, qwave * nw / (nx + nw))); ga = std::min(ga, qwave - gb); }
+        QBP_TRACE_BEGIN(st);
+        if (totals) launch(quantize_pair_kernel<true>, (int)(ga + gb), kThreads, (size_t)x->cols * 2 * sizeof(int), st, ja, jb, (int)gb);
+        else        launch(quantize_pair_kernel<false>, (int)(ga + gb), kThreads, 0, st, ja, jb, (int)gb);
+        QBP_LAUNCH_OK("quantize_kernel");
+        return QBP_OK;
+    }
+    for (int i = 0; i < 2; ++i) {
+        if (!ops[i]) continue;
+        QuantOperand &op = *ops[i];
+        RangeSrc r{parts[i], 0, nullptr, op.qp, nullptr};
+        int rc = launch_range(op.v, op.rows * op.cols, parts[i], &r.nparts, st, zero);
+        if (rc) return rc;
+        zero = ZeroJobs{};
+        if ((rc = launch_quantize(op.v, op.rows * op.cols, op.cols, 0, QBP_ROUND_NEAREST, r, 0, 0, 0, o[i], st))) return rc;
+    }
     return QBP_OK;
 }
 
@@ -1138,9 +1036,10 @@ extern "C" __attribute__((visibility("default"))) int qbp_bifurcate(const float 
                     quant_ws_bytes(cols, QBP_PER_TENSOR), ws_bytes);
     WsCarver w(ws, ws_bytes);
     float2 *parts = w.take<float2>(kMaxParts);
-    int rc = launch_range(g, rows * cols, parts, qp8, qp16, st);
+    RangeSrc r{parts, 0, nullptr, qp8, qp16};
+    int rc = rows * cols > 0 ? launch_range(g, rows * cols, parts, &r.nparts, st) : launch_empty_qparams(qp8, qp16, st);
     if (rc) return rc;
-    return bifurcate_tail(g, rows, cols, seed, tensor_id8, tensor_id16, q8, qp8, row_sums8, hi, lo, qp16, st);
+    return bifurcate_tail(g, rows, cols, seed, tensor_id8, tensor_id16, q8, r, row_sums8, hi, lo, st);
 }
 
 // Both parameter records from clamping values the caller supplies.
@@ -1163,10 +1062,13 @@ extern "C" __attribute__((visibility("default"))) int qbp_bifurcate_shard(const 
     if (rows * cols > 0 && (!g || !q8 || !hi || !lo)) return fail(QBP_ERR_INVALID_ARG, "bifurcate_shard: NULL tensor");
     if (((uintptr_t)g & 3) != 0) return fail(QBP_ERR_INVALID_ARG, "bifurcate_shard: g is not 4-byte aligned");
     if (index_base % 4) return fail(QBP_ERR_INVALID_ARG, "bifurcate_shard: index_base must be a multiple of 4");
-    QBP_TRACE_BEGIN(st);
-    launch(qparams_pair_from_range_kernel, 1, 1, 0, st, range_in, qp8, qp16);
-    QBP_LAUNCH_OK("qparams_pair_from_range_kernel");
-    return bifurcate_tail(g, rows, cols, seed, tensor_id8, tensor_id16, q8, qp8, row_sums8, hi, lo, qp16, st, index_base);
+    if (rows * cols == 0) {
+        QBP_TRACE_BEGIN(st);
+        launch(qparams_pair_from_range_kernel, 1, 1, 0, st, range_in, qp8, qp16);
+        QBP_LAUNCH_OK("qparams_pair_from_range_kernel");
+        return QBP_OK;
+    }
+    return bifurcate_tail(g, rows, cols, seed, tensor_id8, tensor_id16, q8, RangeSrc{nullptr, 0, range_in, qp8, qp16}, row_sums8, hi, lo, st, index_base);
 }
 
 // out = (float)acc * (sa * sb): the dequantisation of a weight gradient whose int64 accumulators were added up

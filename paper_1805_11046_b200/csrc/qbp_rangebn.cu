@@ -10,6 +10,7 @@
 // outputs the ReLU kept.
 #include "qbp_colscan.cuh"
 #include "qbp_mma.cuh"
+#include "qbp_sums.cuh"
 
 #include <cmath>
 
@@ -124,7 +125,28 @@ __global__ void bn_mean_from_sum_kernel(const double *__restrict__ col_sum, cons
 // a power of two <= 32 that covers the row) receives each row's sum of stored codes, which the next product's
 // zero-point correction needs.
 // chansum (nullable, [C], added to with 64-bit atomics): per-channel totals of the stored codes over all rows.
-struct BnRequant { const qbp_qparams *rq; int8_t *q; int32_t *rowsum; int rs_group; unsigned long long *chansum; };
+// own_range: every block works the range of y out itself (C channels: a microsecond or so; a launch for it takes more), and the
+// first one writes *rq.
+struct BnRequant { qbp_qparams *rq; int8_t *q; int32_t *rowsum; int rs_group; unsigned long long *chansum; int own_range; };
+constexpr int kBnOwnRangeMax = 1024;       // channels up to which it is worth it
+
+// The exact range of y over the channels a thread is given, from the per-channel statistics: y is a monotone function of x in
+// each channel, computed with the same rounded operations, so its extremes sit at x = min and x = max.
+__device__ __forceinline__ float2 bn_out_extremes(const float *mean, const float *vmin, const float *vmax, const float *gamma,
+                                                  const float *beta, int C, float Cn, bool relu, int first, int step, float4 *fold)
+{
+    float lo = INFINITY, hi = -INFINITY;
+    for (int c = first; c < C; c += step) {
+        const float s = bn_scale(vmin[c], vmax[c], Cn);
+        const float g = gamma ? gamma[c] : 1.0f, b = beta ? beta[c] : 0.0f;
+        if (fold) fold[c] = make_float4(mean[c], s, g, b);      // what a product's epilogue needs to normalise a column
+        float a = bn_y(bn_xhat(vmin[c], mean[c], s), g, b);
+        float z = bn_y(bn_xhat(vmax[c], mean[c], s), g, b);
+        if (relu) { a = fmaxf(a, 0.0f); z = fmaxf(z, 0.0f); }
+        lo = fminf(lo, fminf(a, z)); hi = fmaxf(hi, fmaxf(a, z));
+    }
+    return make_float2(lo, hi);
+}
 
 template <int VEC, bool RELU, bool REQUANT>
 __global__ void __launch_bounds__(kScanThreads) bn_apply_kernel(const float *__restrict__ x, int64_t rows, int C, int tw,
@@ -137,6 +159,18 @@ __global__ void __launch_bounds__(kScanThreads) bn_apply_kernel(const float *__r
 {
     pdl_enter();
     const ScanPos p = scan_pos<VEC>(C, tw);
+    float inv = 0.0f, zp_u = 0.0f;
+    if (REQUANT) {
+        qbp_qparams qp;
+        if (R.own_range) {
+            const float2 t = bn_out_extremes(mean, vmin, vmax, gamma, beta, C, Cn, RELU, (int)threadIdx.x, kScanThreads, nullptr);
+            const float2 r = block_min_max(t.x, t.y);
+            qp = make_qparams(r.x, r.y, 8);
+            if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *R.rq = qp;
+        } else qp = *R.rq;
+        const QParamsReg t = qparams_reg(qp, 8);
+        inv = t.inv; zp_u = t.zp_u;
+    }
     // (with row sums the idle threads of a ragged last slab take part in the shuffles: tw <= 32 then, one slab)
     if (!p.active && !(REQUANT && (R.rowsum || R.chansum))) return;
     const int rpb = kScanThreads / tw;
@@ -149,8 +183,6 @@ __global__ void __launch_bounds__(kScanThreads) bn_apply_kernel(const float *__r
         g[e] = gamma ? gamma[c] : 1.0f;
         b[e] = beta ? beta[c] : 0.0f;
     }
-    float inv = 0.0f, zp_u = 0.0f;
-    if (REQUANT) { inv = __fdiv_rn(1.0f, R.rq->scale); zp_u = (float)(R.rq->zero_point + 128); }
     int cs[VEC];                                            // totals of the stored codes of this thread's channels
 #pragma unroll
     for (int e = 0; e < VEC; ++e) cs[e] = 0;
@@ -224,9 +256,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_apply_kernel(const float *__r
     }
 }
 
-// Exact range of y over the whole tensor from the per-channel statistics:
-// y is a non-decreasing (gamma >= 0) or non-increasing function of x computed
-// with the same rounded operations, so its extremes sit at x = min and x = max.
+// The same in a launch of its own.
 __global__ void __launch_bounds__(256) bn_out_range_kernel(const float *__restrict__ mean, const float *__restrict__ vmin,
                                                            const float *__restrict__ vmax,
                                                            const float *__restrict__ gamma,
@@ -235,24 +265,11 @@ __global__ void __launch_bounds__(256) bn_out_range_kernel(const float *__restri
                                                            float4 *__restrict__ fold)
 {
     pdl_enter();
-    float lo = INFINITY, hi = -INFINITY;
-    for (int c = threadIdx.x; c < C; c += 256) {
-        float s = bn_scale(vmin[c], vmax[c], Cn);
-        float g = gamma ? gamma[c] : 1.0f, b = beta ? beta[c] : 0.0f;
-        if (fold) fold[c] = make_float4(mean[c], s, g, b);      // what a product's epilogue needs to normalise a column
-        float a = bn_y(bn_xhat(vmin[c], mean[c], s), g, b);
-        float z = bn_y(bn_xhat(vmax[c], mean[c], s), g, b);
-        if (relu) { a = fmaxf(a, 0.0f); z = fmaxf(z, 0.0f); }
-        lo = fminf(lo, fminf(a, z)); hi = fmaxf(hi, fmaxf(a, z));
-    }
-    lo = warp_min(lo); hi = warp_max(hi);
-    __shared__ float s_lo[8], s_hi[8];
-    if ((threadIdx.x & 31) == 0) { s_lo[threadIdx.x >> 5] = lo; s_hi[threadIdx.x >> 5] = hi; }
-    __syncthreads();
+    const float2 t = bn_out_extremes(mean, vmin, vmax, gamma, beta, C, Cn, relu != 0, (int)threadIdx.x, 256, fold);
+    const float2 r = block_min_max(t.x, t.y);
     if (threadIdx.x == 0) {
-        for (int w = 0; w < 8; ++w) { lo = fminf(lo, s_lo[w]); hi = fmaxf(hi, s_hi[w]); }
-        if (out) { out->scale = 0.0f; out->zero_point = 0; out->vmin = lo; out->vmax = hi; }
-        if (qp8_out) *qp8_out = make_qparams(lo, hi, 8);
+        if (out) { out->scale = 0.0f; out->zero_point = 0; out->vmin = r.x; out->vmax = r.y; }
+        if (qp8_out) *qp8_out = make_qparams(r.x, r.y, 8);
     }
 }
 
@@ -271,9 +288,12 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_stats_kernel(const float 
                                                                     const float *__restrict__ beta, float Cn,
                                                                     double *__restrict__ part_dy,
                                                                     double *__restrict__ part_dyx,
-                                                                    float *__restrict__ ext)
+                                                                    float *__restrict__ ext, const ZeroJobs zero)
 {
     pdl_enter();
+    if (EXT)
+        run_zero_jobs(zero, ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kScanThreads + threadIdx.x,
+                      (int64_t)gridDim.x * gridDim.y * kScanThreads);
     const ScanPos p = scan_pos<VEC>(C, tw);
     const int rpb = kScanThreads / tw;
     double sdy[VEC], sdyx[VEC];
@@ -382,9 +402,10 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_stats_kernel(const float 
     }
 }
 
-// One block of 128 threads per channel: dbeta, dgamma, and the two per-channel
+constexpr int kFinThreads = kSumThreads;
+// One block of kFinThreads threads per channel: dbeta, dgamma, and the two per-channel
 // constants of dx: m1 = gamma*dbeta/n, k2 = C(n)*gamma*dgamma.
-__global__ void __launch_bounds__(128) bn_bwd_finalize_kernel(const double *__restrict__ part_dy,
+__global__ void __launch_bounds__(kFinThreads) bn_bwd_finalize_kernel(const double *__restrict__ part_dy,
                                                               const double *__restrict__ part_dyx, int nparts, int C,
                                                               int64_t n, const float *__restrict__ gamma, double Cn,
                                                               float *__restrict__ dgamma, float *__restrict__ dbeta,
@@ -396,23 +417,26 @@ __global__ void __launch_bounds__(128) bn_bwd_finalize_kernel(const double *__re
                                                               float2 *__restrict__ chan_range = nullptr,
                                                               const float *__restrict__ mean = nullptr,
                                                               const float *__restrict__ beta = nullptr,
-                                                              float2 *__restrict__ relu_thr = nullptr)
+                                                              float2 *__restrict__ relu_thr = nullptr,
+                                                              const __grid_constant__ SumJobs J = SumJobs{})
 {
     pdl_enter();
     const int c = blockIdx.x;
+    // (the blocks behind the channels take code sums that a later product needs: C short blocks leave most SMs idle)
+    if (c >= C) { code_sums_block(J, c - C); return; }
     double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += 128) {
+    for (int i = threadIdx.x; i < nparts; i += kFinThreads) {
         const double pa_ = part_dy[(int64_t)i * C + c], pb_ = part_dyx[(int64_t)i * C + c];
         a += pa_; b += pb_;
     }
     // ext (see bn_bwd_stats_kernel): the extremes of dy over the three sets of positions, then (below) the exact range
     // of this channel's dx, left in chan_range[c] for the quantiser of the gradient
     float ev[6];
-    __shared__ float s_e[6][4];
+    __shared__ float s_e[6][kFinThreads / 32];
     if (ext) {
 #pragma unroll
         for (int k = 0; k < 6; ++k) ev[k] = (k & 1) ? -INFINITY : INFINITY;
-        for (int i = threadIdx.x; i < nparts; i += 128) {
+        for (int i = threadIdx.x; i < nparts; i += kFinThreads) {
             float o[6];
 #pragma unroll
             for (int k = 0; k < 6; ++k) o[k] = ext[((int64_t)k * nparts + i) * C + c];
@@ -430,11 +454,11 @@ __global__ void __launch_bounds__(128) bn_bwd_finalize_kernel(const double *__re
         a += __shfl_xor_sync(0xffffffffu, a, o);
         b += __shfl_xor_sync(0xffffffffu, b, o);
     }
-    __shared__ double s_a[4], s_b[4];
+    __shared__ double s_a[kFinThreads / 32], s_b[kFinThreads / 32];
     if ((threadIdx.x & 31) == 0) { s_a[threadIdx.x >> 5] = a; s_b[threadIdx.x >> 5] = b; }
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < 4; ++w) { a += s_a[w]; b += s_b[w]; }
+        for (int w = 1; w < kFinThreads / 32; ++w) { a += s_a[w]; b += s_b[w]; }
         if (sum_dy) {                       // raw sums only: combined over several GPUs before the coefficients
             sum_dy[c] = a; sum_dyx[c] = b;
             return;
@@ -450,7 +474,7 @@ __global__ void __launch_bounds__(128) bn_bwd_finalize_kernel(const double *__re
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 float lo = ev[2 * k], hi = ev[2 * k + 1];
-                for (int w = 1; w < 4; ++w) { lo = fminf(lo, s_e[2 * k][w]); hi = fmaxf(hi, s_e[2 * k + 1][w]); }
+                for (int w = 1; w < kFinThreads / 32; ++w) { lo = fminf(lo, s_e[2 * k][w]); hi = fmaxf(hi, s_e[2 * k + 1][w]); }
                 if (lo <= hi) {              // (a set with no position keeps +inf, -inf)
                     const float ind = k == 0 ? 0.0f : k == 1 ? 1.0f : -1.0f;
                     const float v0 = bn_dx(lo, ind, s, gf, m1, k2), v1 = bn_dx(hi, ind, s, gf, m1, k2);
@@ -485,7 +509,7 @@ __global__ void __launch_bounds__(kScanThreads, 3) bn_bwd_apply_bifurcate_kernel
     const float *__restrict__ dy, const float *__restrict__ x, int64_t rows, int C, int tw, const float *__restrict__ mean,
     const float *__restrict__ vmin, const float *__restrict__ vmax, const float *__restrict__ gamma,
     const float *__restrict__ beta, float Cn, const float2 *__restrict__ coef, float *__restrict__ g_out,
-    const qbp_qparams *__restrict__ qp8, const qbp_qparams *__restrict__ qp16, uint32_t id8, uint32_t id16,
+    const RangeSrc range, uint32_t id8, uint32_t id16,
     const __grid_constant__ PhiloxKeys keys, uint32_t *__restrict__ q8, uint32_t *__restrict__ q_hi, uint32_t *__restrict__ q_lo,
     uint32_t lo_flip, int32_t *__restrict__ rowsum8, unsigned long long *__restrict__ chansum16,
     const float2 *__restrict__ relu_thr)
@@ -509,8 +533,9 @@ __global__ void __launch_bounds__(kScanThreads, 3) bn_bwd_apply_bifurcate_kernel
         thr[e] = th.x; tsg[e] = th.y;
     }
     // both codes in fixed point with 16 fraction bits (quantize_sr8_byte2 / quantize_sr16_top_half)
-    const float inv8 = __fdiv_rn(1.0f, qp8->scale) * 65536.0f, zp8 = (float)(qp8->zero_point + 128) * 65536.0f;
-    const float inv16 = __fdiv_rn(1.0f, qp16->scale) * 65536.0f, zp16 = (float)(qp16->zero_point + 32768) * 65536.0f;
+    QParamsReg q8r, q16r;
+    resolve_range(range, true, true, blockIdx.x == 0 && blockIdx.y == 0, q8r, q16r);
+    const float inv8 = q8r.inv * 65536.0f, zp8 = q8r.zp_u * 65536.0f, inv16 = q16r.inv * 65536.0f, zp16 = q16r.zp_u * 65536.0f;
     const bool one_block = id8 == id16;
     const int64_t step = (int64_t)gridDim.x * rpb;
     // (the loop bound is the block's: every lane takes part in the row-sum shuffles)
@@ -750,13 +775,14 @@ static int bn_fwd_apply_launch(const float *x, int64_t n_rows, int64_t n_stat, i
     const ScanGeom ga = scan_geom(n_rows, C, al, bps);
     const dim3 grid_apply(ga.nbx, ga.slabs);
     const float Cn = (float)(1.0 / std::sqrt(2.0 * std::log((double)n_stat)));
-    if (out_range || requant) {
+    const bool own_range = requant && !out_range && C <= kBnOwnRangeMax;
+    if ((out_range || requant) && !own_range) {
         QBP_TRACE_BEGIN(st);
         launch(bn_out_range_kernel, 1, 256, 0, st, save_mean, save_min, save_max, gamma, beta, (int)C, Cn, relu, out_range,
                                                requant ? rq->qp : nullptr, nullptr);
         QBP_LAUNCH_OK("bn_out_range_kernel");
     }
-    BnRequant R{nullptr, nullptr, nullptr, 1, nullptr};
+    BnRequant R{nullptr, nullptr, nullptr, 1, nullptr, own_range ? 1 : 0};
     bool fused_rowsum = false;
     if (requant) {
         R.rq = rq->qp; R.q = rq->q;
@@ -909,7 +935,8 @@ static int bn_bwd_stats_launch(const float *dy, const float *x, int64_t n_rows, 
                                const float *beta, int relu, const float *save_mean, const float *save_min,
                                const float *save_max, float *dgamma, float *dbeta, float2 *coef, double *sum_dy,
                                double *sum_dyx, double *pa, double *pb, cudaStream_t st, float *ext = nullptr,
-                               float2 *chan_range = nullptr, float2 *relu_thr = nullptr)
+                               float2 *chan_range = nullptr, float2 *relu_thr = nullptr, const ZeroJobs &zero = ZeroJobs{},
+                               const SumJob *extra = nullptr, int extra_count = 0)
 {
     const bool al = aligned16(x) && aligned16(dy);
     const bool v4 = al && C % 4 == 0;
@@ -921,7 +948,7 @@ static int bn_bwd_stats_launch(const float *dy, const float *x, int64_t n_rows, 
     const double Cnd = 1.0 / std::sqrt(2.0 * std::log((double)n_stat));
     const float Cn = (float)Cnd;
     QBP_TRACE_BEGIN(st);
-#define QBP_BN_BSTATS(V, R, E) launch(bn_bwd_stats_kernel<V, R, E>, grid, kScanThreads, 0, st, dy, x, n_rows, (int)C, g.tw, save_mean, save_min, save_max, gamma, beta, Cn, pa, pb, ext)
+#define QBP_BN_BSTATS(V, R, E) launch(bn_bwd_stats_kernel<V, R, E>, grid, kScanThreads, 0, st, dy, x, n_rows, (int)C, g.tw, save_mean, save_min, save_max, gamma, beta, Cn, pa, pb, ext, zero)
     if (ext) {
         if (g.vec != 4) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "rangebn_bwd: the pass with dy extremes needs aligned tensors and C a multiple of 4");
         if (relu) QBP_BN_BSTATS(4, true, true); else QBP_BN_BSTATS(4, false, true);
@@ -930,8 +957,11 @@ static int bn_bwd_stats_launch(const float *dy, const float *x, int64_t n_rows, 
 #undef QBP_BN_BSTATS
     QBP_LAUNCH_OK("bn_bwd_stats_kernel");
     QBP_TRACE_BEGIN(st);
-    launch(bn_bwd_finalize_kernel, (int)C, 128, 0, st, pa, pb, g.nbx, (int)C, n_stat, gamma, Cnd, dgamma, dbeta, coef, sum_dy, sum_dyx,
-                                                   ext, save_min, save_max, Cn, chan_range, save_mean, beta, relu_thr);
+    SumJobs J{};
+    int sum_blocks = 0;
+    if (extra_count) if (int rc = fill_sum_jobs(extra, extra_count, J, &sum_blocks)) return rc;
+    launch(bn_bwd_finalize_kernel, (int)C + sum_blocks, kFinThreads, 0, st, pa, pb, g.nbx, (int)C, n_stat, gamma, Cnd, dgamma, dbeta, coef, sum_dy, sum_dyx,
+                                                   ext, save_min, save_max, Cn, chan_range, save_mean, beta, relu_thr, J);
     QBP_LAUNCH_OK("bn_bwd_finalize_kernel");
     return QBP_OK;
 }
@@ -978,7 +1008,8 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
                                int relu, const float *save_mean, const float *save_min, const float *save_max, float *g_out,
                                float *dgamma, float *dbeta, uint64_t seed, uint32_t id8, uint32_t id16, int8_t *q8,
                                qbp_qparams *qp8, int32_t *row_sums8, int8_t *hi, uint8_t *lo, qbp_qparams *qp16, bool lo_signed,
-                               void *ws, size_t ws_bytes, cudaStream_t st, cudaEvent_t after_range, int64_t *tot16)
+                               void *ws, size_t ws_bytes, cudaStream_t st, int64_t *tot16, void *clear,
+                               int64_t clear_words, const SumJob *extra, int extra_count)
 {
     int rc = check_bn("rangebn_bwd", dy, x, n, C, ws, ws_bytes);
     if (rc) return rc;
@@ -994,23 +1025,23 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
     float *ext = w.take<float>(6 * (size_t)kScanMaxStrips * C);
     float2 *chan_range = w.take<float2>((size_t)C);
     float2 *relu_thr = w.take<float2>((size_t)C);
-    if ((rc = bn_bwd_stats_launch(dy, x, n, n, C, gamma, beta, relu, save_mean, save_min, save_max, dgamma, dbeta, coef, nullptr,
-                                  nullptr, pa, pb, st, ext, chan_range, relu ? relu_thr : nullptr)))
-        return rc;
-    if ((rc = launch_range_finalize(chan_range, (int)C, qp8, qp16, st, after_range))) return rc;
-    if (tot16) QBP_CUDA_OK(cudaMemsetAsync(tot16, 0, sizeof(int64_t) * (size_t)C, st));
     // (three resident blocks per SM by the kernel's launch bounds, whatever the instance)
     const ScanGeom ga = scan_geom(n, C, true, blocks_per_sm(bn_bwd_apply_bifurcate_kernel<true, true, true>, kScanThreads));
+    // each row's code sum by shuffles over the row's lanes of a warp; a row that spans several warps or blocks is
+    // added up from its pieces (integer atomics on the zeroed sums: the result does not depend on the order)
+    ZeroJobs zero{};
+    if (row_sums8 && (ga.tw > 32 || ga.slabs > 1)) { zero.p[0] = reinterpret_cast<uint32_t *>(row_sums8); zero.words[0] = n; }
+    zero.p[1] = static_cast<uint32_t *>(clear); zero.words[1] = clear_words;
+    if ((rc = bn_bwd_stats_launch(dy, x, n, n, C, gamma, beta, relu, save_mean, save_min, save_max, dgamma, dbeta, coef, nullptr,
+                                  nullptr, pa, pb, st, ext, chan_range, relu ? relu_thr : nullptr, zero, extra, extra_count)))
+        return rc;
+    const RangeSrc range{chan_range, (int)C, nullptr, qp8, qp16};
     const dim3 grid(ga.nbx, ga.slabs);
     const float Cn = (float)(1.0 / std::sqrt(2.0 * std::log((double)n)));
     const PhiloxKeys keys = philox_keys_host(seed);
     const uint32_t flip = lo_signed ? 0x80808080u : 0u;
-    // each row's code sum by shuffles over the row's lanes of a warp; a row that spans several warps or blocks is
-    // added up from its pieces (integer atomics on the zeroed sums: the result does not depend on the order)
-    int32_t *row_sums_arg = row_sums8;
-    if (row_sums8 && (ga.tw > 32 || ga.slabs > 1)) QBP_CUDA_OK(cudaMemsetAsync(row_sums8, 0, sizeof(int32_t) * (size_t)n, st));
     QBP_TRACE_BEGIN(st);
-#define QBP_BN_BAB(R, G, T) do { static PerDeviceOnce once_; QBP_SMEM_OPT_IN(once_, (bn_bwd_apply_bifurcate_kernel<R, G, T>), kBabRingBytes); launch(bn_bwd_apply_bifurcate_kernel<R, G, T>, grid, kScanThreads, kBabRingBytes, st, dy, x, n, (int)C, ga.tw, save_mean, save_min, save_max, gamma, beta, Cn, coef, g_out, qp8, qp16, id8, id16, keys, reinterpret_cast<uint32_t *>(q8), reinterpret_cast<uint32_t *>(hi), reinterpret_cast<uint32_t *>(lo), flip, row_sums_arg, reinterpret_cast<unsigned long long *>(tot16), relu_thr); } while (0)
+#define QBP_BN_BAB(R, G, T) do { static PerDeviceOnce once_; QBP_SMEM_OPT_IN(once_, (bn_bwd_apply_bifurcate_kernel<R, G, T>), kBabRingBytes); launch(bn_bwd_apply_bifurcate_kernel<R, G, T>, grid, kScanThreads, kBabRingBytes, st, dy, x, n, (int)C, ga.tw, save_mean, save_min, save_max, gamma, beta, Cn, coef, g_out, range, id8, id16, keys, reinterpret_cast<uint32_t *>(q8), reinterpret_cast<uint32_t *>(hi), reinterpret_cast<uint32_t *>(lo), flip, row_sums8, reinterpret_cast<unsigned long long *>(tot16), relu_thr); } while (0)
 #define QBP_BN_BAB2(R, G) do { if (tot16) QBP_BN_BAB(R, G, true); else QBP_BN_BAB(R, G, false); } while (0)
     if (g_out) { if (relu) QBP_BN_BAB2(true, true); else QBP_BN_BAB2(false, true); }
     else       { if (relu) QBP_BN_BAB2(true, false); else QBP_BN_BAB2(false, false); }

@@ -52,17 +52,18 @@ __device__ __forceinline__ int tern_keep(uint32_t word, float s, float a)
 
 // Sum over `samples` stochastic ternarisations of g: code = sign(g) * (number of samples that keep the element), as
 // int8 (q), and / or as the two byte limbs of the same value as a 16-bit code (hi: 0 or -1, lo: the low byte), which
-// is what the weight-gradient product takes.  *rng holds the tensor's range (s = max(-vmin, vmax)); *qp_out receives
+// is what the weight-gradient product takes.  parts: the range scan's (min, max) pairs (s = max(-vmin, vmax)); *qp_out receives
 // scale = s / samples, zero-point 0, so that scale * code estimates g.
 template <int VEC>
 __global__ void __launch_bounds__(kTbpThreads) stc_ternarize_kernel(const float *__restrict__ g, int64_t n,
-                                                                    const qbp_qparams *__restrict__ rng, int samples,
+                                                                    const float2 *__restrict__ parts, int nparts, int samples,
                                                                     uint32_t tensor_id, const __grid_constant__ PhiloxKeys keys,
                                                                     int8_t *__restrict__ q, int8_t *__restrict__ hi,
                                                                     uint8_t *__restrict__ lo, qbp_qparams *__restrict__ qp_out)
 {
     pdl_enter();
-    const float s = fmaxf(-rng->vmin, rng->vmax);
+    const float2 rng = block_range(parts, nparts);          // (an empty tensor: s = 0)
+    const float s = fmaxf(-fminf(rng.x, 0.0f), fmaxf(rng.y, 0.0f));
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         qbp_qparams r;
         r.scale = s > 0.0f ? __fdiv_rn(s, (float)samples) : 1.0f;
@@ -123,16 +124,16 @@ static int stc_ternarize_impl(const float *g, int64_t n, int samples, uint64_t s
     if (((uintptr_t)g & 3) != 0) return fail(QBP_ERR_INVALID_ARG, "stc_ternarize: g is not 4-byte aligned");
     if (!ws || ws_bytes < tern_ws_bytes())
         return fail(QBP_ERR_WORKSPACE, "stc_ternarize: workspace of %zu bytes needed, %zu given", tern_ws_bytes(), ws_bytes);
-    qbp_qparams *rng = reinterpret_cast<qbp_qparams *>(static_cast<char *>(ws) + range_scan_ws_bytes());
-    int rc = range_scan(g, n, ws, range_scan_ws_bytes(), rng, st);
+    int nparts = 0;
+    int rc = range_scan(g, n, ws, range_scan_ws_bytes(), &nparts, st);
     if (rc) return rc;
     const bool vec = aligned16(g) && (!q || ((uintptr_t)q & 3) == 0) && (!hi || ((uintptr_t)hi & 3) == 0) && (!lo || ((uintptr_t)lo & 3) == 0);
     const int64_t items = vec ? (n + 3) / 4 : n;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((items + kTbpThreads - 1) / kTbpThreads, (int64_t)sm_count() * 8));
     const PhiloxKeys keys = philox_keys_host(seed);
     QBP_TRACE_BEGIN(st);
-    if (vec) launch(stc_ternarize_kernel<4>, grid, kTbpThreads, 0, st, g, n, rng, samples, tensor_id, keys, q, hi, lo, qp_out);
-    else     launch(stc_ternarize_kernel<1>, grid, kTbpThreads, 0, st, g, n, rng, samples, tensor_id, keys, q, hi, lo, qp_out);
+    if (vec) launch(stc_ternarize_kernel<4>, grid, kTbpThreads, 0, st, g, n, static_cast<const float2 *>(ws), nparts, samples, tensor_id, keys, q, hi, lo, qp_out);
+    else     launch(stc_ternarize_kernel<1>, grid, kTbpThreads, 0, st, g, n, static_cast<const float2 *>(ws), nparts, samples, tensor_id, keys, q, hi, lo, qp_out);
     QBP_LAUNCH_OK("stc_ternarize_kernel");
     return QBP_OK;
 }

@@ -23,8 +23,8 @@
 // Convolution: the MMA's 128 rows hold `chunks` filter taps x the input
 // channels of one tap (2 taps x 64 channels, or 1 tap x 128 channels); each
 // tap is its own TMA load of the input, shifted by the tap offset, padding
-// zero-filled.  Zero-points are applied afterwards from per-border-class code
-// sums (a tap near the border sees fewer positions).
+// zero-filled.  Zero-points are applied afterwards from the operands' code sums
+// and those of the images' edges (a tap near the border sees fewer positions).
 //
 // The TMA-issuing lanes run from a small table built once per CTA (one entry per load of a stage); the MMA warp
 // runs whole with an elected issuer and the stage's MMAs fully unrolled for the operand layouts (see
@@ -88,20 +88,15 @@ struct WgradParams {
     int64_t part_stride;             // ma * 128 * bn, padded
     // plain product: code sums over the M rows (acc = raw - zg * sx[k] - zx * (256 * shi[n] + slo[n]) + M * zx * zg)
     CodeSums sx, shi, slo;
+    // convolution: over all positions ([C], [N], [N]) and over the edges of the images ([8][...], see kSumEdges)
+    const long long *cx, *chi, *clo, *ex, *ehi, *elo;
     const qbp_qparams *qx, *qg;
     long long *acc_out; float *dW;
     int dW_vec;                      // dW starts on a 16-byte boundary
     int *status;
     // Convolution: per-channel totals of the stored codes over all positions (x: [C]; the 16-bit gradient codes
-    // 256 * hi + lo: [N]) that the kernels which wrote the codes left.  The class tables then hold the border classes
-    // only, and the interior class is the total minus those.  NULL: the tables hold all sixteen classes.
+    // 256 * hi + lo: [N]) that the kernels which wrote the codes left; NULL: cx / chi / clo hold them.
     const long long *tot_x, *tot_g;
-    // ... and those border classes can be taken by this kernel's epilogue warps while the MMAs run (a few percent of
-    // the positions: the loads hide behind the main loop): cls_x [16][C], cls_hi / cls_lo [16][N] (zeroed beforehand),
-    // the code tensors, and the offset of the CTA's tables in shared memory.  cls_x == NULL: done elsewhere.
-    unsigned long long *cls_x, *cls_hi, *cls_lo;
-    const uint8_t *codes_x, *codes_hi, *codes_lo;
-    uint32_t cls_off;
     // The gradient's per-channel totals from the product itself: when the taps do not fill the last A tile, its first
     // spare chunk is filled with the code 1 once (nothing else writes there), so that the first accumulator row of
     // that chunk is sum over all positions of 1 * g -- MMA rows that were computed and thrown away before.  The
@@ -292,83 +287,6 @@ __device__ __forceinline__ bool wg_mma_dispatch_halo(int nt, int bh, const WgMma
     return wg_mma_loop_halo<R, RBB, (RBB == 128 ? 1 : 4), 4>(A);
 }
 
-// Sixteen per-channel sums from one 16-byte group of codes (dot products that pick one byte each).
-__device__ __forceinline__ void border_add(bool is_signed, const uint4 &v, int *acc)
-{
-    const uint32_t wd[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-            acc[k * 4 + b] = is_signed ? __dp4a((int)wd[k], 1 << (8 * b), acc[k * 4 + b])
-                                       : (int)__dp4a(wd[k], 1u << (8 * b), (unsigned)acc[k * 4 + b]);
-}
-
-// The border classes (first / last row, first / last column, corners; H, W >= 3) of images [img_begin, img_end) of one
-// code tensor of C channels (C / 16 = 2, 4 or 8 groups), by 128 threads (t = 0..127), into tbl [16][C] (shared
-// memory, zeroed).  Thread = (group, slot): it walks every slots-th position of the four edges, two images at a
-// time, with one set of 16 sums per edge in registers.
-__device__ __forceinline__ void wg_border_sums(bool is_signed, const uint8_t *__restrict__ q, int C, int H, int W, int img_begin,
-                                               int img_end, int *tbl, int t)
-{
-    const int cv = C >> 4, slots = 128 / cv;
-    const int g = t % cv, k = t / cv;
-    int top[16], bot[16], lef[16], rig[16];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) { top[e] = 0; bot[e] = 0; lef[e] = 0; rig[e] = 0; }
-    constexpr int U = 2;
-    for (int img0 = img_begin; img0 < img_end; img0 += U) {
-        const uint4 *base[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) base[u] = reinterpret_cast<const uint4 *>(q + (int64_t)min(img0 + u, img_end - 1) * H * W * C) + g;
-        for (int w = 1 + k; w < W - 1; w += slots) {
-            uint4 a[U], b[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) { a[u] = __ldg(base[u] + (int64_t)w * cv); b[u] = __ldg(base[u] + ((int64_t)(H - 1) * W + w) * cv); }
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (img0 + u < img_end) { border_add(is_signed, a[u], top); border_add(is_signed, b[u], bot); }
-        }
-        for (int h = 1 + k; h < H - 1; h += slots) {
-            uint4 a[U], b[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) { a[u] = __ldg(base[u] + (int64_t)h * W * cv); b[u] = __ldg(base[u] + ((int64_t)h * W + W - 1) * cv); }
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (img0 + u < img_end) { border_add(is_signed, a[u], lef); border_add(is_signed, b[u], rig); }
-        }
-        if (k < 4) {
-            // the four corners: classes 5, 9 (first row), 6, 10 (last row)
-            const int h = k < 2 ? 0 : H - 1, w = (k & 1) ? W - 1 : 0;
-            int cor[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) cor[e] = 0;
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (img0 + u < img_end) border_add(is_signed, __ldg(base[u] + ((int64_t)h * W + w) * cv), cor);
-            int *dst = tbl + ((k < 2 ? 1 : 2) | ((k & 1) ? 8 : 4)) * C + g * 16;
-#pragma unroll
-            for (int e = 0; e < 16; ++e)
-                if (cor[e]) atomicAdd(dst + e, cor[e]);
-        }
-    }
-    // the lanes of a warp that hold the same group meet by shuffle (cv is 2, 4 or 8), then one lane per group adds
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        int tt = top[e], bb = bot[e], ll = lef[e], rr = rig[e];
-        for (int off = cv; off < 32; off <<= 1) {
-            tt += __shfl_xor_sync(0xffffffffu, tt, off); bb += __shfl_xor_sync(0xffffffffu, bb, off);
-            ll += __shfl_xor_sync(0xffffffffu, ll, off); rr += __shfl_xor_sync(0xffffffffu, rr, off);
-        }
-        if ((t & 31) < cv) {
-            if (tt) atomicAdd(tbl + 1 * C + g * 16 + e, tt);
-            if (bb) atomicAdd(tbl + 2 * C + g * 16 + e, bb);
-            if (ll) atomicAdd(tbl + 4 * C + g * 16 + e, ll);
-            if (rr) atomicAdd(tbl + 8 * C + g * 16 + e, rr);
-        }
-    }
-}
-
 // One instance per pair of operand layouts: RBA = row bytes of the x chunks, RBB = row bytes of the gradient tiles.
 template <int RBA, int RBB>
 __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_constant__ WgradParams P)
@@ -396,7 +314,6 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
     const uint32_t stage_bytes = a_bytes + 2u * P.b.tile_bytes;
     const bool last_group = ag == P.a_groups - 1;
     const int stages = last_group ? P.stages_last : P.stages, cg = last_group ? P.cg_last : P.cg;
-    const int kk_per_iter = P.kr / 32;
 
     // chunks present in A tile `at`: conv -- taps left in the tap group; plain -- column chunks left in K
     auto chunks_of = [&](int at) {
@@ -523,24 +440,6 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
         // ------------------------------------------------------- epilogue
         const int quad = warp & 3;
         const int row = quad * 32 + lane;
-        if (P.cls_x) {
-            // while the MMAs run: the border classes of this CTA's share of the images (by CTA index, whatever its item)
-            const int t = threadIdx.x - 64;
-            int *tx = reinterpret_cast<int *>(smem + P.cls_off), *th = tx + 16 * P.C, *tl = th + 16 * (int)P.N;
-            for (int i = t; i < 16 * (P.C + 2 * (int)P.N); i += 128) tx[i] = 0;
-            named_barrier(2, 128);
-            const int img_begin = (int)((int64_t)P.Nimg * blockIdx.x / gridDim.x), img_end = (int)((int64_t)P.Nimg * (blockIdx.x + 1) / gridDim.x);
-            wg_border_sums(true, P.codes_x, P.C, P.H, P.W, img_begin, img_end, tx, t);
-            wg_border_sums(true, P.codes_hi, (int)P.N, P.H, P.W, img_begin, img_end, th, t);
-            wg_border_sums(P.lo_signed != 0, P.codes_lo, (int)P.N, P.H, P.W, img_begin, img_end, tl, t);
-            named_barrier(2, 128);
-            for (int i = t; i < 16 * P.C; i += 128)
-                if (tx[i]) atomicAdd(P.cls_x + i, (unsigned long long)(long long)tx[i]);
-            for (int i = t; i < 16 * (int)P.N; i += 128) {
-                if (th[i]) atomicAdd(P.cls_hi + i, (unsigned long long)(long long)th[i]);
-                if (tl[i]) atomicAdd(P.cls_lo + i, (unsigned long long)(long long)tl[i]);
-            }
-        }
         if (P.direct) {
             const int t = threadIdx.x - 64;
             const long long zx = P.qx->zero_point;
@@ -630,270 +529,6 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
     if (warp == 1) { __syncwarp(); tmem_dealloc(tmem_base, (uint32_t)P.tmem_cols); }
 }
 
-// ------------------------------------------------------------ code sums
-// Sums of stored codes per channel and per border class of the pixel the code
-// sits at (bit 1: first row, 2: last row, 4: first column, 8: last column).
-// sums[cls][c] (int64, zeroed beforehand).
-template <bool IS_SIGNED>
-__global__ void __launch_bounds__(256) class_sums_kernel(const uint8_t *__restrict__ q, int pixels, int H, int W,
-                                                         int C, unsigned long long *__restrict__ sums)
-{
-    pdl_enter();
-    extern __shared__ int s_acc[];                       // [16][C]
-    for (int i = threadIdx.x; i < 16 * C; i += 256) s_acc[i] = 0;
-    __syncthreads();
-    const int cv = C >> 4;                               // 16-byte groups per pixel
-    const int tw = cv < 256 ? cv : 256;
-    const int rpb = 256 / tw;
-    const int tx = threadIdx.x % tw, ty = threadIdx.x / tw;
-    constexpr int U = 8;                                 // loads in flight per thread
-    if (ty < rpb) {
-        const int step = (int)gridDim.x * rpb;
-        for (int g = tx; g < cv; g += tw) {
-            int interior[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) interior[e] = 0;
-            for (int p0 = (int)blockIdx.x * rpb + ty; p0 < pixels; p0 += U * step) {
-                uint4 v[U];
-                bool ok[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int p = p0 + u * step;
-                    ok[u] = p < pixels;
-                    if (ok[u]) v[u] = __ldg(reinterpret_cast<const uint4 *>(q + (int64_t)p * C) + g);
-                }
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    if (!ok[u]) continue;
-                    const unsigned p = (unsigned)(p0 + u * step);
-                    const unsigned w = p % (unsigned)W, h = (p / (unsigned)W) % (unsigned)H;
-                    const int cls = (h == 0 ? 1 : 0) | (h == (unsigned)H - 1 ? 2 : 0) | (w == 0 ? 4 : 0) | (w == (unsigned)W - 1 ? 8 : 0);
-                    const uint32_t wd[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-                    if (cls == 0) {
-                        // one byte per dot product: the selector picks it, sign- or zero-extended
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-#pragma unroll
-                            for (int b = 0; b < 4; ++b)
-                                interior[k * 4 + b] = IS_SIGNED ? __dp4a((int)wd[k], 1 << (8 * b), interior[k * 4 + b])
-                                                                : (int)__dp4a(wd[k], 1u << (8 * b), (unsigned)interior[k * 4 + b]);
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-#pragma unroll
-                            for (int b = 0; b < 4; ++b)
-                                atomicAdd(&s_acc[cls * C + g * 16 + k * 4 + b],
-                                          IS_SIGNED ? (int)(int8_t)(wd[k] >> (8 * b)) : (int)((wd[k] >> (8 * b)) & 0xFF));
-                    }
-                }
-            }
-#pragma unroll
-            for (int e = 0; e < 16; ++e) atomicAdd(&s_acc[g * 16 + e], interior[e]);
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 16 * C; i += 256)
-        if (s_acc[i] != 0) atomicAdd(&sums[i], (unsigned long long)(long long)s_acc[i]);
-}
-
-// The same sums, one image row per block step: thread (w, g) owns 16 channels of column w, so its border class
-// in the w direction never changes, and the row's class is the same for the whole block.  The sums over all rows
-// stay in 16 registers; the first and last row of an image (a few percent of the rows) are added to their row sets
-// in shared memory as well.  No division per pixel, and atomics only for those rows.
-// gs = 16-channel groups per block (a power of two, W * gs <= 256); blockIdx.y selects the channel slab.
-template <bool IS_SIGNED>
-__device__ __forceinline__ void row_class_sums_body(const uint8_t *__restrict__ q, int Nimg, int H, int W, int C, int gs,
-                                                    unsigned long long *__restrict__ sums)
-{
-    extern __shared__ int s_acc[];                       // [3 row sets: all, first, last][4 column classes][gs * 16]
-    const int cw = gs * 16;
-    for (int i = threadIdx.x; i < 12 * cw; i += 256) s_acc[i] = 0;
-    __syncthreads();
-    const int w = threadIdx.x / gs, gl = threadIdx.x % gs;
-    const int g = blockIdx.y * gs + gl;
-    const bool active = w < W && g < (C >> 4);
-    const int colclass = (w == 0 ? 1 : 0) | (w == W - 1 ? 2 : 0);
-    const int lane = threadIdx.x & 31;
-    const int64_t row_bytes = (int64_t)W * C;
-    const uint8_t *base = q + (int64_t)(active ? w : 0) * C + (int64_t)(active ? g : 0) * 16;
-    constexpr int U = 8;                                 // rows in flight per thread
-
-    int acc[16];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) acc[e] = 0;
-    const bool interior = active && colclass == 0;
-    {
-        // (every thread walks the rows, the idle ones without loading: the shuffles below need whole warps)
-        const int rows = Nimg * H, step = (int)gridDim.x, hstep = step % H;
-        int h = (int)blockIdx.x % H;
-        for (int r = (int)blockIdx.x; r < rows; r += U * step) {
-            uint4 v[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                v[u] = make_uint4(0, 0, 0, 0);
-                if (active && r + u * step < rows) v[u] = __ldcs(reinterpret_cast<const uint4 *>(base + (int64_t)(r + u * step) * row_bytes));
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (r + u * step >= rows) break;
-                const uint32_t wd[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-#pragma unroll
-                    for (int b = 0; b < 4; ++b)          // one byte per dot product: the selector picks it, sign- or zero-extended
-                        acc[k * 4 + b] = IS_SIGNED ? __dp4a((int)wd[k], 1 << (8 * b), acc[k * 4 + b])
-                                                   : (int)__dp4a(wd[k], 1u << (8 * b), (unsigned)acc[k * 4 + b]);
-                if (active && H > 1 && (h == 0 || h == H - 1)) {
-                    // a first or last row (the same for the whole block, and rare): its codes also go to that row set
-                    int *dst = &s_acc[((h == 0 ? 1 : 2) * 4 + colclass) * cw + gl * 16];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-#pragma unroll
-                        for (int b = 0; b < 4; ++b)
-                            atomicAdd(dst + k * 4 + b, IS_SIGNED ? (int)(int8_t)(wd[k] >> (8 * b)) : (int)((wd[k] >> (8 * b)) & 0xFF));
-                }
-                h += hstep; if (h >= H) h -= H;
-            }
-        }
-    }
-    {
-        // all rows, reduced the same way
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            int r = interior ? acc[e] : 0;
-            for (int off = gs; off < 32; off <<= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
-            const int ch = gl * 16 + e;
-            if (lane < gs && r) atomicAdd(&s_acc[0 * cw + ch], r);
-            if (active && colclass != 0 && acc[e]) atomicAdd(&s_acc[colclass * cw + ch], acc[e]);
-        }
-    }
-    __syncthreads();
-    // exclusive classes (bit 1: first row, 2: last row, 4: first column, 8: last column); a single row is both
-    for (int i = threadIdx.x; i < 4 * cw; i += 256) {
-        const int cc = i / cw, c = (int)blockIdx.y * cw + i % cw;
-        if (c >= C) continue;
-        const int colbits = (cc & 1 ? 4 : 0) | (cc & 2 ? 8 : 0);
-        const int all = s_acc[(0 * 4 + cc) * cw + i % cw], top = s_acc[(1 * 4 + cc) * cw + i % cw], bot = s_acc[(2 * 4 + cc) * cw + i % cw];
-        if (H == 1) {
-            if (all) atomicAdd(&sums[(3 | colbits) * C + c], (unsigned long long)(long long)all);
-        } else {
-            const int mid = all - top - bot;
-            if (mid) atomicAdd(&sums[(0 | colbits) * C + c], (unsigned long long)(long long)mid);
-            if (top) atomicAdd(&sums[(1 | colbits) * C + c], (unsigned long long)(long long)top);
-            if (bot) atomicAdd(&sums[(2 | colbits) * C + c], (unsigned long long)(long long)bot);
-        }
-    }
-}
-
-template <bool IS_SIGNED>
-__global__ void __launch_bounds__(256, 3) row_class_sums_kernel(const uint8_t *__restrict__ q, int Nimg, int H, int W,
-                                                                int C, int gs, unsigned long long *__restrict__ sums)
-{
-    pdl_enter();
-    row_class_sums_body<IS_SIGNED>(q, Nimg, H, W, C, gs, sums);
-}
-
-// The three tensors of a weight gradient with as many input as output channels in one launch (blockIdx.z: the
-// layer input, the gradient's signed high bytes, its unsigned low bytes); sums: three tables of 16 * C, one after another.
-__global__ void __launch_bounds__(256, 3) row_class_sums3_kernel(const uint8_t *__restrict__ x, const uint8_t *__restrict__ hi,
-                                                                 const uint8_t *__restrict__ lo, int Nimg, int H, int W, int C,
-                                                                 int gs, unsigned long long *__restrict__ sums, int lo_signed)
-{
-    pdl_enter();
-    if (blockIdx.z == 0)      row_class_sums_body<true>(x, Nimg, H, W, C, gs, sums);
-    else if (blockIdx.z == 1) row_class_sums_body<true>(hi, Nimg, H, W, C, gs, sums + 16 * C);
-    else if (lo_signed)       row_class_sums_body<true>(lo, Nimg, H, W, C, gs, sums + 32 * C);
-    else                      row_class_sums_body<false>(lo, Nimg, H, W, C, gs, sums + 32 * C);
-}
-
-// The border classes only (first / last row, first / last column and the four corners; H, W >= 3) of the three code
-// tensors of a convolution's weight gradient: a few percent of the positions.  blockIdx.z: the layer input, the
-// gradient's signed high bytes, its unsigned low bytes (tables of 16 * Cx / 16 * Cg / 16 * Cg, zeroed beforehand);
-// blockIdx.x strides over groups of four images.  Thread = (16-channel group g, slot k): it walks positions k,
-// k + slots, ... of each of the four edges (corners excluded) and keeps one set of 16 sums per edge in registers;
-// the corners go straight to shared memory.  Few blocks: each ends with one atomic per table entry.
-__global__ void __launch_bounds__(256) border_class_sums_kernel(const uint8_t *__restrict__ x, const uint8_t *__restrict__ hi,
-                                                                const uint8_t *__restrict__ lo, int Nimg, int H, int W, int Cx,
-                                                                int Cg, unsigned long long *__restrict__ sums_x,
-                                                                unsigned long long *__restrict__ sums_hi,
-                                                                unsigned long long *__restrict__ sums_lo, int lo_signed)
-{
-    pdl_enter();
-    extern __shared__ int s_acc[];                       // [16][C]
-    const uint8_t *q = blockIdx.z == 0 ? x : blockIdx.z == 1 ? hi : lo;
-    unsigned long long *sums = blockIdx.z == 0 ? sums_x : blockIdx.z == 1 ? sums_hi : sums_lo;
-    const int C = blockIdx.z == 0 ? Cx : Cg;
-    const bool is_signed = blockIdx.z != 2 || lo_signed;
-    for (int i = threadIdx.x; i < 16 * C; i += 256) s_acc[i] = 0;
-    __syncthreads();
-    const int cv = C >> 4;
-    const int slots = 256 / cv;                          // (cv <= 256: C <= 4096)
-    const int g = threadIdx.x % cv, k = threadIdx.x / cv;
-    int top[16], bot[16], lef[16], rig[16];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) { top[e] = 0; bot[e] = 0; lef[e] = 0; rig[e] = 0; }
-    if (k < slots) {
-        // four images at a time, all their loads first: the positions are few and far apart, so latency is what counts
-        constexpr int U = 4;
-        for (int img0 = blockIdx.x * U; img0 < Nimg; img0 += gridDim.x * U) {
-            const uint4 *base[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) base[u] = reinterpret_cast<const uint4 *>(q + (int64_t)min(img0 + u, Nimg - 1) * H * W * C) + g;
-            for (int w = 1 + k; w < W - 1; w += slots) {
-                uint4 a[U], b[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) { a[u] = __ldg(base[u] + (int64_t)w * cv); b[u] = __ldg(base[u] + ((int64_t)(H - 1) * W + w) * cv); }
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (img0 + u < Nimg) { border_add(is_signed, a[u], top); border_add(is_signed, b[u], bot); }
-            }
-            for (int h = 1 + k; h < H - 1; h += slots) {
-                uint4 a[U], b[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) { a[u] = __ldg(base[u] + (int64_t)h * W * cv); b[u] = __ldg(base[u] + ((int64_t)h * W + W - 1) * cv); }
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (img0 + u < Nimg) { border_add(is_signed, a[u], lef); border_add(is_signed, b[u], rig); }
-            }
-            if (k < 4) {
-                // the four corners: classes 5, 9 (first row), 6, 10 (last row)
-                const int h = k < 2 ? 0 : H - 1, w = (k & 1) ? W - 1 : 0;
-                int cor[16];
-#pragma unroll
-                for (int e = 0; e < 16; ++e) cor[e] = 0;
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (img0 + u < Nimg) border_add(is_signed, __ldg(base[u] + ((int64_t)h * W + w) * cv), cor);
-                int *dst = s_acc + ((k < 2 ? 1 : 2) | ((k & 1) ? 8 : 4)) * C + g * 16;
-#pragma unroll
-                for (int e = 0; e < 16; ++e)
-                    if (cor[e]) atomicAdd(dst + e, cor[e]);
-            }
-        }
-    }
-    // the lanes of a warp that hold the same channel group meet by shuffle (when cv is a power of two below 32: whole
-    // warps are then inside `k < slots`), then one lane per group adds to the block's table
-    const bool shuffle = cv < 32 && (cv & (cv - 1)) == 0;
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        int t = top[e], b = bot[e], l = lef[e], r = rig[e];
-        if (shuffle)
-            for (int off = cv; off < 32; off <<= 1) {
-                t += __shfl_xor_sync(0xffffffffu, t, off); b += __shfl_xor_sync(0xffffffffu, b, off);
-                l += __shfl_xor_sync(0xffffffffu, l, off); r += __shfl_xor_sync(0xffffffffu, r, off);
-            }
-        if (k < slots && (!shuffle || (threadIdx.x & 31) < cv)) {
-            if (t) atomicAdd(s_acc + 1 * C + g * 16 + e, t);
-            if (b) atomicAdd(s_acc + 2 * C + g * 16 + e, b);
-            if (l) atomicAdd(s_acc + 4 * C + g * 16 + e, l);
-            if (r) atomicAdd(s_acc + 8 * C + g * 16 + e, r);
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 16 * C; i += 256)
-        if (s_acc[i] != 0) atomicAdd(&sums[i], (unsigned long long)(long long)s_acc[i]);
-}
-
 // Adds the CTAs' partials, applies the zero-points and dequantises:
 //   acc = raw - zg * SX - zx * SG + count * zx * zg
 // Plain product [k][n]: SX / SG are the column sums, count = M.  kWgFinalizeLanes lanes per output element share its slices (an
@@ -937,39 +572,32 @@ __global__ void __launch_bounds__(256) wgrad_finalize_kernel(const __grid_consta
     if (P.dW) P.dW[e] = __fmul_rn((float)acc, __fmul_rn(P.qx->scale, P.qg->scale));
 }
 
-// The part of SX (of_x: over the positions of x that tap (r, s) sees) or SG (over the positions of g at which it is inside
-// the image) that four of the sixteen border classes contribute (cls = 4 i + q): with totals, what those classes take off the
-// total; without, what they hold.
-__device__ __forceinline__ long long wg_class_part(const WgradParams &P, bool of_x, int ch, int r, int s, int q,
-                                                   const long long *__restrict__ ta, const long long *__restrict__ tb)
+// SX (of_x: over the positions of x that tap (r, s) sees) or SG (over the positions of g at which it is inside the image) in
+// four parts: all positions, less the row and the column that are out, plus the corner that was taken off twice.
+//   g sees the tap where p - pad + r is in [0, H): not in the first row for r < pad, not in the last for r > pad;
+//   x is seen where h + pad - r is in [0, H):      not in the last row for r < pad, not in the first for r > pad.
+__device__ __forceinline__ long long wg_tap_part(const WgradParams &P, bool of_x, int ch, int r, int s, int part)
 {
-    const int pad = P.pad, width = of_x ? P.C : (int)P.N;
-    const bool totals = P.tot_x != nullptr;
-    long long sum = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int cls = 4 * i + q;
-        const bool top = cls & 1, bottom = cls & 2, left = cls & 4, right = cls & 8;
-        // positions of g that see this tap: p - pad + r in [0,H)  <=>  not (r<pad and first row), not (r>pad and last row);
-        // positions of x that are seen:      h + pad - r in [0,H)  <=>  not (r<pad and last row),  not (r>pad and first row).
-        const bool ok = of_x ? !((r < pad && bottom) || (r > pad && top) || (s < pad && right) || (s > pad && left))
-                             : !((r < pad && top) || (r > pad && bottom) || (s < pad && left) || (s > pad && right));
-        if (ok != totals) {               // (totals: the classes not seen; the interior always is)
-            const long long v = of_x ? ta[cls * width + ch] : 256 * ta[cls * width + ch] + tb[cls * width + ch];
-            sum += totals ? -v : v;
-        }
+    const int dr = r < P.pad ? -1 : r > P.pad ? 1 : 0, ds = s < P.pad ? -1 : s > P.pad ? 1 : 0;
+    if (part == 0 && P.tot_x) {
+        if (of_x) return P.tot_x[ch];
+        return P.tot_g[ch] - (P.lo_signed && P.tot_g_plain ? 128ll * P.Nimg * P.H * P.W : 0);
     }
-    return sum;
+    if (part == 0) return of_x ? P.cx[ch] : 256 * P.chi[ch] + P.clo[ch];
+    if ((part != 2 && dr == 0) || (part != 1 && ds == 0)) return 0;
+    const int row = (dr > 0) != of_x ? 1 : 0, col = (ds > 0) != of_x ? 1 : 0;         // the row / column out: 0 first, 1 last
+    const int edge = part == 1 ? row : part == 2 ? 2 + col : 4 + 2 * row + col;
+    const int64_t at = (int64_t)edge * (of_x ? P.C : P.N) + ch;
+    const long long v = of_x ? P.ex[at] : 256 * P.ehi[at] + P.elo[at];
+    return part == 3 ? v : -v;
 }
 
-// The same for a convolution, output [n][tap][c].  A block takes 64 channels of one tap and NB output channels: the class
-// sums behind SX and SG are added up once per block instead of once per element (thirty and more loads each, which made
-// this kernel 78 us for a 256 -> 256 channel 3x3 filter, five times what its partials take to read), four groups
-// of 64 threads share the slices, each thread with eight loads in flight, and meet in shared memory.
+// The same for a convolution, output [n][tap][c].  A block takes 64 channels of one tap and NB output channels: SX and SG
+// are added up once per block instead of once per element (tens of loads each, which made this kernel 78 us for a
+// 256 -> 256 channel 3x3 filter, five times what its partials take to read), four groups of 64 threads share the slices,
+// each thread with eight loads in flight, and meet in shared memory.
 template <int NB>
-__global__ void __launch_bounds__(256) wgrad_conv_finalize_kernel(const __grid_constant__ WgradParams P, const long long *__restrict__ sx,
-                                                                  const long long *__restrict__ shi,
-                                                                  const long long *__restrict__ slo)
+__global__ void __launch_bounds__(256) wgrad_conv_finalize_kernel(const __grid_constant__ WgradParams P)
 {
     pdl_enter();
     constexpr int U = 8 / NB;                              // slices in flight per output channel
@@ -1014,8 +642,8 @@ __global__ void __launch_bounds__(256) wgrad_conv_finalize_kernel(const __grid_c
     }
 #pragma unroll
     for (int i = 0; i < NB; ++i) s_part[i][q][threadIdx.x & 63] = raw[i];
-    s_sx[q][threadIdx.x & 63] = c_ok ? wg_class_part(P, true, c, r, s, q, sx, nullptr) : 0;
-    if ((threadIdx.x & 63) < NB) s_sg[q][threadIdx.x & 63] = wg_class_part(P, false, min(n0 + (int)(threadIdx.x & 63), (int)P.N - 1), r, s, q, shi, slo);
+    s_sx[q][threadIdx.x & 63] = c_ok ? wg_tap_part(P, true, c, r, s, q) : 0;
+    if ((threadIdx.x & 63) < NB) s_sg[q][threadIdx.x & 63] = wg_tap_part(P, false, min(n0 + (int)(threadIdx.x & 63), (int)P.N - 1), r, s, q);
     __syncthreads();
     // (signed low bytes: the limbs hold g16 - 128, against the zero-point zg - 128)
     const long long zx = P.qx->zero_point, zg = P.qg->zero_point - (P.lo_signed ? 128 : 0);
@@ -1025,11 +653,7 @@ __global__ void __launch_bounds__(256) wgrad_conv_finalize_kernel(const __grid_c
     for (int i = threadIdx.x; i < NB * 64; i += 256) {
         const int cl = i & 63, nl = i >> 6, n = n0 + nl, co = ((int)blockIdx.x % cblocks) * 64 + cl;
         if (n >= P.N || co >= P.C) continue;
-        long long SX = s_sx[0][cl] + s_sx[1][cl] + s_sx[2][cl] + s_sx[3][cl], SG = s_sg[0][nl] + s_sg[1][nl] + s_sg[2][nl] + s_sg[3][nl];
-        if (P.tot_x) {
-            SX += P.tot_x[co]; SG += P.tot_g[n];
-            if (P.lo_signed && P.tot_g_plain) SG -= 128ll * P.Nimg * P.H * P.W;
-        }
+        const long long SX = s_sx[0][cl] + s_sx[1][cl] + s_sx[2][cl] + s_sx[3][cl], SG = s_sg[0][nl] + s_sg[1][nl] + s_sg[2][nl] + s_sg[3][nl];
         const long long acc = s_part[nl][0][cl] + s_part[nl][1][cl] + s_part[nl][2][cl] + s_part[nl][3][cl] - zg * SX - zx * SG + count * zx * zg;
         const int64_t e = ((int64_t)n * P.taps + tap) * P.C + co;
         if (P.acc_out) P.acc_out[e] = acc;
@@ -1065,15 +689,18 @@ struct WgradPlan {
     int bw, bh, bn_img;
 };
 
-// Whether the kernel's epilogue warps can take the border classes themselves: a padded convolution whose x and g
-// tensors have 32, 64 or 128 channels (a pixel is 2, 4 or 8 sixteen-byte groups) and at least 3 x 3 positions.
-static bool wgrad_inline_border(const qbp_conv_desc *d)
-{
-    auto ok = [](int c) { return c == 32 || c == 64 || c == 128; };
-    return d && d->pad > 0 && ok(d->C) && ok(d->K) && d->H >= 3 && d->W >= 3;
-}
-
 }  // namespace qbp
+
+size_t qbp::wgrad_sum_table(const qbp_conv_desc *d) { return d ? (size_t)(d->pad ? 9 : 1) * ((size_t)d->C + 2 * (size_t)d->K) : 0; }
+int qbp::wgrad_sum_jobs(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, const int8_t *x, const int8_t *hi, const uint8_t *lo,
+                        bool lo_signed, int64_t *tab, SumJob (&jobs)[6])
+{
+    const struct { const void *q; int64_t cols; int is_signed; } t[3] = {{x, K, 1}, {hi, N, 1}, {lo, N, lo_signed ? 1 : 0}};
+    for (int i = 0; i < 3; ++i) { jobs[i] = SumJob{t[i].q, M, t[i].cols, kSumCols, t[i].is_signed, nullptr, 0, 0, tab}; if (tab) tab += t[i].cols; }
+    if (!d || !d->pad) return 3;
+    for (int i = 0; i < 3; ++i) { jobs[3 + i] = SumJob{t[i].q, M, t[i].cols, kSumEdges, t[i].is_signed, nullptr, d->H, d->W, tab}; if (tab) tab += 8 * t[i].cols; }
+    return 6;
+}
 
 // Whether the product can take the gradient's per-channel totals itself (a spare chunk in its last A tile).
 bool qbp::wgrad_self_totals(const qbp_conv_desc *d)
@@ -1161,13 +788,11 @@ static void plan_wgrad(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, 
     // pipeline: stages of kr rows; one commit releases `cg` stages (some 24 MMAs between commits while that leaves
     // three groups in the ring).  The CTAs of the last group (fewer A tiles) get a ring of their own shape.
     const int n_last = P.a_tiles - (P.a_groups - 1) * P.ma;                 // A tiles of the last group
-    // (the border-class tables of the epilogue warps sit behind the ring)
-    // (... and behind those the region of ones of the halo variant)
-    const uint32_t cls_only = wgrad_inline_border(d) ? (uint32_t)align_up(sizeof(int) * 16 * (size_t)(K + 2 * N), 1024) : 0u;
-    const uint32_t cls_bytes = cls_only + (P.halo_bh ? P.halo_bytes : 0u);
+    // (the region of ones of the halo variant sits behind the ring)
+    const uint32_t ones_bytes = P.halo_bh ? P.halo_bytes : 0u;
     auto ring = [&](int tiles, int &stages, int &cg) {
         const uint32_t stage_bytes = (P.halo_bh ? P.halo_bytes : P.a_chunk_bytes * P.a_chunks * (uint32_t)tiles) + 2 * P.b.tile_bytes;
-        stages = std::max(2, std::min<int>(kWgMaxStages, (int)((kWgSmem - 1024 - cls_bytes) / stage_bytes)));
+        stages = std::max(2, std::min<int>(kWgMaxStages, (int)((kWgSmem - 1024 - ones_bytes) / stage_bytes)));
         const int mmas = tiles * (int)(kr / 32) * 2;       // (in MMAs of bn columns: a fused one counts twice)
         cg = 1;
         while (cg * mmas < 24 && stages / (cg + 1) >= 3) ++cg;
@@ -1176,9 +801,8 @@ static void plan_wgrad(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, 
     };
     const size_t smem_full = ring(P.ma, P.stages, P.cg);
     const size_t smem_last = ring(n_last, P.stages_last, P.cg_last);
-    P.cls_off = (uint32_t)(std::max(smem_full, smem_last) - 1024);           // behind the longer of the two rings
-    P.ones_off = P.cls_off + cls_only;
-    pl.smem = std::max(smem_full, smem_last) + cls_bytes;
+    P.ones_off = (uint32_t)(std::max(smem_full, smem_last) - 1024);          // behind the longer of the two rings
+    pl.smem = std::max(smem_full, smem_last) + ones_bytes;
     // split of the reductions: at most 65536 rows per CTA; with few items, enough slices to fill the machine
     // once, in proportion to an item's cost per reduction step: a fixed part (waits, the share of a commit)
     // worth about eight MMAs, plus its MMAs
@@ -1206,8 +830,8 @@ static void plan_wgrad(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, 
 
 static size_t wgrad_ws_bytes(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K)
 {
-    const size_t sums = d ? align_up(sizeof(int64_t) * 16 * (size_t)d->C, 256) + 2 * align_up(sizeof(int64_t) * 16 * (size_t)d->K, 256)
-                          : align_up(sizeof(int32_t) * sum_elems(M, K, true), 256) + 2 * align_up(sizeof(int32_t) * sum_elems(M, N, true), 256);
+    const size_t sums = d ? align_up(sizeof(int64_t) * wgrad_sum_table(d), 256)
+                          : align_up(sizeof(int32_t) * sum_elems(M, K, kSumCols), 256) + 2 * align_up(sizeof(int32_t) * sum_elems(M, N, kSumCols), 256);
     // (the split, and with it the partials, may differ between the two forms of the low limb: room for either)
     size_t part = 0;
     for (int lo_signed = 0; lo_signed < 2; ++lo_signed) {
@@ -1216,42 +840,6 @@ static size_t wgrad_ws_bytes(const qbp_conv_desc *d, int64_t M, int64_t N, int64
         part = std::max(part, pl.P.direct ? (size_t)0 : align_up(sizeof(int64_t) * (size_t)pl.grid * (size_t)pl.P.part_stride, 256));
     }
     return 256 + sums + part;
-}
-
-template <bool IS_SIGNED>
-static int launch_class_sums(const void *q, int64_t pixels, int H, int W, int C, int64_t *sums, cudaStream_t st)
-{
-    QBP_CUDA_OK(cudaMemsetAsync(sums, 0, sizeof(int64_t) * 16 * C, st));
-    if ((size_t)C * 16 * sizeof(int) > 200 * 1024) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "wgrad: more than 3200 channels");
-    const size_t smem = (size_t)C * 16 * sizeof(int);
-    static PerDeviceOnce configured;
-    if (smem > 48 * 1024) QBP_SMEM_OPT_IN(configured, class_sums_kernel<IS_SIGNED>, 200 * 1024);
-    if (pixels >= (1ll << 30)) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "wgrad: more than 2^30 positions");
-    if (W <= 256) {
-        // a block step is one image row: W columns x gs channel groups of 16
-        const int cv = C / 16;
-        int gs = 1; while (gs * 2 <= cv && gs * 2 * W <= 256 && gs < 16) gs *= 2;
-        const int slabs = (cv + gs - 1) / gs;
-        const int64_t rows = pixels / W;
-        const int Nimg = (int)(rows / H);
-        // int32 registers: a thread sees at most rows / grid * 255 per channel
-        int64_t grid_x = std::min<int64_t>(rows, std::max<int64_t>(1, (int64_t)sm_count() * 3 / slabs));
-        grid_x = std::max<int64_t>(grid_x, rows / (1 << 22) + 1);
-        QBP_TRACE_BEGIN(st);
-        launch(row_class_sums_kernel<IS_SIGNED>, dim3((unsigned)grid_x, (unsigned)slabs), 256, (size_t)12 * gs * 16 * sizeof(int), st, (const uint8_t *)q, Nimg, H, W, C, gs, (unsigned long long *)sums);
-        QBP_LAUNCH_OK("class_sums_kernel");
-        return QBP_OK;
-    }
-    // int32 partials: a thread sees at most pixels / grid * 255 per channel.  Few blocks (each ends with up to
-    // 16*C atomics on the same 16*C sums), eight 16-byte loads in flight per thread.
-    const int cv = C / 16, tw = cv < 256 ? cv : 256, rpb = 256 / tw;
-    const int bps = std::max(1, std::min(2, (int)((200 * 1024) / std::max<size_t>(smem, 1024))));
-    int64_t grid = std::min<int64_t>((pixels + 8 * rpb - 1) / (8 * rpb), (int64_t)sm_count() * bps);
-    grid = std::max<int64_t>(grid, pixels / (1 << 22) + 1);
-    QBP_TRACE_BEGIN(st);
-    launch(class_sums_kernel<IS_SIGNED>, (unsigned)grid, 256, smem, st, (const uint8_t *)q, (int)pixels, H, W, C, (unsigned long long *)sums);
-    QBP_LAUNCH_OK("class_sums_kernel");
-    return QBP_OK;
 }
 
 }  // namespace qbp
@@ -1280,7 +868,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_wgrad_s16(const qbp_co
 int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qparams *qx,
                         const int8_t *g_hi, const uint8_t *g_lo, const qbp_qparams *qg16, int64_t *acc_out, float *dW,
                         int *ext_status, void *ws, size_t ws_bytes, cudaStream_t st, const int64_t *tot_x, const int64_t *tot_g16,
-                        bool tot_g_filled, bool lo_signed)
+                        bool tot_g_filled, bool lo_signed, const SumJob *done_sums)
 {
     if (!x || !g_hi || !g_lo || !qx || !qg16) return fail(QBP_ERR_INVALID_ARG, "wgrad_s16: NULL operand");
     if (!acc_out && !dW) return fail(QBP_ERR_INVALID_ARG, "wgrad_s16: acc_out and dW are both NULL");
@@ -1291,6 +879,7 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
             return fail(QBP_ERR_UNSUPPORTED_SHAPE,
                         "wgrad_s16: needs stride 1, R = S in {1,3}, pad = (R-1)/2, C and K multiples of 32");
         M = (int64_t)d->N * d->H * d->W; N = d->K; K = d->C;
+        if (M >= (1ll << 30)) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "wgrad: more than 2^30 positions");
     } else {
         if (M <= 0 || N <= 0 || K <= 0) return fail(QBP_ERR_INVALID_ARG, "wgrad_s16: M, N, K must be positive");
         if (N % 16 || K % 16) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "wgrad_s16: N and K must be multiples of 16");
@@ -1307,66 +896,41 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
     WsCarver w(ws, ws_bytes);
     int *status = w.take<int>(1);
     if (ext_status) status = ext_status;         // the caller's sticky word: raised here, never cleared
-    int64_t *sx = nullptr, *shi = nullptr, *slo = nullptr;       // convolution: per border class
-    SumJob jobs[3] = {{x, M, K, 1, 1, nullptr}, {g_hi, M, N, 1, 1, nullptr}, {g_lo, M, N, 1, lo_signed ? 1 : 0, nullptr}};
-    if (d) { sx = w.take<int64_t>(16 * K); shi = w.take<int64_t>(16 * N); slo = w.take<int64_t>(16 * N); }
-    else for (SumJob &j : jobs) j.out = w.take<int32_t>(sum_elems(j.rows, j.cols, true));
+    SumJob all[6], jobs[6];
+    int64_t *tab = d && !done_sums ? w.take<int64_t>(wgrad_sum_table(d)) : nullptr;
+    const int nall = wgrad_sum_jobs(d, M, N, K, x, g_hi, g_lo, lo_signed, tab, all);
+    for (int i = 0; i < nall; ++i) {
+        if (done_sums) all[i] = done_sums[i];
+        else if (!d) all[i].out = w.take<int32_t>(sum_elems(all[i]));
+    }
     int64_t *part = P.direct ? nullptr : w.take<int64_t>((size_t)pl.grid * (size_t)P.part_stride);
 
     // large plain products run on CTA pairs (256 x 256 tiles across two SMs, the whole reduction in one pair)
     const bool pair_kernel = !d && wgrad2_eligible(M, N, K);
-    // code sums for the zero-point terms: per border class (convolution) or plain column sums
+    // code sums for the zero-point terms: of everything, or (the kernels that wrote the codes left their per-channel totals,
+    // or the product takes the gradient's itself: a row of ones in its spare chunk) of the images' edges only
     int rc;
-    // (the border tables stay within int32 per block: a block sees at most Nimg * 2 (W + H) border positions)
-    const bool from_totals = d && tot_x && tot_g16 && d->H >= 3 && d->W >= 3 && std::max(K, N) <= 1536 &&
-                             (int64_t)d->N * 2 * (d->H + d->W) < (1ll << 22) && (tot_g_filled || wgrad_self_totals(d));
+    const bool from_totals = d && tot_x && tot_g16 && (tot_g_filled || wgrad_self_totals(d));
+    int njobs = 0;
+    if (!done_sums)
+        for (int i = from_totals ? 3 : 0; i < nall; ++i) jobs[njobs++] = all[i];
+    if (!d) { P.sx = sums_of(all[0]); P.shi = sums_of(all[1]); P.slo = sums_of(all[2]); }
+    else {
+        P.cx = (const long long *)all[0].out64; P.chi = (const long long *)all[1].out64; P.clo = (const long long *)all[2].out64;
+        if (nall == 6) { P.ex = (const long long *)all[3].out64; P.ehi = (const long long *)all[4].out64; P.elo = (const long long *)all[5].out64; }
+        if (tab) QBP_CUDA_OK(cudaMemsetAsync(tab, 0, sizeof(int64_t) * wgrad_sum_table(d), st));
+    }
+    ZeroJobs zero{};
+    if (!ext_status) { zero.p[0] = reinterpret_cast<uint32_t *>(status); zero.words[0] = 1; }
     if (from_totals) {
-        // the kernels that wrote the codes left their per-channel totals: only the border positions are read again
-        QBP_CUDA_OK(cudaMemsetAsync(sx, 0, (size_t)((char *)(slo + 16 * N) - (char *)sx), st));
-        if (wgrad_inline_border(d)) {
-            // the product kernel's epilogue warps take the border classes while its MMAs run
-            P.cls_x = (unsigned long long *)sx; P.cls_hi = (unsigned long long *)shi; P.cls_lo = (unsigned long long *)slo;
-            P.codes_x = (const uint8_t *)x; P.codes_hi = (const uint8_t *)g_hi; P.codes_lo = g_lo;
-        } else if (d->pad > 0) {         // (without padding every tap sees every position: the totals are all there is)
-            static PerDeviceOnce configured;
-            QBP_SMEM_OPT_IN(configured, border_class_sums_kernel, 96 * 1024);
-            const int gx = (int)std::min<int64_t>((d->N + 3) / 4, 128);      // one group of four images per block when possible
-            QBP_TRACE_BEGIN(st);
-            launch(border_class_sums_kernel, dim3((unsigned)gx, 1, 3), 256, (size_t)std::max(K, N) * 16 * sizeof(int), st, (const uint8_t *)x, (const uint8_t *)g_hi, g_lo, d->N, d->H, d->W, (int)K, (int)N, (unsigned long long *)sx,
-                (unsigned long long *)shi, (unsigned long long *)slo, lo_signed ? 1 : 0);
-            QBP_LAUNCH_OK("border_class_sums_kernel");
-        }
         P.tot_x = (const long long *)tot_x; P.tot_g = (const long long *)tot_g16;
         P.tot_g_plain = tot_g_filled ? 1 : 0;
         if (!tot_g_filled) {
-            // nobody left the gradient's totals: the product takes them itself (a row of ones in its spare chunk)
-            QBP_CUDA_OK(cudaMemsetAsync(const_cast<int64_t *>(tot_g16), 0, sizeof(int64_t) * (size_t)N, st));
             P.ones_tot = (unsigned long long *)const_cast<int64_t *>(tot_g16);
+            if (!done_sums) { zero.p[1] = reinterpret_cast<uint32_t *>(P.ones_tot); zero.words[1] = 2 * N; }
         }
-    } else if (d && K == N && d->W <= 256 && M < (1ll << 30) && shi == sx + 16 * K && slo == shi + 16 * N) {
-        // as many input as output channels: the three tensors in one launch
-        QBP_CUDA_OK(cudaMemsetAsync(sx, 0, sizeof(int64_t) * 48 * K, st));
-        const int cv = (int)K / 16;
-        int gs = 1; while (gs * 2 <= cv && gs * 2 * d->W <= 256 && gs < 16) gs *= 2;
-        const int slabs = (cv + gs - 1) / gs;
-        const int64_t rows = M / d->W;
-        // one wave of three blocks per SM over the three tensors
-        int64_t grid_x = std::min<int64_t>(rows, std::max<int64_t>(1, (int64_t)sm_count() / slabs));
-        grid_x = std::max<int64_t>(grid_x, rows / (1 << 22) + 1);
-        QBP_TRACE_BEGIN(st);
-        launch(row_class_sums3_kernel, dim3((unsigned)grid_x, (unsigned)slabs, 3), 256, (size_t)12 * gs * 16 * sizeof(int), st, (const uint8_t *)x, (const uint8_t *)g_hi, (const uint8_t *)g_lo, (int)(rows / d->H), d->H, d->W, (int)K, gs,
-            (unsigned long long *)sx, lo_signed ? 1 : 0);
-        QBP_LAUNCH_OK("class_sums_kernel");
-    } else if (d) {
-        if ((rc = launch_class_sums<true>(x, M, d->H, d->W, (int)K, sx, st))) return rc;
-        if ((rc = launch_class_sums<true>(g_hi, M, d->H, d->W, (int)N, shi, st))) return rc;
-        if ((rc = lo_signed ? launch_class_sums<true>(g_lo, M, d->H, d->W, (int)N, slo, st)
-                            : launch_class_sums<false>(g_lo, M, d->H, d->W, (int)N, slo, st))) return rc;
-    } else {
-        if ((rc = launch_code_sums(jobs, 3, st))) return rc;
-        P.sx = sums_of(jobs[0]); P.shi = sums_of(jobs[1]); P.slo = sums_of(jobs[2]);
     }
-    if (!ext_status) QBP_CUDA_OK(cudaMemsetAsync(status, 0, sizeof(int), st));
+    if ((rc = launch_code_sums(jobs, njobs, st, zero))) return rc;
     if (pair_kernel)
         return launch_wgrad2(M, N, K, x, qx, g_hi, g_lo, qg16, acc_out, dW, P.sx, P.shi, P.slo, status, st, lo_signed);
 
@@ -1408,9 +972,9 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
         const int nb = per_n * (d->K / 8) >= 4ll * sm_count() ? 8 : per_n * (d->K / 4) >= 4ll * sm_count() ? 4 : 2;
         const dim3 grid((unsigned)per_n, (unsigned)((d->K + nb - 1) / nb));
         QBP_TRACE_BEGIN(st);
-        if (nb == 8)      launch(wgrad_conv_finalize_kernel<8>, grid, 256, 0, st, P, (const long long *)sx, (const long long *)shi, (const long long *)slo);
-        else if (nb == 4) launch(wgrad_conv_finalize_kernel<4>, grid, 256, 0, st, P, (const long long *)sx, (const long long *)shi, (const long long *)slo);
-        else              launch(wgrad_conv_finalize_kernel<2>, grid, 256, 0, st, P, (const long long *)sx, (const long long *)shi, (const long long *)slo);
+        if (nb == 8)      launch(wgrad_conv_finalize_kernel<8>, grid, 256, 0, st, P);
+        else if (nb == 4) launch(wgrad_conv_finalize_kernel<4>, grid, 256, 0, st, P);
+        else              launch(wgrad_conv_finalize_kernel<2>, grid, 256, 0, st, P);
         QBP_LAUNCH_OK("wgrad_finalize_kernel");
     } else if (!P.direct) {
         const int blocks = (int)((outs * kWgFinalizeLanes + 255) / 256);

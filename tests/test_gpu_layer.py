@@ -476,3 +476,12 @@ def test_backward_with_mixed_gamma_and_beta(B, kind):
     ohi, olo = O.limb_split(g16.q)
     assert np.array_equal(to_host(L.g8), g8.q) and np.array_equal(to_host(L.ghi), ohi)
     assert np.array_equal(to_host(L.glo) ^ np.uint8(0x80), olo)
+
+
+@pytest.mark.parametrize("batch,cin,cout", [(16, 16, 16), (48, 4096, 16), (16, 32, 4080), (2064, 144, 272)])
+def test_linear_layers_of_other_shapes_stagewise(B, batch, cin, cout):
+    """Activation and weights quantised in one launch, each tensor with its share of the blocks (much larger activation, much
+    larger weights), the code sums of both products taken beside other kernels: every stage against the oracle."""
+    cfg = dict(x=synth.normal((batch, cin), 95), w=synth.kaiming_uniform_linear(cin, cout, 96), dy=synth.normal((batch, cout), 97, std=0.1),
+               seed=3, id8=5, id16=5)
+    _check_layer(B, cfg, True)

@@ -454,3 +454,17 @@ def test_wgrad_code_sums_in_pieces_of_the_rows(B, M, N, K):
     oacc, oout = O.gemm_s16s8(X, -101, G, 12345, 0.5, 0.25)
     assert B.status_word(ws) == 0
     assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
+
+
+@pytest.mark.parametrize("N,H,W,C,K", [(600, 1, 3, 32, 64), (5, 7, 1, 160, 32), (150, 2, 4, 64, 288), (700, 3, 3, 32, 32)])
+def test_wgrad_conv_edge_sums(B, N, H, W, C, K):
+    """The zero-point terms of a 3x3 weight gradient from the operands' sums over all positions less those over the images'
+    edges: images of one row or column (both edges at once), edges in one and several pieces, strips of 32, 64 and 128
+    channels, partly filled ones."""
+    d = B.conv_desc(N, H, W, C, K, 3, 3, 1, 1); od = O.conv_desc(N, H, W, C, K, 3, 3, 1, 1)
+    X = random_codes((N, H, W, C), 71); G = np.random.Generator(np.random.PCG64(72)).integers(-32768, 32768, (N, H, W, K)).astype(np.int16)
+    hi, lo = O.limb_split(G)
+    acc, dW, ws = B.qbp_wgrad_s16(to_dev(X), _qp(B, 0.5, -90), to_dev(hi), to_dev(lo), _qp(B, 0.25, 2077), d=d, want_acc=True)
+    oacc, oout = O.conv_wgrad_s16(od, X, -90, G, 2077, 0.5, 0.25)
+    assert B.status_word(ws) == 0
+    assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
