@@ -10,6 +10,7 @@ message.
 from __future__ import annotations
 
 import ctypes as C
+import threading
 from pathlib import Path
 
 import torch
@@ -107,14 +108,21 @@ def _check(status: int) -> None:
 
 def _ptr(t) -> C.c_void_p:
     if t is None:
-        return C.c_void_p(0)
+        return _NULL
     if isinstance(t, int):
         return C.c_void_p(t)
     assert t.is_cuda and t.is_contiguous(), "device tensors must be contiguous CUDA tensors"
     return C.c_void_p(t.data_ptr())
 
 
+_NULL = C.c_void_p(0)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream() -> C.c_void_p:
+    # (the raw handle of torch's current stream: building a Stream object for it costs several times as much)
+    if _raw_stream is not None:
+        return C.c_void_p(_raw_stream(torch.cuda.current_device()))
     return C.c_void_p(torch.cuda.current_stream().cuda_stream)
 
 
@@ -124,12 +132,12 @@ _ws_cache: dict = {}
 def workspace(nbytes: int, device=None) -> torch.Tensor:
     """A cached device scratch buffer of at least nbytes (grown on demand, 256-byte aligned by torch); one per
     device and host thread, since calls of different threads may interleave on a stream."""
-    import threading
-    dev = torch.device("cuda", torch.cuda.current_device()) if device is None else torch.device(device)
-    key = (dev, threading.get_ident())
+    dev = None if device is None else torch.device(device)
+    index = torch.cuda.current_device() if dev is None or dev.index is None else dev.index
+    key = (index, threading.get_ident())
     t = _ws_cache.get(key)
     if t is None or t.numel() < nbytes:
-        t = torch.empty(max(nbytes, 1 << 20), dtype=torch.uint8, device=dev)
+        t = torch.empty(max(nbytes, 1 << 20), dtype=torch.uint8, device=torch.device("cuda", index))
         _ws_cache[key] = t
     return t
 
@@ -137,6 +145,11 @@ def workspace(nbytes: int, device=None) -> torch.Tensor:
 def new_qparams(count: int = 1, device="cuda") -> torch.Tensor:
     """Device storage for `count` qbp_qparams records: int32 [count, 4] = (scale bits, zero_point, vmin bits, vmax bits)."""
     return torch.zeros((count, 4), dtype=torch.int32, device=device)
+
+
+def _out_qparams(count, device):
+    """The same for a call that writes every record itself: not cleared (a launch less)."""
+    return torch.empty((count, 4), dtype=torch.int32, device=device)
 
 
 def read_qparams(qp: torch.Tensor):
@@ -175,7 +188,7 @@ def qbp_quantize_s8(x, granularity=QBP_PER_TENSOR, rounding=QBP_ROUND_NEAREST, s
                     range_in=None, q=None, qp_out=None, row_sums=None, col_sums=None, ws=None):
     cols = x.shape[-1]; rows = x.numel() // cols if cols else 0
     if q is None: q = torch.empty(x.shape, dtype=torch.int8, device=x.device)
-    if qp_out is None: qp_out = new_qparams(cols if granularity else 1, x.device)
+    if qp_out is None: qp_out = _out_qparams(cols if granularity else 1, x.device)
     if ws is None: ws = workspace(lib.qbp_quantize_workspace_bytes(rows, cols, granularity), x.device)
     _check(lib.qbp_quantize_s8(_ptr(x), C.c_int64(rows), C.c_int64(cols), granularity, rounding,
                                C.c_uint64(seed), C.c_uint32(tensor_id), _ptr(range_in), _ptr(q), _ptr(qp_out),
@@ -187,7 +200,7 @@ def qbp_range_chunked(x, chunks, range_out=None, ws=None):
     """Appendix B's clamping values for activations (averages of the chunks' minima / maxima over `chunks` equal
     groups of rows) as a qparams record to pass to qbp_quantize_s8(range_in=...)."""
     cols = x.shape[-1]; rows = x.numel() // cols if cols else 0
-    if range_out is None: range_out = new_qparams(1, x.device)
+    if range_out is None: range_out = _out_qparams(1, x.device)
     if ws is None: ws = workspace(lib.qbp_range_chunked_workspace_bytes(), x.device)
     _check(lib.qbp_range_chunked(_ptr(x), C.c_int64(rows), C.c_int64(cols), C.c_int64(chunks), _ptr(range_out), _ptr(ws),
                                  C.c_size_t(ws.numel()), _stream()))
@@ -214,7 +227,7 @@ def qbp_quantize_s16(x, granularity=QBP_PER_TENSOR, rounding=QBP_ROUND_NEAREST, 
     if q is None and "q" in want: q = torch.empty(x.shape, dtype=torch.int16, device=x.device)
     if hi is None and "hi" in want: hi = torch.empty(x.shape, dtype=torch.int8, device=x.device)
     if lo is None and "lo" in want: lo = torch.empty(x.shape, dtype=torch.uint8, device=x.device)
-    if qp_out is None: qp_out = new_qparams(cols if granularity else 1, x.device)
+    if qp_out is None: qp_out = _out_qparams(cols if granularity else 1, x.device)
     if ws is None: ws = workspace(lib.qbp_quantize_workspace_bytes(rows, cols, granularity), x.device)
     _check(lib.qbp_quantize_s16(_ptr(x), C.c_int64(rows), C.c_int64(cols), granularity, rounding,
                                 C.c_uint64(seed), C.c_uint32(tensor_id), _ptr(range_in), _ptr(q), _ptr(hi), _ptr(lo),
@@ -228,8 +241,8 @@ def qbp_bifurcate(g, seed, tensor_id8, tensor_id16, q8=None, hi=None, lo=None, q
     if q8 is None: q8 = torch.empty(g.shape, dtype=torch.int8, device=g.device)
     if hi is None: hi = torch.empty(g.shape, dtype=torch.int8, device=g.device)
     if lo is None: lo = torch.empty(g.shape, dtype=torch.uint8, device=g.device)
-    if qp8 is None: qp8 = new_qparams(1, g.device)
-    if qp16 is None: qp16 = new_qparams(1, g.device)
+    if qp8 is None: qp8 = _out_qparams(1, g.device)
+    if qp16 is None: qp16 = _out_qparams(1, g.device)
     if ws is None: ws = workspace(lib.qbp_quantize_workspace_bytes(rows, cols, 0), g.device)
     _check(lib.qbp_bifurcate(_ptr(g), C.c_int64(rows), C.c_int64(cols), C.c_uint64(seed), C.c_uint32(tensor_id8),
                              C.c_uint32(tensor_id16), _ptr(q8), _ptr(qp8), _ptr(row_sums8), _ptr(hi), _ptr(lo),
@@ -245,8 +258,8 @@ def qbp_bifurcate_shard(g, seed, tensor_id8, tensor_id16, index_base, range_in, 
     if q8 is None: q8 = torch.empty(g.shape, dtype=torch.int8, device=g.device)
     if hi is None: hi = torch.empty(g.shape, dtype=torch.int8, device=g.device)
     if lo is None: lo = torch.empty(g.shape, dtype=torch.uint8, device=g.device)
-    if qp8 is None: qp8 = new_qparams(1, g.device)
-    if qp16 is None: qp16 = new_qparams(1, g.device)
+    if qp8 is None: qp8 = _out_qparams(1, g.device)
+    if qp16 is None: qp16 = _out_qparams(1, g.device)
     _check(lib.qbp_bifurcate_shard(_ptr(g), C.c_int64(rows), C.c_int64(cols), C.c_uint64(seed), C.c_uint32(tensor_id8),
                                    C.c_uint32(tensor_id16), C.c_uint64(index_base), _ptr(range_in), _ptr(q8), _ptr(qp8),
                                    _ptr(row_sums8), _ptr(hi), _ptr(lo), _ptr(qp16), _stream()))
@@ -344,14 +357,14 @@ def qbp_wgrad_s16(x, qx, g_hi, g_lo, qg16, d: ConvDesc | None = None, want_acc=F
 # ------------------------------------------------- Appendix C: 1-bit operands, ternary gradients
 def qbp_binarize_s8(x, q=None, qp_out=None):
     if q is None: q = torch.empty(x.shape, dtype=torch.int8, device=x.device)
-    if qp_out is None: qp_out = new_qparams(1, x.device)
+    if qp_out is None: qp_out = _out_qparams(1, x.device)
     _check(lib.qbp_binarize_s8(_ptr(x), C.c_int64(x.numel()), _ptr(q), _ptr(qp_out), _stream()))
     return q, qp_out
 
 
 def qbp_stc_ternarize_s8(g, samples=1, seed=0, tensor_id=0, q=None, qp_out=None, ws=None):
     if q is None: q = torch.empty(g.shape, dtype=torch.int8, device=g.device)
-    if qp_out is None: qp_out = new_qparams(1, g.device)
+    if qp_out is None: qp_out = _out_qparams(1, g.device)
     if ws is None: ws = workspace(lib.qbp_stc_ternarize_workspace_bytes(), g.device)
     _check(lib.qbp_stc_ternarize_s8(_ptr(g), C.c_int64(g.numel()), int(samples), C.c_uint64(seed), C.c_uint32(tensor_id),
                                     _ptr(q), _ptr(qp_out), _ptr(ws), C.c_size_t(ws.numel()), _stream()))
@@ -366,7 +379,7 @@ def qbp_tbp_weight_gradient(a_codes, qa, g, samples, seed=0, tensor_id=0, d: Con
         rows = d.N * d.H * d.W; K = d.C; N = d.K; shape = (d.K, d.R, d.S, d.C); dref = C.byref(d)
     dev = g.device
     t_hi = torch.empty(g.shape, dtype=torch.int8, device=dev); t_lo = torch.empty(g.shape, dtype=torch.uint8, device=dev)
-    qp_t = new_qparams(1, dev)
+    qp_t = _out_qparams(1, dev)
     acc = torch.empty(shape, dtype=torch.int64, device=dev) if want_acc else None
     gW = torch.empty(shape, dtype=torch.float32, device=dev)
     if ws is None: ws = workspace(lib.qbp_tbp_weight_gradient_workspace_bytes(dref, rows, N, K), dev)
@@ -404,7 +417,7 @@ def qbp_rangebn_fwd(x, gamma=None, beta=None, relu=False, y=None, want_range=Fal
     if y is None: y = torch.empty_like(x)
     mean = torch.empty(Cc, dtype=torch.float32, device=x.device)
     vmin = torch.empty_like(mean); vmax = torch.empty_like(mean)
-    out_range = new_qparams(1, x.device) if want_range else None
+    out_range = _out_qparams(1, x.device) if want_range else None
     if ws is None: ws = workspace(lib.qbp_rangebn_workspace_bytes(n, Cc), x.device)
     _check(lib.qbp_rangebn_fwd(_ptr(x), C.c_int64(n), C.c_int64(Cc), _ptr(gamma), _ptr(beta), int(relu), _ptr(y),
                                _ptr(mean), _ptr(vmin), _ptr(vmax), _ptr(out_range), _ptr(ws), C.c_size_t(ws.numel()),
@@ -419,7 +432,7 @@ def qbp_rangebn_fwd_q8(x, gamma=None, beta=None, relu=False, y=None, want_y=True
     Cc = x.shape[-1]; n = x.numel() // Cc
     if y is None and want_y: y = torch.empty_like(x)
     if q is None: q = torch.empty(x.shape, dtype=torch.int8, device=x.device)
-    if qp is None: qp = new_qparams(1, x.device)
+    if qp is None: qp = _out_qparams(1, x.device)
     if row_sums is None and want_row_sums: row_sums = torch.empty(n, dtype=torch.int32, device=x.device)
     mean = torch.empty(Cc, dtype=torch.float32, device=x.device)
     vmin = torch.empty_like(mean); vmax = torch.empty_like(mean)
@@ -450,7 +463,7 @@ def qbp_rangebn_fwd_apply(x, n_stat, col_sum, col_min, col_max, gamma=None, beta
     if y is None and want_y: y = torch.empty_like(x)
     mean = torch.empty(Cc, dtype=torch.float32, device=x.device)
     vmin = torch.empty_like(mean); vmax = torch.empty_like(mean)
-    out_range = new_qparams(1, x.device) if want_range else None
+    out_range = _out_qparams(1, x.device) if want_range else None
     _check(lib.qbp_rangebn_fwd_apply(_ptr(x), C.c_int64(n), C.c_int64(n_stat), C.c_int64(Cc), _ptr(col_sum), _ptr(col_min),
                                      _ptr(col_max), _ptr(gamma), _ptr(beta), int(relu), _ptr(y), _ptr(mean), _ptr(vmin),
                                      _ptr(vmax), _ptr(out_range), C.byref(rq) if rq is not None else None, _stream()))

@@ -34,15 +34,21 @@ struct ScanGeom {
 
 inline int pow2ceil(int v) { int p = 1; while (p < v) p <<= 1; return p; }
 
-// Resident blocks per SM of a kernel at `threads` threads and no dynamic shared memory.
-template <typename Kernel>
-inline int blocks_per_sm(Kernel kernel, int threads)
+// Resident blocks per SM of a kernel at `threads` threads (always the same for one kernel) and no dynamic shared memory; asked
+// once per kernel and device (the query costs the host most of a microsecond).
+template <auto Kernel>
+inline int blocks_per_sm(int threads)
 {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, 0) != cudaSuccess || n < 1) {
+    static int cache[kMaxDevices] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); dev = -1; }
+    int n = dev < 0 ? 0 : __atomic_load_n(&cache[dev], __ATOMIC_RELAXED);
+    if (n > 0) return n;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, Kernel, threads, 0) != cudaSuccess || n < 1) {
         cudaGetLastError();
-        n = 1;
+        return 1;
     }
+    if (dev >= 0) __atomic_store_n(&cache[dev], n, __ATOMIC_RELAXED);
     return n;
 }
 

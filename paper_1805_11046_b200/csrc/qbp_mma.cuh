@@ -21,7 +21,7 @@ struct CodeSums {
     __device__ __forceinline__ long long at(int64_t i) const
     {
         long long s = 0;
-#pragma unroll 4
+#pragma unroll 8
         for (int k = 0; k < pieces; ++k) s += __ldg(p + (int64_t)k * stride + i);
         return s;
     }

@@ -542,12 +542,12 @@ __global__ void __launch_bounds__(kSumThreads) code_sums_kernel(const __grid_con
 }
 
 // ----------------------------------------------------------------- launchers
-// Pieces of the rows in a column sum: enough blocks for two per SM, at least 128 rows each (four per thread row), at most 32
-// pieces (the reader adds them up) -- but at most 2^22 rows each, so that a piece fits int32 (255 * 2^22 < 2^31).
+// Pieces of the rows in a column sum: enough blocks for four per SM, at least 128 rows each, at most 16 pieces (the reader adds
+// them up) -- but at most 2^22 rows each, so that a piece fits int32 (255 * 2^22 < 2^31).
 int sum_pieces(int64_t rows, int64_t cols)
 {
     const int64_t strips = (cols + 127) / 128;
-    int64_t p = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(2ll * sm_count() / strips, 32), rows / 128));
+    int64_t p = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(4ll * sm_count() / strips, 16), rows / 128));
     return (int)std::max<int64_t>(p, (rows >> 22) + 1);
 }
 
@@ -560,9 +560,13 @@ int edge_pieces(int64_t rows, int H, int W)
 
 int fill_sum_jobs(const SumJob *jobs, int count, SumJobs &J, int *blocks)
 {
-    int first = 0;
+    // (sums over rows first: their blocks run longest; those along rows fill the machine behind them)
+    int first = 0, order[kMaxSumJobs], n = 0;
+    for (int pass = 0; pass < 2; ++pass)
+        for (int i = 0; i < count; ++i)
+            if ((jobs[i].kind == kSumRows) == (pass == 1)) order[n++] = i;
     for (int i = 0; i < count; ++i) {
-        const SumJob &s = jobs[i];
+        const SumJob &s = jobs[order[i]];
         if (s.cols % 16 || !aligned16(s.q)) return fail(QBP_ERR_INVALID_ARG, "code sums need 16-byte aligned rows (cols %% 16 == 0)");
         SumJobDev &j = J.j[i];
         j.q = static_cast<const uint8_t *>(s.q); j.rows = s.rows; j.cols = (int)s.cols; j.kind = s.kind; j.out = s.out; j.out64 = s.out64;
@@ -614,7 +618,7 @@ static int scan_blocks(int64_t n, bool vec)
 {
     if (n <= 0) return 0;
     const int64_t per_block = (int64_t)kThreads * kRangeUnroll * (vec ? 4 : 1);
-    const int g = grid_for(vec ? blocks_per_sm(range_partial_kernel<4>, kThreads) : blocks_per_sm(range_partial_kernel<1>, kThreads), (n + per_block - 1) / per_block);
+    const int g = grid_for(vec ? blocks_per_sm<range_partial_kernel<4>>(kThreads) : blocks_per_sm<range_partial_kernel<1>>(kThreads), (n + per_block - 1) / per_block);
     return std::min(g, kMaxParts);
 }
 
@@ -652,8 +656,8 @@ static int launch_chan_range(const float *x, int64_t rows, int64_t cols, int bit
                              qbp_qparams *qp, cudaStream_t st)
 {
     const bool v4 = aligned16(x) && cols % 4 == 0;
-    ScanGeom g = scan_geom(rows, cols, aligned16(x), v4 ? blocks_per_sm(chan_range_partial_kernel<4>, kScanThreads)
-                                                        : blocks_per_sm(chan_range_partial_kernel<1>, kScanThreads));
+    ScanGeom g = scan_geom(rows, cols, aligned16(x), v4 ? blocks_per_sm<chan_range_partial_kernel<4>>(kScanThreads)
+                                                        : blocks_per_sm<chan_range_partial_kernel<1>>(kScanThreads));
     int nparts = 0;
     if (rows > 0) {
         nparts = g.nbx;
@@ -697,7 +701,7 @@ static int launch_quantize(const float *x, int64_t n, int64_t cols, int perch, i
     const QuantJob J{x, n, (int)cols, r, id8, id16, o, smem_cols, index_base};
 #define QBP_QUANT2(SR_, VEC_, PC_, TOT_)                                                                                \
     do {                                                                                                                \
-        const int grid = grid_for(blocks_per_sm(quantize_kernel<SR_, VEC_, PC_, TOT_>, kThreads), groups);              \
+        const int grid = grid_for(blocks_per_sm<quantize_kernel<SR_, VEC_, PC_, TOT_>>(kThreads), groups);              \
         QBP_TRACE_BEGIN(st);                                                                                            \
         launch(quantize_kernel<SR_, VEC_, PC_, TOT_>, grid, kThreads, smem, st, J, key);                                \
     } while (0)
@@ -888,7 +892,7 @@ int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, s
         const int64_t nx = x->rows * x->cols, nw = w->rows * w->cols;
         ScanJob a{x->v, nx, parts[0], scan_blocks(nx, true), 1}, b{w->v, nw, parts[1], scan_blocks(nw, true), 0};
         // one wave in all: each tensor its share
-        const int wave = std::min(kMaxParts, sm_count() * blocks_per_sm(range_partial_kernel<4>, kThreads));
+        const int wave = std::min(kMaxParts, sm_count() * blocks_per_sm<range_partial_kernel<4>>(kThreads));
         if (a.blocks + b.blocks > wave) {
             b.blocks = std::max(1, std::min(b.blocks, (int)(wave * nw / (nx + nw))));
             a.blocks = std::min(a.blocks, wave - b.blocks);
@@ -900,7 +904,7 @@ int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, s
         const QuantJob jb{w->v, nw, (int)w->cols, RangeSrc{parts[1], b.blocks, nullptr, w->qp, nullptr}, 0, 0, o[1], 0, 0};
         const int64_t per_block = (int64_t)kThreads * 4 * kUnroll;
         const bool totals = o[0].chansum8 != nullptr;
-        const int qwave = sm_count() * (totals ? blocks_per_sm(quantize_pair_kernel<true>, kThreads) : blocks_per_sm(quantize_pair_kernel<false>, kThreads));
+        const int qwave = sm_count() * (totals ? blocks_per_sm<quantize_pair_kernel<true>>(kThreads) : blocks_per_sm<quantize_pair_kernel<false>>(kThreads));
         int64_t ga = (nx + per_block - 1) / per_block, gb = (nw + per_block - 1) / per_block;
         if (ga + gb > qwave) { gb = std::max<int64_t>(1, std::min(gb, qwave * nw / (nx + nw))); ga = std::min(ga, qwave - gb); }
         QBP_TRACE_BEGIN(st);
@@ -973,7 +977,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_range_chunked(const fl
     const bool vec = aligned16(x) && n_chunk % 4 == 0;
     // about one wave of blocks in all, at least one per chunk
     const int64_t per_block = (int64_t)kThreads * kRangeUnroll * (vec ? 4 : 1);
-    const int wave = grid_for(vec ? blocks_per_sm(chunk_range_partial_kernel<4>, kThreads) : blocks_per_sm(chunk_range_partial_kernel<1>, kThreads),
+    const int wave = grid_for(vec ? blocks_per_sm<chunk_range_partial_kernel<4>>(kThreads) : blocks_per_sm<chunk_range_partial_kernel<1>>(kThreads),
                               (rows * cols + per_block - 1) / per_block);
     int bpc = (int)std::max<int64_t>(1, std::min<int64_t>((n_chunk + per_block - 1) / per_block, wave / chunks));
     bpc = (int)std::min<int64_t>(bpc, kMaxParts / chunks);

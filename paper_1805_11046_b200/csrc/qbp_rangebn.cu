@@ -767,11 +767,11 @@ static int bn_fwd_apply_launch(const float *x, int64_t n_rows, int64_t n_stat, i
     if (!y && !requant) return fail(QBP_ERR_INVALID_ARG, "rangebn_fwd: neither y nor 8-bit codes wanted");
     const bool al = aligned16(x) && (!y || aligned16(y)) && (!requant || ((uintptr_t)rq->q & 3) == 0);
     const bool v4 = al && C % 4 == 0;
-    const int bps = v4 ? (requant ? (relu ? blocks_per_sm(bn_apply_kernel<4, true, true>, kScanThreads)
-                                          : blocks_per_sm(bn_apply_kernel<4, false, true>, kScanThreads))
-                                  : (relu ? blocks_per_sm(bn_apply_kernel<4, true, false>, kScanThreads)
-                                          : blocks_per_sm(bn_apply_kernel<4, false, false>, kScanThreads)))
-                       : blocks_per_sm(bn_apply_kernel<1, true, true>, kScanThreads);
+    const int bps = v4 ? (requant ? (relu ? blocks_per_sm<bn_apply_kernel<4, true, true>>(kScanThreads)
+                                          : blocks_per_sm<bn_apply_kernel<4, false, true>>(kScanThreads))
+                                  : (relu ? blocks_per_sm<bn_apply_kernel<4, true, false>>(kScanThreads)
+                                          : blocks_per_sm<bn_apply_kernel<4, false, false>>(kScanThreads)))
+                       : blocks_per_sm<bn_apply_kernel<1, true, true>>(kScanThreads);
     const ScanGeom ga = scan_geom(n_rows, C, al, bps);
     const dim3 grid_apply(ga.nbx, ga.slabs);
     const float Cn = (float)(1.0 / std::sqrt(2.0 * std::log((double)n_stat)));
@@ -821,8 +821,8 @@ static int bn_fwd_stats_launch(const float *x, int64_t n, int64_t C, float *mean
     float *phi = w.take<float>((size_t)kScanMaxStrips * C);
     const bool al = aligned16(x);
     const bool v4 = al && C % 4 == 0;
-    const ScanGeom g = scan_geom(n, C, al, v4 ? blocks_per_sm(bn_stats_kernel<4>, kScanThreads)
-                                              : blocks_per_sm(bn_stats_kernel<1>, kScanThreads));
+    const ScanGeom g = scan_geom(n, C, al, v4 ? blocks_per_sm<bn_stats_kernel<4>>(kScanThreads)
+                                              : blocks_per_sm<bn_stats_kernel<1>>(kScanThreads));
     const dim3 grid(g.nbx, g.slabs);
     QBP_TRACE_BEGIN(st);
     if (g.vec == 4) launch(bn_stats_kernel<4>, grid, kScanThreads, 0, st, x, n, (int)C, g.tw, plo, phi, psum);
@@ -940,10 +940,10 @@ static int bn_bwd_stats_launch(const float *dy, const float *x, int64_t n_rows, 
 {
     const bool al = aligned16(x) && aligned16(dy);
     const bool v4 = al && C % 4 == 0;
-    const ScanGeom g = scan_geom(n_rows, C, al, v4 ? (ext ? blocks_per_sm(bn_bwd_stats_kernel<4, true, true>, kScanThreads)
-                                                          : relu ? blocks_per_sm(bn_bwd_stats_kernel<4, true, false>, kScanThreads)
-                                                                 : blocks_per_sm(bn_bwd_stats_kernel<4, false, false>, kScanThreads))
-                                                   : blocks_per_sm(bn_bwd_stats_kernel<1, true, false>, kScanThreads));
+    const ScanGeom g = scan_geom(n_rows, C, al, v4 ? (ext ? blocks_per_sm<bn_bwd_stats_kernel<4, true, true>>(kScanThreads)
+                                                          : relu ? blocks_per_sm<bn_bwd_stats_kernel<4, true, false>>(kScanThreads)
+                                                                 : blocks_per_sm<bn_bwd_stats_kernel<4, false, false>>(kScanThreads))
+                                                   : blocks_per_sm<bn_bwd_stats_kernel<1, true, false>>(kScanThreads));
     const dim3 grid(g.nbx, g.slabs);
     const double Cnd = 1.0 / std::sqrt(2.0 * std::log((double)n_stat));
     const float Cn = (float)Cnd;
@@ -973,9 +973,9 @@ static int bn_bwd_apply_launch(const float *dy, const float *x, int64_t n_rows, 
 {
     const bool al = aligned16(x) && aligned16(dy) && aligned16(dx);
     const bool v4 = al && C % 4 == 0;
-    const ScanGeom ga = scan_geom(n_rows, C, al, v4 ? (relu ? blocks_per_sm(bn_bwd_apply_kernel<4, true, true>, kScanThreads)
-                                                            : blocks_per_sm(bn_bwd_apply_kernel<4, false, true>, kScanThreads))
-                                                    : blocks_per_sm(bn_bwd_apply_kernel<1, true, true>, kScanThreads));
+    const ScanGeom ga = scan_geom(n_rows, C, al, v4 ? (relu ? blocks_per_sm<bn_bwd_apply_kernel<4, true, true>>(kScanThreads)
+                                                            : blocks_per_sm<bn_bwd_apply_kernel<4, false, true>>(kScanThreads))
+                                                    : blocks_per_sm<bn_bwd_apply_kernel<1, true, true>>(kScanThreads));
     const dim3 grid_apply(ga.nbx, ga.slabs);
     const float Cn = (float)(1.0 / std::sqrt(2.0 * std::log((double)n_stat)));
     QBP_TRACE_BEGIN(st);
@@ -1026,7 +1026,7 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
     float2 *chan_range = w.take<float2>((size_t)C);
     float2 *relu_thr = w.take<float2>((size_t)C);
     // (three resident blocks per SM by the kernel's launch bounds, whatever the instance)
-    const ScanGeom ga = scan_geom(n, C, true, blocks_per_sm(bn_bwd_apply_bifurcate_kernel<true, true, true>, kScanThreads));
+    const ScanGeom ga = scan_geom(n, C, true, blocks_per_sm<bn_bwd_apply_bifurcate_kernel<true, true, true>>(kScanThreads));
     // each row's code sum by shuffles over the row's lanes of a warp; a row that spans several warps or blocks is
     // added up from its pieces (integer atomics on the zeroed sums: the result does not depend on the order)
     ZeroJobs zero{};

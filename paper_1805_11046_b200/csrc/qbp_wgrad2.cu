@@ -222,13 +222,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
             const bool slab_in = (int64_t)o.k0 + 128 * (int)rank + quad * 32 < P.K;
             const long long rterm = valid ? -zg * P.sx.at(k) + P.M * zx * zg : 0;
             const int64_t ncol = P.N - o.n0;
-            // lane l takes the column terms of column l of this warp's four chunks, while the MMAs run
-            long long ct[4];
+            // lane l takes the column terms of column l of this warp's four chunks, while the MMAs run (the sums come in pieces:
+            // two pieces of all eight sums are in flight at a time -- one sum after the other took up to 64 us a tile)
+            long long ct[4] = {0, 0, 0, 0};
+            const int32_t *ph = P.shi.p + o.n0 + half * 128 + lane, *pl = P.slo.p + o.n0 + half * 128 + lane;
+#pragma unroll 2
+            for (int k = 0; k < P.shi.pieces; ++k) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int n = (half * 4 + i) * 32 + lane;
-                ct[i] = n < ncol ? -zx * (256 * P.shi.at(o.n0 + n) + P.slo.at(o.n0 + n)) : 0;
+                for (int i = 0; i < 4; ++i)
+                    if ((half * 4 + i) * 32 + lane < ncol) ct[i] += 256 * (long long)__ldg(ph + 32 * i) + __ldg(pl + 32 * i);
+                ph += P.shi.stride; pl += P.slo.stride;
             }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) ct[i] *= -zx;
             const int nchunks = (int)((ncol < 256 ? ncol : 256) + 31) / 32;
             if (!timed_out && !mbar_wait_warp(&acc_full, fph)) timed_out = true;
             fph ^= 1u;
