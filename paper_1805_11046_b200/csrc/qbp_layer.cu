@@ -275,8 +275,9 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_bwd(const qbp_la
     int nearly = 0, nlate = 0;
     const SumJob w_job = weight_sum_job(L, s, true, saved->w_codes, l.w_sums);
     early[nearly++] = w_job;
+    const bool x_early = !s.conv || !rangebn_bwd_one_launch(s.rows, s.cout);      // (a convolution's are added to what is cleared there)
     for (int i = totals ? 3 : 0; i < l.wg_count; ++i) {
-        if (i % 3 == 0) early[nearly++] = l.wg_sums[i];
+        if (i % 3 == 0 && x_early) early[nearly++] = l.wg_sums[i];
         else            late[nlate++] = l.wg_sums[i];          // ... of the gradient's copies once they are there
     }
     if (!s.conv) late[nlate++] = SumJob{g8, s.rows, s.cout, kSumRows, 1, l.row_sums};

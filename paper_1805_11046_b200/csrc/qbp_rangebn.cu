@@ -402,6 +402,31 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_stats_kernel(const float 
     }
 }
 
+// What the backward's second pass needs of a channel, from its complete sums: dbeta = sum dy, dgamma = sum dy*xhat,
+// m1 = gamma*dbeta/n, k2 = C(n)*gamma*dgamma; with the extremes ev of dy over the three sets of positions (see
+// bn_bwd_stats_kernel) also the exact range of the channel's dx and the rectifier's mask as a threshold on x.
+struct BnBwdOut { float *dgamma, *dbeta; float2 *coef, *chan_range, *relu_thr; };
+__device__ __forceinline__ void bn_bwd_channel(int c, double sdy, double sdyx, int64_t n, double Cn, float g, float b, float mu, float lo,
+                                               float hi, float Cn_f, const float *ev, const BnBwdOut &o)
+{
+    if (o.dbeta) o.dbeta[c] = (float)sdy;
+    if (o.dgamma) o.dgamma[c] = (float)sdyx;
+    const float m1 = (float)((double)g * sdy / (double)n), k2 = (float)(Cn * (double)g * sdyx);
+    o.coef[c] = make_float2(m1, k2);
+    if (!ev) return;
+    const float s = bn_scale(lo, hi, Cn_f);
+    float rlo = INFINITY, rhi = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (!(ev[2 * k] <= ev[2 * k + 1])) continue;           // (a set with no position keeps +inf, -inf)
+        const float ind = k == 0 ? 0.0f : k == 1 ? 1.0f : -1.0f;
+        const float v0 = bn_dx(ev[2 * k], ind, s, g, m1, k2), v1 = bn_dx(ev[2 * k + 1], ind, s, g, m1, k2);
+        rlo = fminf(rlo, fminf(v0, v1)); rhi = fmaxf(rhi, fmaxf(v0, v1));
+    }
+    o.chan_range[c] = make_float2(rlo, rhi);
+    if (o.relu_thr) o.relu_thr[c] = relu_threshold(mu, s, g, b);
+}
+
 constexpr int kFinThreads = kSumThreads;
 // One block of kFinThreads threads per channel: dbeta, dgamma, and the two per-channel
 // constants of dx: m1 = gamma*dbeta/n, k2 = C(n)*gamma*dgamma.
@@ -463,28 +488,14 @@ __global__ void __launch_bounds__(kFinThreads) bn_bwd_finalize_kernel(const doub
             sum_dy[c] = a; sum_dyx[c] = b;
             return;
         }
-        const double g = gamma ? (double)gamma[c] : 1.0;
-        if (dbeta) dbeta[c] = (float)a;
-        if (dgamma) dgamma[c] = (float)b;
-        const float m1 = (float)(g * a / (double)n), k2 = (float)(Cn * g * b);
-        coef[c] = make_float2(m1, k2);
+        BnBwdOut o{dgamma, dbeta, coef, chan_range, relu_thr};
         if (ext) {
-            const float s = bn_scale(vmin[c], vmax[c], Cn_f), gf = gamma ? gamma[c] : 1.0f;
-            float rlo = INFINITY, rhi = -INFINITY;
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                float lo = ev[2 * k], hi = ev[2 * k + 1];
-                for (int w = 1; w < kFinThreads / 32; ++w) { lo = fminf(lo, s_e[2 * k][w]); hi = fmaxf(hi, s_e[2 * k + 1][w]); }
-                if (lo <= hi) {              // (a set with no position keeps +inf, -inf)
-                    const float ind = k == 0 ? 0.0f : k == 1 ? 1.0f : -1.0f;
-                    const float v0 = bn_dx(lo, ind, s, gf, m1, k2), v1 = bn_dx(hi, ind, s, gf, m1, k2);
-                    rlo = fminf(rlo, fminf(v0, v1)); rhi = fmaxf(rhi, fmaxf(v0, v1));
-                }
-            }
-            chan_range[c] = make_float2(rlo, rhi);
-            // (the rectifier's mask of this channel as a threshold on x, for the pass that follows)
-            if (relu_thr) relu_thr[c] = relu_threshold(mean[c], s, gf, beta ? beta[c] : 0.0f);
+            for (int k = 0; k < 6; ++k)
+                for (int w = 1; w < kFinThreads / 32; ++w) ev[k] = (k & 1) ? fmaxf(ev[k], s_e[k][w]) : fminf(ev[k], s_e[k][w]);
         }
+        bn_bwd_channel(c, a, b, n, Cn, gamma ? gamma[c] : 1.0f, beta ? beta[c] : 0.0f, ext ? mean[c] : 0.0f, ext ? vmin[c] : 0.0f,
+                       ext ? vmax[c] : 0.0f, Cn_f, ext ? ev : nullptr, o);
     }
 }
 
@@ -715,6 +726,191 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_apply_kernel(const float 
     }
 }
 
+// ------------------------------------------------------------- few rows
+// With few rows (a linear layer's minibatch, a late stage's last positions) a block takes 16 channels whole: statistics and what
+// follows from them in one launch, where the passes above need a launch for the partials and one to combine them -- 2 to 4 us
+// each, which is what such a tensor costs.  Bound by latency: 512 threads, each row's 64 bytes by four of them, four rows in
+// flight.  Up to kFewRows rows (16 per thread); beyond, one block per 16 channels walks too long (at 7220 x 160 the
+// walk alone would take 17 us, the three launches take 12).
+constexpr int kFewThreads = 512, kFewRows = 2048, kFewHigh = kFewThreads / 4;
+static bool few_rows(int64_t n, int64_t C) { return n <= kFewRows && C % 4 == 0; }
+
+// Sum (fp64), min and max over a block's rows, per channel: the lanes of a warp that hold the same channels by shuffles, the
+// warps in shared memory; all threads end up with their four channels' values.
+template <int NS, int NM>      // sums; (min, max) pairs
+__device__ __forceinline__ void few_reduce(double (&sum)[NS][4], float (&lo)[NM][4], float (&hi)[NM][4])
+{
+    __shared__ double s_sum[NS][kFewThreads / 32][16];
+    __shared__ float s_lo[NM][kFewThreads / 32][16], s_hi[NM][kFewThreads / 32][16];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tx = lane & 3;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+#pragma unroll
+            for (int k = 0; k < NS; ++k) sum[k][e] += __shfl_xor_sync(0xffffffffu, sum[k][e], o);
+#pragma unroll
+            for (int k = 0; k < NM; ++k) {
+                lo[k][e] = fminf(lo[k][e], __shfl_xor_sync(0xffffffffu, lo[k][e], o));
+                hi[k][e] = fmaxf(hi[k][e], __shfl_xor_sync(0xffffffffu, hi[k][e], o));
+            }
+        }
+        if (lane < 4) {
+#pragma unroll
+            for (int k = 0; k < NS; ++k) s_sum[k][warp][tx * 4 + e] = sum[k][e];
+#pragma unroll
+            for (int k = 0; k < NM; ++k) { s_lo[k][warp][tx * 4 + e] = lo[k][e]; s_hi[k][warp][tx * 4 + e] = hi[k][e]; }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            double t = 0.0;
+            for (int w = 0; w < kFewThreads / 32; ++w) t += s_sum[k][w][tx * 4 + e];
+            sum[k][e] = t;
+        }
+#pragma unroll
+        for (int k = 0; k < NM; ++k)
+            for (int w = 0; w < kFewThreads / 32; ++w) { lo[k][e] = fminf(lo[k][e], s_lo[k][w][tx * 4 + e]); hi[k][e] = fmaxf(hi[k][e], s_hi[k][w][tx * 4 + e]); }
+    }
+}
+
+// Forward: the rows wait in registers between the statistics and the normalisation (ROWS per thread, a power of two).
+template <int ROWS>
+__global__ void __launch_bounds__(kFewThreads) bn_fwd_few_kernel(const float *__restrict__ x, int rows, int C, const float *__restrict__ gamma,
+                                                                 const float *__restrict__ beta, int relu, float Cn, float *__restrict__ y,
+                                                                 float *__restrict__ mean, float *__restrict__ vmin, float *__restrict__ vmax)
+{
+    pdl_enter();
+    const int col = (int)blockIdx.x * 16 + (threadIdx.x & 3) * 4, ty = threadIdx.x >> 2;
+    const bool active = col < C;
+    float4 v[ROWS];
+#pragma unroll
+    for (int u = 0; u < ROWS; ++u) {
+        const int r = ty + u * kFewHigh;
+        if (active && r < rows) v[u] = __ldg(reinterpret_cast<const float4 *>(x + (int64_t)r * C + col));
+    }
+    double sum[1][4];
+    float lo[1][4], hi[1][4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { sum[0][e] = 0.0; lo[0][e] = INFINITY; hi[0][e] = -INFINITY; }
+#pragma unroll
+    for (int u = 0; u < ROWS; ++u)
+        if (active && ty + u * kFewHigh < rows) {
+            const float t[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) { sum[0][e] += (double)t[e]; lo[0][e] = fminf(lo[0][e], t[e]); hi[0][e] = fmaxf(hi[0][e], t[e]); }
+        }
+    few_reduce<1, 1>(sum, lo, hi);
+    if (!active) return;
+    float mu[4], s[4], g[4], b[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        mu[e] = (float)(sum[0][e] / (double)rows);
+        s[e] = bn_scale(lo[0][e], hi[0][e], Cn);
+        g[e] = gamma ? gamma[col + e] : 1.0f; b[e] = beta ? beta[col + e] : 0.0f;
+        if (ty == 0) { mean[col + e] = mu[e]; vmin[col + e] = lo[0][e]; vmax[col + e] = hi[0][e]; }
+    }
+#pragma unroll
+    for (int u = 0; u < ROWS; ++u) {
+        const int r = ty + u * kFewHigh;
+        if (r >= rows) break;
+        float t[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            t[e] = bn_y(bn_xhat(t[e], mu[e], s[e]), g[e], b[e]);
+            if (relu) t[e] = fmaxf(t[e], 0.0f);
+        }
+        *reinterpret_cast<float4 *>(y + (int64_t)r * C + col) = make_float4(t[0], t[1], t[2], t[3]);
+    }
+}
+
+// Backward: the channel's sums and the extremes of dy, and what bn_bwd_channel makes of them.  (blocks behind the channels: code
+// sums that a later product needs; `zero`: cleared on the way)
+__global__ void __launch_bounds__(kFewThreads) bn_bwd_few_kernel(const float *__restrict__ dy, const float *__restrict__ x, int rows, int C,
+                                                                 const float *__restrict__ mean, const float *__restrict__ vmin,
+                                                                 const float *__restrict__ vmax, const float *__restrict__ gamma,
+                                                                 const float *__restrict__ beta, int relu, float Cn, double Cnd,
+                                                                 const BnBwdOut out, const ZeroJobs zero, const __grid_constant__ SumJobs J)
+{
+    pdl_enter();
+    const int blocks = (C + 15) / 16;
+    if ((int)blockIdx.x >= blocks) {
+        if (threadIdx.x < kSumThreads) code_sums_block(J, (int)blockIdx.x - blocks);
+        return;
+    }
+    run_zero_jobs(zero, (int64_t)blockIdx.x * kFewThreads + threadIdx.x, (int64_t)blocks * kFewThreads);
+    const int col = (int)blockIdx.x * 16 + (threadIdx.x & 3) * 4, ty = threadIdx.x >> 2;
+    const bool active = col < C;
+    double sum[2][4];
+    float lo[3][4], hi[3][4];             // ordinary positions, those at the channel's maximum, at its minimum
+    float mu[4], s[4], g[4], b[4], cl[4], ch[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int c = active ? col + e : 0;
+        sum[0][e] = sum[1][e] = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { lo[k][e] = INFINITY; hi[k][e] = -INFINITY; }
+        mu[e] = mean[c]; cl[e] = vmin[c]; ch[e] = vmax[c];
+        s[e] = bn_scale(cl[e], ch[e], Cn);
+        g[e] = gamma ? gamma[c] : 1.0f; b[e] = beta ? beta[c] : 0.0f;
+    }
+    constexpr int U = 4;
+    for (int r0 = ty; r0 < rows && active; r0 += U * kFewHigh) {
+        float4 vx[U], vd[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int r = r0 + u * kFewHigh;
+            if (r < rows) {
+                vx[u] = __ldg(reinterpret_cast<const float4 *>(x + (int64_t)r * C + col));
+                vd[u] = __ldg(reinterpret_cast<const float4 *>(dy + (int64_t)r * C + col));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (r0 + u * kFewHigh >= rows) break;
+            const float ax[4] = {vx[u].x, vx[u].y, vx[u].z, vx[u].w}, ad[4] = {vd[u].x, vd[u].y, vd[u].z, vd[u].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float xh = bn_xhat(ax[e], mu[e], s[e]);
+                float d = ad[e];
+                if (relu && !(bn_y(xh, g[e], b[e]) > 0.0f)) d = 0.0f;
+                sum[0][e] += (double)d;
+                sum[1][e] += (double)d * (double)xh;
+                const bool ih = ax[e] == ch[e], il = ax[e] == cl[e];
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    if (k == 0 ? ih == il : k == 1 ? ih && !il : il && !ih) { lo[k][e] = fminf(lo[k][e], d); hi[k][e] = fmaxf(hi[k][e], d); }
+            }
+        }
+    }
+    few_reduce<2, 3>(sum, lo, hi);
+    if (!active || ty > 3) return;
+    // four threads of the first rows per vector, one channel each (picked by selection: a branch per channel would run the
+    // threshold's bisection four times over, 10 us)
+    auto pick = [&](const auto &t) { return ty == 0 ? t[0] : ty == 1 ? t[1] : ty == 2 ? t[2] : t[3]; };
+    const float ev[6] = {pick(lo[0]), pick(hi[0]), pick(lo[1]), pick(hi[1]), pick(lo[2]), pick(hi[2])};
+    bn_bwd_channel(col + ty, pick(sum[0]), pick(sum[1]), rows, Cnd, pick(g), pick(b), pick(mu), pick(cl), pick(ch), Cn,
+                   out.chan_range ? ev : nullptr, out);
+}
+
+static int launch_bwd_few(const float *dy, const float *x, int64_t n, int64_t C, const float *gamma, const float *beta, int relu,
+                          const float *mean, const float *vmin, const float *vmax, const BnBwdOut &out, const ZeroJobs &zero,
+                          const SumJob *extra, int extra_count, cudaStream_t st)
+{
+    SumJobs J{};
+    int sum_blocks = 0;
+    if (extra_count) if (int rc = fill_sum_jobs(extra, extra_count, J, &sum_blocks)) return rc;
+    const double Cnd = 1.0 / std::sqrt(2.0 * std::log((double)n));
+    QBP_TRACE_BEGIN(st);
+    launch(bn_bwd_few_kernel, (int)((C + 15) / 16) + sum_blocks, kFewThreads, 0, st, dy, x, (int)n, (int)C, mean, vmin, vmax, gamma, beta,
+           relu, (float)Cnd, Cnd, out, zero, J);
+    QBP_LAUNCH_OK("bn_bwd_few_kernel");
+    return QBP_OK;
+}
+
 static size_t bn_ws_bytes(int64_t C)
 {
     // forward: lo, hi (float) + sum (double) partials; backward: two double partials + coefficients
@@ -845,6 +1041,18 @@ extern "C" __attribute__((visibility("default"))) int qbp_rangebn_fwd_q8(const f
     if (rc) return rc;
     if (!y && !rq) return fail(QBP_ERR_INVALID_ARG, "rangebn_fwd: NULL tensor");
     if (!save_mean || !save_min || !save_max) return fail(QBP_ERR_INVALID_ARG, "rangebn_fwd: NULL statistics buffer");
+    if (!rq && !out_range && few_rows(n, C) && aligned16(x) && aligned16(y)) {
+        const float Cn = (float)(1.0 / std::sqrt(2.0 * std::log((double)n)));
+        const int grid = (int)((C + 15) / 16);
+        QBP_TRACE_BEGIN(st);
+#define QBP_BN_FEW(ROWS_) launch(bn_fwd_few_kernel<ROWS_>, grid, kFewThreads, 0, st, x, (int)n, (int)C, gamma, beta, relu, Cn, y, save_mean, save_min, save_max)
+        if (n <= kFewHigh)          QBP_BN_FEW(1);
+        else if (n <= 4 * kFewHigh) QBP_BN_FEW(4);
+        else                        QBP_BN_FEW(16);
+#undef QBP_BN_FEW
+        QBP_LAUNCH_OK("bn_fwd_few_kernel");
+        return QBP_OK;
+    }
     if ((rc = bn_fwd_stats_launch(x, n, C, save_mean, save_min, save_max, nullptr, ws, ws_bytes, st))) return rc;
     return bn_fwd_apply_launch(x, n, n, C, gamma, beta, relu, y, save_mean, save_min, save_max, out_range, rq, st);
 }
@@ -993,6 +1201,9 @@ static int bn_bwd_apply_launch(const float *dy, const float *x, int64_t n_rows, 
     return QBP_OK;
 }
 
+// Whether the statistics of rangebn_bwd_bifurcate_impl are one launch: what it clears is then not clear before `extra` runs.
+bool rangebn_bwd_one_launch(int64_t n, int64_t C) { return few_rows(n, C); }
+
 // Whether rangebn_bwd_bifurcate_impl takes a tensor of C channels (row_sums: each row's 8-bit code sum is wanted).
 bool rangebn_bwd_bifurcate_supported(const float *dy, const float *x, const float *g_out, int64_t n, int64_t C, bool row_sums)
 {
@@ -1032,7 +1243,11 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
     ZeroJobs zero{};
     if (row_sums8 && (ga.tw > 32 || ga.slabs > 1)) { zero.p[0] = reinterpret_cast<uint32_t *>(row_sums8); zero.words[0] = n; }
     zero.p[1] = static_cast<uint32_t *>(clear); zero.words[1] = clear_words;
-    if ((rc = bn_bwd_stats_launch(dy, x, n, n, C, gamma, beta, relu, save_mean, save_min, save_max, dgamma, dbeta, coef, nullptr,
+    if (few_rows(n, C)) {
+        if ((rc = launch_bwd_few(dy, x, n, C, gamma, beta, relu, save_mean, save_min, save_max,
+                                 BnBwdOut{dgamma, dbeta, coef, chan_range, relu ? relu_thr : nullptr}, zero, extra, extra_count, st)))
+            return rc;
+    } else if ((rc = bn_bwd_stats_launch(dy, x, n, n, C, gamma, beta, relu, save_mean, save_min, save_max, dgamma, dbeta, coef, nullptr,
                                   nullptr, pa, pb, st, ext, chan_range, relu ? relu_thr : nullptr, zero, extra, extra_count)))
         return rc;
     const RangeSrc range{chan_range, (int)C, nullptr, qp8, qp16};
@@ -1069,7 +1284,11 @@ int qbp::rangebn_bwd_impl(const float *dy, const float *x, int64_t n, int64_t C,
     w.take<float>((size_t)kScanMaxStrips * C);
     w.take<float>((size_t)kScanMaxStrips * C);
     float2 *coef = w.take<float2>((size_t)C);
-    if ((rc = bn_bwd_stats_launch(dy, x, n, n, C, gamma, beta, relu, save_mean, save_min, save_max, dgamma, dbeta, coef,
+    if (few_rows(n, C) && aligned16(x) && aligned16(dy)) {
+        if ((rc = launch_bwd_few(dy, x, n, C, gamma, beta, relu, save_mean, save_min, save_max, BnBwdOut{dgamma, dbeta, coef, nullptr, nullptr},
+                                 ZeroJobs{}, nullptr, 0, st)))
+            return rc;
+    } else if ((rc = bn_bwd_stats_launch(dy, x, n, n, C, gamma, beta, relu, save_mean, save_min, save_max, dgamma, dbeta, coef,
                                   nullptr, nullptr, pa, pb, st)))
         return rc;
     return bn_bwd_apply_launch(dy, x, n, n, C, gamma, beta, relu, save_mean, save_min, save_max, coef, dx, range_parts, nparts, st);

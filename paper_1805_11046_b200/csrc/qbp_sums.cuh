@@ -102,7 +102,7 @@ __device__ __forceinline__ void code_sums_block(const SumJobs &J, int blk)
 #pragma unroll
         for (int e = 0; e < 16; ++e) s_acc[threadIdx.x >> 5][lane * 16 + e] = acc[e];
     }
-    __syncthreads();
+    named_barrier(1, kSumThreads);       // (the block may have more threads than take part)
     const int c = (strip << (j.lg_log2 + 4)) + (int)threadIdx.x;
     if ((int)threadIdx.x < 16 * lg && c < j.cols) {
         int sum = 0;

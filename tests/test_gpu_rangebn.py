@@ -116,3 +116,19 @@ def test_sweep_shapes_full_size(B, hw, C):
     s = 1.0 / (O.rangebn_C(n) * (to_host(vmax).astype(np.float64) - to_host(vmin)))
     want_max = (to_host(vmax).astype(np.float64) - to_host(mean)) * s
     assert np.allclose(yh.max(0), np.maximum(want_max, 0), rtol=1e-5)
+
+
+@pytest.mark.parametrize("n,C", [(2, 4), (127, 20), (128, 16), (129, 36), (512, 12), (513, 64), (2047, 8), (2048, 40), (2049, 40)])
+@pytest.mark.parametrize("relu", [False, True])
+def test_few_rows(B, n, C, relu):
+    """Up to 2048 rows a block takes 16 channels whole (one launch for statistics and normalisation): one, four and sixteen
+    rows per thread and their edges, channel groups partly filled, the first size beyond."""
+    x = synth.channel_gaussian((n, 1, 1, C), 30, 31).reshape(n, C); dy = synth.normal((n, C), 32)
+    gamma = synth.uniform((C,), 33, 1.0) + np.float32(1.5); beta = synth.uniform((C,), 34, 0.5)
+    gamma[::3] *= -1
+    y, mean, vmin, vmax, _ = B.qbp_rangebn_fwd(to_dev(x), to_dev(gamma), to_dev(beta), relu)
+    oy, om, olo, ohi = O.rangebn_fwd(x, gamma, beta, relu)
+    assert np.array_equal(to_host(vmin), olo) and np.array_equal(to_host(vmax), ohi)
+    assert np.abs(to_host(mean) - om).max() <= 1e-6 * max(1.0, np.abs(om).max())
+    assert _per_channel_rel(to_host(y), oy, _scales(x, dy, olo, ohi, gamma, beta)[0]) <= FP32_TOL
+    _run(B, x, dy, gamma, beta, relu)
