@@ -1421,6 +1421,12 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
         }
     }
 
+    int bwl = 0, bhl = 0;
+    pick_pixel_box(d->N, d->H, d->W, bwl, bhl);
+    // 3 x 3 with many channels on both sides: CTA pairs (the epilogue's tail is the single-CTA kernel's)
+    if (conv2_eligible(d, dgrad) && !(tail && (tail->fold || tail->relu || tail->q)))
+        return launch_conv2(dgrad, d, in, q_in, wgt, q_w, acc_out, out, rowterm, colterm, stats, status, bwl, bhl, st);
+
     MmaParams P{};
     P.mode = dgrad ? MODE_DGRAD : MODE_FPROP;
     P.msub = 1; P.ncls = raw_sums ? 1 : 16; P.nslab = 1;
@@ -1448,8 +1454,6 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
     P.tiles_n = (Nout + P.bn - 1) / P.bn;
     P.M = pix; P.N = Nout;
 
-    int bwl = 0, bhl = 0;
-    pick_pixel_box(d->N, d->H, d->W, bwl, bhl);
     // 3 x 3: a box of 16 rows x 8 pixels of one image, loaded once with its border; the nine taps are windows of
     // that tile (a ninth of the operand traffic of one load per tap).  Taken when the filter stays resident and the
     // fixed box does not waste many more MMA rows than the free one.

@@ -158,12 +158,21 @@ int make_map_nhwc(CUtensorMap *map, const void *base, uint64_t N, uint64_t H, ui
 
 // fp32 output matrix [rows x cols] stored by TMA in boxes of 32 rows x 32 columns (128-byte swizzled slabs).
 int make_map_out_2d(CUtensorMap *map, float *base, uint64_t rows, uint64_t cols);
+// fp32 NHWC output stored in boxes of 32 channels x (sw x sh x sn = 32 pixels).
+int make_map_out_nhwc(CUtensorMap *map, float *base, uint64_t N, uint64_t H, uint64_t W, uint64_t C, uint32_t sn,
+                      uint32_t sh, uint32_t sw);
 
 // ---- the dense product on CTA pairs (qbp_mma2.cu) -------------------------------
 bool gemm2_eligible(int64_t M, int64_t N, int64_t K);
 int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,
                  const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const CodeSums &a_sums,
                  const CodeSums &b_sums, int *status, cudaStream_t st);
+
+// ---- the 3 x 3 convolution products on CTA pairs (qbp_conv2.cu); bwl / bhl: log2 of the position box's extents ----
+bool conv2_eligible(const qbp_conv_desc *d, bool dgrad);
+int launch_conv2(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp_qparams *q_in, const int8_t *wgt,
+                 const qbp_qparams *q_w, int32_t *acc_out, float *out, const int32_t *rowterm, const int32_t *colterm,
+                 ColStatParts *stats, int *status, int bwl, int bhl, cudaStream_t st);
 
 // ---- the dense weight gradient on CTA pairs (qbp_wgrad2.cu) ----------------------
 bool wgrad2_eligible(int64_t M, int64_t N, int64_t K);

@@ -468,3 +468,24 @@ def test_wgrad_conv_edge_sums(B, N, H, W, C, K):
     oacc, oout = O.conv_wgrad_s16(od, X, -90, G, 2077, 0.5, 0.25)
     assert B.status_word(ws) == 0
     assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
+
+
+# ------------------------------------------- 3x3 convolutions of many channels (CTA pairs)
+@pytest.mark.parametrize("N,H,W,C,K", [(1, 1, 1, 96, 96), (2, 5, 6, 96, 160), (3, 9, 7, 128, 256), (2, 14, 14, 288, 112), (1, 8, 16, 256, 400),
+                                       (40, 28, 28, 128, 256), (90, 14, 14, 256, 512)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_conv_pairs(B, N, H, W, C, K, mode):
+    """One box and an odd number of boxes per column of tiles, channel chunks and column tiles partly filled on either side, tiles of
+    128 and of 256 channels (the last two fill the machine), more tiles than pairs; accumulators, output and statistics."""
+    d = B.conv_desc(N, H, W, C, K, 3, 3, 1, 1); od = O.conv_desc(N, H, W, C, K, 3, 3, 1, 1)
+    inp = random_codes((N, H, W, C if mode == 0 else K), 81); w = random_codes((K, 3, 3, C), 82)
+    zi, zw = -31, 14
+    acc, out, ws, stats = B.qbp_conv_s8_implicit(mode, d, to_dev(inp), _qp(B, 0.5, zi), to_dev(w), _qp(B, 0.25, zw), want_acc=True, col_stats=True)
+    assert B.status_word(ws) == 0
+    a, o = to_host(acc).ravel(), to_host(out).ravel()
+    idx = np.arange(a.size) if a.size <= 1 << 19 else np.unique(np.concatenate(
+        [[0, a.size - 1], np.random.Generator(np.random.PCG64(83)).integers(0, a.size, 1 << 14)]))
+    oacc, oout, bad = O.conv_s8(mode, od, inp, zi, w, zw, 0.5, 0.25, idx=idx.astype(np.int64))
+    assert bad == 0 and np.array_equal(a[idx], oacc) and np.array_equal(o[idx], oout)
+    assert np.array_equal(o, a.astype(np.float32) * np.float32(0.125))
+    _check_col_stats(out, stats)
