@@ -180,19 +180,20 @@ __device__ __forceinline__ int quantize_code(float x, float inv_scale, float zp_
 // L * 2^16 is the clamp at the top (then nothing can carry).
 // The caller passes inv_scale and zp_u already multiplied by 2^16: scaling by a power of two commutes with the
 // rounding of the fused multiply-add, so fma(x, inv * 2^16, zp * 2^16) is exactly 2^16 * fma(x, inv, zp).
-// 8 bits: the code is byte 2 of the result; the draw is the high half of rnd.
+// What is stored is the code with its top bit flipped (code - 2^(M-1)); that bit is flipped by the same addition.
+// 8 bits: the stored code is byte 2 of the result (byte 3 is not to be used); the draw is the high half of rnd.
 __device__ __forceinline__ uint32_t quantize_sr8_byte2(float x, float inv_scale_2p16, float zp_u_2p16, uint32_t rnd)
 {
     uint32_t tc;
     asm("cvt.rpi.sat.u32.f32 %0, %1;" : "=r"(tc) : "f"(__fmaf_rn(x, inv_scale_2p16, zp_u_2p16)));
-    return min(tc, 0x00FF0000u) + ((~rnd) >> 16);
+    return min(tc, 0x00FF0000u) + 0x0080FFFFu - (rnd >> 16);
 }
-// 16 bits: the code is the upper half of the result (high byte = byte 3, low byte = byte 2); the draw is the low half of rnd.
+// 16 bits: the stored code is the upper half of the result (high byte = byte 3, low byte = byte 2); the draw is the low half of rnd.
 __device__ __forceinline__ uint32_t quantize_sr16_top_half(float x, float inv_scale_2p16, float zp_u_2p16, uint32_t rnd)
 {
     uint32_t tc;
     asm("cvt.rpi.sat.u32.f32 %0, %1;" : "=r"(tc) : "f"(__fmaf_rn(x, inv_scale_2p16, zp_u_2p16)));
-    return min(tc, 0xFFFF0000u) + ((~rnd) & 0xFFFFu);
+    return min(tc, 0xFFFF0000u) + 0x80000000u + ((~rnd) & 0xFFFFu);
 }
 
 // Philox4x32-10 with the ten round keys precomputed (they depend on the key only); passed to a kernel by value,
@@ -218,6 +219,26 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxKeys &k)
     return c;
 }
 
+// Four consecutive elements of a gradient bifurcated (Section 6): the four stored 8-bit codes, and the high and low limbs of the
+// four stored 16-bit codes (the low one XORed with lo_flip).  r8, r16: their Philox words (the same for equal tensor ids: the 8-bit
+// draw is a word's high half, the 16-bit draw its low half).  c16: the 16-bit codes, each in the upper half of its word.
+struct BifWords { uint32_t q8, hi, lo; };
+__device__ __forceinline__ BifWords bifurcate4(const float (&v)[4], float inv8, float zp8, float inv16, float zp16, const uint4 &r8,
+                                               const uint4 &r16, uint32_t lo_flip, uint32_t (&c16)[4])
+{
+    const uint32_t w8[4] = {r8.x, r8.y, r8.z, r8.w}, w16[4] = {r16.x, r16.y, r16.z, r16.w};
+    uint32_t c8[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        c8[e] = quantize_sr8_byte2(v[e], inv8, zp8, w8[e]);
+        c16[e] = quantize_sr16_top_half(v[e], inv16, zp16, w16[e]);
+    }
+    // (low, low, high, high) bytes of two 16-bit codes each, then the two words: four permutes for both limbs
+    const uint32_t t01 = __byte_perm(c16[0], c16[1], 0x7362), t23 = __byte_perm(c16[2], c16[3], 0x7362);
+    return {__byte_perm(__byte_perm(c8[0], c8[1], 0x0062), __byte_perm(c8[2], c8[3], 0x0062), 0x5410), __byte_perm(t01, t23, 0x7632),
+            __byte_perm(t01, t23, 0x5410) ^ lo_flip};
+}
+
 // Range BN (Section 3, Eq. (range)): xhat and y of one element and the per-channel scale 1 / (C(n) (max - min)).
 // The order of operations is part of the contract: every kernel that normalises (the apply passes, the fused
 // epilogue of a product) must produce the same bits, so that forward, backward and requantisation agree.
@@ -227,11 +248,13 @@ __device__ __forceinline__ float bn_y(float xh, float g, float b) { return __fad
 // dx = s * (gamma * dy - m1 - k2 * ind), ind = [x == max] - [x == min].  Every operation is rounded on its own and
 // none is contracted, so the value is a monotone function of dy for fixed (s >= 0, gamma, m1, k2, ind): the extremes of
 // dx over a set of positions are this function of the extremes of dy (which is how the gradient's range is known
-// before the gradient is written).
-__device__ __forceinline__ float bn_dx(float d, float ind, float s, float g, float m1, float k2)
+// before the gradient is written).  t = k2 * ind.
+__device__ __forceinline__ float bn_dx(float d, float t, float s, float g, float m1)
 {
-    return __fmul_rn(s, __fsub_rn(__fsub_rn(__fmul_rn(g, d), m1), __fmul_rn(k2, ind)));
+    return __fmul_rn(s, __fsub_rn(__fsub_rn(__fmul_rn(g, d), m1), t));
 }
+// k2 * ind of a value (in a constant channel, max == min, s is 0 and t does not count)
+__device__ __forceinline__ float bn_k2_ind(float x, float lo, float hi, float k2) { return x == hi ? k2 : x == lo ? -k2 : 0.0f; }
 // Floats as integers that compare the same way (and back): for atomic minima and maxima of floats.
 __device__ __forceinline__ int float_order(float f) { const int b = __float_as_int(f); return b ^ ((b >> 31) & 0x7fffffff); }
 __device__ __forceinline__ float order_float(int i) { return __int_as_float(i ^ ((i >> 31) & 0x7fffffff)); }

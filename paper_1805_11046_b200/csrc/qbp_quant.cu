@@ -356,7 +356,8 @@ __device__ __forceinline__ uint32_t pack_bytes2(const uint32_t (&c)[4])
 // PERCH is a template parameter so that the per-tensor instance (the hot one: it is bound by its instruction
 // count when rounding stochastically) carries none of the per-channel parameter handling.
 // TOTALS: the instance that also leaves the per-channel totals (the others carry none of that work).
-template <bool SR, int VEC, bool PERCH, bool TOTALS>
+// J32: every Philox block index is below 2^32 (the first two rounds then have constant halves).  Four blocks per SM.
+template <bool SR, int VEC, bool PERCH, bool TOTALS, bool J32>
 __device__ __forceinline__ void quantize_body(const QuantJob &J, const PhiloxKeys &keys, int block, int blocks)
 {
     const float *__restrict__ x = J.x;
@@ -392,7 +393,7 @@ __device__ __forceinline__ void quantize_body(const QuantJob &J, const PhiloxKey
     // both copies of a gradient under one tensor id: one Philox block serves the two (disjoint halves of each word)
     const bool one_block = want8 && want16 && id8 == id16;
     int cs8[4] = {0, 0, 0, 0};                               // this thread's channels: totals of the stored 8-bit codes
-    unsigned cs16[4] = {0, 0, 0, 0};                         // ... and of the unsigned 16-bit codes (fewer than 65536 per thread)
+    int cs16[4] = {0, 0, 0, 0};                              // ... and of the stored 16-bit codes (fewer than 65536 per thread)
     const int64_t nv = n >> 2;
     const int64_t stride = (int64_t)blocks * kThreads * kUnroll;
     for (int64_t base = (int64_t)block * kThreads * kUnroll; base < nv; base += stride) {
@@ -419,8 +420,8 @@ __device__ __forceinline__ void quantize_body(const QuantJob &J, const PhiloxKey
             if (SR) {
                 // counter = the block's index in the whole tensor (a shard of a larger tensor starts at index_base)
                 const uint64_t jb = (uint64_t)j + (index_base >> 2);
-                if (want8) b8 = philox4x32_10(make_uint4((uint32_t)jb, (uint32_t)(jb >> 32), id8, 0u), keys);
-                if (want16) b16 = one_block ? b8 : philox4x32_10(make_uint4((uint32_t)jb, (uint32_t)(jb >> 32), id16, 0u), keys);
+                if (want8) b8 = philox4x32_10(make_uint4((uint32_t)jb, J32 ? 0u : (uint32_t)(jb >> 32), id8, 0u), keys);
+                if (want16) b16 = one_block ? b8 : philox4x32_10(make_uint4((uint32_t)jb, J32 ? 0u : (uint32_t)(jb >> 32), id16, 0u), keys);
             }
             if (want8) {
                 const uint32_t r[4] = {b8.x, b8.y, b8.z, b8.w};
@@ -435,7 +436,7 @@ __device__ __forceinline__ void quantize_body(const QuantJob &J, const PhiloxKey
                     c[e] = SR ? quantize_sr8_byte2(xs[e], p8.inv, p8.zp_u, r[e])
                               : (uint32_t)quantize_code<SR>(xs[e], p8.inv, p8.zp_u, 255.0f, r[e]);
                 }
-                const uint32_t packed = (SR ? pack_bytes2(c) : pack_bytes0(c)) ^ 0x80808080u;       // stored = unsigned code - 128
+                const uint32_t packed = SR ? pack_bytes2(c) : pack_bytes0(c) ^ 0x80808080u;       // stored = unsigned code - 128
                 reinterpret_cast<uint32_t *>(o.q8)[j] = packed;
                 if (o.rowsum8) rs[u] = __dp4a((int)packed, 0x01010101, 0);
                 if (TOTALS && o.chansum8) {
@@ -458,21 +459,20 @@ __device__ __forceinline__ void quantize_body(const QuantJob &J, const PhiloxKey
                               : (uint32_t)quantize_code<SR>(xs[e], p16.inv, p16.zp_u, 65535.0f, r[e]);
                 }
                 if (TOTALS && o.chansum16) {
-                    // unsigned codes here (the offset of 32768 per element is taken off when the block adds its totals up)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) cs16[e] += SR ? c[e] >> 16 : c[e];
+                    for (int e = 0; e < 4; ++e) cs16[e] += SR ? (int)c[e] >> 16 : (int)c[e] - 32768;
                 }
                 // stored = unsigned code - 32768: flip the top bit of every code (of every high byte)
                 if (o.q16)
-                    reinterpret_cast<uint2 *>(o.q16)[j] = make_uint2(__byte_perm(c[0], c[1], SR ? 0x7632 : 0x5410) ^ 0x80008000u,
-                                                                     __byte_perm(c[2], c[3], SR ? 0x7632 : 0x5410) ^ 0x80008000u);
+                    reinterpret_cast<uint2 *>(o.q16)[j] = make_uint2(__byte_perm(c[0], c[1], SR ? 0x7632 : 0x5410) ^ (SR ? 0u : 0x80008000u),
+                                                                     __byte_perm(c[2], c[3], SR ? 0x7632 : 0x5410) ^ (SR ? 0u : 0x80008000u));
                 if (SR && o.hi && o.lo) {
                     // (low, low, high, high) bytes of two codes each, then the two words: four permutes for both limbs
                     const uint32_t t01 = __byte_perm(c[0], c[1], 0x7362), t23 = __byte_perm(c[2], c[3], 0x7362);
-                    reinterpret_cast<uint32_t *>(o.hi)[j] = __byte_perm(t01, t23, 0x7632) ^ 0x80808080u;
+                    reinterpret_cast<uint32_t *>(o.hi)[j] = __byte_perm(t01, t23, 0x7632);
                     reinterpret_cast<uint32_t *>(o.lo)[j] = __byte_perm(t01, t23, 0x5410) ^ o.lo_flip;
                 } else {
-                    if (o.hi) reinterpret_cast<uint32_t *>(o.hi)[j] = (SR ? pack_bytes3(c) : pack_bytes1(c)) ^ 0x80808080u;
+                    if (o.hi) reinterpret_cast<uint32_t *>(o.hi)[j] = SR ? pack_bytes3(c) : pack_bytes1(c) ^ 0x80808080u;
                     if (o.lo) reinterpret_cast<uint32_t *>(o.lo)[j] = (SR ? pack_bytes2(c) : pack_bytes0(c)) ^ o.lo_flip;
                 }
             }
@@ -499,14 +499,10 @@ __device__ __forceinline__ void quantize_body(const QuantJob &J, const PhiloxKey
         for (int c = threadIdx.x; c < 2 * cols; c += kThreads) s_cs[c] = 0;
         __syncthreads();
         const int c0 = 4 * (threadIdx.x & ((cols >> 2) - 1));
-        // how many elements this thread quantised per channel: the 16-bit totals were taken over unsigned codes
-        int64_t mine = 0;
-        for (int64_t base = (int64_t)block * kThreads * kUnroll; base < nv; base += stride)
-            for (int u = 0; u < kUnroll; ++u) mine += (base + u * kThreads + threadIdx.x < nv) ? 1 : 0;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             if (o.chansum8 && cs8[e]) atomicAdd(&s_cs[c0 + e], cs8[e]);
-            if (o.chansum16) atomicAdd(&s_cs[cols + c0 + e], (int)((long long)cs16[e] - mine * 32768));
+            if (o.chansum16) atomicAdd(&s_cs[cols + c0 + e], cs16[e]);
         }
         __syncthreads();
         for (int c = threadIdx.x; c < cols; c += kThreads) {
@@ -516,11 +512,54 @@ __device__ __forceinline__ void quantize_body(const QuantJob &J, const PhiloxKey
     }
 }
 
-template <bool SR, int VEC, bool PERCH, bool TOTALS>
-__global__ void __launch_bounds__(kThreads) quantize_kernel(const __grid_constant__ QuantJob J, const __grid_constant__ PhiloxKeys keys)
+template <bool SR, int VEC, bool PERCH, bool TOTALS, bool J32>
+__global__ void __launch_bounds__(kThreads, 4) quantize_kernel(const __grid_constant__ QuantJob J, const __grid_constant__ PhiloxKeys keys)
 {
     pdl_enter();
-    quantize_body<SR, VEC, PERCH, TOTALS>(J, keys, (int)blockIdx.x, (int)gridDim.x);
+    quantize_body<SR, VEC, PERCH, TOTALS, J32>(J, keys, (int)blockIdx.x, (int)gridDim.x);
+}
+
+// A gradient's 8-bit copy and the byte limbs of its 16-bit copy, nothing else (the usual bifurcation): the integer pipes bound
+// it, so the general body's checks and 64-bit indices are left out (26 instructions per element instead of 39) and four blocks
+// share an SM.  25.7 M elements with a range that is known: 50 -> 37 us (4.9 TB/s).  Not better: two vectors per thread with
+// six blocks (41) or with the next two fetched ahead (41).
+// ONE: both copies have one tensor id and share their Philox blocks.
+template <bool ONE>
+__global__ void __launch_bounds__(kThreads, 4) bifurcate_kernel(const __grid_constant__ QuantJob J, const __grid_constant__ PhiloxKeys keys)
+{
+    pdl_enter();
+    QParamsReg p8 = {0, 0}, p16 = {0, 0};
+    resolve_range(J.r, true, true, blockIdx.x == 0, p8, p16);
+    const QParamsReg t8 = p8, t16 = p16;
+    const float inv8 = p8.inv * 65536.0f, zp8 = p8.zp_u * 65536.0f, inv16 = p16.inv * 65536.0f, zp16 = p16.zp_u * 65536.0f;
+    const float4 *const x = reinterpret_cast<const float4 *>(J.x);
+    uint32_t *const q8 = reinterpret_cast<uint32_t *>(J.o.q8), *const hi = reinterpret_cast<uint32_t *>(J.o.hi), *const lo = reinterpret_cast<uint32_t *>(J.o.lo);
+    const uint32_t nv = (uint32_t)(J.n >> 2), first = (uint32_t)(J.index_base >> 2);
+    auto work = [&](const float4 &f, uint32_t j) {
+        const float v[4] = {f.x, f.y, f.z, f.w};
+        const uint4 r8 = philox4x32_10(make_uint4(j + first, 0u, J.id8, 0u), keys);
+        const uint4 r16 = ONE ? r8 : philox4x32_10(make_uint4(j + first, 0u, J.id16, 0u), keys);
+        uint32_t c16[4];
+        const BifWords w = bifurcate4(v, inv8, zp8, inv16, zp16, r8, r16, J.o.lo_flip, c16);
+        q8[j] = w.q8; hi[j] = w.hi; lo[j] = w.lo;
+    };
+    constexpr uint32_t kStep = kThreads * kUnroll;
+    for (uint64_t base = (uint64_t)blockIdx.x * kStep; base < nv; base += (uint64_t)gridDim.x * kStep) {
+        const uint32_t j = (uint32_t)base + threadIdx.x;
+        if (base + kStep <= nv) {
+            float4 v[kUnroll];
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) v[u] = __ldg(x + (j + u * kThreads));
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) work(v[u], j + u * kThreads);
+        } else {
+#pragma unroll 1
+            for (int u = 0; u < kUnroll; ++u)
+                if (base + u * kThreads + threadIdx.x < nv) work(__ldg(x + (j + u * kThreads)), j + u * kThreads);
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        for (int64_t i = (int64_t)nv << 2; i < J.n; ++i) quantize_scalar<true>(J, i, false, t8, t16, keys);
 }
 
 // A layer's weights (the first b_blocks blocks) and activation in one launch; nearest rounding, per tensor.
@@ -529,8 +568,8 @@ __global__ void __launch_bounds__(kThreads) quantize_pair_kernel(const __grid_co
 {
     pdl_enter();
     const PhiloxKeys none = {};
-    if ((int)blockIdx.x < b_blocks) quantize_body<false, 4, false, false>(b, none, (int)blockIdx.x, b_blocks);
-    else                            quantize_body<false, 4, false, TOTALS>(a, none, (int)blockIdx.x - b_blocks, (int)gridDim.x - b_blocks);
+    if ((int)blockIdx.x < b_blocks) quantize_body<false, 4, false, false, false>(b, none, (int)blockIdx.x, b_blocks);
+    else                            quantize_body<false, 4, false, TOTALS, false>(a, none, (int)blockIdx.x - b_blocks, (int)gridDim.x - b_blocks);
 }
 
 // The sums of up to eight code tensors in a launch of their own (see qbp_sums.cuh).
@@ -702,24 +741,32 @@ static int launch_quantize(const float *x, int64_t n, int64_t cols, int perch, i
     const size_t smem = !vec ? 0 : totals ? (size_t)cols * 2 * sizeof(int) : (size_t)smem_cols * 2 * sizeof(float2);
     const int64_t groups = (n + per_block - 1) / per_block;
     const QuantJob J{x, n, (int)cols, r, id8, id16, o, smem_cols, index_base};
-#define QBP_QUANT2(SR_, VEC_, PC_, TOT_)                                                                                \
+    const bool j32 = (((uint64_t)n + index_base) >> 2) < (1ull << 32) - 1;
+#define QBP_QUANT3(SR_, VEC_, PC_, TOT_, J32_)                                                                          \
     do {                                                                                                                \
-        const int grid = grid_for(blocks_per_sm<quantize_kernel<SR_, VEC_, PC_, TOT_>>(kThreads), groups);              \
+        const int grid = grid_for(blocks_per_sm<quantize_kernel<SR_, VEC_, PC_, TOT_, J32_>>(kThreads), groups);        \
         QBP_TRACE_BEGIN(st);                                                                                            \
-        launch(quantize_kernel<SR_, VEC_, PC_, TOT_>, grid, kThreads, smem, st, J, key);                                \
+        launch(quantize_kernel<SR_, VEC_, PC_, TOT_, J32_>, grid, kThreads, smem, st, J, key);                          \
     } while (0)
-#define QBP_QUANT(SR_, VEC_, PC_) QBP_QUANT2(SR_, VEC_, PC_, false)
-    if (totals) {           // (vector path, per tensor: checked above)
-        if (sr) QBP_QUANT2(true, 4, false, true); else QBP_QUANT2(false, 4, false, true);
-    } else if (sr) {
-        if (vec) { if (perch) QBP_QUANT(true, 4, true); else QBP_QUANT(true, 4, false); }
-        else     { if (perch) QBP_QUANT(true, 1, true); else QBP_QUANT(true, 1, false); }
-    } else {
-        if (vec) { if (perch) QBP_QUANT(false, 4, true); else QBP_QUANT(false, 4, false); }
-        else     { if (perch) QBP_QUANT(false, 1, true); else QBP_QUANT(false, 1, false); }
+#define QBP_QUANT(PC_, TOT_)                                                                                            \
+    do {                                                                                                                \
+        if (sr) { if (j32) QBP_QUANT3(true, 4, PC_, TOT_, true); else QBP_QUANT3(true, 4, PC_, TOT_, false); }          \
+        else QBP_QUANT3(false, 4, PC_, TOT_, false);                                                                    \
+    } while (0)
+    if (sr && vec && !perch && !totals && j32 && o.q8 && o.hi && o.lo && !o.q16 && !o.rowsum8) {
+        QBP_TRACE_BEGIN(st);
+        if (id8 == id16) launch(bifurcate_kernel<true>, grid_for(blocks_per_sm<bifurcate_kernel<true>>(kThreads), groups), kThreads, 0, st, J, key);
+        else             launch(bifurcate_kernel<false>, grid_for(blocks_per_sm<bifurcate_kernel<false>>(kThreads), groups), kThreads, 0, st, J, key);
+        QBP_LAUNCH_OK("quantize_kernel");
+        return QBP_OK;
     }
+    if (totals) QBP_QUANT(false, true);           // (vector path, per tensor: checked above)
+    else if (vec && perch) QBP_QUANT(true, false);
+    else if (vec) QBP_QUANT(false, false);
+    else if (sr) { if (perch) QBP_QUANT3(true, 1, true, false, false); else QBP_QUANT3(true, 1, false, false, false); }
+    else         { if (perch) QBP_QUANT3(false, 1, true, false, false); else QBP_QUANT3(false, 1, false, false, false); }
+#undef QBP_QUANT3
 #undef QBP_QUANT
-#undef QBP_QUANT2
     QBP_LAUNCH_OK("quantize_kernel");
     return QBP_OK;
 }

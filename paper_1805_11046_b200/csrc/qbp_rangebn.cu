@@ -12,7 +12,9 @@
 #include "qbp_mma.cuh"
 #include "qbp_sums.cuh"
 
+#include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 namespace qbp {
 
@@ -278,6 +280,10 @@ __global__ void __launch_bounds__(256) bn_out_range_kernel(const float *__restri
 // channel's maximum, where it is its minimum, and everywhere else -- as ext [6][blocks][C] (min, max of the ordinary
 // positions, then of the maxima, then of the minima).  dx is a monotone function of dy on each set (bn_dx), so the
 // finalize kernel knows the exact range of dx from these, before dx is computed.
+// The last kKeepBytes of both tensors are read with loads that leave them in the L2 (the rest passes through, evict-first): the
+// bifurcating pass that follows walks from the end (25.7 M elements of 128 channels with g kept: 74 -> 68 us there, +2 here
+// with 72 MB, nothing with 48; more than the L2 holds beside the writes only costs).
+constexpr int64_t kKeepBytes = 64ll << 20;
 template <int VEC, bool RELU, bool EXT>
 __global__ void __launch_bounds__(kScanThreads) bn_bwd_stats_kernel(const float *__restrict__ dy,
                                                                     const float *__restrict__ x, int64_t rows, int C,
@@ -288,7 +294,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_stats_kernel(const float 
                                                                     const float *__restrict__ beta, float Cn,
                                                                     double *__restrict__ part_dy,
                                                                     double *__restrict__ part_dyx,
-                                                                    float *__restrict__ ext, const ZeroJobs zero)
+                                                                    float *__restrict__ ext, const ZeroJobs zero, int64_t keep_from)
 {
     pdl_enter();
     if (EXT)
@@ -318,14 +324,18 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_stats_kernel(const float 
             b[e] = beta ? beta[p.col + e] : 0.0f;
         }
         const int64_t step = (int64_t)gridDim.x * rpb;
-        for (int64_t r0 = (int64_t)blockIdx.x * rpb + p.ty; r0 < rows; r0 += step * kScanUnroll) {
+        auto pass = [&](auto stream, int64_t &r0, int64_t end) {       // (stream: evict-first loads)
+        for (; r0 < end; r0 += step * kScanUnroll) {
             VecF<VEC> vx[kScanUnroll], vd[kScanUnroll];
             bool ok[kScanUnroll];
 #pragma unroll
             for (int u = 0; u < kScanUnroll; ++u) {
                 int64_t r = r0 + u * step;
                 ok[u] = r < rows;
-                if (ok[u]) { vx[u].load_stream(x + r * C + p.col); vd[u].load_stream(dy + r * C + p.col); }
+                if (ok[u]) {
+                    if (decltype(stream)::value) { vx[u].load_stream(x + r * C + p.col); vd[u].load_stream(dy + r * C + p.col); }
+                    else                         { vx[u].load(x + r * C + p.col); vd[u].load(dy + r * C + p.col); }
+                }
             }
             // (the few rows of one step are added in fp32, the steps in fp64: a quarter of the conversions and fp64
             // additions, and an error of a few ulp of four terms)
@@ -355,6 +365,10 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_stats_kernel(const float 
 #pragma unroll
             for (int e = 0; e < VEC; ++e) { sdy[e] += (double)fs[e]; sdyx[e] += (double)fp[e]; }
         }
+        };
+        int64_t r0 = (int64_t)blockIdx.x * rpb + p.ty;
+        pass(std::true_type{}, r0, keep_from);
+        pass(std::false_type{}, r0, rows);
     }
     __shared__ double s_ab[2 * kScanThreads * VEC];
     double *s_a = s_ab, *s_b = s_ab + kScanThreads * VEC;
@@ -419,8 +433,8 @@ __device__ __forceinline__ void bn_bwd_channel(int c, double sdy, double sdyx, i
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         if (!(ev[2 * k] <= ev[2 * k + 1])) continue;           // (a set with no position keeps +inf, -inf)
-        const float ind = k == 0 ? 0.0f : k == 1 ? 1.0f : -1.0f;
-        const float v0 = bn_dx(ev[2 * k], ind, s, g, m1, k2), v1 = bn_dx(ev[2 * k + 1], ind, s, g, m1, k2);
+        const float t = k == 0 ? 0.0f : k == 1 ? k2 : -k2;
+        const float v0 = bn_dx(ev[2 * k], t, s, g, m1), v1 = bn_dx(ev[2 * k + 1], t, s, g, m1);
         rlo = fminf(rlo, fminf(v0, v1)); rhi = fmaxf(rhi, fmaxf(v0, v1));
     }
     o.chan_range[c] = make_float2(rlo, rhi);
@@ -502,138 +516,199 @@ __global__ void __launch_bounds__(kFinThreads) bn_bwd_finalize_kernel(const doub
 // The Range BN backward apply pass and the bifurcation of the gradient it computes (Sections 3 and 6) in one pass:
 // dx goes from registers into its 8-bit copy (stochastic rounding), the two limbs of its 16-bit copy and each row's
 // 8-bit code sum; the fp32 dx itself is written only when the caller keeps it (g_out).  The parameters of both copies
-// are known beforehand (bn_bwd_finalize_kernel + the range finalize).  Element i of the [rows x C] tensor draws from
+// are known beforehand (from the ranges bn_bwd_finalize_kernel leaves per channel).  Element i of the [rows x C] tensor draws from
 // Philox block i / 4 as in quantize_kernel: a thread's four channels are one block.  rowsum8: a row's lanes
 // of one warp add up by shuffles; when a row spans several warps or blocks (tw > 32 or several slabs) the pieces are added
 // to rowsum8 [rows], zeroed beforehand.
 // TOTALS: also each channel's total of the stored 16-bit codes (256 * hi + lo with lo unsigned, whatever lo_flip) over
 // all rows, added to chansum16 [C] (zeroed beforehand): a thread keeps its four channels for its whole life, a block
 // adds its threads' totals in shared memory and ends with one 64-bit atomic per channel.
-// The pass is bound by arithmetic (Philox), and a thread that computes has no load in flight: the operands come through a
-// ring in shared memory, filled by each thread's own asynchronous copies kBabSlots - 1 steps ahead of the step it
-// computes (a thread reads back only what it copied itself: no barrier), so the memory system always has work.
-constexpr int kBabUnroll = 2;     // rows per thread and step (two operands each)
-constexpr int kBabSlots = 3;      // ring depth in steps
-constexpr size_t kBabRingBytes = (size_t)kBabSlots * kBabUnroll * 2 * kScanThreads * sizeof(float4);
-template <bool RELU, bool STORE_G, bool TOTALS>
-__global__ void __launch_bounds__(kScanThreads, 3) bn_bwd_apply_bifurcate_kernel(
-    const float *__restrict__ dy, const float *__restrict__ x, int64_t rows, int C, int tw, const float *__restrict__ mean,
-    const float *__restrict__ vmin, const float *__restrict__ vmax, const float *__restrict__ gamma,
-    const float *__restrict__ beta, float Cn, const float2 *__restrict__ coef, float *__restrict__ g_out,
-    const RangeSrc range, uint32_t id8, uint32_t id16,
-    const __grid_constant__ PhiloxKeys keys, uint32_t *__restrict__ q8, uint32_t *__restrict__ q_hi, uint32_t *__restrict__ q_lo,
-    uint32_t lo_flip, int32_t *__restrict__ rowsum8, unsigned long long *__restrict__ chansum16,
-    const float2 *__restrict__ relu_thr)
+// The operands come through a ring in shared memory, filled by each thread's own asynchronous copies one tile ahead of the one
+// it computes (a thread reads back only what it copied itself: no barrier), so the memory system always has work.
+// What bounds it: the integer pipes (about 25 instructions per element in Philox and the two roundings alone).  So the rest is
+// kept small: 32-bit indices, no check per row in the whole tiles, the rare terms of the extremes on a path outside the
+// straight line (one branch per tile of four rows, after which all of them are quantised together), the channels' constants
+// read from shared memory once per tile.  Two rows per tile and 69 instructions per element before: 51.4 M elements of 64
+// channels 131 -> 109 us (without Philox at all: 109), 102.8 M of 512 channels 277 -> 209 us (5.5 TB/s), 12.8 M of 256
+// channels 43 -> 35 us.  Not better: four blocks of 64 registers (113, spills with four rows), two of 105 (109), a third slot.
+constexpr int kBabRows = 4;       // rows per thread and tile (an even number)
+constexpr int kBabSlots = 2;      // ring depth in tiles
+constexpr int kBabBlocks = 3;     // blocks per SM (at most 80 registers a thread)
+constexpr size_t kBabRingBytes = (size_t)kBabSlots * 2 * kBabRows * kScanThreads * sizeof(float4);
+// ONE: both copies have one tensor id and share their Philox blocks.
+template <bool RELU, bool STORE_G, bool TOTALS, bool ONE>
+__global__ void __launch_bounds__(kScanThreads, kBabBlocks) bn_bwd_apply_bifurcate_kernel(
+    const float4 *__restrict__ dy, const float4 *__restrict__ x, uint32_t rows, int C, int tw, const float *__restrict__ vmin,
+    const float *__restrict__ vmax, const float *__restrict__ gamma, float Cn, const float2 *__restrict__ coef,
+    float4 *__restrict__ g_out, const RangeSrc range, uint32_t id8, uint32_t id16, const __grid_constant__ PhiloxKeys keys,
+    uint32_t *__restrict__ q8, uint32_t *__restrict__ q_hi, uint32_t *__restrict__ q_lo, uint32_t lo_flip,
+    int32_t *__restrict__ rowsum8, unsigned long long *__restrict__ chansum16, const float2 *__restrict__ relu_thr)
 {
     pdl_enter();
-    const bool rowsum_pieces = tw > 32 || gridDim.y > 1;
     const ScanPos p = scan_pos<4>(C, tw);
-    uint32_t cs16[4] = {0u, 0u, 0u, 0u};          // unsigned codes of this thread's rows (fewer than 65536 rows)
-    int mine = 0;
-    const int rpb = kScanThreads / tw;
-    float s[4], g[4], lo[4], hi[4], m1[4], k2[4], thr[4], tsg[4];
+    int cs16[4] = {0, 0, 0, 0};                   // stored codes of this thread's rows (fewer than 65536 rows)
+    // the channels' constants in shared memory, read again for every step: held in registers (28 of them) they would cost the
+    // fourth block of an SM
+    __shared__ float4 s_const[7][kScanMaxTw];     // scale, gamma, centre, half of the range, m1, the mask's threshold and sign
+    if ((int)threadIdx.x < tw) {
+        float k[7][4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const int c = p.active ? p.col + e : 0;
-        lo[e] = vmin[c]; hi[e] = vmax[c];
-        s[e] = bn_scale(lo[e], hi[e], Cn);
-        g[e] = gamma ? gamma[c] : 1.0f;
-        const float2 cf = coef[c];
-        m1[e] = cf.x; k2[e] = cf.y;
-        const float2 th = RELU ? relu_thr[c] : make_float2(0.0f, 1.0f);   // (the mask y > 0 as sgn * x >= threshold)
-        thr[e] = th.x; tsg[e] = th.y;
+        for (int e = 0; e < 4; ++e) {
+            const int c = p.active ? p.col + e : 0;
+            const float2 th = RELU ? relu_thr[c] : make_float2(0.0f, 1.0f);   // (the mask y > 0 as sgn * x >= threshold)
+            const float lo = vmin[c], hi = vmax[c];
+            k[0][e] = bn_scale(lo, hi, Cn);
+            // |x - centre| >= half holds for the extremes (both sides rounded alike) and for hardly anything else
+            k[2][e] = 0.5f * lo + 0.5f * hi;
+            k[3][e] = fminf(__fsub_rn(hi, k[2][e]), __fsub_rn(k[2][e], lo));
+            k[1][e] = gamma ? gamma[c] : 1.0f;
+            k[4][e] = coef[c].x; k[5][e] = th.x; k[6][e] = th.y;
+        }
+#pragma unroll
+        for (int i = 0; i < 7; ++i) s_const[i][p.tx] = make_float4(k[i][0], k[i][1], k[i][2], k[i][3]);
     }
+    __syncthreads();
     // both codes in fixed point with 16 fraction bits (quantize_sr8_byte2 / quantize_sr16_top_half)
     QParamsReg q8r, q16r;
     resolve_range(range, true, true, blockIdx.x == 0 && blockIdx.y == 0, q8r, q16r);
     const float inv8 = q8r.inv * 65536.0f, zp8 = q8r.zp_u * 65536.0f, inv16 = q16r.inv * 65536.0f, zp16 = q16r.zp_u * 65536.0f;
-    const bool one_block = id8 == id16;
-    const int64_t step = (int64_t)gridDim.x * rpb;
-    // (the loop bound is the block's: every lane takes part in the row-sum shuffles)
-    extern __shared__ __align__(16) float4 bab_ring[];         // [slot][row of the step][x | dy][thread]
-    float4 *const mine_ring = bab_ring + threadIdx.x;
-    const int64_t stride = step * kBabUnroll;
-    auto fetch = [&](int64_t base, int slot) {
+
+    // The gradients of a tile's rows without the terms of the maxima and minima; whether one of those may be among them.
+    auto dx = [&](const float4 *src, float (&v)[kBabRows][4]) {
+        float s[4], g[4], mid[4], half[4], m1[4], thr[4], tsg[4];
+        auto get = [&](int i, float (&k)[4]) { const float4 c = s_const[i][p.tx]; k[0] = c.x; k[1] = c.y; k[2] = c.z; k[3] = c.w; };
+        get(0, s); get(1, g); get(2, mid); get(3, half); get(4, m1);
+        if (RELU) { get(5, thr); get(6, tsg); }
+        bool edge = false;
 #pragma unroll
-        for (int u = 0; u < kBabUnroll; ++u) {
-            const int64_t r = base + p.ty + u * step;
-            if (p.active && r < rows) {
-                cp_async16(mine_ring + ((slot * kBabUnroll + u) * 2 + 0) * kScanThreads, x + r * C + p.col);
-                cp_async16(mine_ring + ((slot * kBabUnroll + u) * 2 + 1) * kScanThreads, dy + r * C + p.col);
+        for (int u = 0; u < kBabRows; ++u) {
+            const float4 fx = src[2 * u * kScanThreads], fd = src[(2 * u + 1) * kScanThreads];
+            const float ax[4] = {fx.x, fx.y, fx.z, fx.w}, ad[4] = {fd.x, fd.y, fd.z, fd.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float d = RELU && !(__fmul_rn(tsg[e], ax[e]) >= thr[e]) ? 0.0f : ad[e];
+                v[u][e] = bn_dx(d, 0.0f, s[e], g[e], m1[e]);
+                edge |= fabsf(__fsub_rn(ax[e], mid[e])) >= half[e];
             }
         }
-        cp_async_commit();                                     // (a group per step, empty past the end: the count below is uniform)
+        return edge;
+    };
+    // ... of one float4, with them.
+    auto dx_edge = [&](const float4 &fx, const float4 &fd, float (&v)[4]) {
+        const float ax[4] = {fx.x, fx.y, fx.z, fx.w}, ad[4] = {fd.x, fd.y, fd.z, fd.w};
+        const float *const k = reinterpret_cast<const float *>(&s_const[0][p.tx]);
+        constexpr int kRow = 4 * kScanMaxTw;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int c = p.active ? p.col + e : 0;
+            const float d = RELU && !(__fmul_rn(k[6 * kRow + e], ax[e]) >= k[5 * kRow + e]) ? 0.0f : ad[e];
+            v[e] = bn_dx(d, bn_k2_ind(ax[e], vmin[c], vmax[c], coef[c].y), k[e], k[kRow + e], k[4 * kRow + e]);
+        }
+    };
+    // The codes and stores of one float4; returns the sum of its 8-bit codes.  store: false for a thread beyond the columns.
+    auto codes = [&](const float (&v)[4], uint32_t j, bool store) {
+        // the thread's Philox block = its float4's index
+        const uint4 r8 = philox4x32_10(make_uint4(j, 0u, id8, 0u), keys);
+        const uint4 r16 = ONE ? r8 : philox4x32_10(make_uint4(j, 0u, id16, 0u), keys);
+        uint32_t c16[4];
+        const BifWords w = bifurcate4(v, inv8, zp8, inv16, zp16, r8, r16, lo_flip, c16);
+        if (store) {
+            if (STORE_G) __stcs(g_out + j, make_float4(v[0], v[1], v[2], v[3]));
+            q8[j] = w.q8; q_hi[j] = w.hi; q_lo[j] = w.lo;
+        }
+        if (TOTALS) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) cs16[e] += (int)c16[e] >> 16;
+        }
+        return store ? __dp4a((int)w.q8, 0x01010101, 0) : 0;
+    };
+    // A row's code sum of a step's rows.  Two of them ride in one word: at most 32 lanes of a warp share a row, four codes each,
+    // offset by 512 per lane.  Lane 0 of the row stores the first row's sum, lane 1 the second's (a single lane, both); of a row
+    // wider than the warp, or than the block, each piece is added to the zeroed sum.
+    const int lanes = tw < 32 ? tw : 32, lane = p.tx & (lanes - 1);
+    const bool rowsum_pieces = tw > 32 || gridDim.y > 1;
+    auto row_sums = [&](int rs0, int rs1, uint32_t r0, uint32_t r1, bool ok0, bool ok1) {
+        uint32_t two = (uint32_t)(rs0 + 512) + ((uint32_t)(rs1 + 512) << 16);
+        if (lanes == 32) two = __reduce_add_sync(0xffffffffu, two);
+        else
+#pragma unroll
+            for (int off = 8; off > 0; off >>= 1)
+                if (off < lanes) two += __shfl_xor_sync(0xffffffffu, two, off);
+        if (lane < 2 && (lane ? ok1 : ok0)) {
+            const int sum = (int)((lane ? two >> 16 : two & 0xFFFFu)) - 512 * lanes;
+            int32_t *const dst = rowsum8 + (lane ? r1 : r0);
+            if (rowsum_pieces) atomicAdd(dst, sum); else *dst = sum;
+            if (lanes == 1 && ok1) rowsum8[r1] = (int)(two >> 16) - 512;
+        }
+    };
+    // A block takes tiles of kBabRows * rpb rows; rows and float4 indices in 32 bits (fewer than 2^32 of either).
+    const uint32_t rpb = kScanThreads / tw, cv = (uint32_t)C >> 2, tile = kBabRows * rpb, jrow = rpb * cv;
+    const uint32_t tiles = rows / tile;                        // whole ones; the rows that are left over come last
+    const uint32_t mine = blockIdx.x < tiles ? (tiles - blockIdx.x - 1) / gridDim.x + 1 : 0;
+    const uint32_t jt = gridDim.x * tile * cv;
+    // (from the last tile to the first: the statistics' pass, just before, left the end of both tensors in the L2)
+    uint32_t r = (tiles - 1 - blockIdx.x) * tile + p.ty, j = r * cv + (uint32_t)((p.active ? p.col : 0) >> 2);
+    extern __shared__ __align__(16) float4 bab_ring[];         // [slot][row][x | dy][thread]
+    float4 *const mine_ring = bab_ring + threadIdx.x;
+    auto fetch = [&](uint32_t jf, int slot) {
+        float4 *const dst = mine_ring + slot * (2 * kBabRows * kScanThreads);
+#pragma unroll
+        for (int u = 0; u < kBabRows; ++u) {
+            cp_async16(dst + (2 * u) * kScanThreads, x + (jf + u * jrow));
+            cp_async16(dst + (2 * u + 1) * kScanThreads, dy + (jf + u * jrow));
+        }
     };
 #pragma unroll
-    for (int k = 0; k < kBabSlots - 1; ++k) fetch((int64_t)blockIdx.x * rpb + k * stride, k);
+    for (uint32_t k = 0; k < kBabSlots - 1; ++k) {
+        if (k < mine) fetch(j - k * jt, (int)k);
+        cp_async_commit();                                     // (a group per tile, empty past the end: the count below is uniform)
+    }
     int slot = 0;
-    for (int64_t base = (int64_t)blockIdx.x * rpb; base < rows; base += stride) {
-        const int64_t r0 = base + p.ty;
-        // the slot this thread emptied in the step before takes the step kBabSlots - 1 ahead; then this step's data is in
-        fetch(base + (kBabSlots - 1) * stride, slot == 0 ? kBabSlots - 1 : slot - 1);
+    for (uint32_t t = 0; t < mine; ++t) {
+        // the slot this thread emptied in the step before takes the tile kBabSlots - 1 ahead; then this step's data is in
+        if (t + (kBabSlots - 1) < mine) fetch(j - (kBabSlots - 1) * jt, slot == 0 ? kBabSlots - 1 : slot - 1);
+        cp_async_commit();
         cp_async_wait<kBabSlots - 1>();
+        const float4 *const src = mine_ring + slot * (2 * kBabRows * kScanThreads);
+        float v[kBabRows][4];
+        if (dx(src, v)) {                                      // (few: two positions per channel, or ties)
 #pragma unroll
-        for (int u = 0; u < kBabUnroll; ++u) {
-            const int64_t r = r0 + u * step;
-            const bool ok_u = p.active && r < rows;
-            int rs = 0;
-            if (ok_u) {
-                const float4 fx = mine_ring[((slot * kBabUnroll + u) * 2 + 0) * kScanThreads];
-                const float4 fd = mine_ring[((slot * kBabUnroll + u) * 2 + 1) * kScanThreads];
-                const float ax[4] = {fx.x, fx.y, fx.z, fx.w}, ad[4] = {fd.x, fd.y, fd.z, fd.w};
-                float v[4];
+            for (int u = 0; u < kBabRows; ++u) dx_edge(src[2 * u * kScanThreads], src[(2 * u + 1) * kScanThreads], v[u]);
+        }
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float xv = ax[e];
-                    float d = ad[e];
-                    if (RELU && !(__fmul_rn(tsg[e], xv) >= thr[e])) d = 0.0f;
-                    const float ind = (xv == hi[e] ? 1.0f : 0.0f) - (xv == lo[e] ? 1.0f : 0.0f);
-                    v[e] = bn_dx(d, ind, s[e], g[e], m1[e], k2[e]);
-                }
-                const int64_t j = (r * C + p.col) >> 2;                 // the thread's Philox block = its float4's index
-                if (STORE_G) __stcs(reinterpret_cast<float4 *>(g_out) + j, make_float4(v[0], v[1], v[2], v[3]));
-                const uint4 r8 = philox4x32_10(make_uint4((uint32_t)j, (uint32_t)((uint64_t)j >> 32), id8, 0u), keys);
-                const uint4 r16 = one_block ? r8 : philox4x32_10(make_uint4((uint32_t)j, (uint32_t)((uint64_t)j >> 32), id16, 0u), keys);
-                const uint32_t w8[4] = {r8.x, r8.y, r8.z, r8.w}, w16[4] = {r16.x, r16.y, r16.z, r16.w};
-                uint32_t c8[4], c16[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    c8[e] = quantize_sr8_byte2(v[e], inv8, zp8, w8[e]);
-                    c16[e] = quantize_sr16_top_half(v[e], inv16, zp16, w16[e]);
-                }
-                // the 8-bit codes are byte 2 of each word; the 16-bit codes bytes 3 (high) and 2 (low)
-                const uint32_t packed = __byte_perm(__byte_perm(c8[0], c8[1], 0x0062), __byte_perm(c8[2], c8[3], 0x0062), 0x5410) ^ 0x80808080u;
-                q8[j] = packed;
-                const uint32_t t01 = __byte_perm(c16[0], c16[1], 0x7362), t23 = __byte_perm(c16[2], c16[3], 0x7362);
-                q_hi[j] = __byte_perm(t01, t23, 0x7632) ^ 0x80808080u;
-                q_lo[j] = __byte_perm(t01, t23, 0x5410) ^ lo_flip;
-                rs = __dp4a((int)packed, 0x01010101, 0);
-                if (TOTALS) {
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) cs16[e] += c16[e] >> 16;
-                    ++mine;
-                }
-            }
-            if (rowsum8) {
-                for (int off = 16; off > 0; off >>= 1)
-                    if (off < tw) rs += __shfl_xor_sync(0xffffffffu, rs, off);
-                // (a row wider than a warp's lanes, or than the block: each piece is added to the zeroed sum)
-                if (ok_u && (p.tx & 31) == 0) {
-                    if (rowsum_pieces) atomicAdd(rowsum8 + r, rs);
-                    else rowsum8[r] = rs;
-                }
-            }
+        for (int u = 0; u < kBabRows; u += 2) {
+            const int rs0 = codes(v[u], j + u * jrow, p.active), rs1 = codes(v[u + 1], j + (u + 1) * jrow, p.active);
+            if (rowsum8) row_sums(rs0, rs1, r + u * rpb, r + (u + 1) * rpb, true, true);
         }
         slot = slot + 1 == kBabSlots ? 0 : slot + 1;
+        j -= jt; r -= gridDim.x * tile;
     }
-    cp_async_wait<0>();
+    // the rows left over (fewer than a tile): the last block's
+    if (blockIdx.x == gridDim.x - 1 && tiles * tile < rows) {
+        const uint32_t rl = tiles * tile + p.ty;
+#pragma unroll 1
+        for (int u = 0; u < kBabRows; u += 2) {
+            int rs[2] = {0, 0};
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t ru = rl + (u + h) * rpb;
+                if (!(p.active && ru < rows)) continue;
+                const uint32_t ju = ru * cv + (uint32_t)(p.col >> 2);
+                float v[4];
+                dx_edge(x[ju], dy[ju], v);
+                rs[h] = codes(v, ju, true);
+            }
+            if (rowsum8) row_sums(rs[0], rs[1], rl + u * rpb, rl + (u + 1) * rpb, rl + u * rpb < rows, rl + (u + 1) * rpb < rows);
+        }
+    }
     if (TOTALS) {
-        __shared__ int s_tot[kScanMaxTw * 4];
+        int *const s_tot = reinterpret_cast<int *>(s_const);     // (the constants' room)
+        __syncthreads();
         for (int i = threadIdx.x; i < tw * 4; i += kScanThreads) s_tot[i] = 0;
         __syncthreads();
-        if (p.active && mine) {
+        if (p.active) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) atomicAdd(&s_tot[p.tx * 4 + e], (int)((long long)cs16[e] - (long long)mine * 32768));
+            for (int e = 0; e < 4; ++e) atomicAdd(&s_tot[p.tx * 4 + e], cs16[e]);
         }
         __syncthreads();
         for (int i = threadIdx.x; i < tw * 4; i += kScanThreads) {
@@ -706,8 +781,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_apply_kernel(const float 
                     const float xv = vx[u].v[e];
                     float d = vd[u].v[e];
                     if (RELU && !(bn_y(bn_xhat(xv, mu[e], s[e]), g[e], b[e]) > 0.0f)) d = 0.0f;
-                    const float ind = (xv == hi[e] ? 1.0f : 0.0f) - (xv == lo[e] ? 1.0f : 0.0f);
-                    vd[u].v[e] = bn_dx(d, ind, s[e], g[e], m1[e], k2[e]);
+                    vd[u].v[e] = bn_dx(d, bn_k2_ind(xv, lo[e], hi[e], k2[e]), s[e], g[e], m1[e]);
                     if (RANGE) { rlo = fminf(rlo, vd[u].v[e]); rhi = fmaxf(rhi, vd[u].v[e]); }
                 }
                 vd[u].store(dx + (r0 + u * step) * C + p.col);
@@ -1155,8 +1229,9 @@ static int bn_bwd_stats_launch(const float *dy, const float *x, int64_t n_rows, 
     const dim3 grid(g.nbx, g.slabs);
     const double Cnd = 1.0 / std::sqrt(2.0 * std::log((double)n_stat));
     const float Cn = (float)Cnd;
+    const int64_t keep_from = std::max<int64_t>(0, n_rows - kKeepBytes / (2 * (int64_t)sizeof(float) * C));
     QBP_TRACE_BEGIN(st);
-#define QBP_BN_BSTATS(V, R, E) launch(bn_bwd_stats_kernel<V, R, E>, grid, kScanThreads, 0, st, dy, x, n_rows, (int)C, g.tw, save_mean, save_min, save_max, gamma, beta, Cn, pa, pb, ext, zero)
+#define QBP_BN_BSTATS(V, R, E) launch(bn_bwd_stats_kernel<V, R, E>, grid, kScanThreads, 0, st, dy, x, n_rows, (int)C, g.tw, save_mean, save_min, save_max, gamma, beta, Cn, pa, pb, ext, zero, keep_from)
     if (ext) {
         if (g.vec != 4) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "rangebn_bwd: the pass with dy extremes needs aligned tensors and C a multiple of 4");
         if (relu) QBP_BN_BSTATS(4, true, true); else QBP_BN_BSTATS(4, false, true);
@@ -1207,7 +1282,7 @@ bool rangebn_bwd_one_launch(int64_t n, int64_t C) { return few_rows(n, C); }
 // Whether rangebn_bwd_bifurcate_impl takes a tensor of C channels (row_sums: each row's 8-bit code sum is wanted).
 bool rangebn_bwd_bifurcate_supported(const float *dy, const float *x, const float *g_out, int64_t n, int64_t C, bool row_sums)
 {
-    if (!aligned16(x) || !aligned16(dy) || (g_out && !aligned16(g_out)) || C % 4 || n < 2 || n * C >= (1ll << 40)) return false;
+    if (!aligned16(x) || !aligned16(dy) || (g_out && !aligned16(g_out)) || C % 4 || n < 2 || n * C >= (1ll << 34)) return false;      // (Philox blocks below 2^32; more does not fit the device)
     (void)row_sums;      // (any row width: rows wider than a warp's lanes are added up from their pieces)
     return true;
 }
@@ -1236,8 +1311,8 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
     float *ext = w.take<float>(6 * (size_t)kScanMaxStrips * C);
     float2 *chan_range = w.take<float2>((size_t)C);
     float2 *relu_thr = w.take<float2>((size_t)C);
-    // (three resident blocks per SM by the kernel's launch bounds, whatever the instance)
-    const ScanGeom ga = scan_geom(n, C, true, blocks_per_sm<bn_bwd_apply_bifurcate_kernel<true, true, true>>(kScanThreads));
+    // (kBabBlocks resident blocks per SM by the kernel's launch bounds, whatever the instance)
+    const ScanGeom ga = scan_geom(n, C, true, blocks_per_sm<bn_bwd_apply_bifurcate_kernel<true, true, true, true>>(kScanThreads));
     // each row's code sum by shuffles over the row's lanes of a warp; a row that spans several warps or blocks is
     // added up from its pieces (integer atomics on the zeroed sums: the result does not depend on the order)
     ZeroJobs zero{};
@@ -1256,11 +1331,13 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
     const PhiloxKeys keys = philox_keys_host(seed);
     const uint32_t flip = lo_signed ? 0x80808080u : 0u;
     QBP_TRACE_BEGIN(st);
-#define QBP_BN_BAB(R, G, T) do { static PerDeviceOnce once_; QBP_SMEM_OPT_IN(once_, (bn_bwd_apply_bifurcate_kernel<R, G, T>), kBabRingBytes); launch(bn_bwd_apply_bifurcate_kernel<R, G, T>, grid, kScanThreads, kBabRingBytes, st, dy, x, n, (int)C, ga.tw, save_mean, save_min, save_max, gamma, beta, Cn, coef, g_out, range, id8, id16, keys, reinterpret_cast<uint32_t *>(q8), reinterpret_cast<uint32_t *>(hi), reinterpret_cast<uint32_t *>(lo), flip, row_sums8, reinterpret_cast<unsigned long long *>(tot16), relu_thr); } while (0)
-#define QBP_BN_BAB2(R, G) do { if (tot16) QBP_BN_BAB(R, G, true); else QBP_BN_BAB(R, G, false); } while (0)
+#define QBP_BN_BAB(R, G, T, O) do { static PerDeviceOnce once_; QBP_SMEM_OPT_IN(once_, (bn_bwd_apply_bifurcate_kernel<R, G, T, O>), kBabRingBytes); launch(bn_bwd_apply_bifurcate_kernel<R, G, T, O>, grid, kScanThreads, kBabRingBytes, st, reinterpret_cast<const float4 *>(dy), reinterpret_cast<const float4 *>(x), (uint32_t)n, (int)C, ga.tw, save_min, save_max, gamma, Cn, coef, reinterpret_cast<float4 *>(g_out), range, id8, id16, keys, reinterpret_cast<uint32_t *>(q8), reinterpret_cast<uint32_t *>(hi), reinterpret_cast<uint32_t *>(lo), flip, row_sums8, reinterpret_cast<unsigned long long *>(tot16), relu_thr); } while (0)
+#define QBP_BN_BAB1(R, G, T) do { if (id8 == id16) QBP_BN_BAB(R, G, T, true); else QBP_BN_BAB(R, G, T, false); } while (0)
+#define QBP_BN_BAB2(R, G) do { if (tot16) QBP_BN_BAB1(R, G, true); else QBP_BN_BAB1(R, G, false); } while (0)
     if (g_out) { if (relu) QBP_BN_BAB2(true, true); else QBP_BN_BAB2(false, true); }
     else       { if (relu) QBP_BN_BAB2(true, false); else QBP_BN_BAB2(false, false); }
 #undef QBP_BN_BAB2
+#undef QBP_BN_BAB1
 #undef QBP_BN_BAB
     QBP_LAUNCH_OK("bn_bwd_apply_bifurcate_kernel");
     return QBP_OK;

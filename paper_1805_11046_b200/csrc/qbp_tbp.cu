@@ -54,7 +54,8 @@ __device__ __forceinline__ int tern_keep(uint32_t word, float s, float a)
 // int8 (q), and / or as the two byte limbs of the same value as a 16-bit code (hi: 0 or -1, lo: the low byte), which
 // is what the weight-gradient product takes.  parts: the range scan's (min, max) pairs (s = max(-vmin, vmax)); *qp_out receives
 // scale = s / samples, zero-point 0, so that scale * code estimates g.
-template <int VEC>
+// J32: every Philox block index is below 2^32 (what the first two rounds have in common for all samples is then taken once).
+template <int VEC, bool J32>
 __global__ void __launch_bounds__(kTbpThreads) stc_ternarize_kernel(const float *__restrict__ g, int64_t n,
                                                                     const float2 *__restrict__ parts, int nparts, int samples,
                                                                     uint32_t tensor_id, const __grid_constant__ PhiloxKeys keys,
@@ -80,7 +81,7 @@ __global__ void __launch_bounds__(kTbpThreads) stc_ternarize_kernel(const float 
 #pragma unroll
             for (int e = 0; e < 4; ++e) p[e] = fabsf(xs[e]);
             for (int k = 0; k < samples; ++k) {
-                const uint4 b = philox4x32_10(make_uint4((uint32_t)j, (uint32_t)((uint64_t)j >> 32), tensor_id, (uint32_t)k), keys);
+                const uint4 b = philox4x32_10(make_uint4((uint32_t)j, J32 ? 0u : (uint32_t)((uint64_t)j >> 32), tensor_id, (uint32_t)k), keys);
                 cnt[0] += tern_keep(b.x, s, p[0]); cnt[1] += tern_keep(b.y, s, p[1]);
                 cnt[2] += tern_keep(b.z, s, p[2]); cnt[3] += tern_keep(b.w, s, p[3]);
             }
@@ -132,8 +133,10 @@ static int stc_ternarize_impl(const float *g, int64_t n, int samples, uint64_t s
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((items + kTbpThreads - 1) / kTbpThreads, (int64_t)sm_count() * 8));
     const PhiloxKeys keys = philox_keys_host(seed);
     QBP_TRACE_BEGIN(st);
-    if (vec) launch(stc_ternarize_kernel<4>, grid, kTbpThreads, 0, st, g, n, static_cast<const float2 *>(ws), nparts, samples, tensor_id, keys, q, hi, lo, qp_out);
-    else     launch(stc_ternarize_kernel<1>, grid, kTbpThreads, 0, st, g, n, static_cast<const float2 *>(ws), nparts, samples, tensor_id, keys, q, hi, lo, qp_out);
+    const bool j32 = n < (1ll << 34);
+    if (vec && j32) launch(stc_ternarize_kernel<4, true>, grid, kTbpThreads, 0, st, g, n, static_cast<const float2 *>(ws), nparts, samples, tensor_id, keys, q, hi, lo, qp_out);
+    else if (vec) launch(stc_ternarize_kernel<4, false>, grid, kTbpThreads, 0, st, g, n, static_cast<const float2 *>(ws), nparts, samples, tensor_id, keys, q, hi, lo, qp_out);
+    else     launch(stc_ternarize_kernel<1, false>, grid, kTbpThreads, 0, st, g, n, static_cast<const float2 *>(ws), nparts, samples, tensor_id, keys, q, hi, lo, qp_out);
     QBP_LAUNCH_OK("stc_ternarize_kernel");
     return QBP_OK;
 }

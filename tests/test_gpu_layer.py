@@ -485,3 +485,20 @@ def test_linear_layers_of_other_shapes_stagewise(B, batch, cin, cout):
     cfg = dict(x=synth.normal((batch, cin), 95), w=synth.kaiming_uniform_linear(cin, cout, 96), dy=synth.normal((batch, cout), 97, std=0.1),
                seed=3, id8=5, id16=5)
     _check_layer(B, cfg, True)
+
+
+@pytest.mark.parametrize("id16", [5, 6])
+@pytest.mark.parametrize("batch,cin,cout", [(32, 16, 16), (256, 16, 16), (272, 32, 16), (400, 64, 48), (48, 16, 528), (2080, 32, 64)])
+def test_backward_where_many_elements_are_extremes(B, batch, cin, cout, id16):
+    """The bifurcating Range BN backward adds the terms of a channel's extremes on a path of its own: a constant channel, and
+    channels that take two values only (every element an extreme), next to ordinary ones.  Fewer rows than a block's tile, whole
+    tiles and remainders; rows of a part of a warp, of several warps and of several slabs."""
+    x = (synth.normal((batch, cin), 71) > 0).astype(np.float32)
+    x[0, :] = 1.0
+    x[1, :] = 0.0
+    w = synth.kaiming_uniform_linear(cin, cout, 72)
+    w[:, 0] = 0.0
+    for c in (1, 2, 5, cout - 1):
+        w[:, c] = 0.0
+        w[c % cin, c] = 0.3
+    _check_layer(B, dict(x=x, w=w, dy=synth.normal((batch, cout), 73, std=0.1), seed=4, id8=5, id16=id16), True)

@@ -126,6 +126,19 @@ def test_bifurcate_and_code_sums(B):
     assert np.array_equal(to_host(cols), on.q.astype(np.int64).sum(0))
 
 
+@pytest.mark.parametrize("id8,id16", [(3, 3), (3, 4)])
+@pytest.mark.parametrize("n", [1, 3, 4, 1023, 4092, 4096, 4099, 8192 + 1028, 592 * 4096 * 2 + 4100])
+def test_bifurcate_at_the_edges_of_a_blocks_share(B, n, id8, id16):
+    """Tensors shorter than a block's step of 4096 elements, whole steps, remainders of vectors and of single elements, and
+    more steps than resident blocks; one Philox block for both copies (equal ids) or one each."""
+    g = synth.normal((1, n), 17, std=0.2)
+    q8, qp8, hi, lo, qp16 = B.qbp_bifurcate(to_dev(g), 5, id8, id16)
+    o8, o16 = O.bifurcate(g, 5, id8, id16)
+    _same_params(B, qp8, o8); _same_params(B, qp16, o16)
+    ohi, olo = O.limb_split(o16.q)
+    assert np.array_equal(to_host(q8), o8.q) and np.array_equal(to_host(hi), ohi) and np.array_equal(to_host(lo), olo)
+
+
 @pytest.mark.parametrize("rows,cols", [(130, 128), (77, 256), (300, 512), (33, 2048), (9, 96), (5, 4096)])
 def test_row_sums_of_rows_of_any_width(B, rows, cols):
     """Row sums taken inside the quantising kernel (power-of-two rows up to 128 elements) or by the pass over the codes
