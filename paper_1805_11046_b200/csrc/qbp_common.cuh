@@ -261,24 +261,31 @@ __device__ __forceinline__ float order_float(int i) { return __int_as_float(i ^ 
 __device__ __forceinline__ float bn_scale(float lo, float hi, float Cn);
 // The rectifier's mask of a Range BN output as a threshold on the input.  y(x) = bn_y(bn_xhat(x, mu, s), g, b) is a
 // monotone function of x (every operation is rounded on its own and monotone, s >= 0): rising for g >= 0, falling for
-// g < 0, so {x : y(x) > 0} is a ray, and its end is found by bisection over the floats in their order (33 evaluations
-// of y).  Returns (t, sgn) with  y(x) > 0  <=>  sgn * x >= t  for finite x (sgn = +-1; t = +-inf: none / all).
+// g < 0, so {x : y(x) > 0} is a ray, and its end is found by a search over the floats in their order.  Returns (t, sgn) with  y(x) > 0  <=>  sgn * x >= t  for finite x (sgn = +-1; t = +-inf: none / all).
 __device__ inline float2 relu_threshold(float mu, float s, float g, float b)
 {
     const bool rising = !(g < 0.0f);
-    long long lo = float_order(-3.402823466e38f), hi = float_order(3.402823466e38f);
-    auto on = [&](long long k) { return bn_y(bn_xhat(order_float((int)k), mu, s), g, b) > 0.0f; };
     const float sgn = rising ? 1.0f : -1.0f;
-    // (towards `far` the output rises: the ray is [threshold, far])
-    const bool at_far = on(rising ? hi : lo), at_near = on(rising ? lo : hi);
-    if (!at_far) return make_float2(INFINITY, sgn);
-    if (at_near) return make_float2(-INFINITY, sgn);
-    if (rising) {                       // smallest key that is on
-        while (hi - lo > 1) { const long long mid = lo + (hi - lo) / 2; if (on(mid)) hi = mid; else lo = mid; }
-        return make_float2(order_float((int)hi), 1.0f);
+    // (the keys of x, or of -x when the output falls: the output then rises with the key; the key of -x is -1 - key)
+    auto on = [&](long long k) { return bn_y(bn_xhat(order_float(rising ? (int)k : -1 - (int)k), mu, s), g, b) > 0.0f; };
+    long long lo = float_order(-3.402823466e38f), hi = float_order(3.402823466e38f);
+    if (!on(hi)) return make_float2(INFINITY, sgn);
+    if (on(lo)) return make_float2(-INFINITY, sgn);
+    // Outwards from where the output is zero in real numbers, in growing steps, then between the last two: a few evaluations
+    // (beta = 0: one) where halving the whole range takes 32, 3 us at the end of every backward statistics' pass.
+    const float x0 = sgn * __fsub_rn(mu, __fdiv_rn(b, __fmul_rn(g, s)));
+    if (fabsf(x0) < 3.0e38f) {
+        const long long k0 = float_order(x0);
+        if (on(k0)) {
+            hi = k0;
+            for (long long step = 1; hi - step > lo; step *= 8) { if (on(hi - step)) hi -= step; else { lo = hi - step; break; } }
+        } else {
+            lo = k0;
+            for (long long step = 1; lo + step < hi; step *= 8) { if (on(lo + step)) { hi = lo + step; break; } lo += step; }
+        }
     }
-    while (hi - lo > 1) { const long long mid = lo + (hi - lo) / 2; if (on(mid)) lo = mid; else hi = mid; }   // largest key that is on
-    return make_float2(-order_float((int)lo), -1.0f);
+    while (hi - lo > 1) { const long long mid = lo + (hi - lo) / 2; if (on(mid)) hi = mid; else lo = mid; }       // smallest key that is on
+    return make_float2(order_float((int)hi), sgn);
 }
 __device__ __forceinline__ float bn_scale(float lo, float hi, float Cn)
 {

@@ -464,24 +464,32 @@ __global__ void __launch_bounds__(kFinThreads) bn_bwd_finalize_kernel(const doub
     // (the blocks behind the channels take code sums that a later product needs: C short blocks leave most SMs idle)
     if (c >= C) { code_sums_block(J, c - C); return; }
     double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += kFinThreads) {
-        const double pa_ = part_dy[(int64_t)i * C + c], pb_ = part_dyx[(int64_t)i * C + c];
-        a += pa_; b += pb_;
-    }
     // ext (see bn_bwd_stats_kernel): the extremes of dy over the three sets of positions, then (below) the exact range
     // of this channel's dx, left in chan_range[c] for the quantiser of the gradient
     float ev[6];
     __shared__ float s_e[6][kFinThreads / 32];
-    if (ext) {
 #pragma unroll
-        for (int k = 0; k < 6; ++k) ev[k] = (k & 1) ? -INFINITY : INFINITY;
-        for (int i = threadIdx.x; i < nparts; i += kFinThreads) {
-            float o[6];
+    for (int k = 0; k < 6; ++k) ev[k] = (k & 1) ? -INFINITY : INFINITY;
+    // (all loads of two partials at once: the whole table in one round trip for up to two blocks per SM)
+    for (int i0 = threadIdx.x; i0 < nparts; i0 += 2 * kFinThreads) {
+        double pa_[2], pb_[2];
+        float o[2][6];
 #pragma unroll
-            for (int k = 0; k < 6; ++k) o[k] = ext[((int64_t)k * nparts + i) * C + c];
+        for (int u = 0; u < 2; ++u) {
+            const int i = i0 + u * kFinThreads;
+            const bool ok = i < nparts;
+            pa_[u] = ok ? part_dy[(int64_t)i * C + c] : 0.0; pb_[u] = ok ? part_dyx[(int64_t)i * C + c] : 0.0;
 #pragma unroll
-            for (int k = 0; k < 6; ++k) ev[k] = (k & 1) ? fmaxf(ev[k], o[k]) : fminf(ev[k], o[k]);
+            for (int k = 0; k < 6; ++k) o[u][k] = ok && ext ? ext[((int64_t)k * nparts + i) * C + c] : (k & 1) ? -INFINITY : INFINITY;
         }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            a += pa_[u]; b += pb_[u];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) ev[k] = (k & 1) ? fmaxf(ev[k], o[u][k]) : fminf(ev[k], o[u][k]);
+        }
+    }
+    if (ext) {
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             ev[k] = (k & 1) ? warp_max(ev[k]) : warp_min(ev[k]);
