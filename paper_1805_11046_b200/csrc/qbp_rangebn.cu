@@ -817,46 +817,58 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_apply_kernel(const float 
 constexpr int kFewThreads = 512, kFewRows = 2048, kFewHigh = kFewThreads / 4;
 static bool few_rows(int64_t n, int64_t C) { return n <= kFewRows && C % 4 == 0; }
 
-// Sum (fp64), min and max over a block's rows, per channel: the lanes of a warp that hold the same channels by shuffles, the
-// warps in shared memory; all threads end up with their four channels' values.
+// Sum (fp64), min and max over a block's rows, per channel: the eight lanes of a warp that hold the same four channels by
+// shuffles (each step halves the channels a lane still carries: four shuffles per quantity instead of twelve), then the warps in
+// shared memory, one thread per quantity and channel (all threads adding up all warps took 6 us of a 64 x 64 tensor's backward).
+// Every thread can then read its channels' results from the table: sums first, then (min, max) pairs.
+template <int NS, int NM> struct FewTable { double sum[NS][16]; float lo[NM][16], hi[NM][16]; };
 template <int NS, int NM>      // sums; (min, max) pairs
-__device__ __forceinline__ void few_reduce(double (&sum)[NS][4], float (&lo)[NM][4], float (&hi)[NM][4])
+__device__ __forceinline__ const FewTable<NS, NM> &few_reduce(double (&sum)[NS][4], float (&lo)[NM][4], float (&hi)[NM][4])
 {
-    __shared__ double s_sum[NS][kFewThreads / 32][16];
-    __shared__ float s_lo[NM][kFewThreads / 32][16], s_hi[NM][kFewThreads / 32][16];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tx = lane & 3;
+    constexpr int kWarps = kFewThreads / 32;
+    __shared__ double s_sum[NS][kWarps][16];
+    __shared__ float s_lo[NM][kWarps][16], s_hi[NM][kWarps][16];
+    __shared__ FewTable<NS, NM> t;
+    static_assert((NS + 2 * NM) * 16 <= kFewThreads, "a thread per quantity and channel");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool b2 = lane & 4, b3 = lane & 8;
+    auto reduce = [&](auto (&v)[4], auto op) {             // of channel 2 * b2 + b3 over the lanes
+        auto r0 = op(b2 ? v[2] : v[0], __shfl_xor_sync(0xffffffffu, b2 ? v[0] : v[2], 4));
+        auto r1 = op(b2 ? v[3] : v[1], __shfl_xor_sync(0xffffffffu, b2 ? v[1] : v[3], 4));
+        auto q = op(b3 ? r1 : r0, __shfl_xor_sync(0xffffffffu, b3 ? r0 : r1, 8));
+        return op(q, __shfl_xor_sync(0xffffffffu, q, 16));
+    };
+    auto add = [](double a, double b) { return a + b; };
+    auto mn = [](float a, float b) { return fminf(a, b); };
+    auto mx = [](float a, float b) { return fmaxf(a, b); };
+    const int ch = (lane & 3) * 4 + (b2 ? 2 : 0) + (b3 ? 1 : 0);
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
+    for (int k = 0; k < NS; ++k) { const double r = reduce(sum[k], add); if (lane < 16) s_sum[k][warp][ch] = r; }
 #pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {
-#pragma unroll
-            for (int k = 0; k < NS; ++k) sum[k][e] += __shfl_xor_sync(0xffffffffu, sum[k][e], o);
-#pragma unroll
-            for (int k = 0; k < NM; ++k) {
-                lo[k][e] = fminf(lo[k][e], __shfl_xor_sync(0xffffffffu, lo[k][e], o));
-                hi[k][e] = fmaxf(hi[k][e], __shfl_xor_sync(0xffffffffu, hi[k][e], o));
-            }
-        }
-        if (lane < 4) {
-#pragma unroll
-            for (int k = 0; k < NS; ++k) s_sum[k][warp][tx * 4 + e] = sum[k][e];
-#pragma unroll
-            for (int k = 0; k < NM; ++k) { s_lo[k][warp][tx * 4 + e] = lo[k][e]; s_hi[k][warp][tx * 4 + e] = hi[k][e]; }
-        }
+    for (int k = 0; k < NM; ++k) {
+        const float l = reduce(lo[k], mn), h = reduce(hi[k], mx);
+        if (lane < 16) { s_lo[k][warp][ch] = l; s_hi[k][warp][ch] = h; }
     }
     __syncthreads();
+    const int q = threadIdx.x >> 4, c = threadIdx.x & 15;
+    if (q < NS) {
+        double r = 0.0;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
+        for (int w = 0; w < kWarps; ++w) r += s_sum[q][w][c];
+        t.sum[q][c] = r;
+    } else if (q < NS + NM) {
+        float r = INFINITY;
 #pragma unroll
-        for (int k = 0; k < NS; ++k) {
-            double t = 0.0;
-            for (int w = 0; w < kFewThreads / 32; ++w) t += s_sum[k][w][tx * 4 + e];
-            sum[k][e] = t;
-        }
+        for (int w = 0; w < kWarps; ++w) r = fminf(r, s_lo[q - NS][w][c]);
+        t.lo[q - NS][c] = r;
+    } else if (q < NS + 2 * NM) {
+        float r = -INFINITY;
 #pragma unroll
-        for (int k = 0; k < NM; ++k)
-            for (int w = 0; w < kFewThreads / 32; ++w) { lo[k][e] = fminf(lo[k][e], s_lo[k][w][tx * 4 + e]); hi[k][e] = fmaxf(hi[k][e], s_hi[k][w][tx * 4 + e]); }
+        for (int w = 0; w < kWarps; ++w) r = fmaxf(r, s_hi[q - NS - NM][w][c]);
+        t.hi[q - NS - NM][c] = r;
     }
+    __syncthreads();
+    return t;
 }
 
 // Forward: the rows wait in registers between the statistics and the normalisation (ROWS per thread, a power of two).
@@ -885,15 +897,17 @@ __global__ void __launch_bounds__(kFewThreads) bn_fwd_few_kernel(const float *__
 #pragma unroll
             for (int e = 0; e < 4; ++e) { sum[0][e] += (double)t[e]; lo[0][e] = fminf(lo[0][e], t[e]); hi[0][e] = fmaxf(hi[0][e], t[e]); }
         }
-    few_reduce<1, 1>(sum, lo, hi);
+    const FewTable<1, 1> &t1 = few_reduce<1, 1>(sum, lo, hi);
     if (!active) return;
+    const int cl = (threadIdx.x & 3) * 4;
     float mu[4], s[4], g[4], b[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        mu[e] = (float)(sum[0][e] / (double)rows);
-        s[e] = bn_scale(lo[0][e], hi[0][e], Cn);
+        const float lo_e = t1.lo[0][cl + e], hi_e = t1.hi[0][cl + e];
+        mu[e] = (float)(t1.sum[0][cl + e] / (double)rows);
+        s[e] = bn_scale(lo_e, hi_e, Cn);
         g[e] = gamma ? gamma[col + e] : 1.0f; b[e] = beta ? beta[col + e] : 0.0f;
-        if (ty == 0) { mean[col + e] = mu[e]; vmin[col + e] = lo[0][e]; vmax[col + e] = hi[0][e]; }
+        if (ty == 0) { mean[col + e] = mu[e]; vmin[col + e] = lo_e; vmax[col + e] = hi_e; }
     }
 #pragma unroll
     for (int u = 0; u < ROWS; ++u) {
@@ -968,13 +982,12 @@ __global__ void __launch_bounds__(kFewThreads) bn_bwd_few_kernel(const float *__
             }
         }
     }
-    few_reduce<2, 3>(sum, lo, hi);
-    if (!active || ty > 3) return;
-    // four threads of the first rows per vector, one channel each (picked by selection: a branch per channel would run the
-    // threshold's bisection four times over, 10 us)
-    auto pick = [&](const auto &t) { return ty == 0 ? t[0] : ty == 1 ? t[1] : ty == 2 ? t[2] : t[3]; };
-    const float ev[6] = {pick(lo[0]), pick(hi[0]), pick(lo[1]), pick(hi[1]), pick(lo[2]), pick(hi[2])};
-    bn_bwd_channel(col + ty, pick(sum[0]), pick(sum[1]), rows, Cnd, pick(g), pick(b), pick(mu), pick(cl), pick(ch), Cn,
+    const FewTable<2, 3> &t = few_reduce<2, 3>(sum, lo, hi);
+    // one thread per channel
+    const int k = threadIdx.x, c = (int)blockIdx.x * 16 + k;
+    if (k >= 16 || c >= C) return;
+    const float ev[6] = {t.lo[0][k], t.hi[0][k], t.lo[1][k], t.hi[1][k], t.lo[2][k], t.hi[2][k]};
+    bn_bwd_channel(c, t.sum[0][k], t.sum[1][k], rows, Cnd, gamma ? gamma[c] : 1.0f, beta ? beta[c] : 0.0f, mean[c], vmin[c], vmax[c], Cn,
                    out.chan_range ? ev : nullptr, out);
 }
 
