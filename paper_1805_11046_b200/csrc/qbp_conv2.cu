@@ -136,7 +136,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kC2Threads, 1) qbp_c
     cluster_sync_all();                  // both CTAs' barriers are initialised before either signals the other
     tc_fence_after();
     pdl_trigger();                       // (tensor memory is allocated, in both CTAs)
-    pdl_wait();
+    // (each role waits for the kernels before at its first use of their results: what it needs of the launch's parameters, and the
+    // code up to there, has then been fetched)
     const uint32_t tmem_base = tmem_slot;
     bool timed_out = false;
 
@@ -145,6 +146,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kC2Threads, 1) qbp_c
             // ---------------------------------------------------- TMA producer (both CTAs)
             const uint32_t cg = (uint32_t)P.cg;
             const int n_mine = n0 + (P.bn >> 1) * (int)rank;
+            bool waited = false;
             uint32_t s = 0, gph = 1, in_group = 0, group = 0;
             for (int tile = pair; tile < P.tiles_total && !timed_out; tile += P.pairs) {
                 const Conv2Box o = conv2_box(P, tile, rank);
@@ -156,6 +158,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kC2Threads, 1) qbp_c
                         const uint32_t bar = map_to_cta(&full_bar[s], 0);
                         if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * stage_bytes);
                         const int c0 = cc * 128, r = tap / 3, t = tap - 3 * r;
+                        if (!waited) { pdl_wait(); waited = true; }
                         // forward: input row p - 1 + r feeds output row p; layer gradient: gradient row h + 1 - r feeds input row h
                         if (!P.dgrad) {
                             tma_load_4d_pair(sa, &P.mapA, bar, c0, o.w0 + t - 1, o.h0 + r - 1, o.img0);
@@ -185,6 +188,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kC2Threads, 1) qbp_c
         const int ew = warp - 2, quad = warp & 3, half = ew >> 2, et = threadIdx.x - 64;
         const int row = quad * 32 + lane, hcols = P.bn >> 1;
         uint8_t *slab = staging + (size_t)ew * kC2Slab;
+        pdl_wait();
         const float scale = __fmul_rn(P.qa->scale, P.qb->scale);
         C2Stat *my_stat = s_stat + (size_t)ew * hcols;
         for (int i = et; i < 16 * P.bn; i += 32 * kC2EpiWarps) {

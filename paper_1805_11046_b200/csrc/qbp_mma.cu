@@ -453,7 +453,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
     __syncthreads();
     tc_fence_after();
     pdl_trigger();                       // (tensor memory is allocated)
-    pdl_wait();
+    // (each role waits for the kernels before at its first use of their results: what it needs of the launch's parameters, and the
+    // code up to there, has then been fetched)
     const uint32_t tmem_base = tmem_slot;
     const uint32_t buf_cols = (uint32_t)(P.msub * P.bn);
     bool timed_out = false;
@@ -462,9 +463,12 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
         // ---------------------------------------------------- TMA producer
         // Lane 0 owns the barriers.  Convolution: the `ips` activation tiles of a stage are issued by
         // `ips` lanes at once, each from its own entry of the k-iteration table.
+        bool waited = false;
+        auto wait_once = [&] { if (!waited) { pdl_wait(); waited = true; } };
         if (P.b_resident && lane == 0) {
             // the filter is the same for every tile of this CTA: fetch it once
             mbar_expect_tx(&b_full, P.b.tile_bytes * (uint32_t)P.k_iters);
+            wait_once();
             for (int it = 0; it < P.k_iters; ++it) {
                 const int4 e = s_iter[it];
                 uint8_t *dst = smem_b + (size_t)it * P.b.tile_bytes;
@@ -486,6 +490,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
                         uint8_t *sb = sa + a_stage;
                         mbar_expect_tx(&full_bar[s], stage_bytes);
                         const int k0 = it * P.kblock;
+                        wait_once();
                         // K-major operands: one box of all rows; M/N-major: one box per 128-byte column chunk
                         if (P.a.major == 0) tma_load_2d(sa, &P.mapA, &full_bar[s], k0, o.m0);
                         else
@@ -510,6 +515,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
                 }
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok) { timed_out = true; break; }
+                wait_once();
                 if (P.halo) {
                     // the pixel box with a border of `pad` pixels, one load per channel chunk; outside the image: zeros
                     if (lane < P.ips)
@@ -593,6 +599,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
         const int row = quad * 32 + lane;
         uint8_t *slab0 = staging + (size_t)(ew * P.nslab) * kStageSlab;
         uint32_t slab_i = 0;
+        pdl_wait();
         const float scale = __fmul_rn(P.qa->scale, P.qb->scale);
         ColStat *my_stat = s_stat + (size_t)ew * P.stat_cols;
         const int stat_base = P.stat_local ? (int)(blockIdx.x % (unsigned)P.tiles_n) * P.bn : 0;     // first column this CTA keeps

@@ -149,7 +149,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
     cluster_sync_all();                  // both CTAs' barriers are initialised before either signals the other
     tc_fence_after();
     pdl_trigger();                       // (tensor memory is allocated, in both CTAs)
-    pdl_wait();
+    // (each role waits for the kernels before at its first use of their results: what it needs of the launch's parameters, and the
+    // code up to there, has then been fetched)
     const uint32_t tmem_base = tmem_slot;
     bool timed_out = false;
 
@@ -157,6 +158,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
         if (lane == 0) {
             // ---------------------------------------------------- TMA producer (both CTAs)
             const uint32_t cg = (uint32_t)P.cg;
+            bool waited = false;
             uint32_t s = 0, gph = 1, in_group = 0, group = 0;
             for (int tile = pair; tile < P.tiles_total && !timed_out; tile += P.pairs) {
                 const Tile2 o = tile2_origin(P, tile);
@@ -169,6 +171,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
                     const uint32_t bar = map_to_cta(&full_bar[s], 0);
                     if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * stage_bytes);
                     const int k0 = it * 128;
+                    if (!waited) { pdl_wait(); waited = true; }
                     for (int sub = 0; sub < P.msub; ++sub) {
                         if (P.a.major == 0) tma_load_2d_pair(sa + sub * P.a.tile_bytes, &P.mapA, bar, k0, m_mine + 256 * sub);
                         else                tma_load_2d_pair(sa + sub * P.a.tile_bytes, &P.mapA, bar, m_mine + 256 * sub, k0);
@@ -207,6 +210,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
         const int et = threadIdx.x - 64;
         const int row = quad * 32 + lane;
         uint8_t *slab = staging + (size_t)ew * k2Slab;
+        pdl_wait();
         const float scale = __fmul_rn(P.qa->scale, P.qb->scale);
         const int neg_za = -P.qa->zero_point, neg_zb = -P.qb->zero_point, k_zz = P.k_len * neg_za * neg_zb;
         const uint32_t leader_empty0 = map_to_cta(&acc_empty[0], 0), leader_empty1 = map_to_cta(&acc_empty[1], 0);

@@ -364,7 +364,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
     __syncthreads();
     tc_fence_after();
     pdl_trigger();                       // (tensor memory is allocated)
-    pdl_wait();
+    // (each role waits for the kernels before at its first use of their results: what it needs of the launch's parameters, and the
+    // code up to there, has then been fetched)
     const uint32_t tmem_base = tmem_slot;
     bool timed_out = false;
 
@@ -387,6 +388,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
             if (++in_group == (uint32_t)cg) { in_group = 0; ++group; }
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) { timed_out = true; break; }
+            if (i == 0) pdl_wait();
             if (lane < n_loads) {
                 uint8_t *dst = smem + (size_t)s * stage_bytes + ld.x;
                 const int it = it_begin + i;
@@ -440,6 +442,22 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
         // ------------------------------------------------------- epilogue
         const int quad = warp & 3;
         const int row = quad * 32 + lane;
+        pdl_wait();
+        // what the epilogue needs of other kernels' results is fetched beside the products: the scale, the zero-points (signed
+        // low bytes: the limbs hold g16 - 128, against the zero-point zg - 128) and, one tile of rows ahead, the row terms
+        const float scale = P.direct ? __fmul_rn(P.qx->scale, P.qg->scale) : 0.0f;
+        const long long zg_d = P.direct ? P.qg->zero_point - (P.lo_signed ? 128 : 0) : 0, zz_d = P.direct ? P.M * P.qx->zero_point * zg_d : 0;
+        auto row_of = [&](int at, int64_t &k) {                     // whether this thread's row of A tile `at` is one of the result's
+            const bool valid = row / P.rb_a < chunks_of(at);
+            k = (int64_t)at * 128 + row;                            // plain: output row
+            if (!P.conv) return valid && k < P.K;
+            return valid && (at % P.tiles_c) * P.rb_a + row % P.rb_a < P.C;
+        };
+        auto row_term = [&](int at) {
+            int64_t k;
+            return P.direct && row_of(at, k) ? -zg_d * P.sx.at(k) + zz_d : 0ll;
+        };
+        long long rterm = n_tiles > 0 ? row_term(ag * P.ma) : 0;
         if (P.direct) {
             const int t = threadIdx.x - 64;
             const long long zx = P.qx->zero_point;
@@ -449,17 +467,12 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
         if (k_iters > 0 && !mbar_wait_warp(&acc_bar, 0)) timed_out = true;
         tc_fence_after();
         if (!timed_out && k_iters > 0) {
-            const float scale = P.direct ? __fmul_rn(P.qx->scale, P.qg->scale) : 0.0f;
-            // (signed low bytes: the limbs hold g16 - 128, against the zero-point zg - 128)
-            const long long zg_d = P.direct ? P.qg->zero_point - (P.lo_signed ? 128 : 0) : 0, zz_d = P.direct ? P.M * P.qx->zero_point * zg_d : 0;
             long long *part = P.part + (int64_t)blockIdx.x * P.part_stride;
             for (int j = 0; j < n_tiles; ++j) {
                 const int at = ag * P.ma + j;
-                bool valid = row / P.rb_a < chunks_of(at);
-                const int64_t k = (int64_t)at * 128 + row;                  // plain: output row
-                if (!P.conv) valid = valid && k < P.K;
-                else         valid = valid && (at % P.tiles_c) * P.rb_a + row % P.rb_a < P.C;
-                const long long rterm = (P.direct && valid) ? -zg_d * P.sx.at(k) + zz_d : 0;
+                int64_t k;
+                const bool valid = row_of(at, k);
+                const long long rterm_next = j + 1 < n_tiles ? row_term(at + 1) : 0;
                 const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(j * 2 * P.bn);
                 for (int c0 = 0; c0 < P.bn; c0 += 32) {
                     uint32_t rh[32], rl[32];
@@ -516,6 +529,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
                         }
                     }
                 }
+                rterm = rterm_next;
             }
         }
     }

@@ -153,13 +153,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
     w2_cluster_sync();                   // both CTAs' barriers are initialised before either signals the other
     tc_fence_after();
     pdl_trigger();                       // (tensor memory is allocated, in both CTAs)
-    pdl_wait();
+    // (each role waits for the kernels before at its first use of their results: what it needs of the launch's parameters, and the
+    // code up to there, has then been fetched)
     const uint32_t tmem_base = tmem_slot;
     bool timed_out = false;
 
     if (warp == 0) {
         if (lane == 0) {
             // ---------------------------------------------------- TMA producer (both CTAs)
+            bool waited = false;
             uint32_t s = 0, gph = 1, in_group = 0, group = 0;
             for (int tile = pair; tile < P.tiles_total && !timed_out; tile += P.pairs) {
                 const W2Tile o = w2_tile(P, tile);
@@ -171,6 +173,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
                     const uint32_t bar = w2_map_to_cta(&full_bar[s], 0);
                     if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * kW2StageBytes);
                     const int m0 = it * 128;
+                    if (!waited) { pdl_wait(); waited = true; }
                     w2_tma_load_2d(sa, &P.mapX, bar, k_mine, m0);
                     w2_tma_load_2d(sa + 16384, &P.mapHi, bar, n_mine, m0);
                     w2_tma_load_2d(sa + 32768, &P.mapLo, bar, n_mine, m0);
@@ -211,6 +214,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
         const int ew = warp - 2, quad = warp & 3, half = ew >> 2;
         const int row = quad * 32 + lane;
         uint8_t *slab = staging + (size_t)ew * kW2Slab;
+        pdl_wait();
         const float scale = __fmul_rn(P.qx->scale, P.qg->scale);
         const long long zx = P.qx->zero_point, zg = P.qg->zero_point - P.zg_shift;
         const uint32_t leader_empty = w2_map_to_cta(&acc_empty, 0);
