@@ -50,6 +50,17 @@ __device__ __forceinline__ int tern_keep(uint32_t word, float s, float a)
     return __fmul_rn(__fmul_rn((float)(word >> 8), 0x1p-24f), s) < a ? 1 : 0;
 }
 
+// The same with s24 = s * 2^-24 (exact), as 1 or 0 in fp32: the comparison gives the number that is added up, and the sum runs
+// on the floating-point pipe (with a predicate, a selection and an integer sum the integer pipe, which Philox fills, had 36
+// instructions per four draws, now 26: six samples of 6.4 M elements 43 -> 39 us; the two pipes that Philox uses do not
+// overlap, and are 90 % busy together).
+__device__ __forceinline__ float tern_keep1(uint32_t word, float s24, float a)
+{
+    float r;
+    asm("set.lt.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(__fmul_rn((float)(word >> 8), s24)), "f"(a));
+    return r;
+}
+
 // Sum over `samples` stochastic ternarisations of g: code = sign(g) * (number of samples that keep the element), as
 // int8 (q), and / or as the two byte limbs of the same value as a 16-bit code (hi: 0 or -1, lo: the low byte), which
 // is what the weight-gradient product takes.  parts: the range scan's (min, max) pairs (s = max(-vmin, vmax)); *qp_out receives
@@ -72,23 +83,25 @@ __global__ void __launch_bounds__(kTbpThreads) stc_ternarize_kernel(const float 
         *qp_out = r;
     }
     const int64_t stride = (int64_t)gridDim.x * kTbpThreads;
-    if (VEC == 4) {
+    const float s24 = __fmul_rn(s, 0x1p-24f);
+    const bool vector = VEC == 4 && __fmul_rn(s24, 0x1p24f) == s;       // (s below 2^-102 or so: s24 is not exact)
+    if (vector) {
         const int64_t nv = n >> 2;
         for (int64_t j = (int64_t)blockIdx.x * kTbpThreads + threadIdx.x; j < nv; j += stride) {
             const float4 v = __ldcs(reinterpret_cast<const float4 *>(g) + j);
             const float xs[4] = {v.x, v.y, v.z, v.w};
-            float p[4]; int cnt[4] = {0, 0, 0, 0};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) p[e] = fabsf(xs[e]);
+            float cnt[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 2
             for (int k = 0; k < samples; ++k) {
                 const uint4 b = philox4x32_10(make_uint4((uint32_t)j, J32 ? 0u : (uint32_t)((uint64_t)j >> 32), tensor_id, (uint32_t)k), keys);
-                cnt[0] += tern_keep(b.x, s, p[0]); cnt[1] += tern_keep(b.y, s, p[1]);
-                cnt[2] += tern_keep(b.z, s, p[2]); cnt[3] += tern_keep(b.w, s, p[3]);
+                const uint32_t w[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) cnt[e] += tern_keep1(w[e], s24, fabsf(xs[e]));
             }
             uint32_t w8 = 0, whi = 0;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const int c = xs[e] > 0.0f ? cnt[e] : -cnt[e];
+                const int c = (int)copysignf(cnt[e], xs[e]);        // (nothing keeps a zero or a NaN)
                 w8 |= ((uint32_t)c & 0xFFu) << (8 * e);
                 whi |= (c < 0 ? 0xFFu : 0u) << (8 * e);
             }
@@ -97,8 +110,8 @@ __global__ void __launch_bounds__(kTbpThreads) stc_ternarize_kernel(const float 
             if (lo) reinterpret_cast<uint32_t *>(lo)[j] = w8;
         }
     }
-    // elements the vector loop leaves (all of them when VEC == 1)
-    const int64_t first = VEC == 4 ? (n >> 2) << 2 : 0;
+    // elements the vector loop leaves (all of them without it)
+    const int64_t first = vector ? (n >> 2) << 2 : 0;
     for (int64_t i = first + (int64_t)blockIdx.x * kTbpThreads + threadIdx.x; i < n; i += stride) {
         const float p = fabsf(g[i]);
         const int64_t j = i >> 2;
