@@ -184,6 +184,8 @@ struct MmaParams {
     int b_stage_tiles;            // filter tiles consumed per stage (resident filter)
     uint32_t stage_tx;            // bytes the TMA loads of one stage deliver
     int egroups;                  // msub == 1: groups of four epilogue warps that take tiles in turn (at most 3, at most nbuf)
+    int one_tile;                 // no CTA has more than one tile (known before the launch's shape is)
+    int split;                    // msub == 1, one tile per CTA: the groups share its column chunks
     int ewarps;                   // epilogue warps at work (the rest of the kEpiWarps idle): 8 when msub == 2, else 4 * egroups
     int nslab;                    // epilogue staging slabs per warp (2: a store is still reading one while the next is filled)
     // Per-column statistics of the fp32 output (for the Range BN that follows, Section 3): every working epilogue
@@ -592,7 +594,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
         // msub == 2: two groups of four warps work on every tile, one 128-row sub-tile each.
         // msub == 1: the groups take tiles (and accumulator buffers) in turn: a warp's read-out, arithmetic and
         //            store of a tile is one long dependent chain, so the epilogue's throughput is the number of
-        //            tiles in flight.
+        //            tiles in flight.  A CTA's only tile (split): the groups take its chunks in turn, 1100 cycles each.
         const int ew = warp - 2;                         // 0 .. P.ewarps-1
         const int quad = warp & 3;                       // the tensor-memory lanes this warp may read
         const int group = ew >> 2;
@@ -653,9 +655,9 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
         };
 
         const int tile_step = (int)gridDim.x * lt_step;
-        int tile = blockIdx.x + (P.msub == 2 ? 0 : group * (int)gridDim.x);
+        int tile = blockIdx.x + (P.msub == 2 || P.split ? 0 : group * (int)gridDim.x);
         // this group's accumulator buffer and the parity of its "full" barrier; msub == 1: buffers of the group's own parity
-        uint32_t buf = P.msub == 2 ? 0u : (uint32_t)group, fph = 0;
+        uint32_t buf = P.msub == 2 || P.split ? 0u : (uint32_t)group, fph = 0;
         TileOrigin o = tile_origin(P, tile < P.tiles_total ? tile : 0);
         RowInfo ri = row_info(o);
         int rterm = (tile < P.tiles_total && ri.valid) ? row_term(ri.m) : 0;
@@ -682,7 +684,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
                 tc_fence_after();
                 const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + buf * buf_cols + (uint32_t)(sub * P.bn);
                 int row_code_sum = 0;                   // of this thread's output row's 8-bit codes (one column tile)
-                for (int c = 0; c < nchunks; ++c) {
+                for (int c = P.split ? group : 0; c < nchunks; c += P.split ? P.egroups : 1) {
                     const int c0 = c * 32;
                     uint32_t r[32];
                     tmem_ld_32x32(t_addr + (uint32_t)c0, r);
@@ -1018,7 +1020,8 @@ static uint32_t fixed_smem(MmaParams &P)
     P.egroups = P.msub == 2 ? 2 : std::min(kEpiWarps / 4, P.nbuf);
     if (P.msub == 1) P.nbuf -= P.nbuf % P.egroups;
     P.ewarps = 4 * P.egroups;
-    P.cterm_all = (size_t)P.ncls * P.N * sizeof(int32_t) <= 32u * 1024u ? 1 : 0;
+    // (a CTA with one tile of a product needs that tile's columns only)
+    P.cterm_all = (size_t)P.ncls * P.N * sizeof(int32_t) <= 32u * 1024u && !P.one_tile ? 1 : 0;
     const size_t cterm_bytes = P.cterm_all ? ((size_t)P.ncls * P.N + 64) * sizeof(int32_t)
                                            : (size_t)(P.msub == 1 ? P.egroups : 1) * P.ncls * P.bn * sizeof(int32_t);
     P.iter_entries = P.mode == MODE_GEMM ? 0 : (int)align_up((size_t)P.k_iters, 64);
@@ -1099,6 +1102,8 @@ static int launch_mma(MmaParams &P, int tiles_m, cudaStream_t st)
         grid -= grid % P.tiles_n;
     }
     P.grid = grid;
+    // (a row's code sum is one thread's: such a tile stays with one group)
+    P.split = P.msub == 1 && P.tiles_total <= grid && !P.ep_rowsum ? 1 : 0;
     QBP_TRACE_BEGIN(st);
     launch(kernel, grid, kMmaThreads, smem, st, P);
     QBP_LAUNCH_OK("qbp_mma_kernel");
@@ -1264,7 +1269,14 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
     P.kblock = 128;
     P.k_iters = (int)((K + 127) / 128);
     P.mma_per_iter = 4;
-    P.msub = M > 128 ? 2 : 1;            // 256-row CTA tiles halve the operand traffic per multiply-add
+    // 256-row CTA tiles halve the operand traffic per multiply-add; where tiles of 128 rows fit the machine once, and then where
+    // tiles of half as many columns do (32 at least), the smaller tiles: their rings and epilogues are shorter (64 x 256 x 128,
+    // traced with its launch: 12.8 us as one tile of 256 columns, 10.6 as eight of 32.  Not for what the pair kernel takes:
+    // 1024 x 1008 x 2048 on 128 CTAs is no faster than on its 16 pairs)
+    const auto tiles_of = [&](int64_t m, int64_t n) { return ((M + m - 1) / m) * ((N + n - 1) / n); };
+    P.msub = M > 128 && tiles_of(128, 256) > sm_count() ? 2 : 1;
+    int64_t cols = 256;
+    while (!has_tail && P.msub == 1 && cols > 32 && tiles_of(128, cols / 2) <= sm_count()) cols /= 2;
     P.ncls = 1; P.nslab = 1;
     // A: stored [M x K] -> K-major rows of 128 reduction bytes; stored [K x M] -> M-major, one box per sub-tile
     if (!transA) {
@@ -1277,13 +1289,14 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
     }
     if (rc) return rc;
     if (transB) {
-        P.bn = (int)std::min<int64_t>(256, N);
+        P.bn = (int)std::min<int64_t>(cols, N);
         P.b = layout_kmajor((uint32_t)P.bn, 128);
         rc = make_map_2d(&P.mapB, B, N, K, (uint32_t)P.bn, 128);
     } else {
         // N-contiguous operand: one swizzled row holds min(128, N) output columns; two such chunks make 256
-        const uint32_t rb = N >= 128 ? 128u : N >= 64 ? 64u : 32u;
-        const uint32_t chunks = (rb == 128 && N >= 256) ? 2u : 1u;
+        const int64_t nb = std::min(cols, N);
+        const uint32_t rb = nb >= 128 ? 128u : nb >= 64 ? 64u : 32u;
+        const uint32_t chunks = (rb == 128 && nb >= 256) ? 2u : 1u;
         P.bn = (int)(rb * chunks);
         P.b = layout_mnmajor(128, rb, chunks, 128 * rb);
         P.b_loads = (int)chunks; P.b_load_bytes = 128 * rb;
@@ -1293,6 +1306,7 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
     if (C && (rc = make_map_out_2d(&P.mapC, C, M, N))) return rc;
     P.idesc = make_idesc(true, true, P.a.major, P.b.major, 128, (uint32_t)P.bn);
     P.tiles_n = (int)((N + P.bn - 1) / P.bn);
+    P.one_tile = P.msub == 1 && (M + 127) / 128 * P.tiles_n <= sm_count() ? 1 : 0;
     P.M = M; P.N = N;
     P.acc_out = acc_out; P.out = C;
     P.raw_sums = 1; P.k_len = (int)K; P.a_sums = asum; P.b_sums = bsum; P.qa = qa; P.qb = qb; P.status = status;

@@ -734,7 +734,10 @@ static void plan_wgrad(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, 
     P.conv = d ? 1 : 0;
     P.M = M; P.N = N; P.K = K;
     // g side: one swizzled row holds bn output channels
-    const uint32_t rb_b = N >= 128 ? 128u : N >= 64 ? 64u : 32u;
+    uint32_t rb_b = N >= 128 ? 128u : N >= 64 ? 64u : 32u;
+    // (a short plain reduction -- done whole, see below -- whose tiles of half as many columns still fit the machine once: the
+    // epilogue takes 1900 cycles per 32 columns)
+    while (!d && M <= 8 * kWgRows && rb_b > 32 && ((K + 127) / 128) * ((N + rb_b / 2 - 1) / (rb_b / 2)) <= sm_count()) rb_b /= 2;
     P.bn = (int)rb_b;
     P.tiles_b = (int)((N + P.bn - 1) / P.bn);
     // x side: 128 MMA rows = a_chunks chunks of rb_a columns / channels

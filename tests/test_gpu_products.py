@@ -489,3 +489,28 @@ def test_conv_pairs(B, N, H, W, C, K, mode):
     assert bad == 0 and np.array_equal(a[idx], oacc) and np.array_equal(o[idx], oout)
     assert np.array_equal(o, a.astype(np.float32) * np.float32(0.125))
     _check_col_stats(out, stats)
+
+
+# ------------------------------------------------- products that leave most of the machine idle: smaller tiles
+@pytest.mark.parametrize("M,N,K", [(48, 4736, 64), (48, 4752, 64), (128, 9488, 32), (240, 96, 160), (2304, 240, 48), (2432, 240, 48),
+                                   (16, 37888, 16), (16, 37904, 16)])
+@pytest.mark.parametrize("tB", [False, True])
+def test_gemm_tiles_that_fit_the_machine_once(B, M, N, K, tB):
+    """128-row tiles of 32, 64, 128 and 256 columns are taken while they fit 148 SMs once, each size just inside and just outside;
+    a CTA's only tile is read out by all epilogue groups, its columns in chunks that do not divide evenly among them."""
+    A = random_codes((M, K), 61); Bm = random_codes((N, K) if tB else (K, N), 62)
+    acc, out, ws = B.qbp_gemm_s8(to_dev(A), _qp(B, 0.5, 7), to_dev(Bm), _qp(B, 0.25, -19), transB=tB, want_acc=True)
+    oacc, oout, bad = O.gemm_s8(A, 7, Bm, -19, 0.5, 0.25, transB=tB)
+    assert bad == 0 and B.status_word(ws) == 0
+    assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(out), oout)
+
+
+@pytest.mark.parametrize("M,N,K", [(64, 32, 128), (128, 4736, 16), (128, 4752, 16), (1024, 1184, 512), (1024, 1200, 512), (144, 176, 240)])
+def test_wgrad_tiles_that_fit_the_machine_once(B, M, N, K):
+    """Short reductions over tiles of 32, 64 and 128 columns, each size just inside and just outside one wave."""
+    X = random_codes((M, K), 63); G = _g16((M, N), 64)
+    hi, lo = O.limb_split(G)
+    acc, dW, ws = B.qbp_wgrad_s16(to_dev(X), _qp(B, 0.5, -3), to_dev(hi), to_dev(lo), _qp(B, 0.25, 1234), want_acc=True)
+    oacc, oout = O.gemm_s16s8(X, -3, G, 1234, 0.5, 0.25)
+    assert B.status_word(ws) == 0
+    assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
