@@ -475,6 +475,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
                 const long long rterm_next = j + 1 < n_tiles ? row_term(at + 1) : 0;
                 const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(j * 2 * P.bn);
                 for (int c0 = 0; c0 < P.bn; c0 += 32) {
+                    if ((int64_t)n0 + c0 >= P.N) break;                     // (a ragged last tile: nothing reads those)
                     uint32_t rh[32], rl[32];
                     tmem_ld_32x32(t_addr + (uint32_t)c0, rh);
                     tmem_ld_32x32(t_addr + (uint32_t)(P.bn + c0), rl);
@@ -753,15 +754,6 @@ static void plan_wgrad(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, 
         P.tiles_c = (d->C + (int)rb_a - 1) / (int)rb_a;
         P.a_tiles = ((P.taps + P.a_chunks - 1) / P.a_chunks) * P.tiles_c;
     }
-    // A tiles per CTA: at most what tensor memory holds (two accumulators of bn columns each), spread evenly over
-    // the groups that takes (5 tiles: 3 + 2 rather than 4 + 1 -- a stage of few MMAs is bound by its fixed costs)
-    const int ma_max = std::max(1, std::min({kWgMaxTiles, 512 / (2 * P.bn), P.a_tiles}));
-    P.a_groups = (P.a_tiles + ma_max - 1) / ma_max;
-    // (a plain product whose tiles do not fill the machine: one A tile per CTA)
-    if (!d && (int64_t)P.a_tiles * P.tiles_b <= sm_count()) P.a_groups = P.a_tiles;
-    P.ma = (P.a_tiles + P.a_groups - 1) / P.a_groups;
-    int cols = 32; while (cols < P.ma * 2 * P.bn) cols <<= 1;
-    P.tmem_cols = cols;
     // reduction rows per stage: kWgRows (the ring is shallower than with 64, but a stage holds twice the MMAs)
     const uint32_t kr = kWgRows;
     P.kr = (int)kr;
@@ -802,6 +794,33 @@ static void plan_wgrad(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, 
         P.iters_total = P.tiles_w * P.tiles_h * ((d->N + pl.bn_img - 1) / pl.bn_img);
         P.d_tiles_w = make_fastdiv(P.tiles_w); P.d_tiles_h = make_fastdiv(P.tiles_h);
     }
+    // A tiles per CTA: at most what tensor memory holds (two accumulators of bn columns each), spread evenly over
+    // the groups that takes (5 tiles: 3 + 2 rather than 4 + 1 -- a stage of few MMAs is bound by its fixed costs)
+    const int ma_max = std::max(1, std::min({kWgMaxTiles, 512 / (2 * P.bn), P.a_tiles}));
+    P.a_groups = (P.a_tiles + ma_max - 1) / ma_max;
+    // (a plain product whose tiles do not fill the machine: one A tile per CTA)
+    if (!d && (int64_t)P.a_tiles * P.tiles_b <= sm_count()) P.a_groups = P.a_tiles;
+    // A convolution's reduction is split over the machine, and every CTA reads out and writes a partial of all its A tiles: more of
+    // them share the gradient's tiles in the loop, fewer leave less to read out, write and add up.  In cycles: an operand row of the
+    // loop 2.7 (what the copies reach), a tile's read-out 6000, the partials at 2.6 KB a cycle over the machine.  (20 images of
+    // 19 x 19, 96 -> 160: kernel and finalize 22.9 + 14.7 us with two tiles, 18.9 + 12.8 with one, launches included; 64 images of
+    // 28 x 28, 128 -> 128: 31 + 16 and 25 + 13; 256 of 14 x 14, 256 -> 256 stays with two: 52 + 21.)
+    if (d && !P.halo_bh) {
+        int64_t best = -1;
+        int groups = P.a_groups;
+        for (int ma = ma_max; ma >= 1; --ma) {
+            const int64_t ag = (P.a_tiles + ma - 1) / ma, items = ag * P.tiles_b;
+            const int64_t slices = std::max<int64_t>(1, std::min<int64_t>(sm_count() / items, P.iters_total));
+            const int64_t waves = (items * slices + sm_count() - 1) / sm_count(), iters = (P.iters_total + slices - 1) / slices;
+            const int64_t loop = iters * (int64_t)kr * (ma * P.a_chunks + 2) * 27 / 10, part = items * slices * ma * 128 * P.bn * 8;
+            const int64_t cost = waves * (loop + ma * 6000) + part / 2600;
+            if (best < 0 || cost < best) { best = cost; groups = (int)ag; }
+        }
+        P.a_groups = groups;
+    }
+    P.ma = (P.a_tiles + P.a_groups - 1) / P.a_groups;
+    int cols = 32; while (cols < P.ma * 2 * P.bn) cols <<= 1;
+    P.tmem_cols = cols;
     // pipeline: stages of kr rows; one commit releases `cg` stages (some 24 MMAs between commits while that leaves
     // three groups in the ring).  The CTAs of the last group (fewer A tiles) get a ring of their own shape.
     const int n_last = P.a_tiles - (P.a_groups - 1) * P.ma;                 // A tiles of the last group

@@ -514,3 +514,10 @@ def test_wgrad_tiles_that_fit_the_machine_once(B, M, N, K):
     oacc, oout = O.gemm_s16s8(X, -3, G, 1234, 0.5, 0.25)
     assert B.status_word(ws) == 0
     assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
+
+
+@pytest.mark.parametrize("N,H,W,C,K,R", [(1, 8, 16, 128, 128, 3), (2, 12, 12, 128, 160, 3), (6, 16, 16, 256, 96, 1), (5, 11, 13, 96, 160, 3)])
+def test_wgrad_conv_one_tile_per_block_and_ragged_columns(B, N, H, W, C, K, R):
+    """Reductions short enough that each block takes one tile of 128 rows, from a single step on; output channels that leave most
+    of the last tile's columns out."""
+    test_wgrad_conv_finalize_block_shapes(B, N, H, W, C, K, R)
