@@ -515,6 +515,19 @@ int qbp_layer_bwd(const qbp_layer_desc *L, const qbp_layer_ctx *saved, const flo
 int qbp_sgd_update(float *w, const float *dw, float *momentum_buf, int64_t count,
                    float lr, float momentum, float weight_decay, void *stream);
 
+/* The same for several tensors at once (a model's step in few launches); the
+ * tensors must not overlap.  `tensors` is host memory, read before the call
+ * returns. */
+typedef struct qbp_sgd_tensor {
+    float *w;
+    const float *dw;
+    float *momentum_buf;      /* nullable */
+    int64_t count;
+    float weight_decay;
+    int32_t reserved;         /* 0 */
+} qbp_sgd_tensor;
+int qbp_sgd_update_many(const qbp_sgd_tensor *tensors, int n_tensors, float lr, float momentum, void *stream);
+
 /* ------------------------------------------------------------------------
  * Appendix C -- Ternarized Back-Propagation: 1-bit weights and activations,
  * ternary gradients, every forward MAC an XNOR + popcount.

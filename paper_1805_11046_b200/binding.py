@@ -26,7 +26,7 @@ EXPORTS = (
     "qbp_last_error", "qbp_trace_enable", "qbp_trace_count", "qbp_trace_read",
     "qbp_device_status", "qbp_selftest_bounded_wait",
     "qbp_quantize_workspace_bytes", "qbp_quantize_s8", "qbp_quantize_s8_static", "qbp_quantize_s16", "qbp_bifurcate",
-    "qbp_bifurcate_shard", "qbp_dequant_s64", "qbp_sgd_update",
+    "qbp_bifurcate_shard", "qbp_dequant_s64", "qbp_sgd_update", "qbp_sgd_update_many",
     "qbp_range_chunked_workspace_bytes", "qbp_range_chunked",
     "qbp_gemm_s8_workspace_bytes", "qbp_gemm_s8", "qbp_gemm_s8_sums",
     "qbp_conv_s8_workspace_bytes", "qbp_conv_s8_implicit",
@@ -510,6 +510,19 @@ def qbp_sgd_update(w, dw, momentum_buf=None, lr=0.1, momentum=0.0, weight_decay=
     _check(lib.qbp_sgd_update(_ptr(w), _ptr(dw), _ptr(momentum_buf), C.c_int64(w.numel()), C.c_float(lr),
                               C.c_float(momentum), C.c_float(weight_decay), _stream()))
     return w
+
+
+class SgdTensor(C.Structure):
+    _fields_ = [("w", C.c_void_p), ("dw", C.c_void_p), ("momentum_buf", C.c_void_p), ("count", C.c_int64),
+                ("weight_decay", C.c_float), ("reserved", C.c_int32)]
+
+
+def qbp_sgd_update_many(tensors, lr=0.1, momentum=0.0):
+    """qbp_sgd_update for several tensors at once: (w, dw, momentum_buf or None, weight_decay) each."""
+    a = (SgdTensor * len(tensors))()
+    for t, (w, dw, v, wd) in zip(a, tensors):
+        t.w, t.dw, t.momentum_buf, t.count, t.weight_decay = _ptr(w), _ptr(dw), _ptr(v), w.numel(), wd
+    _check(lib.qbp_sgd_update_many(a, len(tensors), C.c_float(lr), C.c_float(momentum), _stream()))
 
 
 # ---------------------------------------------------------------------- layer

@@ -1152,14 +1152,26 @@ extern "C" __attribute__((visibility("default"))) int qbp_dequant_s64(const int6
 // fp32 master-weight update (Section 6 "Putting it all together": the updates stay in float32 and run once per
 // minibatch): g = dw + wd * w;  v = mu * v + g (with a momentum buffer);  w = w - lr * v.  Every operation is
 // rounded on its own, in this order.
-__global__ void __launch_bounds__(256) sgd_update_kernel(float *__restrict__ w, const float *__restrict__ dw,
-                                                         float *__restrict__ vbuf, int64_t n, float lr, float mu, float wd)
+// A launch takes up to kSgdTensors tensors, each with its share of the blocks (the nine tensors of three layers: 2 us each as
+// launches of their own, which is all they take).
+constexpr int kSgdTensors = 32;
+struct SgdTensor { float *w; const float *dw; float *v; int64_t n; float wd; int first_block; };
+struct SgdTensors { SgdTensor t[kSgdTensors]; int count; };
+__global__ void __launch_bounds__(256) sgd_update_kernel(const __grid_constant__ SgdTensors J, float lr, float mu)
 {
     pdl_enter();
-    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+    int k = 0;
+    while (k + 1 < J.count && (int)blockIdx.x >= J.t[k + 1].first_block) ++k;
+    const SgdTensor &T = J.t[k];
+    const int last = k + 1 < J.count ? J.t[k + 1].first_block : (int)gridDim.x;
+    float *const w = T.w, *const v = T.v;
+    const float *const dw = T.dw;
+    const int64_t n = T.n, step = (int64_t)(last - T.first_block) * 256;
+    const float wd = T.wd;
+    for (int64_t i = (int64_t)((int)blockIdx.x - T.first_block) * 256 + threadIdx.x; i < n; i += step) {
         const float wi = w[i];
         float g = __fadd_rn(dw[i], __fmul_rn(wd, wi));
-        if (vbuf) { g = __fadd_rn(__fmul_rn(mu, vbuf[i]), g); vbuf[i] = g; }
+        if (v) { g = __fadd_rn(__fmul_rn(mu, v[i]), g); v[i] = g; }
         w[i] = __fsub_rn(wi, __fmul_rn(lr, g));
     }
 }
@@ -1167,13 +1179,34 @@ __global__ void __launch_bounds__(256) sgd_update_kernel(float *__restrict__ w, 
 extern "C" __attribute__((visibility("default"))) int qbp_sgd_update(float *w, const float *dw, float *momentum_buf, int64_t count,
                               float lr, float momentum, float weight_decay, void *stream)
 {
-    cudaStream_t st = (cudaStream_t)stream;
     if (count < 0 || (count > 0 && (!w || !dw))) return fail(QBP_ERR_INVALID_ARG, "sgd_update: NULL tensor");
     if (count == 0) return QBP_OK;
-    const int grid = (int)std::min<int64_t>((count + 255) / 256, (int64_t)sm_count() * 8);
-    QBP_TRACE_BEGIN(st);
-    launch(sgd_update_kernel, grid, 256, 0, st, w, dw, momentum_buf, count, lr, momentum, weight_decay);
-    QBP_LAUNCH_OK("sgd_update_kernel");
+    const qbp_sgd_tensor t{w, dw, momentum_buf, count, weight_decay, 0};
+    return qbp_sgd_update_many(&t, 1, lr, momentum, stream);
+}
+
+extern "C" __attribute__((visibility("default"))) int qbp_sgd_update_many(const qbp_sgd_tensor *tensors, int n_tensors, float lr, float momentum,
+                                                                          void *stream)
+{
+    cudaStream_t st = (cudaStream_t)stream;
+    if (n_tensors < 0 || (n_tensors > 0 && !tensors)) return fail(QBP_ERR_INVALID_ARG, "sgd_update_many: NULL tensors or a negative count");
+    for (int i = 0; i < n_tensors; ++i)
+        if (tensors[i].count < 0 || (tensors[i].count > 0 && (!tensors[i].w || !tensors[i].dw)))
+            return fail(QBP_ERR_INVALID_ARG, "sgd_update_many: tensor %d is NULL or of negative size", i);
+    for (int i = 0; i < n_tensors;) {
+        SgdTensors J{};
+        int blocks = 0;
+        for (; i < n_tensors && J.count < kSgdTensors; ++i) {
+            const qbp_sgd_tensor &t = tensors[i];
+            if (t.count == 0) continue;
+            J.t[J.count++] = SgdTensor{t.w, t.dw, t.momentum_buf, t.count, t.weight_decay, blocks};
+            blocks += (int)std::min<int64_t>((t.count + 255) / 256, (int64_t)sm_count() * 8);
+        }
+        if (!J.count) break;
+        QBP_TRACE_BEGIN(st);
+        launch(sgd_update_kernel, blocks, 256, 0, st, J, lr, momentum);
+        QBP_LAUNCH_OK("sgd_update_kernel");
+    }
     return QBP_OK;
 }
 

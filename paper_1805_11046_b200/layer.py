@@ -133,10 +133,10 @@ class QuantizedStack:
         return d
 
     def update(self):
+        tensors = []
         for L, w, g, b, vw, vg, vb in zip(self.layers, self.w, self.gamma, self.beta, self.vw, self.vg, self.vb):
-            B.qbp_sgd_update(w, L.dw, vw, self.lr, self.momentum, self.weight_decay)
-            B.qbp_sgd_update(g, L.dgamma, vg, self.lr, self.momentum, 0.0)
-            B.qbp_sgd_update(b, L.dbeta, vb, self.lr, self.momentum, 0.0)
+            tensors += [(w, L.dw, vw, self.weight_decay), (g, L.dgamma, vg, 0.0), (b, L.dbeta, vb, 0.0)]
+        B.qbp_sgd_update_many(tensors, self.lr, self.momentum)
 
     def train_step(self, x, dy):
         self.forward(x)

@@ -502,3 +502,17 @@ def test_backward_where_many_elements_are_extremes(B, batch, cin, cout, id16):
         w[:, c] = 0.0
         w[c % cin, c] = 0.3
     _check_layer(B, dict(x=x, w=w, dy=synth.normal((batch, cout), 73, std=0.1), seed=4, id8=5, id16=id16), True)
+
+
+@pytest.mark.parametrize("momentum", [0.0, 0.9])
+def test_sgd_update_of_many_tensors(B, momentum):
+    """More tensors than one launch takes, empty ones and single elements among them: each as if updated alone."""
+    sizes = [1, 255, 256, 257, 0, 4099, 70000] * 5 + [3]
+    w = [synth.normal((n,), 90 + i) for i, n in enumerate(sizes)]
+    dw = [synth.normal((n,), 200 + i, std=0.01) for i, n in enumerate(sizes)]
+    v = [synth.normal((n,), 300 + i, std=0.01) if momentum else None for i, n in enumerate(sizes)]
+    dev = [(to_dev(a), to_dev(b), to_dev(c) if momentum else None, 1e-4 * (i % 3)) for i, (a, b, c) in enumerate(zip(w, dw, v))]
+    B.qbp_sgd_update_many(dev, lr=0.05, momentum=momentum)
+    for (wd_, _, vd, decay), a, b, c in zip(dev, w, dw, v):
+        ow, ov = O.sgd_update(a, b, c, lr=0.05, momentum=momentum, weight_decay=decay)
+        assert np.array_equal(to_host(wd_), ow) and (not momentum or np.array_equal(to_host(vd), ov))
