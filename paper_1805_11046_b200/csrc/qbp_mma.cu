@@ -454,7 +454,6 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_trigger();                       // (tensor memory is allocated)
     // (each role waits for the kernels before at its first use of their results: what it needs of the launch's parameters, and the
     // code up to there, has then been fetched)
     const uint32_t tmem_base = tmem_slot;
@@ -870,7 +869,7 @@ struct ConvTerms {
 // The first `sum_blocks` blocks take code sums that a later product needs (a launch less, and they overlap).
 __global__ void __launch_bounds__(256, 6) conv_terms_kernel(const __grid_constant__ ConvTerms T, const __grid_constant__ SumJobs J, int sum_blocks)
 {
-    pdl_enter();
+    pdl_wait();
     if ((int)blockIdx.x < sum_blocks) { code_sums_block(J, (int)blockIdx.x); return; }
     const int block = (int)blockIdx.x - sum_blocks;
     if (block >= T.row_blocks) {
@@ -922,7 +921,7 @@ __global__ void __launch_bounds__(128) colstat_finalize_kernel(const float *__re
                                                                double *__restrict__ col_sum, float *__restrict__ col_min,
                                                                float *__restrict__ col_max)
 {
-    pdl_enter();
+    pdl_wait();
     const int c = blockIdx.x;
     float lo = INFINITY, hi = -INFINITY;
     double sum = 0.0;
@@ -967,7 +966,7 @@ static size_t colstat_ws_bytes(int64_t N, bool conv = false)
 // Parameters of the requantisation in a product's epilogue from the caller's clamping values.
 __global__ void epilogue_qparams_kernel(const qbp_qparams *__restrict__ range, qbp_qparams *__restrict__ qp8)
 {
-    pdl_enter();
+    pdl_wait();
     *qp8 = make_qparams(range->vmin, range->vmax, 8);
 }
 

@@ -88,7 +88,7 @@ template <int VEC>
 __global__ void __launch_bounds__(kThreads) range_partial_kernel(const __grid_constant__ ScanJob a, const __grid_constant__ ScanJob b,
                                                                  const __grid_constant__ ZeroJobs zero)
 {
-    pdl_enter();
+    pdl_wait();
     const bool second = (int)blockIdx.x < b.blocks;
     const ScanJob &J = second ? b : a;
     const int block = second ? (int)blockIdx.x : (int)blockIdx.x - b.blocks;
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kThreads) range_partial_kernel(const __grid_co
 // The parameters of an empty tensor.
 __global__ void empty_qparams_kernel(qbp_qparams *qp8, qbp_qparams *qp16)
 {
-    pdl_enter();
+    pdl_wait();
     if (qp8) *qp8 = make_qparams(0.0f, 0.0f, 8);
     if (qp16) *qp16 = make_qparams(0.0f, 0.0f, 16);
 }
@@ -134,7 +134,7 @@ template <int VEC>
 __global__ void __launch_bounds__(kThreads) chunk_range_partial_kernel(const float *__restrict__ x, int64_t n_chunk,
                                                                        float2 *__restrict__ partials)
 {
-    pdl_enter();
+    pdl_wait();
     x += (int64_t)blockIdx.y * n_chunk;
     float lo = INFINITY, hi = -INFINITY;
     const int64_t nv = n_chunk / VEC;              // (VEC = 4 only when n_chunk is a multiple of 4)
@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(kThreads) chunk_range_finalize_kernel(const fl
                                                                         int blocks_per_chunk, float2 *__restrict__ per_chunk,
                                                                         qbp_qparams *__restrict__ out)
 {
-    pdl_enter();
+    pdl_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int k = warp; k < chunks; k += kThreads / 32) {
         float lo = INFINITY, hi = -INFINITY;
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kThreads) chunk_range_finalize_kernel(const fl
 __global__ void qparams_from_range_kernel(const qbp_qparams *__restrict__ in, int count, int bits,
                                           qbp_qparams *__restrict__ out)
 {
-    pdl_enter();
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < count) out[i] = make_qparams(in[i].vmin, in[i].vmax, bits);
 }
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kScanThreads) chan_range_partial_kernel(const 
                                                                           int C, int tw, float *__restrict__ part_lo,
                                                                           float *__restrict__ part_hi)
 {
-    pdl_enter();
+    pdl_wait();
     const ScanPos p = scan_pos<VEC>(C, tw);
     const int rpb = kScanThreads / tw;
     float lo[VEC], hi[VEC];
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kThreads) chan_range_finalize_kernel(const flo
                                                                        const float *__restrict__ part_hi, int nparts,
                                                                        int C, int bits, qbp_qparams *__restrict__ qp)
 {
-    pdl_enter();
+    pdl_wait();
     int c = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
     if (c >= C) return;
     float lo = INFINITY, hi = -INFINITY;
@@ -515,7 +515,7 @@ __device__ __forceinline__ void quantize_body(const QuantJob &J, const PhiloxKey
 template <bool SR, int VEC, bool PERCH, bool TOTALS, bool J32>
 __global__ void __launch_bounds__(kThreads, 4) quantize_kernel(const __grid_constant__ QuantJob J, const __grid_constant__ PhiloxKeys keys)
 {
-    pdl_enter();
+    pdl_wait();
     quantize_body<SR, VEC, PERCH, TOTALS, J32>(J, keys, (int)blockIdx.x, (int)gridDim.x);
 }
 
@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(kThreads, 4) quantize_kernel(const __grid_cons
 template <bool ONE>
 __global__ void __launch_bounds__(kThreads, 4) bifurcate_kernel(const __grid_constant__ QuantJob J, const __grid_constant__ PhiloxKeys keys)
 {
-    pdl_enter();
+    pdl_wait();
     QParamsReg p8 = {0, 0}, p16 = {0, 0};
     resolve_range(J.r, true, true, blockIdx.x == 0, p8, p16);
     const QParamsReg t8 = p8, t16 = p16;
@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(kThreads, 4) bifurcate_kernel(const __grid_con
 template <bool TOTALS>
 __global__ void __launch_bounds__(kThreads) quantize_pair_kernel(const __grid_constant__ QuantJob a, const __grid_constant__ QuantJob b, int b_blocks)
 {
-    pdl_enter();
+    pdl_wait();
     const PhiloxKeys none = {};
     if ((int)blockIdx.x < b_blocks) quantize_body<false, 4, false, false, false>(b, none, (int)blockIdx.x, b_blocks);
     else                            quantize_body<false, 4, false, TOTALS, false>(a, none, (int)blockIdx.x - b_blocks, (int)gridDim.x - b_blocks);
@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(kThreads) quantize_pair_kernel(const __grid_co
 // The sums of up to eight code tensors in a launch of their own (see qbp_sums.cuh).
 __global__ void __launch_bounds__(kSumThreads) code_sums_kernel(const __grid_constant__ SumJobs J)
 {
-    pdl_enter();
+    pdl_wait();
     run_zero_jobs(J.zero, (int64_t)blockIdx.x * kSumThreads + threadIdx.x, (int64_t)gridDim.x * kSumThreads);
     code_sums_block(J, (int)blockIdx.x);
 }
@@ -1100,7 +1100,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_bifurcate(const float 
 __global__ void qparams_pair_from_range_kernel(const qbp_qparams *__restrict__ in, qbp_qparams *__restrict__ qp8,
                                                qbp_qparams *__restrict__ qp16)
 {
-    pdl_enter();
+    pdl_wait();
     *qp8 = make_qparams(in->vmin, in->vmax, 8);
     *qp16 = make_qparams(in->vmin, in->vmax, 16);
 }
@@ -1130,7 +1130,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_bifurcate_shard(const 
 __global__ void dequant_s64_kernel(const long long *__restrict__ acc, int64_t n, const qbp_qparams *qa,
                                    const qbp_qparams *qb, float *__restrict__ out)
 {
-    pdl_enter();
+    pdl_wait();
     const float s = __fmul_rn(qa->scale, qb->scale);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         out[i] = __fmul_rn((float)acc[i], s);
@@ -1159,7 +1159,7 @@ struct SgdTensor { float *w; const float *dw; float *v; int64_t n; float wd; int
 struct SgdTensors { SgdTensor t[kSgdTensors]; int count; };
 __global__ void __launch_bounds__(256) sgd_update_kernel(const __grid_constant__ SgdTensors J, float lr, float mu)
 {
-    pdl_enter();
+    pdl_wait();
     int k = 0;
     while (k + 1 < J.count && (int)blockIdx.x >= J.t[k + 1].first_block) ++k;
     const SgdTensor &T = J.t[k];

@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_stats_kernel(const float *__r
                                                                 float *__restrict__ part_lo, float *__restrict__ part_hi,
                                                                 double *__restrict__ part_sum)
 {
-    pdl_enter();
+    pdl_wait();
     const ScanPos p = scan_pos<VEC>(C, tw);
     const int rpb = kScanThreads / tw;
     float lo[VEC], hi[VEC];
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(128) bn_stats_finalize_kernel(const float *__r
                                                                 float *__restrict__ vmin, float *__restrict__ vmax,
                                                                 double *__restrict__ sum_out)
 {
-    pdl_enter();
+    pdl_wait();
     const int c = blockIdx.x;
     float lo = INFINITY, hi = -INFINITY;
     double sum = 0.0;
@@ -114,7 +114,7 @@ __global__ void bn_mean_from_sum_kernel(const double *__restrict__ col_sum, cons
                                         const float *__restrict__ col_max, int C, int64_t n, float *__restrict__ mean,
                                         float *__restrict__ vmin, float *__restrict__ vmax)
 {
-    pdl_enter();
+    pdl_wait();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= C) return;
     mean[c] = (float)(col_sum[c] / (double)n);
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_apply_kernel(const float *__r
                                                                 const float *__restrict__ beta, float Cn,
                                                                 float *__restrict__ y, BnRequant R, int reverse)
 {
-    pdl_enter();
+    pdl_wait();
     const ScanPos p = scan_pos<VEC>(C, tw);
     float inv = 0.0f, zp_u = 0.0f;
     if (REQUANT) {
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(256) bn_out_range_kernel(const float *__restri
                                                            qbp_qparams *__restrict__ out, qbp_qparams *__restrict__ qp8_out,
                                                            float4 *__restrict__ fold)
 {
-    pdl_enter();
+    pdl_wait();
     const float2 t = bn_out_extremes(mean, vmin, vmax, gamma, beta, C, Cn, relu != 0, (int)threadIdx.x, 256, fold);
     const float2 r = block_min_max(t.x, t.y);
     if (threadIdx.x == 0) {
@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_stats_kernel(const float 
                                                                     double *__restrict__ part_dyx,
                                                                     float *__restrict__ ext, const ZeroJobs zero, int64_t keep_from)
 {
-    pdl_enter();
+    pdl_wait();
     if (EXT)
         run_zero_jobs(zero, ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kScanThreads + threadIdx.x,
                       (int64_t)gridDim.x * gridDim.y * kScanThreads);
@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(kFinThreads) bn_bwd_finalize_kernel(const doub
                                                               float2 *__restrict__ relu_thr = nullptr,
                                                               const __grid_constant__ SumJobs J = SumJobs{})
 {
-    pdl_enter();
+    pdl_wait();
     const int c = blockIdx.x;
     // (the blocks behind the channels take code sums that a later product needs: C short blocks leave most SMs idle)
     if (c >= C) { code_sums_block(J, c - C); return; }
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(kScanThreads, kBabBlocks) bn_bwd_apply_bifurca
     uint32_t *__restrict__ q8, uint32_t *__restrict__ q_hi, uint32_t *__restrict__ q_lo, uint32_t lo_flip,
     int32_t *__restrict__ rowsum8, unsigned long long *__restrict__ chansum16, const float2 *__restrict__ relu_thr)
 {
-    pdl_enter();
+    pdl_wait();
     const ScanPos p = scan_pos<4>(C, tw);
     int cs16[4] = {0, 0, 0, 0};                   // stored codes of this thread's rows (fewer than 65536 rows)
     // the channels' constants in shared memory, read again for every step: held in registers (28 of them) they would cost the
@@ -731,7 +731,7 @@ __global__ void bn_bwd_coef_kernel(const double *__restrict__ sum_dy, const doub
                                    const float *__restrict__ gamma, double Cn, float *__restrict__ dgamma,
                                    float *__restrict__ dbeta, float2 *__restrict__ coef)
 {
-    pdl_enter();
+    pdl_wait();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= C) return;
     const double a = sum_dy[c], b = sum_dyx[c];
@@ -755,7 +755,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_apply_kernel(const float 
                                                                     float *__restrict__ dx,
                                                                     float2 *__restrict__ range_parts)
 {
-    pdl_enter();
+    pdl_wait();
     const ScanPos p = scan_pos<VEC>(C, tw);
     float rlo = INFINITY, rhi = -INFINITY;
     if (p.active) {
@@ -877,7 +877,7 @@ __global__ void __launch_bounds__(kFewThreads) bn_fwd_few_kernel(const float *__
                                                                  const float *__restrict__ beta, int relu, float Cn, float *__restrict__ y,
                                                                  float *__restrict__ mean, float *__restrict__ vmin, float *__restrict__ vmax)
 {
-    pdl_enter();
+    pdl_wait();
     const int col = (int)blockIdx.x * 16 + (threadIdx.x & 3) * 4, ty = threadIdx.x >> 2;
     const bool active = col < C;
     float4 v[ROWS];
@@ -931,7 +931,7 @@ __global__ void __launch_bounds__(kFewThreads) bn_bwd_few_kernel(const float *__
                                                                  const float *__restrict__ beta, int relu, float Cn, double Cnd,
                                                                  const BnBwdOut out, const ZeroJobs zero, const __grid_constant__ SumJobs J)
 {
-    pdl_enter();
+    pdl_wait();
     const int blocks = (C + 15) / 16;
     if ((int)blockIdx.x >= blocks) {
         if (threadIdx.x < kSumThreads) code_sums_block(J, (int)blockIdx.x - blocks);

@@ -21,7 +21,7 @@ template <int VEC>
 __global__ void __launch_bounds__(kTbpThreads) binarize_kernel(const float *__restrict__ x, int64_t n, int8_t *__restrict__ q,
                                                                qbp_qparams *__restrict__ qp_out)
 {
-    pdl_enter();
+    pdl_wait();
     if (qp_out && blockIdx.x == 0 && threadIdx.x == 0) {
         qbp_qparams r; r.scale = 1.0f; r.zero_point = 0; r.vmin = -1.0f; r.vmax = 1.0f;
         *qp_out = r;
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kTbpThreads) stc_ternarize_kernel(const float 
                                                                     int8_t *__restrict__ q, int8_t *__restrict__ hi,
                                                                     uint8_t *__restrict__ lo, qbp_qparams *__restrict__ qp_out)
 {
-    pdl_enter();
+    pdl_wait();
     const float2 rng = block_range(parts, nparts);          // (an empty tensor: s = 0)
     const float s = fmaxf(-fminf(rng.x, 0.0f), fmaxf(rng.y, 0.0f));
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -160,7 +160,7 @@ static int stc_ternarize_impl(const float *g, int64_t n, int samples, uint64_t s
 __global__ void __launch_bounds__(256) pack_bits_kernel(const int8_t *__restrict__ codes, int64_t rows, int64_t cols, int mask,
                                                         uint32_t *__restrict__ words)
 {
-    pdl_enter();
+    pdl_wait();
     const int64_t wpr = (cols + 31) / 32;
     const int lane = threadIdx.x & 31;
     for (int64_t word = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); word < rows * wpr; word += (int64_t)gridDim.x * 8) {
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(256) xnor_gemm_bits_kernel(int M, int N, int K
                                                              const uint32_t *__restrict__ S, const uint32_t *__restrict__ B,
                                                              int32_t *__restrict__ C)
 {
-    pdl_enter();
+    pdl_wait();
     __shared__ uint32_t sA[64][33], sB[64][33], sS[GATED ? 64 : 1][33];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;

@@ -363,7 +363,6 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    pdl_trigger();                       // (tensor memory is allocated)
     // (each role waits for the kernels before at its first use of their results: what it needs of the launch's parameters, and the
     // code up to there, has then been fetched)
     const uint32_t tmem_base = tmem_slot;
@@ -550,7 +549,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
 // element's partials are few hundred bytes each, far apart: one thread walking them alone is bound by latency).
 __global__ void __launch_bounds__(256) wgrad_finalize_kernel(const __grid_constant__ WgradParams P, int64_t total)
 {
-    pdl_enter();
+    pdl_wait();
     constexpr int kLanes = kWgFinalizeLanes;
     const int64_t e_raw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kLanes;
     const int part_lane = threadIdx.x % kLanes;
@@ -614,7 +613,7 @@ __device__ __forceinline__ long long wg_tap_part(const WgradParams &P, bool of_x
 template <int NB>
 __global__ void __launch_bounds__(256) wgrad_conv_finalize_kernel(const __grid_constant__ WgradParams P)
 {
-    pdl_enter();
+    pdl_wait();
     constexpr int U = 8 / NB;                              // slices in flight per output channel
     __shared__ long long s_part[NB][4][64], s_sx[4][64], s_sg[4][NB];
     const int cblocks = (P.C + 63) / 64;

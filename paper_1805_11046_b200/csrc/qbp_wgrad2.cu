@@ -152,7 +152,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
     __syncthreads();
     w2_cluster_sync();                   // both CTAs' barriers are initialised before either signals the other
     tc_fence_after();
-    pdl_trigger();                       // (tensor memory is allocated, in both CTAs)
     // (each role waits for the kernels before at its first use of their results: what it needs of the launch's parameters, and the
     // code up to there, has then been fetched)
     const uint32_t tmem_base = tmem_slot;
