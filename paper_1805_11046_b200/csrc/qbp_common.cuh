@@ -41,9 +41,10 @@ void trace_end(const char *name, cudaStream_t st);
 // Kernels of one stream run one after another, but a kernel's launch need not wait until the one before has been retired:
 // launch() marks every kernel as a programmatic dependent of its predecessor, whose blocks let it go as they exit, and each kernel
 // waits, before it touches the predecessor's results, until those are visible (pdl_wait).  A chain of dependent small kernels then
-// costs about 2 us each instead of 4 to 5.  No kernel lets its successor go earlier: blocks that wait on an SM beside the running
-// kernel made that kernel slower (per-channel statistics of 51 MB 14.5 -> 20 us, the layer of 56 x 56 x 64 543 -> 577 us, three
-// layers' inference at batch 8 105.6 -> 117 us).  While launches are timed one by one the dependency is the ordinary one.
+// costs about 2 us each instead of 4 to 5.  Only the short kernels whose successor is a product (code sums and zero-point terms) let
+// it go at their start (pdl_trigger), so that it allocates its tensor memory beside them (ternary layer 212 -> 206 us, layer
+// 14 x 14 x 256 255 -> 251): elsewhere blocks that wait on an SM beside the running kernel made that kernel slower (per-channel
+// statistics of 51 MB 14.5 -> 20 us, the layer of 56 x 56 x 64 543 -> 577 us, three layers' inference at batch 8 106 -> 117 us).  While launches are timed one by one the dependency is the ordinary one.
 bool trace_is_on();
 template <typename... P, typename... A>
 inline void launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A &&...args)
@@ -112,6 +113,7 @@ struct ZeroJobs { uint32_t *p[2]; int64_t words[2]; };
 
 // The two halves of a programmatic launch (see launch()).  A kernel that allocates tensor memory triggers only once it
 // has it: its successor could otherwise take it first and then wait for a kernel that cannot go on.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Philox4x32-10 (Salmon et al., SC'11): ten rounds of two 32x32->64 multiplies

@@ -869,6 +869,7 @@ struct ConvTerms {
 // The first `sum_blocks` blocks take code sums that a later product needs (a launch less, and they overlap).
 __global__ void __launch_bounds__(256, 6) conv_terms_kernel(const __grid_constant__ ConvTerms T, const __grid_constant__ SumJobs J, int sum_blocks)
 {
+    pdl_trigger();                       // (see launch())
     pdl_wait();
     if ((int)blockIdx.x < sum_blocks) { code_sums_block(J, (int)blockIdx.x); return; }
     const int block = (int)blockIdx.x - sum_blocks;

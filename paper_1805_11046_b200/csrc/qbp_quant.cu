@@ -575,6 +575,7 @@ __global__ void __launch_bounds__(kThreads) quantize_pair_kernel(const __grid_co
 // The sums of up to eight code tensors in a launch of their own (see qbp_sums.cuh).
 __global__ void __launch_bounds__(kSumThreads) code_sums_kernel(const __grid_constant__ SumJobs J)
 {
+    pdl_trigger();                       // (see launch())
     pdl_wait();
     run_zero_jobs(J.zero, (int64_t)blockIdx.x * kSumThreads + threadIdx.x, (int64_t)gridDim.x * kSumThreads);
     code_sums_block(J, (int)blockIdx.x);
