@@ -441,10 +441,12 @@ __device__ __forceinline__ void bn_bwd_channel(int c, double sdy, double sdyx, i
     if (o.relu_thr) o.relu_thr[c] = relu_threshold(mu, s, g, b);
 }
 
-constexpr int kFinThreads = kSumThreads;
-// One block of kFinThreads threads per channel: dbeta, dgamma, and the two per-channel
+// One block of T threads per channel: kSumThreads, or, when there are no code sums to take, as few as have every partial in flight
+// at once, two per thread (statistics and this of 25.7 M elements in 2048 channels of 37 partials 44.3 -> 38.6 us with 64, of 6.4 M
+// in 512 channels of 148 17.0 -> 15.3 with 128; 128 channels of 296 37.3 with 128, 36.6 with 256): dbeta, dgamma, and the two per-channel
 // constants of dx: m1 = gamma*dbeta/n, k2 = C(n)*gamma*dgamma.
-__global__ void __launch_bounds__(kFinThreads) bn_bwd_finalize_kernel(const double *__restrict__ part_dy,
+template <int T>
+__global__ void __launch_bounds__(T) bn_bwd_finalize_kernel(const double *__restrict__ part_dy,
                                                               const double *__restrict__ part_dyx, int nparts, int C,
                                                               int64_t n, const float *__restrict__ gamma, double Cn,
                                                               float *__restrict__ dgamma, float *__restrict__ dbeta,
@@ -462,21 +464,21 @@ __global__ void __launch_bounds__(kFinThreads) bn_bwd_finalize_kernel(const doub
     pdl_wait();
     const int c = blockIdx.x;
     // (the blocks behind the channels take code sums that a later product needs: C short blocks leave most SMs idle)
-    if (c >= C) { code_sums_block(J, c - C); return; }
+    if (T == kSumThreads && c >= C) { code_sums_block(J, c - C); return; }
     double a = 0.0, b = 0.0;
     // ext (see bn_bwd_stats_kernel): the extremes of dy over the three sets of positions, then (below) the exact range
     // of this channel's dx, left in chan_range[c] for the quantiser of the gradient
     float ev[6];
-    __shared__ float s_e[6][kFinThreads / 32];
+    __shared__ float s_e[6][T / 32];
 #pragma unroll
     for (int k = 0; k < 6; ++k) ev[k] = (k & 1) ? -INFINITY : INFINITY;
     // (all loads of two partials at once: the whole table in one round trip for up to two blocks per SM)
-    for (int i0 = threadIdx.x; i0 < nparts; i0 += 2 * kFinThreads) {
+    for (int i0 = threadIdx.x; i0 < nparts; i0 += 2 * T) {
         double pa_[2], pb_[2];
         float o[2][6];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const int i = i0 + u * kFinThreads;
+            const int i = i0 + u * T;
             const bool ok = i < nparts;
             pa_[u] = ok ? part_dy[(int64_t)i * C + c] : 0.0; pb_[u] = ok ? part_dyx[(int64_t)i * C + c] : 0.0;
 #pragma unroll
@@ -501,11 +503,11 @@ __global__ void __launch_bounds__(kFinThreads) bn_bwd_finalize_kernel(const doub
         a += __shfl_xor_sync(0xffffffffu, a, o);
         b += __shfl_xor_sync(0xffffffffu, b, o);
     }
-    __shared__ double s_a[kFinThreads / 32], s_b[kFinThreads / 32];
+    __shared__ double s_a[T / 32], s_b[T / 32];
     if ((threadIdx.x & 31) == 0) { s_a[threadIdx.x >> 5] = a; s_b[threadIdx.x >> 5] = b; }
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < kFinThreads / 32; ++w) { a += s_a[w]; b += s_b[w]; }
+        for (int w = 1; w < T / 32; ++w) { a += s_a[w]; b += s_b[w]; }
         if (sum_dy) {                       // raw sums only: combined over several GPUs before the coefficients
             sum_dy[c] = a; sum_dyx[c] = b;
             return;
@@ -514,7 +516,7 @@ __global__ void __launch_bounds__(kFinThreads) bn_bwd_finalize_kernel(const doub
         if (ext) {
 #pragma unroll
             for (int k = 0; k < 6; ++k)
-                for (int w = 1; w < kFinThreads / 32; ++w) ev[k] = (k & 1) ? fmaxf(ev[k], s_e[k][w]) : fminf(ev[k], s_e[k][w]);
+                for (int w = 1; w < T / 32; ++w) ev[k] = (k & 1) ? fmaxf(ev[k], s_e[k][w]) : fminf(ev[k], s_e[k][w]);
         }
         bn_bwd_channel(c, a, b, n, Cn, gamma ? gamma[c] : 1.0f, beta ? beta[c] : 0.0f, ext ? mean[c] : 0.0f, ext ? vmin[c] : 0.0f,
                        ext ? vmax[c] : 0.0f, Cn_f, ext ? ev : nullptr, o);
@@ -1264,8 +1266,9 @@ static int bn_bwd_stats_launch(const float *dy, const float *x, int64_t n_rows, 
     SumJobs J{};
     int sum_blocks = 0;
     if (extra_count) if (int rc = fill_sum_jobs(extra, extra_count, J, &sum_blocks)) return rc;
-    launch(bn_bwd_finalize_kernel, (int)C + sum_blocks, kFinThreads, 0, st, pa, pb, g.nbx, (int)C, n_stat, gamma, Cnd, dgamma, dbeta, coef, sum_dy, sum_dyx,
-                                                   ext, save_min, save_max, Cn, chan_range, save_mean, beta, relu_thr, J);
+#define QBP_BN_BFIN(T) launch(bn_bwd_finalize_kernel<T>, (int)C + sum_blocks, T, 0, st, pa, pb, g.nbx, (int)C, n_stat, gamma, Cnd, dgamma, dbeta, coef, sum_dy, sum_dyx, ext, save_min, save_max, Cn, chan_range, save_mean, beta, relu_thr, J)
+    if (sum_blocks || g.nbx > 256) QBP_BN_BFIN(kSumThreads); else if (g.nbx > 128) QBP_BN_BFIN(128); else QBP_BN_BFIN(64);
+#undef QBP_BN_BFIN
     QBP_LAUNCH_OK("bn_bwd_finalize_kernel");
     return QBP_OK;
 }
