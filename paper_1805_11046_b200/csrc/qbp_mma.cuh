@@ -41,7 +41,6 @@ enum { kSumRows = 0, kSumCols = 1, kSumEdges = 2 };
 struct SumJob { const void *q; int64_t rows, cols; int kind, is_signed; int32_t *out; int H = 0, W = 0; int64_t *out64 = nullptr; };
 constexpr int kMaxSumJobs = 8;
 int sum_pieces(int64_t rows, int64_t cols);
-int edge_pieces(int64_t rows, int H, int W);
 inline size_t sum_elems(int64_t rows, int64_t cols, int kind)
 {
     return kind == kSumRows ? (size_t)rows : kind == kSumCols ? (size_t)sum_pieces(rows, cols) * (size_t)cols : 8 * (size_t)cols;
