@@ -280,9 +280,10 @@ __global__ void __launch_bounds__(256) bn_out_range_kernel(const float *__restri
 // channel's maximum, where it is its minimum, and everywhere else -- as ext [6][blocks][C] (min, max of the ordinary
 // positions, then of the maxima, then of the minima).  dx is a monotone function of dy on each set (bn_dx), so the
 // finalize kernel knows the exact range of dx from these, before dx is computed.
-// The last kKeepBytes of both tensors are read with loads that leave them in the L2 (the rest passes through, evict-first): the
-// bifurcating pass that follows walks from the end (25.7 M elements of 128 channels with g kept: 74 -> 68 us there, +2 here
-// with 72 MB, nothing with 48; more than the L2 holds beside the writes only costs).
+// The last kKeepBytes of both tensors are read with loads that leave them in the L2 (the rest passes through, evict-first) when the
+// second pass is bound by HBM, which then starts with them: the plain one (51 MB: 33 -> 31 us) and the bifurcating one that also
+// writes the gradient (25.7 M elements 74 -> 68 us).  The bifurcating pass alone is bound by arithmetic and gains nothing (the layers of
+// 56 x 56 x 64 and 14 x 14 x 256 lose a microsecond).  More than the L2 holds beside the writes (88 MB) only costs.
 constexpr int64_t kKeepBytes = 64ll << 20;
 template <int VEC, bool RELU, bool EXT>
 __global__ void __launch_bounds__(kScanThreads) bn_bwd_stats_kernel(const float *__restrict__ dy,
@@ -1241,7 +1242,7 @@ static int bn_bwd_stats_launch(const float *dy, const float *x, int64_t n_rows, 
                                const float *save_max, float *dgamma, float *dbeta, float2 *coef, double *sum_dy,
                                double *sum_dyx, double *pa, double *pb, cudaStream_t st, float *ext = nullptr,
                                float2 *chan_range = nullptr, float2 *relu_thr = nullptr, const ZeroJobs &zero = ZeroJobs{},
-                               const SumJob *extra = nullptr, int extra_count = 0)
+                               const SumJob *extra = nullptr, int extra_count = 0, bool keep_tail = true)
 {
     const bool al = aligned16(x) && aligned16(dy);
     const bool v4 = al && C % 4 == 0;
@@ -1252,7 +1253,7 @@ static int bn_bwd_stats_launch(const float *dy, const float *x, int64_t n_rows, 
     const dim3 grid(g.nbx, g.slabs);
     const double Cnd = 1.0 / std::sqrt(2.0 * std::log((double)n_stat));
     const float Cn = (float)Cnd;
-    const int64_t keep_from = std::max<int64_t>(0, n_rows - kKeepBytes / (2 * (int64_t)sizeof(float) * C));
+    const int64_t keep_from = keep_tail ? std::max<int64_t>(0, n_rows - kKeepBytes / (2 * (int64_t)sizeof(float) * C)) : n_rows;
     QBP_TRACE_BEGIN(st);
 #define QBP_BN_BSTATS(V, R, E) launch(bn_bwd_stats_kernel<V, R, E>, grid, kScanThreads, 0, st, dy, x, n_rows, (int)C, g.tw, save_mean, save_min, save_max, gamma, beta, Cn, pa, pb, ext, zero, keep_from)
     if (ext) {
@@ -1347,7 +1348,7 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
                                  BnBwdOut{dgamma, dbeta, coef, chan_range, relu ? relu_thr : nullptr}, zero, extra, extra_count, st)))
             return rc;
     } else if ((rc = bn_bwd_stats_launch(dy, x, n, n, C, gamma, beta, relu, save_mean, save_min, save_max, dgamma, dbeta, coef, nullptr,
-                                  nullptr, pa, pb, st, ext, chan_range, relu ? relu_thr : nullptr, zero, extra, extra_count)))
+                                  nullptr, pa, pb, st, ext, chan_range, relu ? relu_thr : nullptr, zero, extra, extra_count, g_out != nullptr)))
         return rc;
     const RangeSrc range{chan_range, (int)C, nullptr, qp8, qp16};
     const dim3 grid(ga.nbx, ga.slabs);
