@@ -253,6 +253,9 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_bwd(const qbp_la
     if (!saved || !dy || !dx || !dw) return fail(QBP_ERR_INVALID_ARG, "layer_bwd: NULL argument");
     if (!saved->g8 || !saved->qg8 || !saved->g_hi || !saved->g_lo || !saved->qg16 || !saved->z)
         return fail(QBP_ERR_INVALID_ARG, "layer_bwd: the saved-state record has a NULL buffer (the backward pass needs z and the gradient buffers)");
+    // (the forward's codes are summed up beside the first pass, and its statistics are read there)
+    if (!saved->x_codes || !saved->qx || !saved->w_codes || !saved->qw || !saved->save_mean || !saved->save_min || !saved->save_max)
+        return fail(QBP_ERR_INVALID_ARG, "layer_bwd: the saved-state record has a NULL buffer (codes, parameters or statistics of the forward)");
     float *g = saved->g;
     int8_t *g8 = saved->g8, *ghi = saved->g_hi;
     uint8_t *glo = saved->g_lo;

@@ -109,6 +109,18 @@ def test_epilogue_statistics_need_all_three_buffers_the_output_and_few_columns(l
                            C.c_size_t(1 << 30), null) == -1              # requantisation without clamping values
 
 
+@pytest.mark.parametrize("conv", [False, True])
+@pytest.mark.parametrize("missing", ["x_codes", "qx", "w_codes", "qw", "save_mean", "save_min", "save_max", "z", "g8", "qg8", "g_hi", "g_lo", "qg16"])
+def test_layer_backward_refuses_a_record_with_a_missing_buffer(lib, conv, missing):
+    """Before anything is launched: the first launches of the backward already read the forward's codes and statistics."""
+    from paper_1805_11046_b200.binding import ConvDesc, LayerCtx, LayerDesc
+    fake = C.c_void_p(4096); null = C.c_void_p(0)
+    L = LayerDesc(conv=ConvDesc(1, 8, 8, 32, 32, 3, 3, 1, 1)) if conv else LayerDesc(batch=64, in_features=32, out_features=32)
+    ctx = LayerCtx(**{f: None if f in (missing, "g", "x_chan_sums") else 4096 for f, _ in LayerCtx._fields_})
+    assert lib.qbp_layer_bwd(C.byref(L), C.byref(ctx), fake, null, null, fake, fake, fake, fake, fake, C.c_size_t(1 << 40), null) == -1
+    assert "NULL buffer" in _err(lib)
+
+
 def test_workspace_queries_are_pure(lib):
     for name in ("qbp_quantize_workspace_bytes", "qbp_gemm_s8_workspace_bytes", "qbp_rangebn_workspace_bytes"):
         getattr(lib, name).restype = C.c_size_t
