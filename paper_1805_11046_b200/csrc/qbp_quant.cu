@@ -591,7 +591,7 @@ int sum_pieces(int64_t rows, int64_t cols)
     return (int)std::max<int64_t>(p, (rows >> 22) + 1);
 }
 
-// The same for the edges of N images (always added up by atomics): some 256 positions of the longest edge each, at most 64; of
+// The same for the long edges of N images (always added up by atomics): some 256 positions of the longest edge each, at most 64; of
 // short edges up to four, as long as a block of `high` rows has all of its piece in flight at once.  (256 images of 56 x 56: with
 // 16 pieces of 896 positions the layer took 530 us, with 56 526; of 14 x 14, 256 channels: 14 pieces 250.5, 28 of them 254.)
 static int edge_pieces(int64_t rows, int H, int W, int high)
@@ -599,6 +599,11 @@ static int edge_pieces(int64_t rows, int H, int W, int high)
     const int64_t longest = rows / ((int64_t)H * W) * std::max(H, W);
     const int64_t p = std::max<int64_t>(std::min<int64_t>(64, longest / 256), std::min<int64_t>(4, longest / (4 * high)));
     return (int)std::max<int64_t>(std::max<int64_t>(1, p), (longest >> 22) + 1);
+}
+// ... and for their corners: one position per image.
+static int corner_pieces(int64_t images)
+{
+    return (int)std::max<int64_t>(std::max<int64_t>(1, std::min<int64_t>(64, images / 256)), (images >> 22) + 1);
 }
 
 int fill_sum_jobs(const SumJob *jobs, int count, SumJobs &J, int *blocks)
@@ -613,7 +618,7 @@ int fill_sum_jobs(const SumJob *jobs, int count, SumJobs &J, int *blocks)
         if (s.cols % 16 || !aligned16(s.q)) return fail(QBP_ERR_INVALID_ARG, "code sums need 16-byte aligned rows (cols %% 16 == 0)");
         SumJobDev &j = J.j[i];
         j.q = static_cast<const uint8_t *>(s.q); j.rows = s.rows; j.cols = (int)s.cols; j.kind = s.kind; j.out = s.out; j.out64 = s.out64;
-        j.flip = s.is_signed ? 0u : 0x80808080u; j.first = first; j.G = 1; j.pieces = 1; j.H = s.H; j.W = s.W;
+        j.flip = s.is_signed ? 0u : 0x80808080u; j.first = first; j.G = 1; j.pieces = j.corner_pieces = 1; j.H = s.H; j.W = s.W;
         while ((16 << j.lg_log2) < s.cols && j.lg_log2 < 3) ++j.lg_log2;
         const int strips = (int)((s.cols / 16 + (1 << j.lg_log2) - 1) >> j.lg_log2);
         if (s.kind == kSumRows) {
@@ -625,7 +630,8 @@ int fill_sum_jobs(const SumJob *jobs, int count, SumJobs &J, int *blocks)
             // added up by atomics, nobody reads the pieces one by one: as many blocks as the rows give work to (the sums of
             // 200704 x 128 codes with 16 pieces: 31 us, now 16)
             if (s.out64 && s.kind == kSumCols) j.pieces = (int)std::max<int64_t>(j.pieces, std::min<int64_t>(4ll * sm_count() / strips, s.rows / 128));
-            j.blocks = strips * (s.kind == kSumCols ? j.pieces : 4 * j.pieces + 4);
+            if (s.kind == kSumEdges) j.corner_pieces = corner_pieces(s.rows / ((int64_t)s.H * s.W));
+            j.blocks = strips * (s.kind == kSumCols ? j.pieces : 4 * (j.pieces + j.corner_pieces));
         }
         first += j.blocks;
     }

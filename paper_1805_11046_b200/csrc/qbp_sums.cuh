@@ -8,7 +8,7 @@
 namespace qbp {
 
 constexpr int kSumThreads = 256;
-struct SumJobDev { const uint8_t *q; int64_t rows; int cols, kind, first, blocks, G, pieces, H, W, lg_log2; uint32_t flip; int32_t *out; int64_t *out64; };
+struct SumJobDev { const uint8_t *q; int64_t rows; int cols, kind, first, blocks, G, pieces, corner_pieces, H, W, lg_log2; uint32_t flip; int32_t *out; int64_t *out64; };
 struct SumJobs { SumJobDev j[kMaxSumJobs]; int count; ZeroJobs zero; };
 // The device form of `count` jobs; *blocks: the blocks they take.  (qbp_quant.cu)
 int fill_sum_jobs(const SumJob *jobs, int count, SumJobs &J, int *blocks);
@@ -59,10 +59,12 @@ __device__ __forceinline__ void code_sums_block(const SumJobs &J, int blk)
     // a strip is 16 * lg columns wide (lg = 8, or the channels' groups when they are fewer: no lane idles) and 256 / lg rows high
     __shared__ int s_acc[kSumThreads / 32][128];
     const int lg = 1 << j.lg_log2, strips = (cv + lg - 1) >> j.lg_log2, strip = bid % strips;
-    // (edges: the pieces of the four long ones, then the corners whole)
+    // (edges: the pieces of the four long ones, then those of the corners)
     const int unit = bid / strips, long_units = 4 * j.pieces;
-    const int edge = j.kind != kSumEdges ? 0 : unit < long_units ? unit % 4 : 4 + unit - long_units;
-    const int piece = j.kind != kSumEdges ? unit : unit < long_units ? unit / 4 : 0, pieces = edge < 4 ? j.pieces : 1;
+    const bool corner = j.kind == kSumEdges && unit >= long_units;
+    const int nth = corner ? unit - long_units : unit;
+    const int edge = j.kind != kSumEdges ? 0 : (corner ? 4 : 0) + nth % 4;
+    const int piece = j.kind != kSumEdges ? unit : nth / 4, pieces = corner ? j.corner_pieces : j.pieces;
     // an edge: `len` positions of every image, `step` apart, from `off`
     const int HW = j.H * j.W;
     const int len = edge < 2 ? j.W : edge < 4 ? j.H : 1, step = edge < 2 ? 1 : j.W;

@@ -470,6 +470,22 @@ def test_wgrad_conv_edge_sums(B, N, H, W, C, K):
     assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
 
 
+@pytest.mark.parametrize("side", [1, 2])
+def test_wgrad_conv_corner_sums_of_many_small_images(B, side):
+    """So many images that the low bytes of one corner alone add up to more than an int32 holds (255 * N > 2^31): constant
+    codes, whose accumulators are a count of positions times one product."""
+    import torch
+    N, C, zx, zg = (1 << 31) // 255 + 128, 32, -90, 2077
+    d = B.conv_desc(N, side, side, C, C, 3, 3, 1, 1)
+    code = lambda v, dt: torch.full((N, side, side, C), v, dtype=dt, device="cuda")
+    acc, _, ws = B.qbp_wgrad_s16(code(1, torch.int8), _qp(B, 0.5, zx), code(0, torch.int8), code(255, torch.uint8), _qp(B, 0.25, zg), d=d,
+                                 want_acc=True, want_out=False)
+    assert B.status_word(ws) == 0
+    seen = np.array([side - 1, side, side - 1], np.int64)          # rows (columns) that each tap row (column) sees
+    want = N * np.outer(seen, seen) * (1 - zx) * (255 - zg)
+    assert np.array_equal(to_host(acc), np.broadcast_to(want[None, :, :, None], (C, 3, 3, C)))
+
+
 # ------------------------------------------- 3x3 convolutions of many channels (CTA pairs)
 @pytest.mark.parametrize("N,H,W,C,K", [(1, 1, 1, 96, 96), (2, 5, 6, 96, 160), (3, 9, 7, 128, 256), (2, 14, 14, 288, 112), (1, 8, 16, 256, 400),
                                        (40, 28, 28, 128, 256), (90, 14, 14, 256, 512)])
