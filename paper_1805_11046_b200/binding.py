@@ -126,19 +126,29 @@ def _stream() -> C.c_void_p:
     return C.c_void_p(torch.cuda.current_stream().cuda_stream)
 
 
-_ws_cache: dict = {}
+class _Workspaces(threading.local):
+    """A host thread's default scratch buffers by (device, raw stream handle); given back when the thread ends."""
+
+    def __init__(self):
+        self.by_stream = {}
+
+
+_workspaces = _Workspaces()
 
 
 def workspace(nbytes: int, device=None) -> torch.Tensor:
-    """A cached device scratch buffer of at least nbytes (grown on demand, 256-byte aligned by torch); one per
-    device and host thread, since calls of different threads may interleave on a stream."""
+    """A cached device scratch buffer of at least nbytes (grown on demand, 256-byte aligned by torch) for the current
+    stream: one per device, stream and host thread.  Calls on different streams run at the same time, and calls of
+    different threads may interleave on one stream; both would overwrite each other's scratch.  A buffer that is outgrown
+    was allocated on the stream that used it, so the allocator hands its memory on in that stream's order.  (A captured
+    graph keeps the addresses of its calls: give those calls a `ws` of their own.)"""
     dev = None if device is None else torch.device(device)
     index = torch.cuda.current_device() if dev is None or dev.index is None else dev.index
-    key = (index, threading.get_ident())
-    t = _ws_cache.get(key)
+    key = (index, _stream().value)
+    t = _workspaces.by_stream.get(key)
     if t is None or t.numel() < nbytes:
         t = torch.empty(max(nbytes, 1 << 20), dtype=torch.uint8, device=torch.device("cuda", index))
-        _ws_cache[key] = t
+        _workspaces.by_stream[key] = t
     return t
 
 
