@@ -115,6 +115,15 @@ struct ZeroJobs { uint32_t *p[2]; int64_t words[2]; };
 // has it: its successor could otherwise take it first and then wait for a kernel that cannot go on.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A load of what a kernel that let this one go at its start writes (code sums, zero-point terms): an ordinary global load that
+// stays behind pdl_wait().  __ldg would take the non-coherent path, which is for memory that nothing writes while the reading
+// kernel is resident; everything else that a kernel reads was written by blocks that had ended before it started.
+__device__ __forceinline__ int32_t load_after_wait(const int32_t *p)
+{
+    int32_t v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
 
 // Philox4x32-10 (Salmon et al., SC'11): ten rounds of two 32x32->64 multiplies
 // (one wide multiply each); the round keys are key + r * (0x9E3779B9, 0xBB67AE85).

@@ -192,7 +192,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kC2Threads, 1) qbp_c
         C2Stat *my_stat = s_stat + (size_t)ew * hcols;
         for (int i = et; i < 16 * P.bn; i += 32 * kC2EpiWarps) {
             const int cls = i / P.bn, n = n0 + i - cls * P.bn;
-            s_cterm[i] = n < P.N ? __ldg(P.colterm + (int64_t)cls * P.N + n) : 0;
+            s_cterm[i] = n < P.N ? load_after_wait(P.colterm + (int64_t)cls * P.N + n) : 0;
         }
         if (P.st_sum)
             for (int i = lane; i < hcols; i += 32) { my_stat[i].sum = 0.0; my_stat[i].lo = INFINITY; my_stat[i].hi = -INFINITY; }
@@ -220,12 +220,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kC2Threads, 1) qbp_c
         const int c_begin = half * (hcols >> 5), c_end = min((ncol + 31) >> 5, (half + 1) * (hcols >> 5));
         uint32_t buf = 0, fph = 0;
         RowInfo ri = row_info(pair < P.tiles_total ? pair : 0);
-        int rterm = (pair < P.tiles_total && ri.valid) ? __ldg(P.rowterm + ri.m) : 0;
+        int rterm = (pair < P.tiles_total && ri.valid) ? load_after_wait(P.rowterm + ri.m) : 0;
         for (int tile = pair; tile < P.tiles_total; tile += P.pairs) {
             // the next tile's row term is fetched now, so that its latency hides behind this tile
             const int tile_next = tile + P.pairs;
             const RowInfo ri_next = row_info(tile_next < P.tiles_total ? tile_next : 0);
-            const int rterm_next = (tile_next < P.tiles_total && ri_next.valid) ? __ldg(P.rowterm + ri_next.m) : 0;
+            const int rterm_next = (tile_next < P.tiles_total && ri_next.valid) ? load_after_wait(P.rowterm + ri_next.m) : 0;
             const int32_t *cterm = s_cterm + ri.cls * P.bn;
             if (!timed_out && !mbar_wait_warp(&acc_full[buf], fph)) timed_out = true;
             if (!timed_out) {

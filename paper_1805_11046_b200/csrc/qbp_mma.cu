@@ -615,8 +615,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
         int32_t *region = s_cterm + (P.cterm_all || P.msub == 2 ? 0 : group * P.ncls * P.bn);
         int neg_za = 0, neg_zb = 0, k_zz = 0;
         if (RAW) { neg_za = -P.qa->zero_point; neg_zb = -P.qb->zero_point; k_zz = P.k_len * neg_za * neg_zb; }
-        auto row_term = [&](int64_t m) { return RAW ? neg_zb * (int)P.a_sums.at(m) + k_zz : __ldg(P.rowterm + m); };
-        auto col_term = [&](int64_t i) { return RAW ? neg_za * (int)P.b_sums.at(i) : __ldg(P.colterm + i); };
+        auto row_term = [&](int64_t m) { return RAW ? neg_zb * (int)P.a_sums.at(m) + k_zz : load_after_wait(P.rowterm + m); };
+        auto col_term = [&](int64_t i) { return RAW ? neg_za * (int)P.b_sums.at(i) : load_after_wait(P.colterm + i); };
         if (P.cterm_all || (TAIL && P.ep_fold)) {
             // the whole column-term table fits: fill it once (and the per-column constants of the normalisation)
             if (P.cterm_all)
@@ -898,18 +898,18 @@ __global__ void __launch_bounds__(256, 6) conv_terms_kernel(const __grid_constan
     const int m = img * T.HW + i;                            // (fewer than 2^31 positions)
     const bool up = p > 0, down = p + 1 < T.H, left = q > 0, right = q + 1 < T.W;
     const int32_t *c = T.chan_sum + m;
-    int box = __ldg(c);
-    if (left) box += __ldg(c - 1);
-    if (right) box += __ldg(c + 1);
+    int box = load_after_wait(c);
+    if (left) box += load_after_wait(c - 1);
+    if (right) box += load_after_wait(c + 1);
     if (up) {
-        box += __ldg(c - T.W);
-        if (left) box += __ldg(c - T.W - 1);
-        if (right) box += __ldg(c - T.W + 1);
+        box += load_after_wait(c - T.W);
+        if (left) box += load_after_wait(c - T.W - 1);
+        if (right) box += load_after_wait(c - T.W + 1);
     }
     if (down) {
-        box += __ldg(c + T.W);
-        if (left) box += __ldg(c + T.W - 1);
-        if (right) box += __ldg(c + T.W + 1);
+        box += load_after_wait(c + T.W);
+        if (left) box += load_after_wait(c + T.W - 1);
+        if (right) box += load_after_wait(c + T.W + 1);
     }
     const int taps = (1 + (up ? 1 : 0) + (down ? 1 : 0)) * (1 + (left ? 1 : 0) + (right ? 1 : 0));
     const int za = T.q_in->zero_point, zb = T.q_w->zero_point;

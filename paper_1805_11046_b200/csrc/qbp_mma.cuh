@@ -22,7 +22,7 @@ struct CodeSums {
     {
         long long s = 0;
 #pragma unroll 8
-        for (int k = 0; k < pieces; ++k) s += __ldg(p + (int64_t)k * stride + i);
+        for (int k = 0; k < pieces; ++k) s += load_after_wait(p + (int64_t)k * stride + i);
         return s;
     }
 #endif

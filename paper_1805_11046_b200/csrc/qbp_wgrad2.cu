@@ -233,7 +233,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
             for (int k = 0; k < P.shi.pieces; ++k) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    if ((half * 4 + i) * 32 + lane < ncol) ct[i] += 256 * (long long)__ldg(ph + 32 * i) + __ldg(pl + 32 * i);
+                    if ((half * 4 + i) * 32 + lane < ncol) ct[i] += 256 * (long long)load_after_wait(ph + 32 * i) + load_after_wait(pl + 32 * i);
                 ph += P.shi.stride; pl += P.slo.stride;
             }
 #pragma unroll

@@ -1,0 +1,61 @@
+"""What the kernels must keep to because each is launched as a programmatic dependent of the one before it (and may be resident
+while that one, or a caller's kernel, still runs): read from the sources, since a violation would be a race on the device."""
+import re
+from pathlib import Path
+
+CSRC = Path(__file__).resolve().parent.parent / "paper_1805_11046_b200" / "csrc"
+
+
+def _sources():
+    out = {}
+    for f in sorted(CSRC.glob("*.cu*")):
+        out[f.name] = re.sub(r"//[^\n]*", "", f.read_text())
+    return out
+
+
+def _body(text, at):
+    """The braces that open at or after `at`, with what is in them."""
+    start = text.index("{", at)
+    depth = 0
+    for i in range(start, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        if depth == 0:
+            return text[start:i + 1]
+    raise AssertionError("unbalanced braces")
+
+
+def _kernels():
+    out = {}
+    for name, text in _sources().items():
+        for m in re.finditer(r"__global__[^;{]*?\bvoid\b[^;{]*?(\w+_kernel)\s*\(", text):
+            i, depth = m.end(), 1                      # to the end of the parameter list (default arguments may hold braces)
+            while depth:
+                depth += {"(": 1, ")": -1}.get(text[i], 0)
+                i += 1
+            out[m.group(1)] = _body(text, i)
+    return out
+
+
+EARLY = {"code_sums_kernel", "conv_terms_kernel"}        # the kernels that let their successor go at their start
+
+
+def test_every_kernel_waits_for_the_one_before():
+    kernels = _kernels()
+    assert len(kernels) > 30
+    for name, body in kernels.items():
+        if name != "bounded_wait_selftest_kernel":       # (launched in the ordinary way)
+            assert "pdl_wait()" in body, name
+    assert {n for n, b in kernels.items() if "pdl_trigger()" in b} == EARLY
+    for name in EARLY:
+        assert "tmem_alloc" not in kernels[name]         # a successor could take the tensor memory it waits for
+
+
+def test_what_an_early_kernel_writes_is_read_by_ordinary_loads():
+    """Code sums and zero-point terms: their reader is resident while they are written, which the non-coherent path excludes."""
+    sources, kernels = _sources(), _kernels()
+    at = _body(sources["qbp_mma.cuh"], sources["qbp_mma.cuh"].index("long long at(int64_t i) const"))
+    assert "load_after_wait(" in at and "__ldg" not in at
+    assert "__ldg" not in kernels["conv_terms_kernel"]   # (reads the code sums of the launch before)
+    for name in ("qbp_mma_kernel", "qbp_conv2_kernel", "qbp_mma2_kernel", "qbp_wgrad_kernel", "qbp_wgrad2_kernel"):
+        for m in re.finditer(r"__ldg\(([^;]*);", kernels[name]):
+            assert m.group(1).startswith("P.ep_fold"), (name, m.group(0))      # (written by bn_out_range_kernel)
