@@ -179,6 +179,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kC2Threads, 1) qbp_c
             A.a_desc_lo = P.a_desc_lo; A.b_desc_lo = P.b_desc_lo; A.idesc = P.idesc; A.bn = (uint32_t)P.bn;
             A.k_iters = P.k_iters; A.stages = (uint32_t)P.stages; A.cg = (uint32_t)P.cg; A.nbuf = (uint32_t)P.nbuf;
             A.tile0 = pair; A.tiles_total = P.tiles_total; A.tile_step = P.pairs;
+            // (a barrier's wait is bounded: its clock starts once the producer's copies can)
+            pdl_wait();
             timed_out = !(!P.dgrad ? conv2_mma_loop<2, 128>(A) : P.bn == 256 ? conv2_mma_loop<256, 128>(A) : conv2_mma_loop<128, 64>(A));
         }
     } else {

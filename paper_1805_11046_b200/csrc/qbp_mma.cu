@@ -550,6 +550,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
         // ------------------------------------------------------ MMA issuer
         // The whole warp walks the tiles and stages in step, so that ring positions, descriptors and accumulator
         // addresses stay warp-uniform; an elected lane issues the MMAs and the commits.
+        // (a barrier's wait is bounded: its clock starts once the producer's copies can)
+        pdl_wait();
         if (P.b_resident && !mbar_wait_uniform(&b_full, 0)) timed_out = true;
         const uint32_t bres_addr = smem_u32(smem_b);
         const uint32_t ring_addr = smem_u32(smem);

@@ -192,6 +192,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
             A.k_iters = P.k_iters; A.stages = (uint32_t)P.stages; A.cg = (uint32_t)P.cg; A.nbuf = (uint32_t)P.nbuf;
             A.tile0 = pair; A.tiles_total = P.tiles_total; A.tile_step = P.pairs;
             bool ok;
+            // (a barrier's wait is bounded: its clock starts once the producer's copies can)
+            pdl_wait();
             if (P.msub == 2) {
                 if (P.a.major == 0) ok = P.b.major == 0 ? pair_mma_loop<2, 2, 2>(A) : pair_mma_loop<2, 256, 2>(A);
                 else                ok = P.b.major == 0 ? pair_mma_loop<256, 2, 2>(A) : pair_mma_loop<256, 256, 2>(A);

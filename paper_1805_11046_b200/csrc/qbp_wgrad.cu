@@ -411,6 +411,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
         A.ring = smem_u32(smem); A.stage_bytes = stage_bytes; A.a_bytes = a_bytes; A.tmem = tmem_base;
         A.k_iters = k_iters; A.stages = (uint32_t)stages; A.cg = (uint32_t)cg;
         A.a_desc_lo = P.a.desc_lo;
+        // (a barrier's wait is bounded: its clock starts once the producer's copies can)
+        pdl_wait();
         if (P.halo_bh) {
             // where each A tile's taps start in the halo tile (tap (r, s): r tile rows and s positions in)
             for (int j = 0; j < 4; ++j) {

@@ -186,6 +186,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
             uint32_t s = 0, ph = 0, in_group = 0, group = 0, eph = 1;
             const uint32_t ring = smem_u32(smem);
             uint32_t a_addr = ring;
+            // (a barrier's wait is bounded: its clock starts once the producer's copies can)
+            pdl_wait();
             for (int tile = pair; tile < P.tiles_total && !timed_out; tile += P.pairs) {
                 if (!mbar_wait_uniform(&acc_empty, eph)) { timed_out = true; break; }
                 eph ^= 1u;

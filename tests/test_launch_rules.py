@@ -59,3 +59,22 @@ def test_what_an_early_kernel_writes_is_read_by_ordinary_loads():
     for name in ("qbp_mma_kernel", "qbp_conv2_kernel", "qbp_mma2_kernel", "qbp_wgrad_kernel", "qbp_wgrad2_kernel"):
         for m in re.finditer(r"__ldg\(([^;]*);", kernels[name]):
             assert m.group(1).startswith("P.ep_fold"), (name, m.group(0))      # (written by bn_out_range_kernel)
+
+
+def test_no_bounded_wait_starts_its_clock_before_the_kernel_may_work():
+    """The waits on barriers give up after about a second.  Every role therefore waits for the kernels before this one, however
+    long those run, ahead of the first barrier that only completes once copies have been issued.  (The producer's first waits are
+    on stages that nothing has filled yet: they pass at once.)"""
+    sources = {f.name: f.read_text() for f in CSRC.glob("*.cu")}
+    seen = 0
+    for name, text in sources.items():
+        if "-- MMA issuer" not in text:
+            continue
+        issuer, epilogue = text.index("-- MMA issuer"), re.search(r"//\s-+ epilogue", text).start()
+        assert issuer < epilogue, name
+        waiting = r"mbar_wait|_mma_loop|mma_loop_|_dispatch"
+        for role in (text[issuer:epilogue], text[epilogue:]):
+            assert "pdl_wait();" in role, name
+            assert role.index("pdl_wait();") < re.search(waiting, role).start(), name
+        seen += 1
+    assert seen == 5                                     # the products' files
