@@ -84,7 +84,7 @@ struct LayerWs {
     ColStatParts parts;          // per-channel (sum, min, max) partials of the output, from the convolution's epilogue
     float4 *fold;                // per-channel constants of the normalisation, for the recompute fusion
     int64_t *tot_g;              // [cout] per-channel totals of the 16-bit gradient codes, and behind them ...
-    int64_t *wg_table;           // ... the table of the weight gradient's sums (convolution): cleared together
+    int64_t *wg_table;           // ... the table of the weight gradient's sums (NULL: in pieces): cleared together
     int64_t clear_words;
     int32_t *w_sums;             // the weights' code sums: forward, then layer gradient
     SumJob wg_sums[6];           // the weight gradient's code sums (count: wg_count)
@@ -110,12 +110,13 @@ static LayerWs layer_ws(const qbp_layer_desc *L, const LayerShape &s, void *ws, 
     if (cells) { l.parts.lo = c.take<float>(cells); l.parts.hi = c.take<float>(cells); l.parts.sum = c.take<double>(cells); }
     l.fold = c.take<float4>((size_t)s.cout);
     const qbp_conv_desc *d = s.conv ? &L->conv : nullptr;
-    l.tot_g = c.take<int64_t>((size_t)s.cout + wgrad_sum_table(d));
-    l.wg_table = l.tot_g + s.cout;
-    l.clear_words = 2 * ((int64_t)s.cout + (int64_t)wgrad_sum_table(d));
+    const size_t table = wgrad_sum_table(d, s.rows, s.cout, s.cin);
+    l.tot_g = c.take<int64_t>((size_t)s.cout + table);
+    l.wg_table = table ? l.tot_g + s.cout : nullptr;
+    l.clear_words = table ? 2 * ((int64_t)s.cout + (int64_t)table) : 0;
     l.w_sums = c.take<int32_t>(std::max(sum_elems(weight_sum_job(L, s, false, nullptr, nullptr)), sum_elems(weight_sum_job(L, s, true, nullptr, nullptr))));
-    l.wg_count = wgrad_sum_jobs(d, s.rows, s.cout, s.cin, x, hi, lo, true, d ? l.wg_table : nullptr, l.wg_sums);
-    for (int i = 0; i < l.wg_count && !d; ++i) l.wg_sums[i].out = c.take<int32_t>(sum_elems(l.wg_sums[i]));
+    l.wg_count = wgrad_sum_jobs(d, s.rows, s.cout, s.cin, x, hi, lo, true, l.wg_table, l.wg_sums);
+    for (int i = 0; i < l.wg_count && !table; ++i) l.wg_sums[i].out = c.take<int32_t>(sum_elems(l.wg_sums[i]));
     l.bytes = c.off;
     return l;
 }
@@ -294,10 +295,10 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_bwd(const qbp_la
         rc = rangebn_bwd_bifurcate_impl(dy, saved->z, s.rows, s.cout, gamma, beta, L->relu, saved->save_mean, saved->save_min,
                                         saved->save_max, g, dgamma, dbeta, L->seed, L->tensor_id8, L->tensor_id16, g8, qp8,
                                         s.conv ? l.row_sums : nullptr, ghi, glo, qp16, true, l.scratch, l.scratch_bytes, st,
-                                        self_totals ? nullptr : tot_g, l.tot_g, s.conv ? l.clear_words : 0, early, nearly);
+                                        self_totals ? nullptr : tot_g, l.tot_g, l.clear_words, early, nearly);
     } else {
         if (!g) return fail(QBP_ERR_INVALID_ARG, "layer_bwd: this shape needs saved->g (the fp32 gradient is written and read back)");
-        if (s.conv) QBP_CUDA_OK(cudaMemsetAsync(l.tot_g, 0, sizeof(uint32_t) * (size_t)l.clear_words, st));
+        if (l.clear_words) QBP_CUDA_OK(cudaMemsetAsync(l.tot_g, 0, sizeof(uint32_t) * (size_t)l.clear_words, st));
         int nparts = 0;
         rc = rangebn_bwd_impl(dy, saved->z, s.rows, s.cout, gamma, beta, L->relu, saved->save_mean, saved->save_min,
                               saved->save_max, g, dgamma, dbeta, l.scratch, l.scratch_bytes, l.range_parts, &nparts, st);

@@ -129,13 +129,13 @@ int wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, cons
                    int *ext_status, void *ws, size_t ws_bytes, cudaStream_t st, const int64_t *tot_x = nullptr,
                    const int64_t *tot_g16 = nullptr, bool tot_g_filled = true, bool lo_signed = false,
                    const SumJob *done_sums = nullptr);
-// The sums behind the zero-point terms.  Plain product: the columns of x, hi, lo in pieces (3 jobs).  Convolution: the same
-// added to one cleared table of int64 (tab: x [C], hi [N], lo [N]; 3 x 3: then [8][C], [8][N], [8][N] over the images' edges;
-// 3 or 6 jobs); with totals (tot_x, tot_g16) the first three are not needed.  done_sums (above): the caller has run the needed
+// The sums behind the zero-point terms.  Plain product: the columns of x, hi, lo in pieces (3 jobs), or, when that would make the
+// pieces long, as for a convolution: added to one cleared table of int64 (tab: x [C], hi [N], lo [N]; 3 x 3: then [8][C], [8][N],
+// [8][N] over the images' edges; 3 or 6 jobs); with totals (tot_x, tot_g16) the first three are not needed.  done_sums (above): the caller has run the needed
 // ones into these buffers, and has cleared tot_g16 when tot_g_filled is false.
 int wgrad_sum_jobs(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, const int8_t *x, const int8_t *hi, const uint8_t *lo,
                    bool lo_signed, int64_t *tab, SumJob (&jobs)[6]);
-size_t wgrad_sum_table(const qbp_conv_desc *d);        // int64 entries of tab (0: plain)
+size_t wgrad_sum_table(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K);        // int64 entries of tab (0: sums in pieces)
 // tot_g_filled == false: tot_g16 is a cleared buffer [K] that the product fills itself (possible when wgrad_self_totals(d)).
 bool wgrad_self_totals(const qbp_conv_desc *d);
 // Shapes the convolution products / the convolution weight gradient implement.

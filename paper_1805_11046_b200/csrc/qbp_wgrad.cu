@@ -86,9 +86,9 @@ struct WgradParams {
     int64_t M, N, K;
     long long *part;                 // int64 partials, one block of part_stride values per CTA
     int64_t part_stride;             // ma * 128 * bn, padded
-    // plain product: code sums over the M rows (acc = raw - zg * sx[k] - zx * (256 * shi[n] + slo[n]) + M * zx * zg)
+    // plain product: code sums over the M rows, in pieces or (cx set) as for a convolution (acc = raw - zg * sx[k] - zx * (256 * shi[n] + slo[n]) + M * zx * zg)
     CodeSums sx, shi, slo;
-    // convolution: over all positions ([C], [N], [N]) and over the edges of the images ([8][...], see kSumEdges)
+    // over all positions ([C], [N], [N]); convolution: and over the edges of the images ([8][...], see kSumEdges)
     const long long *cx, *chi, *clo, *ex, *ehi, *elo;
     const qbp_qparams *qx, *qg;
     long long *acc_out; float *dW;
@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(256) wgrad_finalize_kernel(const __grid_consta
 #pragma unroll
     for (int o = 1; o < kLanes; o <<= 1) raw += __shfl_xor_sync(0xffffffffu, raw, o);
     if (!live || part_lane != 0) return;
-    const long long SX = P.sx.at(k), SG = 256 * P.shi.at(n) + P.slo.at(n);
+    const long long SX = P.cx ? P.cx[k] : P.sx.at(k), SG = P.cx ? 256 * P.chi[n] + P.clo[n] : 256 * P.shi.at(n) + P.slo.at(n);
     const long long acc = raw - zg * SX - zx * SG + P.M * zx * zg;
     if (P.acc_out) P.acc_out[e] = acc;
     if (P.dW) P.dW[e] = __fmul_rn((float)acc, __fmul_rn(P.qx->scale, P.qg->scale));
@@ -707,7 +707,16 @@ struct WgradPlan {
 
 }  // namespace qbp
 
-size_t qbp::wgrad_sum_table(const qbp_conv_desc *d) { return d ? (size_t)(d->pad ? 9 : 1) * ((size_t)d->C + 2 * (size_t)d->K) : 0; }
+// Plain products of more than kWgPieceRows rows: the sums by atomics into a table, from as many blocks as the rows fill.  The 16
+// pieces that a reader adds up would be longer than the whole product takes (2^20 rows, 128 x 32 columns: 521 us with pieces, 115
+// with the table; the clearing it needs is what shorter ones save).  Such a product never finishes in one launch and is never the pair
+// kernel's: only wgrad_finalize_kernel reads the sums.
+constexpr int64_t kWgPieceRows = 65536;
+size_t qbp::wgrad_sum_table(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K)
+{
+    if (!d) return M > kWgPieceRows ? (size_t)(K + 2 * N) : 0;
+    return (size_t)(d->pad ? 9 : 1) * ((size_t)d->C + 2 * (size_t)d->K);
+}
 int qbp::wgrad_sum_jobs(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, const int8_t *x, const int8_t *hi, const uint8_t *lo,
                         bool lo_signed, int64_t *tab, SumJob (&jobs)[6])
 {
@@ -867,8 +876,9 @@ static void plan_wgrad(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K, 
 
 static size_t wgrad_ws_bytes(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K)
 {
-    const size_t sums = d ? align_up(sizeof(int64_t) * wgrad_sum_table(d), 256)
-                          : align_up(sizeof(int32_t) * sum_elems(M, K, kSumCols), 256) + 2 * align_up(sizeof(int32_t) * sum_elems(M, N, kSumCols), 256);
+    const size_t table = wgrad_sum_table(d, M, N, K);
+    const size_t sums = table ? align_up(sizeof(int64_t) * table, 256)
+                              : align_up(sizeof(int32_t) * sum_elems(M, K, kSumCols), 256) + 2 * align_up(sizeof(int32_t) * sum_elems(M, N, kSumCols), 256);
     // (the split, and with it the partials, may differ between the two forms of the low limb: room for either)
     size_t part = 0;
     for (int lo_signed = 0; lo_signed < 2; ++lo_signed) {
@@ -934,11 +944,12 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
     int *status = w.take<int>(1);
     if (ext_status) status = ext_status;         // the caller's sticky word: raised here, never cleared
     SumJob all[6], jobs[6];
-    int64_t *tab = d && !done_sums ? w.take<int64_t>(wgrad_sum_table(d)) : nullptr;
+    const size_t table = wgrad_sum_table(d, M, N, K);
+    int64_t *tab = table && !done_sums ? w.take<int64_t>(table) : nullptr;
     const int nall = wgrad_sum_jobs(d, M, N, K, x, g_hi, g_lo, lo_signed, tab, all);
     for (int i = 0; i < nall; ++i) {
         if (done_sums) all[i] = done_sums[i];
-        else if (!d) all[i].out = w.take<int32_t>(sum_elems(all[i]));
+        else if (!table) all[i].out = w.take<int32_t>(sum_elems(all[i]));
     }
     int64_t *part = P.direct ? nullptr : w.take<int64_t>((size_t)pl.grid * (size_t)P.part_stride);
 
@@ -951,11 +962,11 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
     int njobs = 0;
     if (!done_sums)
         for (int i = from_totals ? 3 : 0; i < nall; ++i) jobs[njobs++] = all[i];
-    if (!d) { P.sx = sums_of(all[0]); P.shi = sums_of(all[1]); P.slo = sums_of(all[2]); }
+    if (!table) { P.sx = sums_of(all[0]); P.shi = sums_of(all[1]); P.slo = sums_of(all[2]); }
     else {
         P.cx = (const long long *)all[0].out64; P.chi = (const long long *)all[1].out64; P.clo = (const long long *)all[2].out64;
         if (nall == 6) { P.ex = (const long long *)all[3].out64; P.ehi = (const long long *)all[4].out64; P.elo = (const long long *)all[5].out64; }
-        if (tab) QBP_CUDA_OK(cudaMemsetAsync(tab, 0, sizeof(int64_t) * wgrad_sum_table(d), st));
+        if (tab) QBP_CUDA_OK(cudaMemsetAsync(tab, 0, sizeof(int64_t) * table, st));
     }
     ZeroJobs zero{};
     if (!ext_status) { zero.p[0] = reinterpret_cast<uint32_t *>(status); zero.words[0] = 1; }

@@ -487,6 +487,12 @@ def test_linear_layers_of_other_shapes_stagewise(B, batch, cin, cout):
     _check_layer(B, cfg, True)
 
 
+@pytest.mark.parametrize("batch", [65536, 65552])
+def test_linear_layer_of_a_long_minibatch_stagewise(B, batch):
+    """Either side of 65536 rows, where the weight gradient's column sums go to a table that the backward clears on the way."""
+    test_linear_layers_of_other_shapes_stagewise(B, batch, 32, 48)
+
+
 @pytest.mark.parametrize("id16", [5, 6])
 @pytest.mark.parametrize("batch,cin,cout", [(32, 16, 16), (256, 16, 16), (272, 32, 16), (400, 64, 48), (48, 16, 528), (2080, 32, 64)])
 def test_backward_where_many_elements_are_extremes(B, batch, cin, cout, id16):

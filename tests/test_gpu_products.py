@@ -456,6 +456,13 @@ def test_wgrad_code_sums_in_pieces_of_the_rows(B, M, N, K):
     assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
 
 
+@pytest.mark.parametrize("M", [65535, 65536, 65537, 300001])
+@pytest.mark.parametrize("N,K", [(16, 144), (144, 32)])
+def test_wgrad_code_sums_of_long_reductions(B, M, N, K):
+    """Beyond 65536 rows the column sums are added up in a table instead of pieces: either side of that, many rows."""
+    test_wgrad_code_sums_in_pieces_of_the_rows(B, M, N, K)
+
+
 @pytest.mark.parametrize("N,H,W,C,K", [(600, 1, 3, 32, 64), (5, 7, 1, 160, 32), (150, 2, 4, 64, 288), (700, 3, 3, 32, 32)])
 def test_wgrad_conv_edge_sums(B, N, H, W, C, K):
     """The zero-point terms of a 3x3 weight gradient from the operands' sums over all positions less those over the images'
