@@ -119,11 +119,13 @@ _NULL = C.c_void_p(0)
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
-def _stream() -> C.c_void_p:
+def _stream_handle(device: int) -> int:
     # (the raw handle of torch's current stream: building a Stream object for it costs several times as much)
-    if _raw_stream is not None:
-        return C.c_void_p(_raw_stream(torch.cuda.current_device()))
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return _raw_stream(device) if _raw_stream is not None else torch.cuda.current_stream(device).cuda_stream
+
+
+def _stream() -> C.c_void_p:
+    return C.c_void_p(_stream_handle(torch.cuda.current_device()))
 
 
 class _Workspaces(threading.local):
@@ -144,7 +146,7 @@ def workspace(nbytes: int, device=None) -> torch.Tensor:
     graph keeps the addresses of its calls: give those calls a `ws` of their own.)"""
     dev = None if device is None else torch.device(device)
     index = torch.cuda.current_device() if dev is None or dev.index is None else dev.index
-    key = (index, _stream().value)
+    key = (index, _stream_handle(index))
     t = _workspaces.by_stream.get(key)
     if t is None or t.numel() < nbytes:
         t = torch.empty(max(nbytes, 1 << 20), dtype=torch.uint8, device=torch.device("cuda", index))
