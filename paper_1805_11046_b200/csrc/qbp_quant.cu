@@ -798,6 +798,7 @@ int launch_rowsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int
 }
 int launch_colsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int64_t *sums, cudaStream_t st)
 {
+    if (cols % 16 || !aligned16(q)) return fail(QBP_ERR_INVALID_ARG, "column sums need cols %% 16 == 0 and 16-byte aligned codes");
     const SumJob job{q, rows, cols, kSumCols, is_signed ? 1 : 0, nullptr, 0, 0, sums};
     QBP_CUDA_OK(cudaMemsetAsync(sums, 0, sizeof(int64_t) * (size_t)cols, st));
     return rows == 0 ? QBP_OK : launch_code_sums(&job, 1, st);

@@ -109,6 +109,16 @@ def test_chunk_averaged_clamp_refuses_rows_that_do_not_divide(B):
         B.qbp_range_chunked(to_dev(synth.normal((10, 8), 1)), 3)
 
 
+@pytest.mark.parametrize("rows", [0, 5])
+def test_column_sums_that_are_refused_leave_their_buffer_alone(B, rows):
+    import torch
+    x = torch.ones((rows, 24), dtype=torch.float32, device="cuda")
+    cols = torch.full((24,), 7, dtype=torch.int64, device="cuda")
+    with pytest.raises(B.QbpError):
+        B.qbp_quantize_s8(x, col_sums=cols)          # 24 columns are no multiple of 16
+    assert bool((cols == 7).all())
+
+
 def test_bifurcate_and_code_sums(B):
     import torch
     g = synth.normal((130, 64), 12, std=0.1)
