@@ -22,11 +22,14 @@ def B():
 def _run_layer(B, cfg, relu, conv=None):
     import torch
     from paper_1805_11046_b200 import layer
-    x, w, dy = cfg["x"], cfg["w"], cfg["dy"]
+    x, w, dy = cfg["x"], cfg["w"], to_dev(cfg["dy"])
+    if cfg.get("dy_off"):                           # (that many floats behind a 16-byte boundary)
+        dy = torch.cat([dy.new_zeros(cfg["dy_off"]), dy.flatten()])[cfg["dy_off"]:].view(dy.shape)
+        assert dy.data_ptr() % 16 == 4 * cfg["dy_off"]
     L = layer.QuantizedLayer(conv=conv, batch=x.shape[0], in_features=x.shape[-1], out_features=w.shape[-1] if conv is None else None,
                              relu=relu, seed=cfg["seed"], tensor_id8=cfg["id8"], tensor_id16=cfg["id16"])
     y = L.forward(to_dev(x), to_dev(w))
-    dx, dw, dgamma, dbeta = L.backward(to_dev(dy))
+    dx, dw, dgamma, dbeta = L.backward(dy)
     torch.cuda.synchronize()
     return L, y, dx, dw, dgamma, dbeta
 
@@ -491,6 +494,23 @@ def test_linear_layers_of_other_shapes_stagewise(B, batch, cin, cout):
 def test_linear_layer_of_a_long_minibatch_stagewise(B, batch):
     """Either side of 65536 rows, where the weight gradient's column sums go to a table that the backward clears on the way."""
     test_linear_layers_of_other_shapes_stagewise(B, batch, 32, 48)
+
+
+@pytest.mark.parametrize("relu", [False, True])
+@pytest.mark.parametrize("shape", [(48, 64, 80), (2080, 32, 64), (65552, 16, 16), (2, 9, 32, 96, 3), (3, 14, 64, 32, 1), (12, 14, 96, 64, 3), (12, 14, 64, 64, 1)])
+def test_backward_of_a_gradient_off_the_vector_boundary(B, shape, relu):
+    """dy 4 bytes behind a 16-byte boundary: the gradient is written by a pass of its own and bifurcated from memory, with its own
+    clearing and order of the code sums -- linear layers and convolutions of few and of many rows."""
+    if len(shape) == 3:
+        batch, cin, cout = shape
+        cfg, conv = dict(x=synth.normal((batch, cin), 95), w=synth.kaiming_uniform_linear(cin, cout, 96), dy=synth.normal((batch, cout), 97, std=0.1)), None
+    else:
+        n, hw, cin, cout, r = shape
+        cfg = synth.conv3x3_layer(batch=n, hw=hw, c_in=cin, k_out=cout)
+        conv = dict(N=n, H=hw, W=hw, C=cin, K=cout, R=r, S=r, stride=1, pad=(r - 1) // 2)
+        if r == 1:
+            cfg["w"] = np.ascontiguousarray(cfg["w"][:, 1:2, 1:2, :])
+    _check_layer(B, dict(x=cfg["x"], w=cfg["w"], dy=cfg["dy"], seed=3, id8=5, id16=5, dy_off=1), relu, conv, _sampler(98))
 
 
 @pytest.mark.parametrize("id16", [5, 6])
