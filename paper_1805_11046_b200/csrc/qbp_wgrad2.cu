@@ -18,6 +18,7 @@
 // that arrives in both CTAs; warps 2..9 drain this CTA's accumulator rows.  Every wait is bounded; on expiry the
 // CTA raises the status word and leaves through the normal exit.  No TMA load here uses cluster multicast.
 #include "qbp_mma.cuh"
+#include "qbp_pair.cuh"
 
 #include <algorithm>
 
@@ -48,50 +49,6 @@ struct Wgrad2Params {
     int *status;
 };
 
-__device__ __forceinline__ uint32_t w2_cluster_ctarank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void w2_cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t w2_map_to_cta(const void *p, uint32_t rank)
-{
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void w2_arrive_cluster(uint32_t cluster_addr)
-{
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// TMA load of this CTA's box whose completion is reported to an mbarrier of either CTA of the pair (no multicast)
-__device__ __forceinline__ void w2_tma_load_2d(void *dst, const void *map, uint32_t bar_cluster_addr, int x, int y)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-        ::"r"(smem_u32(dst)), "l"(map), "r"(bar_cluster_addr), "r"(x), "r"(y)
-        : "memory");
-}
-__device__ __forceinline__ void w2_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
-}
-__device__ __forceinline__ void w2_commit(uint64_t *bar)
-{
-    const uint16_t mask = 3;
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(smem_u32(bar)), "h"(mask)
-                 : "memory");
-}
-
 // The eight pair MMAs of a stage (128 reduction rows = four k steps per limb), the limb outermost: switching
 // between the two instruction descriptors stalls the MMA pipe.  Offsets in 16-byte units: 256 per k step of an
 // M/N-major 128-byte-row tile, 1024 per 128 x 128 tile.
@@ -104,7 +61,7 @@ __device__ __forceinline__ void w2_issue_stage(uint32_t tmem, uint32_t a_lo, uin
     for (int i = 0; i < 8; ++i) {
         const int limb = i >> 2, kk = i & 3;
         if (elect_one())
-            w2_mma(tmem + 256u * (uint32_t)limb, ((uint64_t)hi << 32) | (uint64_t)(a_lo + (uint32_t)kk * 256u),
+            mma_i8_pair(tmem + 256u * (uint32_t)limb, ((uint64_t)hi << 32) | (uint64_t)(a_lo + (uint32_t)kk * 256u),
                    ((uint64_t)hi << 32) | (uint64_t)(b_lo + (uint32_t)limb * 1024u + (uint32_t)kk * 256u),
                    limb ? idesc_lo : idesc_hi, (FIRST && kk == 0) ? 0u : 1u);
     }
@@ -132,7 +89,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
     uint8_t *smem = smem_raw + ((1024u - (raw_addr & 1023u)) & 1023u);
     uint8_t *staging = smem + (size_t)kW2Stages * kW2StageBytes;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = w2_cluster_ctarank();
+    const uint32_t rank = cluster_ctarank();
     const int pair = blockIdx.x >> 1;
 
     if (threadIdx.x == 0) {
@@ -144,13 +101,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
         tma_prefetch_desc(&P.mapX); tma_prefetch_desc(&P.mapHi); tma_prefetch_desc(&P.mapLo);
         if (P.dW) tma_prefetch_desc(&P.mapC);
     }
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512u) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    }
+    if (warp == 1) { tmem_alloc_pair(&tmem_slot, 512); tmem_relinquish_pair(); }
     tc_fence_before();
     __syncthreads();
-    w2_cluster_sync();                   // both CTAs' barriers are initialised before either signals the other
+    cluster_sync_all();                   // both CTAs' barriers are initialised before either signals the other
     tc_fence_after();
     // (each role waits for the kernels before at its first use of their results: what it needs of the launch's parameters, and the
     // code up to there, has then been fetched)
@@ -169,13 +123,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
                     if (in_group == 0 && !mbar_wait(&empty_bar[group], gph)) { timed_out = true; break; }
                     if (++in_group == (uint32_t)kW2Cg) { in_group = 0; ++group; }
                     uint8_t *sa = smem + (size_t)s * kW2StageBytes;
-                    const uint32_t bar = w2_map_to_cta(&full_bar[s], 0);
+                    const uint32_t bar = map_to_cta(&full_bar[s], 0);
                     if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * kW2StageBytes);
                     const int m0 = it * 128;
                     if (!waited) { pdl_wait(); waited = true; }
-                    w2_tma_load_2d(sa, &P.mapX, bar, k_mine, m0);
-                    w2_tma_load_2d(sa + 16384, &P.mapHi, bar, n_mine, m0);
-                    w2_tma_load_2d(sa + 32768, &P.mapLo, bar, n_mine, m0);
+                    tma_load_2d_pair(sa, &P.mapX, bar, k_mine, m0);
+                    tma_load_2d_pair(sa + 16384, &P.mapHi, bar, n_mine, m0);
+                    tma_load_2d_pair(sa + 32768, &P.mapLo, bar, n_mine, m0);
                     if (++s == (uint32_t)kW2Stages) { s = 0; gph ^= 1u; group = 0; }
                 }
             }
@@ -200,13 +154,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
                     if (it == 0) w2_issue_stage<true>(tmem_base, a_lo, b_lo, P.idesc_hi, P.lo_flip);
                     else         w2_issue_stage<false>(tmem_base, a_lo, b_lo, P.idesc_hi, P.lo_flip);
                     if (++in_group == (uint32_t)kW2Cg) {
-                        if (elect_one()) w2_commit(&empty_bar[group]);
+                        if (elect_one()) mma_commit_pair(&empty_bar[group]);
                         in_group = 0; ++group;
                     }
                     a_addr += kW2StageBytes;
                     if (++s == (uint32_t)kW2Stages) { s = 0; ph ^= 1u; group = 0; a_addr = ring; }
                 }
-                if (!timed_out && elect_one()) w2_commit(&acc_full);
+                if (!timed_out && elect_one()) mma_commit_pair(&acc_full);
             }
         }
     } else {
@@ -218,7 +172,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
         pdl_wait();
         const float scale = __fmul_rn(P.qx->scale, P.qg->scale);
         const long long zx = P.qx->zero_point, zg = P.qg->zero_point - P.zg_shift;
-        const uint32_t leader_empty = w2_map_to_cta(&acc_empty, 0);
+        const uint32_t leader_empty = map_to_cta(&acc_empty, 0);
         uint32_t fph = 0;
         for (int tile = pair; tile < P.tiles_total; tile += P.pairs) {
             const W2Tile o = w2_tile(P, tile);
@@ -250,7 +204,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
                 if (c_begin >= c_end) {
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) w2_arrive_cluster(leader_empty);
+                    if (lane == 0) mbar_arrive_cluster(leader_empty);
                 }
                 for (int c = c_begin; c < c_end; ++c) {
                     const int c0 = c * 32;
@@ -262,7 +216,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
                         // this warp has read its part of the accumulators: tell the leader's MMA warp
                         tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) w2_arrive_cluster(leader_empty);
+                        if (lane == 0) mbar_arrive_cluster(leader_empty);
                     }
                     const int lim = (int)(ncol - c0 < 32 ? ncol - c0 : 32);
                     // (lane l holds the column term of column c0 + l; the row's 32 sums take them by shuffle)
@@ -317,10 +271,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
     }
     tc_fence_before();
     __syncthreads();
-    w2_cluster_sync();                   // neither CTA retires while the other may still read its memory or signal it
+    cluster_sync_all();                   // neither CTA retires while the other may still read its memory or signal it
     if (warp == 1) {
         __syncwarp();
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+        tmem_dealloc_pair(tmem_base, 512);
     }
 }
 
