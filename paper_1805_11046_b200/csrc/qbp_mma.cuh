@@ -66,7 +66,7 @@ int rangebn_bwd_impl(const float *dy, const float *x, int64_t n, int64_t C, cons
 size_t rangebn_range_parts_capacity(int64_t C);
 // Range BN backward and the bifurcation of the gradient in two passes, the fp32 gradient optional (qbp_rangebn.cu).
 bool rangebn_bwd_one_launch(int64_t n, int64_t C);
-bool rangebn_bwd_bifurcate_supported(const float *dy, const float *x, const float *g_out, int64_t n, int64_t C, bool row_sums);
+bool rangebn_bwd_bifurcate_supported(const float *dy, const float *x, const float *g_out, int64_t n, int64_t C);
 int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64_t C, const float *gamma, const float *beta,
                                int relu, const float *save_mean, const float *save_min, const float *save_max, float *g_out,
                                float *dgamma, float *dbeta, uint64_t seed, uint32_t id8, uint32_t id16, int8_t *q8,

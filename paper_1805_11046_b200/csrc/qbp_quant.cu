@@ -628,7 +628,7 @@ int fill_sum_jobs(const SumJob *jobs, int count, SumJobs &J, int *blocks)
         } else {
             j.pieces = s.kind == kSumEdges ? edge_pieces(s.rows, s.H, s.W, kSumThreads >> j.lg_log2) : sum_pieces(s.rows, s.cols);
             // added up by atomics, nobody reads the pieces one by one: as many blocks as the rows give work to (the sums of
-            // 200704 x 128 codes with 16 pieces: 31 us, now 16)
+            // 200704 x 128 codes: 31 us with 16 pieces, 16 so)
             if (s.out64 && s.kind == kSumCols) j.pieces = (int)std::max<int64_t>(j.pieces, std::min<int64_t>(4ll * sm_count() / strips, s.rows / 128));
             if (s.kind == kSumEdges) j.corner_pieces = corner_pieces(s.rows / ((int64_t)s.H * s.W));
             j.blocks = strips * (s.kind == kSumCols ? j.pieces : 4 * (j.pieces + j.corner_pieces));

@@ -541,13 +541,13 @@ __global__ void __launch_bounds__(T) bn_bwd_finalize_kernel(const double *__rest
 // What bounds it: the integer pipes (about 25 instructions per element in Philox and the two roundings alone).  So the rest is
 // kept small: 32-bit indices, no check per row in the whole tiles, the rare terms of the extremes on a path outside the
 // straight line (one branch per tile of four rows, after which all of them are quantised together), the channels' constants
-// read from shared memory once per tile.  Two rows per tile and 69 instructions per element before: 51.4 M elements of 64
-// channels 131 -> 109 us (without Philox at all: 109), 102.8 M of 512 channels 277 -> 209 us (5.5 TB/s), 12.8 M of 256
-// channels 43 -> 35 us.  Not better: four blocks of 64 registers (113, spills with four rows), two of 105 (109), a third slot.
+// read from shared memory once per tile.  With tiles of two rows and checks per row (69 instructions per element, now 47) 51.4 M
+// elements of 64 channels take 131 us, so 109; 102.8 M of 512 channels 277 and 209 (5.5 TB/s), 12.8 M of 256 channels 43 and 35.  Not better: four blocks of 64 registers (113, spills with four rows), two of 105 (109), a third slot.
 constexpr int kBabRows = 4;       // rows per thread and tile (an even number)
 constexpr int kBabSlots = 2;      // ring depth in tiles
 constexpr int kBabBlocks = 3;     // blocks per SM (at most 80 registers a thread)
 constexpr size_t kBabRingBytes = (size_t)kBabSlots * 2 * kBabRows * kScanThreads * sizeof(float4);
+static_assert(kBabBlocks * (kBabRingBytes + 8192 + 1024) <= 228 * 1024, "the rings of an SM's blocks, their 7.3 KB of static shared memory beside them");
 // ONE: both copies have one tensor id and share their Philox blocks.
 template <bool RELU, bool STORE_G, bool TOTALS, bool ONE>
 __global__ void __launch_bounds__(kScanThreads, kBabBlocks) bn_bwd_apply_bifurcate_kernel(
@@ -560,8 +560,7 @@ __global__ void __launch_bounds__(kScanThreads, kBabBlocks) bn_bwd_apply_bifurca
     pdl_wait();
     const ScanPos p = scan_pos<4>(C, tw);
     int cs16[4] = {0, 0, 0, 0};                   // stored codes of this thread's rows (fewer than 65536 rows)
-    // the channels' constants in shared memory, read again for every step: held in registers (28 of them) they would cost the
-    // fourth block of an SM
+    // the channels' constants in shared memory, read again for every tile: 28 registers that the 80 of a thread have no room for
     __shared__ float4 s_const[7][kScanMaxTw];     // scale, gamma, centre, half of the range, m1, the mask's threshold and sign
     if ((int)threadIdx.x < tw) {
         float k[7][4];
@@ -1308,12 +1307,10 @@ static int bn_bwd_apply_launch(const float *dy, const float *x, int64_t n_rows, 
 // Whether the statistics of rangebn_bwd_bifurcate_impl are one launch: what it clears is then not clear before `extra` runs.
 bool rangebn_bwd_one_launch(int64_t n, int64_t C) { return few_rows(n, C); }
 
-// Whether rangebn_bwd_bifurcate_impl takes a tensor of C channels (row_sums: each row's 8-bit code sum is wanted).
-bool rangebn_bwd_bifurcate_supported(const float *dy, const float *x, const float *g_out, int64_t n, int64_t C, bool row_sums)
+// Whether rangebn_bwd_bifurcate_impl takes these tensors.  (Philox blocks below 2^32: more elements do not fit the device)
+bool rangebn_bwd_bifurcate_supported(const float *dy, const float *x, const float *g_out, int64_t n, int64_t C)
 {
-    if (!aligned16(x) || !aligned16(dy) || (g_out && !aligned16(g_out)) || C % 4 || n < 2 || n * C >= (1ll << 34)) return false;      // (Philox blocks below 2^32; more does not fit the device)
-    (void)row_sums;      // (any row width: rows wider than a warp's lanes are added up from their pieces)
-    return true;
+    return aligned16(x) && aligned16(dy) && (!g_out || aligned16(g_out)) && C % 4 == 0 && n >= 2 && n * C < (1ll << 34);
 }
 
 // Range BN backward and the bifurcation of its result in two passes over (dy, x): statistics with the extremes of dy
@@ -1328,7 +1325,7 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
 {
     int rc = check_bn("rangebn_bwd", dy, x, n, C, ws, ws_bytes);
     if (rc) return rc;
-    if (!rangebn_bwd_bifurcate_supported(dy, x, g_out, n, C, row_sums8 != nullptr) || ((uintptr_t)q8 & 3) || ((uintptr_t)hi & 3) || ((uintptr_t)lo & 3))
+    if (!rangebn_bwd_bifurcate_supported(dy, x, g_out, n, C) || ((uintptr_t)q8 & 3) || ((uintptr_t)hi & 3) || ((uintptr_t)lo & 3))
         return fail(QBP_ERR_UNSUPPORTED_SHAPE, "rangebn_bwd (bifurcating): shape or alignment not taken");
     WsCarver w(ws, ws_bytes);
     double *pa = w.take<double>((size_t)kScanMaxStrips * C);
@@ -1340,8 +1337,8 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
     float *ext = w.take<float>(6 * (size_t)kScanMaxStrips * C);
     float2 *chan_range = w.take<float2>((size_t)C);
     float2 *relu_thr = w.take<float2>((size_t)C);
-    // (kBabBlocks resident blocks per SM by the kernel's launch bounds, whatever the instance)
-    const ScanGeom ga = scan_geom(n, C, true, blocks_per_sm<bn_bwd_apply_bifurcate_kernel<true, true, true, true>>(kScanThreads));
+    // (kBabBlocks resident blocks per SM, by the kernel's launch bounds and its ring, whatever the instance)
+    const ScanGeom ga = scan_geom(n, C, true, kBabBlocks);
     // each row's code sum by shuffles over the row's lanes of a warp; a row that spans several warps or blocks is
     // added up from its pieces (integer atomics on the zeroed sums: the result does not depend on the order)
     ZeroJobs zero{};
@@ -1360,7 +1357,16 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
     const PhiloxKeys keys = philox_keys_host(seed);
     const uint32_t flip = lo_signed ? 0x80808080u : 0u;
     QBP_TRACE_BEGIN(st);
-#define QBP_BN_BAB(R, G, T, O) do { static PerDeviceOnce once_; QBP_SMEM_OPT_IN(once_, (bn_bwd_apply_bifurcate_kernel<R, G, T, O>), kBabRingBytes); launch(bn_bwd_apply_bifurcate_kernel<R, G, T, O>, grid, kScanThreads, kBabRingBytes, st, reinterpret_cast<const float4 *>(dy), reinterpret_cast<const float4 *>(x), (uint32_t)n, (int)C, ga.tw, save_min, save_max, gamma, Cn, coef, reinterpret_cast<float4 *>(g_out), range, id8, id16, keys, reinterpret_cast<uint32_t *>(q8), reinterpret_cast<uint32_t *>(hi), reinterpret_cast<uint32_t *>(lo), flip, row_sums8, reinterpret_cast<unsigned long long *>(tot16), relu_thr); } while (0)
+#define QBP_BN_BAB(R, G, T, O)                                                                                          \
+    do {                                                                                                                \
+        static PerDeviceOnce once_;                                                                                     \
+        QBP_SMEM_OPT_IN(once_, (bn_bwd_apply_bifurcate_kernel<R, G, T, O>), kBabRingBytes);                             \
+        launch(bn_bwd_apply_bifurcate_kernel<R, G, T, O>, grid, kScanThreads, kBabRingBytes, st,                        \
+               reinterpret_cast<const float4 *>(dy), reinterpret_cast<const float4 *>(x), (uint32_t)n, (int)C, ga.tw,   \
+               save_min, save_max, gamma, Cn, coef, reinterpret_cast<float4 *>(g_out), range, id8, id16, keys,          \
+               reinterpret_cast<uint32_t *>(q8), reinterpret_cast<uint32_t *>(hi), reinterpret_cast<uint32_t *>(lo),    \
+               flip, row_sums8, reinterpret_cast<unsigned long long *>(tot16), relu_thr);                               \
+    } while (0)
 #define QBP_BN_BAB1(R, G, T) do { if (id8 == id16) QBP_BN_BAB(R, G, T, true); else QBP_BN_BAB(R, G, T, false); } while (0)
 #define QBP_BN_BAB2(R, G) do { if (tot16) QBP_BN_BAB1(R, G, true); else QBP_BN_BAB1(R, G, false); } while (0)
     if (g_out) { if (relu) QBP_BN_BAB2(true, true); else QBP_BN_BAB2(false, true); }

@@ -609,8 +609,8 @@ __device__ __forceinline__ long long wg_tap_part(const WgradParams &P, bool of_x
 }
 
 // The same for a convolution, output [n][tap][c].  A block takes 64 channels of one tap and NB output channels: SX and SG
-// are added up once per block instead of once per element (tens of loads each, which made this kernel 78 us for a
-// 256 -> 256 channel 3x3 filter, five times what its partials take to read), four groups of 64 threads share the slices,
+// are added up once per block (once per element they are tens of loads each: 78 us for a 256 -> 256 channel 3x3 filter, five times
+// what its partials take to read), four groups of 64 threads share the slices,
 // each thread with eight loads in flight, and meet in shared memory.
 template <int NB>
 __global__ void __launch_bounds__(256) wgrad_conv_finalize_kernel(const __grid_constant__ WgradParams P)

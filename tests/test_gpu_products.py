@@ -446,7 +446,7 @@ def test_wgrad_conv_finalize_block_shapes(B, N, H, W, C, K, R):
 @pytest.mark.parametrize("M", [1, 31, 127, 128, 255, 256, 257, 4095, 8200])
 @pytest.mark.parametrize("N,K", [(16, 144), (272, 16)])
 def test_wgrad_code_sums_in_pieces_of_the_rows(B, M, N, K):
-    """The zero-point terms come from column sums taken in up to 32 pieces of the rows, in strips of 128 columns: one and
+    """The zero-point terms come from column sums taken in up to 16 pieces of the rows, in strips of 128 columns: one and
     several pieces, uneven ones, strips of one 16-column group and partly filled; signed and unsigned bytes."""
     X = random_codes((M, K), 61); G = np.random.Generator(np.random.PCG64(62)).integers(-32768, 32768, (M, N)).astype(np.int16)
     hi, lo = O.limb_split(G)
