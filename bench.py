@@ -108,11 +108,11 @@ def conv_workload(batch):
 # move O(channels) or O(pixels) bytes only.
 OPS_PER_ELEMENT_CONV = 2 * 9 * CIN          # 2*K per output element of fprop / dgrad
 KERNEL_WORK = {
-    ("range_partial_kernel", 0): (4, 0), ("quantize_kernel", 0): (5, 0),            # x: scan, then codes (+ per-pixel sums, per-channel totals)
+    ("range_partial_kernel", 0): (4, 0), ("quantize_pair_kernel", 0): (5, 0),       # x: scan, then codes (+ per-pixel sums, per-channel totals)
     ("qbp_mma_kernel", 0): (5, OPS_PER_ELEMENT_CONV),                               # fprop: 1 B codes in, 4 B fp32 out
     ("bn_stats_kernel", 0): (4, 0), ("bn_apply_kernel", 0): (8, 0),
     ("bn_bwd_stats_kernel", 0): (8, 0), ("bn_bwd_apply_kernel", 0): (12, 0),
-    ("quantize_kernel", 1): (7, 0),                                                 # bifurcation: 4 B in, 1 + 2 B out
+    ("bifurcate_kernel", 0): (7, 0),                                                # bifurcation: 4 B in, 1 + 2 B out
     ("bn_bwd_apply_bifurcate_kernel", 0): (11, 0),                                  # dy and z in (8 B), the gradient's 8-bit copy and two limbs out (3 B)
     ("qbp_mma_kernel", 1): (5, OPS_PER_ELEMENT_CONV),                               # dgrad
     ("qbp_wgrad_kernel", 0): (3, 2 * OPS_PER_ELEMENT_CONV),                         # two int8 products per 16x8-bit product
@@ -513,7 +513,7 @@ def tbp_block(B, batch, hbm_peak, peaks, launches=30):
     out["xnor_forward_4096"] = {"ms": round(ms, 4), "tera_bit_macs_per_s": round(n ** 3 / (ms * 1e-3) / 1e12, 1),
                                 "int8_tops": round(2 * n ** 3 / (ms * 1e-3) / 1e12, 1),
                                 "frac_of_measured_burst": round(2 * n ** 3 / (ms * 1e-3) / 1e12 / (2 * float(peaks["bf16_tflops"])), 3),
-                                "includes": "the two code-sum kernels and the terms kernel of the call"}
+                                "includes": "the code-sum kernel of the call"}
     # the same product from bit rows on the popcount unit of the CUDA cores
     ab, bb = B.qbp_pack_bits(qa), B.qbp_pack_bits(qb.t().contiguous())
     oc = torch.empty((n, n), dtype=torch.int32, device="cuda")

@@ -767,7 +767,7 @@ static int launch_quantize(const float *x, int64_t n, int64_t cols, int perch, i
         QBP_TRACE_BEGIN(st);
         if (id8 == id16) launch(bifurcate_kernel<true>, grid_for(blocks_per_sm<bifurcate_kernel<true>>(kThreads), groups), kThreads, 0, st, J, key);
         else             launch(bifurcate_kernel<false>, grid_for(blocks_per_sm<bifurcate_kernel<false>>(kThreads), groups), kThreads, 0, st, J, key);
-        QBP_LAUNCH_OK("quantize_kernel");
+        QBP_LAUNCH_OK("bifurcate_kernel");
         return QBP_OK;
     }
     if (totals) QBP_QUANT(false, true);           // (vector path, per tensor: checked above)
@@ -971,7 +971,7 @@ int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, s
         QBP_TRACE_BEGIN(st);
         if (totals) launch(quantize_pair_kernel<true>, (int)(ga + gb), kThreads, (size_t)x->cols * 2 * sizeof(int), st, ja, jb, (int)gb);
         else        launch(quantize_pair_kernel<false>, (int)(ga + gb), kThreads, 0, st, ja, jb, (int)gb);
-        QBP_LAUNCH_OK("quantize_kernel");
+        QBP_LAUNCH_OK("quantize_pair_kernel");
         return QBP_OK;
     }
     for (int i = 0; i < 2; ++i) {

@@ -1023,7 +1023,7 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
         if (nb == 8)      launch(wgrad_conv_finalize_kernel<8>, grid, 256, 0, st, P);
         else if (nb == 4) launch(wgrad_conv_finalize_kernel<4>, grid, 256, 0, st, P);
         else              launch(wgrad_conv_finalize_kernel<2>, grid, 256, 0, st, P);
-        QBP_LAUNCH_OK("wgrad_finalize_kernel");
+        QBP_LAUNCH_OK("wgrad_conv_finalize_kernel");
     } else if (!P.direct) {
         const int blocks = (int)((outs * kWgFinalizeLanes + 255) / 256);
         QBP_TRACE_BEGIN(st);
