@@ -280,12 +280,10 @@ __global__ void __launch_bounds__(256) bn_out_range_kernel(const float *__restri
 // channel's maximum, where it is its minimum, and everywhere else -- as ext [6][blocks][C] (min, max of the ordinary
 // positions, then of the maxima, then of the minima).  dx is a monotone function of dy on each set (bn_dx), so the
 // finalize kernel knows the exact range of dx from these, before dx is computed.
-// Loads that leave their lines in the L2 (the others pass through, evict-first) where the second pass is bound by HBM and finds them
-// there.  Before the bifurcating pass that also writes the gradient, which walks from the end: the last kKeepBytes of the two tensors
-// (25.7 M elements 74 -> 68 us).  Before the plain pass, which walks from the front: both tensors, when they fit kKeepBytes together
-// (two of 26 MB, statistics and second pass 31.4 -> 28.4 us; keeping the end of larger ones changes nothing, 2 x 51 to 2 x 206 MB).
-// The bifurcating pass alone is bound by arithmetic and gains nothing (the layers of 56 x 56 x 64 and 14 x 14 x 256 lose a
-// microsecond).  More than the L2 holds beside the writes (88 MB) only costs.
+// The last kKeepBytes of both tensors are read with loads that leave them in the L2 (the rest passes through, evict-first) when the
+// second pass is bound by HBM, which then starts with them: the plain one (51 MB: 33 -> 31 us) and the bifurcating one that also
+// writes the gradient (25.7 M elements 74 -> 68 us).  The bifurcating pass alone is bound by arithmetic and gains nothing (the layers of
+// 56 x 56 x 64 and 14 x 14 x 256 lose a microsecond).  More than the L2 holds beside the writes (88 MB) only costs.
 constexpr int64_t kKeepBytes = 64ll << 20;
 template <int VEC, bool RELU, bool EXT>
 __global__ void __launch_bounds__(kScanThreads) bn_bwd_stats_kernel(const float *__restrict__ dy,
@@ -1254,9 +1252,7 @@ static int bn_bwd_stats_launch(const float *dy, const float *x, int64_t n_rows, 
     const dim3 grid(g.nbx, g.slabs);
     const double Cnd = 1.0 / std::sqrt(2.0 * std::log((double)n_stat));
     const float Cn = (float)Cnd;
-    const int64_t keep_rows = kKeepBytes / (2 * (int64_t)sizeof(float) * C);
-    const bool keep = ext ? keep_tail : n_rows <= keep_rows;
-    const int64_t keep_from = keep ? std::max<int64_t>(0, n_rows - keep_rows) : n_rows;
+    const int64_t keep_from = keep_tail ? std::max<int64_t>(0, n_rows - kKeepBytes / (2 * (int64_t)sizeof(float) * C)) : n_rows;
     QBP_TRACE_BEGIN(st);
 #define QBP_BN_BSTATS(V, R, E) launch(bn_bwd_stats_kernel<V, R, E>, grid, kScanThreads, 0, st, dy, x, n_rows, (int)C, g.tw, save_mean, save_min, save_max, gamma, beta, Cn, pa, pb, ext, zero, keep_from)
     if (ext) {
