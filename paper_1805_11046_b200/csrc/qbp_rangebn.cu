@@ -281,9 +281,11 @@ __global__ void __launch_bounds__(256) bn_out_range_kernel(const float *__restri
 // positions, then of the maxima, then of the minima).  dx is a monotone function of dy on each set (bn_dx), so the
 // finalize kernel knows the exact range of dx from these, before dx is computed.
 // The last kKeepBytes of both tensors are read with loads that leave them in the L2 (the rest passes through, evict-first) when the
-// second pass is bound by HBM, which then starts with them: the plain one (51 MB: 33 -> 31 us) and the bifurcating one that also
-// writes the gradient (25.7 M elements 74 -> 68 us).  The bifurcating pass alone is bound by arithmetic and gains nothing (the layers of
-// 56 x 56 x 64 and 14 x 14 x 256 lose a microsecond).  More than the L2 holds beside the writes (88 MB) only costs.
+// second pass is bound by HBM.  The bifurcating pass that also writes the gradient starts with them (25.7 M elements 74 -> 68 us).  The
+// plain pass walks from the front: it gains where both tensors fit (two of 26 MB, statistics and second pass 31.4 -> 28.4 us), a little
+// where half of them does (two of 51 MB with their forward 86.4 -> 86.0), and nothing of larger ones.  The bifurcating pass alone is
+// bound by arithmetic and gains nothing (the layers of 56 x 56 x 64 and 14 x 14 x 256 lose a microsecond).  More than the L2 holds
+// beside the writes (88 MB) only costs.
 constexpr int64_t kKeepBytes = 64ll << 20;
 template <int VEC, bool RELU, bool EXT>
 __global__ void __launch_bounds__(kScanThreads) bn_bwd_stats_kernel(const float *__restrict__ dy,
