@@ -42,9 +42,13 @@ void trace_end(const char *name, cudaStream_t st);
 // launch() marks every kernel as a programmatic dependent of its predecessor, whose blocks let it go as they exit, and each kernel
 // waits, before it touches the predecessor's results, until those are visible (pdl_wait).  A chain of dependent small kernels then
 // costs about 2 us each instead of 4 to 5.  Only the short kernels whose successor is a product (code sums and zero-point terms) let
-// it go at their start (pdl_trigger), so that it allocates its tensor memory beside them (ternary layer 212 -> 206 us, layer
-// 14 x 14 x 256 255 -> 251): elsewhere blocks that wait on an SM beside the running kernel made that kernel slower (per-channel
-// statistics of 51 MB 14.5 -> 20 us, the layer of 56 x 56 x 64 543 -> 577 us, three layers' inference at batch 8 106 -> 117 us).  While launches are timed one by one the dependency is the ordinary one.
+// it go while they run (pdl_trigger): elsewhere blocks that wait on an SM beside the running kernel made that kernel slower (per-channel
+// statistics of 51 MB 14.5 -> 20 us, the layer of 56 x 56 x 64 543 -> 577 us, three layers' inference at batch 8 106 -> 117 us).  They do
+// so behind their own wait: all that was launched before them is complete then, the product's operands and parameters among it, and
+// the product, told that its launch follows one of them (`beside`), starts on its operands at once; only its epilogue, which reads
+// the sums or terms and writes the output, waits for their end.  (Layer gradient of 16 x 7 x 7, 512 -> 512 channels, with its terms:
+// 27.6 -> 21.6 us; the layer of 20 x 19 x 19, 96 -> 160, 92.8 -> 91.2; the low-bit layer 196.5 -> 194.4.)
+// While launches are timed one by one the dependency is the ordinary one.
 bool trace_is_on();
 template <typename... P, typename... A>
 inline void launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A &&...args)
@@ -111,7 +115,7 @@ struct ZeroJobs { uint32_t *p[2]; int64_t words[2]; };
 // -------------------------------------------------------------- device side
 #ifdef __CUDACC__
 
-// The two halves of a programmatic launch (see launch()).  Only code_sums_kernel and conv_terms_kernel trigger.  A kernel that
+// The two halves of a programmatic launch (see launch()).  Only code_sums_kernel and conv_terms_kernel trigger, behind their wait.  A kernel that
 // allocates tensor memory never does: its successor could take that memory first and then wait for a kernel that cannot go on.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -582,6 +586,17 @@ __device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, uint32_t (&r)[32])
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
           "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr)
+        : "memory");
+}
+// ... 16 columns
+__device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t (&r)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr)
         : "memory");
 }

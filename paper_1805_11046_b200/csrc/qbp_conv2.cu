@@ -39,6 +39,7 @@ struct Conv2Params {
     const int32_t *rowterm, *colterm;              // [positions], [16 border classes][N]
     const qbp_qparams *qa, *qb;
     float *st_lo, *st_hi; double *st_sum;          // per-channel statistics of the output, a row per CTA (NULL: not wanted)
+    int beside;                      // the launch before writes the terms and neither operands nor parameters: only the epilogue waits for it
     int *status;
 };
 
@@ -157,7 +158,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kC2Threads, 1) qbp_c
                         const uint32_t bar = map_to_cta(&full_bar[s], 0);
                         if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * stage_bytes);
                         const int c0 = cc * 128, r = tap / 3, t = tap - 3 * r;
-                        if (!waited) { pdl_wait(); waited = true; }
+                        if (!waited) { if (!P.beside) pdl_wait(); waited = true; }
                         // forward: input row p - 1 + r feeds output row p; layer gradient: gradient row h + 1 - r feeds input row h
                         if (!P.dgrad) {
                             tma_load_4d_pair(sa, &P.mapA, bar, c0, o.w0 + t - 1, o.h0 + r - 1, o.img0);
@@ -180,7 +181,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kC2Threads, 1) qbp_c
             A.k_iters = P.k_iters; A.stages = (uint32_t)P.stages; A.cg = (uint32_t)P.cg; A.nbuf = (uint32_t)P.nbuf;
             A.tile0 = pair; A.tiles_total = P.tiles_total; A.tile_step = P.pairs;
             // (a barrier's wait is bounded: its clock starts once the producer's copies can)
-            pdl_wait();
+            if (!P.beside) pdl_wait();
             timed_out = !(!P.dgrad ? conv2_mma_loop<2, 128>(A) : P.bn == 256 ? conv2_mma_loop<256, 128>(A) : conv2_mma_loop<128, 64>(A));
         }
     } else {
@@ -341,6 +342,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kC2Threads, 1) qbp_c
     }
 
     if (timed_out) {
+        pdl_wait();                      // (a launch before may clear the word)
         raise_timeout(P.status);
         __nanosleep(1000000);
     }
@@ -367,14 +369,14 @@ bool conv2_eligible(const qbp_conv_desc *d, bool dgrad)
 
 int launch_conv2(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp_qparams *q_in, const int8_t *wgt,
                  const qbp_qparams *q_w, int32_t *acc_out, float *out, const int32_t *rowterm, const int32_t *colterm,
-                 ColStatParts *stats, int *status, int bwl, int bhl, cudaStream_t st)
+                 ColStatParts *stats, int *status, int bwl, int bhl, bool beside, cudaStream_t st)
 {
     Conv2Params P{};
     const int Cred = dgrad ? d->K : d->C, Nout = dgrad ? d->C : d->K;
     const int bw = 1 << bwl, bh = 1 << bhl, bimg = 128 >> (bwl + bhl);
     const int tiles_w = (d->W + bw - 1) / bw, tiles_h = (d->H + bh - 1) / bh;
     const int64_t boxes = (int64_t)tiles_w * tiles_h * ((d->N + bimg - 1) / bimg);
-    P.dgrad = dgrad ? 1 : 0;
+    P.dgrad = dgrad ? 1 : 0; P.beside = beside ? 1 : 0;
     P.bn = conv2_bn(boxes, Nout);
     P.nbuf = 512 / P.bn;
     int rc;

@@ -129,10 +129,10 @@ static int conv_rangebn_recompute(const qbp_conv_desc *d, const int8_t *x_codes,
                                   const int8_t *w_codes, const qbp_qparams *qw, const float *gamma, const float *beta, int relu,
                                   float *save_mean, float *save_min, float *save_max, const qbp_requant *out,
                                   ColStatParts parts, float4 *fold, const CodeSums &w_sums, int *status, void *ws, size_t scratch,
-                                  cudaStream_t st)
+                                  bool beside, cudaStream_t st)
 {
     const int64_t rows = (int64_t)d->N * d->H * d->W;
-    const EpilogueTail first{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums};
+    const EpilogueTail first{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums, nullptr, 0, beside};
     int rc = conv_s8_impl(QBP_CONV_FPROP, d, x_codes, qx, w_codes, qw, nullptr, nullptr, in_sums, &parts, status, ws, scratch, st,
                           &first);
     if (rc) return rc;
@@ -219,20 +219,21 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_fwd_chained(cons
     if (!wo.row_sums_left) jobs[njobs++] = w_job;
     if ((want_totals && x && !xo.tot_left) || chained_totals)
         jobs[njobs++] = SumJob{saved->x_codes, s.rows, s.cin, kSumCols, 1, nullptr, 0, 0, saved->x_chan_sums};
-    if (njobs && (rc = launch_code_sums(jobs, njobs, st))) return rc;
+    bool beside = false;
+    if (njobs && (rc = launch_code_sums(jobs, njobs, st, ZeroJobs{}, &beside))) return rc;
     const CodeSums w_sums = sums_of(w_job), x_sums = sums_of(in_sums);
     ColStatParts parts = l.parts;
     if (recompute)
         return conv_rangebn_recompute(&L->conv, saved->x_codes, saved->qx, in_sums, saved->w_codes, saved->qw, gamma, beta, L->relu,
                                       saved->save_mean, saved->save_min, saved->save_max, out, parts, l.fold, w_sums, status,
-                                      l.scratch, l.scratch_bytes, st);
-    const EpilogueTail with_sums{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums};
+                                      l.scratch, l.scratch_bytes, beside, st);
+    const EpilogueTail with_sums{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums, nullptr, 0, beside};
     if (s.conv)
         rc = conv_s8_impl(QBP_CONV_FPROP, &L->conv, saved->x_codes, saved->qx, saved->w_codes, saved->qw, nullptr, saved->z,
                           in_sums, parts.sum ? &parts : nullptr, status, l.scratch, l.scratch_bytes, st, &with_sums);
     else
         rc = gemm_s8_impl(0, 0, s.rows, s.cout, s.cin, saved->x_codes, saved->qx, saved->w_codes, saved->qw, nullptr,
-                          saved->z, nullptr, status, l.scratch, l.scratch_bytes, st, &x_sums, &w_sums);
+                          saved->z, nullptr, status, l.scratch, l.scratch_bytes, st, &x_sums, &w_sums, beside);
     if (rc) return rc;
     // the convolution's epilogue has left the statistics of z: no pass over z for them
     if (parts.sum)
@@ -311,10 +312,11 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_bwd(const qbp_la
     if (rc) return rc;
     // (a 3 x 3 convolution: in the launch of the layer gradient's correction terms)
     const bool with_terms = s.conv && L->conv.R == 3;
-    if (!with_terms && nlate && (rc = launch_code_sums(late, nlate, st))) return rc;
+    bool beside = false;
+    if (!with_terms && nlate && (rc = launch_code_sums(late, nlate, st, ZeroJobs{}, &beside))) return rc;
     const CodeSums w_sums = sums_of(w_job), g_sums = sums_of(l.row_sums);
     if (s.conv) {
-        const EpilogueTail with_sums{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums, late, with_terms ? nlate : 0};
+        const EpilogueTail with_sums{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums, late, with_terms ? nlate : 0, beside};
         rc = conv_s8_impl(QBP_CONV_DGRAD, &L->conv, g8, qp8, saved->w_codes, saved->qw, nullptr, dx, l.row_sums, nullptr, status,
                           l.scratch, l.scratch_bytes, st, &with_sums);
         if (rc) return rc;
@@ -323,7 +325,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_bwd(const qbp_la
     }
     // dx [batch x in] = g8 [batch x out] . w^T, w stored [in x out]
     rc = gemm_s8_impl(0, 1, s.rows, s.cin, s.cout, g8, qp8, saved->w_codes, saved->qw, nullptr, dx, nullptr, status, l.scratch,
-                      l.scratch_bytes, st, &g_sums, &w_sums);
+                      l.scratch_bytes, st, &g_sums, &w_sums, beside);
     if (rc) return rc;
     return wgrad_s16_impl(nullptr, s.rows, s.cout, s.cin, saved->x_codes, saved->qx, ghi, glo, qp16, nullptr, dw, status, l.scratch,
                           l.scratch_bytes, st, nullptr, nullptr, true, true, l.wg_sums);

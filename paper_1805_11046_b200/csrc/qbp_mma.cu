@@ -220,6 +220,7 @@ struct MmaParams {
     const int32_t *rowterm;       // [M]
     const int32_t *colterm;       // [ncls][N]
     int raw_sums, k_len;
+    int beside;                   // the launch before makes the sums or terms: only the epilogue waits for it
     CodeSums a_sums, b_sums;
     const qbp_qparams *qa, *qb;
     int *status;
@@ -465,7 +466,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
         // Lane 0 owns the barriers.  Convolution: the `ips` activation tiles of a stage are issued by
         // `ips` lanes at once, each from its own entry of the k-iteration table.
         bool waited = false;
-        auto wait_once = [&] { if (!waited) { pdl_wait(); waited = true; } };
+        auto wait_once = [&] { if (!waited) { if (!P.beside) pdl_wait(); waited = true; } };
         if (P.b_resident && lane == 0) {
             // the filter is the same for every tile of this CTA: fetch it once
             mbar_expect_tx(&b_full, P.b.tile_bytes * (uint32_t)P.k_iters);
@@ -551,7 +552,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
         // The whole warp walks the tiles and stages in step, so that ring positions, descriptors and accumulator
         // addresses stay warp-uniform; an elected lane issues the MMAs and the commits.
         // (a barrier's wait is bounded: its clock starts once the producer's copies can)
-        pdl_wait();
+        if (!P.beside) pdl_wait();
         if (P.b_resident && !mbar_wait_uniform(&b_full, 0)) timed_out = true;
         const uint32_t bres_addr = smem_u32(smem_b);
         const uint32_t ring_addr = smem_u32(smem);
@@ -843,6 +844,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) qbp_mma_kernel(const __grid_co
     }
 
     if (timed_out) {
+        pdl_wait();                    // (the launch before may clear the word)
         raise_timeout(P.status);
         __nanosleep(1000000);          // let copies already in flight land before the CTA retires
     }
@@ -871,8 +873,8 @@ struct ConvTerms {
 // The first `sum_blocks` blocks take code sums that a later product needs (a launch less, and they overlap).
 __global__ void __launch_bounds__(256, 6) conv_terms_kernel(const __grid_constant__ ConvTerms T, const __grid_constant__ SumJobs J, int sum_blocks)
 {
-    pdl_trigger();                       // (see launch())
     pdl_wait();
+    pdl_trigger();                       // (see launch())
     if ((int)blockIdx.x < sum_blocks) { code_sums_block(J, (int)blockIdx.x); return; }
     const int block = (int)blockIdx.x - sum_blocks;
     if (block >= T.row_blocks) {
@@ -1219,7 +1221,8 @@ extern "C" __attribute__((visibility("default"))) int qbp_gemm_s8_sums(int trans
 
 int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,
                       const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const qbp_epilogue *ep,
-                      int *ext_status, void *ws, size_t ws_bytes, cudaStream_t st, const CodeSums *a_sums, const CodeSums *b_sums)
+                      int *ext_status, void *ws, size_t ws_bytes, cudaStream_t st, const CodeSums *a_sums, const CodeSums *b_sums,
+                      bool beside)
 {
     if (M <= 0 || N <= 0 || K <= 0) return fail(QBP_ERR_INVALID_ARG, "gemm_s8: M, N, K must be positive");
     if (M % 16 || N % 16 || K % 16) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "gemm_s8: M, N, K must be multiples of 16");
@@ -1259,12 +1262,14 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
     int rc = QBP_OK;
     ZeroJobs zero{};
     if (!ext_status) { zero.p[0] = reinterpret_cast<uint32_t *>(status); zero.words[0] = 1; }
-    if ((rc = launch_code_sums(jobs, njobs, st, zero))) return rc;
+    bool own = false;
+    if ((rc = launch_code_sums(jobs, njobs, st, zero, &own))) return rc;
+    beside = njobs ? own : beside && !zero.words[0];         // (a tail's launch for its parameters comes in between)
 
     // large products run on CTA pairs (256 x 256 tiles across two SMs); the column statistics are the
     // single-CTA kernel's (at most 256 columns: narrow either way)
     if (gemm2_eligible(M, N, K) && !stats && !has_tail)
-        return launch_gemm2(transA, transB, M, N, K, A, qa, B, qb, acc_out, C, asum, bsum, status, st);
+        return launch_gemm2(transA, transB, M, N, K, A, qa, B, qb, acc_out, C, asum, bsum, status, beside, st);
 
     MmaParams P{};
     P.mode = MODE_GEMM;
@@ -1311,6 +1316,7 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
     P.one_tile = P.msub == 1 && (M + 127) / 128 * P.tiles_n <= sm_count() ? 1 : 0;
     P.M = M; P.N = N;
     P.acc_out = acc_out; P.out = C;
+    P.beside = beside && !has_tail ? 1 : 0;
     P.raw_sums = 1; P.k_len = (int)K; P.a_sums = asum; P.b_sums = bsum; P.qa = qa; P.qb = qb; P.status = status;
     if (stats) { P.st_lo = parts.lo; P.st_hi = parts.hi; P.st_sum = parts.sum; }
     bool fused_row_sums = false;
@@ -1422,13 +1428,16 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
     if (in_chan_sum) chan_sum = const_cast<int32_t *>(in_chan_sum);
     ZeroJobs zero{};
     if (!ext_status) { zero.p[0] = reinterpret_cast<uint32_t *>(status); zero.words[0] = 1; }
+    bool beside = tail && tail->beside && !zero.words[0];    // (whether the launch before the product is one that it may run beside)
     if (tail && tail->keep_terms) { if ((rc = launch_code_sums(nullptr, 0, st, zero))) return rc; }
     else {
         SumJob jobs[2];
         int njobs = 0;
         if (!in_chan_sum) jobs[njobs++] = SumJob{in, pix, Cred, kSumRows, 1, chan_sum};
         if (own_wsums) jobs[njobs++] = w_job;
-        if ((rc = launch_code_sums(jobs, njobs, st, zero))) return rc;
+        bool own = false;
+        if ((rc = launch_code_sums(jobs, njobs, st, zero, &own))) return rc;
+        beside = njobs ? own : beside;
         if (!raw_sums) {
             ConvTerms T{};
             const int per_img = (d->H * d->W + 255) / 256;
@@ -1441,6 +1450,7 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
             QBP_TRACE_BEGIN(st);
             launch(conv_terms_kernel, sum_blocks + T.row_blocks + (16 * Nout + 255) / 256, 256, 0, st, T, J, sum_blocks);
             QBP_LAUNCH_OK("conv_terms_kernel");
+            beside = true;
         }
     }
 
@@ -1448,7 +1458,7 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
     pick_pixel_box(d->N, d->H, d->W, bwl, bhl);
     // 3 x 3 with many channels on both sides: CTA pairs (the epilogue's tail is the single-CTA kernel's)
     if (conv2_eligible(d, dgrad) && !(tail && (tail->fold || tail->relu || tail->q)))
-        return launch_conv2(dgrad, d, in, q_in, wgt, q_w, acc_out, out, rowterm, colterm, stats, status, bwl, bhl, st);
+        return launch_conv2(dgrad, d, in, q_in, wgt, q_w, acc_out, out, rowterm, colterm, stats, status, bwl, bhl, beside, st);
 
     MmaParams P{};
     P.mode = dgrad ? MODE_DGRAD : MODE_FPROP;
@@ -1516,6 +1526,7 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
     P.idesc = make_idesc(true, true, P.a.major, P.b.major, 128, (uint32_t)P.bn);
     P.acc_out = acc_out; P.out = out;
     P.rowterm = rowterm; P.colterm = colterm; P.qa = q_in; P.qb = q_w; P.status = status;
+    P.beside = beside ? 1 : 0;
     P.raw_sums = raw_sums ? 1 : 0; P.k_len = Cred; P.a_sums = sums_of(chan_sum); P.b_sums = w_sums;
     // each row's code sum comes from the epilogue when one column tile holds the whole row, else from a pass over the codes
     const bool fused_row_sums = want_codes && tail->row_sums && P.tiles_n == 1;

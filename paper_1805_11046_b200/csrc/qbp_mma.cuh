@@ -50,7 +50,11 @@ inline CodeSums sums_of(const SumJob &j)
 {
     return j.kind == kSumRows ? sums_of(j.out) : CodeSums{j.out, sum_pieces(j.rows, j.cols), j.cols};
 }
-int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st, const ZeroJobs &zero = ZeroJobs{});
+// beside (nullable): set when the product launched next may run beside this kernel (see launch()).  Sums of fewer bytes than
+// kSumsBesideBytes take a microsecond or two, less than the product's launch: they let it go at their start, and it waits for them
+// (a linear layer of 64 x 256 -> 128 37.6 us otherwise, 37.4 so; of 1024 x 2048 -> 1008 77.6 beside, 78.3 waiting).
+constexpr int64_t kSumsBesideBytes = 1 << 20;
+int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st, const ZeroJobs &zero = ZeroJobs{}, bool *beside = nullptr);
 
 // ---- per-tensor range scan (qbp_quant.cu): leaves *nparts (min, max) pairs at ws, for RangeSrc::parts -------------
 size_t range_scan_ws_bytes();
@@ -104,8 +108,9 @@ int rangebn_fold_from_parts(int64_t n, int64_t C, const float *gamma, const floa
 // call just before on the same workspace and are not run again.
 // w_sums (nullable): the filter's code sums (forward [K * taps], layer gradient [taps * C]) are there already.
 // extra [extra_count] (3 x 3): code sums of a later product, taken in the launch that makes this one's correction terms.
+// beside: the launch before the call was code_sums_kernel (see launch()).
 struct EpilogueTail { const float4 *fold; int relu; const qbp_qparams *rq; int8_t *q; int32_t *row_sums; int keep_terms; const CodeSums *w_sums;
-                      const SumJob *extra = nullptr; int extra_count = 0; };
+                      const SumJob *extra = nullptr; int extra_count = 0; bool beside = false; };
 size_t filter_sum_elems(const qbp_conv_desc *d);
 SumJob filter_sum_job(const qbp_conv_desc *d, bool dgrad, const int8_t *w, int32_t *out);
 
@@ -117,7 +122,7 @@ int conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const qbp_q
 int gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,
                  const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const qbp_epilogue *ep,
                  int *ext_status, void *ws, size_t ws_bytes, cudaStream_t st, const CodeSums *a_sums = nullptr,
-                 const CodeSums *b_sums = nullptr);
+                 const CodeSums *b_sums = nullptr, bool beside = false);
 // tot_x [C] / tot_g16 [K] (convolution; nullable, both or none): per-channel totals of the stored x codes and of the
 // stored 16-bit gradient codes (256 * hi + lo) over all positions, left by the kernels that wrote the codes.
 // lo_signed: g_lo holds the low bytes with the top bit flipped, i.e. the signed bytes lo - 128 (lo_signed in
@@ -165,19 +170,19 @@ int make_map_out_nhwc(CUtensorMap *map, float *base, uint64_t N, uint64_t H, uin
 bool gemm2_eligible(int64_t M, int64_t N, int64_t K);
 int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,
                  const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const CodeSums &a_sums,
-                 const CodeSums &b_sums, int *status, cudaStream_t st);
+                 const CodeSums &b_sums, int *status, bool beside, cudaStream_t st);
 
 // ---- the 3 x 3 convolution products on CTA pairs (qbp_conv2.cu); bwl / bhl: log2 of the position box's extents ----
 bool conv2_eligible(const qbp_conv_desc *d, bool dgrad);
 int launch_conv2(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp_qparams *q_in, const int8_t *wgt,
                  const qbp_qparams *q_w, int32_t *acc_out, float *out, const int32_t *rowterm, const int32_t *colterm,
-                 ColStatParts *stats, int *status, int bwl, int bhl, cudaStream_t st);
+                 ColStatParts *stats, int *status, int bwl, int bhl, bool beside, cudaStream_t st);
 
 // ---- the dense weight gradient on CTA pairs (qbp_wgrad2.cu) ----------------------
 bool wgrad2_eligible(int64_t M, int64_t N, int64_t K);
 int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qparams *qx, const int8_t *g_hi,
                   const uint8_t *g_lo, const qbp_qparams *qg16, int64_t *acc_out, float *dW, const CodeSums &sx,
-                  const CodeSums &shi, const CodeSums &slo, int *status, cudaStream_t st, bool lo_signed = false);
+                  const CodeSums &shi, const CodeSums &slo, int *status, bool beside, cudaStream_t st, bool lo_signed = false);
 
 // ---- shared-memory operand descriptors ---------------------------------------
 // How one operand tile of a pipeline stage is laid out and walked by the MMAs.

@@ -41,6 +41,7 @@ struct Mma2Params {
     int32_t *acc_out; float *out;
     CodeSums a_sums, b_sums;         // along the reduction: rowterm = -zb * a_sums[m] + K * za * zb, colterm = -za * b_sums[n]
     int k_len;
+    int beside;                      // the launch before makes the code sums: only the epilogue waits for it
     const qbp_qparams *qa, *qb;
     int *status;
 };
@@ -170,7 +171,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
                     const uint32_t bar = map_to_cta(&full_bar[s], 0);
                     if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * stage_bytes);
                     const int k0 = it * 128;
-                    if (!waited) { pdl_wait(); waited = true; }
+                    if (!waited) { if (!P.beside) pdl_wait(); waited = true; }
                     for (int sub = 0; sub < P.msub; ++sub) {
                         if (P.a.major == 0) tma_load_2d_pair(sa + sub * P.a.tile_bytes, &P.mapA, bar, k0, m_mine + 256 * sub);
                         else                tma_load_2d_pair(sa + sub * P.a.tile_bytes, &P.mapA, bar, m_mine + 256 * sub, k0);
@@ -193,7 +194,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
             A.tile0 = pair; A.tiles_total = P.tiles_total; A.tile_step = P.pairs;
             bool ok;
             // (a barrier's wait is bounded: its clock starts once the producer's copies can)
-            pdl_wait();
+            if (!P.beside) pdl_wait();
             if (P.msub == 2) {
                 if (P.a.major == 0) ok = P.b.major == 0 ? pair_mma_loop<2, 2, 2>(A) : pair_mma_loop<2, 256, 2>(A);
                 else                ok = P.b.major == 0 ? pair_mma_loop<256, 2, 2>(A) : pair_mma_loop<256, 256, 2>(A);
@@ -294,6 +295,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
     }
 
     if (timed_out) {
+        pdl_wait();                      // (the launch before may clear the word)
         raise_timeout(P.status);
         __nanosleep(1000000);
     }
@@ -312,7 +314,7 @@ bool gemm2_eligible(int64_t M, int64_t N, int64_t K)
 
 int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,
                  const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const CodeSums &a_sums,
-                 const CodeSums &b_sums, int *status, cudaStream_t st)
+                 const CodeSums &b_sums, int *status, bool beside, cudaStream_t st)
 {
     Mma2Params P{};
     int rc;
@@ -342,7 +344,7 @@ int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const 
     if (stages < 2 * P.cg) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "gemm_s8: the pair kernel's ring does not fit");
     P.stages = stages;
     P.M = M; P.N = N; P.acc_out = acc_out; P.out = C;
-    P.a_sums = a_sums; P.b_sums = b_sums; P.k_len = (int)K; P.qa = qa; P.qb = qb; P.status = status;
+    P.a_sums = a_sums; P.b_sums = b_sums; P.k_len = (int)K; P.beside = beside ? 1 : 0; P.qa = qa; P.qb = qb; P.status = status;
     const size_t smem = 1024 + (size_t)stages * stage_bytes + k2EpiWarps * k2Slab;
     static PerDeviceOnce configured;
     QBP_SMEM_OPT_IN(configured, qbp_mma2_kernel, k2Smem);

@@ -575,8 +575,9 @@ __global__ void __launch_bounds__(kThreads) quantize_pair_kernel(const __grid_co
 // The sums of up to eight code tensors in a launch of their own (see qbp_sums.cuh).
 __global__ void __launch_bounds__(kSumThreads) code_sums_kernel(const __grid_constant__ SumJobs J)
 {
-    pdl_trigger();                       // (see launch())
+    if (!J.beside) pdl_trigger();        // (see launch())
     pdl_wait();
+    if (J.beside) pdl_trigger();
     run_zero_jobs(J.zero, (int64_t)blockIdx.x * kSumThreads + threadIdx.x, (int64_t)gridDim.x * kSumThreads);
     code_sums_block(J, (int)blockIdx.x);
 }
@@ -640,8 +641,9 @@ int fill_sum_jobs(const SumJob *jobs, int count, SumJobs &J, int *blocks)
     return QBP_OK;
 }
 
-int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st, const ZeroJobs &zero)
+int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st, const ZeroJobs &zero, bool *beside)
 {
+    if (beside) *beside = false;
     if (count == 0) {
         for (int k = 0; k < 2; ++k)
             if (zero.words[k]) QBP_CUDA_OK(cudaMemsetAsync(zero.p[k], 0, sizeof(uint32_t) * (size_t)zero.words[k], st));
@@ -651,6 +653,9 @@ int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st, const ZeroJ
     int blocks = 0;
     if (int rc = fill_sum_jobs(jobs, count, J, &blocks)) return rc;
     J.zero = zero;
+    int64_t bytes = 0;
+    for (int i = 0; i < count; ++i) bytes += jobs[i].rows * jobs[i].cols;
+    if (beside && bytes >= kSumsBesideBytes) { *beside = true; J.beside = 1; }
     QBP_TRACE_BEGIN(st);
     launch(code_sums_kernel, blocks, kSumThreads, 0, st, J);
     QBP_LAUNCH_OK("code_sums_kernel");

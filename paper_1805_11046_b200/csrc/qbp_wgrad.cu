@@ -978,9 +978,10 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
             if (!done_sums) { zero.p[1] = reinterpret_cast<uint32_t *>(P.ones_tot); zero.words[1] = 2 * N; }
         }
     }
-    if ((rc = launch_code_sums(jobs, njobs, st, zero))) return rc;
+    bool beside = false;
+    if ((rc = launch_code_sums(jobs, njobs, st, zero, &beside))) return rc;
     if (pair_kernel)
-        return launch_wgrad2(M, N, K, x, qx, g_hi, g_lo, qg16, acc_out, dW, P.sx, P.shi, P.slo, status, st, lo_signed);
+        return launch_wgrad2(M, N, K, x, qx, g_hi, g_lo, qg16, acc_out, dW, P.sx, P.shi, P.slo, status, beside, st, lo_signed);
 
     P.part = (long long *)part; P.status = status;
     P.qx = qx; P.qg = qg16; P.acc_out = (long long *)acc_out; P.dW = dW; P.dW_vec = aligned16(dW) ? 1 : 0;

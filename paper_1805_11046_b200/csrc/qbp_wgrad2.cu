@@ -44,6 +44,7 @@ struct Wgrad2Params {
     int64_t M, N, K;                 // reduction rows; output columns; output rows
     long long *acc_out; float *dW;
     CodeSums sx, shi, slo;           // code sums over the M rows: rowterm = -zg * sx[k] + M * zx * zg, colterm = -zx * (256 * shi[n] + slo[n])
+    int beside;                      // the launch before makes the code sums: only the epilogue waits for it
     int zg_shift;                    // 128 for signed low bytes (lo - 128 against zg - 128)
     const qbp_qparams *qx, *qg;
     int *status;
@@ -126,7 +127,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
                     const uint32_t bar = map_to_cta(&full_bar[s], 0);
                     if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * kW2StageBytes);
                     const int m0 = it * 128;
-                    if (!waited) { pdl_wait(); waited = true; }
+                    if (!waited) { if (!P.beside) pdl_wait(); waited = true; }
                     tma_load_2d_pair(sa, &P.mapX, bar, k_mine, m0);
                     tma_load_2d_pair(sa + 16384, &P.mapHi, bar, n_mine, m0);
                     tma_load_2d_pair(sa + 32768, &P.mapLo, bar, n_mine, m0);
@@ -141,7 +142,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
             const uint32_t ring = smem_u32(smem);
             uint32_t a_addr = ring;
             // (a barrier's wait is bounded: its clock starts once the producer's copies can)
-            pdl_wait();
+            if (!P.beside) pdl_wait();
             for (int tile = pair; tile < P.tiles_total && !timed_out; tile += P.pairs) {
                 if (!mbar_wait_uniform(&acc_empty, eph)) { timed_out = true; break; }
                 eph ^= 1u;
@@ -266,6 +267,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
     }
 
     if (timed_out) {
+        pdl_wait();                       // (the launch before may clear the word)
         raise_timeout(P.status);
         __nanosleep(1000000);
     }
@@ -287,7 +289,7 @@ bool wgrad2_eligible(int64_t M, int64_t N, int64_t K)
 
 int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qparams *qx, const int8_t *g_hi,
                   const uint8_t *g_lo, const qbp_qparams *qg16, int64_t *acc_out, float *dW, const CodeSums &sx,
-                  const CodeSums &shi, const CodeSums &slo, int *status, cudaStream_t st, bool lo_signed)
+                  const CodeSums &shi, const CodeSums &slo, int *status, bool beside, cudaStream_t st, bool lo_signed)
 {
     Wgrad2Params P{};
     int rc;
@@ -307,7 +309,7 @@ int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qp
     P.d_group = make_fastdiv(kW2GroupM * P.tiles_n);
     P.M = M; P.N = N; P.K = K;
     P.acc_out = (long long *)acc_out; P.dW = dW;
-    P.sx = sx; P.shi = shi; P.slo = slo; P.zg_shift = lo_signed ? 128 : 0; P.qx = qx; P.qg = qg16; P.status = status;
+    P.beside = beside ? 1 : 0; P.sx = sx; P.shi = shi; P.slo = slo; P.zg_shift = lo_signed ? 128 : 0; P.qx = qx; P.qg = qg16; P.status = status;
     static PerDeviceOnce configured;
     QBP_SMEM_OPT_IN(configured, qbp_wgrad2_kernel, kW2Smem);
     QBP_TRACE_BEGIN(st);

@@ -514,6 +514,21 @@ def test_conv_pairs(B, N, H, W, C, K, mode):
     _check_col_stats(out, stats)
 
 
+@pytest.mark.parametrize("N,H,W,C,K", [(5, 1, 9, 96, 128), (130, 9, 1, 128, 96), (300, 1, 1, 256, 112), (70, 2, 2, 96, 96), (2, 15, 15, 128, 256),
+                                       (1, 3, 64, 96, 272), (2, 3, 65, 96, 128), (1, 6, 130, 160, 96), (3, 1, 200, 96, 96), (1, 2, 255, 128, 128)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_conv_pairs_numbering_of_the_positions(B, N, H, W, C, K, mode):
+    """Images of one row or column (no padding that way, fewer taps), of a tile's exact size, one and several panels of columns with a
+    narrower last one: every accumulator, the output and its statistics."""
+    d = B.conv_desc(N, H, W, C, K, 3, 3, 1, 1); od = O.conv_desc(N, H, W, C, K, 3, 3, 1, 1)
+    inp = random_codes((N, H, W, C if mode == 0 else K), 84); w = random_codes((K, 3, 3, C), 85)
+    acc, out, ws, stats = B.qbp_conv_s8_implicit(mode, d, to_dev(inp), _qp(B, 0.5, 17), to_dev(w), _qp(B, 0.25, -23), want_acc=True, col_stats=True)
+    assert B.status_word(ws) == 0
+    oacc, oout, bad = O.conv_s8(mode, od, inp, 17, w, -23, 0.5, 0.25)
+    assert bad == 0 and np.array_equal(to_host(acc).ravel(), oacc.ravel()) and np.array_equal(to_host(out).ravel(), oout.ravel())
+    _check_col_stats(out, stats)
+
+
 # ------------------------------------------------- products that leave most of the machine idle: smaller tiles
 @pytest.mark.parametrize("M,N,K", [(48, 4736, 64), (48, 4752, 64), (128, 9488, 32), (240, 96, 160), (2304, 240, 48), (2432, 240, 48),
                                    (16, 37888, 16), (16, 37904, 16)])
