@@ -416,4 +416,554 @@ int launch_conv2(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp
     return QBP_OK;
 }
 
+// ============================================== without statistics: channels as the accumulator's rows
+// The same products where nobody wants the statistics of their output (layer gradients, the low-bit layer, plain calls).
+//
+// The accumulator's rows (tensor-memory lanes) are output channels, its columns output positions: the filter is the A operand and
+// the activation the B operand.  A tile is 256 channels x npos positions on a CTA pair (CTA r holds 128 channels of the filter, half
+// of the positions and the accumulator of its channels) or 128 channels x npos positions on a CTA of its own, npos at most 256.
+// An epilogue thread then owns a channel: the channel's zero-point term is a register, a position's a broadcast, and a position's 32
+// channels of a warp go out as one 128-byte line, where positions as rows stage every value in shared memory beside the operand
+// reads and copies that want its port.  (Statistics would stay in registers too, but in sums of other 32 values: the mean's last
+// bit changes with their grouping, and chained layers amplify that through their stochastic codes.  They keep the kernel above.)
+//
+// The positions of all images lie in one row of numbers: an image row takes W + 1 of them and an image H + 1 rows, the last
+// column and the last row being padding that the neighbours share, so that the input position of a tap is the output position
+// plus a constant.  A CTA's consecutive numbers and their neighbours (its window) are copied once per channel chunk, in boxes of 8,
+// 4, 2 and 1 image rows, and a tap's operand is the window read from a shifted start: the shared-memory swizzle is a function of the
+// address, so a start at any whole position reads what TMA wrote there.  The padding is then filled with the input's zero-point
+// code, so that it adds zero to every corrected sum and one term per channel serves all positions.
+// What bounds it: the operand bytes that all SMs together draw from the L2 (some 10 TB/s; 128 filter rows and a ninth of the window
+// per tap against 128 + bn / 2 rows above), then the epilogue's instructions; the MMAs of a tile run at the pipe's rate.  Measured
+// with the terms' kernel, before and after: 256 x 28 x 28, 128 -> 128 channels 55.5 -> 44.4 us, 8 x 40 x 40, 288 -> 288 37.8 -> 29.4,
+// 20 x 19 x 19, 160 -> 96 16.2 -> 14.3, 16 x 7 x 7, 512 -> 512 21.6 -> 18.5, 1024 x 1 x 1, 256 -> 256 16.3 -> 13.1.
+//
+// Roles per CTA: warp 0 copies filter tiles, warp 18 windows, warp 19 fills their padding, warp 1 issues the MMAs, warps 2..17 are
+// the epilogue.  Every wait is bounded; no TMA load uses cluster multicast.
+constexpr int kCtEpiWarps = 16;                 // (their chains of conversions, stores and comparisons are bound by latency: four warps a scheduler)
+constexpr int kCtThreads = 32 * (kCtEpiWarps + 4);
+constexpr int kCtMaxStages = 8;
+constexpr int kCtMaxWindows = 3;
+constexpr int kCtPanelWidth = 96;               // columns of an image taken together at most (two windows must fit)
+constexpr int kCtChunks = 4;                    // of 16 positions per epilogue warp and tile, at most
+constexpr int kCtBoxHeights = 4;                // windows are copied in boxes of 8, 4, 2 and 1 image rows
+constexpr uint32_t kCtTapBytes = 128u * 128u;   // a filter tile of one tap: 128 output x 128 reduction channels
+constexpr uint32_t kCtSmem = 225u * 1024u;
+
+// Where a number lies: panels of at most kCtPanelWidth columns of an image follow one another, hp rows of s numbers each.
+// One panel: number j of a row is column j, the last one padding.  Several: column first - 1 + j, a neighbour on either side.
+struct ConvTGrid {
+    int s, hp, np, wp, off;          // numbers per row, rows per panel, panels per image, columns per panel, its first column's j
+    int pr, pc;                      // rows / columns on either side that the taps reach (0: one row / column, one tap row / column)
+    FastDiv d_s, d_hp, d_np;
+    int64_t total;                   // numbers in all
+};
+struct CtRun { unsigned vmask; int second; int64_t m1, m2; };         // a chunk's positions: see the epilogue
+struct CtEpiShared { int32_t term[kCtEpiWarps][kCtChunks][16]; CtRun run[kCtEpiWarps][kCtChunks]; };
+
+struct ConvTParams {
+    CUtensorMap mapF, mapX[kCtBoxHeights];     // filter, activation
+    uint32_t f_desc_lo, x_desc_lo, idesc;
+    uint32_t window_bytes, window_start;       // room of a window; where its first number lies (the row it is in starts up to s - 1 before)
+    int dgrad;
+    int npos, npos_cta;              // positions of a tile, of a CTA's window
+    int stages, windows;             // ring stages of a tap row's filter tiles; windows in flight
+    int cchunks;                     // channel chunks of 128 (of a ragged last one the rest is zero on the activation side)
+    int tiles_n, tiles_total, units; // units (pairs or CTAs): a multiple of tiles_n, so that a unit meets one channel tile only
+    FastDiv d_tiles_n;
+    ConvTGrid g;
+    int Nimg, H, W, C, N, Cred;      // C: channels of the filter's innermost extent; N: channels produced
+    int32_t *acc_out; float *out;
+    const int32_t *rowterm, *colterm;          // [positions], [16 border classes][N]
+    const qbp_qparams *qa, *qb;
+    int beside;                      // the launch before writes the terms and neither operands nor parameters: only the epilogue waits for it
+    int *status;
+};
+
+// ---- MMA issue ------------------------------------------------------------------
+// The MMA takes its operands from the warp's few uniform registers: what the direction and the operand layouts fix is spelled as
+// constants and a tap's MMAs are unrolled.  With a tap's place in the window and in the filter's ring worked out per tap from
+// the parameters, four MMAs of 64 cycles took the warp 750.
+// The MMAs of one tap, in column T of COLS: 128 reduction channels.
+template <bool PAIR, bool DGRAD, int T, int COLS, bool FIRST>
+__device__ __forceinline__ void convt_issue_tap(uint32_t d_tmem, uint32_t f_lo, uint32_t x_lo, uint32_t idesc)
+{
+    constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);           // 128-byte swizzle, groups of eight rows 1024 bytes apart
+    constexpr uint32_t f_kstep = DGRAD ? 256u : 2u;                           // 32 reduction channels, in 16-byte units: rows of the tile, or inside one
+    constexpr uint32_t col = DGRAD ? COLS - 1 - T : T;
+#pragma unroll
+    for (uint32_t kk = 0; kk < 4; ++kk) {
+        const uint64_t f = ((uint64_t)hi << 32) | (uint64_t)(f_lo + T * (kCtTapBytes >> 4) + kk * f_kstep);
+        const uint64_t x = ((uint64_t)hi << 32) | (uint64_t)(x_lo + col * 8u + kk * 2u);
+        if (elect_one()) {
+            if (PAIR) mma_i8_pair(d_tmem, f, x, idesc, (FIRST && kk == 0) ? 0u : 1u);
+            else      mma_i8(d_tmem, f, x, idesc, (FIRST && kk == 0) ? 0u : 1u);
+        }
+    }
+}
+
+struct ConvTMmaArgs {
+    uint64_t *full_bar, *empty_bar, *win_full, *win_empty, *acc_full, *acc_empty;
+    uint32_t windows_at, window_bytes, window_start, ring, tmem, f_desc_lo, x_desc_lo, idesc;
+    int cchunks, tap_rows;
+    int tap0, row_step;              // the first tap row's start in the window, from tap row to tap row, in 16-byte units
+    uint32_t stages, windows;
+    int tile0, tiles_total, tile_step;
+};
+template <bool PAIR>
+__device__ __forceinline__ void convt_commit(uint64_t *bar)
+{
+    if (elect_one()) { if (PAIR) mma_commit_pair(bar); else mma_commit(bar); }
+}
+// False when a wait ran out.
+template <bool PAIR, bool DGRAD, int COLS>
+__device__ __forceinline__ bool convt_mma_loop(const ConvTMmaArgs &A)
+{
+    constexpr uint32_t stage_bytes = kCtTapBytes * COLS;
+    uint32_t s = 0, ph = 0, buf = 0, bph = 1, f_addr = A.ring, win = 0, wph = 0, w_addr = A.windows_at;
+    for (int tile = A.tile0; tile < A.tiles_total; tile += A.tile_step) {
+        if (!mbar_wait_uniform(&A.acc_empty[buf], bph)) return false;
+        tc_fence_after();
+        const uint32_t d_tmem = A.tmem + buf * 256u;
+        bool first = true;
+        for (int cc = 0; cc < A.cchunks; ++cc) {
+            if (!mbar_wait_uniform(&A.win_full[win], wph)) return false;
+            uint32_t x_lo = ((((w_addr + A.window_start) >> 4) + (uint32_t)A.tap0) & 0x3FFFu) | A.x_desc_lo;
+            for (int r = 0; r < A.tap_rows; ++r, x_lo += (uint32_t)A.row_step) {
+                const uint32_t f_lo = ((f_addr >> 4) & 0x3FFFu) | A.f_desc_lo;
+                if (!mbar_wait_uniform(&A.full_bar[3 * s], ph)) return false;
+                tc_fence_after();
+                if (first) convt_issue_tap<PAIR, DGRAD, 0, COLS, true>(d_tmem, f_lo, x_lo, A.idesc);
+                else       convt_issue_tap<PAIR, DGRAD, 0, COLS, false>(d_tmem, f_lo, x_lo, A.idesc);
+                first = false;
+                if (COLS == 3) {
+                    if (!mbar_wait_uniform(&A.full_bar[3 * s + 1], ph)) return false;
+                    tc_fence_after();
+                    convt_issue_tap<PAIR, DGRAD, COLS == 3 ? 1 : 0, COLS, false>(d_tmem, f_lo, x_lo, A.idesc);
+                    if (!mbar_wait_uniform(&A.full_bar[3 * s + 2], ph)) return false;
+                    tc_fence_after();
+                    convt_issue_tap<PAIR, DGRAD, COLS == 3 ? 2 : 0, COLS, false>(d_tmem, f_lo, x_lo, A.idesc);
+                }
+                convt_commit<PAIR>(&A.empty_bar[s]);
+                f_addr += stage_bytes;
+                if (++s == A.stages) { s = 0; ph ^= 1u; f_addr = A.ring; }
+            }
+            convt_commit<PAIR>(&A.win_empty[win]);
+            w_addr += A.window_bytes;
+            if (++win == A.windows) { win = 0; wph ^= 1u; w_addr = A.windows_at; }
+        }
+        convt_commit<PAIR>(&A.acc_full[buf]);
+        buf ^= 1u;
+        if (buf == 0) bph ^= 1u;
+    }
+    return true;
+}
+
+// A position's value under a predicate: stored, and the pointer moved on.
+__device__ __forceinline__ void put_if(unsigned cond, uint32_t bits, char *&p, int64_t stride)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p st.global.b32 [%0], %2;\n\t@p add.s64 %0, %0, %3;\n\t}"
+                 : "+l"(p) : "r"(cond), "r"(bits), "l"(stride) : "memory");
+}
+
+// The image rows (of s numbers, counted through all panels, -1 the one before the first) that a CTA's window of a tile touches.
+struct ConvTRows { int first, count, start; };       // start: the window's first number
+__device__ __forceinline__ ConvTRows convt_rows(const ConvTParams &P, int tile_m, uint32_t rank)
+{
+    ConvTRows w;
+    const int reach = P.g.pr * P.g.s + P.g.pc;
+    w.start = tile_m * P.npos + P.npos_cta * (int)rank - reach;
+    w.first = P.g.d_s.div(w.start + 2 * P.g.s) - 2;                      // (reach <= 2 s)
+    w.count = P.g.d_s.div(w.start + P.npos_cta - 1 + 2 * reach + 2 * P.g.s) - 2 - w.first + 1;
+    return w;
+}
+
+template <bool PAIR>
+__global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(kCtThreads, 1) qbp_conv2t_kernel(const __grid_constant__ ConvTParams P)
+{
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t full_bar[3 * kCtMaxStages], empty_bar[kCtMaxStages], win_landed[kCtMaxWindows], win_full[kCtMaxWindows],
+        win_empty[kCtMaxWindows], acc_full[2], acc_empty[2];
+    __shared__ uint32_t tmem_slot;
+
+    const uint32_t raw_addr = smem_u32(smem_raw);
+    uint8_t *windows = smem_raw + ((1024u - (raw_addr & 1023u)) & 1023u);
+    uint8_t *ring = windows + (size_t)P.windows * P.window_bytes;
+    const uint32_t stage_bytes = kCtTapBytes * (P.g.pc ? 3u : 1u);
+    CtEpiShared &E = *reinterpret_cast<CtEpiShared *>(ring + (size_t)P.stages * stage_bytes);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
+    const int unit = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+    const int n_mine = (unit % P.tiles_n) * (PAIR ? 256 : 128) + 128 * (int)rank;                     // this CTA's first channel
+    constexpr uint32_t kCtas = PAIR ? 2u : 1u;
+
+    if (threadIdx.x == 0) {
+        // (pairs: the leader's "full" barriers count its own arrival and the bytes of both CTAs, "win_full" a window of each CTA, the
+        // "empty" ones a multicast commit, "acc_empty" the epilogue warps of both)
+        for (int s = 0; s < P.stages; ++s) { for (int t = 0; t < 3; ++t) mbar_init(&full_bar[3 * s + t], 1); mbar_init(&empty_bar[s], 1); }
+        for (int w = 0; w < P.windows; ++w) { mbar_init(&win_landed[w], 1); mbar_init(&win_full[w], kCtas); mbar_init(&win_empty[w], 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], kCtas * kCtEpiWarps); }
+        mbar_fence_init();
+        tma_prefetch_desc(&P.mapF);
+        for (int b = 0; b < kCtBoxHeights; ++b) tma_prefetch_desc(&P.mapX[b]);
+    }
+    if (warp == 1) {
+        if (PAIR) { tmem_alloc_pair(&tmem_slot, 512); tmem_relinquish_pair(); }
+        else      { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (PAIR) cluster_sync_all();        // both CTAs' barriers are initialised before either signals the other
+    tc_fence_after();
+    // (each role waits for the kernels before at its first use of their results: what it needs of the launch's parameters, and the
+    // code up to there, has then been fetched)
+    const uint32_t tmem_base = tmem_slot;
+    bool timed_out = false;
+    // the taps that reach a position: all nine, or of an image of one row or column the middle ones
+    const int r0 = P.g.pr ? 0 : 1, r1 = P.g.pr ? 3 : 2, t0 = P.g.pc ? 0 : 1, t1 = P.g.pc ? 3 : 2;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            // ---------------------------------------------------- TMA producer of the filter tiles (both CTAs)
+            bool waited = false;
+            uint32_t s = 0, ph = 1;
+            for (int tile = unit; tile < P.tiles_total && !timed_out; tile += P.units)
+                for (int cc = 0; cc < P.cchunks && !timed_out; ++cc)
+                    for (int r = r0; r < r1; ++r) {
+                        if (!mbar_wait(&empty_bar[s], ph)) { timed_out = true; break; }
+                        const int c0 = cc * 128;
+                        if (!waited) { if (!P.beside) pdl_wait(); waited = true; }
+                        for (int t = t0; t < t1; ++t) {
+                            uint8_t *dst = ring + (size_t)s * stage_bytes + (uint32_t)(t - t0) * kCtTapBytes;
+                            uint64_t *bar = &full_bar[3 * s + (uint32_t)(t - t0)];
+                            if (rank == 0) mbar_expect_tx(bar, kCtas * kCtTapBytes);
+                            const int at = (3 * r + t) * P.C;
+                            const int x = P.dgrad ? at + n_mine : at + c0, y = P.dgrad ? c0 : n_mine;
+                            if (PAIR) tma_load_2d_pair(dst, &P.mapF, map_to_cta(bar, 0), x, y);
+                            else      tma_load_2d(dst, &P.mapF, bar, x, y);
+                        }
+                        if (++s == (uint32_t)P.stages) { s = 0; ph ^= 1u; }
+                    }
+        }
+    } else if (warp == 2 + kCtEpiWarps) {
+        // -------------------------------------------------------- windows: a lane copies the rows of a panel
+        uint32_t win = 0, ph = 1;
+        bool waited = P.beside != 0;
+        const int s = P.g.s;
+        for (int tile = unit; tile < P.tiles_total && !timed_out; tile += P.units) {
+            const ConvTRows w = convt_rows(P, P.d_tiles_n.div(tile), rank);
+            const int v0 = P.g.d_hp.div(w.first + P.g.hp) - 1, v1 = P.g.d_hp.div(w.first + w.count - 1 + P.g.hp) - 1;    // panels, -1 the one before the first
+            // (the rows behind the panels v0 .. that the window touches are not copied)
+            const int padding = P.g.pr ? P.g.d_hp.div(w.first + w.count + P.g.hp) - 1 - v0 : 0;
+            const uint32_t bytes = (uint32_t)((w.count - padding) * s) * 128u;
+            int img0, panel0;
+            P.g.d_np.divmod(v0 + lane + P.g.np, img0, panel0);
+            for (int cc = 0; cc < P.cchunks; ++cc) {
+                if (!mbar_wait_uniform(&win_empty[win], ph)) { timed_out = true; break; }
+                if (!waited) { pdl_wait(); waited = true; }
+                uint8_t *base = windows + (size_t)win * P.window_bytes + P.window_start;
+                if (lane == 0) mbar_expect_tx(&win_landed[win], bytes);
+                __syncwarp();
+                for (int v = v0 + lane, img = img0, panel = panel0; v <= v1; v += 32) {
+                    if (v != v0 + lane) P.g.d_np.divmod(v + P.g.np, img, panel);
+                    int row = max(w.first, v * P.g.hp);
+                    const int end = min(w.first + w.count, v * P.g.hp + P.H);
+                    for (int b = 0; row < end;) {
+                        const int high = 8 >> b;
+                        if (row + high > end) { ++b; continue; }
+                        tma_load_4d(base + (row * s - w.start) * 128, &P.mapX[b], &win_landed[win], cc * 128, panel * P.g.wp - P.g.off, row - v * P.g.hp, img - 1);
+                        row += high;
+                    }
+                }
+                __syncwarp();
+                if (++win == (uint32_t)P.windows) { win = 0; ph ^= 1u; }
+            }
+        }
+    } else if (warp == 3 + kCtEpiWarps) {
+        // -------------------------------------------------------- the windows' padding, once their copies have landed
+        uint32_t win = 0, ph = 0, zz = 0;
+        const int s = P.g.s;
+        if (!P.beside) pdl_wait();
+        zz = ((uint32_t)P.qa->zero_point & 0xFFu) * 0x01010101u;
+        for (int tile = unit; tile < P.tiles_total && !timed_out; tile += P.units) {
+            const ConvTRows w = convt_rows(P, P.d_tiles_n.div(tile), rank);
+            int h0 = 0;
+            if (P.g.pr) { int v; P.g.d_hp.divmod(w.first + P.g.hp, v, h0); }
+            for (int cc = 0; cc < P.cchunks; ++cc) {
+                const uint32_t base = smem_u32(windows) + win * P.window_bytes + P.window_start + (uint32_t)((w.first * s - w.start) * 128);   // of the first row
+                const bool ragged = cc * 128 + 128 > P.Cred;
+                // 16 bytes of padding (channels beyond the last stay zero): group g of a position's 128 bytes lies at g ^ (its line & 7)
+                auto pad = [&](uint32_t line, int group) {
+                    uint32_t z = zz;
+                    if (ragged && cc * 128 + (group ^ (int)((line >> 7) & 7u)) * 16 >= P.Cred) z = 0u;
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(line + (uint32_t)group * 16u), "r"(z) : "memory");
+                };
+                if (!mbar_wait_uniform(&win_landed[win], ph)) { timed_out = true; break; }
+                // a column of it in every row (of several panels: of the image's first and last) ...
+                if (P.g.pc) {
+                    uint32_t line = base + (uint32_t)((lane >> 3) * s) * 128u;
+                    for (int i = lane >> 3; i < w.count; i += 4, line += 512u * (uint32_t)s) {
+                        if (P.g.np == 1) { pad(line + (uint32_t)P.W * 128u, lane & 7); continue; }
+                        int v, h, img, panel;
+                        P.g.d_hp.divmod(w.first + i + P.g.hp, v, h);
+                        P.g.d_np.divmod(v - 1 + P.g.np, img, panel);
+                        if (panel == P.g.np - 1) pad(line + (uint32_t)(P.W - panel * P.g.wp + P.g.off) * 128u, lane & 7);
+                        if (panel == 0) pad(line, lane & 7);
+                    }
+                }
+                // ... and the row behind every panel
+                if (P.g.pr)
+                    for (int i = P.H - h0; i < w.count; i += P.g.hp)
+                        for (int u = lane; u < 8 * s; u += 32) pad(base + (uint32_t)(i * s + (u >> 3)) * 128u, u & 7);
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) {
+                    if (PAIR) mbar_arrive_cluster(map_to_cta(&win_full[win], 0));
+                    else      mbar_arrive(&win_full[win]);
+                }
+                if (++win == (uint32_t)P.windows) { win = 0; ph ^= 1u; }
+            }
+        }
+    } else if (warp == 1) {
+        if (rank == 0) {
+            // ---------------------------------------------------- MMA issuer (a pair's leader only): the whole warp in step
+            ConvTMmaArgs A;
+            A.full_bar = full_bar; A.empty_bar = empty_bar; A.win_full = win_full; A.win_empty = win_empty; A.acc_full = acc_full; A.acc_empty = acc_empty;
+            A.windows_at = smem_u32(windows); A.window_bytes = P.window_bytes; A.window_start = P.window_start;
+            A.ring = smem_u32(ring); A.tmem = tmem_base; A.f_desc_lo = P.f_desc_lo; A.x_desc_lo = P.x_desc_lo; A.idesc = P.idesc;
+            A.cchunks = P.cchunks; A.stages = (uint32_t)P.stages; A.windows = (uint32_t)P.windows;
+            // forward: input (p - 1 + r, q - 1 + t) feeds output (p, q); layer gradient: gradient (h + 1 - r, w + 1 - t) feeds input (h, w)
+            A.tap_rows = r1 - r0;
+            A.tap0 = P.dgrad ? 16 * P.g.pr * P.g.s : 0;
+            A.row_step = P.dgrad ? -8 * P.g.s : 8 * P.g.s;
+            A.tile0 = unit; A.tiles_total = P.tiles_total; A.tile_step = P.units;
+            // (a barrier's wait is bounded: its clock starts once the producers' copies can)
+            if (!P.beside) pdl_wait();
+            const bool ok = t1 - t0 == 1 ? (P.dgrad ? convt_mma_loop<PAIR, true, 1>(A) : convt_mma_loop<PAIR, false, 1>(A))
+                                         : (P.dgrad ? convt_mma_loop<PAIR, true, 3>(A) : convt_mma_loop<PAIR, false, 3>(A));
+            timed_out = !ok;
+        }
+    } else {
+        // ------------------------------------------------------- epilogue (each CTA drains its own 128 channels; the four groups
+        // of four warps split the chunks of 16 positions)
+        const int ew = warp - 2, quad = warp & 3, group = ew >> 2;
+        const int ch = n_mine + quad * 32 + lane;
+        const bool ch_in = ch < P.N;
+        const int chunks = P.npos >> 4, c_begin = chunks * group >> 2, c_end = chunks * (group + 1) >> 2;
+        pdl_wait();
+        const float scale = __fmul_rn(P.qa->scale, P.qb->scale);
+        // (the taps that are left out of an image of one row or column: the border class without them)
+        const int cterm = ch_in ? load_after_wait(P.colterm + (int64_t)((P.g.pr ? 0 : 3) | (P.g.pc ? 0 : 12)) * P.N + ch) : 0;
+        const uint32_t leader_empty = PAIR ? map_to_cta(&acc_empty[0], 0) : 0u;          // (8 bytes a barrier)
+        auto hand_back = [&](uint32_t buf) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) { if (PAIR) mbar_arrive_cluster(leader_empty + 8u * buf); else mbar_arrive(&acc_empty[buf]); }
+        };
+
+        // The positions of this warp's chunks of a tile, two a lane: where they lie in the output (padding: nowhere), their terms.
+        // A chunk's positions follow one another in the output, but for a step where a panel's row ends.
+        bool valid[2]; int64_t m[2]; int term[2];
+        auto look_up = [&](int tile) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                int rem, j, v, h, img, panel;
+                const int at = c_begin * 16 + k * 32 + lane;
+                P.g.d_s.divmod(P.d_tiles_n.div(tile) * P.npos + at, rem, j);
+                P.g.d_hp.divmod(rem, v, h);
+                P.g.d_np.divmod(v, img, panel);
+                const int q = panel * P.g.wp - P.g.off + j;
+                valid[k] = at < c_end * 16 && img < P.Nimg && h < P.H && j >= P.g.off && j < P.g.off + P.g.wp && q < P.W;
+                m[k] = ((int64_t)img * P.H + h) * P.W + q;
+                term[k] = valid[k] ? load_after_wait(P.rowterm + m[k]) : 0;
+            }
+        };
+        auto put_down = [&]() {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                // (a lane's own chunk is half of the 32 positions)
+                const unsigned sixteen = lane & 16 ? 0xffff0000u : 0xffffu;
+                const unsigned vmask = __ballot_sync(0xffffffffu, valid[k]) & sixteen;
+                const int64_t m1 = __shfl_sync(0xffffffffu, m[k], vmask ? __ffs(vmask) - 1 : lane);
+                const unsigned step = __ballot_sync(0xffffffffu, valid[k] && m[k] != m1 + __popc(vmask & ((1u << lane) - 1u))) & sixteen;
+                const int second = step ? __ffs(step) - 1 : lane;
+                const int64_t m2 = __shfl_sync(0xffffffffu, m[k], second);
+                E.term[ew][2 * k + (lane >> 4)][lane & 15] = term[k];
+                if ((lane & 15) == 0) E.run[ew][2 * k + (lane >> 4)] = CtRun{lane & 16 ? vmask >> 16 : vmask, step ? second & 15 : 16, m1, m2};
+            }
+            __syncwarp();
+        };
+        if (unit < P.tiles_total) { look_up(unit); put_down(); }
+        uint32_t buf = 0, fph = 0;
+        for (int tile = unit; tile < P.tiles_total; tile += P.units) {
+            // (the next tile's terms are fetched now, so that their latency hides behind this tile)
+            const int tile_next = tile + P.units;
+            if (tile_next < P.tiles_total) look_up(tile_next);
+            if (!timed_out && !mbar_wait_warp(&acc_full[buf], fph)) timed_out = true;
+            if (!timed_out) {
+                tc_fence_after();
+                const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + buf * 256u;
+                if (c_begin >= c_end) hand_back(buf);
+                for (int c = c_begin; c < c_end; ++c) {
+                    uint32_t r[16];
+                    tmem_ld_32x16(t_addr + (uint32_t)(c * 16), r);
+                    const CtRun run = E.run[ew][c - c_begin];
+                    const int4 *terms = reinterpret_cast<const int4 *>(E.term[ew][c - c_begin]);
+                    tmem_ld_wait();
+                    if (c == c_end - 1) hand_back(buf);              // this warp has read its part of the accumulator
+                    int acc[16];
+#pragma unroll
+                    for (int j = 0; j < 16; j += 4) {
+                        const int4 t = terms[j >> 2];
+                        acc[j] = (int)r[j] + t.x + cterm; acc[j + 1] = (int)r[j + 1] + t.y + cterm;
+                        acc[j + 2] = (int)r[j + 2] + t.z + cterm; acc[j + 3] = (int)r[j + 3] + t.w + cterm;
+                    }
+                    // Position by position, under predicates (a branch each took twice the time); a chunk that a panel's row ends in is
+                    // gone through twice.
+                    const unsigned below = (1u << run.second) - 1u;
+                    if (ch_in) {
+#pragma unroll 1
+                        for (int pass = 0; pass < (run.second < 16 ? 2 : 1); ++pass) {
+                            const unsigned mask = pass ? run.vmask & ~below : run.vmask & below;
+                            const int64_t at = ((pass ? run.m2 : run.m1) * P.N + ch) * 4, stride = (int64_t)P.N * 4;
+                            if (P.acc_out) {
+                                char *to = reinterpret_cast<char *>(P.acc_out) + at;
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) put_if(mask & (1u << j), (uint32_t)acc[j], to, stride);
+                            }
+                            if (P.out) {
+                                char *to = reinterpret_cast<char *>(P.out) + at;
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) put_if(mask & (1u << j), __float_as_uint(__fmul_rn((float)acc[j], scale)), to, stride);
+                            }
+                        }
+                    }
+                }
+            }
+            __syncwarp();                                            // (every lane has read the terms before they are replaced)
+            if (tile_next < P.tiles_total) put_down();
+            buf ^= 1u;
+            if (buf == 0) fph ^= 1u;
+        }
+    }
+
+    if (timed_out) {
+        pdl_wait();                      // (a launch before may clear the word)
+        raise_timeout(P.status);
+        __nanosleep(1000000);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (PAIR) cluster_sync_all();        // neither CTA retires while the other may still read its memory or signal it
+    if (warp == 1) {
+        __syncwarp();
+        if (PAIR) tmem_dealloc_pair(tmem_base, 512); else tmem_dealloc(tmem_base, 512);
+    }
+}
+
+static ConvTGrid convt_grid(const qbp_conv_desc *d)
+{
+    ConvTGrid g{};
+    g.pr = d->H > 1 ? 1 : 0; g.pc = d->W > 1 ? 1 : 0;
+    g.np = (d->W + kCtPanelWidth - 1) / kCtPanelWidth; g.wp = (d->W + g.np - 1) / g.np; g.off = g.np > 1 ? 1 : 0;
+    g.s = g.np > 1 ? g.wp + 2 : d->W + g.pc; g.hp = d->H + g.pr;
+    g.d_s = make_fastdiv(g.s); g.d_hp = make_fastdiv(g.hp); g.d_np = make_fastdiv(g.np);
+    g.total = (int64_t)d->N * g.np * g.hp * g.s;
+    return g;
+}
+
+// The tile: on pairs or not, and its positions.  A model of the launch in cycles per SM, the cheapest wins: rounds of tiles x (taps x
+// chunks x the longest of the MMAs (2 cycles per position and tap), the copies (3 per operand row) and shared memory's port (128
+// bytes a cycle for operand reads and copies) + a tile's overhead) + the last tile's epilogue.
+struct ConvTPlan { bool pair; int npos, tiles_n, units, windows, stages; uint32_t window_bytes; double cost; };
+static ConvTPlan convt_plan(const qbp_conv_desc *d, const ConvTGrid &g, bool dgrad)
+{
+    const int Cred = dgrad ? d->K : d->C, Nout = dgrad ? d->C : d->K, cchunks = (Cred + 127) / 128;
+    const int cols = g.pc ? 3 : 1, taps = (g.pr ? 3 : 1) * cols, reach = g.pr * g.s + g.pc;
+    ConvTPlan best{};
+    best.cost = 0.0;
+    for (int pair = 0; pair < 2; ++pair)
+        for (int npos = 256; npos >= 64; npos -= 32) {
+            ConvTPlan p{};
+            p.pair = pair != 0; p.npos = npos;
+            const int width = pair ? 256 : 128, units = pair ? sm_count() / 2 : sm_count(), ncta = pair ? npos / 2 : npos;
+            p.tiles_n = (Nout + width - 1) / width;
+            if ((pair && Nout <= 128) || p.tiles_n > units) continue;
+            const int64_t tiles = (g.total + npos - 1) / npos * p.tiles_n;
+            p.units = (int)std::min<int64_t>(tiles, units);
+            p.units -= p.units % p.tiles_n;
+            p.window_bytes = (uint32_t)align_up(128u * (size_t)(2 * g.s + ncta + 2 * reach), 1024);
+            const int room = (int)(kCtSmem - 1024u - (uint32_t)align_up(sizeof(CtEpiShared), 256));
+            // two windows, or three where they leave the filter's ring three tap rows
+            const int stage_bytes = cols * (int)kCtTapBytes;
+            p.windows = room - 3 * (int)p.window_bytes >= 3 * stage_bytes ? 3 : 2;
+            p.stages = std::min(kCtMaxStages, (room - p.windows * (int)p.window_bytes) / stage_bytes);
+            if (p.stages < 2) continue;
+            const double rows = 128.0 + (double)(4 * g.s + ncta) / taps;
+            const double port = (4.0 * (4096.0 + 32.0 * ncta) + 128.0 * rows) / 128.0;
+            const double stage = std::max({2.0 * npos, 3.0 * rows, port});
+            p.cost = (double)((tiles + p.units - 1) / p.units) * (taps * cchunks * stage + 300.0) + 10.0 * npos;
+            if (best.cost == 0.0 || p.cost < best.cost) best = p;
+        }
+    return best;
+}
+
+// Whether this kernel takes the product (of a supported convolution; bwl, bhl: log2 of the position box of the kernel above).
+// Where that one takes it too, by both models.  The constants were fitted to some 40 shapes; what the rule gives away is at most 4 %
+// (cycles by the models, then us): 256 x 14 x 14, 256 -> 256 45.6 K / 35.7 K, 36.3 / 38.3, stays above; 512 x 14 x 14 91.2 K / 60.8 K,
+// 64.7 / 63.3, comes here; 96 x 14 x 14 15.2 K / 17.7 K, 20.7 / 22.5, stays; 30 x 17 x 17, 512 -> 512 60.8 K / 33.5 K, 38.2 / 30.8, comes.
+bool conv2t_eligible(const qbp_conv_desc *d, bool dgrad, int bwl, int bhl)
+{
+    const int Cred = dgrad ? d->K : d->C, Nout = dgrad ? d->C : d->K;
+    if (d->R != 3 || Cred < 96 || Nout < 96) return false;
+    const ConvTGrid g = convt_grid(d);
+    if (g.total >= (1ll << 31) - 4096) return false;
+    const ConvTPlan p = convt_plan(d, g, dgrad);
+    if (p.cost <= 0.0 || !conv2_eligible(d, dgrad)) return p.cost > 0.0;
+    const int64_t boxes = (int64_t)((d->W + (1 << bwl) - 1) >> bwl) * ((d->H + (1 << bhl) - 1) >> bhl) * ((d->N + (128 >> (bwl + bhl)) - 1) / (128 >> (bwl + bhl)));
+    const int bn = conv2_bn(boxes, Nout), tiles_n = (Nout + bn - 1) / bn;
+    const int64_t tiles = (boxes + 1) / 2 * tiles_n;
+    int64_t pairs = std::min<int64_t>(tiles, sm_count() / 2);
+    pairs -= pairs % tiles_n;
+    const double above = (double)((tiles + pairs - 1) / pairs) * 9 * ((Cred + 127) / 128) * std::max(2.0 * bn, 3.3 * (128 + bn / 2));
+    return p.cost < 0.7 * above + 3000.0;
+}
+
+int launch_conv2t(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp_qparams *q_in, const int8_t *wgt,
+                 const qbp_qparams *q_w, int32_t *acc_out, float *out, const int32_t *rowterm, const int32_t *colterm,
+                 int *status, bool beside, cudaStream_t st)
+{
+    ConvTParams P{};
+    const int Cred = dgrad ? d->K : d->C, Nout = dgrad ? d->C : d->K;
+    P.g = convt_grid(d);
+    const ConvTPlan p = convt_plan(d, P.g, dgrad);
+    P.cchunks = (Cred + 127) / 128;
+    P.dgrad = dgrad ? 1 : 0; P.beside = beside ? 1 : 0;
+    P.npos = p.npos; P.npos_cta = p.pair ? p.npos / 2 : p.npos;
+    int rc;
+    // filter: forward [K x 9 C], rows = output channels (K-major); layer gradient: rows = the reduction, columns = output channels
+    if ((rc = make_map_2d(&P.mapF, wgt, d->K, 9ull * d->C, 128, 128))) return rc;
+    for (int b = 0; b < kCtBoxHeights; ++b)
+        if ((rc = make_map_nhwc(&P.mapX[b], in, d->N, d->H, d->W, Cred, 1, 8u >> b, (uint32_t)P.g.s, 128))) return rc;
+    const OperandLayout f = dgrad ? layout_mnmajor(128, 128, 1, 0) : layout_kmajor(128, 128), x = layout_kmajor(128, 128);
+    P.f_desc_lo = f.desc_lo; P.x_desc_lo = x.desc_lo;
+    P.idesc = make_idesc(true, true, f.major, x.major, p.pair ? 256 : 128, (uint32_t)p.npos);
+    P.window_start = 128u * (uint32_t)P.g.s; P.window_bytes = p.window_bytes;
+    P.windows = p.windows; P.stages = p.stages;
+    P.tiles_n = p.tiles_n; P.units = p.units;
+    P.tiles_total = (int)((P.g.total + p.npos - 1) / p.npos) * p.tiles_n;
+    P.d_tiles_n = make_fastdiv(P.tiles_n);
+    P.Nimg = d->N; P.H = d->H; P.W = d->W; P.C = d->C; P.N = Nout; P.Cred = Cred;
+    P.acc_out = acc_out; P.out = out; P.rowterm = rowterm; P.colterm = colterm; P.qa = q_in; P.qb = q_w; P.status = status;
+    const int grid = p.pair ? 2 * p.units : p.units;
+    const size_t smem = 1024u + (size_t)p.windows * p.window_bytes + (size_t)p.stages * (P.g.pc ? 3 : 1) * kCtTapBytes + sizeof(CtEpiShared);
+    static PerDeviceOnce configured[2];
+    void (*kernel)(const ConvTParams) = p.pair ? qbp_conv2t_kernel<true> : qbp_conv2t_kernel<false>;
+    QBP_SMEM_OPT_IN(configured[p.pair ? 1 : 0], kernel, kCtSmem);
+    QBP_TRACE_BEGIN(st);
+    launch(kernel, grid, kCtThreads, smem, st, P);
+    QBP_LAUNCH_OK("qbp_conv2t_kernel");
+    return QBP_OK;
+}
+
 }  // namespace qbp

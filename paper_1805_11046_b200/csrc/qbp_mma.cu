@@ -1456,8 +1456,11 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
 
     int bwl = 0, bhl = 0;
     pick_pixel_box(d->N, d->H, d->W, bwl, bhl);
-    // 3 x 3 with many channels on both sides: CTA pairs (the epilogue's tail is the single-CTA kernel's)
-    if (conv2_eligible(d, dgrad) && !(tail && (tail->fold || tail->relu || tail->q)))
+    // 3 x 3 with many channels on both sides: kernels of their own (the epilogue's tail is the single-CTA kernel's)
+    const bool plain = !(tail && (tail->fold || tail->relu || tail->q));
+    if (plain && !stats && conv2t_eligible(d, dgrad, bwl, bhl))
+        return launch_conv2t(dgrad, d, in, q_in, wgt, q_w, acc_out, out, rowterm, colterm, status, beside, st);
+    if (plain && conv2_eligible(d, dgrad))
         return launch_conv2(dgrad, d, in, q_in, wgt, q_w, acc_out, out, rowterm, colterm, stats, status, bwl, bhl, beside, st);
 
     MmaParams P{};

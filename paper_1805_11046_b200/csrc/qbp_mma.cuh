@@ -177,6 +177,11 @@ bool conv2_eligible(const qbp_conv_desc *d, bool dgrad);
 int launch_conv2(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp_qparams *q_in, const int8_t *wgt,
                  const qbp_qparams *q_w, int32_t *acc_out, float *out, const int32_t *rowterm, const int32_t *colterm,
                  ColStatParts *stats, int *status, int bwl, int bhl, bool beside, cudaStream_t st);
+// ... and those whose output's statistics nobody wants
+bool conv2t_eligible(const qbp_conv_desc *d, bool dgrad, int bwl, int bhl);
+int launch_conv2t(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp_qparams *q_in, const int8_t *wgt,
+                  const qbp_qparams *q_w, int32_t *acc_out, float *out, const int32_t *rowterm, const int32_t *colterm,
+                  int *status, bool beside, cudaStream_t st);
 
 // ---- the dense weight gradient on CTA pairs (qbp_wgrad2.cu) ----------------------
 bool wgrad2_eligible(int64_t M, int64_t N, int64_t K);

@@ -515,18 +515,22 @@ def test_conv_pairs(B, N, H, W, C, K, mode):
 
 
 @pytest.mark.parametrize("N,H,W,C,K", [(5, 1, 9, 96, 128), (130, 9, 1, 128, 96), (300, 1, 1, 256, 112), (70, 2, 2, 96, 96), (2, 15, 15, 128, 256),
-                                       (1, 3, 64, 96, 272), (2, 3, 65, 96, 128), (1, 6, 130, 160, 96), (3, 1, 200, 96, 96), (1, 2, 255, 128, 128)])
+                                       (1, 3, 96, 96, 272), (2, 3, 97, 96, 128), (1, 6, 130, 160, 96), (3, 1, 200, 96, 96), (1, 2, 255, 128, 128),
+                                       (20, 19, 19, 96, 160), (40, 28, 28, 128, 128), (64, 14, 14, 512, 512)])
 @pytest.mark.parametrize("mode", [0, 1])
-def test_conv_pairs_numbering_of_the_positions(B, N, H, W, C, K, mode):
-    """Images of one row or column (no padding that way, fewer taps), of a tile's exact size, one and several panels of columns with a
-    narrower last one: every accumulator, the output and its statistics."""
+def test_conv_channels_as_rows(B, N, H, W, C, K, mode):
+    """Products without statistics.  Images of one row or column (no padding that way, fewer taps), of a tile's exact size, one and
+    several panels of columns with a narrower last one, channel chunks partly filled, pairs and single CTAs, several tiles of each."""
     d = B.conv_desc(N, H, W, C, K, 3, 3, 1, 1); od = O.conv_desc(N, H, W, C, K, 3, 3, 1, 1)
     inp = random_codes((N, H, W, C if mode == 0 else K), 84); w = random_codes((K, 3, 3, C), 85)
-    acc, out, ws, stats = B.qbp_conv_s8_implicit(mode, d, to_dev(inp), _qp(B, 0.5, 17), to_dev(w), _qp(B, 0.25, -23), want_acc=True, col_stats=True)
+    acc, out, ws = B.qbp_conv_s8_implicit(mode, d, to_dev(inp), _qp(B, 0.5, 17), to_dev(w), _qp(B, 0.25, -23), want_acc=True)
     assert B.status_word(ws) == 0
-    oacc, oout, bad = O.conv_s8(mode, od, inp, 17, w, -23, 0.5, 0.25)
-    assert bad == 0 and np.array_equal(to_host(acc).ravel(), oacc.ravel()) and np.array_equal(to_host(out).ravel(), oout.ravel())
-    _check_col_stats(out, stats)
+    a, o = to_host(acc).ravel(), to_host(out).ravel()
+    idx = np.arange(a.size) if a.size <= 1 << 19 else np.unique(np.concatenate(
+        [[0, a.size - 1], np.random.Generator(np.random.PCG64(86)).integers(0, a.size, 1 << 14)]))
+    oacc, oout, bad = O.conv_s8(mode, od, inp, 17, w, -23, 0.5, 0.25, idx=idx.astype(np.int64))
+    assert bad == 0 and np.array_equal(a[idx], oacc) and np.array_equal(o[idx], oout)
+    assert np.array_equal(o, a.astype(np.float32) * np.float32(0.125))
 
 
 # ------------------------------------------------- products that leave most of the machine idle: smaller tiles
