@@ -124,7 +124,8 @@ int gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, const 
                  int *ext_status, void *ws, size_t ws_bytes, cudaStream_t st, const CodeSums *a_sums = nullptr,
                  const CodeSums *b_sums = nullptr, bool beside = false);
 // tot_x [C] / tot_g16 [K] (convolution; nullable, both or none): per-channel totals of the stored x codes and of the
-// stored 16-bit gradient codes (256 * hi + lo) over all positions, left by the kernels that wrote the codes.
+// stored 16-bit gradient codes (256 * hi + lo) over all positions, left by the kernels that wrote the codes.  tot_g16 [N] alone:
+// a plain product's, of at most kWgPieceRows rows.
 // lo_signed: g_lo holds the low bytes with the top bit flipped, i.e. the signed bytes lo - 128 (lo_signed in
 // bifurcate_with_range_partials): g16 - zg = 256 * hi + (lo - 128) - (zg - 128), so the two limbs have one operand
 // type and run as one product of twice the columns (the x tile is read from shared memory once, not once per limb),
@@ -187,7 +188,7 @@ int launch_conv2t(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qb
 bool wgrad2_eligible(int64_t M, int64_t N, int64_t K);
 int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qparams *qx, const int8_t *g_hi,
                   const uint8_t *g_lo, const qbp_qparams *qg16, int64_t *acc_out, float *dW, const CodeSums &sx,
-                  const CodeSums &shi, const CodeSums &slo, int *status, bool beside, cudaStream_t st, bool lo_signed = false);
+                  const CodeSums &shi, const CodeSums &slo, const int64_t *tot_g, int *status, bool beside, cudaStream_t st, bool lo_signed = false);
 
 // ---- shared-memory operand descriptors ---------------------------------------
 // How one operand tile of a pipeline stage is laid out and walked by the MMAs.

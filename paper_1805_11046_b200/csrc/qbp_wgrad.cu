@@ -104,6 +104,13 @@ struct WgradParams {
     unsigned long long *ones_tot;
 };
 
+// A plain product: the sum of a gradient column's codes as the limbs are stored.
+__device__ __forceinline__ long long wg_plain_sum_g(const WgradParams &P, int n)
+{
+    if (P.tot_g) return P.tot_g[n] - (P.lo_signed ? 128 * P.M : 0);
+    return P.cx ? 256 * P.chi[n] + P.clo[n] : 256 * P.shi.at(n) + P.slo.at(n);
+}
+
 // Which item and slice a CTA works on.
 struct WgItem { int ag, tb, slice, slices; };
 
@@ -462,7 +469,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) qbp_wgrad_kernel(const __grid_c
         if (P.direct) {
             const int t = threadIdx.x - 64;
             const long long zx = P.qx->zero_point;
-            if (t < P.bn) s_cterm[t] = (int64_t)n0 + t < P.N ? -zx * (256 * P.shi.at(n0 + t) + P.slo.at(n0 + t)) : 0;
+            if (t < P.bn) s_cterm[t] = (int64_t)n0 + t < P.N ? -zx * wg_plain_sum_g(P, n0 + t) : 0;
             named_barrier(3, 128);
         }
         if (k_iters > 0 && !mbar_wait_warp(&acc_bar, 0)) timed_out = true;
@@ -582,7 +589,7 @@ __global__ void __launch_bounds__(256) wgrad_finalize_kernel(const __grid_consta
 #pragma unroll
     for (int o = 1; o < kLanes; o <<= 1) raw += __shfl_xor_sync(0xffffffffu, raw, o);
     if (!live || part_lane != 0) return;
-    const long long SX = P.cx ? P.cx[k] : P.sx.at(k), SG = P.cx ? 256 * P.chi[n] + P.clo[n] : 256 * P.shi.at(n) + P.slo.at(n);
+    const long long SX = P.cx ? P.cx[k] : P.sx.at(k), SG = wg_plain_sum_g(P, n);
     const long long acc = raw - zg * SX - zx * SG + P.M * zx * zg;
     if (P.acc_out) P.acc_out[e] = acc;
     if (P.dW) P.dW[e] = __fmul_rn((float)acc, __fmul_rn(P.qx->scale, P.qg->scale));
@@ -959,6 +966,7 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
     // or the product takes the gradient's itself: a row of ones in its spare chunk) of the images' edges only
     int rc;
     const bool from_totals = d && tot_x && tot_g16 && (tot_g_filled || wgrad_self_totals(d));
+    const int64_t *plain_tot_g = !d && !table && done_sums ? tot_g16 : nullptr;
     int njobs = 0;
     if (!done_sums)
         for (int i = from_totals ? 3 : 0; i < nall; ++i) jobs[njobs++] = all[i];
@@ -981,7 +989,8 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
     bool beside = false;
     if ((rc = launch_code_sums(jobs, njobs, st, zero, &beside))) return rc;
     if (pair_kernel)
-        return launch_wgrad2(M, N, K, x, qx, g_hi, g_lo, qg16, acc_out, dW, P.sx, P.shi, P.slo, status, beside, st, lo_signed);
+        return launch_wgrad2(M, N, K, x, qx, g_hi, g_lo, qg16, acc_out, dW, P.sx, P.shi, P.slo, plain_tot_g, status, beside, st, lo_signed);
+    if (!d) P.tot_g = (const long long *)plain_tot_g;
 
     P.part = (long long *)part; P.status = status;
     P.qx = qx; P.qg = qg16; P.acc_out = (long long *)acc_out; P.dW = dW; P.dW_vec = aligned16(dW) ? 1 : 0;

@@ -44,6 +44,7 @@ struct Wgrad2Params {
     int64_t M, N, K;                 // reduction rows; output columns; output rows
     long long *acc_out; float *dW;
     CodeSums sx, shi, slo;           // code sums over the M rows: rowterm = -zg * sx[k] + M * zx * zg, colterm = -zx * (256 * shi[n] + slo[n])
+    const long long *tot_g;          // [N]: totals of 256 * hi + (unsigned low byte) over the rows, in place of shi and slo (NULL: not there)
     int beside;                      // the launch before makes the code sums: only the epilogue waits for it
     int zg_shift;                    // 128 for signed low bytes (lo - 128 against zg - 128)
     const qbp_qparams *qx, *qg;
@@ -186,6 +187,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
             // two pieces of all eight sums are in flight at a time -- one sum after the other took up to 64 us a tile)
             long long ct[4] = {0, 0, 0, 0};
             const int32_t *ph = P.shi.p + o.n0 + half * 128 + lane, *pl = P.slo.p + o.n0 + half * 128 + lane;
+            if (P.tot_g) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if ((half * 4 + i) * 32 + lane < ncol) ct[i] = P.tot_g[o.n0 + (half * 4 + i) * 32 + lane] - P.zg_shift * P.M;
+            } else
 #pragma unroll 2
             for (int k = 0; k < P.shi.pieces; ++k) {
 #pragma unroll
@@ -289,7 +295,7 @@ bool wgrad2_eligible(int64_t M, int64_t N, int64_t K)
 
 int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qparams *qx, const int8_t *g_hi,
                   const uint8_t *g_lo, const qbp_qparams *qg16, int64_t *acc_out, float *dW, const CodeSums &sx,
-                  const CodeSums &shi, const CodeSums &slo, int *status, bool beside, cudaStream_t st, bool lo_signed)
+                  const CodeSums &shi, const CodeSums &slo, const int64_t *tot_g, int *status, bool beside, cudaStream_t st, bool lo_signed)
 {
     Wgrad2Params P{};
     int rc;
@@ -309,7 +315,7 @@ int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qp
     P.d_group = make_fastdiv(kW2GroupM * P.tiles_n);
     P.M = M; P.N = N; P.K = K;
     P.acc_out = (long long *)acc_out; P.dW = dW;
-    P.beside = beside ? 1 : 0; P.sx = sx; P.shi = shi; P.slo = slo; P.zg_shift = lo_signed ? 128 : 0; P.qx = qx; P.qg = qg16; P.status = status;
+    P.beside = beside ? 1 : 0; P.tot_g = (const long long *)tot_g; P.sx = sx; P.shi = shi; P.slo = slo; P.zg_shift = lo_signed ? 128 : 0; P.qx = qx; P.qg = qg16; P.status = status;
     static PerDeviceOnce configured;
     QBP_SMEM_OPT_IN(configured, qbp_wgrad2_kernel, kW2Smem);
     QBP_TRACE_BEGIN(st);

@@ -490,6 +490,13 @@ def test_linear_layers_of_other_shapes_stagewise(B, batch, cin, cout):
     _check_layer(B, cfg, True)
 
 
+@pytest.mark.parametrize("batch,cin,cout", [(528, 256, 256), (1040, 272, 1008), (2048, 1040, 400), (1024, 128, 2064)])
+def test_wide_linear_layers_stagewise(B, batch, cin, cout):
+    """The weight gradient on CTA pairs and off them, its gradient totals and the layer gradient's row sums left by the second backward
+    pass: channel counts that fill one, part of a second and several slabs of columns."""
+    _check_layer(B, synth.linear_layer(batch, cin, cout), True)
+
+
 @pytest.mark.parametrize("batch", [65536, 65552])
 def test_linear_layer_of_a_long_minibatch_stagewise(B, batch):
     """Either side of 65536 rows, where the weight gradient's column sums go to a table that the backward clears on the way."""
