@@ -110,7 +110,12 @@ struct WsCarver {
 // a launch of its own for it costs two and more) and the first block leaves the records at qp8 / qp16 (each nullable).
 struct RangeSrc { const float2 *parts; int nparts; const qbp_qparams *given; qbp_qparams *qp8, *qp16; };
 // Regions of 32-bit words that a kernel clears on the way (a status word, sums that a later kernel adds to).
-struct ZeroJobs { uint32_t *p[2]; int64_t words[2]; };
+constexpr int kMaxZeroJobs = 5;
+struct ZeroJobs {
+    int count;
+    uint32_t *p[kMaxZeroJobs]; int64_t words[kMaxZeroJobs];
+    void add(void *at, int64_t n) { if (n > 0) { p[count] = static_cast<uint32_t *>(at); words[count++] = n; } }
+};
 
 // -------------------------------------------------------------- device side
 #ifdef __CUDACC__
@@ -342,7 +347,7 @@ __device__ __forceinline__ float2 block_range(const float2 *__restrict__ parts, 
 __device__ __forceinline__ void run_zero_jobs(const ZeroJobs &z, int64_t thread, int64_t threads)
 {
 #pragma unroll
-    for (int k = 0; k < 2; ++k)
+    for (int k = 0; k < kMaxZeroJobs && k < z.count; ++k)        // (unrolled: an index into a parameter would copy it to local memory)
         for (int64_t i = thread; i < z.words[k]; i += threads) z.p[k][i] = 0u;
 }
 struct QParamsReg { float inv, zp_u; };       // 1 / scale and the unsigned zero-point

@@ -605,7 +605,8 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(kCtThread
         for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], kCtas * kCtEpiWarps); }
         mbar_fence_init();
         tma_prefetch_desc(&P.mapF);
-        for (int b = 0; b < kCtBoxHeights; ++b) tma_prefetch_desc(&P.mapX[b]);
+        for (int b = 0; b < kCtBoxHeights; ++b)
+            if ((8 >> b) <= P.H) tma_prefetch_desc(&P.mapX[b]);
     }
     if (warp == 1) {
         if (PAIR) { tmem_alloc_pair(&tmem_slot, 512); tmem_relinquish_pair(); }
@@ -875,7 +876,6 @@ static ConvTGrid convt_grid(const qbp_conv_desc *d)
 // The tile: on pairs or not, and its positions.  A model of the launch in cycles per SM, the cheapest wins: rounds of tiles x (taps x
 // chunks x the longest of the MMAs (2 cycles per position and tap), the copies (3 per operand row) and shared memory's port (128
 // bytes a cycle for operand reads and copies) + a tile's overhead) + the last tile's epilogue.
-struct ConvTPlan { bool pair; int npos, tiles_n, units, windows, stages; uint32_t window_bytes; double cost; };
 static ConvTPlan convt_plan(const qbp_conv_desc *d, const ConvTGrid &g, bool dgrad)
 {
     const int Cred = dgrad ? d->K : d->C, Nout = dgrad ? d->C : d->K, cchunks = (Cred + 127) / 128;
@@ -912,13 +912,13 @@ static ConvTPlan convt_plan(const qbp_conv_desc *d, const ConvTGrid &g, bool dgr
 // Where that one takes it too, by both models.  The constants were fitted to some 40 shapes; what the rule gives away is at most 4 %
 // (cycles by the models, then us): 256 x 14 x 14, 256 -> 256 45.6 K / 35.7 K, 36.3 / 38.3, stays above; 512 x 14 x 14 91.2 K / 60.8 K,
 // 64.7 / 63.3, comes here; 96 x 14 x 14 15.2 K / 17.7 K, 20.7 / 22.5, stays; 30 x 17 x 17, 512 -> 512 60.8 K / 33.5 K, 38.2 / 30.8, comes.
-bool conv2t_eligible(const qbp_conv_desc *d, bool dgrad, int bwl, int bhl)
+bool conv2t_eligible(const qbp_conv_desc *d, bool dgrad, int bwl, int bhl, ConvTPlan &p)
 {
     const int Cred = dgrad ? d->K : d->C, Nout = dgrad ? d->C : d->K;
     if (d->R != 3 || Cred < 96 || Nout < 96) return false;
     const ConvTGrid g = convt_grid(d);
     if (g.total >= (1ll << 31) - 4096) return false;
-    const ConvTPlan p = convt_plan(d, g, dgrad);
+    p = convt_plan(d, g, dgrad);
     if (p.cost <= 0.0 || !conv2_eligible(d, dgrad)) return p.cost > 0.0;
     const int64_t boxes = (int64_t)((d->W + (1 << bwl) - 1) >> bwl) * ((d->H + (1 << bhl) - 1) >> bhl) * ((d->N + (128 >> (bwl + bhl)) - 1) / (128 >> (bwl + bhl)));
     const int bn = conv2_bn(boxes, Nout), tiles_n = (Nout + bn - 1) / bn;
@@ -931,12 +931,11 @@ bool conv2t_eligible(const qbp_conv_desc *d, bool dgrad, int bwl, int bhl)
 
 int launch_conv2t(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp_qparams *q_in, const int8_t *wgt,
                  const qbp_qparams *q_w, int32_t *acc_out, float *out, const int32_t *rowterm, const int32_t *colterm,
-                 int *status, bool beside, cudaStream_t st)
+                 const ConvTPlan &p, int *status, bool beside, cudaStream_t st)
 {
     ConvTParams P{};
     const int Cred = dgrad ? d->K : d->C, Nout = dgrad ? d->C : d->K;
     P.g = convt_grid(d);
-    const ConvTPlan p = convt_plan(d, P.g, dgrad);
     P.cchunks = (Cred + 127) / 128;
     P.dgrad = dgrad ? 1 : 0; P.beside = beside ? 1 : 0;
     P.npos = p.npos; P.npos_cta = p.pair ? p.npos / 2 : p.npos;
@@ -944,7 +943,7 @@ int launch_conv2t(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qb
     // filter: forward [K x 9 C], rows = output channels (K-major); layer gradient: rows = the reduction, columns = output channels
     if ((rc = make_map_2d(&P.mapF, wgt, d->K, 9ull * d->C, 128, 128))) return rc;
     for (int b = 0; b < kCtBoxHeights; ++b)
-        if ((rc = make_map_nhwc(&P.mapX[b], in, d->N, d->H, d->W, Cred, 1, 8u >> b, (uint32_t)P.g.s, 128))) return rc;
+        if ((8 >> b) <= d->H && (rc = make_map_nhwc(&P.mapX[b], in, d->N, d->H, d->W, Cred, 1, 8u >> b, (uint32_t)P.g.s, 128))) return rc;
     const OperandLayout f = dgrad ? layout_mnmajor(128, 128, 1, 0) : layout_kmajor(128, 128), x = layout_kmajor(128, 128);
     P.f_desc_lo = f.desc_lo; P.x_desc_lo = x.desc_lo;
     P.idesc = make_idesc(true, true, f.major, x.major, p.pair ? 256 : 128, (uint32_t)p.npos);

@@ -129,10 +129,10 @@ static int conv_rangebn_recompute(const qbp_conv_desc *d, const int8_t *x_codes,
                                   const int8_t *w_codes, const qbp_qparams *qw, const float *gamma, const float *beta, int relu,
                                   float *save_mean, float *save_min, float *save_max, const qbp_requant *out,
                                   ColStatParts parts, float4 *fold, const CodeSums &w_sums, int *status, void *ws, size_t scratch,
-                                  bool beside, cudaStream_t st)
+                                  bool beside, const SumJob *extra, int extra_count, cudaStream_t st)
 {
     const int64_t rows = (int64_t)d->N * d->H * d->W;
-    const EpilogueTail first{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums, nullptr, 0, beside};
+    const EpilogueTail first{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums, extra, extra_count, beside};
     int rc = conv_s8_impl(QBP_CONV_FPROP, d, x_codes, qx, w_codes, qw, nullptr, nullptr, in_sums, &parts, status, ws, scratch, st,
                           &first);
     if (rc) return rc;
@@ -140,7 +140,7 @@ static int conv_rangebn_recompute(const qbp_conv_desc *d, const int8_t *x_codes,
     const EpilogueTail tail{fold, relu, out->qp, out->q, out->row_sums, 1, &w_sums};
     rc = conv_s8_impl(QBP_CONV_FPROP, d, x_codes, qx, w_codes, qw, nullptr, nullptr, in_sums, nullptr, status, ws, scratch, st, &tail);
     if (rc || !out->chan_sums) return rc;
-    return launch_colsum(out->q, true, rows, d->K, out->chan_sums, st);
+    return launch_colsum(out->q, true, rows, d->K, out->chan_sums, st, true);
 }
 
 }  // namespace qbp
@@ -202,12 +202,16 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_fwd_chained(cons
     // activations: nearest rounding, clamping values = min and max (Appendix B) -- or already quantised by the
     // Range BN of the layer before (Section 4); weights the same.  (the first launch also clears the status word)
     const int64_t w_rows = s.conv ? (int64_t)L->conv.K * L->conv.R * L->conv.S : s.cin;
-    QuantOperand xo{x, s.rows, s.cin, saved->x_codes, saved->qx, l.row_sums, want_totals ? saved->x_chan_sums : nullptr};
-    QuantOperand wo{w, w_rows, s.w_elems / w_rows, saved->w_codes, saved->qw, s.conv ? l.w_sums : nullptr, nullptr};
+    QuantOperand xo{x, s.rows, s.cin, saved->x_codes, saved->qx, in && in->row_sums ? nullptr : l.row_sums, want_totals ? saved->x_chan_sums : nullptr, nullptr};
+    QuantOperand wo{w, w_rows, s.w_elems / w_rows, saved->w_codes, saved->qw, s.conv ? l.w_sums : nullptr, nullptr, s.conv ? nullptr : l.w_sums};
     // (an input that came without its channel totals: cleared with the rest, summed up below; a filter has cin columns)
     const bool chained_totals = !x && want_totals && !in->chan_sums;
     if (chained_totals) wo.tot = saved->x_chan_sums;
-    if ((rc = quantize_operands(x ? &xo : nullptr, &wo, status, l.scratch, l.scratch_bytes, st))) return rc;
+    // ... and the totals that the last kernel of this call adds to, so that no memset stands between two kernels
+    const bool clear_out = out && out->chan_sums;
+    const bool no_launch = !s.conv || L->conv.R == 3 || !want_totals || (x ? quantizer_totals_supported(s.cin) : !chained_totals);
+    if ((rc = quantize_operands(x ? &xo : nullptr, &wo, status, l.scratch, l.scratch_bytes, st, no_launch, clear_out ? out->chan_sums : nullptr,
+                                clear_out ? 2 * s.cout : 0))) return rc;
     // what the products need beside the codes: each input row's code sum (convolution: each pixel's), the weights' sums,
     // each input channel's total -- whatever the quantising kernel did not leave, in one launch
     SumJob jobs[3];
@@ -216,9 +220,11 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_fwd_chained(cons
     if (in && in->row_sums) in_sums = in->row_sums;
     else if (!xo.row_sums_left) jobs[njobs++] = SumJob{saved->x_codes, s.rows, s.cin, kSumRows, 1, l.row_sums};
     const SumJob w_job = weight_sum_job(L, s, false, saved->w_codes, l.w_sums);
-    if (!wo.row_sums_left) jobs[njobs++] = w_job;
-    if ((want_totals && x && !xo.tot_left) || chained_totals)
-        jobs[njobs++] = SumJob{saved->x_codes, s.rows, s.cin, kSumCols, 1, nullptr, 0, 0, saved->x_chan_sums};
+    if (!wo.row_sums_left && !wo.col_sums_left) jobs[njobs++] = w_job;
+    // (the totals alone, of a 3 x 3 convolution: in the launch of its correction terms)
+    const SumJob tot_job{saved->x_codes, s.rows, s.cin, kSumCols, 1, nullptr, 0, 0, saved->x_chan_sums};
+    const bool tot_wanted = (want_totals && x && !xo.tot_left) || chained_totals, tot_with_terms = tot_wanted && !njobs && L->conv.R == 3;
+    if (tot_wanted && !tot_with_terms) jobs[njobs++] = tot_job;
     bool beside = false;
     if (njobs && (rc = launch_code_sums(jobs, njobs, st, ZeroJobs{}, &beside))) return rc;
     const CodeSums w_sums = sums_of(w_job), x_sums = sums_of(in_sums);
@@ -226,8 +232,8 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_fwd_chained(cons
     if (recompute)
         return conv_rangebn_recompute(&L->conv, saved->x_codes, saved->qx, in_sums, saved->w_codes, saved->qw, gamma, beta, L->relu,
                                       saved->save_mean, saved->save_min, saved->save_max, out, parts, l.fold, w_sums, status,
-                                      l.scratch, l.scratch_bytes, beside, st);
-    const EpilogueTail with_sums{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums, nullptr, 0, beside};
+                                      l.scratch, l.scratch_bytes, beside, &tot_job, tot_with_terms ? 1 : 0, st);
+    const EpilogueTail with_sums{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums, &tot_job, tot_with_terms ? 1 : 0, beside};
     if (s.conv)
         rc = conv_s8_impl(QBP_CONV_FPROP, &L->conv, saved->x_codes, saved->qx, saved->w_codes, saved->qw, nullptr, saved->z,
                           in_sums, parts.sum ? &parts : nullptr, status, l.scratch, l.scratch_bytes, st, &with_sums);
@@ -238,7 +244,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_fwd_chained(cons
     // the convolution's epilogue has left the statistics of z: no pass over z for them
     if (parts.sum)
         return rangebn_fwd_from_parts(saved->z, s.rows, s.cout, gamma, beta, L->relu, y, saved->save_mean, saved->save_min,
-                                      saved->save_max, parts, nullptr, out, st);
+                                      saved->save_max, parts, nullptr, out, st, clear_out);
     return qbp_rangebn_fwd_q8(saved->z, s.rows, s.cout, gamma, beta, L->relu, y, saved->save_mean, saved->save_min,
                               saved->save_max, nullptr, out, l.scratch, l.scratch_bytes, stream);
 }
@@ -304,7 +310,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_bwd(const qbp_la
                                         self_totals ? nullptr : tot_g, l.tot_g, clear_words, early, nearly);
     } else {
         if (!g) return fail(QBP_ERR_INVALID_ARG, "layer_bwd: this shape needs saved->g (the fp32 gradient is written and read back)");
-        if (l.clear_words) QBP_CUDA_OK(cudaMemsetAsync(l.tot_g, 0, sizeof(uint32_t) * (size_t)l.clear_words, st));
+        if ((rc = launch_clear(l.tot_g, l.clear_words, st))) return rc;
         int nparts = 0;
         rc = rangebn_bwd_impl(dy, saved->z, s.rows, s.cout, gamma, beta, L->relu, saved->save_mean, saved->save_min,
                               saved->save_max, g, dgamma, dbeta, l.scratch, l.scratch_bytes, l.range_parts, &nparts, st);

@@ -1261,10 +1261,10 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
 
     int rc = QBP_OK;
     ZeroJobs zero{};
-    if (!ext_status) { zero.p[0] = reinterpret_cast<uint32_t *>(status); zero.words[0] = 1; }
+    if (!ext_status) zero.add(status, 1);
     bool own = false;
     if ((rc = launch_code_sums(jobs, njobs, st, zero, &own))) return rc;
-    beside = njobs ? own : beside && !zero.words[0];         // (a tail's launch for its parameters comes in between)
+    beside = njobs ? own : beside && !zero.count;         // (a tail's launch for its parameters comes in between)
 
     // large products run on CTA pairs (256 x 256 tiles across two SMs); the column statistics are the
     // single-CTA kernel's (at most 256 columns: narrow either way)
@@ -1427,8 +1427,8 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
     int rc = QBP_OK;
     if (in_chan_sum) chan_sum = const_cast<int32_t *>(in_chan_sum);
     ZeroJobs zero{};
-    if (!ext_status) { zero.p[0] = reinterpret_cast<uint32_t *>(status); zero.words[0] = 1; }
-    bool beside = tail && tail->beside && !zero.words[0];    // (whether the launch before the product is one that it may run beside)
+    if (!ext_status) zero.add(status, 1);
+    bool beside = tail && tail->beside && !zero.count;    // (whether the launch before the product is one that it may run beside)
     if (tail && tail->keep_terms) { if ((rc = launch_code_sums(nullptr, 0, st, zero))) return rc; }
     else {
         SumJob jobs[2];
@@ -1458,8 +1458,9 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
     pick_pixel_box(d->N, d->H, d->W, bwl, bhl);
     // 3 x 3 with many channels on both sides: kernels of their own (the epilogue's tail is the single-CTA kernel's)
     const bool plain = !(tail && (tail->fold || tail->relu || tail->q));
-    if (plain && !stats && conv2t_eligible(d, dgrad, bwl, bhl))
-        return launch_conv2t(dgrad, d, in, q_in, wgt, q_w, acc_out, out, rowterm, colterm, status, beside, st);
+    ConvTPlan tp;
+    if (plain && !stats && conv2t_eligible(d, dgrad, bwl, bhl, tp))
+        return launch_conv2t(dgrad, d, in, q_in, wgt, q_w, acc_out, out, rowterm, colterm, tp, status, beside, st);
     if (plain && conv2_eligible(d, dgrad))
         return launch_conv2(dgrad, d, in, q_in, wgt, q_w, acc_out, out, rowterm, colterm, stats, status, bwl, bhl, beside, st);
 

@@ -11,7 +11,10 @@ namespace qbp {
 
 // ---- sums of stored codes (qbp_quant.cu) -------------------------------------
 int launch_rowsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int32_t *sums, cudaStream_t st);
-int launch_colsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int64_t *sums, cudaStream_t st);
+// (cleared: sums is zero already)
+int launch_colsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int64_t *sums, cudaStream_t st, bool cleared = false);
+// Clears 32-bit words in a kernel: a memset node between two kernels costs the stream 4 to 5 us, since neither overlaps it.
+int launch_clear(void *p, int64_t words, cudaStream_t st);
 // Sums of stored codes as a product takes them for its zero-point correction: element i is the sum of `pieces` int32
 // values p[i], p[i + stride], ... (sums along the rows of a tensor in pieces of its columns, so that nothing has to start at
 // zero and no atomics are needed).
@@ -35,7 +38,7 @@ inline CodeSums sums_of(const int32_t *p) { return CodeSums{p, 1, 0}; }
 //              row, first column, last column and the four corners (first row: first, last column; last row: the same) of
 //              every image: added to out64 [8][cols], which is zero beforehand
 // out64 (kSumCols): the whole sums are added to out64 [cols], which is zero beforehand, instead.
-// cols a multiple of 16, q 16-byte aligned, fewer than 2^31 rows.  zero: up to two regions of 32-bit words the launch clears (a
+// cols a multiple of 16, q 16-byte aligned, fewer than 2^31 rows.  zero: regions of 32-bit words the launch clears (a
 // status word, sums that a later kernel adds to).
 enum { kSumRows = 0, kSumCols = 1, kSumEdges = 2 };
 struct SumJob { const void *q; int64_t rows, cols; int kind, is_signed; int32_t *out; int H = 0, W = 0; int64_t *out64 = nullptr; };
@@ -84,14 +87,17 @@ int bifurcate_with_range_partials(const float *g, int64_t rows, int64_t cols, ui
                                   uint8_t *lo, qbp_qparams *qp16, const float2 *partials, int nparts, cudaStream_t st,
                                   int64_t *tot16 = nullptr, bool lo_signed = false);
 // The layer's operands quantised to 8 bits (nearest rounding, clamping values = min and max): the activation (nullable) and the
-// weights, in two launches.  row_sums [rows] / tot [cols] (each nullable): wanted sums of the stored codes; *_left: whether the
-// quantising kernel left them (it depends on the shape; the caller sums the codes up otherwise).  tot is cleared either way.
+// weights, in two launches.  row_sums [rows] / tot [cols] / col_sums [sum_pieces(rows, cols)][cols] (each nullable): wanted sums of the
+// stored codes; *_left: whether the quantising kernel left them (it depends on the shape; the caller sums the codes up otherwise).
+// tot is cleared either way, and so are clear_words 32-bit words at `clear`.  add_rows: row sums may be added up in pieces (slower
+// than whole rows; worth it where no launch for other sums follows).
 struct QuantOperand {
-    const float *v; int64_t rows, cols; int8_t *q; qbp_qparams *qp; int32_t *row_sums; int64_t *tot;
-    bool row_sums_left = false, tot_left = false;
+    const float *v; int64_t rows, cols; int8_t *q; qbp_qparams *qp; int32_t *row_sums; int64_t *tot; int32_t *col_sums;
+    bool row_sums_left = false, tot_left = false, col_sums_left = false;
 };
 size_t quantize_operands_ws_bytes();
-int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, size_t ws_bytes, cudaStream_t st);
+int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, size_t ws_bytes, cudaStream_t st, bool add_rows,
+                      void *clear = nullptr, int64_t clear_words = 0);
 bool quantizer_totals_supported(int64_t cols);
 // The convolution products with the per-pixel channel sums of the input codes supplied by the caller
 // (nullable: computed here) (qbp_mma.cu).
@@ -148,10 +154,11 @@ bool wgrad_self_totals(const qbp_conv_desc *d);
 bool conv_supported(const qbp_conv_desc *d);
 bool wgrad_conv_supported(const qbp_conv_desc *d);
 // Range BN forward from such partials instead of a statistics pass over x (qbp_rangebn.cu).
-// out_range / rq (each nullable): the exact range of y / its 8-bit codes for the next layer (see qbp_requant).
+// out_range / rq (each nullable): the exact range of y / its 8-bit codes for the next layer (see qbp_requant); totals_cleared:
+// rq->chan_sums is zero already.
 int rangebn_fwd_from_parts(const float *x, int64_t n, int64_t C, const float *gamma, const float *beta, int relu, float *y,
                            float *save_mean, float *save_min, float *save_max, const ColStatParts &parts,
-                           qbp_qparams *out_range, const qbp_requant *rq, cudaStream_t st);
+                           qbp_qparams *out_range, const qbp_requant *rq, cudaStream_t st, bool totals_cleared = false);
 
 // ---- TMA tensor maps ---------------------------------------------------------
 // A dense byte matrix [rows x cols] (cols innermost) read in boxes of
@@ -179,10 +186,11 @@ int launch_conv2(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp
                  const qbp_qparams *q_w, int32_t *acc_out, float *out, const int32_t *rowterm, const int32_t *colterm,
                  ColStatParts *stats, int *status, int bwl, int bhl, bool beside, cudaStream_t st);
 // ... and those whose output's statistics nobody wants
-bool conv2t_eligible(const qbp_conv_desc *d, bool dgrad, int bwl, int bhl);
+struct ConvTPlan { bool pair; int npos, tiles_n, units, windows, stages; uint32_t window_bytes; double cost; };
+bool conv2t_eligible(const qbp_conv_desc *d, bool dgrad, int bwl, int bhl, ConvTPlan &p);
 int launch_conv2t(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp_qparams *q_in, const int8_t *wgt,
                   const qbp_qparams *q_w, int32_t *acc_out, float *out, const int32_t *rowterm, const int32_t *colterm,
-                  int *status, bool beside, cudaStream_t st);
+                  const ConvTPlan &p, int *status, bool beside, cudaStream_t st);
 
 // ---- the dense weight gradient on CTA pairs (qbp_wgrad2.cu) ----------------------
 bool wgrad2_eligible(int64_t M, int64_t N, int64_t K);

@@ -278,9 +278,13 @@ struct QuantOut {
     int16_t *q16;    // 16-bit codes (nullable)
     int8_t *hi;      // high byte of the 16-bit code (nullable)
     uint8_t *lo;     // low byte (nullable)
-    int32_t *rowsum8;   // sums of the stored 8-bit codes over each row of `cols` (nullable; vector path only)
-    int rs_group;       // lanes that share a row: cols / 4, a power of two <= 32
-    int rs_shift;       // log2(rs_group)
+    // Sums of the stored 8-bit codes over each row of `cols` (nullable; vector path only).  rs_group lanes (a power of two that
+    // divides cols / 4, at most 32) add up.  rs_shift >= 0: they are a whole row, cols / 4 = 2^rs_shift.  Else the sums are zero
+    // beforehand and pieces are added: per group, or (rs_group 0: 128 columns or more, no multiple of 128) per warp, whose 128
+    // elements meet at most two (in groups of the four lanes that divide 4080 columns the atomics of 4096 such rows took 40 us).
+    int32_t *rowsum8;
+    int rs_group, rs_shift;
+    FastDiv rs_div;             // by cols / 4
     // Per-channel totals of the stored codes over all rows, added (64-bit atomics) to chansum8 [cols] / chansum16
     // [cols] (nullable; vector path, per tensor, cols / 4 a power of two <= 256: a thread then keeps its four
     // channels for its whole life).  The weight gradient's zero-point terms are built from such totals.
@@ -289,6 +293,16 @@ struct QuantOut {
     // gradient then runs both limbs as one s8 x s8 product); 0: plain unsigned low bytes.
     uint32_t lo_flip;
 };
+
+static QuantOut quant_out(int8_t *q8, int16_t *q16, int8_t *hi, uint8_t *lo, uint32_t lo_flip = 0u)
+{
+    QuantOut o{};
+    o.q8 = q8; o.q16 = q16; o.hi = hi; o.lo = lo; o.lo_flip = lo_flip;
+    return o;
+}
+
+// Column sums beside the codes of a quantising launch's second tensor (NULL: not wanted).
+struct StripJob { int64_t rows; int pieces; int32_t *col_sums; };
 
 // One tensor of a quantising launch.
 struct QuantJob {
@@ -477,8 +491,8 @@ __device__ __forceinline__ void quantize_body(const QuantJob &J, const PhiloxKey
                 }
             }
         }
-        if (o.rowsum8) {
-            // a row is rs_group consecutive lanes (groups are aligned: the lane index is j mod 32)
+        if (o.rowsum8 && o.rs_group) {
+            // (groups are aligned: the lane index is j mod 32)
 #pragma unroll
             for (int u = 0; u < kUnroll; ++u) {
                 int sum = rs[u];
@@ -486,7 +500,20 @@ __device__ __forceinline__ void quantize_body(const QuantJob &J, const PhiloxKey
                 for (int off = 16; off > 0; off >>= 1)
                     if (off < o.rs_group) sum += __shfl_xor_sync(0xffffffffu, sum, off);
                 const int64_t j = base + u * kThreads + threadIdx.x;
-                if (ok[u] && (threadIdx.x & (o.rs_group - 1)) == 0) o.rowsum8[j >> o.rs_shift] = sum;
+                if (ok[u] && (threadIdx.x & (o.rs_group - 1)) == 0) {
+                    if (o.rs_shift >= 0) o.rowsum8[j >> o.rs_shift] = sum;
+                    else                 atomicAdd(o.rowsum8 + o.rs_div.div((int)j), sum);
+                }
+            }
+        } else if (o.rowsum8) {
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) {
+                const int row = o.rs_div.div((int)(base + u * kThreads + threadIdx.x)), first = __shfl_sync(0xffffffffu, row, 0);
+                const int all = __reduce_add_sync(0xffffffffu, rs[u]), here = __reduce_add_sync(0xffffffffu, row == first ? rs[u] : 0);
+                if ((threadIdx.x & 31) == 0) {
+                    if (here) atomicAdd(o.rowsum8 + first, here);
+                    if (all != here) atomicAdd(o.rowsum8 + first + 1, all - here);
+                }
             }
         }
     }
@@ -562,14 +589,68 @@ __global__ void __launch_bounds__(kThreads, 4) bifurcate_kernel(const __grid_con
         for (int64_t i = (int64_t)nv << 2; i < J.n; ++i) quantize_scalar<true>(J, i, false, t8, t16, keys);
 }
 
-// A layer's weights (the first b_blocks blocks) and activation in one launch; nearest rounding, per tensor.
+// A matrix [rows x cols] (cols a multiple of 4) quantised to 8 bits by nearest rounding, with the sums of its columns in pieces of
+// its rows: block = (strip of 64 columns, piece), 16 rows at a time, four of them in flight per thread.
+__device__ __forceinline__ void quantize_strip(const QuantJob &J, const StripJob &S, int block)
+{
+    QParamsReg p8 = {0, 0}, none = {0, 0};
+    resolve_range(J.r, true, false, block == 0, p8, none);
+    const int cv = J.cols >> 2, strips = (cv + 15) >> 4, strip = block % strips, piece = block / strips;
+    const int v = strip * 16 + (threadIdx.x & 15), ty = threadIdx.x >> 4;
+    const int64_t r_begin = S.rows * piece / S.pieces, r_end = S.rows * (piece + 1) / S.pieces;
+    int acc[4] = {0, 0, 0, 0};
+    for (int64_t r = r_begin + ty; r < r_end && v < cv; r += 16 * kUnroll) {
+        float4 f[kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u)
+            if (r + 16 * u < r_end) f[u] = __ldcs(reinterpret_cast<const float4 *>(J.x) + (r + 16 * u) * cv + v);
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            if (r + 16 * u >= r_end) break;
+            const float e4[4] = {f[u].x, f[u].y, f[u].z, f[u].w};
+            uint32_t c[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                c[e] = (uint32_t)quantize_code<false>(e4[e], p8.inv, p8.zp_u, 255.0f, 0u);
+                acc[e] += (int)c[e] - 128;
+            }
+            reinterpret_cast<uint32_t *>(J.o.q8)[(r + 16 * u) * cv + v] = pack_bytes0(c) ^ 0x80808080u;
+        }
+    }
+    __shared__ int s_acc[kThreads / 32][64];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 16);              // (a warp holds two rows)
+        if ((threadIdx.x & 31) < 16) s_acc[threadIdx.x >> 5][(threadIdx.x & 15) * 4 + e] = acc[e];
+    }
+    __syncthreads();
+    const int col = strip * 64 + (int)threadIdx.x;
+    if (threadIdx.x < 64 && col < J.cols) {
+        int sum = 0;
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w) sum += s_acc[w][threadIdx.x];
+        S.col_sums[(int64_t)piece * J.cols + col] = sum;
+    }
+}
+
+// A layer's weights (the first b_blocks blocks; with the sums of their columns when S.col_sums is given) and activation in one
+// launch; nearest rounding, per tensor.
 template <bool TOTALS>
-__global__ void __launch_bounds__(kThreads) quantize_pair_kernel(const __grid_constant__ QuantJob a, const __grid_constant__ QuantJob b, int b_blocks)
+__global__ void __launch_bounds__(kThreads) quantize_pair_kernel(const __grid_constant__ QuantJob a, const __grid_constant__ QuantJob b, int b_blocks,
+                                                                 const __grid_constant__ StripJob S)
 {
     pdl_wait();
     const PhiloxKeys none = {};
-    if ((int)blockIdx.x < b_blocks) quantize_body<false, 4, false, false, false>(b, none, (int)blockIdx.x, b_blocks);
-    else                            quantize_body<false, 4, false, TOTALS, false>(a, none, (int)blockIdx.x - b_blocks, (int)gridDim.x - b_blocks);
+    if ((int)blockIdx.x >= b_blocks) quantize_body<false, 4, false, TOTALS, false>(a, none, (int)blockIdx.x - b_blocks, (int)gridDim.x - b_blocks);
+    else if (!TOTALS && S.col_sums)  quantize_strip(b, S, (int)blockIdx.x);
+    else                             quantize_body<false, 4, false, false, false>(b, none, (int)blockIdx.x, b_blocks);
+}
+
+// Regions cleared between two kernels (see launch_clear).
+__global__ void __launch_bounds__(kThreads) clear_kernel(const __grid_constant__ ZeroJobs zero)
+{
+    pdl_wait();
+    run_zero_jobs(zero, (int64_t)blockIdx.x * kThreads + threadIdx.x, (int64_t)gridDim.x * kThreads);
 }
 
 // The sums of up to eight code tensors in a launch of their own (see qbp_sums.cuh).
@@ -641,12 +722,24 @@ int fill_sum_jobs(const SumJob *jobs, int count, SumJobs &J, int *blocks)
     return QBP_OK;
 }
 
+int launch_clear(void *p, int64_t words, cudaStream_t st)
+{
+    if (words <= 0) return QBP_OK;
+    ZeroJobs zero{};
+    zero.add(p, words);
+    const int grid = (int)std::min<int64_t>(sm_count(), (words + kThreads - 1) / kThreads);
+    QBP_TRACE_BEGIN(st);
+    launch(clear_kernel, grid, kThreads, 0, st, zero);
+    QBP_LAUNCH_OK("clear_kernel");
+    return QBP_OK;
+}
+
 int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st, const ZeroJobs &zero, bool *beside)
 {
     if (beside) *beside = false;
     if (count == 0) {
-        for (int k = 0; k < 2; ++k)
-            if (zero.words[k]) QBP_CUDA_OK(cudaMemsetAsync(zero.p[k], 0, sizeof(uint32_t) * (size_t)zero.words[k], st));
+        for (int k = 0; k < zero.count; ++k)
+            if (int rc = launch_clear(zero.p[k], zero.words[k], st)) return rc;
         return QBP_OK;
     }
     SumJobs J{};
@@ -786,13 +879,20 @@ static int launch_quantize(const float *x, int64_t n, int64_t cols, int perch, i
     return QBP_OK;
 }
 
-// Whether the quantising kernel itself can emit the row sums of its 8-bit codes: per-tensor, 16-byte aligned
-// tensors whose rows are 4, 8, ..., 128 elements (a row is then a power-of-two group of lanes of one warp).
-static bool can_fuse_rowsums(const float *x, const void *q8, int64_t cols, const QuantOut &o)
+// Whether the quantising kernel itself can emit the row sums of its 8-bit codes: per-tensor, 16-byte aligned tensors whose rows are
+// 4, 8, ..., 128 elements (a row is then a power-of-two group of lanes of one warp) or, where the sums are cleared beforehand
+// (`add`), a multiple of 16 (added in pieces).  Fills the record in.
+static bool fuse_rowsums(const float *x, int64_t n, int64_t cols, bool add, int32_t *row_sums, QuantOut &o)
 {
-    const int64_t g = cols / 4;
-    return cols % 4 == 0 && g >= 1 && g <= 32 && (g & (g - 1)) == 0 && aligned16(x) && ((uintptr_t)q8 & 3) == 0 &&
-           (!o.q16 || ((uintptr_t)o.q16 & 7) == 0) && (!o.hi || ((uintptr_t)o.hi & 3) == 0) && (!o.lo || ((uintptr_t)o.lo & 3) == 0);
+    const int64_t v = cols / 4, group = std::min<int64_t>(v & -v, 32);
+    const bool whole = group == v;
+    if (cols % 4 || v < 1 || (!whole && !(add && cols % 16 == 0 && n / 4 < (1ll << 31) - 2048)) || !aligned16(x) || ((uintptr_t)o.q8 & 3) ||
+        (o.q16 && ((uintptr_t)o.q16 & 7)) || (o.hi && ((uintptr_t)o.hi & 3)) || (o.lo && ((uintptr_t)o.lo & 3)))
+        return false;
+    o.rowsum8 = row_sums; o.rs_group = !whole && v >= 32 && group < 32 ? 0 : (int)group;
+    o.rs_shift = -1; o.rs_div = FastDiv{};
+    if (whole) o.rs_shift = 31 - __builtin_clz((unsigned)v); else o.rs_div = make_fastdiv((int)v);
+    return true;
 }
 
 // Row / column sums of stored codes, complete.
@@ -801,11 +901,12 @@ int launch_rowsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int
     const SumJob job{q, rows, cols, kSumRows, is_signed ? 1 : 0, sums};
     return rows == 0 ? QBP_OK : launch_code_sums(&job, 1, st);
 }
-int launch_colsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int64_t *sums, cudaStream_t st)
+int launch_colsum(const void *q, bool is_signed, int64_t rows, int64_t cols, int64_t *sums, cudaStream_t st, bool cleared)
 {
     if (cols % 16 || !aligned16(q)) return fail(QBP_ERR_INVALID_ARG, "column sums need cols %% 16 == 0 and 16-byte aligned codes");
     const SumJob job{q, rows, cols, kSumCols, is_signed ? 1 : 0, nullptr, 0, 0, sums};
-    QBP_CUDA_OK(cudaMemsetAsync(sums, 0, sizeof(int64_t) * (size_t)cols, st));
+    if (!cleared)
+        if (int rc = launch_clear(sums, 2 * cols, st)) return rc;
     return rows == 0 ? QBP_OK : launch_code_sums(&job, 1, st);
 }
 
@@ -901,11 +1002,10 @@ static int bifurcate_tail(const float *g, int64_t rows, int64_t cols, uint64_t s
                           uint32_t tensor_id16, int8_t *q8, const RangeSrc &r, int32_t *row_sums8, int8_t *hi, uint8_t *lo,
                           cudaStream_t st, uint64_t index_base = 0, int64_t *tot16 = nullptr, bool lo_signed = false)
 {
-    QuantOut o = {q8, nullptr, hi, lo, nullptr, 0, 0, nullptr, nullptr, lo_signed ? 0x80808080u : 0u};
+    QuantOut o = quant_out(q8, nullptr, hi, lo, lo_signed ? 0x80808080u : 0u);
     if (tot16 && rows * cols > 0)                         // (cleared by the caller, who asked quantizer_totals_supported(cols) first)
         o.chansum16 = reinterpret_cast<unsigned long long *>(tot16);
-    const bool fused = row_sums8 && rows * cols > 0 && can_fuse_rowsums(g, q8, cols, o);
-    if (fused) { o.rowsum8 = row_sums8; o.rs_group = (int)(cols / 4); o.rs_shift = 31 - __builtin_clz((unsigned)o.rs_group); }
+    const bool fused = row_sums8 && rows * cols > 0 && fuse_rowsums(g, rows * cols, cols, false, row_sums8, o);
     int rc = launch_quantize(g, rows * cols, cols, 0, QBP_ROUND_STOCHASTIC, r, tensor_id8, tensor_id16, seed, o, st, index_base);
     if (rc) return rc;
     if (row_sums8 && !fused) return launch_rowsum(q8, true, rows, cols, row_sums8, st);
@@ -928,7 +1028,7 @@ bool quantizer_totals_supported(int64_t cols)
 }
 
 size_t quantize_operands_ws_bytes() { return 2 * align_up(sizeof(float2) * kMaxParts, 256); }
-int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, size_t ws_bytes, cudaStream_t st)
+int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, size_t ws_bytes, cudaStream_t st, bool add_rows, void *clear, int64_t clear_words)
 {
     if (!ws || ws_bytes < quantize_operands_ws_bytes()) return fail(QBP_ERR_WORKSPACE, "quantize: workspace too small");
     WsCarver c(ws, ws_bytes);
@@ -936,20 +1036,32 @@ int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, s
     QuantOut o[2];
     float2 *parts[2];
     bool vec[2] = {true, true};
-    ZeroJobs zero{{reinterpret_cast<uint32_t *>(status), nullptr}, {status ? 1 : 0, 0}};
+    // The weights' column sums beside their codes: of at most 3 M elements, in blocks of at most 64 K (a launch and its reading of the
+    // codes less: 3 us; 64 x 4080 -> 4080, whose 16.6 M the strips read at two thirds of the bandwidth, 158 -> 165 us).  Where they are
+    // not taken, a launch for code sums follows anyway, and takes the activation's rows as well.
+    StripJob S{w->rows, sum_pieces(w->rows, w->cols), nullptr};
+    const int64_t strip_blocks = (w->cols + 63) / 64 * S.pieces;
+    if (w->col_sums) {
+        if (x && w->cols % 4 == 0 && w->rows * w->cols <= std::min<int64_t>(strip_blocks * 65536, 3ll << 20) && aligned16(w->v) &&
+            ((uintptr_t)w->q & 3) == 0 && aligned16(x->v) && ((uintptr_t)x->q & 3) == 0 && !x->tot) S.col_sums = w->col_sums;
+        w->col_sums_left = S.col_sums != nullptr;
+        add_rows = add_rows && w->col_sums_left;
+    }
+    // (the status word, the caller's, the activation's or the weights' totals, either operand's row sums in pieces)
+    ZeroJobs zero{};
+    if (status) zero.add(status, 1);
+    zero.add(clear, clear_words);
     for (int i = 0; i < 2; ++i) {
         parts[i] = c.take<float2>(kMaxParts);
         if (!ops[i]) continue;
         QuantOperand &op = *ops[i];
         if (int rc = check_common(op.v, op.rows, op.cols, QBP_PER_TENSOR, QBP_ROUND_NEAREST, op.qp)) return rc;
-        o[i] = QuantOut{op.q, nullptr, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr, 0u};
-        if (op.row_sums && can_fuse_rowsums(op.v, op.q, op.cols, o[i])) {
-            o[i].rowsum8 = op.row_sums; o[i].rs_group = (int)(op.cols / 4); o[i].rs_shift = 31 - __builtin_clz((unsigned)o[i].rs_group);
-            op.row_sums_left = true;
-        }
+        o[i] = quant_out(op.q, nullptr, nullptr, nullptr);
+        op.row_sums_left = op.row_sums && fuse_rowsums(op.v, op.rows * op.cols, op.cols, add_rows, op.row_sums, o[i]);
+        if (op.row_sums_left && o[i].rs_shift < 0) zero.add(op.row_sums, op.rows);
         vec[i] = quant_vec(op.v, op.cols, 0, o[i]);
         if (op.tot) {
-            zero.p[1] = reinterpret_cast<uint32_t *>(op.tot); zero.words[1] = 2 * op.cols;
+            zero.add(op.tot, 2 * op.cols);
             if (i == 0 && vec[i] && quantizer_totals_supported(op.cols)) { o[i].chansum8 = reinterpret_cast<unsigned long long *>(op.tot); op.tot_left = true; }
         }
     }
@@ -972,10 +1084,13 @@ int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, s
         const bool totals = o[0].chansum8 != nullptr;
         const int qwave = sm_count() * (totals ? blocks_per_sm<quantize_pair_kernel<true>>(kThreads) : blocks_per_sm<quantize_pair_kernel<false>>(kThreads));
         int64_t ga = (nx + per_block - 1) / per_block, gb = (nw + per_block - 1) / per_block;
-        if (ga + gb > qwave) { gb = std::max<int64_t>(1, std::min(gb, qwave * nw / (nx + nw))); ga = std::min(ga, qwave - gb); }
+        if (S.col_sums) {
+            gb = strip_blocks;
+            ga = std::max<int64_t>(1, std::min<int64_t>(ga, qwave));
+        } else if (ga + gb > qwave) { gb = std::max<int64_t>(1, std::min(gb, qwave * nw / (nx + nw))); ga = std::min(ga, qwave - gb); }
         QBP_TRACE_BEGIN(st);
-        if (totals) launch(quantize_pair_kernel<true>, (int)(ga + gb), kThreads, (size_t)x->cols * 2 * sizeof(int), st, ja, jb, (int)gb);
-        else        launch(quantize_pair_kernel<false>, (int)(ga + gb), kThreads, 0, st, ja, jb, (int)gb);
+        if (totals) launch(quantize_pair_kernel<true>, (int)(ga + gb), kThreads, (size_t)x->cols * 2 * sizeof(int), st, ja, jb, (int)gb, S);
+        else        launch(quantize_pair_kernel<false>, (int)(ga + gb), kThreads, 0, st, ja, jb, (int)gb, S);
         QBP_LAUNCH_OK("quantize_pair_kernel");
         return QBP_OK;
     }
@@ -1072,9 +1187,8 @@ extern "C" __attribute__((visibility("default"))) int qbp_quantize_s8(const floa
     if (!q && rows * cols > 0) return fail(QBP_ERR_INVALID_ARG, "quantize_s8: q is NULL");
     if ((row_sums || col_sums) && granularity != QBP_PER_TENSOR)
         return fail(QBP_ERR_INVALID_ARG, "quantize_s8: row/column sums are per-tensor only");
-    QuantOut o = {q, nullptr, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr};
-    const bool fused = row_sums && rows * cols > 0 && can_fuse_rowsums(x, q, cols, o);
-    if (fused) { o.rowsum8 = row_sums; o.rs_group = (int)(cols / 4); o.rs_shift = 31 - __builtin_clz((unsigned)o.rs_group); }
+    QuantOut o = quant_out(q, nullptr, nullptr, nullptr);
+    const bool fused = row_sums && rows * cols > 0 && fuse_rowsums(x, rows * cols, cols, false, row_sums, o);
     int rc = quantize_any(8, x, rows, cols, granularity, rounding, seed, tensor_id, range_in, o, qp_out, ws, ws_bytes, st);
     if (rc) return rc;
     if (row_sums && !fused) { rc = launch_rowsum(q, true, rows, cols, row_sums, st); if (rc) return rc; }
@@ -1087,7 +1201,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_quantize_s16(const flo
                                 int8_t *hi, uint8_t *lo, qbp_qparams *qp_out, void *ws, size_t ws_bytes, void *stream)
 {
     if (!q && !hi && !lo) return fail(QBP_ERR_INVALID_ARG, "quantize_s16: q, hi and lo are all NULL");
-    QuantOut o = {nullptr, q, hi, lo, nullptr, 0, 0, nullptr, nullptr};
+    QuantOut o = quant_out(nullptr, q, hi, lo);
     return quantize_any(16, x, rows, cols, granularity, rounding, seed, tensor_id, range_in, o, qp_out, ws, ws_bytes,
                         (cudaStream_t)stream);
 }
@@ -1245,7 +1359,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_quantize_s8_static(con
     rc = static_scratch_address(&scratch);
     if (rc) return rc;
     // every partial the finalising kernel reads was written by this call's scan: nothing has to start at zero
-    QuantOut o = {q, nullptr, nullptr, nullptr, nullptr, 0, 0, nullptr, nullptr};
+    QuantOut o = quant_out(q, nullptr, nullptr, nullptr);
     return quantize_any(8, x, rows, cols, granularity, rounding, seed, tensor_id, nullptr, o, qp_out, scratch,
                         kStaticScratchBytes, (cudaStream_t)stream);
 }

@@ -1055,7 +1055,7 @@ namespace qbp {
 static int bn_fwd_apply_launch(const float *x, int64_t n_rows, int64_t n_stat, int64_t C, const float *gamma,
                                const float *beta, int relu, float *y, const float *save_mean, const float *save_min,
                                const float *save_max, qbp_qparams *out_range, const qbp_requant *rq, cudaStream_t st,
-                               bool reverse = false)
+                               bool reverse = false, bool totals_cleared = false)
 {
     const bool requant = rq != nullptr;
     if (requant && (!rq->q || !rq->qp)) return fail(QBP_ERR_INVALID_ARG, "rangebn_fwd: the requantisation record needs q and qp");
@@ -1086,7 +1086,8 @@ static int bn_fwd_apply_launch(const float *x, int64_t n_rows, int64_t n_stat, i
         if (fused_rowsum) { R.rowsum = rq->row_sums; R.rs_group = ga.tw; }
         if (rq->chan_sums) {
             if (n_rows >= (1ll << 22)) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "rangebn_fwd: per-channel code totals for fewer than 2^22 rows");
-            QBP_CUDA_OK(cudaMemsetAsync(rq->chan_sums, 0, sizeof(int64_t) * (size_t)C, st));
+            if (!totals_cleared)
+                if (int rc = launch_clear(rq->chan_sums, 2 * C, st)) return rc;
             R.chansum = reinterpret_cast<unsigned long long *>(rq->chan_sums);
         }
     }
@@ -1215,7 +1216,7 @@ int qbp::rangebn_fold_from_parts(int64_t n, int64_t C, const float *gamma, const
 // pass over x: finalize, then the apply pass.
 int qbp::rangebn_fwd_from_parts(const float *x, int64_t n, int64_t C, const float *gamma, const float *beta, int relu,
                                 float *y, float *save_mean, float *save_min, float *save_max, const ColStatParts &parts,
-                                qbp_qparams *out_range, const qbp_requant *rq, cudaStream_t st)
+                                qbp_qparams *out_range, const qbp_requant *rq, cudaStream_t st, bool totals_cleared)
 {
     if (!x || !save_mean || !save_min || !save_max || !parts.lo || !parts.hi || !parts.sum || parts.rows <= 0)
         return fail(QBP_ERR_INVALID_ARG, "rangebn_fwd: NULL tensor");
@@ -1224,7 +1225,7 @@ int qbp::rangebn_fwd_from_parts(const float *x, int64_t n, int64_t C, const floa
     launch(bn_stats_finalize_kernel, (int)C, 128, 0, st, parts.lo, parts.hi, parts.sum, parts.rows, (int)C, n, save_mean, save_min, save_max, nullptr);
     QBP_LAUNCH_OK("bn_stats_finalize_kernel");
     // (the product that left the statistics has just written x: its tail is in the L2)
-    return bn_fwd_apply_launch(x, n, n, C, gamma, beta, relu, y, save_mean, save_min, save_max, out_range, rq, st, true);
+    return bn_fwd_apply_launch(x, n, n, C, gamma, beta, relu, y, save_mean, save_min, save_max, out_range, rq, st, true, totals_cleared);
 }
 
 extern "C" __attribute__((visibility("default"))) int qbp_rangebn_bwd(const float *dy, const float *x, int64_t n, int64_t C, const float *gamma,
@@ -1340,8 +1341,8 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
     // each row's code sum by shuffles over the row's lanes of a warp; a row that spans several warps or blocks is
     // added up from its pieces (integer atomics on the zeroed sums: the result does not depend on the order)
     ZeroJobs zero{};
-    if (row_sums8 && (ga.tw > 32 || ga.slabs > 1)) { zero.p[0] = reinterpret_cast<uint32_t *>(row_sums8); zero.words[0] = n; }
-    zero.p[1] = static_cast<uint32_t *>(clear); zero.words[1] = clear_words;
+    if (row_sums8 && (ga.tw > 32 || ga.slabs > 1)) zero.add(row_sums8, n);
+    zero.add(clear, clear_words);
     if (few_rows(n, C)) {
         if ((rc = launch_bwd_few(dy, x, n, C, gamma, beta, relu, save_mean, save_min, save_max,
                                  BnBwdOut{dgamma, dbeta, coef, chan_range, relu ? relu_thr : nullptr}, zero, extra, extra_count, st)))

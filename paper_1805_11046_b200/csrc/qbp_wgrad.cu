@@ -974,16 +974,16 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
     else {
         P.cx = (const long long *)all[0].out64; P.chi = (const long long *)all[1].out64; P.clo = (const long long *)all[2].out64;
         if (nall == 6) { P.ex = (const long long *)all[3].out64; P.ehi = (const long long *)all[4].out64; P.elo = (const long long *)all[5].out64; }
-        if (tab) QBP_CUDA_OK(cudaMemsetAsync(tab, 0, sizeof(int64_t) * table, st));
+        if (tab && (rc = launch_clear(tab, 2 * (int64_t)table, st))) return rc;
     }
     ZeroJobs zero{};
-    if (!ext_status) { zero.p[0] = reinterpret_cast<uint32_t *>(status); zero.words[0] = 1; }
+    if (!ext_status) zero.add(status, 1);
     if (from_totals) {
         P.tot_x = (const long long *)tot_x; P.tot_g = (const long long *)tot_g16;
         P.tot_g_plain = tot_g_filled ? 1 : 0;
         if (!tot_g_filled) {
             P.ones_tot = (unsigned long long *)const_cast<int64_t *>(tot_g16);
-            if (!done_sums) { zero.p[1] = reinterpret_cast<uint32_t *>(P.ones_tot); zero.words[1] = 2 * N; }
+            if (!done_sums) zero.add(P.ones_tot, 2 * N);
         }
     }
     bool beside = false;
