@@ -18,11 +18,20 @@
 
 namespace qbp {
 
+// The second pass of either direction walks the rows from the last to the first and finds in the L2 what the statistics pass read
+// last: its rows from keep_from on (kKeepBytes of what the second pass reads), with loads that leave the lines there; the rest passes
+// through, evict-first, and so does all that the second passes read for the last time and write.  A forward's second pass leaves
+// the head of x for the backward of the same call site in the same way (keep_head).  Forward + backward, with the forward's pass
+// from the front and all of its loads evict-first, the backward's from the front with ordinary loads and stores, and so: 50176 x 256
+// 86.5 -> 72.4 us, 802816 x 64 272.5 -> 261.5, 12544 x 2048 151.6 -> 139.0.  48, 88 or 104 MB: within 0.5 us.
+constexpr int64_t kKeepBytes = 64ll << 20;
+static int64_t keep_from_row(int64_t rows, int64_t row_bytes) { return std::max<int64_t>(0, rows - kKeepBytes / row_bytes); }
+
 // ---------------------------------------------------------------- forward
 template <int VEC>
 __global__ void __launch_bounds__(kScanThreads) bn_stats_kernel(const float *__restrict__ x, int64_t rows, int C, int tw,
                                                                 float *__restrict__ part_lo, float *__restrict__ part_hi,
-                                                                double *__restrict__ part_sum)
+                                                                double *__restrict__ part_sum, int64_t keep_from)
 {
     pdl_wait();
     const ScanPos p = scan_pos<VEC>(C, tw);
@@ -40,7 +49,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_stats_kernel(const float *__r
             for (int u = 0; u < kScanUnroll; ++u) {
                 int64_t r = r0 + u * step;
                 ok[u] = r < rows;
-                if (ok[u]) v[u].load_stream(x + r * C + p.col);
+                if (ok[u]) { if (r0 < keep_from) v[u].load_stream(x + r * C + p.col); else v[u].load(x + r * C + p.col); }
             }
 #pragma unroll
             for (int u = 0; u < kScanUnroll; ++u)
@@ -157,7 +166,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_apply_kernel(const float *__r
                                                                 const float *__restrict__ vmax,
                                                                 const float *__restrict__ gamma,
                                                                 const float *__restrict__ beta, float Cn,
-                                                                float *__restrict__ y, BnRequant R, int reverse)
+                                                                float *__restrict__ y, BnRequant R, int reverse, int64_t keep_head)
 {
     pdl_wait();
     const ScanPos p = scan_pos<VEC>(C, tw);
@@ -198,9 +207,10 @@ __global__ void __launch_bounds__(kScanThreads) bn_apply_kernel(const float *__r
         for (int u = 0; u < kScanUnroll; ++u) {
             int64_t r = r0 + u * step;
             ok[u] = p.active && r < rows;
-            // (reverse: rows from the last to the first, when the kernel that wrote x ran just before and has left the
-            // tail of x in the L2)
-            if (ok[u]) v[u].load_stream(x + (reverse ? rows - 1 - r : r) * C + p.col);
+            // (reverse: rows from the last to the first, when the kernel that wrote or read x just before has left the tail of x
+            // in the L2; of those, the first keep_head rows stay)
+            const float *const at = x + (reverse ? rows - 1 - r : r) * C + p.col;
+            if (ok[u]) { if (rows - rb <= keep_head) v[u].load(at); else v[u].load_stream(at); }
         }
 #pragma unroll
         for (int u = 0; u < kScanUnroll; ++u) {
@@ -280,13 +290,9 @@ __global__ void __launch_bounds__(256) bn_out_range_kernel(const float *__restri
 // channel's maximum, where it is its minimum, and everywhere else -- as ext [6][blocks][C] (min, max of the ordinary
 // positions, then of the maxima, then of the minima).  dx is a monotone function of dy on each set (bn_dx), so the
 // finalize kernel knows the exact range of dx from these, before dx is computed.
-// The last kKeepBytes of both tensors are read with loads that leave them in the L2 (the rest passes through, evict-first) when the
-// second pass is bound by HBM.  The bifurcating pass that also writes the gradient starts with them (25.7 M elements 74 -> 68 us).  The
-// plain pass walks from the front: it gains where both tensors fit (two of 26 MB, statistics and second pass 31.4 -> 28.4 us), a little
-// where half of them does (two of 51 MB with their forward 86.4 -> 86.0), and nothing of larger ones.  The bifurcating pass alone is
-// bound by arithmetic and gains nothing (the layers of 56 x 56 x 64 and 14 x 14 x 256 lose a microsecond).  More than the L2 holds
-// beside the writes (88 MB) only costs.
-constexpr int64_t kKeepBytes = 64ll << 20;
+// The last kKeepBytes of both tensors stay in the L2 for the second pass (see above) where that is bound by HBM: the plain one, and
+// the bifurcating one that also writes the gradient (25.7 M elements 74 -> 68 us).  The bifurcating pass alone is bound by arithmetic
+// and gains nothing (the layers of 56 x 56 x 64 and 14 x 14 x 256 lose a microsecond).
 template <int VEC, bool RELU, bool EXT>
 __global__ void __launch_bounds__(kScanThreads) bn_bwd_stats_kernel(const float *__restrict__ dy,
                                                                     const float *__restrict__ x, int64_t rows, int C,
@@ -783,7 +789,8 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_apply_kernel(const float 
         for (int u = 0; u < kScanUnroll; ++u) {
             int64_t r = r0 + u * step;
             ok[u] = r < rows;
-            if (ok[u]) { vx[u].load(x + r * C + p.col); vd[u].load(dy + r * C + p.col); }
+            // (from the last row to the first)
+            if (ok[u]) { vx[u].load_stream(x + (rows - 1 - r) * C + p.col); vd[u].load_stream(dy + (rows - 1 - r) * C + p.col); }
         }
 #pragma unroll
         for (int u = 0; u < kScanUnroll; ++u)
@@ -796,7 +803,7 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_apply_kernel(const float 
                     vd[u].v[e] = bn_dx(d, bn_k2_ind(xv, lo[e], hi[e], k2[e]), s[e], g[e], m1[e]);
                     if (RANGE) { rlo = fminf(rlo, vd[u].v[e]); rhi = fmaxf(rhi, vd[u].v[e]); }
                 }
-                vd[u].store(dx + (r0 + u * step) * C + p.col);
+                vd[u].store_stream(dx + (rows - 1 - (r0 + u * step)) * C + p.col);
             }
     }
     }
@@ -1055,7 +1062,7 @@ namespace qbp {
 static int bn_fwd_apply_launch(const float *x, int64_t n_rows, int64_t n_stat, int64_t C, const float *gamma,
                                const float *beta, int relu, float *y, const float *save_mean, const float *save_min,
                                const float *save_max, qbp_qparams *out_range, const qbp_requant *rq, cudaStream_t st,
-                               bool reverse = false, bool totals_cleared = false)
+                               bool reverse, int64_t keep_head = 0, bool totals_cleared = false)
 {
     const bool requant = rq != nullptr;
     if (requant && (!rq->q || !rq->qp)) return fail(QBP_ERR_INVALID_ARG, "rangebn_fwd: the requantisation record needs q and qp");
@@ -1092,7 +1099,7 @@ static int bn_fwd_apply_launch(const float *x, int64_t n_rows, int64_t n_stat, i
         }
     }
     QBP_TRACE_BEGIN(st);
-#define QBP_BN_APPLY(V, RL, RQ) launch(bn_apply_kernel<V, RL, RQ>, grid_apply, kScanThreads, 0, st, x, n_rows, (int)C, ga.tw, save_mean, save_min, save_max, gamma, beta, Cn, y, R, reverse ? 1 : 0)
+#define QBP_BN_APPLY(V, RL, RQ) launch(bn_apply_kernel<V, RL, RQ>, grid_apply, kScanThreads, 0, st, x, n_rows, (int)C, ga.tw, save_mean, save_min, save_max, gamma, beta, Cn, y, R, reverse ? 1 : 0, keep_head)
     if (ga.vec == 4) {
         if (requant) { if (relu) QBP_BN_APPLY(4, true, true); else QBP_BN_APPLY(4, false, true); }
         else         { if (relu) QBP_BN_APPLY(4, true, false); else QBP_BN_APPLY(4, false, false); }
@@ -1121,8 +1128,8 @@ static int bn_fwd_stats_launch(const float *x, int64_t n, int64_t C, float *mean
                                               : blocks_per_sm<bn_stats_kernel<1>>(kScanThreads));
     const dim3 grid(g.nbx, g.slabs);
     QBP_TRACE_BEGIN(st);
-    if (g.vec == 4) launch(bn_stats_kernel<4>, grid, kScanThreads, 0, st, x, n, (int)C, g.tw, plo, phi, psum);
-    else            launch(bn_stats_kernel<1>, grid, kScanThreads, 0, st, x, n, (int)C, g.tw, plo, phi, psum);
+    if (g.vec == 4) launch(bn_stats_kernel<4>, grid, kScanThreads, 0, st, x, n, (int)C, g.tw, plo, phi, psum, keep_from_row(n, 4 * C));
+    else            launch(bn_stats_kernel<1>, grid, kScanThreads, 0, st, x, n, (int)C, g.tw, plo, phi, psum, keep_from_row(n, 4 * C));
     QBP_LAUNCH_OK("bn_stats_kernel");
     QBP_TRACE_BEGIN(st);
     launch(bn_stats_finalize_kernel, (int)C, 128, 0, st, plo, phi, psum, g.nbx, (int)C, n, mean, vmin, vmax, sum_out);
@@ -1154,7 +1161,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_rangebn_fwd_q8(const f
         return QBP_OK;
     }
     if ((rc = bn_fwd_stats_launch(x, n, C, save_mean, save_min, save_max, nullptr, ws, ws_bytes, st))) return rc;
-    return bn_fwd_apply_launch(x, n, n, C, gamma, beta, relu, y, save_mean, save_min, save_max, out_range, rq, st);
+    return bn_fwd_apply_launch(x, n, n, C, gamma, beta, relu, y, save_mean, save_min, save_max, out_range, rq, st, true, kKeepBytes / (4 * C));
 }
 
 extern "C" __attribute__((visibility("default"))) int qbp_rangebn_fwd(const float *x, int64_t n, int64_t C, const float *gamma, const float *beta, int relu,
@@ -1189,7 +1196,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_rangebn_fwd_apply(cons
     QBP_TRACE_BEGIN(st);
     launch(bn_mean_from_sum_kernel, (int)((C + 255) / 256), 256, 0, st, col_sum, col_min, col_max, (int)C, n_stat, save_mean, save_min, save_max);
     QBP_LAUNCH_OK("bn_mean_from_sum_kernel");
-    return bn_fwd_apply_launch(x, n_rows, n_stat, C, gamma, beta, relu, y, save_mean, save_min, save_max, out_range, rq, st);
+    return bn_fwd_apply_launch(x, n_rows, n_stat, C, gamma, beta, relu, y, save_mean, save_min, save_max, out_range, rq, st, true, kKeepBytes / (4 * C));
 }
 
 // The statistics half of the recompute fusion (a convolution run twice: once for the statistics, once to write
@@ -1225,7 +1232,7 @@ int qbp::rangebn_fwd_from_parts(const float *x, int64_t n, int64_t C, const floa
     launch(bn_stats_finalize_kernel, (int)C, 128, 0, st, parts.lo, parts.hi, parts.sum, parts.rows, (int)C, n, save_mean, save_min, save_max, nullptr);
     QBP_LAUNCH_OK("bn_stats_finalize_kernel");
     // (the product that left the statistics has just written x: its tail is in the L2)
-    return bn_fwd_apply_launch(x, n, n, C, gamma, beta, relu, y, save_mean, save_min, save_max, out_range, rq, st, true, totals_cleared);
+    return bn_fwd_apply_launch(x, n, n, C, gamma, beta, relu, y, save_mean, save_min, save_max, out_range, rq, st, true, 0, totals_cleared);
 }
 
 extern "C" __attribute__((visibility("default"))) int qbp_rangebn_bwd(const float *dy, const float *x, int64_t n, int64_t C, const float *gamma,
@@ -1255,7 +1262,7 @@ static int bn_bwd_stats_launch(const float *dy, const float *x, int64_t n_rows, 
     const dim3 grid(g.nbx, g.slabs);
     const double Cnd = 1.0 / std::sqrt(2.0 * std::log((double)n_stat));
     const float Cn = (float)Cnd;
-    const int64_t keep_from = keep_tail ? std::max<int64_t>(0, n_rows - kKeepBytes / (2 * (int64_t)sizeof(float) * C)) : n_rows;
+    const int64_t keep_from = keep_tail ? keep_from_row(n_rows, 8 * C) : n_rows;
     QBP_TRACE_BEGIN(st);
 #define QBP_BN_BSTATS(V, R, E) launch(bn_bwd_stats_kernel<V, R, E>, grid, kScanThreads, 0, st, dy, x, n_rows, (int)C, g.tw, save_mean, save_min, save_max, gamma, beta, Cn, pa, pb, ext, zero, keep_from)
     if (ext) {
