@@ -615,72 +615,77 @@ __device__ __forceinline__ long long wg_tap_part(const WgradParams &P, bool of_x
     return part == 3 ? v : -v;
 }
 
-// The same for a convolution, output [n][tap][c].  A block takes 64 channels of one tap and NB output channels: SX and SG
-// are added up once per block (once per element they are tens of loads each: 78 us for a 256 -> 256 channel 3x3 filter, five times
-// what its partials take to read), four groups of 64 threads share the slices,
-// each thread with eight loads in flight, and meet in shared memory.
-template <int NB>
-__global__ void __launch_bounds__(256) wgrad_conv_finalize_kernel(const __grid_constant__ WgradParams P)
+// The same for a convolution, output [n][tap][c].  A block takes 64 channels of one tap and NB output channels per group of 64 threads:
+// SX and SG are added up once per block (once per element they are tens of loads each: 78 us for a 256 -> 256 channel 3x3 filter).
+// Q = 4: the groups share the slices of the same NB output channels and meet in shared memory; Q = 1, for items of one or two slices:
+// each takes all slices of NB channels of its own (three of four groups had nothing to load).
+// Bound by latency: rounds of resident blocks, each a few dependent loads long.  So four blocks share an SM (one pointer for the NB
+// columns of a tile, 128 values apart: at 124 registers, two blocks), eight or more loads are in flight per thread, and NB is as
+// large as leaves four blocks per SM.  256 -> 256 channels, 8 slices: 16.5 -> 10.0 us; 512 -> 512 with
+// 64 x 7 x 7 positions, 1 slice: 46.9 -> 11.0.
+template <int NB, int Q>
+__global__ void __launch_bounds__(256, 4) wgrad_conv_finalize_kernel(const __grid_constant__ WgradParams P)
 {
     pdl_wait();
-    constexpr int U = 8 / NB;                              // slices in flight per output channel
-    __shared__ long long s_part[NB][4][64], s_sx[4][64], s_sg[4][NB];
+    constexpr int U = NB == 8 ? 2 : 8 / NB;                // slices in flight per output channel
+    constexpr int NN = Q == 1 ? 4 * NB : NB;               // output channels of the block
+    __shared__ long long s_part[Q == 1 ? 1 : NB][4][64], s_sx[4][64], s_sg[4][NN];
     const int cblocks = (P.C + 63) / 64;
-    const int tap = (int)blockIdx.x / cblocks, c = ((int)blockIdx.x % cblocks) * 64 + (threadIdx.x & 63);
+    const int tap = (int)blockIdx.x / cblocks, cl = threadIdx.x & 63, c = ((int)blockIdx.x % cblocks) * 64 + cl;
     const int q = threadIdx.x >> 6;
-    const int n0 = (int)blockIdx.y * NB;
+    const int n0 = (int)blockIdx.y * NN, n_mine = n0 + (Q == 1 ? q * NB : 0);
     const int r = tap / P.S, s = tap % P.S, pad = P.pad;
-    const bool c_ok = c < P.C;
+    const bool c_ok = c < P.C && n_mine < P.N;
     // the CTAs of this channel's items
     const int at = (tap / P.a_chunks) * P.tiles_c + (c_ok ? c : 0) / P.rb_a, row = (tap % P.a_chunks) * P.rb_a + (c_ok ? c : 0) % P.rb_a;
     const int ag = at / P.ma, j = at % P.ma, full_items = P.ctas_full / P.s_full;
     long long raw[NB];
-    const long long *src[NB];
-    int slices = 0;
 #pragma unroll
-    for (int i = 0; i < NB; ++i) {
-        const int n = min(n0 + i, (int)P.N - 1);
-        const int item = ag * P.tiles_b + n / P.bn;
-        const int first = item < full_items ? item * P.s_full : P.ctas_full + (item - full_items) * P.s_last;
-        slices = item < full_items ? P.s_full : P.s_last;  // (the same for all: it depends on the A group alone)
-        src[i] = P.part + (int64_t)first * P.part_stride + ((int64_t)j * P.bn + n % P.bn) * 128 + row;
-        raw[i] = 0;
-    }
+    for (int i = 0; i < NB; ++i) raw[i] = 0;
     if (c_ok) {
-        int sl = q;
-        for (; sl + 4 * (U - 1) < slices; sl += 4 * U) {
+        // (N and a tile's columns are multiples of NB: these output channels lie in one tile)
+        const int item = ag * P.tiles_b + n_mine / P.bn;
+        const int first = item < full_items ? item * P.s_full : P.ctas_full + (item - full_items) * P.s_last;
+        const int slices = item < full_items ? P.s_full : P.s_last;
+        const long long *const src = P.part + (int64_t)first * P.part_stride + ((int64_t)j * P.bn + n_mine % P.bn) * 128 + row;
+        for (int sl = Q == 1 ? 0 : q; sl < slices; sl += Q * U) {
             long long v[NB][U];
 #pragma unroll
-            for (int i = 0; i < NB; ++i)
+            for (int u = 0; u < U; ++u)
 #pragma unroll
-                for (int u = 0; u < U; ++u) v[i][u] = __ldcs(src[i] + (int64_t)(sl + 4 * u) * P.part_stride);
+                for (int i = 0; i < NB; ++i) v[i][u] = sl + Q * u < slices ? __ldcs(src + (int64_t)(sl + Q * u) * P.part_stride + i * 128) : 0;
 #pragma unroll
             for (int i = 0; i < NB; ++i)
 #pragma unroll
                 for (int u = 0; u < U; ++u) raw[i] += v[i][u];
         }
-        for (; sl < slices; sl += 4)
-#pragma unroll
-            for (int i = 0; i < NB; ++i) raw[i] += __ldcs(src[i] + (int64_t)sl * P.part_stride);
     }
+    if (Q != 1) {
 #pragma unroll
-    for (int i = 0; i < NB; ++i) s_part[i][q][threadIdx.x & 63] = raw[i];
-    s_sx[q][threadIdx.x & 63] = c_ok ? wg_tap_part(P, true, c, r, s, q) : 0;
-    if ((threadIdx.x & 63) < NB) s_sg[q][threadIdx.x & 63] = wg_tap_part(P, false, min(n0 + (int)(threadIdx.x & 63), (int)P.N - 1), r, s, q);
+        for (int i = 0; i < NB; ++i) s_part[Q == 1 ? 0 : i][q][cl] = raw[i];
+    }
+    s_sx[q][cl] = c < P.C ? wg_tap_part(P, true, c, r, s, q) : 0;
+    if (cl < NN) s_sg[q][cl] = wg_tap_part(P, false, min(n0 + cl, (int)P.N - 1), r, s, q);
     __syncthreads();
     // (signed low bytes: the limbs hold g16 - 128, against the zero-point zg - 128)
     const long long zx = P.qx->zero_point, zg = P.qg->zero_point - (P.lo_signed ? 128 : 0);
     const long long rows_ok = P.H - (r < pad ? pad - r : r - pad), cols_ok = P.W - (s < pad ? pad - s : s - pad);
     const long long count = (long long)P.Nimg * (rows_ok > 0 ? rows_ok : 0) * (cols_ok > 0 ? cols_ok : 0);
     const float scale = __fmul_rn(P.qx->scale, P.qg->scale);
-    for (int i = threadIdx.x; i < NB * 64; i += 256) {
-        const int cl = i & 63, nl = i >> 6, n = n0 + nl, co = ((int)blockIdx.x % cblocks) * 64 + cl;
-        if (n >= P.N || co >= P.C) continue;
-        const long long SX = s_sx[0][cl] + s_sx[1][cl] + s_sx[2][cl] + s_sx[3][cl], SG = s_sg[0][nl] + s_sg[1][nl] + s_sg[2][nl] + s_sg[3][nl];
-        const long long acc = s_part[nl][0][cl] + s_part[nl][1][cl] + s_part[nl][2][cl] + s_part[nl][3][cl] - zg * SX - zx * SG + count * zx * zg;
-        const int64_t e = ((int64_t)n * P.taps + tap) * P.C + co;
+    const long long xterm = count * zx * zg - zg * (s_sx[0][cl] + s_sx[1][cl] + s_sx[2][cl] + s_sx[3][cl]);
+    auto finish = [&](int nl, long long part) {
+        const int n = n0 + nl;
+        if (n >= P.N || c >= P.C) return;
+        const long long acc = part + xterm - zx * (s_sg[0][nl] + s_sg[1][nl] + s_sg[2][nl] + s_sg[3][nl]);
+        const int64_t e = ((int64_t)n * P.taps + tap) * P.C + c;
         if (P.acc_out) P.acc_out[e] = acc;
         if (P.dW) P.dW[e] = __fmul_rn((float)acc, scale);
+    };
+    if (Q == 1) {
+#pragma unroll
+        for (int i = 0; i < NB; ++i) finish(q * NB + i, raw[i]);
+    } else {
+        for (int nl = q; nl < NB; nl += 4) finish(nl, s_part[nl][0][cl] + s_part[nl][1][cl] + s_part[nl][2][cl] + s_part[nl][3][cl]);
     }
 }
 
@@ -1025,14 +1030,21 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
     launch(kernel, pl.grid, kWgThreads, pl.smem, st, P);
     QBP_LAUNCH_OK("qbp_wgrad_kernel");
     if (d) {
-        // output channels per block: as many as still leave four blocks per SM
         const int64_t per_n = (int64_t)P.taps * ((d->C + 63) / 64);
-        const int nb = per_n * (d->K / 8) >= 4ll * sm_count() ? 8 : per_n * (d->K / 4) >= 4ll * sm_count() ? 4 : 2;
-        const dim3 grid((unsigned)per_n, (unsigned)((d->K + nb - 1) / nb));
+        const bool whole = std::max(P.s_full, P.s_last) <= 2;
+        const int groups = whole ? 4 : 1;
+        const int nb = per_n * (d->K / (8 * groups)) >= 4ll * sm_count() ? 8 : per_n * (d->K / (4 * groups)) >= 4ll * sm_count() ? 4 : 2;
+        const dim3 grid((unsigned)per_n, (unsigned)((d->K + nb * groups - 1) / (nb * groups)));
         QBP_TRACE_BEGIN(st);
-        if (nb == 8)      launch(wgrad_conv_finalize_kernel<8>, grid, 256, 0, st, P);
-        else if (nb == 4) launch(wgrad_conv_finalize_kernel<4>, grid, 256, 0, st, P);
-        else              launch(wgrad_conv_finalize_kernel<2>, grid, 256, 0, st, P);
+        if (whole) {
+            if (nb == 8)      launch(wgrad_conv_finalize_kernel<8, 1>, grid, 256, 0, st, P);
+            else if (nb == 4) launch(wgrad_conv_finalize_kernel<4, 1>, grid, 256, 0, st, P);
+            else              launch(wgrad_conv_finalize_kernel<2, 1>, grid, 256, 0, st, P);
+        } else {
+            if (nb == 8)      launch(wgrad_conv_finalize_kernel<8, 4>, grid, 256, 0, st, P);
+            else if (nb == 4) launch(wgrad_conv_finalize_kernel<4, 4>, grid, 256, 0, st, P);
+            else              launch(wgrad_conv_finalize_kernel<2, 4>, grid, 256, 0, st, P);
+        }
         QBP_LAUNCH_OK("wgrad_conv_finalize_kernel");
     } else if (!P.direct) {
         const int blocks = (int)((outs * kWgFinalizeLanes + 255) / 256);

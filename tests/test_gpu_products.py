@@ -443,6 +443,13 @@ def test_wgrad_conv_finalize_block_shapes(B, N, H, W, C, K, R):
     assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
 
 
+@pytest.mark.parametrize("N,H,W,C,K,R", [(2, 7, 7, 512, 512, 3), (3, 5, 4, 416, 480, 3), (1, 6, 6, 256, 544, 3), (2, 4, 4, 1056, 1024, 1), (9, 8, 8, 480, 96, 3)])
+def test_wgrad_conv_finalize_of_whole_items(B, N, H, W, C, K, R):
+    """Many output tiles, one or two slices each: every group of threads finishes output channels of its own (several groups of them per
+    block, ragged channels on either side, one slice and two, the groups sharing slices beside them)."""
+    test_wgrad_conv_finalize_block_shapes(B, N, H, W, C, K, R)
+
+
 @pytest.mark.parametrize("M", [1, 31, 127, 128, 255, 256, 257, 4095, 8200])
 @pytest.mark.parametrize("N,K", [(16, 144), (272, 16)])
 def test_wgrad_code_sums_in_pieces_of_the_rows(B, M, N, K):
