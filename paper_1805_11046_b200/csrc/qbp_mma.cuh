@@ -53,10 +53,11 @@ inline CodeSums sums_of(const SumJob &j)
 {
     return j.kind == kSumRows ? sums_of(j.out) : CodeSums{j.out, sum_pieces(j.rows, j.cols), j.cols};
 }
-// beside (nullable): set when the product launched next may run beside this kernel (see launch()).  Sums of fewer bytes than
-// kSumsBesideBytes take a microsecond or two, less than the product's launch: they let it go at their start, and it waits for them
-// (a linear layer of 64 x 256 -> 128 37.6 us otherwise, 37.4 so; of 1024 x 2048 -> 1008 77.6 beside, 78.3 waiting).
-constexpr int64_t kSumsBesideBytes = 1 << 20;
+// beside (nullable): set when the product launched next may run beside this kernel (see launch()).  Sums of fewer than a megabyte
+// take a microsecond or two, less than the product's launch: they let it go at their start, and it waits for them.  Sums of more than
+// 32 want HBM for themselves (weight gradient 8192 x 2048 x 4096 with its 67 MB 123.7 us beside them, 122.8 behind; linear layer
+// 1024 x 2048 -> 1008 with 4 MB 77.6 and 78.3).
+constexpr int64_t kSumsBesideMin = 1 << 20, kSumsBesideMax = 32 << 20;
 int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st, const ZeroJobs &zero = ZeroJobs{}, bool *beside = nullptr);
 
 // ---- per-tensor range scan (qbp_quant.cu): leaves *nparts (min, max) pairs at ws, for RangeSrc::parts -------------

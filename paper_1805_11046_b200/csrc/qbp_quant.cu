@@ -7,6 +7,7 @@
 // fill every SM.  Also hosts the library's error-reporting state.
 #include "qbp_colscan.cuh"
 #include "qbp_mma.cuh"
+#include "qbp_pair.cuh"
 #include "qbp_sums.cuh"
 
 #include <algorithm>
@@ -368,6 +369,28 @@ __device__ __forceinline__ uint32_t pack_bytes2(const uint32_t (&c)[4])
     return __byte_perm(__byte_perm(c[0], c[1], 0x0062), __byte_perm(c[2], c[3], 0x0062), 0x5410);
 }
 
+// A warp's share of the row sums: lane l has the codes of vector j = j of lane 0 + l (ok: inside the tensor), sum their sum.
+__device__ __forceinline__ void put_row_sum_group(const QuantOut &o, int64_t j, bool ok, int sum)          // rs_group > 0
+{
+    // (groups are aligned: the lane index is j mod 32)
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+        if (off < o.rs_group) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    if (ok && (threadIdx.x & (o.rs_group - 1)) == 0) {
+        if (o.rs_shift >= 0) o.rowsum8[j >> o.rs_shift] = sum;
+        else                 atomicAdd(o.rowsum8 + o.rs_div.div((int)j), sum);
+    }
+}
+__device__ __forceinline__ void put_row_sum_wide(const QuantOut &o, int64_t j, int sum)                    // rs_group == 0
+{
+    const int row = o.rs_div.div((int)j), first = __shfl_sync(0xffffffffu, row, 0);
+    const int all = __reduce_add_sync(0xffffffffu, sum), here = __reduce_add_sync(0xffffffffu, row == first ? sum : 0);
+    if ((threadIdx.x & 31) == 0) {
+        if (here) atomicAdd(o.rowsum8 + first, here);
+        if (all != here) atomicAdd(o.rowsum8 + first + 1, all - here);
+    }
+}
+
 // PERCH is a template parameter so that the per-tensor instance (the hot one: it is bound by its instruction
 // count when rounding stochastically) carries none of the per-channel parameter handling.
 // TOTALS: the instance that also leaves the per-channel totals (the others carry none of that work).
@@ -493,29 +516,11 @@ __device__ __forceinline__ void quantize_body(const QuantJob &J, const PhiloxKey
             }
         }
         if (o.rowsum8 && o.rs_group) {
-            // (groups are aligned: the lane index is j mod 32)
 #pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-                int sum = rs[u];
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1)
-                    if (off < o.rs_group) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-                const int64_t j = base + u * kThreads + threadIdx.x;
-                if (ok[u] && (threadIdx.x & (o.rs_group - 1)) == 0) {
-                    if (o.rs_shift >= 0) o.rowsum8[j >> o.rs_shift] = sum;
-                    else                 atomicAdd(o.rowsum8 + o.rs_div.div((int)j), sum);
-                }
-            }
+            for (int u = 0; u < kUnroll; ++u) put_row_sum_group(o, base + u * kThreads + threadIdx.x, ok[u], rs[u]);
         } else if (o.rowsum8) {
 #pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-                const int row = o.rs_div.div((int)(base + u * kThreads + threadIdx.x)), first = __shfl_sync(0xffffffffu, row, 0);
-                const int all = __reduce_add_sync(0xffffffffu, rs[u]), here = __reduce_add_sync(0xffffffffu, row == first ? rs[u] : 0);
-                if ((threadIdx.x & 31) == 0) {
-                    if (here) atomicAdd(o.rowsum8 + first, here);
-                    if (all != here) atomicAdd(o.rowsum8 + first + 1, all - here);
-                }
-            }
+            for (int u = 0; u < kUnroll; ++u) put_row_sum_wide(o, base + u * kThreads + threadIdx.x, rs[u]);
         }
     }
     if (block == 0 && threadIdx.x == 0)
@@ -647,6 +652,102 @@ __global__ void __launch_bounds__(kThreads) quantize_pair_kernel(const __grid_co
     else                             quantize_body<false, 4, false, false, false>(b, none, (int)blockIdx.x, b_blocks);
 }
 
+// A layer's activation and weights, each of at most kSmallElems elements: range, codes and their sums in one launch.  A tensor is a
+// cluster of eight CTAs that holds it in registers (two float4 a thread); their ranges meet in distributed shared memory.  What the
+// sums are added to is cleared before the cluster's barrier.  (A scan and a quantiser are two launches of 2 and 4 us for such tensors,
+// of which the reading is a fraction: the layer of 64 x 256 -> 128 33.4 -> 32.3 us a step.  Not for larger tensors, whose bytes eight
+// SMs take too long to read: weights of 147 K elements 6.7 us against 6.4, the layer of 512 x 512 -> 512 53.0 against 51.9.)
+// colsum [cols]: column sums, 32 bits, added to the first of `pieces` rows; o.chansum8: 64 bits.
+struct SmallOperand { const float *x; int n4, cols; QuantOut o; qbp_qparams *qp; int32_t *colsum; int pieces; };
+struct SmallJob { SmallOperand op[2]; ZeroJobs zero; };
+constexpr int kSmallCtas = 8, kSmallThreads = 1024, kSmallVecs = 2, kSmallMaxCols = 8192;
+constexpr int64_t kSmallElems = 4ll * kSmallCtas * kSmallThreads * kSmallVecs;
+__device__ __forceinline__ void quantize_small_body(const SmallJob &J)
+{
+    extern __shared__ int s_cols[];                          // [cols] when column sums or totals are wanted
+    __shared__ float2 s_range;
+    const SmallOperand &op = J.op[blockIdx.x / kSmallCtas];
+    const QuantOut &o = op.o;
+    const int rank = (int)cluster_ctarank(), t = rank * kSmallThreads + (int)threadIdx.x;
+    constexpr int kAll = kSmallCtas * kSmallThreads;
+    const bool columns = op.colsum || o.chansum8;
+    float4 v[kSmallVecs];
+    float lo = INFINITY, hi = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < kSmallVecs; ++k)
+        if (t + k * kAll < op.n4) v[k] = __ldg(reinterpret_cast<const float4 *>(op.x) + t + k * kAll);
+    if (blockIdx.x < kSmallCtas) run_zero_jobs(J.zero, t, kAll);
+    if (o.rowsum8 && o.rs_shift < 0)
+        for (int i = t; i < op.n4 / (op.cols >> 2); i += kAll) o.rowsum8[i] = 0;
+    if (op.colsum)
+        for (int i = t; i < op.pieces * op.cols; i += kAll) op.colsum[i] = 0;
+    if (o.chansum8)
+        for (int i = t; i < op.cols; i += kAll) o.chansum8[i] = 0;
+    if (columns)
+        for (int i = threadIdx.x; i < op.cols; i += kSmallThreads) s_cols[i] = 0;
+#pragma unroll
+    for (int k = 0; k < kSmallVecs; ++k)
+        if (t + k * kAll < op.n4) {
+            lo = fminf(fminf(lo, fminf(v[k].x, v[k].y)), fminf(v[k].z, v[k].w));
+            hi = fmaxf(fmaxf(hi, fmaxf(v[k].x, v[k].y)), fmaxf(v[k].z, v[k].w));
+        }
+    const float2 mine = block_min_max(lo, hi);
+    if (threadIdx.x == 0) s_range = mine;
+    __syncthreads();
+    cluster_sync_all();
+    {
+        const int lane = threadIdx.x & 31;
+        float2 r = make_float2(INFINITY, -INFINITY);
+        if (lane < kSmallCtas) {
+            const uint32_t at = map_to_cta(&s_range, (uint32_t)lane);
+            asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(r.x), "=f"(r.y) : "r"(at) : "memory");
+        }
+        lo = warp_min(r.x); hi = warp_max(r.y);
+    }
+    // (a CTA's range may be read until all have read it: the wait for this is at the end)
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    const qbp_qparams qp = make_qparams(lo, hi, 8);
+    if (t == 0) *op.qp = qp;
+    const QParamsReg p = qparams_reg(qp, 8);
+    const int cv = op.cols >> 2;
+#pragma unroll
+    for (int k = 0; k < kSmallVecs; ++k) {
+        const int j = t + k * kAll;
+        if (j - (int)(threadIdx.x & 31) >= op.n4) break;     // (the warp's)
+        const bool ok = j < op.n4;
+        int sum = 0;
+        if (ok) {
+            const float e4[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+            uint32_t c[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) c[e] = (uint32_t)quantize_code<false>(e4[e], p.inv, p.zp_u, 255.0f, 0u);
+            const uint32_t packed = pack_bytes0(c) ^ 0x80808080u;
+            reinterpret_cast<uint32_t *>(o.q8)[j] = packed;
+            sum = __dp4a((int)packed, 0x01010101, 0);
+            if (columns) {
+                const int c0 = (j % cv) * 4;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) atomicAdd(&s_cols[c0 + e], (int)c[e] - 128);
+            }
+        }
+        if (o.rowsum8) { if (o.rs_group) put_row_sum_group(o, j, ok, sum); else put_row_sum_wide(o, j, sum); }
+    }
+    if (columns) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < op.cols; i += kSmallThreads) {
+            const int sum = s_cols[i];
+            if (sum && op.colsum) atomicAdd(op.colsum + i, sum);
+            if (sum && o.chansum8) atomicAdd(o.chansum8 + i, (unsigned long long)(long long)sum);
+        }
+    }
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads, 1) operands_prep_kernel(const __grid_constant__ SmallJob J)
+{
+    pdl_wait();
+    quantize_small_body(J);
+}
+
 // Regions cleared between two kernels (see launch_clear).
 __global__ void __launch_bounds__(kThreads) clear_kernel(const __grid_constant__ ZeroJobs zero)
 {
@@ -749,7 +850,7 @@ int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st, const ZeroJ
     J.zero = zero;
     int64_t bytes = 0;
     for (int i = 0; i < count; ++i) bytes += jobs[i].rows * jobs[i].cols;
-    if (beside && bytes >= kSumsBesideBytes) { *beside = true; J.beside = 1; }
+    if (beside && bytes >= kSumsBesideMin && bytes <= kSumsBesideMax) { *beside = true; J.beside = 1; }
     QBP_TRACE_BEGIN(st);
     launch(code_sums_kernel, blocks, kSumThreads, 0, st, J);
     QBP_LAUNCH_OK("code_sums_kernel");
@@ -1038,6 +1139,39 @@ int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, s
     QuantOut o[2];
     float2 *parts[2];
     bool vec[2] = {true, true};
+    // (the status word, the caller's, the activation's or the weights' totals, either operand's row sums in pieces)
+    ZeroJobs zero{};
+    if (status) zero.add(status, 1);
+    zero.add(clear, clear_words);
+    // small tensors: everything in one launch
+    {
+        SmallJob J{};
+        J.zero = zero;
+        bool small = x != nullptr;
+        int count = 0, cols = 0;
+        for (int i = 0; i < 2 && small; ++i) {
+            if (!ops[i]) continue;
+            QuantOperand &op = *ops[i];
+            if (int rc = check_common(op.v, op.rows, op.cols, QBP_PER_TENSOR, QBP_ROUND_NEAREST, op.qp)) return rc;
+            SmallOperand &s = J.op[count++];
+            const int64_t n = op.rows * op.cols;
+            s = SmallOperand{op.v, (int)(n / 4), (int)op.cols, quant_out(op.q, nullptr, nullptr, nullptr), op.qp, op.col_sums, 0};
+            small = n > 0 && n <= kSmallElems && op.cols % 4 == 0 && op.cols <= kSmallMaxCols && quant_vec(op.v, op.cols, 0, s.o) &&
+                    (!op.row_sums || fuse_rowsums(op.v, n, op.cols, true, op.row_sums, s.o));
+            if (op.col_sums) s.pieces = sum_pieces(op.rows, op.cols);
+            if (op.tot && i == 0) s.o.chansum8 = reinterpret_cast<unsigned long long *>(op.tot);
+            else if (op.tot) J.zero.add(op.tot, 2 * op.cols);
+            if (s.colsum || s.o.chansum8) cols = std::max(cols, s.cols);
+        }
+        if (small) {
+            for (int i = 0; i < 2; ++i)
+                if (ops[i]) { ops[i]->row_sums_left = ops[i]->row_sums != nullptr; ops[i]->tot_left = ops[i]->tot && i == 0; ops[i]->col_sums_left = ops[i]->col_sums != nullptr; }
+            QBP_TRACE_BEGIN(st);
+            launch(operands_prep_kernel, count * kSmallCtas, kSmallThreads, (size_t)cols * sizeof(int), st, J);
+            QBP_LAUNCH_OK("operands_prep_kernel");
+            return QBP_OK;
+        }
+    }
     // The weights' column sums beside their codes: of at most 3 M elements, in blocks of at most 64 K (a launch and its reading of the
     // codes less: 3 us; 64 x 4080 -> 4080, whose 16.6 M the strips read at two thirds of the bandwidth, 158 -> 165 us).  Where they are
     // not taken, a launch for code sums follows anyway, and takes the activation's rows as well.
@@ -1049,10 +1183,6 @@ int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, s
         w->col_sums_left = S.col_sums != nullptr;
         add_rows = add_rows && w->col_sums_left;
     }
-    // (the status word, the caller's, the activation's or the weights' totals, either operand's row sums in pieces)
-    ZeroJobs zero{};
-    if (status) zero.add(status, 1);
-    zero.add(clear, clear_words);
     for (int i = 0; i < 2; ++i) {
         parts[i] = c.take<float2>(kMaxParts);
         if (!ops[i]) continue;
