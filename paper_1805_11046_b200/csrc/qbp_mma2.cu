@@ -1,8 +1,9 @@
 // The dense 8-bit product y = W x (Section 1) on CTA pairs: tcgen05.mma.cta_group::2.
 //
-// Two CTAs of a cluster (two neighbouring SMs) compute one 256 x 256 output tile: CTA r of the pair holds rows
-// [128 r, 128 r + 128) of the A tile and columns [128 r, 128 r + 128) of the B tile in its shared memory and
-// the accumulator of its 128 rows (256 columns) in its tensor memory.  One thread of the pair's first CTA (the
+// Two CTAs of a cluster (two neighbouring SMs) compute one 256 x 256 output tile (512 x 256 or narrower ones by the size of
+// the product, see launch_gemm2): CTA r of the pair holds rows [128 r, 128 r + 128) of the A tile and columns
+// [128 r, 128 r + 128) of the B tile in its shared memory and the accumulator of its 128 rows (256 columns) in its tensor
+// memory.  One thread of the pair's first CTA (the
 // leader) issues every MMA; the tensor cores of both SMs read the B halves of both CTAs.  Against the
 // single-CTA kernel this halves the B bytes each SM reads per MMA, halves the instructions and commits per
 // multiply-add, and leaves room in tensor memory for a second accumulator, so that the epilogue of a tile
@@ -29,8 +30,9 @@ constexpr uint32_t k2Smem = 225u * 1024u;     // dynamic; about 1.2 KB of static
 
 struct Mma2Params {
     CUtensorMap mapA, mapB, mapC;
-    OperandLayout a, b;              // per-CTA halves: A 128 rows, B 128 columns, 128 reduction bytes
-    uint32_t idesc;                  // M = 256, N = 256
+    OperandLayout a, b;              // per-CTA halves: A 128 rows, B bn / 2 columns, 128 reduction bytes
+    uint32_t idesc;                  // M = 256, N = bn
+    int bn;                          // columns of a pair tile: 256, or 128 or 64 (msub == 1)
     int stages, cg;                  // ring stages of one k block; stages released per commit
     int msub;                        // 256-row sub-tiles of the pair tile (2: 512 x 256, one accumulator set)
     int nbuf;                        // accumulator sets in tensor memory (2 when msub == 1)
@@ -50,7 +52,8 @@ struct Mma2Params {
 // The MMA takes its operands from the warp's few uniform registers: the loop is written for a whole converged warp
 // with an elected issuer, its MMAs unrolled with constant offsets, and what the operand layout fixes (the k step:
 // 2 sixteen-byte units inside a K-major row, 256 between the 32-row blocks of an M/N-major tile; the upper descriptor
-// word: 128-byte swizzle, 8-row groups 1024 bytes apart) is spelled as constants.
+// word: 128-byte swizzle, 8-row groups 1024 bytes apart; of an M/N-major B tile of RB bytes a row, the swizzle of RB
+// bytes and groups of 8 RB) is spelled as constants.
 struct Pair2MmaArgs {
     uint64_t *full_bar, *empty_bar, *acc_full, *acc_empty;
     uint32_t ring, stage_bytes, a_bytes, tmem, a_desc_lo, b_desc_lo, idesc;
@@ -59,22 +62,23 @@ struct Pair2MmaArgs {
     int tile0, tiles_total, tile_step;
 };
 
-template <uint32_t AK, uint32_t BK, int MSUB, bool FIRST>
+template <uint32_t AK, uint32_t BK, uint32_t RB, int MSUB, bool FIRST>
 __device__ __forceinline__ void pair_issue_stage(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc)
 {
     constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+    constexpr uint32_t b_hi = ((8u * RB) >> 4) | (1u << 14) | ((RB == 128 ? 2u : RB == 64 ? 4u : 6u) << 29);
     constexpr uint32_t a_tile16 = 128u * 128u / 16u;              // a CTA's half of one 256-row sub-tile
 #pragma unroll
     for (int i = 0; i < 4 * MSUB; ++i) {
         const int kk = i / MSUB, sub = i % MSUB;
         if (elect_one())
             mma_i8_pair(d_tmem + 256u * (uint32_t)sub, ((uint64_t)hi << 32) | (uint64_t)(a_lo + (uint32_t)sub * a_tile16 + (uint32_t)kk * AK),
-                        ((uint64_t)hi << 32) | (uint64_t)(b_lo + (uint32_t)kk * BK), idesc, (FIRST && kk == 0) ? 0u : 1u);
+                        ((uint64_t)b_hi << 32) | (uint64_t)(b_lo + (uint32_t)kk * BK), idesc, (FIRST && kk == 0) ? 0u : 1u);
     }
 }
 
 // False when a wait ran out.
-template <uint32_t AK, uint32_t BK, int MSUB>
+template <uint32_t AK, uint32_t BK, int MSUB, uint32_t RB = 128>
 __device__ __forceinline__ bool pair_mma_loop(const Pair2MmaArgs &A)
 {
     uint32_t s = 0, ph = 0, buf = 0, bph = 1;
@@ -89,8 +93,8 @@ __device__ __forceinline__ bool pair_mma_loop(const Pair2MmaArgs &A)
             tc_fence_after();
             const uint32_t a_lo = ((a_addr >> 4) & 0x3FFFu) | A.a_desc_lo;
             const uint32_t b_lo = (((a_addr + A.a_bytes) >> 4) & 0x3FFFu) | A.b_desc_lo;
-            if (it == 0) pair_issue_stage<AK, BK, MSUB, true>(d_tmem, a_lo, b_lo, A.idesc);
-            else         pair_issue_stage<AK, BK, MSUB, false>(d_tmem, a_lo, b_lo, A.idesc);
+            if (it == 0) pair_issue_stage<AK, BK, RB, MSUB, true>(d_tmem, a_lo, b_lo, A.idesc);
+            else         pair_issue_stage<AK, BK, RB, MSUB, false>(d_tmem, a_lo, b_lo, A.idesc);
             // release the group of stages this one completes, in both CTAs (the last group of a tile too: the
             // commit of acc_full below covers the same MMAs, but the producers wait on "empty")
             if (++in_group == A.cg) {
@@ -114,7 +118,7 @@ __device__ __forceinline__ Tile2 tile2_origin(const Mma2Params &P, int tile)
     const int rows_here = min(k2GroupM, P.tiles_m - g * k2GroupM);
     if (rows_here == k2GroupM) { tile_n = r / k2GroupM; tile_m = g * k2GroupM + r % k2GroupM; }
     else                       { tile_n = r / rows_here; tile_m = g * k2GroupM + r % rows_here; }
-    Tile2 t; t.m0 = tile_m * 256 * P.msub; t.n0 = tile_n * 256;
+    Tile2 t; t.m0 = tile_m * 256 * P.msub; t.n0 = tile_n * P.bn;
     return t;
 }
 
@@ -129,7 +133,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
     uint8_t *smem = smem_raw + ((1024u - (raw_addr & 1023u)) & 1023u);
     const uint32_t a_bytes = P.a.tile_bytes * (uint32_t)P.msub;
     const uint32_t stage_bytes = a_bytes + P.b.tile_bytes;                   // this CTA's halves
-    uint8_t *staging = smem + (size_t)P.stages * stage_bytes;                // 1024-aligned: stage_bytes is 32 KB
+    uint8_t *staging = smem + (size_t)P.stages * stage_bytes;                // 1024-aligned: stage_bytes is a multiple of 4 KB
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();                                 // 0: leader of the pair
     const int pair = blockIdx.x >> 1;
@@ -162,7 +166,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
             uint32_t s = 0, gph = 1, in_group = 0, group = 0;
             for (int tile = pair; tile < P.tiles_total && !timed_out; tile += P.pairs) {
                 const Tile2 o = tile2_origin(P, tile);
-                const int m_mine = o.m0 + 128 * (int)rank, n_mine = o.n0 + 128 * (int)rank;   // sub-tile s: + 256 s rows
+                const int m_mine = o.m0 + 128 * (int)rank, n_mine = o.n0 + (P.bn >> 1) * (int)rank;   // sub-tile s: + 256 s rows
                 for (int it = 0; it < P.k_iters; ++it) {
                     if (in_group == 0 && !mbar_wait(&empty_bar[group], gph)) { timed_out = true; break; }
                     if (++in_group == cg) { in_group = 0; ++group; }
@@ -198,15 +202,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
             if (P.msub == 2) {
                 if (P.a.major == 0) ok = P.b.major == 0 ? pair_mma_loop<2, 2, 2>(A) : pair_mma_loop<2, 256, 2>(A);
                 else                ok = P.b.major == 0 ? pair_mma_loop<256, 2, 2>(A) : pair_mma_loop<256, 256, 2>(A);
-            } else {
+            } else if (P.b.major == 0 || P.bn == 256) {
                 if (P.a.major == 0) ok = P.b.major == 0 ? pair_mma_loop<2, 2, 1>(A) : pair_mma_loop<2, 256, 1>(A);
                 else                ok = P.b.major == 0 ? pair_mma_loop<256, 2, 1>(A) : pair_mma_loop<256, 256, 1>(A);
+            } else if (P.bn == 128) {
+                ok = P.a.major == 0 ? pair_mma_loop<2, 128, 1, 64>(A) : pair_mma_loop<256, 128, 1, 64>(A);
+            } else {
+                ok = P.a.major == 0 ? pair_mma_loop<2, 64, 1, 32>(A) : pair_mma_loop<256, 64, 1, 32>(A);
             }
             timed_out = !ok;
         }
     } else {
         // ------------------------------------------------------- epilogue (each CTA drains its own 128 rows)
-        // msub == 1: the two groups of four warps split the column chunks (0..3, 4..7); msub == 2: one sub-tile each
+        // msub == 1: the two groups of four warps split the column chunks in halves; msub == 2: one sub-tile each
         const int ew = warp - 2, quad = warp & 3, half = ew >> 2;
         const int sub = P.msub == 2 ? half : 0;
         const int et = threadIdx.x - 64;
@@ -225,15 +233,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
             const int rterm = valid ? neg_zb * (int)P.a_sums.at(m) + k_zz : 0;
             // column terms of this tile (the previous tile's readers are done first)
             named_barrier(1, 32 * k2EpiWarps);
-            if (et < 256) s_cterm[et] = o.n0 + et < P.N ? neg_za * (int)P.b_sums.at(o.n0 + et) : 0;
+            if (et < P.bn) s_cterm[et] = o.n0 + et < P.N ? neg_za * (int)P.b_sums.at(o.n0 + et) : 0;
             named_barrier(1, 32 * k2EpiWarps);
             const int64_t ncol = P.N - o.n0;
-            const int nchunks = (int)((ncol < 256 ? ncol : 256) + 31) / 32;
+            const int nchunks = (int)((ncol < P.bn ? ncol : P.bn) + 31) / 32, per_group = P.bn >> 6;
             if (!timed_out && !mbar_wait_warp(&acc_full[buf], fph)) timed_out = true;
             if (!timed_out) {
                 tc_fence_after();
                 const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16) + buf * 256u + 256u * (uint32_t)sub;
-                const int c_begin = P.msub == 2 ? 0 : half * 4, c_end = P.msub == 2 ? nchunks : min(nchunks, half * 4 + 4);
+                const int c_begin = P.msub == 2 ? 0 : half * per_group, c_end = P.msub == 2 ? nchunks : min(nchunks, (half + 1) * per_group);
                 if (c_begin >= c_end) {
                     tc_fence_before();
                     __syncwarp();
@@ -318,25 +326,34 @@ int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const 
 {
     Mma2Params P{};
     int rc;
-    // per-CTA operand halves: 128 rows of A, 128 columns of B, 128 reduction bytes per stage
+    // Tiles.  512 x 256 pair tiles (two accumulators per CTA fill tensor memory: no second set) cut the operand bytes per
+    // multiply-add by a quarter against 256 x 256; worth it once the product is large enough to be fetch-bound.  Where tiles of
+    // 256 x 256 fit the pairs once, they and tiles of half as many columns (64 at least) as long as they do: rings and epilogues
+    // get shorter, and SMs that had none take part.  Times of a call with its sums, 256 or 512 rows by 256 -> by this rule:
+    // 4096 x 256 x 1024 15.4 -> 9.8 us, 2048 x 2048 x 2048 20.2 -> 15.3, 4096 x 1024 x 4096 30.0 -> 21.8, 1024 x 1024 x 1024
+    // 11.3 -> 9.5; the same where it changes nothing (2048 x 2560 x 1024: 16.6).
+    const auto tiles_of = [&](int64_t m, int64_t n) { return ((M + m - 1) / m) * ((N + n - 1) / n); };
+    const int pairs = sm_count() / 2;
+    P.msub = M >= 2048 && tiles_of(256, 256) > pairs ? 2 : 1;
+    P.bn = 256;
+    while (P.msub == 1 && P.bn > 64 && tiles_of(256, P.bn / 2) <= pairs) P.bn /= 2;
+    // per-CTA operand halves: 128 rows of A, bn / 2 columns of B, 128 reduction bytes per stage
+    const uint32_t half = (uint32_t)P.bn / 2;
     if (!transA) { P.a = layout_kmajor(128, 128);        rc = make_map_2d(&P.mapA, A, M, K, 128, 128); }
     else         { P.a = layout_mnmajor(128, 128, 1, 0); rc = make_map_2d(&P.mapA, A, K, M, 128, 128); }
     if (rc) return rc;
-    if (transB)  { P.b = layout_kmajor(128, 128);        rc = make_map_2d(&P.mapB, B, N, K, 128, 128); }
-    else         { P.b = layout_mnmajor(128, 128, 1, 0); rc = make_map_2d(&P.mapB, B, K, N, 128, 128); }
+    if (transB)  { P.b = layout_kmajor(half, 128);         rc = make_map_2d(&P.mapB, B, N, K, half, 128); }
+    else         { P.b = layout_mnmajor(128, half, 1, 0);  rc = make_map_2d(&P.mapB, B, K, N, 128, half); }
     if (rc) return rc;
     if (C && (rc = make_map_out_2d(&P.mapC, C, M, N))) return rc;
-    P.idesc = make_idesc(true, true, P.a.major, P.b.major, 256, 256);
+    P.idesc = make_idesc(true, true, P.a.major, P.b.major, 256, (uint32_t)P.bn);
     P.k_iters = (int)((K + 127) / 128);
-    // 512 x 256 pair tiles (two accumulators per CTA fill tensor memory: no second set) cut the operand bytes per
-    // multiply-add by a quarter against 256 x 256; worth it once the product is large enough to be fetch-bound
-    P.msub = M >= 2048 ? 2 : 1;
     P.nbuf = P.msub == 2 ? 1 : 2;
-    P.tiles_m = (int)((M + 256 * P.msub - 1) / (256 * P.msub)); P.tiles_n = (int)((N + 255) / 256);
+    P.tiles_m = (int)((M + 256 * P.msub - 1) / (256 * P.msub)); P.tiles_n = (int)((N + P.bn - 1) / P.bn);
     P.tiles_total = P.tiles_m * P.tiles_n;
     P.pairs = std::min(P.tiles_total, sm_count() / 2);
     P.d_group = make_fastdiv(k2GroupM * P.tiles_n);
-    const uint32_t stage_bytes = P.a.tile_bytes * P.msub + P.b.tile_bytes;  // 32 KB or 48 KB
+    const uint32_t stage_bytes = P.a.tile_bytes * P.msub + P.b.tile_bytes;  // 20, 24, 32 or 48 KB
     int stages = (int)((k2Smem - 1024 - k2EpiWarps * k2Slab) / stage_bytes);
     stages = std::min(stages, k2MaxStages);
     P.cg = 2;                           // sixteen (msub 2) or eight pair MMAs, 1024 cycles or more, between commits

@@ -162,6 +162,23 @@ def test_gemm_s8_pair_kernel_ragged_sampled_rows(B, M, N, K, tA, tB):
     assert np.array_equal(to_host(acc[rows]), oacc) and np.array_equal(to_host(out[rows]), oout)
 
 
+# Products that fit the SM pairs once: pair tiles of 64, 128 and 256 columns, ragged in every dimension (the last one has
+# more than 2048 rows and still takes tiles of 256).
+SMALL_PAIR_GEMMS = [(272, 304, 144), (256, 256, 1040), (2064, 1008, 144), (4368, 784, 272)]
+
+
+@pytest.mark.parametrize("M,N,K", SMALL_PAIR_GEMMS)
+@pytest.mark.parametrize("tA,tB", [(False, False), (False, True), (True, False), (True, True)])
+def test_gemm_s8_pair_kernel_narrow_tiles(B, M, N, K, tA, tB):
+    A = random_codes((K, M) if tA else (M, K), 13); Bm = random_codes((N, K) if tB else (K, N), 14)
+    za, zb, sa, sb = 23, -5, 0.25, 0.5
+    acc, out, ws = B.qbp_gemm_s8(to_dev(A), _qp(B, sa, za), to_dev(Bm), _qp(B, sb, zb), transA=tA, transB=tB, want_acc=True)
+    assert B.status_word(ws) == 0
+    oacc, oout, bad = O.gemm_s8(A, za, Bm, zb, sa, sb, transA=tA, transB=tB)
+    assert bad == 0
+    assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(out), oout)
+
+
 # ------------------------------------------- column statistics from the epilogue
 def _check_col_stats(out, stats):
     o = to_host(out).reshape(-1, out.shape[-1]).astype(np.float64)
