@@ -5,7 +5,7 @@
 // exactly in int64 in the epilogue.  The reduction runs over the M rows, so both operands are M/N-major in shared
 // memory (TMA boxes [reduction rows x columns]).
 //
-// Two CTAs of a cluster compute one 256 x 256 output tile: CTA r holds columns [128 r, 128 r + 128) of the X block
+// Two CTAs of a cluster compute one 256 x 256 output tile (or a narrower one, see launch_wgrad2): CTA r holds columns [128 r, 128 r + 128) of the X block
 // (= output rows) and columns [128 r, 128 r + 128) of both limb blocks, and the accumulators of its 128 output rows
 // (256 columns of the high product, 256 of the low one: all 512 columns of its tensor memory).  One thread of the
 // leader issues every MMA; against the single-CTA kernel (256 x 128 tiles) each SM fetches a third fewer operand
@@ -21,23 +21,27 @@
 #include "qbp_pair.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace qbp {
 
 constexpr int kW2Threads = 320;
 constexpr int kW2EpiWarps = 8;
-constexpr int kW2Stages = 4;                    // of 48 KB: 128 reduction rows x (128 X + 128 hi + 128 lo columns)
+constexpr int kW2MaxStages = 8;                 // of 24, 32 or 48 KB: 128 reduction rows x (128 X + bn / 2 hi + bn / 2 lo columns)
+constexpr uint32_t kW2Ring = 192u * 1024u;
 constexpr int kW2Cg = 2;                        // stages released per commit
 constexpr int kW2GroupM = 8;
 constexpr uint32_t kW2Slab = 32 * 128;
-constexpr uint32_t kW2StageBytes = 3u * 128u * 128u;
-constexpr uint32_t kW2Smem = 1024u + kW2Stages * kW2StageBytes + kW2EpiWarps * kW2Slab;
+constexpr uint32_t kW2XBytes = 128u * 128u;
+constexpr uint32_t kW2Smem = 1024u + kW2Ring + kW2EpiWarps * kW2Slab;
 
 struct Wgrad2Params {
     CUtensorMap mapX, mapHi, mapLo, mapC;
-    uint32_t desc_lo;                // descriptor bits 16..31 of the M/N-major 128 x 128 tiles
-    uint32_t idesc_hi;               // s8 x s8, M = 256, N = 256, both operands M/N-major
+    uint32_t x_desc_lo, g_desc_lo;   // descriptor bits 16..31 of the M/N-major tiles of 128 and of bn / 2 columns
+    uint32_t idesc_hi;               // s8 x s8, M = 256, N = bn, both operands M/N-major
     uint32_t lo_flip;                // the low limb's descriptor = idesc_hi ^ lo_flip: the B sign bit for unsigned low bytes, 0 for lo - 128
+    int bn, stages;                  // columns of a pair tile (256, 128 or 64); ring stages
+    uint32_t stage_bytes;
     int k_iters;                     // reduction steps of 128 rows
     int tiles_m, tiles_n, tiles_total, pairs;
     FastDiv d_group;
@@ -53,18 +57,20 @@ struct Wgrad2Params {
 
 // The eight pair MMAs of a stage (128 reduction rows = four k steps per limb), the limb outermost: switching
 // between the two instruction descriptors stalls the MMA pipe.  Offsets in 16-byte units: 256 per k step of an
-// M/N-major 128-byte-row tile, 1024 per 128 x 128 tile.
-template <bool FIRST>
+// M/N-major 128-byte-row tile, 2 RB of one of RB columns (bn / 2) of a limb, 8 RB per limb tile; the upper descriptor word is the
+// swizzle of that many bytes and groups of eight rows.
+template <uint32_t RB, bool FIRST>
 __device__ __forceinline__ void w2_issue_stage(uint32_t tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc_hi, uint32_t lo_flip)
 {
     constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
+    constexpr uint32_t g_hi = ((8u * RB) >> 4) | (1u << 14) | ((RB == 128 ? 2u : RB == 64 ? 4u : 6u) << 29);
     const uint32_t idesc_lo = idesc_hi ^ lo_flip;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int limb = i >> 2, kk = i & 3;
         if (elect_one())
             mma_i8_pair(tmem + 256u * (uint32_t)limb, ((uint64_t)hi << 32) | (uint64_t)(a_lo + (uint32_t)kk * 256u),
-                   ((uint64_t)hi << 32) | (uint64_t)(b_lo + (uint32_t)limb * 1024u + (uint32_t)kk * 256u),
+                   ((uint64_t)g_hi << 32) | (uint64_t)(b_lo + (uint32_t)limb * (8u * RB) + (uint32_t)kk * (2u * RB)),
                    limb ? idesc_lo : idesc_hi, (FIRST && kk == 0) ? 0u : 1u);
     }
 }
@@ -77,19 +83,19 @@ __device__ __forceinline__ W2Tile w2_tile(const Wgrad2Params &P, int tile)
     const int rows_here = min(kW2GroupM, P.tiles_m - g * kW2GroupM);
     if (rows_here == kW2GroupM) { tile_n = r / kW2GroupM; tile_m = g * kW2GroupM + r % kW2GroupM; }
     else                        { tile_n = r / rows_here; tile_m = g * kW2GroupM + r % rows_here; }
-    W2Tile t; t.k0 = tile_m * 256; t.n0 = tile_n * 256;
+    W2Tile t; t.k0 = tile_m * 256; t.n0 = tile_n * P.bn;
     return t;
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_wgrad2_kernel(const __grid_constant__ Wgrad2Params P)
 {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t full_bar[kW2Stages], empty_bar[kW2Stages], acc_full, acc_empty;
+    __shared__ uint64_t full_bar[kW2MaxStages], empty_bar[kW2MaxStages], acc_full, acc_empty;
     __shared__ uint32_t tmem_slot;
 
     const uint32_t raw_addr = smem_u32(smem_raw);
     uint8_t *smem = smem_raw + ((1024u - (raw_addr & 1023u)) & 1023u);
-    uint8_t *staging = smem + (size_t)kW2Stages * kW2StageBytes;
+    uint8_t *staging = smem + kW2Ring;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const int pair = blockIdx.x >> 1;
@@ -97,7 +103,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
     if (threadIdx.x == 0) {
         // "full": the leader's arrive + the bytes of both CTAs; "empty": one multicast commit per stage group;
         // "acc_full": one multicast commit per tile; "acc_empty" (the leader's is waited on): 8 warps of each CTA
-        for (int s = 0; s < kW2Stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
+        for (int s = 0; s < kW2MaxStages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
         mbar_init(&acc_full, 1); mbar_init(&acc_empty, 2 * kW2EpiWarps);
         mbar_fence_init();
         tma_prefetch_desc(&P.mapX); tma_prefetch_desc(&P.mapHi); tma_prefetch_desc(&P.mapLo);
@@ -120,55 +126,61 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
             uint32_t s = 0, gph = 1, in_group = 0, group = 0;
             for (int tile = pair; tile < P.tiles_total && !timed_out; tile += P.pairs) {
                 const W2Tile o = w2_tile(P, tile);
-                const int k_mine = o.k0 + 128 * (int)rank, n_mine = o.n0 + 128 * (int)rank;
+                const int k_mine = o.k0 + 128 * (int)rank, n_mine = o.n0 + (P.bn >> 1) * (int)rank;
                 for (int it = 0; it < P.k_iters; ++it) {
                     if (in_group == 0 && !mbar_wait(&empty_bar[group], gph)) { timed_out = true; break; }
                     if (++in_group == (uint32_t)kW2Cg) { in_group = 0; ++group; }
-                    uint8_t *sa = smem + (size_t)s * kW2StageBytes;
+                    uint8_t *sa = smem + (size_t)s * P.stage_bytes;
                     const uint32_t bar = map_to_cta(&full_bar[s], 0);
-                    if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * kW2StageBytes);
+                    if (rank == 0) mbar_expect_tx(&full_bar[s], 2u * P.stage_bytes);
                     const int m0 = it * 128;
                     if (!waited) { if (!P.beside) pdl_wait(); waited = true; }
                     tma_load_2d_pair(sa, &P.mapX, bar, k_mine, m0);
-                    tma_load_2d_pair(sa + 16384, &P.mapHi, bar, n_mine, m0);
-                    tma_load_2d_pair(sa + 32768, &P.mapLo, bar, n_mine, m0);
-                    if (++s == (uint32_t)kW2Stages) { s = 0; gph ^= 1u; group = 0; }
+                    tma_load_2d_pair(sa + kW2XBytes, &P.mapHi, bar, n_mine, m0);
+                    tma_load_2d_pair(sa + kW2XBytes + 64 * P.bn, &P.mapLo, bar, n_mine, m0);
+                    if (++s == (uint32_t)P.stages) { s = 0; gph ^= 1u; group = 0; }
                 }
             }
         }
     } else if (warp == 1) {
         if (rank == 0) {
             // ---------------------------------------------------- MMA issuer (leader CTA only): the whole warp in step
-            uint32_t s = 0, ph = 0, in_group = 0, group = 0, eph = 1;
-            const uint32_t ring = smem_u32(smem);
-            uint32_t a_addr = ring;
             // (a barrier's wait is bounded: its clock starts once the producer's copies can)
             if (!P.beside) pdl_wait();
-            for (int tile = pair; tile < P.tiles_total && !timed_out; tile += P.pairs) {
-                if (!mbar_wait_uniform(&acc_empty, eph)) { timed_out = true; break; }
-                eph ^= 1u;
-                tc_fence_after();
-                for (int it = 0; it < P.k_iters; ++it) {
-                    if (!mbar_wait_uniform(&full_bar[s], ph)) { timed_out = true; break; }
+            const auto issue = [&](auto columns) {
+                constexpr uint32_t RB = decltype(columns)::value;
+                uint32_t s = 0, ph = 0, in_group = 0, group = 0, eph = 1;
+                const uint32_t ring = smem_u32(smem);
+                uint32_t a_addr = ring;
+                for (int tile = pair; tile < P.tiles_total; tile += P.pairs) {
+                    if (!mbar_wait_uniform(&acc_empty, eph)) return false;
+                    eph ^= 1u;
                     tc_fence_after();
-                    const uint32_t a_lo = ((a_addr >> 4) & 0x3FFFu) | P.desc_lo;
-                    const uint32_t b_lo = (((a_addr + 16384u) >> 4) & 0x3FFFu) | P.desc_lo;
-                    if (it == 0) w2_issue_stage<true>(tmem_base, a_lo, b_lo, P.idesc_hi, P.lo_flip);
-                    else         w2_issue_stage<false>(tmem_base, a_lo, b_lo, P.idesc_hi, P.lo_flip);
-                    if (++in_group == (uint32_t)kW2Cg) {
-                        if (elect_one()) mma_commit_pair(&empty_bar[group]);
-                        in_group = 0; ++group;
+                    for (int it = 0; it < P.k_iters; ++it) {
+                        if (!mbar_wait_uniform(&full_bar[s], ph)) return false;
+                        tc_fence_after();
+                        const uint32_t a_lo = ((a_addr >> 4) & 0x3FFFu) | P.x_desc_lo;
+                        const uint32_t b_lo = (((a_addr + kW2XBytes) >> 4) & 0x3FFFu) | P.g_desc_lo;
+                        if (it == 0) w2_issue_stage<RB, true>(tmem_base, a_lo, b_lo, P.idesc_hi, P.lo_flip);
+                        else         w2_issue_stage<RB, false>(tmem_base, a_lo, b_lo, P.idesc_hi, P.lo_flip);
+                        if (++in_group == (uint32_t)kW2Cg) {
+                            if (elect_one()) mma_commit_pair(&empty_bar[group]);
+                            in_group = 0; ++group;
+                        }
+                        a_addr += P.stage_bytes;
+                        if (++s == (uint32_t)P.stages) { s = 0; ph ^= 1u; group = 0; a_addr = ring; }
                     }
-                    a_addr += kW2StageBytes;
-                    if (++s == (uint32_t)kW2Stages) { s = 0; ph ^= 1u; group = 0; a_addr = ring; }
+                    if (elect_one()) mma_commit_pair(&acc_full);
                 }
-                if (!timed_out && elect_one()) mma_commit_pair(&acc_full);
-            }
+                return true;
+            };
+            timed_out = !(P.bn == 256 ? issue(std::integral_constant<uint32_t, 128>{})
+                          : P.bn == 128 ? issue(std::integral_constant<uint32_t, 64>{}) : issue(std::integral_constant<uint32_t, 32>{}));
         }
     } else {
         // ------------------------------------------------------- epilogue (each CTA drains its own 128 output rows)
-        // the two groups of four warps split the eight column chunks of 32
-        const int ew = warp - 2, quad = warp & 3, half = ew >> 2;
+        // the two groups of four warps split the column chunks of 32
+        const int ew = warp - 2, quad = warp & 3, half = ew >> 2, per_group = P.bn >> 6;
         const int row = quad * 32 + lane;
         uint8_t *slab = staging + (size_t)ew * kW2Slab;
         pdl_wait();
@@ -186,28 +198,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
             // lane l takes the column terms of column l of this warp's four chunks, while the MMAs run (the sums come in pieces:
             // two pieces of all eight sums are in flight at a time -- one sum after the other took up to 64 us a tile)
             long long ct[4] = {0, 0, 0, 0};
-            const int32_t *ph = P.shi.p + o.n0 + half * 128 + lane, *pl = P.slo.p + o.n0 + half * 128 + lane;
+            const int32_t *ph = P.shi.p + o.n0 + half * per_group * 32 + lane, *pl = P.slo.p + o.n0 + half * per_group * 32 + lane;
             if (P.tot_g) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    if ((half * 4 + i) * 32 + lane < ncol) ct[i] = P.tot_g[o.n0 + (half * 4 + i) * 32 + lane] - P.zg_shift * P.M;
+                    if (i < per_group && (half * per_group + i) * 32 + lane < ncol) ct[i] = P.tot_g[o.n0 + (half * per_group + i) * 32 + lane] - P.zg_shift * P.M;
             } else
 #pragma unroll 2
             for (int k = 0; k < P.shi.pieces; ++k) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    if ((half * 4 + i) * 32 + lane < ncol) ct[i] += 256 * (long long)load_after_wait(ph + 32 * i) + load_after_wait(pl + 32 * i);
+                    if (i < per_group && (half * per_group + i) * 32 + lane < ncol) ct[i] += 256 * (long long)load_after_wait(ph + 32 * i) + load_after_wait(pl + 32 * i);
                 ph += P.shi.stride; pl += P.slo.stride;
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) ct[i] *= -zx;
-            const int nchunks = (int)((ncol < 256 ? ncol : 256) + 31) / 32;
+            const int nchunks = (int)((ncol < P.bn ? ncol : P.bn) + 31) / 32;
             if (!timed_out && !mbar_wait_warp(&acc_full, fph)) timed_out = true;
             fph ^= 1u;
             if (!timed_out) {
                 tc_fence_after();
                 const uint32_t t_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
-                const int c_begin = half * 4, c_end = min(nchunks, half * 4 + 4);
+                const int c_begin = half * per_group, c_end = min(nchunks, (half + 1) * per_group);
                 if (c_begin >= c_end) {
                     tc_fence_before();
                     __syncwarp();
@@ -299,18 +311,27 @@ int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qp
 {
     Wgrad2Params P{};
     int rc;
-    // per-CTA operand parts: 128 reduction rows x 128 columns, M/N-major
-    const OperandLayout L = layout_mnmajor(128, 128, 1, 0);
-    if ((rc = make_map_2d(&P.mapX, x, M, K, 128, 128))) return rc;
-    if ((rc = make_map_2d(&P.mapHi, g_hi, M, N, 128, 128))) return rc;
-    if ((rc = make_map_2d(&P.mapLo, g_lo, M, N, 128, 128))) return rc;
-    if (dW && (rc = make_map_out_2d(&P.mapC, dW, K, N))) return rc;
-    P.desc_lo = L.desc_lo;
-    P.idesc_hi = make_idesc(true, true, 1, 1, 256, 256);
-    P.lo_flip = lo_signed ? 0u : (1u << 10);
-    P.k_iters = (int)((M + 127) / 128);
-    P.tiles_m = (int)((K + 255) / 256); P.tiles_n = (int)((N + 255) / 256);
+    // where tiles of 256 columns fit the pairs once, tiles of half as many (64 at least) as long as they do: rings and epilogues get
+    // shorter, and SMs that had none take part.  Call with its sums, 256 columns -> by this rule: 1024 rows for 2048 x 1008 18.3 ->
+    // 15.6 us, 4096 for 1024 x 1024 31.7 -> 24.1, 16384 for 256 x 512 84.9 -> 57.0
+    const auto tiles_n_of = [&](int bn) { return (N + bn - 1) / bn; };
+    P.tiles_m = (int)((K + 255) / 256);
+    P.bn = 256;
+    while (P.bn > 64 && P.tiles_m * tiles_n_of(P.bn / 2) <= sm_count() / 2) P.bn /= 2;
+    P.tiles_n = (int)tiles_n_of(P.bn);
     P.tiles_total = P.tiles_m * P.tiles_n;
+    // per-CTA operand parts: 128 reduction rows x 128 columns of X, x bn / 2 of each limb, M/N-major
+    const uint32_t half = (uint32_t)P.bn / 2;
+    if ((rc = make_map_2d(&P.mapX, x, M, K, 128, 128))) return rc;
+    if ((rc = make_map_2d(&P.mapHi, g_hi, M, N, 128, half))) return rc;
+    if ((rc = make_map_2d(&P.mapLo, g_lo, M, N, 128, half))) return rc;
+    if (dW && (rc = make_map_out_2d(&P.mapC, dW, K, N))) return rc;
+    P.x_desc_lo = layout_mnmajor(128, 128, 1, 0).desc_lo; P.g_desc_lo = layout_mnmajor(128, half, 1, 0).desc_lo;
+    P.idesc_hi = make_idesc(true, true, 1, 1, 256, (uint32_t)P.bn);
+    P.lo_flip = lo_signed ? 0u : (1u << 10);
+    P.stage_bytes = kW2XBytes + 2u * 128u * half;
+    P.stages = (int)(kW2Ring / P.stage_bytes);            // 4, 6 or 8: a multiple of kW2Cg
+    P.k_iters = (int)((M + 127) / 128);
     P.pairs = std::min(P.tiles_total, sm_count() / 2);
     P.d_group = make_fastdiv(kW2GroupM * P.tiles_n);
     P.M = M; P.N = N; P.K = K;

@@ -295,6 +295,19 @@ def test_wgrad_plain(B, M, N, K):
     assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
 
 
+# The CTA-pair kernel where it fits the SM pairs once: tiles of 64, 128 and 256 columns, ragged in every dimension, fewer
+# reduction steps than the ring has stages and more.
+@pytest.mark.parametrize("M,N,K", [(528, 272, 304), (2064, 256, 256), (560, 1008, 2064), (1536, 784, 4368)])
+def test_wgrad_plain_pair_kernel_narrow_tiles(B, M, N, K):
+    X = random_codes((M, K), 7); G = _g16((M, N), 8)
+    hi, lo = O.limb_split(G)
+    zx, zg = 11, -77
+    acc, dW, ws = B.qbp_wgrad_s16(to_dev(X), _qp(B, 0.5, zx), to_dev(hi), to_dev(lo), _qp(B, 0.25, zg), want_acc=True)
+    oacc, oout = O.gemm_s16s8(X, zx, G, zg, 0.5, 0.25)
+    assert B.status_word(ws) == 0
+    assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
+
+
 def test_wgrad_long_reduction_extreme_codes(B):
     """131072 rows of extreme codes: each CTA's int32 chunk stays in range, the int64 total is exact."""
     M, N, K = 131072, 32, 32
