@@ -2,8 +2,8 @@
 //   y = W x and g_{l-1} = g_l W^T (Section 1; Eq. (grad_layer)) for linear
 //   layers (GEMM) and for convolutions (implicit GEMM over the filter taps).
 //
-// This file: the persistent single-CTA kernel (convolutions, narrow GEMMs) and the entry points; the dense GEMM of
-// at least one 256 x 256 tile runs on CTA pairs (qbp_mma2.cu).  One CTA per SM walks output tiles of 128 (or 2 x 128)
+// This file: the persistent single-CTA kernel (convolutions, small GEMMs) and the entry points; dense GEMMs of at least
+// one 256 x 256 tile and deep ones run on CTA pairs (qbp_mma2.cu).  One CTA per SM walks output tiles of 128 (or 2 x 128)
 // rows x BN columns.  Warp 0 drives TMA (cp.async.bulk.tensor into 128B/64B/32B-swizzled shared-memory stages),
 // warp 1 issues tcgen05.mma kind::i8 with int32 accumulators in tensor memory (the whole warp runs the loop, an
 // elected lane issues: see issue_stage), up to twelve epilogue warps read accumulators back (tcgen05.ld), apply the
@@ -1266,7 +1266,7 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
     if ((rc = launch_code_sums(jobs, njobs, st, zero, &own))) return rc;
     beside = njobs ? own : beside && !zero.count;         // (a tail's launch for its parameters comes in between)
 
-    // large products run on CTA pairs (256 x 256 tiles across two SMs); the column statistics are the
+    // large and deep products run on CTA pairs (tiles across two SMs); the column statistics are the
     // single-CTA kernel's (at most 256 columns: narrow either way)
     if (gemm2_eligible(M, N, K) && !stats && !has_tail)
         return launch_gemm2(transA, transB, M, N, K, A, qa, B, qb, acc_out, C, asum, bsum, status, beside, st);

@@ -313,11 +313,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
     if (warp == 1) { __syncwarp(); tmem_dealloc_pair(tmem_base, 512); }
 }
 
-// Whether the pair kernel takes this product: anything with at least one whole pair tile's worth of rows and columns
-// (it is the faster kernel from 1024^3 up; the single-CTA kernel keeps the narrow shapes).
+// Whether the pair kernel takes this product: anything of at least a whole 256 x 256 tile, and every reduction of 1024 and
+// more but for the narrowest outputs, where its deeper ring counts for more than the rows and columns of a tile that lie
+// outside (call with its sums, single-CTA -> pair kernel: 8192 x 128 x 8192 45.4 -> 34.0 us, 64 x 512 x 4096 21.7 -> 16.1,
+// 16 x 1024 x 1024 9.0 -> 8.5, 1024 x 48 x 2048 with A transposed 15.0 -> 16.0).  The short ones stay with the single-CTA kernel
+// (256 x 128 x 256: 7.4 against 8.0, 8192 x 208 x 128: 8.4 against 8.8).
 bool gemm2_eligible(int64_t M, int64_t N, int64_t K)
 {
-    return M >= 256 && N >= 256 && K >= 128;
+    return (M >= 256 && N >= 256 && K >= 128) || (N >= 64 && K >= 1024);
 }
 
 int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,

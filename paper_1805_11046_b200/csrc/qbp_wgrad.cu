@@ -965,7 +965,7 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
     }
     int64_t *part = P.direct ? nullptr : w.take<int64_t>((size_t)pl.grid * (size_t)P.part_stride);
 
-    // large plain products run on CTA pairs (256 x 256 tiles across two SMs, the whole reduction in one pair)
+    // most plain products run on CTA pairs (tiles across two SMs, the whole reduction in one pair)
     const bool pair_kernel = !d && wgrad2_eligible(M, N, K);
     // code sums for the zero-point terms: of everything, or (the kernels that wrote the codes left their per-channel totals,
     // or the product takes the gradient's itself: a row of ones in its spare chunk) of the images' edges only

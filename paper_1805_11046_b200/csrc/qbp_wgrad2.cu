@@ -298,11 +298,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
     }
 }
 
-// Whether the pair kernel takes this plain product: whole pair tiles in both output directions, a reduction one
-// pair can hold in int32 chunks, 16-byte aligned rows.
+// Whether the pair kernel takes this plain product: a reduction that one pair can hold in int32, and one of
+//   - fewer than 512 rows: large outputs (64 rows for 2048 x 2048: 15.7 us with the single-CTA kernel, 13.3 with this one; 384 for
+//     256 x 256: 9.2 against 9.6);
+//   - more: where the longer walk of a pair over all rows, about 2.9 us per 1000, costs less than the single-CTA kernel's
+//     partial sums, about 1 us per 10000 outputs (8192 rows for 4096 x 128: 68.9 us -> 39.6, 2048 for 1024 x 208: 35.2 -> 16.3,
+//     512 for 128 x 128: 9.1 against 9.4, 8192 for 128 x 128: 20.5 against 31.9, 65536 for 256 x 256: 49.6 against 228).
 bool wgrad2_eligible(int64_t M, int64_t N, int64_t K)
 {
-    return M >= 512 && M <= 65536 && N >= 256 && K >= 256;
+    if (M > 65536 || N < 64 || K < 64) return false;
+    return M < 512 ? N * K >= (1 << 20) : N * K >= (1 << 15) && 29 * M <= 30000 + N * K;
 }
 
 int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qparams *qx, const int8_t *g_hi,

@@ -162,9 +162,9 @@ def test_gemm_s8_pair_kernel_ragged_sampled_rows(B, M, N, K, tA, tB):
     assert np.array_equal(to_host(acc[rows]), oacc) and np.array_equal(to_host(out[rows]), oout)
 
 
-# Products that fit the SM pairs once: pair tiles of 64, 128 and 256 columns, ragged in every dimension (the last one has
-# more than 2048 rows and still takes tiles of 256).
-SMALL_PAIR_GEMMS = [(272, 304, 144), (256, 256, 1040), (2064, 1008, 144), (4368, 784, 272)]
+# Products that fit the SM pairs once: pair tiles of 64, 128 and 256 columns, ragged in every dimension (the fourth has
+# more than 2048 rows and still takes tiles of 256), and deep ones smaller than a tile.
+SMALL_PAIR_GEMMS = [(272, 304, 144), (256, 256, 1040), (2064, 1008, 144), (4368, 784, 272), (16, 64, 1024), (144, 208, 1040)]
 
 
 @pytest.mark.parametrize("M,N,K", SMALL_PAIR_GEMMS)
@@ -296,8 +296,9 @@ def test_wgrad_plain(B, M, N, K):
 
 
 # The CTA-pair kernel where it fits the SM pairs once: tiles of 64, 128 and 256 columns, ragged in every dimension, fewer
-# reduction steps than the ring has stages and more.
-@pytest.mark.parametrize("M,N,K", [(528, 272, 304), (2064, 256, 256), (560, 1008, 2064), (1536, 784, 4368)])
+# reduction steps than the ring has stages and more; outputs smaller than a tile, the fewest rows; the last is just too deep for it.
+@pytest.mark.parametrize("M,N,K", [(528, 272, 304), (2064, 256, 256), (560, 1008, 2064), (1536, 784, 4368), (1040, 208, 160),
+                                   (512, 64, 528), (16, 1024, 1024), (3312, 256, 256)])
 def test_wgrad_plain_pair_kernel_narrow_tiles(B, M, N, K):
     X = random_codes((M, K), 7); G = _g16((M, N), 8)
     hi, lo = O.limb_split(G)
