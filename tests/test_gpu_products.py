@@ -141,7 +141,7 @@ def test_wgrad_dense_sweep_noncube_sampled_columns(B, M, N, K):
 
 
 # Shapes the CTA-pair kernel takes (at least eight rounds of 256 x 256 tiles over the SM pairs) with ragged edges in
-# every dimension: 512 x 256 pair tiles (M >= 2048) and 256 x 256 pair tiles (short M, wide N).
+# every dimension: 512 x 256 pair tiles, several rounds of them.
 PAIR_GEMMS = [(8208, 8464, 208), (1104, 38000, 144), (2048, 19216, 400)]
 
 
@@ -163,8 +163,9 @@ def test_gemm_s8_pair_kernel_ragged_sampled_rows(B, M, N, K, tA, tB):
 
 
 # Products that fit the SM pairs once: pair tiles of 64, 128 and 256 columns, ragged in every dimension (the fourth has
-# more than 2048 rows and still takes tiles of 256), and deep ones smaller than a tile.
-SMALL_PAIR_GEMMS = [(272, 304, 144), (256, 256, 1040), (2064, 1008, 144), (4368, 784, 272), (16, 64, 1024), (144, 208, 1040)]
+# more than 2048 rows and still takes tiles of 256), and deep ones smaller than a tile; then two rounds of 256 x 256
+# tiles of more than 2048 rows, and one of 512 x 256 tiles of fewer.
+SMALL_PAIR_GEMMS = [(272, 304, 144), (256, 256, 1040), (2064, 1008, 144), (4368, 784, 272), (16, 64, 1024), (144, 208, 1040), (2320, 4112, 144), (592, 8208, 144)]
 
 
 @pytest.mark.parametrize("M,N,K", SMALL_PAIR_GEMMS)
