@@ -820,48 +820,55 @@ __global__ void __launch_bounds__(kScanThreads) bn_bwd_apply_kernel(const float 
 }
 
 // ------------------------------------------------------------- few rows
-// With few rows (a linear layer's minibatch, a late stage's last positions) a block takes 16 channels whole: statistics and what
-// follows from them in one launch, where the passes above need a launch for the partials and one to combine them -- 2 to 4 us
+// With few rows (a linear layer's minibatch, a late stage's last positions) a block takes CH = 16 channels whole: statistics and
+// what follows from them in one launch, where the passes above need a launch for the partials and one to combine them -- 2 to 4 us
 // each, which is what such a tensor costs.  Bound by latency: 512 threads, each row's 64 bytes by four of them, four rows in
 // flight.  Up to kFewRows rows (16 per thread); beyond, one block per 16 channels walks too long (at 7220 x 160 the
-// walk alone would take 17 us, the three launches take 12).
-constexpr int kFewThreads = 512, kFewRows = 2048, kFewHigh = kFewThreads / 4;
+// walk alone would take 17 us, the three launches take 12).  Eight channels (a sector of 32 bytes a row) where a
+// block of 16 would give its threads more than one row and the blocks, code sums included, still fit the SMs once: half the walk
+// and half the conversions per SM (forward 1024 x 1008 6.5 -> 5.1 us, 2048 x 1024 8.4 -> 6.7; backward 640 x 768 6.6 -> 6.1; with
+// code sums beyond the SMs the 1024 x 1008 backward would go from 9.2 to 10.6).
+constexpr int kFewThreads = 512, kFewRows = 2048;
+template <int CH> constexpr int kFewHigh = kFewThreads / (CH / 4);        // rows taken at a time
+static bool few_narrow(int64_t n, int64_t C, int beside) { return n > kFewHigh<16> && (C + 7) / 8 + beside <= sm_count(); }
 static bool few_rows(int64_t n, int64_t C) { return n <= kFewRows && C % 4 == 0; }
 
-// Sum (fp64), min and max over a block's rows, per channel: the eight lanes of a warp that hold the same four channels by
-// shuffles (each step halves the channels a lane still carries: four shuffles per quantity instead of twelve), then the warps in
+// Sum (fp64), min and max over a block's rows, per channel: the 128 / CH lanes of a warp that hold the same four channels by
+// shuffles (the first two steps halve the channels a lane still carries: four shuffles per quantity instead of twelve), then the warps in
 // shared memory, one thread per quantity and channel (all threads adding up all warps took 6 us of a 64 x 64 tensor's backward).
 // Every thread can then read its channels' results from the table: sums first, then (min, max) pairs.
-template <int NS, int NM> struct FewTable { double sum[NS][16]; float lo[NM][16], hi[NM][16]; };
-template <int NS, int NM>      // sums; (min, max) pairs
-__device__ __forceinline__ const FewTable<NS, NM> &few_reduce(double (&sum)[NS][4], float (&lo)[NM][4], float (&hi)[NM][4])
+template <int CH, int NS, int NM> struct FewTable { double sum[NS][CH]; float lo[NM][CH], hi[NM][CH]; };
+template <int CH, int NS, int NM>      // channels; sums; (min, max) pairs
+__device__ __forceinline__ const FewTable<CH, NS, NM> &few_reduce(double (&sum)[NS][4], float (&lo)[NM][4], float (&hi)[NM][4])
 {
-    constexpr int kWarps = kFewThreads / 32;
-    __shared__ double s_sum[NS][kWarps][16];
-    __shared__ float s_lo[NM][kWarps][16], s_hi[NM][kWarps][16];
-    __shared__ FewTable<NS, NM> t;
-    static_assert((NS + 2 * NM) * 16 <= kFewThreads, "a thread per quantity and channel");
+    constexpr int kWarps = kFewThreads / 32, kQuads = CH / 4;
+    __shared__ double s_sum[NS][kWarps][CH];
+    __shared__ float s_lo[NM][kWarps][CH], s_hi[NM][kWarps][CH];
+    __shared__ FewTable<CH, NS, NM> t;
+    static_assert((NS + 2 * NM) * CH <= kFewThreads, "a thread per quantity and channel");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool b2 = lane & 4, b3 = lane & 8;
-    auto reduce = [&](auto (&v)[4], auto op) {             // of channel 2 * b2 + b3 over the lanes
-        auto r0 = op(b2 ? v[2] : v[0], __shfl_xor_sync(0xffffffffu, b2 ? v[0] : v[2], 4));
-        auto r1 = op(b2 ? v[3] : v[1], __shfl_xor_sync(0xffffffffu, b2 ? v[1] : v[3], 4));
-        auto q = op(b3 ? r1 : r0, __shfl_xor_sync(0xffffffffu, b3 ? r0 : r1, 8));
-        return op(q, __shfl_xor_sync(0xffffffffu, q, 16));
+    const bool ba = lane & kQuads, bb = lane & (2 * kQuads);
+    auto reduce = [&](auto (&v)[4], auto op) {             // of channel 2 * ba + bb over the lanes
+        auto r0 = op(ba ? v[2] : v[0], __shfl_xor_sync(0xffffffffu, ba ? v[0] : v[2], kQuads));
+        auto r1 = op(ba ? v[3] : v[1], __shfl_xor_sync(0xffffffffu, ba ? v[1] : v[3], kQuads));
+        auto q = op(bb ? r1 : r0, __shfl_xor_sync(0xffffffffu, bb ? r0 : r1, 2 * kQuads));
+#pragma unroll
+        for (int m = 4 * kQuads; m < 32; m *= 2) q = op(q, __shfl_xor_sync(0xffffffffu, q, m));
+        return q;
     };
     auto add = [](double a, double b) { return a + b; };
     auto mn = [](float a, float b) { return fminf(a, b); };
     auto mx = [](float a, float b) { return fmaxf(a, b); };
-    const int ch = (lane & 3) * 4 + (b2 ? 2 : 0) + (b3 ? 1 : 0);
+    const int ch = (lane & (kQuads - 1)) * 4 + (ba ? 2 : 0) + (bb ? 1 : 0);
 #pragma unroll
-    for (int k = 0; k < NS; ++k) { const double r = reduce(sum[k], add); if (lane < 16) s_sum[k][warp][ch] = r; }
+    for (int k = 0; k < NS; ++k) { const double r = reduce(sum[k], add); if (lane < CH) s_sum[k][warp][ch] = r; }
 #pragma unroll
     for (int k = 0; k < NM; ++k) {
         const float l = reduce(lo[k], mn), h = reduce(hi[k], mx);
-        if (lane < 16) { s_lo[k][warp][ch] = l; s_hi[k][warp][ch] = h; }
+        if (lane < CH) { s_lo[k][warp][ch] = l; s_hi[k][warp][ch] = h; }
     }
     __syncthreads();
-    const int q = threadIdx.x >> 4, c = threadIdx.x & 15;
+    const int q = threadIdx.x / CH, c = threadIdx.x % CH;
     if (q < NS) {
         double r = 0.0;
 #pragma unroll
@@ -883,18 +890,19 @@ __device__ __forceinline__ const FewTable<NS, NM> &few_reduce(double (&sum)[NS][
 }
 
 // Forward: the rows wait in registers between the statistics and the normalisation (ROWS per thread, a power of two).
-template <int ROWS>
+template <int CH, int ROWS>
 __global__ void __launch_bounds__(kFewThreads) bn_fwd_few_kernel(const float *__restrict__ x, int rows, int C, const float *__restrict__ gamma,
                                                                  const float *__restrict__ beta, int relu, float Cn, float *__restrict__ y,
                                                                  float *__restrict__ mean, float *__restrict__ vmin, float *__restrict__ vmax)
 {
     pdl_wait();
-    const int col = (int)blockIdx.x * 16 + (threadIdx.x & 3) * 4, ty = threadIdx.x >> 2;
+    constexpr int kQuads = CH / 4;
+    const int col = (int)blockIdx.x * CH + (threadIdx.x % kQuads) * 4, ty = threadIdx.x / kQuads;
     const bool active = col < C;
     float4 v[ROWS];
 #pragma unroll
     for (int u = 0; u < ROWS; ++u) {
-        const int r = ty + u * kFewHigh;
+        const int r = ty + u * kFewHigh<CH>;
         if (active && r < rows) v[u] = __ldg(reinterpret_cast<const float4 *>(x + (int64_t)r * C + col));
     }
     double sum[1][4];
@@ -903,14 +911,14 @@ __global__ void __launch_bounds__(kFewThreads) bn_fwd_few_kernel(const float *__
     for (int e = 0; e < 4; ++e) { sum[0][e] = 0.0; lo[0][e] = INFINITY; hi[0][e] = -INFINITY; }
 #pragma unroll
     for (int u = 0; u < ROWS; ++u)
-        if (active && ty + u * kFewHigh < rows) {
+        if (active && ty + u * kFewHigh<CH> < rows) {
             const float t[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) { sum[0][e] += (double)t[e]; lo[0][e] = fminf(lo[0][e], t[e]); hi[0][e] = fmaxf(hi[0][e], t[e]); }
         }
-    const FewTable<1, 1> &t1 = few_reduce<1, 1>(sum, lo, hi);
+    const FewTable<CH, 1, 1> &t1 = few_reduce<CH, 1, 1>(sum, lo, hi);
     if (!active) return;
-    const int cl = (threadIdx.x & 3) * 4;
+    const int cl = (threadIdx.x % kQuads) * 4;
     float mu[4], s[4], g[4], b[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -922,7 +930,7 @@ __global__ void __launch_bounds__(kFewThreads) bn_fwd_few_kernel(const float *__
     }
 #pragma unroll
     for (int u = 0; u < ROWS; ++u) {
-        const int r = ty + u * kFewHigh;
+        const int r = ty + u * kFewHigh<CH>;
         if (r >= rows) break;
         float t[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
 #pragma unroll
@@ -936,6 +944,7 @@ __global__ void __launch_bounds__(kFewThreads) bn_fwd_few_kernel(const float *__
 
 // Backward: the channel's sums and the extremes of dy, and what bn_bwd_channel makes of them.  (blocks behind the channels: code
 // sums that a later product needs; `zero`: cleared on the way)
+template <int CH>
 __global__ void __launch_bounds__(kFewThreads) bn_bwd_few_kernel(const float *__restrict__ dy, const float *__restrict__ x, int rows, int C,
                                                                  const float *__restrict__ mean, const float *__restrict__ vmin,
                                                                  const float *__restrict__ vmax, const float *__restrict__ gamma,
@@ -943,14 +952,28 @@ __global__ void __launch_bounds__(kFewThreads) bn_bwd_few_kernel(const float *__
                                                                  const BnBwdOut out, const ZeroJobs zero, const __grid_constant__ SumJobs J)
 {
     pdl_wait();
-    const int blocks = (C + 15) / 16;
+    const int blocks = (C + CH - 1) / CH;
     if ((int)blockIdx.x >= blocks) {
         if (threadIdx.x < kSumThreads) code_sums_block(J, (int)blockIdx.x - blocks);
         return;
     }
     run_zero_jobs(zero, (int64_t)blockIdx.x * kFewThreads + threadIdx.x, (int64_t)blocks * kFewThreads);
-    const int col = (int)blockIdx.x * 16 + (threadIdx.x & 3) * 4, ty = threadIdx.x >> 2;
+    constexpr int kQuads = CH / 4;
+    const int col = (int)blockIdx.x * CH + (threadIdx.x % kQuads) * 4, ty = threadIdx.x / kQuads;
     const bool active = col < C;
+    constexpr int U = 4;
+    float4 vx[U], vd[U];
+    auto fetch = [&](int r0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int r = r0 + u * kFewHigh<CH>;
+            if (r < rows && active) {
+                vx[u] = __ldg(reinterpret_cast<const float4 *>(x + (int64_t)r * C + col));
+                vd[u] = __ldg(reinterpret_cast<const float4 *>(dy + (int64_t)r * C + col));
+            }
+        }
+    };
+    fetch(ty);                            // (on their way while the channels' constants are)
     double sum[2][4];
     float lo[3][4], hi[3][4];             // ordinary positions, those at the channel's maximum, at its minimum
     float mu[4], s[4], g[4], b[4], cl[4], ch[4];
@@ -964,20 +987,11 @@ __global__ void __launch_bounds__(kFewThreads) bn_bwd_few_kernel(const float *__
         s[e] = bn_scale(cl[e], ch[e], Cn);
         g[e] = gamma ? gamma[c] : 1.0f; b[e] = beta ? beta[c] : 0.0f;
     }
-    constexpr int U = 4;
-    for (int r0 = ty; r0 < rows && active; r0 += U * kFewHigh) {
-        float4 vx[U], vd[U];
+    for (int r0 = ty; r0 < rows && active; r0 += U * kFewHigh<CH>) {
+        if (r0 != ty) fetch(r0);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int r = r0 + u * kFewHigh;
-            if (r < rows) {
-                vx[u] = __ldg(reinterpret_cast<const float4 *>(x + (int64_t)r * C + col));
-                vd[u] = __ldg(reinterpret_cast<const float4 *>(dy + (int64_t)r * C + col));
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (r0 + u * kFewHigh >= rows) break;
+            if (r0 + u * kFewHigh<CH> >= rows) break;
             const float ax[4] = {vx[u].x, vx[u].y, vx[u].z, vx[u].w}, ad[4] = {vd[u].x, vd[u].y, vd[u].z, vd[u].w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -993,10 +1007,10 @@ __global__ void __launch_bounds__(kFewThreads) bn_bwd_few_kernel(const float *__
             }
         }
     }
-    const FewTable<2, 3> &t = few_reduce<2, 3>(sum, lo, hi);
+    const FewTable<CH, 2, 3> &t = few_reduce<CH, 2, 3>(sum, lo, hi);
     // one thread per channel
-    const int k = threadIdx.x, c = (int)blockIdx.x * 16 + k;
-    if (k >= 16 || c >= C) return;
+    const int k = threadIdx.x, c = (int)blockIdx.x * CH + k;
+    if (k >= CH || c >= C) return;
     const float ev[6] = {t.lo[0][k], t.hi[0][k], t.lo[1][k], t.hi[1][k], t.lo[2][k], t.hi[2][k]};
     bn_bwd_channel(c, t.sum[0][k], t.sum[1][k], rows, Cnd, gamma ? gamma[c] : 1.0f, beta ? beta[c] : 0.0f, mean[c], vmin[c], vmax[c], Cn,
                    out.chan_range ? ev : nullptr, out);
@@ -1011,8 +1025,10 @@ static int launch_bwd_few(const float *dy, const float *x, int64_t n, int64_t C,
     if (extra_count) if (int rc = fill_sum_jobs(extra, extra_count, J, &sum_blocks)) return rc;
     const double Cnd = 1.0 / std::sqrt(2.0 * std::log((double)n));
     QBP_TRACE_BEGIN(st);
-    launch(bn_bwd_few_kernel, (int)((C + 15) / 16) + sum_blocks, kFewThreads, 0, st, dy, x, (int)n, (int)C, mean, vmin, vmax, gamma, beta,
-           relu, (float)Cnd, Cnd, out, zero, J);
+#define QBP_BN_FEW(CH_) launch(bn_bwd_few_kernel<CH_>, (int)((C + CH_ - 1) / CH_) + sum_blocks, kFewThreads, 0, st, dy, x, (int)n, (int)C, mean, vmin, \
+                               vmax, gamma, beta, relu, (float)Cnd, Cnd, out, zero, J)
+    if (few_narrow(n, C, sum_blocks)) QBP_BN_FEW(8); else QBP_BN_FEW(16);
+#undef QBP_BN_FEW
     QBP_LAUNCH_OK("bn_bwd_few_kernel");
     return QBP_OK;
 }
@@ -1150,12 +1166,13 @@ extern "C" __attribute__((visibility("default"))) int qbp_rangebn_fwd_q8(const f
     if (!save_mean || !save_min || !save_max) return fail(QBP_ERR_INVALID_ARG, "rangebn_fwd: NULL statistics buffer");
     if (!rq && !out_range && few_rows(n, C) && aligned16(x) && aligned16(y)) {
         const float Cn = (float)(1.0 / std::sqrt(2.0 * std::log((double)n)));
-        const int grid = (int)((C + 15) / 16);
         QBP_TRACE_BEGIN(st);
-#define QBP_BN_FEW(ROWS_) launch(bn_fwd_few_kernel<ROWS_>, grid, kFewThreads, 0, st, x, (int)n, (int)C, gamma, beta, relu, Cn, y, save_mean, save_min, save_max)
-        if (n <= kFewHigh)          QBP_BN_FEW(1);
-        else if (n <= 4 * kFewHigh) QBP_BN_FEW(4);
-        else                        QBP_BN_FEW(16);
+#define QBP_BN_FEW(CH_, ROWS_) launch(bn_fwd_few_kernel<CH_, ROWS_>, (int)((C + CH_ - 1) / CH_), kFewThreads, 0, st, x, (int)n, (int)C, gamma, beta, \
+                                      relu, Cn, y, save_mean, save_min, save_max)
+        if (few_narrow(n, C, 0)) { if (n <= 4 * kFewHigh<8>) QBP_BN_FEW(8, 4); else QBP_BN_FEW(8, 8); }
+        else if (n <= kFewHigh<16>)     QBP_BN_FEW(16, 1);
+        else if (n <= 4 * kFewHigh<16>) QBP_BN_FEW(16, 4);
+        else                            QBP_BN_FEW(16, 16);
 #undef QBP_BN_FEW
         QBP_LAUNCH_OK("bn_fwd_few_kernel");
         return QBP_OK;

@@ -132,3 +132,17 @@ def test_few_rows(B, n, C, relu):
     assert np.abs(to_host(mean) - om).max() <= 1e-6 * max(1.0, np.abs(om).max())
     assert _per_channel_rel(to_host(y), oy, _scales(x, dy, olo, ohi, gamma, beta)[0]) <= FP32_TOL
     _run(B, x, dy, gamma, beta, relu)
+
+
+@pytest.mark.parametrize("n,C", [(129, 1184), (1025, 1180), (2048, 52), (129, 1188), (700, 1204)])
+def test_few_rows_block_widths(B, n, C):
+    """Blocks of 8 channels up to the widest tensor that has them (148 blocks), of 16 beyond; channel groups partly filled."""
+    x = synth.channel_gaussian((n, 1, 1, C), 35, 36).reshape(n, C); dy = synth.normal((n, C), 37)
+    gamma = synth.uniform((C,), 38, 1.0) + np.float32(1.5); beta = synth.uniform((C,), 39, 0.5)
+    gamma[::3] *= -1
+    y, mean, vmin, vmax, _ = B.qbp_rangebn_fwd(to_dev(x), to_dev(gamma), to_dev(beta), True)
+    oy, om, olo, ohi = O.rangebn_fwd(x, gamma, beta, True)
+    assert np.array_equal(to_host(vmin), olo) and np.array_equal(to_host(vmax), ohi)
+    assert np.abs(to_host(mean) - om).max() <= 1e-6 * max(1.0, np.abs(om).max())
+    assert _per_channel_rel(to_host(y), oy, _scales(x, dy, olo, ohi, gamma, beta)[0]) <= FP32_TOL
+    _run(B, x, dy, gamma, beta, True)
