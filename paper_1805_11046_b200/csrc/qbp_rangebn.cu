@@ -1213,7 +1213,8 @@ extern "C" __attribute__((visibility("default"))) int qbp_rangebn_fwd_apply(cons
     QBP_TRACE_BEGIN(st);
     launch(bn_mean_from_sum_kernel, (int)((C + 255) / 256), 256, 0, st, col_sum, col_min, col_max, (int)C, n_stat, save_mean, save_min, save_max);
     QBP_LAUNCH_OK("bn_mean_from_sum_kernel");
-    return bn_fwd_apply_launch(x, n_rows, n_stat, C, gamma, beta, relu, y, save_mean, save_min, save_max, out_range, rq, st, true, kKeepBytes / (4 * C));
+    // (nothing kept for a backward call, which here comes after other layers: 103 MB statistics + apply 55.4 us with it, 53.2 without)
+    return bn_fwd_apply_launch(x, n_rows, n_stat, C, gamma, beta, relu, y, save_mean, save_min, save_max, out_range, rq, st, true, 0);
 }
 
 // The statistics half of the recompute fusion (a convolution run twice: once for the statistics, once to write
