@@ -314,7 +314,9 @@ int qbp_conv_s8_implicit(int mode, const qbp_conv_desc *d,
  * int32 accumulator over at most 65536 reduction rows at a time (the low
  * limb's bound is 128*255*rows <= 2^31-1, rows <= 65793); partial results
  * are combined in int64, exactly.  acc_out (int64) and dW each nullable, not
- * both; dW = (float)acc * (sx*sg).
+ * both, at any address of their element's alignment (off a 16-byte boundary
+ * the faster kernel for plain products is not taken);
+ * dW = (float)acc * (sx*sg).
  * ---------------------------------------------------------------------- */
 size_t qbp_wgrad_s16_workspace_bytes(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K);
 

@@ -965,8 +965,9 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
     }
     int64_t *part = P.direct ? nullptr : w.take<int64_t>((size_t)pl.grid * (size_t)P.part_stride);
 
-    // most plain products run on CTA pairs (tiles across two SMs, the whole reduction in one pair)
-    const bool pair_kernel = !d && wgrad2_eligible(M, N, K);
+    // most plain products run on CTA pairs (tiles across two SMs, the whole reduction in one pair), whose stores (TMA for dW, 16 bytes
+    // at a time for acc_out) want both outputs on a 16-byte boundary; the single-CTA kernel takes any float- and int64-aligned ones
+    const bool pair_kernel = !d && wgrad2_eligible(M, N, K) && aligned16(dW) && aligned16(acc_out);
     // code sums for the zero-point terms: of everything, or (the kernels that wrote the codes left their per-channel totals,
     // or the product takes the gradient's itself: a row of ones in its spare chunk) of the images' edges only
     int rc;

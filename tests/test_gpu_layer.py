@@ -28,6 +28,9 @@ def _run_layer(B, cfg, relu, conv=None):
         assert dy.data_ptr() % 16 == 4 * cfg["dy_off"]
     L = layer.QuantizedLayer(conv=conv, batch=x.shape[0], in_features=x.shape[-1], out_features=w.shape[-1] if conv is None else None,
                              relu=relu, seed=cfg["seed"], tensor_id8=cfg["id8"], tensor_id16=cfg["id16"])
+    if cfg.get("dw_off"):
+        L.dw = torch.cat([L.dw.new_empty(cfg["dw_off"]), L.dw.flatten()])[cfg["dw_off"]:].view(L.dw.shape)
+        assert L.dw.data_ptr() % 16 == 4 * cfg["dw_off"]
     y = L.forward(to_dev(x), to_dev(w))
     dx, dw, dgamma, dbeta = L.backward(dy)
     torch.cuda.synchronize()
@@ -496,6 +499,14 @@ def test_wide_linear_layers_stagewise(B, batch, cin, cout):
     pass: channel counts that fill one, part of a second and several slabs of columns."""
     cfg = dict(x=synth.normal((batch, cin), 65), w=synth.kaiming_uniform_linear(cin, cout, 66), dy=synth.normal((batch, cout), 67, std=0.1),
                seed=4, id8=6, id16=6)
+    _check_layer(B, cfg, True)
+
+
+@pytest.mark.parametrize("batch,cin,cout", [(2048, 1024, 208), (528, 256, 256), (64, 256, 128)])
+def test_linear_layer_weight_gradient_in_a_flat_buffer(B, batch, cin, cout):
+    """dw 4 bytes behind a 16-byte boundary, with the gradient's totals from the pass that writes its codes."""
+    cfg = dict(x=synth.normal((batch, cin), 65), w=synth.kaiming_uniform_linear(cin, cout, 66), dy=synth.normal((batch, cout), 67, std=0.1),
+               seed=4, id8=6, id16=6, dw_off=1)
     _check_layer(B, cfg, True)
 
 

@@ -597,6 +597,25 @@ def test_wgrad_tiles_that_fit_the_machine_once(B, M, N, K):
     assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
 
 
+@pytest.mark.parametrize("dw_off,acc_off", [(1, 0), (0, 1), (1, 1)])
+@pytest.mark.parametrize("M,N,K", [(2048, 208, 1024), (48, 1024, 1024), (528, 272, 304), (1040, 128, 272), (2048, 64, 48)])
+def test_wgrad_outputs_off_the_vector_boundary(B, M, N, K, dw_off, acc_off):
+    """dW one float, acc_out one int64 behind a 16-byte boundary, as slices of flat buffers are: shapes that the kernel on CTA pairs
+    takes where both lie on one, and shapes that it does not take; what lies before and behind the slices stays."""
+    import torch
+    X = random_codes((M, K), 65); G = _g16((M, N), 66)
+    hi, lo = O.limb_split(G)
+    flat_w = torch.full((K * N + 8,), 7.0, dtype=torch.float32, device="cuda"); flat_a = torch.full((K * N + 4,), 7, dtype=torch.int64, device="cuda")
+    dW, acc = flat_w[dw_off:dw_off + K * N].view(K, N), flat_a[acc_off:acc_off + K * N].view(K, N)
+    assert dW.data_ptr() % 16 == 4 * dw_off and acc.data_ptr() % 16 == 8 * acc_off
+    _, _, ws = B.qbp_wgrad_s16(to_dev(X), _qp(B, 0.5, -3), to_dev(hi), to_dev(lo), _qp(B, 0.25, 1234), acc_out=acc, dW=dW)
+    oacc, oout = O.gemm_s16s8(X, -3, G, 1234, 0.5, 0.25)
+    assert B.status_word(ws) == 0
+    assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
+    for flat, off in ((flat_w, dw_off), (flat_a, acc_off)):
+        assert bool((flat[:off] == 7).all()) and bool((flat[off + K * N:] == 7).all())
+
+
 @pytest.mark.parametrize("N,H,W,C,K,R", [(1, 8, 16, 128, 128, 3), (2, 12, 12, 128, 160, 3), (6, 16, 16, 256, 96, 1), (5, 11, 13, 96, 160, 3)])
 def test_wgrad_conv_one_tile_per_block_and_ragged_columns(B, N, H, W, C, K, R):
     """Reductions short enough that each block takes one tile of 128 rows, from a single step on; output channels that leave most
