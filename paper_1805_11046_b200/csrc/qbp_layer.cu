@@ -129,7 +129,7 @@ static int conv_rangebn_recompute(const qbp_conv_desc *d, const int8_t *x_codes,
                                   const int8_t *w_codes, const qbp_qparams *qw, const float *gamma, const float *beta, int relu,
                                   float *save_mean, float *save_min, float *save_max, const qbp_requant *out,
                                   ColStatParts parts, float4 *fold, const CodeSums &w_sums, int *status, void *ws, size_t scratch,
-                                  bool beside, const SumJob *extra, int extra_count, cudaStream_t st)
+                                  bool beside, const SumJob *extra, int extra_count, bool totals_cleared, cudaStream_t st)
 {
     const int64_t rows = (int64_t)d->N * d->H * d->W;
     const EpilogueTail first{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums, extra, extra_count, beside};
@@ -140,7 +140,7 @@ static int conv_rangebn_recompute(const qbp_conv_desc *d, const int8_t *x_codes,
     const EpilogueTail tail{fold, relu, out->qp, out->q, out->row_sums, 1, &w_sums};
     rc = conv_s8_impl(QBP_CONV_FPROP, d, x_codes, qx, w_codes, qw, nullptr, nullptr, in_sums, nullptr, status, ws, scratch, st, &tail);
     if (rc || !out->chan_sums) return rc;
-    return launch_colsum(out->q, true, rows, d->K, out->chan_sums, st, true);
+    return launch_colsum(out->q, true, rows, d->K, out->chan_sums, st, totals_cleared);
 }
 
 }  // namespace qbp
@@ -207,8 +207,18 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_fwd_chained(cons
     // (an input that came without its channel totals: cleared with the rest, summed up below; a filter has cin columns)
     const bool chained_totals = !x && want_totals && !in->chan_sums;
     if (chained_totals) wo.tot = saved->x_chan_sums;
-    // ... and the totals that the last kernel of this call adds to, so that no memset stands between two kernels
-    const bool clear_out = out && out->chan_sums;
+    // ... and the totals that the last kernel of this call adds to, so that no launch for it stands between two kernels -- unless a
+    // later step of this call refuses it (they then stay as they are), or their memory holds what the steps before that kernel still
+    // read or add to
+    const bool goes_through = aligned16(saved->x_codes) && aligned16(saved->w_codes) &&
+                              (recompute ? aligned16(out->q) : aligned16(saved->z) && s.rows < (1ll << 22));
+    const auto apart = [&](const void *p, int64_t bytes) {
+        const uintptr_t a = (uintptr_t)p, o = (uintptr_t)out->chan_sums;
+        return !p || o + sizeof(int64_t) * (size_t)s.cout <= a || a + (size_t)bytes <= o;
+    };
+    const bool clear_out = out && out->chan_sums && goes_through && apart(x, 4 * s.x_elems) && apart(w, 4 * s.w_elems) &&
+                           apart(saved->x_codes, s.x_elems) && apart(saved->w_codes, s.w_elems) &&
+                           apart(want_totals ? saved->x_chan_sums : nullptr, 8 * s.cin) && apart(in ? in->row_sums : nullptr, 4 * s.rows);
     const bool no_launch = !s.conv || L->conv.R == 3 || !want_totals || (x ? quantizer_totals_supported(s.cin) : !chained_totals);
     if ((rc = quantize_operands(x ? &xo : nullptr, &wo, status, l.scratch, l.scratch_bytes, st, no_launch, clear_out ? out->chan_sums : nullptr,
                                 clear_out ? 2 * s.cout : 0))) return rc;
@@ -232,7 +242,7 @@ extern "C" __attribute__((visibility("default"))) int qbp_layer_fwd_chained(cons
     if (recompute)
         return conv_rangebn_recompute(&L->conv, saved->x_codes, saved->qx, in_sums, saved->w_codes, saved->qw, gamma, beta, L->relu,
                                       saved->save_mean, saved->save_min, saved->save_max, out, parts, l.fold, w_sums, status,
-                                      l.scratch, l.scratch_bytes, beside, &tot_job, tot_with_terms ? 1 : 0, st);
+                                      l.scratch, l.scratch_bytes, beside, &tot_job, tot_with_terms ? 1 : 0, clear_out, st);
     const EpilogueTail with_sums{nullptr, 0, nullptr, nullptr, nullptr, 0, &w_sums, &tot_job, tot_with_terms ? 1 : 0, beside};
     if (s.conv)
         rc = conv_s8_impl(QBP_CONV_FPROP, &L->conv, saved->x_codes, saved->qx, saved->w_codes, saved->qw, nullptr, saved->z,

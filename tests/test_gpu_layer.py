@@ -426,6 +426,62 @@ def test_recompute_fusion_writes_the_same_codes_without_storing_the_product(B, b
         lean.backward(to_dev(cfg["dy"]))
 
 
+@pytest.mark.parametrize("shared", ["input totals", "handed-on input without totals", "input", "weights", "row sums"])
+@pytest.mark.parametrize("n,hw,r,keep_z", [(2, 9, 3, True), (8, 28, 3, True), (8, 28, 1, True), (2, 9, 3, False), (8, 28, 3, False)])
+def test_output_totals_in_memory_the_forward_is_done_with(B, n, hw, r, keep_z, shared):
+    """A forward-only caller that has no use for the input's totals (nor its input, weights or row sums) any more lets the output's
+    totals take their place: small and large operands, with and without a pass over the product."""
+    import torch
+    from paper_1805_11046_b200 import layer
+    c = 64
+    conv, x, w = B.conv_desc(n, hw, hw, c, c, r, r, 1, (r - 1) // 2), to_dev(synth.normal((n, hw, hw, c), 31)), to_dev(synth.normal((c, r, r, c), 32))
+    x0, w0 = x.clone(), w.clone()
+    first = layer.QuantizedLayer(conv=conv, relu=True, emit_codes=True, keep_y=False)
+    first.forward(x, w)
+    handed_on = shared in ("handed-on input without totals", "row sums")
+    outs = []
+    for alias in (False, True):
+        x.copy_(x0); w.copy_(w0)
+        L = layer.QuantizedLayer(conv=conv, relu=True, emit_codes=True, keep_y=False, keep_z=keep_z, input_from=first if handed_on else None)
+        sums = first.out_row_sums.clone()
+        if handed_on:
+            L.rq_in = B.requant(first.out_codes, first.q_out, sums if shared == "row sums" else None, None)
+        if alias:
+            tot = {"input totals": L.out_chan_sums, "handed-on input without totals": L.out_chan_sums, "input": x.view(-1)[:2 * c].view(torch.int64),
+                   "weights": w.view(-1)[:2 * c].view(torch.int64), "row sums": sums[:2 * c].view(torch.int64)}[shared]
+            L.out_chan_sums, L.rq_out = tot, B.requant(L.out_codes, L.q_out, L.out_row_sums, tot)
+            if "totals" in shared:
+                L.ctx.x_chan_sums = tot.data_ptr()
+        L.forward(None if handed_on else x, w)
+        assert L.status() == 0
+        outs.append((to_host(L.out_codes).copy(), to_host(L.out_chan_sums).copy()))
+    assert np.array_equal(outs[0][0], outs[1][0])
+    for codes, tot in outs:
+        assert np.array_equal(tot, codes.reshape(-1, c).astype(np.int64).sum(0))
+
+
+@pytest.mark.parametrize("kind", ["2^22 rows", "codes off a 16-byte boundary", "product off a 16-byte boundary"])
+def test_output_totals_of_a_refused_forward_stay(B, kind):
+    import torch
+    from paper_1805_11046_b200 import layer
+    if kind == "2^22 rows":
+        L = layer.QuantizedLayer(batch=1 << 22, in_features=16, out_features=16, emit_codes=True, keep_y=False, keep_g=False)
+        x, w, codes = torch.randn(L.x_shape, device="cuda"), torch.randn(L.w_shape, device="cuda"), L.out_codes
+    else:
+        L = layer.QuantizedLayer(conv=B.conv_desc(2, 9, 9, 32, 32, 3, 3, 1, 1), emit_codes=True, keep_y=False, keep_z=kind.startswith("product"))
+        x, w, codes = torch.randn(L.x_shape, device="cuda"), torch.randn(L.w_shape, device="cuda"), L.out_codes
+        if kind.startswith("codes"):
+            codes = torch.empty(codes.numel() + 4, dtype=torch.int8, device="cuda")[4:]
+        else:
+            off = torch.empty(L.z.numel() + 1, device="cuda")
+            L.ctx.z = off.data_ptr() + 4
+    tot = torch.full((L.cout,), 7, dtype=torch.int64, device="cuda")
+    L.rq_out = B.requant(codes, L.q_out, L.out_row_sums, tot)
+    with pytest.raises(B.QbpError):
+        L.forward(x, w)
+    assert bool((tot == 7).all())
+
+
 @pytest.mark.parametrize("batch,hw,cin,cout,R", [(3, 9, 32, 96, 3), (2, 12, 64, 32, 3), (2, 7, 96, 64, 3), (4, 6, 128, 128, 3),
                                                    (3, 10, 64, 128, 1), (2, 5, 32, 32, 3), (2, 6, 32, 320, 1)])
 def test_conv_layers_of_other_shapes_stagewise(B, batch, hw, cin, cout, R):
