@@ -298,12 +298,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
     }
 }
 
-// Whether the pair kernel takes this plain product: a reduction that one pair can hold in int32, and one of
-//   - fewer than 512 rows: large outputs (64 rows for 2048 x 2048: 15.7 us with the single-CTA kernel, 13.3 with this one; 384 for
-//     256 x 256: 9.2 against 9.6);
+// Whether the pair kernel takes this plain product: a reduction that one pair can hold in int32, and one of (call with its sums, first
+// with the single-CTA kernel, then with this one)
+//   - fewer than 512 rows: large outputs (64 rows for 2048 x 2048: 15.7 and 13.3 us; not 384 for 256 x 256: 9.2 and 9.6);
 //   - more: where the longer walk of a pair over all rows, about 2.9 us per 1000, costs less than the single-CTA kernel's
-//     partial sums, about 1 us per 10000 outputs (8192 rows for 4096 x 128: 68.9 us -> 39.6, 2048 for 1024 x 208: 35.2 -> 16.3,
-//     512 for 128 x 128: 9.1 against 9.4, 8192 for 128 x 128: 20.5 against 31.9, 65536 for 256 x 256: 49.6 against 228).
+//     partial sums, about 1 us per 10000 outputs (8192 rows for 4096 x 128: 68.9 and 39.6, 2048 for 1024 x 208: 35.2 and 16.3; not
+//     512 for 128 x 128: 9.1 and 9.4, 8192 for 128 x 128: 20.5 and 31.9, 65536 for 256 x 256: 49.6 and 228).
 bool wgrad2_eligible(int64_t M, int64_t N, int64_t K)
 {
     if (M > 65536 || N < 64 || K < 64) return false;
@@ -318,11 +318,13 @@ int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qp
     int rc;
     // where tiles of 256 columns fit the pairs once, tiles of half as many (64 at least) as long as they do: rings and epilogues get
     // shorter, and SMs that had none take part.  Call with its sums, 256 columns -> by this rule: 1024 rows for 2048 x 1008 18.3 ->
-    // 15.6 us, 4096 for 1024 x 1024 31.7 -> 24.1, 16384 for 256 x 512 84.9 -> 57.0
+    // 15.6 us, 4096 for 1024 x 1024 31.7 -> 24.1, 16384 for 256 x 512 84.9 -> 57.0.  And never wider than the columns there are, also
+    // where the row tiles alone do not fit: 4096 rows for 20000 x 128 68.4 -> 54.7 (single-CTA kernel 52.3), 1024 for 65536 x 128
+    // 55.9 -> 44.3 (49.3), 8192 for 65536 x 64 264 -> 216 (200)
     const auto tiles_n_of = [&](int bn) { return (N + bn - 1) / bn; };
     P.tiles_m = (int)((K + 255) / 256);
     P.bn = 256;
-    while (P.bn > 64 && P.tiles_m * tiles_n_of(P.bn / 2) <= sm_count() / 2) P.bn /= 2;
+    while (P.bn > 64 && (N <= P.bn / 2 || P.tiles_m * tiles_n_of(P.bn / 2) <= sm_count() / 2)) P.bn /= 2;
     P.tiles_n = (int)tiles_n_of(P.bn);
     P.tiles_total = P.tiles_m * P.tiles_n;
     // per-CTA operand parts: 128 reduction rows x 128 columns of X, x bn / 2 of each limb, M/N-major

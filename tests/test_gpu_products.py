@@ -296,6 +296,12 @@ def test_wgrad_plain(B, M, N, K):
     assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(dW), oout)
 
 
+@pytest.mark.parametrize("M,N,K", [(48, 64, 18960), (528, 112, 18960), (512, 128, 18944), (64, 144, 18960)])
+def test_wgrad_pair_kernel_more_row_tiles_than_pairs(B, M, N, K):
+    """Outputs whose 256-row tiles alone fill the SM pairs or do not fit them once: tiles as wide as the columns there are."""
+    test_wgrad_plain_pair_kernel_narrow_tiles(B, M, N, K)
+
+
 # The CTA-pair kernel where it fits the SM pairs once: tiles of 64, 128 and 256 columns, ragged in every dimension, fewer
 # reduction steps than the ring has stages and more; outputs smaller than a tile, the fewest rows; the last is just too deep for it.
 @pytest.mark.parametrize("M,N,K", [(528, 272, 304), (2064, 256, 256), (560, 1008, 2064), (1536, 784, 4368), (1040, 208, 160),
