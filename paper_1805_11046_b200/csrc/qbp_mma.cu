@@ -1268,7 +1268,7 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
 
     // large and deep products run on CTA pairs (tiles across two SMs); the column statistics are the
     // single-CTA kernel's (at most 256 columns: narrow either way)
-    if (gemm2_eligible(M, N, K) && !stats && !has_tail)
+    if (gemm2_eligible(transB, M, N, K) && !stats && !has_tail)
         return launch_gemm2(transA, transB, M, N, K, A, qa, B, qb, acc_out, C, asum, bsum, status, beside, st);
 
     MmaParams P{};

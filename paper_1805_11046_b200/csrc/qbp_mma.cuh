@@ -176,7 +176,7 @@ int make_map_out_nhwc(CUtensorMap *map, float *base, uint64_t N, uint64_t H, uin
                       uint32_t sh, uint32_t sw);
 
 // ---- the dense product on CTA pairs (qbp_mma2.cu) -------------------------------
-bool gemm2_eligible(int64_t M, int64_t N, int64_t K);
+bool gemm2_eligible(int transB, int64_t M, int64_t N, int64_t K);
 int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,
                  const int8_t *B, const qbp_qparams *qb, int32_t *acc_out, float *C, const CodeSums &a_sums,
                  const CodeSums &b_sums, int *status, bool beside, cudaStream_t st);

@@ -317,10 +317,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k2Threads, 1) qbp_mm
 // more but for the narrowest outputs, where its deeper ring counts for more than the rows and columns of a tile that lie
 // outside (call with its sums, single-CTA -> pair kernel: 8192 x 128 x 8192 45.4 -> 34.0 us, 64 x 512 x 4096 21.7 -> 16.1,
 // 16 x 1024 x 1024 9.0 -> 8.5, 1024 x 48 x 2048 with A transposed 15.0 -> 16.0).  The short ones stay with the single-CTA kernel
-// (256 x 128 x 256: 7.4 against 8.0, 8192 x 208 x 128: 8.4 against 8.8).
-bool gemm2_eligible(int64_t M, int64_t N, int64_t K)
+// (256 x 128 x 256: 7.4 against 8.0, 8192 x 208 x 128: 8.4 against 8.8), and from 64 K rows on those of up to 4096 whose columns just
+// fit a tile of it: 64, 128, or any of B along the reduction (131072 x 64 x 1024: 75.4 against 79.1, 131072 x 128 x 2048 112.5 against
+// 116.1, 136736 x 112 x 1024 with B transposed 80.2 against 87.8; not transposed 103.0 against 89.1).
+bool gemm2_eligible(int transB, int64_t M, int64_t N, int64_t K)
 {
-    return (M >= 256 && N >= 256 && K >= 128) || (N >= 64 && K >= 1024);
+    if (M >= 256 && N >= 256 && K >= 128) return true;
+    const bool fits = N <= 128 && (transB || N == 64 || N == 128);
+    return N >= 64 && K >= 1024 && !(fits && M >= 65536 && K < 4096);
 }
 
 int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const int8_t *A, const qbp_qparams *qa,
@@ -337,12 +341,16 @@ int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const 
     // 256 x 256 fit the pairs once, they and tiles of half as many columns (64 at least) as long as they do: rings and epilogues
     // get shorter, and SMs that had none take part.  Times of a call with its sums, 256 or 512 rows by 256 -> by this rule:
     // 4096 x 256 x 1024 15.4 -> 9.8 us, 2048 x 2048 x 2048 20.2 -> 15.3, 4096 x 1024 x 4096 30.0 -> 21.8, 1024 x 1024 x 1024
-    // 11.3 -> 9.5; the same where it changes nothing (2048 x 2560 x 1024: 16.6).
+    // 11.3 -> 9.5; the same where it changes nothing (2048 x 2560 x 1024: 16.6).  Of outputs of at most 128 columns whose row tiles
+    // alone do not fit the pairs once, tiles of 256 rows by the columns' own width instead of 512 x 256 where the operand rows a CTA
+    // fetches for them, and a fifth for the additional rounds, are fewer: 40000 x 128 x 2048 41.9 -> 35.6 us, 54784 x 128 x 3072 78.8 ->
+    // 68.4; not 20000 x 64 x 4096 (32.6 as 512 x 256, 34.8) nor 37888 x 128 x 1024 (20.0 and 21.0).
     const auto tiles_of = [&](int64_t m, int64_t n) { return ((M + m - 1) / m) * ((N + n - 1) / n); };
     const int pairs = sm_count() / 2;
     const auto rounds = [&](int64_t m) { return (tiles_of(m, 256) + pairs - 1) / pairs; };
-    P.msub = tiles_of(256, 256) > pairs && 3 * rounds(512) < 2 * rounds(256) + (K >= 1024) ? 2 : 1;
-    P.bn = 256;
+    P.bn = N <= 64 ? 64 : N <= 128 ? 128 : 256;
+    if (P.bn < 256 && 6 * (128 + P.bn / 2) * rounds(256) >= 5 * 384 * rounds(512)) P.bn = 256;
+    P.msub = P.bn == 256 && tiles_of(256, 256) > pairs && 3 * rounds(512) < 2 * rounds(256) + (K >= 1024) ? 2 : 1;
     while (P.msub == 1 && P.bn > 64 && tiles_of(256, P.bn / 2) <= pairs) P.bn /= 2;
     // per-CTA operand halves: 128 rows of A, bn / 2 columns of B, 128 reduction bytes per stage
     const uint32_t half = (uint32_t)P.bn / 2;

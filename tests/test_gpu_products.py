@@ -592,6 +592,21 @@ def test_gemm_tiles_that_fit_the_machine_once(B, M, N, K, tB):
     assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(out), oout)
 
 
+@pytest.mark.parametrize("M,N,K", [(18960, 64, 1040), (18960, 128, 1040), (37904, 64, 1040), (37904, 112, 1040), (37904, 144, 1040), (65520, 64, 1024),
+                                   (65536, 64, 1024), (65536, 80, 1024)])
+@pytest.mark.parametrize("tA,tB", [(False, False), (False, True), (True, False)])
+def test_gemm_pair_kernel_more_row_tiles_than_pairs(B, M, N, K, tA, tB):
+    """Outputs whose 256-row tiles alone do not fit the SM pairs once: 512 x 256 tiles, 256-row tiles as wide as the columns, the
+    single-CTA kernel; sampled rows, those at the edges of the first and last tiles among them."""
+    rows = np.unique(np.concatenate([[0, 127, 128, 255, 256, 511, 512, M - 1, M - 16, M - 17, M // 512 * 512 - 1, M // 256 * 256 - 1],
+                                     np.random.Generator(np.random.PCG64(66)).integers(0, M, 120)]))
+    A = random_codes((M, K), 67); Bm = random_codes((N, K) if tB else (K, N), 68)
+    acc, out, ws = B.qbp_gemm_s8(to_dev(A.T if tA else A), _qp(B, 0.5, 7), to_dev(Bm), _qp(B, 0.25, -19), transA=tA, transB=tB, want_acc=True)
+    oacc, oout, bad = O.gemm_s8(A[rows], 7, Bm, -19, 0.5, 0.25, transB=tB)
+    assert bad == 0 and B.status_word(ws) == 0
+    assert np.array_equal(to_host(acc)[rows], oacc) and np.array_equal(to_host(out)[rows], oout)
+
+
 @pytest.mark.parametrize("M,N,K", [(64, 32, 128), (128, 4736, 16), (128, 4752, 16), (1024, 1184, 512), (1024, 1200, 512), (144, 176, 240)])
 def test_wgrad_tiles_that_fit_the_machine_once(B, M, N, K):
     """Short reductions over tiles of 32, 64 and 128 columns, each size just inside and just outside one wave."""
