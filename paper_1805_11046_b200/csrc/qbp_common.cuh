@@ -114,7 +114,13 @@ constexpr int kMaxZeroJobs = 5;
 struct ZeroJobs {
     int count;
     uint32_t *p[kMaxZeroJobs]; int64_t words[kMaxZeroJobs];
-    void add(void *at, int64_t n) { if (n > 0) { p[count] = static_cast<uint32_t *>(at); words[count++] = n; } }
+    [[nodiscard]] int add(void *at, int64_t n)
+    {
+        if (n <= 0) return QBP_OK;
+        if (count == kMaxZeroJobs) return fail(QBP_ERR_INVALID_ARG, "more than %d regions to clear in one launch", kMaxZeroJobs);
+        p[count] = static_cast<uint32_t *>(at); words[count++] = n;
+        return QBP_OK;
+    }
 };
 
 // -------------------------------------------------------------- device side

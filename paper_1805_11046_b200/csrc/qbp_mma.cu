@@ -1261,7 +1261,7 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
 
     int rc = QBP_OK;
     ZeroJobs zero{};
-    if (!ext_status) zero.add(status, 1);
+    if (!ext_status && (rc = zero.add(status, 1))) return rc;
     bool own = false;
     if ((rc = launch_code_sums(jobs, njobs, st, zero, &own))) return rc;
     beside = njobs ? own : beside && !zero.count;         // (a tail's launch for its parameters comes in between)
@@ -1427,7 +1427,7 @@ int qbp::conv_s8_impl(int mode, const qbp_conv_desc *d, const int8_t *in, const 
     int rc = QBP_OK;
     if (in_chan_sum) chan_sum = const_cast<int32_t *>(in_chan_sum);
     ZeroJobs zero{};
-    if (!ext_status) zero.add(status, 1);
+    if (!ext_status && (rc = zero.add(status, 1))) return rc;
     bool beside = tail && tail->beside && !zero.count;    // (whether the launch before the product is one that it may run beside)
     if (tail && tail->keep_terms) { if ((rc = launch_code_sums(nullptr, 0, st, zero))) return rc; }
     else {

@@ -828,7 +828,7 @@ int launch_clear(void *p, int64_t words, cudaStream_t st)
 {
     if (words <= 0) return QBP_OK;
     ZeroJobs zero{};
-    zero.add(p, words);
+    if (int rc = zero.add(p, words)) return rc;
     const int grid = (int)std::min<int64_t>(sm_count(), (words + kThreads - 1) / kThreads);
     QBP_TRACE_BEGIN(st);
     launch(clear_kernel, grid, kThreads, 0, st, zero);
@@ -1141,8 +1141,8 @@ int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, s
     bool vec[2] = {true, true};
     // (the status word, the caller's, the activation's or the weights' totals, either operand's row sums in pieces)
     ZeroJobs zero{};
-    if (status) zero.add(status, 1);
-    zero.add(clear, clear_words);
+    int rc = status ? zero.add(status, 1) : QBP_OK;
+    if (rc || (rc = zero.add(clear, clear_words))) return rc;
     // small tensors: everything in one launch
     {
         SmallJob J{};
@@ -1152,7 +1152,7 @@ int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, s
         for (int i = 0; i < 2 && small; ++i) {
             if (!ops[i]) continue;
             QuantOperand &op = *ops[i];
-            if (int rc = check_common(op.v, op.rows, op.cols, QBP_PER_TENSOR, QBP_ROUND_NEAREST, op.qp)) return rc;
+            if ((rc = check_common(op.v, op.rows, op.cols, QBP_PER_TENSOR, QBP_ROUND_NEAREST, op.qp))) return rc;
             SmallOperand &s = J.op[count++];
             const int64_t n = op.rows * op.cols;
             s = SmallOperand{op.v, (int)(n / 4), (int)op.cols, quant_out(op.q, nullptr, nullptr, nullptr), op.qp, op.col_sums, 0};
@@ -1160,7 +1160,7 @@ int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, s
                     (!op.row_sums || fuse_rowsums(op.v, n, op.cols, true, op.row_sums, s.o));
             if (op.col_sums) s.pieces = sum_pieces(op.rows, op.cols);
             if (op.tot && i == 0) s.o.chansum8 = reinterpret_cast<unsigned long long *>(op.tot);
-            else if (op.tot) J.zero.add(op.tot, 2 * op.cols);
+            else if (op.tot && (rc = J.zero.add(op.tot, 2 * op.cols))) return rc;
             if (s.colsum || s.o.chansum8) cols = std::max(cols, s.cols);
         }
         if (small) {
@@ -1187,13 +1187,13 @@ int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, s
         parts[i] = c.take<float2>(kMaxParts);
         if (!ops[i]) continue;
         QuantOperand &op = *ops[i];
-        if (int rc = check_common(op.v, op.rows, op.cols, QBP_PER_TENSOR, QBP_ROUND_NEAREST, op.qp)) return rc;
+        if ((rc = check_common(op.v, op.rows, op.cols, QBP_PER_TENSOR, QBP_ROUND_NEAREST, op.qp))) return rc;
         o[i] = quant_out(op.q, nullptr, nullptr, nullptr);
         op.row_sums_left = op.row_sums && fuse_rowsums(op.v, op.rows * op.cols, op.cols, add_rows, op.row_sums, o[i]);
-        if (op.row_sums_left && o[i].rs_shift < 0) zero.add(op.row_sums, op.rows);
+        if (op.row_sums_left && o[i].rs_shift < 0 && (rc = zero.add(op.row_sums, op.rows))) return rc;
         vec[i] = quant_vec(op.v, op.cols, 0, o[i]);
         if (op.tot) {
-            zero.add(op.tot, 2 * op.cols);
+            if ((rc = zero.add(op.tot, 2 * op.cols))) return rc;
             if (i == 0 && vec[i] && quantizer_totals_supported(op.cols)) { o[i].chansum8 = reinterpret_cast<unsigned long long *>(op.tot); op.tot_left = true; }
         }
     }
@@ -1230,8 +1230,7 @@ int quantize_operands(QuantOperand *x, QuantOperand *w, int *status, void *ws, s
         if (!ops[i]) continue;
         QuantOperand &op = *ops[i];
         RangeSrc r{parts[i], 0, nullptr, op.qp, nullptr};
-        int rc = launch_range(op.v, op.rows * op.cols, parts[i], &r.nparts, st, zero);
-        if (rc) return rc;
+        if ((rc = launch_range(op.v, op.rows * op.cols, parts[i], &r.nparts, st, zero))) return rc;
         zero = ZeroJobs{};
         if ((rc = launch_quantize(op.v, op.rows * op.cols, op.cols, 0, QBP_ROUND_NEAREST, r, 0, 0, 0, o[i], st))) return rc;
     }

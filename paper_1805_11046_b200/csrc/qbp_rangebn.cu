@@ -1366,8 +1366,8 @@ int rangebn_bwd_bifurcate_impl(const float *dy, const float *x, int64_t n, int64
     // each row's code sum by shuffles over the row's lanes of a warp; a row that spans several warps or blocks is
     // added up from its pieces (integer atomics on the zeroed sums: the result does not depend on the order)
     ZeroJobs zero{};
-    if (row_sums8 && (ga.tw > 32 || ga.slabs > 1)) zero.add(row_sums8, n);
-    zero.add(clear, clear_words);
+    if (row_sums8 && (ga.tw > 32 || ga.slabs > 1) && (rc = zero.add(row_sums8, n))) return rc;
+    if ((rc = zero.add(clear, clear_words))) return rc;
     if (few_rows(n, C)) {
         if ((rc = launch_bwd_few(dy, x, n, C, gamma, beta, relu, save_mean, save_min, save_max,
                                  BnBwdOut{dgamma, dbeta, coef, chan_range, relu ? relu_thr : nullptr}, zero, extra, extra_count, st)))

@@ -983,13 +983,13 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
         if (tab && (rc = launch_clear(tab, 2 * (int64_t)table, st))) return rc;
     }
     ZeroJobs zero{};
-    if (!ext_status) zero.add(status, 1);
+    if (!ext_status && (rc = zero.add(status, 1))) return rc;
     if (from_totals) {
         P.tot_x = (const long long *)tot_x; P.tot_g = (const long long *)tot_g16;
         P.tot_g_plain = tot_g_filled ? 1 : 0;
         if (!tot_g_filled) {
             P.ones_tot = (unsigned long long *)const_cast<int64_t *>(tot_g16);
-            if (!done_sums) zero.add(P.ones_tot, 2 * N);
+            if (!done_sums && (rc = zero.add(P.ones_tot, 2 * N))) return rc;
         }
     }
     bool beside = false;

@@ -1,6 +1,7 @@
 """What the kernels must keep to because each is launched as a programmatic dependent of the one before it (and may be resident
 while that one, or a caller's kernel, still runs): read from the sources, since a violation would be a race on the device."""
 import re
+import subprocess
 from pathlib import Path
 
 CSRC = Path(__file__).resolve().parent.parent / "paper_1805_11046_b200" / "csrc"
@@ -78,3 +79,27 @@ def test_no_bounded_wait_starts_its_clock_before_the_kernel_may_work():
             assert role.index("pdl_wait();") < re.search(waiting, role).start(), name
         seen += 1
     assert seen == 5                                     # the products' files
+
+
+def test_regions_to_clear_beyond_the_room_for_them_are_refused(tmp_path):
+    """The record that travels with a launch by value: one region too many is an error of the call, and what lies behind stays."""
+    src = tmp_path / "zero.cpp"
+    src.write_text("""
+        #include "qbp_common.cuh"
+        #include <cstring>
+        namespace qbp { int fail(int status, const char *, ...) { return status; } }
+        struct Guarded { qbp::ZeroJobs z; unsigned char behind[256]; };
+        int main()
+        {
+            Guarded g{};
+            memset(g.behind, 7, sizeof g.behind);
+            uint32_t word = 0;
+            for (int i = 0; i < qbp::kMaxZeroJobs; ++i) if (g.z.add(&word, i + 1) != QBP_OK) return 1;
+            if (g.z.add(&word, 0) != QBP_OK || g.z.count != qbp::kMaxZeroJobs) return 2;       // nothing to clear: no room needed
+            if (g.z.add(&word, 1) == QBP_OK || g.z.count != qbp::kMaxZeroJobs) return 3;
+            for (int i = 0; i < qbp::kMaxZeroJobs; ++i) if (g.z.p[i] != &word || g.z.words[i] != i + 1) return 4;
+            for (unsigned char b : g.behind) if (b != 7) return 5;
+            return 0;
+        }""")
+    subprocess.run(["g++", "-std=c++17", "-I", str(CSRC), "-I", "/usr/local/cuda/include", str(src), "-o", str(tmp_path / "zero")], check=True)
+    assert subprocess.run([str(tmp_path / "zero")]).returncode == 0
