@@ -7,10 +7,11 @@ from pathlib import Path
 CSRC = Path(__file__).resolve().parent.parent / "paper_1805_11046_b200" / "csrc"
 
 
-def _sources():
+def _sources(comments=False):
     out = {}
     for f in sorted(CSRC.glob("*.cu*")):
-        out[f.name] = re.sub(r"//[^\n]*", "", f.read_text())
+        text = f.read_text()
+        out[f.name] = text if comments else re.sub(r"//[^\n]*", "", text)
     return out
 
 
@@ -25,9 +26,9 @@ def _body(text, at):
     raise AssertionError("unbalanced braces")
 
 
-def _kernels():
+def _kernels(comments=False):
     out = {}
-    for name, text in _sources().items():
+    for name, text in _sources(comments).items():
         for m in re.finditer(r"__global__[^;{]*?\bvoid\b[^;{]*?(\w+_kernel)\s*\(", text):
             i, depth = m.end(), 1                      # to the end of the parameter list (default arguments may hold braces)
             while depth:
@@ -37,7 +38,8 @@ def _kernels():
     return out
 
 
-EARLY = {"code_sums_kernel", "conv_terms_kernel"}        # the kernels that let their successor go at their start
+EARLY = {"code_sums_kernel", "conv_terms_kernel"}        # the kernels that let their successor go before they end
+PRODUCTS = {"qbp_mma_kernel", "qbp_mma2_kernel", "qbp_conv2_kernel", "qbp_conv2t_kernel", "qbp_wgrad_kernel", "qbp_wgrad2_kernel"}
 
 
 def test_every_kernel_waits_for_the_one_before():
@@ -51,34 +53,81 @@ def test_every_kernel_waits_for_the_one_before():
         assert "tmem_alloc" not in kernels[name]         # a successor could take the tensor memory it waits for
 
 
+def test_a_successor_that_does_not_wait_starts_behind_the_wait_of_the_kernel_before_it():
+    """A product told that its launch follows its sums or terms (`beside`) reads its operands without a wait of its own: the kernel
+    that makes them may let it go only once everything before is complete.  Without that, letting go ahead of the wait is allowed:
+    the successor waits itself."""
+    kernels, sources = _kernels(), _sources()
+    steps = lambda name: re.findall(r"(if \([^;]*?\) )?(pdl_trigger|pdl_wait)\(\)", kernels[name])
+    assert steps("conv_terms_kernel") == [("", "pdl_wait"), ("", "pdl_trigger")]
+    assert steps("code_sums_kernel") == [("if (!J.beside) ", "pdl_trigger"), ("", "pdl_wait"), ("if (J.beside) ", "pdl_trigger")]
+    # who tells it: the launch of the sums, with the kernel's own flag, and the launch of the terms, right behind which the product comes
+    quant, mma = sources["qbp_quant.cu"], sources["qbp_mma.cu"]
+    assert quant.count("*beside = true") == 1 and "{ *beside = true; J.beside = 1; }" in quant
+    assert len(re.findall(r"\bbeside = true", mma)) == 1
+    assert "launch" not in re.sub(r"QBP_LAUNCH_OK", "", mma[mma.index("launch(conv_terms_kernel,") + 6:mma.index("beside = true")])
+
+
 def test_what_an_early_kernel_writes_is_read_by_ordinary_loads():
     """Code sums and zero-point terms: their reader is resident while they are written, which the non-coherent path excludes."""
     sources, kernels = _sources(), _kernels()
     at = _body(sources["qbp_mma.cuh"], sources["qbp_mma.cuh"].index("long long at(int64_t i) const"))
     assert "load_after_wait(" in at and "__ldg" not in at
     assert "__ldg" not in kernels["conv_terms_kernel"]   # (reads the code sums of the launch before)
-    for name in ("qbp_mma_kernel", "qbp_conv2_kernel", "qbp_mma2_kernel", "qbp_wgrad_kernel", "qbp_wgrad2_kernel"):
+    assert PRODUCTS <= {n for n, b in kernels.items() if "load_after_wait(" in b or ".at(" in b}
+    for name in PRODUCTS:
         for m in re.finditer(r"__ldg\(([^;]*);", kernels[name]):
             assert m.group(1).startswith("P.ep_fold"), (name, m.group(0))      # (written by bn_out_range_kernel)
 
 
+def _roles(name, body):
+    """A product's kernel (with its comments): what comes before the MMA issuer, the issuer, the epilogue, what ends the kernel."""
+    assert body.count("-- MMA issuer") == 1, name
+    issuer, epilogue = body.index("-- MMA issuer"), [m.start() for m in re.finditer(r"//\s-+ epilogue", body)]
+    end = body.rindex("if (timed_out) {")
+    assert len(epilogue) == 1 and issuer < epilogue[0] < end, name
+    cut = lambda a, b: re.sub(r"//[^\n]*", "", body[a:b])
+    return cut(0, issuer), cut(issuer, epilogue[0]), cut(epilogue[0], end), cut(end, len(body))
+
+
 def test_no_bounded_wait_starts_its_clock_before_the_kernel_may_work():
     """The waits on barriers give up after about a second.  Every role therefore waits for the kernels before this one, however
-    long those run, ahead of the first barrier that only completes once copies have been issued.  (The producer's first waits are
-    on stages that nothing has filled yet: they pass at once.)"""
-    sources = {f.name: f.read_text() for f in CSRC.glob("*.cu")}
-    seen = 0
-    for name, text in sources.items():
-        if "-- MMA issuer" not in text:
+    long those run, ahead of the first barrier that only completes once copies have been issued; the issuer of a product that runs
+    beside its sums need not, since its copies do not wait either.  (The producer's first waits are on stages that nothing has filled
+    yet: they pass at once.)"""
+    kernels = _kernels(comments=True)
+    assert {n for n, b in kernels.items() if "-- MMA issuer" in b} == PRODUCTS
+    waiting = r"mbar_wait|_mma_loop|mma_loop_|_dispatch"
+    for name in PRODUCTS:
+        before, issuer, epilogue, _ = _roles(name, kernels[name])
+        guard, = re.findall(r"(if \([^;]*\) )?pdl_wait\(\);", issuer)
+        assert guard in ("", "if (!P.beside) "), name
+        assert issuer.index("pdl_wait();") < re.search(waiting, issuer).start(), name
+        assert epilogue.index("pdl_wait();") < re.search(waiting, epilogue).start(), name
+        # (the roles that copy operands or read their parameters, under the same condition, at their first use)
+        working = [r for r in re.split(r"(?m)^    (?:\} else )?if \(warp", before)[1:] if re.search(r"tma_load|P\.qa->", r)]
+        assert working and all("pdl_wait();" in r for r in working), name
+        assert bool(guard) == all("P.beside" in r for r in working), name
+
+
+def test_a_product_beside_its_sums_waits_before_it_reads_them_or_writes():
+    """Its epilogue, unconditionally and first; nothing else reads sums or terms, or writes; the status word, which the launch before
+    may clear, is raised behind a wait as well."""
+    kernels, seen = _kernels(comments=True), 0
+    touching = r"load_after_wait\(|\.at\(|rowterm|colterm|tot_g|acc_out|P\.out\b|P\.dW|P\.mapC|st_sum|tma_store|st\.global|raise_timeout|atomicAdd"
+    for name in sorted(PRODUCTS):
+        before, issuer, epilogue, end = _roles(name, kernels[name])
+        wait = re.search(r"(?m)^\s*pdl_wait\(\);", epilogue)
+        assert wait and "{" not in re.sub(r"\{[^{}]*\}", "", epilogue[:wait.start()]), name      # (not inside a branch of the role)
+        assert not re.search(touching, epilogue[:wait.start()]), name
+        if "P.beside" not in kernels[name]:
             continue
-        issuer, epilogue = text.index("-- MMA issuer"), re.search(r"//\s-+ epilogue", text).start()
-        assert issuer < epilogue, name
-        waiting = r"mbar_wait|_mma_loop|mma_loop_|_dispatch"
-        for role in (text[issuer:epilogue], text[epilogue:]):
-            assert "pdl_wait();" in role, name
-            assert role.index("pdl_wait();") < re.search(waiting, role).start(), name
         seen += 1
-    assert seen == 5                                     # the products' files
+        for role in (re.sub(r"(if \([^;]*\) )?tma_prefetch_desc\([^;]*;", "", before), issuer):
+            assert not re.search(touching, role), (name, re.search(touching, role).group(0))
+        raised = end.index("raise_timeout(")
+        assert re.search(r"(?m)^\s*pdl_wait\(\);", end[:raised]), name
+    assert seen == 5
 
 
 def test_regions_to_clear_beyond_the_room_for_them_are_refused(tmp_path):
