@@ -281,7 +281,7 @@ int qbp_gemm_s8(int transA, int transB, int64_t M, int64_t N, int64_t K,
 
 /* qbp_gemm_s8 with the code sums along the reduction supplied by the caller
  * (the zero-point correction of Appendix B's scheme needs them; qbp_gemm_s8
- * computes them in two small kernels per call).  a_sums [M] (nullable): the
+ * computes them in a small kernel per call).  a_sums [M] (nullable): the
  * sum over k of the stored codes of row m of op(A); b_sums [N] (nullable): the
  * sum over k of column n of op(B); int32 (K <= 33025 codes always fit).  The
  * row_sums output of qbp_quantize_s8 / qbp_requant is a_sums of a

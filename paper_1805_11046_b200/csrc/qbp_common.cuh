@@ -43,10 +43,15 @@ void trace_end(const char *name, cudaStream_t st);
 // waits, before it touches the predecessor's results, until those are visible (pdl_wait).  A chain of dependent small kernels then
 // costs about 2 us each instead of 4 to 5.  Only the short kernels whose successor is a product (code sums and zero-point terms) let
 // it go while they run (pdl_trigger): elsewhere blocks that wait on an SM beside the running kernel made that kernel slower (per-channel
-// statistics of 51 MB 14.5 -> 20 us, the layer of 56 x 56 x 64 543 -> 577 us, three layers' inference at batch 8 106 -> 117 us).  They do
-// so behind their own wait: all that was launched before them is complete then, the product's operands and parameters among it, and
-// the product, told that its launch follows one of them (`beside`), starts on its operands at once; only its epilogue, which reads
-// the sums or terms and writes the output, waits for their end.  (Layer gradient of 16 x 7 x 7, 512 -> 512 channels, with its terms:
+// statistics of 51 MB 14.5 -> 20 us, the layer of 56 x 56 x 64 543 -> 577 us, three layers' inference at batch 8 106 -> 117 us).
+// There are two forms of it.
+//   - Terms always, and code sums whose launch was asked for it (SumJobs::beside, sums of 1 to 32 MB), let the product go behind their
+//     own wait: all that was launched before them is complete then, the product's operands and parameters among it.  The product is
+//     told so (`beside`) and starts on its operands at once; only its epilogue, which reads the sums or terms and writes the output,
+//     waits for their end, and so does whoever raises its status word, which they may clear.
+//   - Other code sums let it go at their start, ahead of their wait: the kernels before them may still run, so the product is not told
+//     and waits in every role before its first access; it has only set itself up by then (barriers, tensor memory, parameters).
+// Any other successor of either form waits like the second.  (Layer gradient of 16 x 7 x 7, 512 -> 512 channels, with its terms:
 // 27.6 -> 21.6 us; the layer of 20 x 19 x 19, 96 -> 160, 92.8 -> 91.2; the low-bit layer 196.5 -> 194.4.)
 // While launches are timed one by one the dependency is the ordinary one.
 bool trace_is_on();
@@ -109,7 +114,7 @@ struct WsCarver {
 // first two cases every block works out the parameters itself (about a microsecond, most of it behind its first loads;
 // a launch of its own for it costs two and more) and the first block leaves the records at qp8 / qp16 (each nullable).
 struct RangeSrc { const float2 *parts; int nparts; const qbp_qparams *given; qbp_qparams *qp8, *qp16; };
-// Regions of 32-bit words that a kernel clears on the way (a status word, sums that a later kernel adds to).
+// Regions of 32-bit words that a kernel clears on the way (a status word, sums that a later kernel adds to); one too many is an error.
 constexpr int kMaxZeroJobs = 5;
 struct ZeroJobs {
     int count;
@@ -126,11 +131,12 @@ struct ZeroJobs {
 // -------------------------------------------------------------- device side
 #ifdef __CUDACC__
 
-// The two halves of a programmatic launch (see launch()).  Only code_sums_kernel and conv_terms_kernel trigger, behind their wait.  A kernel that
-// allocates tensor memory never does: its successor could take that memory first and then wait for a kernel that cannot go on.
+// The two halves of a programmatic launch (see launch()).  Only code_sums_kernel and conv_terms_kernel trigger: the terms behind their
+// wait, the sums behind or ahead of it.  A kernel that allocates tensor memory never does: its successor could take that memory first
+// and then wait for a kernel that cannot go on.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// A load of what a kernel that let this one go at its start writes (code sums, zero-point terms): an ordinary global load that
+// A load of what a kernel that let this one go while it ran writes (code sums, zero-point terms): an ordinary global load that
 // stays behind pdl_wait().  __ldg would take the non-coherent path, which is for memory that nothing writes while the reading
 // kernel is resident; everything else that a kernel reads was written by blocks that had ended before it started.
 __device__ __forceinline__ int32_t load_after_wait(const int32_t *p)

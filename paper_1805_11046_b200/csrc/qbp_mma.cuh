@@ -54,8 +54,8 @@ inline CodeSums sums_of(const SumJob &j)
     return j.kind == kSumRows ? sums_of(j.out) : CodeSums{j.out, sum_pieces(j.rows, j.cols), j.cols};
 }
 // beside (nullable): set when the product launched next may run beside this kernel (see launch()).  Sums of fewer than a megabyte
-// take a microsecond or two, less than the product's launch: they let it go at their start, and it waits for them.  Sums of more than
-// 32 want HBM for themselves (weight gradient 8192 x 2048 x 4096 with its 67 MB 123.7 us beside them, 122.8 behind; linear layer
+// take a microsecond or two, less than the product's launch, and sums of more than 32 want HBM for themselves: both let it go at their
+// start, ahead of their own wait, and it waits for them in every role (weight gradient 8192 x 2048 x 4096 with its 67 MB 123.7 us beside them, 122.8 behind; linear layer
 // 1024 x 2048 -> 1008 with 4 MB 77.6 and 78.3).
 constexpr int64_t kSumsBesideMin = 1 << 20, kSumsBesideMax = 32 << 20;
 int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st, const ZeroJobs &zero = ZeroJobs{}, bool *beside = nullptr);

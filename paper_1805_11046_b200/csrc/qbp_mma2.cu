@@ -371,7 +371,7 @@ int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const 
     const uint32_t stage_bytes = P.a.tile_bytes * P.msub + P.b.tile_bytes;  // 20, 24, 32 or 48 KB
     int stages = (int)((k2Smem - 1024 - k2EpiWarps * k2Slab) / stage_bytes);
     stages = std::min(stages, k2MaxStages);
-    P.cg = 2;                           // sixteen (msub 2) or eight pair MMAs, 1024 cycles or more, between commits
+    P.cg = 2;                           // sixteen (msub 2) or eight pair MMAs between commits: 2048 or 1024 cycles, of 128 and 64 columns 512 and 256
     stages -= stages % P.cg;
     if (stages < 2 * P.cg) return fail(QBP_ERR_UNSUPPORTED_SHAPE, "gemm_s8: the pair kernel's ring does not fit");
     P.stages = stages;

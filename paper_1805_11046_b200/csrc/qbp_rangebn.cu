@@ -22,8 +22,10 @@ namespace qbp {
 // last: its rows from keep_from on (kKeepBytes of what the second pass reads), with loads that leave the lines there; the rest passes
 // through, evict-first, and so does all that the second passes read for the last time and write.  A forward's second pass leaves
 // the head of x for the backward of the same call site in the same way (keep_head).  Forward + backward, with the forward's pass
-// from the front and all of its loads evict-first, the backward's from the front with ordinary loads and stores, and so: 50176 x 256
-// 86.5 -> 72.4 us, 802816 x 64 272.5 -> 261.5, 12544 x 2048 151.6 -> 139.0.  48, 88 or 104 MB: within 0.5 us.
+// from the front and all of its loads evict-first, the backward's from the front with ordinary loads and stores, and so, on the same
+// buffers again and again: 50176 x 256 86.5 -> 72.4 us, 802816 x 64 272.5 -> 261.5, 12544 x 2048 151.6 -> 139.0; alone on inputs that
+// another kernel has just written 84.0 -> 73.8, 272.4 -> 264.2, 151.6 -> 141.3, on ones out of HBM 94.2 -> 77.8, 280.6 -> 268.3, 157.7 ->
+// 145.4.  48, 88 or 104 MB: within 0.5 us.
 constexpr int64_t kKeepBytes = 64ll << 20;
 static int64_t keep_from_row(int64_t rows, int64_t row_bytes) { return std::max<int64_t>(0, rows - kKeepBytes / row_bytes); }
 
