@@ -1263,7 +1263,7 @@ int qbp::gemm_s8_impl(int transA, int transB, int64_t M, int64_t N, int64_t K, c
     ZeroJobs zero{};
     if (!ext_status && (rc = zero.add(status, 1))) return rc;
     bool own = false;
-    if ((rc = launch_code_sums(jobs, njobs, st, zero, &own))) return rc;
+    if ((rc = launch_code_sums(jobs, njobs, st, zero, has_tail ? nullptr : &own))) return rc;
     beside = njobs ? own : beside && !zero.count;         // (a tail's launch for its parameters comes in between)
 
     // large and deep products run on CTA pairs (tiles across two SMs); the column statistics are the

@@ -756,11 +756,12 @@ __global__ void __launch_bounds__(kThreads) clear_kernel(const __grid_constant__
 }
 
 // The sums of up to eight code tensors in a launch of their own (see qbp_sums.cuh).
+template <bool BESIDE>
 __global__ void __launch_bounds__(kSumThreads) code_sums_kernel(const __grid_constant__ SumJobs J)
 {
-    if (!J.beside) pdl_trigger();        // (see launch())
+    if (!BESIDE) pdl_trigger();          // (see launch(); without a look at a parameter, which cost every small product 0.3 us)
     pdl_wait();
-    if (J.beside) pdl_trigger();
+    if (BESIDE) pdl_trigger();
     run_zero_jobs(J.zero, (int64_t)blockIdx.x * kSumThreads + threadIdx.x, (int64_t)gridDim.x * kSumThreads);
     code_sums_block(J, (int)blockIdx.x);
 }
@@ -850,9 +851,11 @@ int launch_code_sums(const SumJob *jobs, int count, cudaStream_t st, const ZeroJ
     J.zero = zero;
     int64_t bytes = 0;
     for (int i = 0; i < count; ++i) bytes += jobs[i].rows * jobs[i].cols;
-    if (beside && bytes >= kSumsBesideMin && bytes <= kSumsBesideMax) { *beside = true; J.beside = 1; }
+    const bool ahead = beside && bytes >= kSumsBesideMin && bytes <= kSumsBesideMax;
+    if (beside) *beside = ahead;
     QBP_TRACE_BEGIN(st);
-    launch(code_sums_kernel, blocks, kSumThreads, 0, st, J);
+    if (ahead) launch(code_sums_kernel<true>, blocks, kSumThreads, 0, st, J);
+    else       launch(code_sums_kernel<false>, blocks, kSumThreads, 0, st, J);
     QBP_LAUNCH_OK("code_sums_kernel");
     return QBP_OK;
 }

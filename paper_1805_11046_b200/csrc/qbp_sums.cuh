@@ -9,7 +9,7 @@ namespace qbp {
 
 constexpr int kSumThreads = 256;
 struct SumJobDev { const uint8_t *q; int64_t rows; int cols, kind, first, blocks, G, pieces, corner_pieces, H, W, lg_log2; uint32_t flip; int32_t *out; int64_t *out64; };
-struct SumJobs { SumJobDev j[kMaxSumJobs]; int count, beside; ZeroJobs zero; };
+struct SumJobs { SumJobDev j[kMaxSumJobs]; int count; ZeroJobs zero; };
 // The device form of `count` jobs; *blocks: the blocks they take.  (qbp_quant.cu)
 int fill_sum_jobs(const SumJob *jobs, int count, SumJobs &J, int *blocks);
 

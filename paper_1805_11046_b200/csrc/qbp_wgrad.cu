@@ -993,7 +993,7 @@ int qbp::wgrad_s16_impl(const qbp_conv_desc *d, int64_t M, int64_t N, int64_t K,
         }
     }
     bool beside = false;
-    if ((rc = launch_code_sums(jobs, njobs, st, zero, &beside))) return rc;
+    if ((rc = launch_code_sums(jobs, njobs, st, zero, pair_kernel ? &beside : nullptr))) return rc;      // (the single-CTA kernel waits)
     if (pair_kernel)
         return launch_wgrad2(M, N, K, x, qx, g_hi, g_lo, qg16, acc_out, dW, P.sx, P.shi, P.slo, plain_tot_g, status, beside, st, lo_signed);
     if (!d) P.tot_g = (const long long *)plain_tot_g;

@@ -60,10 +60,11 @@ def test_a_successor_that_does_not_wait_starts_behind_the_wait_of_the_kernel_bef
     kernels, sources = _kernels(), _sources()
     steps = lambda name: re.findall(r"(if \([^;]*?\) )?(pdl_trigger|pdl_wait)\(\)", kernels[name])
     assert steps("conv_terms_kernel") == [("", "pdl_wait"), ("", "pdl_trigger")]
-    assert steps("code_sums_kernel") == [("if (!J.beside) ", "pdl_trigger"), ("", "pdl_wait"), ("if (J.beside) ", "pdl_trigger")]
-    # who tells it: the launch of the sums, with the kernel's own flag, and the launch of the terms, right behind which the product comes
+    assert steps("code_sums_kernel") == [("if (!BESIDE) ", "pdl_trigger"), ("", "pdl_wait"), ("if (BESIDE) ", "pdl_trigger")]
+    # who tells it: the launch of the sums, with the kernel's own form, and the launch of the terms, right behind which the product comes
     quant, mma = sources["qbp_quant.cu"], sources["qbp_mma.cu"]
-    assert quant.count("*beside = true") == 1 and "{ *beside = true; J.beside = 1; }" in quant
+    assert quant.count("*beside = ahead") == 1 and quant.count("*beside =") == 2
+    assert "if (ahead) launch(code_sums_kernel<true>," in quant and "else       launch(code_sums_kernel<false>," in quant
     assert len(re.findall(r"\bbeside = true", mma)) == 1
     assert "launch" not in re.sub(r"QBP_LAUNCH_OK", "", mma[mma.index("launch(conv_terms_kernel,") + 6:mma.index("beside = true")])
 
