@@ -335,10 +335,11 @@ int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const 
     int rc;
     // Tiles.  512 x 256 pair tiles (two accumulators per CTA fill tensor memory: no second set) cut the operand bytes per
     // multiply-add by a quarter against 256 x 256: a round of them over the pairs takes 3 units of fetching, one of 256 x 256
-    // takes 2, and the fewer units win (on a tie the large tiles from 1024 reduction bytes, whose epilogues the next tile cannot
-    // hide).  Call with its sums, large tiles from 2048 rows on -> by this rule: 2304 x 4096 x 2048 38.0 -> 26.9 us (128 small
-    // tiles), 1024 x 8192 x 1024 21.4 -> 19.1 (64 large ones), 1536 x 8192 x 256 19.9 (a tie; large: 20.6).  Where tiles of
-    // 256 x 256 fit the pairs once, they and tiles of half as many columns (64 at least) as long as they do: rings and epilogues
+    // takes 2, and the fewer units win; on a tie the small ones, whose epilogues the next tile hides (1488 x 7232 x 5824 with B
+    // transposed 70.0 us, large tiles 81.0; 2368 x 5216 x 8192 88.0 and 100.4), but for A transposed alone up to 4096 reduction bytes
+    // (4320 x 3328 x 2048 43.8 and 41.9; 1696 x 7680 x 6144 74.8 and 85.4).  Call with its sums, large tiles from 2048 rows on -> by
+    // this rule: 2304 x 4096 x 2048 38.0 -> 26.9 us (128 small tiles), 1024 x 8192 x 1024 21.4 -> 19.1 (64 large ones).  Where tiles
+    // of 256 x 256 fit the pairs once, they and tiles of half as many columns (64 at least) as long as they do: rings and epilogues
     // get shorter, and SMs that had none take part.  Times of a call with its sums, 256 or 512 rows by 256 -> by this rule:
     // 4096 x 256 x 1024 15.4 -> 9.8 us, 2048 x 2048 x 2048 20.2 -> 15.3, 4096 x 1024 x 4096 30.0 -> 21.8, 1024 x 1024 x 1024
     // 11.3 -> 9.5; the same where it changes nothing (2048 x 2560 x 1024: 16.6).  Of outputs of at most 128 columns whose row tiles
@@ -350,7 +351,7 @@ int launch_gemm2(int transA, int transB, int64_t M, int64_t N, int64_t K, const 
     const auto rounds = [&](int64_t m) { return (tiles_of(m, 256) + pairs - 1) / pairs; };
     P.bn = N <= 64 ? 64 : N <= 128 ? 128 : 256;
     if (P.bn < 256 && 6 * (128 + P.bn / 2) * rounds(256) >= 5 * 384 * rounds(512)) P.bn = 256;
-    P.msub = P.bn == 256 && tiles_of(256, 256) > pairs && 3 * rounds(512) < 2 * rounds(256) + (K >= 1024) ? 2 : 1;
+    P.msub = P.bn == 256 && tiles_of(256, 256) > pairs && 3 * rounds(512) < 2 * rounds(256) + (transA && !transB && K < 4096) ? 2 : 1;
     while (P.msub == 1 && P.bn > 64 && tiles_of(256, P.bn / 2) <= pairs) P.bn /= 2;
     // per-CTA operand halves: 128 rows of A, bn / 2 columns of B, 128 reduction bytes per stage
     const uint32_t half = (uint32_t)P.bn / 2;

@@ -592,12 +592,12 @@ def test_gemm_tiles_that_fit_the_machine_once(B, M, N, K, tB):
     assert np.array_equal(to_host(acc), oacc) and np.array_equal(to_host(out), oout)
 
 
-@pytest.mark.parametrize("M,N,K", [(18960, 64, 1040), (18960, 128, 1040), (37904, 64, 1040), (37904, 112, 1040), (37904, 144, 1040), (65520, 64, 1024),
+@pytest.mark.parametrize("M,N,K", [(2400, 3600, 1040), (2400, 3600, 4096), (18960, 64, 1040), (18960, 128, 1040), (37904, 64, 1040), (37904, 112, 1040), (37904, 144, 1040), (65520, 64, 1024),
                                    (65536, 64, 1024), (65536, 80, 1024)])
 @pytest.mark.parametrize("tA,tB", [(False, False), (False, True), (True, False)])
 def test_gemm_pair_kernel_more_row_tiles_than_pairs(B, M, N, K, tA, tB):
     """Outputs whose 256-row tiles alone do not fit the SM pairs once: 512 x 256 tiles, 256-row tiles as wide as the columns, the
-    single-CTA kernel; sampled rows, those at the edges of the first and last tiles among them."""
+    single-CTA kernel; first, two of as many rounds' worth of large as of small tiles; sampled rows, those at the edges of the first and last tiles among them."""
     rows = np.unique(np.concatenate([[0, 127, 128, 255, 256, 511, 512, M - 1, M - 16, M - 17, M // 512 * 512 - 1, M // 256 * 256 - 1],
                                      np.random.Generator(np.random.PCG64(66)).integers(0, M, 120)]))
     A = random_codes((M, K), 67); Bm = random_codes((N, K) if tB else (K, N), 68)
