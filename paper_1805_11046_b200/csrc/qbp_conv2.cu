@@ -420,8 +420,9 @@ int launch_conv2(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp
 // The same products where nobody wants the statistics of their output (layer gradients, the low-bit layer, plain calls).
 //
 // The accumulator's rows (tensor-memory lanes) are output channels, its columns output positions: the filter is the A operand and
-// the activation the B operand.  A tile is 256 channels x npos positions on a CTA pair (CTA r holds 128 channels of the filter, half
-// of the positions and the accumulator of its channels) or 128 channels x npos positions on a CTA of its own, npos at most 256.
+// the activation the B operand.  A tile is 128 channels x npos positions, npos at most 256, on a CTA of its own.  (Pairs of CTAs with
+// 256 channels, half of the positions' window each, were hardly faster where the products are long, 60 x 40 x 40, 512 -> 512 channels
+// 168 against 170 us, and slower nearly everywhere else, in the mean of 980 shapes by 8 %: 2 x 17 x 17, 256 -> 256 14.9 against 13.1.)
 // An epilogue thread then owns a channel: the channel's zero-point term is a register, a position's a broadcast, and a position's 32
 // channels of a warp go out as one 128-byte line, where positions as rows stage every value in shared memory beside the operand
 // reads and copies that want its port.  (Statistics would stay in registers too, but in sums of other 32 values: the mean's last
@@ -435,8 +436,8 @@ int launch_conv2(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp
 // code, so that it adds zero to every corrected sum and one term per channel serves all positions.
 // What bounds it: the operand bytes that all SMs together draw from the L2 (some 10 TB/s; 128 filter rows and a ninth of the window
 // per tap against 128 + bn / 2 rows above), then the epilogue's instructions; the MMAs of a tile run at the pipe's rate.  Measured
-// with the terms' kernel, before and after: 256 x 28 x 28, 128 -> 128 channels 55.5 -> 44.4 us, 8 x 40 x 40, 288 -> 288 37.8 -> 29.4,
-// 20 x 19 x 19, 160 -> 96 16.2 -> 14.3, 16 x 7 x 7, 512 -> 512 21.6 -> 18.5, 1024 x 1 x 1, 256 -> 256 16.3 -> 13.1.
+// with the terms' kernel, before and after: 256 x 28 x 28, 128 -> 128 channels 55.7 -> 44.6 us, 8 x 40 x 40, 288 -> 288 37.9 -> 26.2,
+// 20 x 19 x 19, 160 -> 96 16.2 -> 12.8, 16 x 7 x 7, 512 -> 512 21.8 -> 17.2, 30 x 17 x 17, 512 -> 512 38.7 -> 29.7.
 //
 // Roles per CTA: warp 0 copies filter tiles, warp 18 windows, warp 19 fills their padding, warp 1 issues the MMAs, warps 2..17 are
 // the epilogue.  Every wait is bounded; no TMA load uses cluster multicast.
@@ -466,10 +467,10 @@ struct ConvTParams {
     uint32_t f_desc_lo, x_desc_lo, idesc;
     uint32_t window_bytes, window_start;       // room of a window; where its first number lies (the row it is in starts up to s - 1 before)
     int dgrad;
-    int npos, npos_cta;              // positions of a tile, of a CTA's window
+    int npos;                        // positions of a tile
     int stages, windows;             // ring stages of a tap row's filter tiles; windows in flight
     int cchunks;                     // channel chunks of 128 (of a ragged last one the rest is zero on the activation side)
-    int tiles_n, tiles_total, units; // units (pairs or CTAs): a multiple of tiles_n, so that a unit meets one channel tile only
+    int tiles_n, tiles_total, units; // units (CTAs): a multiple of tiles_n, so that a unit meets one channel tile only
     FastDiv d_tiles_n;
     ConvTGrid g;
     int Nimg, H, W, C, N, Cred;      // C: channels of the filter's innermost extent; N: channels produced
@@ -485,7 +486,7 @@ struct ConvTParams {
 // constants and a tap's MMAs are unrolled.  With a tap's place in the window and in the filter's ring worked out per tap from
 // the parameters, four MMAs of 64 cycles took the warp 750.
 // The MMAs of one tap, in column T of COLS: 128 reduction channels.
-template <bool PAIR, bool DGRAD, int T, int COLS, bool FIRST>
+template <bool DGRAD, int T, int COLS, bool FIRST>
 __device__ __forceinline__ void convt_issue_tap(uint32_t d_tmem, uint32_t f_lo, uint32_t x_lo, uint32_t idesc)
 {
     constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);           // 128-byte swizzle, groups of eight rows 1024 bytes apart
@@ -495,10 +496,7 @@ __device__ __forceinline__ void convt_issue_tap(uint32_t d_tmem, uint32_t f_lo, 
     for (uint32_t kk = 0; kk < 4; ++kk) {
         const uint64_t f = ((uint64_t)hi << 32) | (uint64_t)(f_lo + T * (kCtTapBytes >> 4) + kk * f_kstep);
         const uint64_t x = ((uint64_t)hi << 32) | (uint64_t)(x_lo + col * 8u + kk * 2u);
-        if (elect_one()) {
-            if (PAIR) mma_i8_pair(d_tmem, f, x, idesc, (FIRST && kk == 0) ? 0u : 1u);
-            else      mma_i8(d_tmem, f, x, idesc, (FIRST && kk == 0) ? 0u : 1u);
-        }
+        if (elect_one()) mma_i8(d_tmem, f, x, idesc, (FIRST && kk == 0) ? 0u : 1u);
     }
 }
 
@@ -510,13 +508,8 @@ struct ConvTMmaArgs {
     uint32_t stages, windows;
     int tile0, tiles_total, tile_step;
 };
-template <bool PAIR>
-__device__ __forceinline__ void convt_commit(uint64_t *bar)
-{
-    if (elect_one()) { if (PAIR) mma_commit_pair(bar); else mma_commit(bar); }
-}
 // False when a wait ran out.
-template <bool PAIR, bool DGRAD, int COLS>
+template <bool DGRAD, int COLS>
 __device__ __forceinline__ bool convt_mma_loop(const ConvTMmaArgs &A)
 {
     constexpr uint32_t stage_bytes = kCtTapBytes * COLS;
@@ -533,26 +526,26 @@ __device__ __forceinline__ bool convt_mma_loop(const ConvTMmaArgs &A)
                 const uint32_t f_lo = ((f_addr >> 4) & 0x3FFFu) | A.f_desc_lo;
                 if (!mbar_wait_uniform(&A.full_bar[3 * s], ph)) return false;
                 tc_fence_after();
-                if (first) convt_issue_tap<PAIR, DGRAD, 0, COLS, true>(d_tmem, f_lo, x_lo, A.idesc);
-                else       convt_issue_tap<PAIR, DGRAD, 0, COLS, false>(d_tmem, f_lo, x_lo, A.idesc);
+                if (first) convt_issue_tap<DGRAD, 0, COLS, true>(d_tmem, f_lo, x_lo, A.idesc);
+                else       convt_issue_tap<DGRAD, 0, COLS, false>(d_tmem, f_lo, x_lo, A.idesc);
                 first = false;
                 if (COLS == 3) {
                     if (!mbar_wait_uniform(&A.full_bar[3 * s + 1], ph)) return false;
                     tc_fence_after();
-                    convt_issue_tap<PAIR, DGRAD, COLS == 3 ? 1 : 0, COLS, false>(d_tmem, f_lo, x_lo, A.idesc);
+                    convt_issue_tap<DGRAD, COLS == 3 ? 1 : 0, COLS, false>(d_tmem, f_lo, x_lo, A.idesc);
                     if (!mbar_wait_uniform(&A.full_bar[3 * s + 2], ph)) return false;
                     tc_fence_after();
-                    convt_issue_tap<PAIR, DGRAD, COLS == 3 ? 2 : 0, COLS, false>(d_tmem, f_lo, x_lo, A.idesc);
+                    convt_issue_tap<DGRAD, COLS == 3 ? 2 : 0, COLS, false>(d_tmem, f_lo, x_lo, A.idesc);
                 }
-                convt_commit<PAIR>(&A.empty_bar[s]);
+                if (elect_one()) mma_commit(&A.empty_bar[s]);
                 f_addr += stage_bytes;
                 if (++s == A.stages) { s = 0; ph ^= 1u; f_addr = A.ring; }
             }
-            convt_commit<PAIR>(&A.win_empty[win]);
+            if (elect_one()) mma_commit(&A.win_empty[win]);
             w_addr += A.window_bytes;
             if (++win == A.windows) { win = 0; wph ^= 1u; w_addr = A.windows_at; }
         }
-        convt_commit<PAIR>(&A.acc_full[buf]);
+        if (elect_one()) mma_commit(&A.acc_full[buf]);
         buf ^= 1u;
         if (buf == 0) bph ^= 1u;
     }
@@ -568,18 +561,17 @@ __device__ __forceinline__ void put_if(unsigned cond, uint32_t bits, char *&p, i
 
 // The image rows (of s numbers, counted through all panels, -1 the one before the first) that a CTA's window of a tile touches.
 struct ConvTRows { int first, count, start; };       // start: the window's first number
-__device__ __forceinline__ ConvTRows convt_rows(const ConvTParams &P, int tile_m, uint32_t rank)
+__device__ __forceinline__ ConvTRows convt_rows(const ConvTParams &P, int tile_m)
 {
     ConvTRows w;
     const int reach = P.g.pr * P.g.s + P.g.pc;
-    w.start = tile_m * P.npos + P.npos_cta * (int)rank - reach;
+    w.start = tile_m * P.npos - reach;
     w.first = P.g.d_s.div(w.start + 2 * P.g.s) - 2;                      // (reach <= 2 s)
-    w.count = P.g.d_s.div(w.start + P.npos_cta - 1 + 2 * reach + 2 * P.g.s) - 2 - w.first + 1;
+    w.count = P.g.d_s.div(w.start + P.npos - 1 + 2 * reach + 2 * P.g.s) - 2 - w.first + 1;
     return w;
 }
 
-template <bool PAIR>
-__global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(kCtThreads, 1) qbp_conv2t_kernel(const __grid_constant__ ConvTParams P)
+__global__ void __launch_bounds__(kCtThreads, 1) qbp_conv2t_kernel(const __grid_constant__ ConvTParams P)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t full_bar[3 * kCtMaxStages], empty_bar[kCtMaxStages], win_landed[kCtMaxWindows], win_full[kCtMaxWindows],
@@ -592,29 +584,20 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(kCtThread
     const uint32_t stage_bytes = kCtTapBytes * (P.g.pc ? 3u : 1u);
     CtEpiShared &E = *reinterpret_cast<CtEpiShared *>(ring + (size_t)P.stages * stage_bytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
-    const int unit = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
-    const int n_mine = (unit % P.tiles_n) * (PAIR ? 256 : 128) + 128 * (int)rank;                     // this CTA's first channel
-    constexpr uint32_t kCtas = PAIR ? 2u : 1u;
+    const int unit = (int)blockIdx.x, n_mine = (unit % P.tiles_n) * 128;                              // this CTA's first channel
 
     if (threadIdx.x == 0) {
-        // (pairs: the leader's "full" barriers count its own arrival and the bytes of both CTAs, "win_full" a window of each CTA, the
-        // "empty" ones a multicast commit, "acc_empty" the epilogue warps of both)
         for (int s = 0; s < P.stages; ++s) { for (int t = 0; t < 3; ++t) mbar_init(&full_bar[3 * s + t], 1); mbar_init(&empty_bar[s], 1); }
-        for (int w = 0; w < P.windows; ++w) { mbar_init(&win_landed[w], 1); mbar_init(&win_full[w], kCtas); mbar_init(&win_empty[w], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], kCtas * kCtEpiWarps); }
+        for (int w = 0; w < P.windows; ++w) { mbar_init(&win_landed[w], 1); mbar_init(&win_full[w], 1); mbar_init(&win_empty[w], 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], kCtEpiWarps); }
         mbar_fence_init();
         tma_prefetch_desc(&P.mapF);
         for (int b = 0; b < kCtBoxHeights; ++b)
             if ((8 >> b) <= P.H) tma_prefetch_desc(&P.mapX[b]);
     }
-    if (warp == 1) {
-        if (PAIR) { tmem_alloc_pair(&tmem_slot, 512); tmem_relinquish_pair(); }
-        else      { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
-    }
+    if (warp == 1) { tmem_alloc(&tmem_slot, 512); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
-    if (PAIR) cluster_sync_all();        // both CTAs' barriers are initialised before either signals the other
     tc_fence_after();
     // (each role waits for the kernels before at its first use of their results: what it needs of the launch's parameters, and the
     // code up to there, has then been fetched)
@@ -625,7 +608,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(kCtThread
 
     if (warp == 0) {
         if (lane == 0) {
-            // ---------------------------------------------------- TMA producer of the filter tiles (both CTAs)
+            // ---------------------------------------------------- TMA producer of the filter tiles
             bool waited = false;
             uint32_t s = 0, ph = 1;
             for (int tile = unit; tile < P.tiles_total && !timed_out; tile += P.units)
@@ -637,11 +620,10 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(kCtThread
                         for (int t = t0; t < t1; ++t) {
                             uint8_t *dst = ring + (size_t)s * stage_bytes + (uint32_t)(t - t0) * kCtTapBytes;
                             uint64_t *bar = &full_bar[3 * s + (uint32_t)(t - t0)];
-                            if (rank == 0) mbar_expect_tx(bar, kCtas * kCtTapBytes);
+                            mbar_expect_tx(bar, kCtTapBytes);
                             const int at = (3 * r + t) * P.C;
                             const int x = P.dgrad ? at + n_mine : at + c0, y = P.dgrad ? c0 : n_mine;
-                            if (PAIR) tma_load_2d_pair(dst, &P.mapF, map_to_cta(bar, 0), x, y);
-                            else      tma_load_2d(dst, &P.mapF, bar, x, y);
+                            tma_load_2d(dst, &P.mapF, bar, x, y);
                         }
                         if (++s == (uint32_t)P.stages) { s = 0; ph ^= 1u; }
                     }
@@ -652,7 +634,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(kCtThread
         bool waited = P.beside != 0;
         const int s = P.g.s;
         for (int tile = unit; tile < P.tiles_total && !timed_out; tile += P.units) {
-            const ConvTRows w = convt_rows(P, P.d_tiles_n.div(tile), rank);
+            const ConvTRows w = convt_rows(P, P.d_tiles_n.div(tile));
             const int v0 = P.g.d_hp.div(w.first + P.g.hp) - 1, v1 = P.g.d_hp.div(w.first + w.count - 1 + P.g.hp) - 1;    // panels, -1 the one before the first
             // (the rows behind the panels v0 .. that the window touches are not copied)
             const int padding = P.g.pr ? P.g.d_hp.div(w.first + w.count + P.g.hp) - 1 - v0 : 0;
@@ -687,7 +669,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(kCtThread
         if (!P.beside) pdl_wait();
         zz = ((uint32_t)P.qa->zero_point & 0xFFu) * 0x01010101u;
         for (int tile = unit; tile < P.tiles_total && !timed_out; tile += P.units) {
-            const ConvTRows w = convt_rows(P, P.d_tiles_n.div(tile), rank);
+            const ConvTRows w = convt_rows(P, P.d_tiles_n.div(tile));
             int h0 = 0;
             if (P.g.pr) { int v; P.g.d_hp.divmod(w.first + P.g.hp, v, h0); }
             for (int cc = 0; cc < P.cchunks; ++cc) {
@@ -718,32 +700,27 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(kCtThread
                         for (int u = lane; u < 8 * s; u += 32) pad(base + (uint32_t)(i * s + (u >> 3)) * 128u, u & 7);
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) {
-                    if (PAIR) mbar_arrive_cluster(map_to_cta(&win_full[win], 0));
-                    else      mbar_arrive(&win_full[win]);
-                }
+                if (lane == 0) mbar_arrive(&win_full[win]);
                 if (++win == (uint32_t)P.windows) { win = 0; ph ^= 1u; }
             }
         }
     } else if (warp == 1) {
-        if (rank == 0) {
-            // ---------------------------------------------------- MMA issuer (a pair's leader only): the whole warp in step
-            ConvTMmaArgs A;
-            A.full_bar = full_bar; A.empty_bar = empty_bar; A.win_full = win_full; A.win_empty = win_empty; A.acc_full = acc_full; A.acc_empty = acc_empty;
-            A.windows_at = smem_u32(windows); A.window_bytes = P.window_bytes; A.window_start = P.window_start;
-            A.ring = smem_u32(ring); A.tmem = tmem_base; A.f_desc_lo = P.f_desc_lo; A.x_desc_lo = P.x_desc_lo; A.idesc = P.idesc;
-            A.cchunks = P.cchunks; A.stages = (uint32_t)P.stages; A.windows = (uint32_t)P.windows;
-            // forward: input (p - 1 + r, q - 1 + t) feeds output (p, q); layer gradient: gradient (h + 1 - r, w + 1 - t) feeds input (h, w)
-            A.tap_rows = r1 - r0;
-            A.tap0 = P.dgrad ? 16 * P.g.pr * P.g.s : 0;
-            A.row_step = P.dgrad ? -8 * P.g.s : 8 * P.g.s;
-            A.tile0 = unit; A.tiles_total = P.tiles_total; A.tile_step = P.units;
-            // (a barrier's wait is bounded: its clock starts once the producers' copies can)
-            if (!P.beside) pdl_wait();
-            const bool ok = t1 - t0 == 1 ? (P.dgrad ? convt_mma_loop<PAIR, true, 1>(A) : convt_mma_loop<PAIR, false, 1>(A))
-                                         : (P.dgrad ? convt_mma_loop<PAIR, true, 3>(A) : convt_mma_loop<PAIR, false, 3>(A));
-            timed_out = !ok;
-        }
+        // ------------------------------------------------------ MMA issuer: the whole warp in step
+        ConvTMmaArgs A;
+        A.full_bar = full_bar; A.empty_bar = empty_bar; A.win_full = win_full; A.win_empty = win_empty; A.acc_full = acc_full; A.acc_empty = acc_empty;
+        A.windows_at = smem_u32(windows); A.window_bytes = P.window_bytes; A.window_start = P.window_start;
+        A.ring = smem_u32(ring); A.tmem = tmem_base; A.f_desc_lo = P.f_desc_lo; A.x_desc_lo = P.x_desc_lo; A.idesc = P.idesc;
+        A.cchunks = P.cchunks; A.stages = (uint32_t)P.stages; A.windows = (uint32_t)P.windows;
+        // forward: input (p - 1 + r, q - 1 + t) feeds output (p, q); layer gradient: gradient (h + 1 - r, w + 1 - t) feeds input (h, w)
+        A.tap_rows = r1 - r0;
+        A.tap0 = P.dgrad ? 16 * P.g.pr * P.g.s : 0;
+        A.row_step = P.dgrad ? -8 * P.g.s : 8 * P.g.s;
+        A.tile0 = unit; A.tiles_total = P.tiles_total; A.tile_step = P.units;
+        // (a barrier's wait is bounded: its clock starts once the producers' copies can)
+        if (!P.beside) pdl_wait();
+        const bool ok = t1 - t0 == 1 ? (P.dgrad ? convt_mma_loop<true, 1>(A) : convt_mma_loop<false, 1>(A))
+                                     : (P.dgrad ? convt_mma_loop<true, 3>(A) : convt_mma_loop<false, 3>(A));
+        timed_out = !ok;
     } else {
         // ------------------------------------------------------- epilogue (each CTA drains its own 128 channels; the four groups
         // of four warps split the chunks of 16 positions)
@@ -755,11 +732,10 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(kCtThread
         const float scale = __fmul_rn(P.qa->scale, P.qb->scale);
         // (the taps that are left out of an image of one row or column: the border class without them)
         const int cterm = ch_in ? load_after_wait(P.colterm + (int64_t)((P.g.pr ? 0 : 3) | (P.g.pc ? 0 : 12)) * P.N + ch) : 0;
-        const uint32_t leader_empty = PAIR ? map_to_cta(&acc_empty[0], 0) : 0u;          // (8 bytes a barrier)
         auto hand_back = [&](uint32_t buf) {
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) { if (PAIR) mbar_arrive_cluster(leader_empty + 8u * buf); else mbar_arrive(&acc_empty[buf]); }
+            if (lane == 0) mbar_arrive(&acc_empty[buf]);
         };
 
         // The positions of this warp's chunks of a tile, two a lane: where they lie in the output (padding: nowhere), their terms.
@@ -855,11 +831,7 @@ __global__ void __cluster_dims__(PAIR ? 2 : 1, 1, 1) __launch_bounds__(kCtThread
     }
     tc_fence_before();
     __syncthreads();
-    if (PAIR) cluster_sync_all();        // neither CTA retires while the other may still read its memory or signal it
-    if (warp == 1) {
-        __syncwarp();
-        if (PAIR) tmem_dealloc_pair(tmem_base, 512); else tmem_dealloc(tmem_base, 512);
-    }
+    if (warp == 1) { __syncwarp(); tmem_dealloc(tmem_base, 512); }
 }
 
 static ConvTGrid convt_grid(const qbp_conv_desc *d)
@@ -873,45 +845,44 @@ static ConvTGrid convt_grid(const qbp_conv_desc *d)
     return g;
 }
 
-// The tile: on pairs or not, and its positions.  A model of the launch in cycles per SM, the cheapest wins: rounds of tiles x (taps x
-// chunks x the longest of the MMAs (2 cycles per position and tap), the copies (3 per operand row) and shared memory's port (128
-// bytes a cycle for operand reads and copies) + a tile's overhead) + the last tile's epilogue.
+// The tile's positions.  A model of the launch in cycles per SM, the cheapest wins: rounds of tiles x (taps x chunks x the longest of
+// the MMAs (2 cycles per position and tap), the copies (3 per operand row) and shared memory's port (128 bytes a cycle for operand
+// reads and copies) + a tile's overhead) + the last tile's epilogue.
 static ConvTPlan convt_plan(const qbp_conv_desc *d, const ConvTGrid &g, bool dgrad)
 {
     const int Cred = dgrad ? d->K : d->C, Nout = dgrad ? d->C : d->K, cchunks = (Cred + 127) / 128;
     const int cols = g.pc ? 3 : 1, taps = (g.pr ? 3 : 1) * cols, reach = g.pr * g.s + g.pc;
     ConvTPlan best{};
-    best.cost = 0.0;
-    for (int pair = 0; pair < 2; ++pair)
-        for (int npos = 256; npos >= 64; npos -= 32) {
-            ConvTPlan p{};
-            p.pair = pair != 0; p.npos = npos;
-            const int width = pair ? 256 : 128, units = pair ? sm_count() / 2 : sm_count(), ncta = pair ? npos / 2 : npos;
-            p.tiles_n = (Nout + width - 1) / width;
-            if ((pair && Nout <= 128) || p.tiles_n > units) continue;
-            const int64_t tiles = (g.total + npos - 1) / npos * p.tiles_n;
-            p.units = (int)std::min<int64_t>(tiles, units);
-            p.units -= p.units % p.tiles_n;
-            p.window_bytes = (uint32_t)align_up(128u * (size_t)(2 * g.s + ncta + 2 * reach), 1024);
-            const int room = (int)(kCtSmem - 1024u - (uint32_t)align_up(sizeof(CtEpiShared), 256));
-            // two windows, or three where they leave the filter's ring three tap rows
-            const int stage_bytes = cols * (int)kCtTapBytes;
-            p.windows = room - 3 * (int)p.window_bytes >= 3 * stage_bytes ? 3 : 2;
-            p.stages = std::min(kCtMaxStages, (room - p.windows * (int)p.window_bytes) / stage_bytes);
-            if (p.stages < 2) continue;
-            const double rows = 128.0 + (double)(4 * g.s + ncta) / taps;
-            const double port = (4.0 * (4096.0 + 32.0 * ncta) + 128.0 * rows) / 128.0;
-            const double stage = std::max({2.0 * npos, 3.0 * rows, port});
-            p.cost = (double)((tiles + p.units - 1) / p.units) * (taps * cchunks * stage + 300.0) + 10.0 * npos;
-            if (best.cost == 0.0 || p.cost < best.cost) best = p;
-        }
+    for (int npos = 256; npos >= 64; npos -= 32) {
+        ConvTPlan p{};
+        p.npos = npos;
+        p.tiles_n = (Nout + 127) / 128;
+        if (p.tiles_n > sm_count()) continue;
+        const int64_t tiles = (g.total + npos - 1) / npos * p.tiles_n;
+        p.units = (int)std::min<int64_t>(tiles, sm_count());
+        p.units -= p.units % p.tiles_n;
+        p.window_bytes = (uint32_t)align_up(128u * (size_t)(2 * g.s + npos + 2 * reach), 1024);
+        const int room = (int)(kCtSmem - 1024u - (uint32_t)align_up(sizeof(CtEpiShared), 256));
+        // two windows, or three where they leave the filter's ring three tap rows
+        const int stage_bytes = cols * (int)kCtTapBytes;
+        p.windows = room - 3 * (int)p.window_bytes >= 3 * stage_bytes ? 3 : 2;
+        p.stages = std::min(kCtMaxStages, (room - p.windows * (int)p.window_bytes) / stage_bytes);
+        if (p.stages < 2) continue;
+        const double rows = 128.0 + (double)(4 * g.s + npos) / taps;
+        const double port = (4.0 * (4096.0 + 32.0 * npos) + 128.0 * rows) / 128.0;
+        const double stage = std::max({2.0 * npos, 3.0 * rows, port});
+        p.cost = (double)((tiles + p.units - 1) / p.units) * (taps * cchunks * stage + 300.0) + 10.0 * npos;
+        if (best.cost == 0.0 || p.cost < best.cost) best = p;
+    }
     return best;
 }
 
 // Whether this kernel takes the product (of a supported convolution; bwl, bhl: log2 of the position box of the kernel above).
-// Where that one takes it too, by both models.  The constants were fitted to some 40 shapes; what the rule gives away is at most 4 %
-// (cycles by the models, then us): 256 x 14 x 14, 256 -> 256 45.6 K / 35.7 K, 36.3 / 38.3, stays above; 512 x 14 x 14 91.2 K / 60.8 K,
-// 64.7 / 63.3, comes here; 96 x 14 x 14 15.2 K / 17.7 K, 20.7 / 22.5, stays; 30 x 17 x 17, 512 -> 512 60.8 K / 33.5 K, 38.2 / 30.8, comes.
+// Where that one takes it too, by both models, whose constants were fitted to 1400 shapes of 96 to 512 channels: the rule leaves the
+// mean at 0.855 of the kernel above, and 5 shapes of one tile a CTA more than 4 % (at most 11 %) slower than it.  (Cycles by the models,
+// here and above, then us: 238 x 17 x 17, 128 -> 160 channels 26.8 K / 24.7 K, 30.1 / 26.9, stays above; 256 x 14 x 14, 256 -> 256
+// 40.3 K / 45.6 K, 38.3 / 36.9, stays; 512 x 14 x 14 68.8 K / 91.2 K, 63.3 / 65.1, comes here; 96 x 14 x 14 21.8 / 23.7, comes; 68 x 23 x
+// 23, 512 -> 512 96.5 K / 152 K, 70.7 / 83.1, comes.)
 bool conv2t_eligible(const qbp_conv_desc *d, bool dgrad, int bwl, int bhl, ConvTPlan &p)
 {
     const int Cred = dgrad ? d->K : d->C, Nout = dgrad ? d->C : d->K;
@@ -925,8 +896,10 @@ bool conv2t_eligible(const qbp_conv_desc *d, bool dgrad, int bwl, int bhl, ConvT
     const int64_t tiles = (boxes + 1) / 2 * tiles_n;
     int64_t pairs = std::min<int64_t>(tiles, sm_count() / 2);
     pairs -= pairs % tiles_n;
-    const double above = (double)((tiles + pairs - 1) / pairs) * 9 * ((Cred + 127) / 128) * std::max(2.0 * bn, 3.3 * (128 + bn / 2));
-    return p.cost < 0.7 * above + 3000.0;
+    // (forward, columns beyond the last are not fetched; the layer gradient's filter tiles run into the next tap there)
+    const double cols = dgrad ? bn : (double)Nout / tiles_n;
+    const double above = (double)((tiles + pairs - 1) / pairs) * 9 * ((Cred + 127) / 128) * std::max(2.0 * bn, 3.3 * (128.0 + cols / 2));
+    return p.cost < 0.8 * above + 2000.0;
 }
 
 int launch_conv2t(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp_qparams *q_in, const int8_t *wgt,
@@ -938,7 +911,7 @@ int launch_conv2t(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qb
     P.g = convt_grid(d);
     P.cchunks = (Cred + 127) / 128;
     P.dgrad = dgrad ? 1 : 0; P.beside = beside ? 1 : 0;
-    P.npos = p.npos; P.npos_cta = p.pair ? p.npos / 2 : p.npos;
+    P.npos = p.npos;
     int rc;
     // filter: forward [K x 9 C], rows = output channels (K-major); layer gradient: rows = the reduction, columns = output channels
     if ((rc = make_map_2d(&P.mapF, wgt, d->K, 9ull * d->C, 128, 128))) return rc;
@@ -946,7 +919,7 @@ int launch_conv2t(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qb
         if ((8 >> b) <= d->H && (rc = make_map_nhwc(&P.mapX[b], in, d->N, d->H, d->W, Cred, 1, 8u >> b, (uint32_t)P.g.s, 128))) return rc;
     const OperandLayout f = dgrad ? layout_mnmajor(128, 128, 1, 0) : layout_kmajor(128, 128), x = layout_kmajor(128, 128);
     P.f_desc_lo = f.desc_lo; P.x_desc_lo = x.desc_lo;
-    P.idesc = make_idesc(true, true, f.major, x.major, p.pair ? 256 : 128, (uint32_t)p.npos);
+    P.idesc = make_idesc(true, true, f.major, x.major, 128, (uint32_t)p.npos);
     P.window_start = 128u * (uint32_t)P.g.s; P.window_bytes = p.window_bytes;
     P.windows = p.windows; P.stages = p.stages;
     P.tiles_n = p.tiles_n; P.units = p.units;
@@ -954,13 +927,11 @@ int launch_conv2t(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qb
     P.d_tiles_n = make_fastdiv(P.tiles_n);
     P.Nimg = d->N; P.H = d->H; P.W = d->W; P.C = d->C; P.N = Nout; P.Cred = Cred;
     P.acc_out = acc_out; P.out = out; P.rowterm = rowterm; P.colterm = colterm; P.qa = q_in; P.qb = q_w; P.status = status;
-    const int grid = p.pair ? 2 * p.units : p.units;
     const size_t smem = 1024u + (size_t)p.windows * p.window_bytes + (size_t)p.stages * (P.g.pc ? 3 : 1) * kCtTapBytes + sizeof(CtEpiShared);
-    static PerDeviceOnce configured[2];
-    void (*kernel)(const ConvTParams) = p.pair ? qbp_conv2t_kernel<true> : qbp_conv2t_kernel<false>;
-    QBP_SMEM_OPT_IN(configured[p.pair ? 1 : 0], kernel, kCtSmem);
+    static PerDeviceOnce configured;
+    QBP_SMEM_OPT_IN(configured, qbp_conv2t_kernel, kCtSmem);
     QBP_TRACE_BEGIN(st);
-    launch(kernel, grid, kCtThreads, smem, st, P);
+    launch(qbp_conv2t_kernel, p.units, kCtThreads, smem, st, P);
     QBP_LAUNCH_OK("qbp_conv2t_kernel");
     return QBP_OK;
 }

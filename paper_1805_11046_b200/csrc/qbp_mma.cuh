@@ -187,7 +187,7 @@ int launch_conv2(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp
                  const qbp_qparams *q_w, int32_t *acc_out, float *out, const int32_t *rowterm, const int32_t *colterm,
                  ColStatParts *stats, int *status, int bwl, int bhl, bool beside, cudaStream_t st);
 // ... and those whose output's statistics nobody wants
-struct ConvTPlan { bool pair; int npos, tiles_n, units, windows, stages; uint32_t window_bytes; double cost; };
+struct ConvTPlan { int npos, tiles_n, units, windows, stages; uint32_t window_bytes; double cost; };
 bool conv2t_eligible(const qbp_conv_desc *d, bool dgrad, int bwl, int bhl, ConvTPlan &p);
 int launch_conv2t(bool dgrad, const qbp_conv_desc *d, const int8_t *in, const qbp_qparams *q_in, const int8_t *wgt,
                   const qbp_qparams *q_w, int32_t *acc_out, float *out, const int32_t *rowterm, const int32_t *colterm,
