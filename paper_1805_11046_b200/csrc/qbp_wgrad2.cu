@@ -298,16 +298,35 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kW2Threads, 1) qbp_w
     }
 }
 
+// Columns of a pair tile: where tiles of 256 fit the pairs once, half as many (64 at least) as long as they do: rings and epilogues get
+// shorter, and SMs that had none take part.  Call with its sums, 256 columns -> by this rule: 1024 rows for 2048 x 1008 18.3 ->
+// 15.6 us, 4096 for 1024 x 1024 31.7 -> 24.1, 16384 for 256 x 512 84.9 -> 57.0.  And never wider than the columns there are, also
+// where the row tiles alone do not fit: 4096 rows for 20000 x 128 68.4 -> 54.7 (single-CTA kernel 52.3), 1024 for 65536 x 128
+// 55.9 -> 44.3 (49.3), 8192 for 65536 x 64 264 -> 216 (200)
+static int w2_columns(int64_t N, int64_t K)
+{
+    const int64_t tiles_m = (K + 255) / 256;
+    int bn = 256;
+    while (bn > 64 && (N <= bn / 2 || tiles_m * ((N + bn / 2 - 1) / (bn / 2)) <= sm_count() / 2)) bn /= 2;
+    return bn;
+}
+
 // Whether the pair kernel takes this plain product: a reduction that one pair can hold in int32, and one of (call with its sums, first
 // with the single-CTA kernel, then with this one)
-//   - fewer than 512 rows: large outputs (64 rows for 2048 x 2048: 15.7 and 13.3 us; not 384 for 256 x 256: 9.2 and 9.6);
+//   - fewer than 512 rows (or 640): large outputs (64 rows for 2048 x 2048: 15.7 and 13.3 us; not 384 for 256 x 256: 9.2 and 9.6, nor
+//     539 for 192 x 672: 9.7 and 10.4);
 //   - more: where the longer walk of a pair over all rows, about 2.9 us per 1000, costs less than the single-CTA kernel's
 //     partial sums, about 1 us per 10000 outputs (8192 rows for 4096 x 128: 68.9 and 39.6, 2048 for 1024 x 208: 35.2 and 16.3; not
 //     512 for 128 x 128: 9.1 and 9.4, 8192 for 128 x 128: 20.5 and 31.9, 65536 for 256 x 256: 49.6 and 228).
+//   - and not where its tiles stay 256 columns wide although 128 x 128 tiles of the other kernel fit the SMs once: those leave half as
+//     much to read out per CTA, on nearly all SMs (558 rows for 1568 x 1328: 14.2 and 16.8, 16 for 1568 x 1296 11.2 and 13.2, 1162 for
+//     832 x 2480 18.6 and 20.8).
 bool wgrad2_eligible(int64_t M, int64_t N, int64_t K)
 {
     if (M > 65536 || N < 64 || K < 64) return false;
-    return M < 512 ? N * K >= (1 << 20) : N * K >= (1 << 15) && 29 * M <= 30000 + N * K;
+    if (N * K < (M < 512 ? 1 << 20 : M < 640 ? 1 << 18 : 1 << 15) || (M >= 512 && 29 * M > 30000 + N * K)) return false;
+    const bool once = (K + 255) / 256 * ((N + 255) / 256) <= sm_count() / 2;
+    return !(once && w2_columns(N, K) == 256 && (K + 127) / 128 * ((N + 127) / 128) <= sm_count());
 }
 
 int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qparams *qx, const int8_t *g_hi,
@@ -316,16 +335,8 @@ int launch_wgrad2(int64_t M, int64_t N, int64_t K, const int8_t *x, const qbp_qp
 {
     Wgrad2Params P{};
     int rc;
-    // where tiles of 256 columns fit the pairs once, tiles of half as many (64 at least) as long as they do: rings and epilogues get
-    // shorter, and SMs that had none take part.  Call with its sums, 256 columns -> by this rule: 1024 rows for 2048 x 1008 18.3 ->
-    // 15.6 us, 4096 for 1024 x 1024 31.7 -> 24.1, 16384 for 256 x 512 84.9 -> 57.0.  And never wider than the columns there are, also
-    // where the row tiles alone do not fit: 4096 rows for 20000 x 128 68.4 -> 54.7 (single-CTA kernel 52.3), 1024 for 65536 x 128
-    // 55.9 -> 44.3 (49.3), 8192 for 65536 x 64 264 -> 216 (200)
-    const auto tiles_n_of = [&](int bn) { return (N + bn - 1) / bn; };
-    P.tiles_m = (int)((K + 255) / 256);
-    P.bn = 256;
-    while (P.bn > 64 && (N <= P.bn / 2 || P.tiles_m * tiles_n_of(P.bn / 2) <= sm_count() / 2)) P.bn /= 2;
-    P.tiles_n = (int)tiles_n_of(P.bn);
+    P.bn = w2_columns(N, K);
+    P.tiles_m = (int)((K + 255) / 256); P.tiles_n = (int)((N + P.bn - 1) / P.bn);
     P.tiles_total = P.tiles_m * P.tiles_n;
     // per-CTA operand parts: 128 reduction rows x 128 columns of X, x bn / 2 of each limb, M/N-major
     const uint32_t half = (uint32_t)P.bn / 2;

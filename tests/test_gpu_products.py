@@ -302,6 +302,13 @@ def test_wgrad_pair_kernel_more_row_tiles_than_pairs(B, M, N, K):
     test_wgrad_plain_pair_kernel_narrow_tiles(B, M, N, K)
 
 
+@pytest.mark.parametrize("M,N,K", [(640, 64, 528), (656, 272, 304), (624, 512, 512), (624, 496, 512), (558, 1328, 1568), (1162, 1328, 1568)])
+def test_wgrad_either_side_of_the_pair_kernels_rule(B, M, N, K):
+    """The fewest rows for small and middle outputs, one step short of the latter, tiles that would stay 256 columns wide where the
+    single-CTA kernel's fit the SMs once."""
+    test_wgrad_plain_pair_kernel_narrow_tiles(B, M, N, K)
+
+
 # The CTA-pair kernel where it fits the SM pairs once: tiles of 64, 128 and 256 columns, ragged in every dimension, fewer
 # reduction steps than the ring has stages and more; outputs smaller than a tile, the fewest rows; the last is just too deep for it.
 @pytest.mark.parametrize("M,N,K", [(528, 272, 304), (2064, 256, 256), (560, 1008, 2064), (1536, 784, 4368), (1040, 208, 160),
