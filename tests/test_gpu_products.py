@@ -572,7 +572,7 @@ def test_conv_pairs(B, N, H, W, C, K, mode):
 @pytest.mark.parametrize("mode", [0, 1])
 def test_conv_channels_as_rows(B, N, H, W, C, K, mode):
     """Products without statistics.  Images of one row or column (no padding that way, fewer taps), of a tile's exact size, one and
-    several panels of columns with a narrower last one, channel chunks partly filled, pairs and single CTAs, several tiles of each."""
+    several panels of columns with a narrower last one, channel chunks partly filled, one and several tiles of a CTA, of one and several tiles of channels."""
     d = B.conv_desc(N, H, W, C, K, 3, 3, 1, 1); od = O.conv_desc(N, H, W, C, K, 3, 3, 1, 1)
     inp = random_codes((N, H, W, C if mode == 0 else K), 84); w = random_codes((K, 3, 3, C), 85)
     acc, out, ws = B.qbp_conv_s8_implicit(mode, d, to_dev(inp), _qp(B, 0.5, 17), to_dev(w), _qp(B, 0.25, -23), want_acc=True)
